@@ -329,6 +329,9 @@ struct NttFinish {
 // out_double (forward, N = 2^16 only): such rows are left as doubles with |x| <= q/2 for a consumer that computes in FP64.
 int ntt_launch(fesc_ctx* ctx, u64* d_data, size_t rows, const RowMap& map, bool inverse, cudaStream_t st,
                bool in_double = false, bool out_double = false, const NttFinish* finish = nullptr);
+// N = 2^16 kernels (ntt16.cu)
+int ntt16_launch(fesc_ctx* ctx, u64* data, size_t rows, const RowMap& map, bool inverse, cudaStream_t st, bool in_double,
+                 bool out_double, const NttFinish& fin, uint64_t& launches);
 // double with |x| <= q/2 as handed to the forward transform
 __device__ __forceinline__ u64 fp_handoff(double s, double q, double qinv) {
     return (u64)__double_as_longlong(fp_reduce(s, q, qinv));
