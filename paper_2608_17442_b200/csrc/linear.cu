@@ -595,13 +595,63 @@ static int bsgs_kernel() {
     return v;
 }
 // Larger groups re-read the diagonals less often and give the key-switch kernels larger batches; every token block
-// of a group needs its rotated inputs and its partial sums resident.  Budget: 28 GiB of scratch for them (37 GiB with packed operands, whose packed inputs
-// and key-switch chunk count as well; 44 GiB allows groups of 8; a fixed figure, so the launch shape does not depend on what else holds memory); if the device cannot provide the scratch,
-// the group is halved until it fits.
-static size_t bsgs_group_bytes(bool packed) {
+// of a group needs its rotated inputs and its partial sums resident.  Budget for residue operands: 28 GiB of scratch (a
+// fixed figure, so the launch shape does not depend on what else holds memory).
+static size_t bsgs_group_bytes() {
     const char* e = getenv("FESC_BSGS_GROUP_GIB");
     if (e && atoi(e) > 0) return (size_t)atoi(e) << 30;
-    return (size_t)(packed ? 37 : 28) << 30;
+    return (size_t)28 << 30;
+}
+// Packed operands: the budget is what an image of in_proj's size (110 GiB) leaves on a device of 178 GiB, 37 GiB, and
+// grows by what a smaller image leaves free, up to 64 GiB.
+static size_t packed_group_bytes(size_t image_bytes) {
+    const char* e = getenv("FESC_BSGS_GROUP_GIB");
+    if (e && atoi(e) > 0) return (size_t)atoi(e) << 30;
+    const size_t full = (size_t)111 << 30, least = (size_t)37 << 30, most = (size_t)64 << 30;
+    const size_t b = image_bytes < full ? least + (full - image_bytes) : least;
+    return b < most ? b : most;
+}
+
+// How a projection on packed diagonals is cut: token blocks per group and output blocks per part of a group.
+struct PackedPlan {
+    uint32_t tbg, nb_part;
+    size_t rot_words, acc_words, xpk_words, total;      // words; bytes of scratch in all
+};
+// Every cut is charged what its accumulate launches have to read plus the tensor work of its tiles of 4 token blocks in the
+// same unit (an image's tensor work takes about half as long as reading it at full size: 13.5 against 21 ms; periodic
+// images keep the tensor work and lose the reading): per group the image once and the packed inputs once per part, and the
+// tiles, full or not.  A group of 1 or 2 pays for a whole tile, which is why a projection whose rotated inputs are large (189
+// terms, 210 accumulators per token block) is worth 58 GiB of scratch: 1086 ms with groups of 1, 592 ms with groups of 4
+// (8 token blocks).
+static PackedPlan packed_plan(const fesc_ctx* ctx, const fesc_bsgs_desc* desc, uint32_t tbg_max, size_t budget) {
+    const uint32_t n2 = desc->n2, gin = desc->in_blocks, nout = desc->out_blocks, tbs = desc->token_blocks;
+    const uint32_t level = desc->n_limbs, N = ctx->N, terms = gin * desc->n1;
+    const size_t ctw = (size_t)2 * level * N;
+    uint32_t bstep = 8;                    // a part starts at a (b,p) pair that is a multiple of 8
+    while (bstep > 1 && (bstep / 2) * n2 % 8 == 0) bstep /= 2;
+    const double image = (double)bsgs_packed_bytes(N >> desc->diag_run_log2, level, nout * n2, terms);
+    const double tensor = 0.5 * (double)bsgs_packed_bytes(N, level, nout * n2, terms);
+    PackedPlan best{};
+    double best_cost = 0;
+    for (uint32_t tbg = tbg_max;; tbg = tbg > 4 ? 4 : (tbg + 1) / 2) {
+        const uint32_t tiles = (tbg + 3) / 4, sub = tbg < 4 ? tbg : 4, groups = (tbs + tbg - 1) / tbg;
+        for (uint32_t nb = (nout + bstep - 1) / bstep * bstep;; nb -= bstep) {
+            PackedPlan p;
+            p.tbg = tbg, p.nb_part = nb < nout ? nb : nout;
+            const uint32_t parts = (nout + p.nb_part - 1) / p.nb_part;
+            const uint32_t max_batch = sub * gin > tbg * p.nb_part ? sub * gin : tbg * p.nb_part;
+            const size_t ks_words = ks_scratch_words(ctx, level, ks_chunk(ctx, max_batch), desc->defer ? giant_ext_buffers(n2) : 1);
+            const size_t rs_words = (size_t)(p.nb_part < 16384 ? p.nb_part : 16384) * 2 * N;
+            p.rot_words = (size_t)sub * terms * ctw, p.acc_words = (size_t)tbg * p.nb_part * n2 * ctw;
+            p.xpk_words = bsgs_packed_bytes(N, level, 2 * tbg, terms) / 8;
+            p.total = (p.rot_words + p.acc_words + p.xpk_words + (ks_words > rs_words ? ks_words : rs_words)) * sizeof(u64);
+            const double cost = groups * (image + parts * 8.0 * (double)p.xpk_words + tiles * tensor);
+            const bool least = tbg == 1 && nb <= bstep;
+            if ((p.total <= budget && (best.tbg == 0 || cost < best_cost)) || (best.tbg == 0 && least)) best = p, best_cost = cost;
+            if (nb <= bstep) break;
+        }
+        if (tbg == 1) return best;
+    }
 }
 
 // Projection on packed diagonals.  Token blocks are processed in groups of up to 8 = two tiles of 4: the baby rotations
@@ -615,37 +665,21 @@ static int linear_packed(fesc_ctx* ctx, const u64* in, const uint8_t* image, con
     const uint32_t n1 = desc->n1, n2 = desc->n2, gin = desc->in_blocks, nout = desc->out_blocks;
     const uint32_t tbs = desc->token_blocks, level = desc->n_limbs, N = ctx->N, terms = gin * n1;
     const size_t ctw = (size_t)2 * level * N, ctw_out = (size_t)2 * (level - 1) * N;
-    uint32_t bstep = 8;                    // a part starts at a (b,p) pair that is a multiple of 8
-    while (bstep > 1 && (bstep / 2) * n2 % 8 == 0) bstep /= 2;
-    if (n2 % 8 == 0) bstep = 1;
-    u64 *scratch = nullptr, *rot = nullptr, *acc = nullptr, *ks = nullptr;
-    uint8_t* xpk = nullptr;
-    uint32_t tbg = tbs >= 8 ? 8 : tbs, nb_part = nout;
+    u64* scratch = nullptr;
+    const size_t budget = packed_group_bytes(bsgs_packed_bytes(N >> desc->diag_run_log2, level, nout * n2, terms));
+    PackedPlan plan;
     int rc = FESC_ENOMEM;
-    for (;; tbg = tbg > 4 ? 4 : (tbg + 1) / 2) {
-        const uint32_t parts = (tbg + 3) / 4, sub = tbg < 4 ? tbg : 4;
-        nb_part = (nout + parts - 1) / parts;
-        nb_part = (nb_part + bstep - 1) / bstep * bstep;
-        if (nb_part > nout) nb_part = nout;
-        const uint32_t max_batch = sub * gin > tbg * nb_part ? sub * gin : tbg * nb_part;
-        const size_t ks_words = ks_scratch_words(ctx, level, ks_chunk(ctx, max_batch), desc->defer ? giant_ext_buffers(n2) : 1);
-        const size_t rs_words = (size_t)(nb_part < 16384 ? nb_part : 16384) * 2 * N;
-        const size_t rot_words = (size_t)sub * terms * ctw, acc_words = (size_t)tbg * nb_part * n2 * ctw;
-        const size_t xpk_words = bsgs_packed_bytes(N, level, 2 * tbg, terms) / 8;
-        const size_t total = (rot_words + acc_words + xpk_words + (ks_words > rs_words ? ks_words : rs_words)) * sizeof(u64);
-        if (total <= bsgs_group_bytes(true) || tbg == 1) {
-            rc = ctx_scratch(ctx, total, &scratch);
-            if (rc == FESC_OK) {
-                rot = scratch;
-                acc = rot + rot_words;
-                xpk = (uint8_t*)(acc + acc_words);
-                ks = acc + acc_words + xpk_words;
-                break;
-            }
-            if (rc != FESC_ENOMEM) return rc;
-        }
-        if (tbg == 1) return rc;
+    for (uint32_t most = tbs >= 8 ? 8 : tbs;; most = most > 4 ? 4 : (most + 1) / 2) {     // smaller groups until the scratch can be had
+        plan = packed_plan(ctx, desc, most, budget);
+        most = plan.tbg;
+        rc = ctx_scratch(ctx, plan.total, &scratch);
+        if (rc == FESC_OK) break;
+        if (rc != FESC_ENOMEM || most == 1) return rc;
     }
+    const uint32_t tbg = plan.tbg, nb_part = plan.nb_part;
+    u64 *rot = scratch, *acc = rot + plan.rot_words;
+    uint8_t* xpk = (uint8_t*)(acc + plan.acc_words);
+    u64* ks = acc + plan.acc_words + plan.xpk_words;
     ctx->counters[5] = tbg;
     const size_t tile_bytes = bsgs_packed_bytes(N, level, 8, terms);     // one tile of 8 rows of packed inputs
     const uint32_t dshift = desc->diag_run_log2;
@@ -728,7 +762,7 @@ extern "C" int fesc_linear(fesc_ctx* ctx, const uint64_t* d_ct_in, const uint64_
     }
     // residue diagonals from here on; token blocks per group, from the scratch budget
     const size_t per_tb = ((size_t)gin * n1 + (size_t)nout * n2) * ctw * sizeof(u64);
-    uint32_t tbg = (uint32_t)(bsgs_group_bytes(false) / per_tb);
+    uint32_t tbg = (uint32_t)(bsgs_group_bytes() / per_tb);
     if (tbg < 1) tbg = 1;
     if (tbg > tbs) tbg = tbs;
     u64 *scratch = nullptr, *rot = nullptr, *acc = nullptr, *ks = nullptr;
