@@ -63,6 +63,12 @@ struct PrimeConst {
     double ninvd;
     double ninvwd;
 };
+// Constants of an inverse transform's last stage (N^-1 and N^-1 psi^-brev(1), times a factor of the caller's): Shoup pairs, and
+// centred doubles for primes below 2^50.
+struct InvScale {
+    u64 n, ns, w, ws;
+    double nd, wd;
+};
 
 // ---------------------------------------------------------------------------------------
 // Device arithmetic.  All moduli are < 2^62, so 4q fits in 64 bits.
@@ -192,12 +198,17 @@ struct RowMap {
 // ---------------------------------------------------------------------------------------
 // Basis-conversion tables (device copies; built on the host in ctx.cu)
 // ---------------------------------------------------------------------------------------
+struct alignas(16) ModUpTerm {      // read with one 16-byte load
+    long long m;     // (Q_j/q_i) mod q_t in [-q_t/2, q_t/2]
+    double mq;       // m / q_t
+};
 // One key-switch digit at one level: source limbs [first, first+n_src), Q_j = their product.
 struct ModUpDigit {
     uint32_t n_src, first;
     u64 inv[FESC_MAX_ALPHA], invs[FESC_MAX_ALPHA];   // (Q_j/q_i)^-1 mod q_i and its Shoup companion
     u64 mat[FESC_MAX_ALPHA][FESC_MAX_PRIMES];        // (Q_j/q_i) mod q_t, t = prime index
     double matd[FESC_MAX_ALPHA][FESC_MAX_PRIMES];    // the same as doubles (exact for targets below 2^53)
+    ModUpTerm term[FESC_MAX_ALPHA][FESC_MAX_PRIMES]; // the same centred (modup16.cu)
 };
 // Division by P = product of the special primes p_k.
 struct ModDownTab {
@@ -219,6 +230,7 @@ struct RescaleTab {
 };
 struct Tables {
     ModUpDigit* d_modup;      // [(level-1) * beta_max + digit], level = 1..n_q
+    InvScale* d_up_scale;     // [(level-1) * n_q + limb]: factor (Q_j/q_limb)^-1 mod q_limb
     ModDownTab* d_moddown;
     RescaleTab* d_rescale;    // [level], level = 2..n_q (index 0,1 unused)
     u64* d_Pmod_all;          // P mod q_t for every prime index (0 on special primes)
@@ -249,7 +261,8 @@ struct fesc_ctx {
     std::vector<u64> q;           // host primes
     std::vector<PrimeConst> pc;   // host copy
     PrimeConst* d_pc;             // device [n_primes]
-    ulonglong2* d_tw;             // forward twiddles [n_primes][N] (w, shoup)
+    ulonglong2* d_tw;             // forward twiddles [n_primes][N] (w, shoup); N = 2^16: entries from 4096 on regrouped
+                                  // (ntt16_twiddle_slot), here and in the three tables below
     ulonglong2* d_itw;            // inverse twiddles [n_primes][N]
     double* d_twf;                // the same twiddles as doubles, rows of primes >= 2^50 unused
     double* d_itwf;
@@ -326,12 +339,24 @@ struct NttFinish {
 // rows: number of N-word rows starting at d_data; map gives the prime per row.
 // in_double (forward, N = 2^16 only): rows on primes below 2^50 hold doubles with |x| <= q/2 (bit patterns) written by a
 // basis-conversion kernel instead of canonical words.
+// scale (inverse, N = 2^16 only): per prime index, constants in place of those of the last stage.  skip_cols (forward, N = 2^16 only): the first eight stages are already done.
 // out_double (forward, N = 2^16 only): such rows are left as doubles with |x| <= q/2 for a consumer that computes in FP64.
 int ntt_launch(fesc_ctx* ctx, u64* d_data, size_t rows, const RowMap& map, bool inverse, cudaStream_t st,
-               bool in_double = false, bool out_double = false, const NttFinish* finish = nullptr);
+               bool in_double = false, bool out_double = false, const NttFinish* finish = nullptr,
+               const InvScale* scale = nullptr, bool skip_cols = false);
+// Where twiddle i of a row of N = 2^16 points is kept.  The last four forward stages read, per 512-point block and lane, one
+// twiddle of stage 12, two of stage 13, four and eight: 15 values that lie up to 120 bytes apart between lanes.  They are
+// stored lane by lane within the block instead, in pairs for the FP64 table (16-byte loads, 512 contiguous bytes per warp), one
+// by one for the 16-byte integer entries; i < 4096 stays where it is.
+static inline uint32_t ntt16_twiddle_slot(uint32_t i, bool pairs) {
+    if (i < 4096) return i;
+    const uint32_t s = 31 - __builtin_clz(i) - 12, g = (i >> s) - 4096, j = i & ((1u << s) - 1), blk = g >> 5, lane = g & 31;
+    if (!pairs || s == 0) return 4096 + 480 * blk + 32 * ((1u << s) - 1 + j) + lane;
+    return 4096 + 480 * blk + 32 + 64 * ((1u << (s - 1)) - 1 + (j >> 1)) + 2 * lane + (j & 1);
+}
 // N = 2^16 kernels (ntt16.cu)
 int ntt16_launch(fesc_ctx* ctx, u64* data, size_t rows, const RowMap& map, bool inverse, cudaStream_t st, bool in_double,
-                 bool out_double, const NttFinish& fin, uint64_t& launches);
+                 bool out_double, const NttFinish& fin, uint64_t& launches, const InvScale* scale, bool skip_cols);
 // double with |x| <= q/2 as handed to the forward transform
 __device__ __forceinline__ u64 fp_handoff(double s, double q, double qinv) {
     return (u64)__double_as_longlong(fp_reduce(s, q, qinv));

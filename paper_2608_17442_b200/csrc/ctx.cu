@@ -316,6 +316,15 @@ static void bconv_fragments(uint4* out, F C) {
             }
 }
 
+// constants of the inverse transform's last stage times f
+static InvScale inv_scale(const PrimeConst& pc, u64 f) {
+    auto centred = [&](u64 v) { return v > pc.q / 2 ? -(double)(pc.q - v) : (double)v; };
+    InvScale s;
+    s.n = h_mul(pc.ninv, f, pc.q), s.ns = h_shoup(s.n, pc.q);
+    s.w = h_mul(pc.ninvw, f, pc.q), s.ws = h_shoup(s.w, pc.q);
+    s.nd = centred(s.n), s.wd = centred(s.w);
+    return s;
+}
 static int build_tables(fesc_ctx* ctx) {
     const uint32_t nq = ctx->n_q, np = ctx->n_primes, K = ctx->n_p, alpha = ctx->alpha;
     const std::vector<u64>& q = ctx->q;
@@ -323,6 +332,7 @@ static int build_tables(fesc_ctx* ctx) {
     // ModUp: for every level and digit
     std::vector<ModUpDigit> mu((size_t)nq * ctx->beta_max);
     memset(mu.data(), 0, mu.size() * sizeof(ModUpDigit));
+    std::vector<InvScale> scale((size_t)nq * nq, InvScale{});
     for (uint32_t level = 1; level <= nq; level++) {
         for (uint32_t j = 0; j * alpha < level; j++) {
             ModUpDigit& d = mu[(size_t)(level - 1) * ctx->beta_max + j];
@@ -338,12 +348,16 @@ static int build_tables(fesc_ctx* ctx) {
                         if (b != a) m = h_mul(m, q[d.first + b] % q[t], q[t]);
                     d.mat[a][t] = m;
                     d.matd[a][t] = (double)m;
+                    d.term[a][t].m = m > q[t] / 2 ? -(long long)(q[t] - m) : (long long)m;
+                    d.term[a][t].mq = (double)((long double)d.term[a][t].m / (long double)q[t]);
                 }
                 d.inv[a] = h_inv(d.mat[a][i], q[i]);
                 d.invs[a] = h_shoup(d.inv[a], q[i]);
+                scale[(size_t)(level - 1) * nq + i] = inv_scale(ctx->pc[i], d.inv[a]);
             }
         }
     }
+    if ((rc = upload(ctx, &ctx->tabs.d_up_scale, scale)) != FESC_OK) return rc;
     if ((rc = upload(ctx, &ctx->tabs.d_modup, mu)) != FESC_OK) return rc;
     // ModDown
     std::vector<ModDownTab> mdv(1);
@@ -407,6 +421,7 @@ static int build_tables(fesc_ctx* ctx) {
 }
 static void free_tables(fesc_ctx* ctx) {
     dev_free(ctx->tabs.d_modup);
+    dev_free(ctx->tabs.d_up_scale);
     dev_free(ctx->tabs.d_moddown);
     dev_free(ctx->tabs.d_rescale);
     dev_free(ctx->tabs.d_Pmod_all);
@@ -519,12 +534,13 @@ extern "C" int fesc_ctx_create(fesc_ctx** out, uint32_t log_n, const uint64_t* p
         }
         for (uint32_t k = 0; k < N; k++) {
             uint32_t r = h_brev(k, log_n);
-            tw[(size_t)i * N + k] = make_ulonglong2(pw[r], h_shoup(pw[r], q));
-            itw[(size_t)i * N + k] = make_ulonglong2(ipw[r], h_shoup(ipw[r], q));
+            const uint32_t ki = log_n == 16 ? ntt16_twiddle_slot(k, false) : k, kf = log_n == 16 ? ntt16_twiddle_slot(k, true) : k;
+            tw[(size_t)i * N + ki] = make_ulonglong2(pw[r], h_shoup(pw[r], q));
+            itw[(size_t)i * N + ki] = make_ulonglong2(ipw[r], h_shoup(ipw[r], q));
             if (q < (1ull << 50)) {
                 // centred representatives (|w| <= q/2) halve the rounding term of the exact FP64 product
-                twf[(size_t)i * N + k] = pw[r] > q / 2 ? -(double)(q - pw[r]) : (double)pw[r];
-                itwf[(size_t)i * N + k] = ipw[r] > q / 2 ? -(double)(q - ipw[r]) : (double)ipw[r];
+                twf[(size_t)i * N + kf] = pw[r] > q / 2 ? -(double)(q - pw[r]) : (double)pw[r];
+                itwf[(size_t)i * N + kf] = ipw[r] > q / 2 ? -(double)(q - ipw[r]) : (double)ipw[r];
             }
         }
         pc.ninvw = h_mul(pc.ninv, ipw[h_brev(1, log_n)], q);

@@ -1,0 +1,163 @@
+// ModUp fused with the first pass of the forward transform (N = 2^16, data primes below 2^50, at most 4 limbs per digit).
+//
+// Per digit j and target modulus q_t:  ext_t = sum_a y_a m_a mod q_t,  y_a = d_a (Q_j/q_a)^-1 mod q_a (left by the inverse
+// transform, whose last stage multiplies by N^-1 (Q_j/q_a)^-1),  m_a = (Q_j/q_a) mod q_t.  The converted rows are formed in
+// the registers of the transform's first eight stages: they never exist in memory, which saves writing and reading
+// (level + K - n_src) rows per digit.
+//
+// The sum is an exact mixed-pipe product: its quotient c = rint(sum_a y_a (m_a / q)) comes from the FP64 pipe (one
+// multiply-add per term, m centred; |sum| < 2^51, so the error stays below 0.75 and |v| <= 1.25 q < 2^63), its value
+// v = sum_a y_a m_a - c q from wrapping 64-bit integer products on the multiplier pipe, which the FP64 butterflies leave idle.
+//
+// A CTA owns 4 columns of one digit of one ciphertext: the source columns (8 KB per limb) are read once into shared memory
+// and serve all targets; six groups of 64 threads take targets from a counter, the slower rows on the 60-bit primes first.
+//
+// What bounds it: the dispatch of wide operands (an FP64 multiply-add of three registers holds its port for three cycles), which
+// conversion and butterflies share; 0.38 us per converted row at 24 limbs and 16 ciphertexts against 0.41 for a conversion kernel
+// and a first pass of their own, and 1.2 GB less traffic per launch.  8 columns with 8 groups 0.39; four exact FP64 products
+// per word instead of the mixed sum 0.53 (the rounding unit takes nine cycles per product); byte planes on the tensor cores,
+// eight targets at a time through shared memory, 0.45; the same for the division by P 0.51 against 0.36 unfused.
+#define FESC_DBG_FILE 12   // file id in the sites a debug build reports
+#include "ntt16.cuh"
+#include "ops.cuh"
+
+#define MU_GROUPS 6
+#define MU_COLS 4
+#define MU_TARGET_THREADS (MU_COLS * 16)
+#define MU_THREADS (MU_GROUPS * MU_TARGET_THREADS)
+#define MU_SRC (256 * MU_COLS)      // words of one source limb's columns
+
+struct GroupBarrier {
+    uint32_t id;
+    __device__ __forceinline__ void operator()() const { asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(MU_TARGET_THREADS) : "memory"); }
+};
+
+#define FP_MAGIC 6755399441055744.0      // 1.5 * 2^52: the low mantissa bits of FP_MAGIC + c hold the integer c, |c| < 2^51
+#define FP_MAGIC_HI 0x43380000u
+
+// v[0..3] = sum_a y_a m_a - c q (two's complement) for the points p, p + 16 MU_COLS, ... of the source columns
+template <int A>
+__device__ __forceinline__ void convert4(const u64* p, uint32_t n_src, const ModUpTerm (*__restrict__ term)[FESC_MAX_PRIMES], uint32_t pt,
+                                         u64 q, u64* v) {
+    u64 acc[4];            // low product words, and the cross terms of weight 2^32 apart from them
+    uint32_t cross[4];
+    double s[4];
+#pragma unroll
+    for (int e = 0; e < 4; e++) acc[e] = 0, cross[e] = 0, s[e] = 0.0;
+#pragma unroll
+    for (int a = 0; a < A; a++) {
+        if (a >= n_src) break;
+        const ulonglong2 t = __ldg(reinterpret_cast<const ulonglong2*>(&term[a][pt]));
+        const uint32_t ml = (uint32_t)t.x, mh = (uint32_t)(t.x >> 32);
+        const double mq = __longlong_as_double((long long)t.y);
+#pragma unroll
+        for (int e = 0; e < 4; e++) {
+            const u64 y = p[a * MU_SRC + e * 16 * MU_COLS];
+            const uint32_t yl = (uint32_t)y, yh = (uint32_t)(y >> 32);
+            s[e] = __fma_rn(fp_from_u64(y), mq, s[e]);
+            asm("mad.wide.u32 %0, %1, %2, %0;" : "+l"(acc[e]) : "r"(yl), "r"(ml));
+            asm("mad.lo.u32 %0, %1, %2, %0;" : "+r"(cross[e]) : "r"(yl), "r"(mh));
+            asm("mad.lo.u32 %0, %1, %2, %0;" : "+r"(cross[e]) : "r"(yh), "r"(ml));
+        }
+    }
+    const u64 nq = 0 - q;
+    const uint32_t ql = (uint32_t)nq, qh = (uint32_t)(nq >> 32);
+#pragma unroll
+    for (int e = 0; e < 4; e++) {
+        const u64 c = (u64)__double_as_longlong(__dadd_rn(s[e], FP_MAGIC));
+        const uint32_t cl = (uint32_t)c, ch = (uint32_t)(c >> 32) - FP_MAGIC_HI;
+        asm("mad.wide.u32 %0, %1, %2, %0;" : "+l"(acc[e]) : "r"(cl), "r"(ql));
+        const uint32_t hi = (uint32_t)(acc[e] >> 32) + (cross[e] + cl * qh + ch * ql);
+        v[e] = ((u64)hi << 32) | (uint32_t)acc[e];
+    }
+}
+
+template <int A>
+__global__ void __launch_bounds__(MU_THREADS, 2)
+    k_modup_cols(const u64* __restrict__ y, u64* __restrict__ ext, const ModUpDigit* __restrict__ tab, const double* __restrict__ twf,
+                 const ulonglong2* __restrict__ tw, const PrimeConst* __restrict__ pcs, uint32_t level, uint32_t n_q, uint32_t K,
+                 uint32_t beta, uint32_t splits) {
+    extern __shared__ __align__(16) u64 smem[];      // [A][MU_SRC] source columns, then one exchange buffer per group
+    __shared__ uint32_t next, taken[MU_GROUPS];
+    const uint32_t tid = threadIdx.x, tile = blockIdx.x / splits, part = blockIdx.x % splits, j = blockIdx.y, b = blockIdx.z;
+    const ModUpDigit* dg = tab + j;
+    const uint32_t first = dg->first, n_src = dg->n_src, rows = level + K, others = rows - n_src;
+    const u64* src = y + ((size_t)b * level + first) * N16 + tile * MU_COLS;
+    u64* out = ext + ((size_t)b * beta + j) * rows * N16 + tile * MU_COLS;
+    if (!DBG_REGION(dg, sizeof(ModUpDigit)) || !DBG_REGION(src - tile * MU_COLS, (size_t)n_src * N16 * sizeof(u64)) ||
+        !DBG_REGION(out - tile * MU_COLS, (size_t)rows * N16 * sizeof(u64)))
+        return;                                     // the same for the whole CTA
+    for (uint32_t i = tid; i < n_src * (MU_SRC / 2); i += MU_THREADS) {
+        const uint32_t a = i / (MU_SRC / 2), r = (i / (MU_COLS / 2)) & 255, c = 2 * (i % (MU_COLS / 2));
+        *reinterpret_cast<ulonglong2*>(smem + a * MU_SRC + r * MU_COLS + c) =
+            *reinterpret_cast<const ulonglong2*>(src + (size_t)a * N16 + r * 256 + c);
+    }
+    if (tid == 0) next = 0;
+    __syncthreads();
+    const uint32_t group = tid / MU_TARGET_THREADS, gt = tid % MU_TARGET_THREADS, col = gt % MU_COLS, sub = gt / MU_COLS;
+    const GroupBarrier bar{1 + group};
+    u64* sm = smem + A * MU_SRC + group * COL_SMEM(MU_COLS);
+    const u64* ys = smem + sub * MU_COLS + col;
+    for (;;) {
+        if (gt == 0) taken[group] = atomicAdd(&next, 1u);
+        bar();
+        const uint32_t o = taken[group] * splits + part;      // (the exchange's barrier keeps the next write behind this read)
+        if (o >= others) return;
+        const uint32_t d = o < K ? 0 : o - K;
+        const uint32_t t = o < K ? level + o : (d < first ? d : d + n_src), pt = o < K ? n_q + o : t;
+        u64* p = out + (size_t)t * N16 + col;
+        const u64 q = pcs[pt].q;
+        if (q < FESC_FP_LIMIT) {
+            FpRow r{twf + (size_t)pt * N16, pcs[pt].qd, pcs[pt].qinvd};
+            double x[16];
+#pragma unroll
+            for (int k = 0; k < 16; k += 4) {
+                u64 v[4];
+                convert4<A>(ys + k * 16 * MU_COLS, n_src, dg->term, pt, q, v);
+#pragma unroll
+                for (int e = 0; e < 4; e++) x[k + e] = __dadd_rn(FpRow::value(v[e] + ((u64)FP_MAGIC_HI << 32)), -FP_MAGIC);
+            }
+            fwd_cols<MU_COLS>(r, x, sm, col, sub, bar);
+#pragma unroll
+            for (int k = 0; k < 16; k++) p[(16 * sub + k) * 256] = FpRow::bits(x[k]);
+        } else {
+            IntRow r{tw + (size_t)pt * N16, q, 2 * q};
+            u64 x[16];
+#pragma unroll
+            for (int k = 0; k < 16; k += 4) {
+                convert4<A>(ys + k * 16 * MU_COLS, n_src, dg->term, pt, q, x + k);
+#pragma unroll
+                for (int e = 0; e < 4; e++) x[k + e] += r.q2;      // |v| <= 1.25 q: below 4q
+            }
+            fwd_cols<MU_COLS>(r, x, sm, col, sub, bar);
+#pragma unroll
+            for (int k = 0; k < 16; k++) p[(16 * sub + k) * 256] = x[k];
+        }
+    }
+}
+
+bool modup16_supported(const fesc_ctx* ctx, uint32_t level) {
+    if (ctx->log_n != 16 || ctx->alpha > 4 || ctx->n_p > 4) return false;
+    for (uint32_t i = 0; i < level; i++)
+        if (ctx->q[i] >= FESC_FP_LIMIT) return false;
+    return true;
+}
+
+template <int A>
+static int launch(fesc_ctx* ctx, const u64* y, u64* ext, uint32_t level, uint32_t batch, cudaStream_t st) {
+    const uint32_t beta = (level + ctx->alpha - 1) / ctx->alpha, tiles = 256 / MU_COLS;
+    const size_t smem = ((size_t)A * MU_SRC + MU_GROUPS * COL_SMEM(MU_COLS)) * sizeof(u64);
+    auto kern = k_modup_cols<A>;
+    FESC_CHECK_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    // two CTAs per SM: with few ciphertexts the targets of a tile are shared by up to four CTAs, so that the last wave is full
+    uint32_t splits = 1;
+    while (splits < 4 && tiles * beta * batch * splits < 8 * 148) splits++;
+    kern<<<dim3(tiles * splits, beta, batch), MU_THREADS, smem, st>>>(y, ext, ctx->tabs.d_modup + (size_t)(level - 1) * ctx->beta_max,
+                                                                     ctx->d_twf, ctx->d_tw, ctx->d_pc, level, ctx->n_q, ctx->n_p, beta, splits);
+    return FESC_OK;
+}
+int modup16_cols_launch(fesc_ctx* ctx, const u64* y, u64* ext, uint32_t level, uint32_t batch, cudaStream_t st) {
+    if (ctx->alpha <= 1) return launch<1>(ctx, y, ext, level, batch, st);
+    if (ctx->alpha <= 2) return launch<2>(ctx, y, ext, level, batch, st);
+    return launch<4>(ctx, y, ext, level, batch, st);
+}

@@ -84,9 +84,10 @@ __global__ void __launch_bounds__(256) ntt_small(u64* __restrict__ data, const u
 }
 
 int ntt_launch(fesc_ctx* ctx, u64* d_data, size_t rows, const RowMap& map, bool inverse, cudaStream_t st, bool in_double,
-               bool out_double, const NttFinish* finish) {
+               bool out_double, const NttFinish* finish, const InvScale* scale, bool skip_cols) {
     const NttFinish fin = finish ? *finish : NttFinish();
     if (fin.acc && (inverse || ctx->log_n != 16)) return fesc_fail(ctx, FESC_EINVAL, "ntt: the fused epilogue belongs to a forward N = 2^16 transform");
+    if ((scale || skip_cols) && ctx->log_n != 16) return fesc_fail(ctx, FESC_EINVAL, "ntt: N = 2^16 only");
     if (rows == 0) return FESC_OK;
     if (rows > 0x7fffffffu) return fesc_fail(ctx, FESC_EINVAL, "ntt: too many rows");
     const ulonglong2* tw = inverse ? ctx->d_itw : ctx->d_tw;
@@ -96,7 +97,7 @@ int ntt_launch(fesc_ctx* ctx, u64* d_data, size_t rows, const RowMap& map, bool 
     prof_begin(ctx, PF_NTT, st);
     uint64_t launches = 0;
     if (ctx->log_n == 16) {
-        const int rc = ntt16_launch(ctx, d_data, rows, map, inverse, st, in_double, out_double, fin, launches);
+        const int rc = ntt16_launch(ctx, d_data, rows, map, inverse, st, in_double, out_double, fin, launches, scale, skip_cols);
         if (rc != FESC_OK) return rc;
     } else {
         size_t smem = sizeof(u64) << ctx->log_n;

@@ -23,215 +23,6 @@
 #include "common.cuh"
 #include "ntt16.cuh"
 
-#define N16 65536u
-#ifndef NTT_COLS
-#define NTT_COLS 8                  // columns per CTA of ntt16_cols (x 16 threads)
-#endif
-#ifndef NTT_WARPS
-#define NTT_WARPS 4                 // warps per CTA of ntt16_rows
-#endif
-#define COL_THREADS (NTT_COLS * 16)
-#define COL_SMEM (256 * NTT_COLS + 16 * 8)
-#define ROW_THREADS (NTT_WARPS * 32)
-#define ROW_SMEM 576                // words per warp: 512 points, two words of padding after every 16
-
-__device__ __forceinline__ uint32_t pad16(uint32_t e) { return e + 2 * (e >> 4); }
-
-// ---------------------------------------------------------------------------------------
-// Arithmetic of a row.  w(i): twiddle i of the row's table.
-// FpRow: primes below 2^50, exact products on the FP64 pipe.  |product| <= (1/2 + 1.5 |y| 2^-53) q with centred twiddles,
-// so a forward stage takes a bound B q to (1.1875 B + 1/2) q: four stages from 2.8 q reach 8 q, seven from q/2 reach 7.88 q,
-// and everything below 8 q < 2^53 is exact.  Forward rows are folded back to q/2 twice (after four and after eleven
-// stages; the first bound leaves room for a conversion's lazy sum at the input); an inverse stage doubles the bound, so four stages from q/2 end at 8 q and every inverse
-// round folds back.
-// IntRow: any prime below 2^62, lazy Shoup butterflies, values below 4q (forward) or 2q (inverse).
-// ---------------------------------------------------------------------------------------
-struct FpRow {
-    typedef double T;
-    const double* __restrict__ tw;
-    double q, qinv;
-    __device__ __forceinline__ void ct(T& x, T& y, double w) const {
-        const double v = fp_modmul(y, w, q, qinv), u = x;
-        x = u + v;
-        y = u - v;
-    }
-    __device__ __forceinline__ void gs(T& x, T& y, double w) const {
-        const double u = x, v = y;
-        x = u + v;
-        y = fp_modmul(u - v, w, q, qinv);
-    }
-    template <int S>
-    __device__ __forceinline__ void load(double (&w)[8], uint32_t i) const {      // 2^S twiddles from i on
-        if (S == 0) {
-            w[0] = __ldg(tw + i);
-        } else {
-#pragma unroll
-            for (int k = 0; k < (1 << S) / 2; k++) {
-                const double2 v = __ldg(reinterpret_cast<const double2*>(tw + i) + k);
-                w[2 * k] = v.x, w[2 * k + 1] = v.y;
-            }
-        }
-    }
-    typedef double W;
-    __device__ __forceinline__ T fold(T x) const { return fp_reduce(x, q, qinv); }
-    static __device__ __forceinline__ u64 bits(T x) { return (u64)__double_as_longlong(x); }
-    static __device__ __forceinline__ T value(u64 b) { return __longlong_as_double((long long)b); }
-};
-struct IntRow {
-    typedef u64 T;
-    typedef ulonglong2 W;
-    const ulonglong2* __restrict__ tw;
-    u64 q, q2;
-    __device__ __forceinline__ void ct(T& x, T& y, const W& w) const {
-        const u64 u = csub(x, q2), v = shoup_lazy(y, w.x, w.y, q);
-        x = u + v;
-        y = u - v + q2;
-    }
-    __device__ __forceinline__ void gs(T& x, T& y, const W& w) const {
-        const u64 u = x, v = y;
-        x = csub(u + v, q2);
-        y = shoup_lazy(u - v + q2, w.x, w.y, q);
-    }
-    template <int S>
-    __device__ __forceinline__ void load(W (&w)[8], uint32_t i) const {
-#pragma unroll
-        for (int k = 0; k < (1 << S); k++) w[k] = __ldg(tw + i + k);
-    }
-    __device__ __forceinline__ T fold(T x) const { return x; }
-    static __device__ __forceinline__ u64 bits(T x) { return x; }
-    static __device__ __forceinline__ T value(u64 b) { return b; }
-};
-
-// Stage S (0..3) of a forward round: distance 8 >> S, twiddles (i0 << S) + j for the j-th group of 16 >> S registers.
-template <int S, class R>
-__device__ __forceinline__ void fwd_stage(const R& r, typename R::T (&x)[16], uint32_t i0) {
-    typename R::W w[8];
-    r.template load<S>(w, i0 << S);
-    constexpr int d = 8 >> S;
-#pragma unroll
-    for (int k = 0; k < 8; k++) {
-        const int i = (k / d) * 2 * d + k % d;
-        r.ct(x[i], x[i + d], w[k / d]);
-    }
-}
-template <int S, class R>
-__device__ __forceinline__ void inv_stage(const R& r, typename R::T (&x)[16], uint32_t i0) {
-    typename R::W w[8];
-    r.template load<S>(w, i0 << S);
-    constexpr int d = 8 >> S;
-#pragma unroll
-    for (int k = 0; k < 8; k++) {
-        const int i = (k / d) * 2 * d + k % d;
-        r.gs(x[i], x[i + d], w[k / d]);
-    }
-}
-template <class R>
-__device__ __forceinline__ void fold16(const R& r, typename R::T (&x)[16]) {
-#pragma unroll
-    for (int k = 0; k < 16; k++) x[k] = r.fold(x[k]);
-}
-
-// position of (hi, col) in the exchange buffer of ntt16_cols: a row of 16 hi values is shifted by 8 words, so that both
-// sides of the exchange are free of bank conflicts
-__device__ __forceinline__ uint32_t col_slot(uint32_t hi, uint32_t col) { return hi * NTT_COLS + (hi >> 4) * 8 + col; }
-
-// Rounds A and B on the registers of one thread (column, sub = 0..15).
-template <class R>
-__device__ __forceinline__ void fwd_cols(const R& r, typename R::T (&x)[16], u64* sm, uint32_t col, uint32_t sub) {
-    fwd_stage<0>(r, x, 1);
-    fwd_stage<1>(r, x, 1);
-    fwd_stage<2>(r, x, 1);
-    fwd_stage<3>(r, x, 1);
-    fold16(r, x);
-#pragma unroll
-    for (int k = 0; k < 16; k++) sm[col_slot(16 * k, col) + sub * NTT_COLS] = R::bits(x[k]);
-    __syncthreads();
-    const u64* s = sm + col_slot(16 * sub, col);
-#pragma unroll
-    for (int k = 0; k < 16; k++) x[k] = R::value(s[k * NTT_COLS]);
-    const uint32_t i0 = 16 + sub;
-    fwd_stage<0>(r, x, i0);
-    fwd_stage<1>(r, x, i0);
-    fwd_stage<2>(r, x, i0);
-    fwd_stage<3>(r, x, i0);
-}
-// Rounds B and A without the last stage.
-template <class R>
-__device__ __forceinline__ void inv_cols(const R& r, typename R::T (&x)[16], u64* sm, uint32_t col, uint32_t sub) {
-    const uint32_t i0 = 16 + sub;
-    inv_stage<3>(r, x, i0);
-    inv_stage<2>(r, x, i0);
-    inv_stage<1>(r, x, i0);
-    inv_stage<0>(r, x, i0);
-    fold16(r, x);
-    u64* s = sm + col_slot(16 * sub, col);
-#pragma unroll
-    for (int k = 0; k < 16; k++) s[k * NTT_COLS] = R::bits(x[k]);
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < 16; k++) x[k] = R::value(sm[col_slot(16 * k, col) + sub * NTT_COLS]);
-    inv_stage<3>(r, x, 1);
-    inv_stage<2>(r, x, 1);
-    inv_stage<1>(r, x, 1);
-}
-// Rounds C and D of one warp's 512 points (blk = index of the 512-point block in the row).  x holds round C's points on
-// entry; on return the warp's padded buffer holds the transformed points, unreduced.
-template <class R>
-__device__ __forceinline__ void fwd_rows(const R& r, typename R::T (&x)[16], u64* sm, uint32_t blk, uint32_t lane) {
-    const uint32_t i1 = 256 + 2 * blk + (lane >> 4);
-    fwd_stage<0>(r, x, i1);
-    fwd_stage<1>(r, x, i1);
-    fwd_stage<2>(r, x, i1);
-    fold16(r, x);
-    fwd_stage<3>(r, x, i1);
-    u64* c = sm + 288 * (lane >> 4) + (lane & 15);
-#pragma unroll
-    for (int k = 0; k < 16; k++) c[18 * k] = R::bits(x[k]);
-    __syncwarp();
-    ulonglong2* d = reinterpret_cast<ulonglong2*>(sm + 18 * lane);
-#pragma unroll
-    for (int k = 0; k < 8; k++) {
-        const ulonglong2 v = d[k];
-        x[2 * k] = R::value(v.x), x[2 * k + 1] = R::value(v.y);
-    }
-    const uint32_t i2 = 4096 + 32 * blk + lane;
-    fwd_stage<0>(r, x, i2);
-    fwd_stage<1>(r, x, i2);
-    fwd_stage<2>(r, x, i2);
-    fwd_stage<3>(r, x, i2);
-#pragma unroll
-    for (int k = 0; k < 8; k++) d[k] = make_ulonglong2(R::bits(x[2 * k]), R::bits(x[2 * k + 1]));
-    __syncwarp();
-}
-// Rounds D and C: the warp's padded buffer holds the points on entry, x round C's points on return.
-template <class R>
-__device__ __forceinline__ void inv_rows(const R& r, typename R::T (&x)[16], u64* sm, uint32_t blk, uint32_t lane) {
-    ulonglong2* d = reinterpret_cast<ulonglong2*>(sm + 18 * lane);
-#pragma unroll
-    for (int k = 0; k < 8; k++) {
-        const ulonglong2 v = d[k];
-        x[2 * k] = R::value(v.x), x[2 * k + 1] = R::value(v.y);
-    }
-    const uint32_t i2 = 4096 + 32 * blk + lane;
-    inv_stage<3>(r, x, i2);
-    inv_stage<2>(r, x, i2);
-    inv_stage<1>(r, x, i2);
-    inv_stage<0>(r, x, i2);
-    fold16(r, x);
-#pragma unroll
-    for (int k = 0; k < 8; k++) d[k] = make_ulonglong2(R::bits(x[2 * k]), R::bits(x[2 * k + 1]));
-    __syncwarp();
-    const u64* c = sm + 288 * (lane >> 4) + (lane & 15);
-#pragma unroll
-    for (int k = 0; k < 16; k++) x[k] = R::value(c[18 * k]);
-    const uint32_t i1 = 256 + 2 * blk + (lane >> 4);
-    inv_stage<3>(r, x, i1);
-    inv_stage<2>(r, x, i1);
-    inv_stage<1>(r, x, i1);
-    inv_stage<0>(r, x, i1);
-    fold16(r, x);
-}
-
 __device__ __forceinline__ uint32_t list_row(const RowList& list, uint32_t y, uint32_t& prime) {
     const uint32_t rep = y / list.count, e = y - rep * list.count;
     prime = list.prime[e];
@@ -243,7 +34,7 @@ template <bool FP>
 __global__ void __launch_bounds__(COL_THREADS, 1024 / COL_THREADS)
     ntt16_cols_fwd(u64* __restrict__ data, const void* __restrict__ tw, const PrimeConst* __restrict__ pcs, RowList list,
                    uint32_t y0, int in_double) {
-    __shared__ u64 sm[COL_SMEM];
+    __shared__ u64 sm[COL_SMEM(NTT_COLS)];
     uint32_t pi;
     const uint32_t row = list_row(list, y0 + blockIdx.y, pi);
     const uint32_t col = threadIdx.x % NTT_COLS, sub = threadIdx.x / NTT_COLS;
@@ -257,7 +48,7 @@ __global__ void __launch_bounds__(COL_THREADS, 1024 / COL_THREADS)
             const u64 v = p[(16 * k + sub) * 256];
             x[k] = in_double ? FpRow::value(v) : fp_from_u64(v);
         }
-        fwd_cols(r, x, sm, col, sub);
+        fwd_cols<NTT_COLS>(r, x, sm, col, sub, CtaBarrier());
 #pragma unroll
         for (int k = 0; k < 16; k++) p[(16 * sub + k) * 256] = FpRow::bits(x[k]);      // doubles below 3.7q
     } else {
@@ -266,7 +57,7 @@ __global__ void __launch_bounds__(COL_THREADS, 1024 / COL_THREADS)
         u64 x[16];
 #pragma unroll
         for (int k = 0; k < 16; k++) x[k] = p[(16 * k + sub) * 256];
-        fwd_cols(r, x, sm, col, sub);
+        fwd_cols<NTT_COLS>(r, x, sm, col, sub, CtaBarrier());
 #pragma unroll
         for (int k = 0; k < 16; k++) p[(16 * sub + k) * 256] = x[k];                   // below 4q
     }
@@ -274,8 +65,9 @@ __global__ void __launch_bounds__(COL_THREADS, 1024 / COL_THREADS)
 
 template <bool FP>
 __global__ void __launch_bounds__(COL_THREADS, 1024 / COL_THREADS)
-    ntt16_cols_inv(u64* __restrict__ data, const void* __restrict__ tw, const PrimeConst* __restrict__ pcs, RowList list, uint32_t y0) {
-    __shared__ u64 sm[COL_SMEM];
+    ntt16_cols_inv(u64* __restrict__ data, const void* __restrict__ tw, const PrimeConst* __restrict__ pcs, RowList list, uint32_t y0,
+                   const InvScale* __restrict__ scale) {
+    __shared__ u64 sm[COL_SMEM(NTT_COLS)];
     uint32_t pi;
     const uint32_t row = list_row(list, y0 + blockIdx.y, pi);
     const uint32_t col = threadIdx.x % NTT_COLS, sub = threadIdx.x / NTT_COLS;
@@ -287,8 +79,8 @@ __global__ void __launch_bounds__(COL_THREADS, 1024 / COL_THREADS)
         double x[16];
 #pragma unroll
         for (int k = 0; k < 16; k++) x[k] = FpRow::value(p[(16 * sub + k) * 256]);
-        inv_cols(r, x, sm, col, sub);
-        const double ninv = pc.ninvd, ninvw = pc.ninvwd;
+        inv_cols<NTT_COLS>(r, x, sm, col, sub);
+        const double ninv = scale ? scale[pi].nd : pc.ninvd, ninvw = scale ? scale[pi].wd : pc.ninvwd;
 #pragma unroll
         for (int k = 0; k < 8; k++) {        // last stage, N^-1 folded in
             const double u = x[k], v = x[k + 8];
@@ -301,8 +93,9 @@ __global__ void __launch_bounds__(COL_THREADS, 1024 / COL_THREADS)
         u64 x[16];
 #pragma unroll
         for (int k = 0; k < 16; k++) x[k] = p[(16 * sub + k) * 256];
-        inv_cols(r, x, sm, col, sub);
-        const u64 n = pc.ninv, ns = pc.ninvs, nw = pc.ninvw, nws = pc.ninvws;
+        inv_cols<NTT_COLS>(r, x, sm, col, sub);
+        const u64 n = scale ? scale[pi].n : pc.ninv, ns = scale ? scale[pi].ns : pc.ninvs;
+        const u64 nw = scale ? scale[pi].w : pc.ninvw, nws = scale ? scale[pi].ws : pc.ninvws;
 #pragma unroll
         for (int k = 0; k < 8; k++) {
             const u64 u = x[k], v = x[k + 8];
@@ -427,7 +220,7 @@ __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
 }
 
 int ntt16_launch(fesc_ctx* ctx, u64* data, size_t rows, const RowMap& map, bool inverse, cudaStream_t st, bool in_double,
-                 bool out_double, const NttFinish& fin, uint64_t& launches) {
+                 bool out_double, const NttFinish& fin, uint64_t& launches, const InvScale* scale, bool skip_cols) {
     RowList kind[2];                  // 0: primes below 2^50, 1: the rest
     for (RowList& l : kind) l.period = map.period, l.count = 0;
     for (uint32_t i = 0; i < map.period; i++) {
@@ -445,20 +238,20 @@ int ntt16_launch(fesc_ctx* ctx, u64* data, size_t rows, const RowMap& map, bool 
             const dim3 gc(256 / NTT_COLS, n), gr(128 / NTT_WARPS, n);
             const uint32_t y = (uint32_t)y0;
             if (f == 0 && !inverse) {
-                ntt16_cols_fwd<true><<<gc, COL_THREADS, 0, st>>>(data, ctx->d_twf, ctx->d_pc, l, y, in_double);
+                if (!skip_cols) ntt16_cols_fwd<true><<<gc, COL_THREADS, 0, st>>>(data, ctx->d_twf, ctx->d_pc, l, y, in_double);
                 if (fin.acc) ntt16_rows_fwd<true, true><<<gr, ROW_THREADS, 0, st>>>(data, ctx->d_twf, ctx->d_pc, l, y, out_double, fin);
                 else ntt16_rows_fwd<true, false><<<gr, ROW_THREADS, 0, st>>>(data, ctx->d_twf, ctx->d_pc, l, y, out_double, fin);
             } else if (f == 0) {
                 ntt16_rows_inv<true><<<gr, ROW_THREADS, 0, st>>>(data, ctx->d_itwf, ctx->d_pc, l, y);
-                ntt16_cols_inv<true><<<gc, COL_THREADS, 0, st>>>(data, ctx->d_itwf, ctx->d_pc, l, y);
+                ntt16_cols_inv<true><<<gc, COL_THREADS, 0, st>>>(data, ctx->d_itwf, ctx->d_pc, l, y, scale);
             } else if (!inverse) {
-                ntt16_cols_fwd<false><<<gc, COL_THREADS, 0, st>>>(data, ctx->d_tw, ctx->d_pc, l, y, 0);
+                if (!skip_cols) ntt16_cols_fwd<false><<<gc, COL_THREADS, 0, st>>>(data, ctx->d_tw, ctx->d_pc, l, y, 0);
                 ntt16_rows_fwd<false, false><<<gr, ROW_THREADS, 0, st>>>(data, ctx->d_tw, ctx->d_pc, l, y, 0, fin);
             } else {
                 ntt16_rows_inv<false><<<gr, ROW_THREADS, 0, st>>>(data, ctx->d_itw, ctx->d_pc, l, y);
-                ntt16_cols_inv<false><<<gc, COL_THREADS, 0, st>>>(data, ctx->d_itw, ctx->d_pc, l, y);
+                ntt16_cols_inv<false><<<gc, COL_THREADS, 0, st>>>(data, ctx->d_itw, ctx->d_pc, l, y, scale);
             }
-            launches += 2;
+            launches += skip_cols ? 1 : 2;
         }
     }
     return FESC_OK;

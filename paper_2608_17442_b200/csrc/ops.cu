@@ -731,8 +731,24 @@ static int ks_decompose(fesc_ctx* ctx, const KsScratch& ws, uint32_t level, uint
     // 1. d -> COEFF
     m.period = level;
     for (uint32_t i = 0; i < level; i++) m.prime[i] = (uint8_t)i;
-    if ((rc = ntt_launch(ctx, ws.dcoef, (size_t)batch * level, m, true, st)) != FESC_OK) return rc;
-    // 2. ModUp
+    const bool fused = modup16_supported(ctx, level);
+    if ((rc = ntt_launch(ctx, ws.dcoef, (size_t)batch * level, m, true, st, false, false, nullptr,
+                         fused ? ctx->tabs.d_up_scale + (size_t)(level - 1) * nq : nullptr)) != FESC_OK)
+        return rc;
+    // 2. ModUp, 3. NTT of the converted rows
+    if (beta * rows > sizeof(RowMap::prime)) return fesc_fail(ctx, FESC_EINVAL, "key switch: too many digit rows");
+    m.period = beta * rows;
+    for (uint32_t j = 0; j < beta; j++)
+        for (uint32_t t = 0; t < rows; t++) {
+            bool own = t < level && t / alpha == j;
+            m.prime[j * rows + t] = own ? 0xFF : (uint8_t)(t < level ? t : nq + (t - level));
+        }
+    if (fused) {      // the conversion feeds the transform's first pass
+        prof_begin(ctx, PF_MODUP, st);
+        if ((rc = modup16_cols_launch(ctx, ws.dcoef, ws.ext, level, batch, st)) != FESC_OK) return rc;
+        prof_end(ctx, PF_MODUP, st);
+        return ntt_launch(ctx, ws.ext, (size_t)batch * beta * rows, m, false, st, false, true, nullptr, nullptr, true);
+    }
     const ModUpDigit* tab = ctx->tabs.d_modup + (size_t)(level - 1) * ctx->beta_max;
     const int dbl = ctx->log_n == 16;   // the N = 2^16 forward transform takes doubles straight from the conversion
     const bool vec2 = N % (256 * KS_VEC) == 0;
@@ -750,14 +766,6 @@ static int ks_decompose(fesc_ctx* ctx, const KsScratch& ws, uint32_t level, uint
     else MODUP(8);
 #undef MODUP
     prof_end(ctx, PF_MODUP, st);
-    // 3. NTT of the converted rows
-    if (beta * rows > sizeof(RowMap::prime)) return fesc_fail(ctx, FESC_EINVAL, "key switch: too many digit rows");
-    m.period = beta * rows;
-    for (uint32_t j = 0; j < beta; j++)
-        for (uint32_t t = 0; t < rows; t++) {
-            bool own = t < level && t / alpha == j;
-            m.prime[j * rows + t] = own ? 0xFF : (uint8_t)(t < level ? t : nq + (t - level));
-        }
     if ((rc = ntt_launch(ctx, ws.ext, (size_t)batch * beta * rows, m, false, st, dbl != 0, dbl != 0)) != FESC_OK) return rc;
     FESC_CHECK_CUDA(ctx, cudaGetLastError());
     return FESC_OK;

@@ -102,6 +102,11 @@ __device__ __forceinline__ u64 imma_recombine(const int (&d)[4][7][4], int sel, 
 bool bconv_supported(const fesc_ctx* ctx, uint32_t level);
 void moddown_conv_imma_launch(fesc_ctx* ctx, const u64* acc, u64* u, uint32_t level, uint32_t batch, int out_double, cudaStream_t st);
 
+// ModUp fused with the first eight stages of the forward transform (N = 2^16, modup16.cu): y = the COEFF rows times
+// (Q_j/q_a)^-1
+bool modup16_supported(const fesc_ctx* ctx, uint32_t level);
+int modup16_cols_launch(fesc_ctx* ctx, const u64* y, u64* ext, uint32_t level, uint32_t batch, cudaStream_t st);
+
 // packed-operand BSGS accumulate (packed.cu)
 size_t bsgs_packed_bytes(uint32_t N, uint32_t level, uint32_t rows, uint32_t terms);
 bool bsgs_packed_supported(const fesc_ctx* ctx, uint32_t level, uint32_t terms, uint32_t dshift);
