@@ -231,6 +231,7 @@ struct RescaleTab {
 struct Tables {
     ModUpDigit* d_modup;      // [(level-1) * beta_max + digit], level = 1..n_q
     InvScale* d_up_scale;     // [(level-1) * n_q + limb]: factor (Q_j/q_limb)^-1 mod q_limb
+    InvScale* d_down_scale;   // [prime index]: factor (P/p_k)^-1 mod p_k (special primes)
     ModDownTab* d_moddown;
     RescaleTab* d_rescale;    // [level], level = 2..n_q (index 0,1 unused)
     u64* d_Pmod_all;          // P mod q_t for every prime index (0 on special primes)
@@ -357,6 +358,9 @@ static inline uint32_t ntt16_twiddle_slot(uint32_t i, bool pairs) {
 // N = 2^16 kernels (ntt16.cu)
 int ntt16_launch(fesc_ctx* ctx, u64* data, size_t rows, const RowMap& map, bool inverse, cudaStream_t st, bool in_double,
                  bool out_double, const NttFinish& fin, uint64_t& launches, const InvScale* scale, bool skip_cols);
+// N = 2^10 .. 2^12 (small.cu)
+bool small_ring(const fesc_ctx* ctx);
+int small_ntt_launch(fesc_ctx* ctx, u64* data, size_t rows, const RowMap& map, bool inverse, cudaStream_t st);
 // double with |x| <= q/2 as handed to the forward transform
 __device__ __forceinline__ u64 fp_handoff(double s, double q, double qinv) {
     return (u64)__double_as_longlong(fp_reduce(s, q, qinv));

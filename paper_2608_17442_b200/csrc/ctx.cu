@@ -393,6 +393,9 @@ static int build_tables(fesc_ctx* ctx) {
         md.pinvd[i] = (double)md.pinv[i];
     }
     if ((rc = upload(ctx, &ctx->tabs.d_moddown, mdv)) != FESC_OK) return rc;
+    std::vector<InvScale> ds(np, InvScale{});
+    for (uint32_t k = 0; k < K; k++) ds[nq + k] = inv_scale(ctx->pc[nq + k], md.inv[k]);
+    if ((rc = upload(ctx, &ctx->tabs.d_down_scale, ds)) != FESC_OK) return rc;
     if (K <= 4) {
         std::vector<uint4> df(512);
         bconv_fragments(df.data(), [&](uint32_t row, uint32_t k, uint32_t b) -> u64 {
@@ -422,6 +425,7 @@ static int build_tables(fesc_ctx* ctx) {
 static void free_tables(fesc_ctx* ctx) {
     dev_free(ctx->tabs.d_modup);
     dev_free(ctx->tabs.d_up_scale);
+    dev_free(ctx->tabs.d_down_scale);
     dev_free(ctx->tabs.d_moddown);
     dev_free(ctx->tabs.d_rescale);
     dev_free(ctx->tabs.d_Pmod_all);

@@ -1,5 +1,5 @@
-// Negacyclic NTT / inverse NTT over RNS limbs for sm_100a: rings N <= 2^12 and the entry point of both ring sizes
-// (N = 2^16 lives in ntt16.cu).
+// Negacyclic NTT / inverse NTT over RNS limbs for sm_100a: rings N <= 2^9 and the entry point of all ring sizes
+// (N = 2^16 lives in ntt16.cu, N = 2^10 .. 2^12 in small.cu).
 //
 // Forward: Cooley-Tukey butterflies with psi merged into the twiddles (natural order in, bit-reversed evaluation order
 // out); inverse: Gentleman-Sande with the inverse twiddles and N^-1 folded into the last stage.
@@ -28,7 +28,7 @@ __device__ __forceinline__ void gs_bfly(u64& x, u64& y, const Tw& t, u64 q, u64 
 }
 
 // ---------------------------------------------------------------------------------------
-// N <= 2^12: one CTA per row, radix-2 stages in shared memory.
+// N <= 2^9: one CTA per row, radix-2 stages in shared memory.
 // ---------------------------------------------------------------------------------------
 template <bool INV>
 __global__ void __launch_bounds__(256) ntt_small(u64* __restrict__ data, const ulonglong2* __restrict__ tw_all,
@@ -99,6 +99,10 @@ int ntt_launch(fesc_ctx* ctx, u64* d_data, size_t rows, const RowMap& map, bool 
     if (ctx->log_n == 16) {
         const int rc = ntt16_launch(ctx, d_data, rows, map, inverse, st, in_double, out_double, fin, launches, scale, skip_cols);
         if (rc != FESC_OK) return rc;
+    } else if (small_ring(ctx)) {
+        const int rc = small_ntt_launch(ctx, d_data, rows, map, inverse, st);
+        if (rc != FESC_OK) return rc;
+        launches = 1;
     } else {
         size_t smem = sizeof(u64) << ctx->log_n;
         if (!inverse)

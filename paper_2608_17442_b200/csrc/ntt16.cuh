@@ -73,6 +73,7 @@ struct FpRow {
             }
         }
     }
+    __device__ __forceinline__ void one(double& w, uint32_t i) const { w = __ldg(tw + i); }
     typedef double W;
     __device__ __forceinline__ T fold(T x) const { return fp_reduce(x, q, qinv); }
     static __device__ __forceinline__ u64 bits(T x) { return (u64)__double_as_longlong(x); }
@@ -104,6 +105,7 @@ struct IntRow {
 #pragma unroll
         for (int k = 0; k < (1 << S); k++) w[k] = __ldg(t + 32 * ((1 << S) - 1 + k));
     }
+    __device__ __forceinline__ void one(W& w, uint32_t i) const { w = __ldg(tw + i); }
     __device__ __forceinline__ T fold(T x) const { return x; }
     static __device__ __forceinline__ u64 bits(T x) { return x; }
     static __device__ __forceinline__ T value(u64 b) { return b; }
@@ -167,6 +169,12 @@ __device__ __forceinline__ void fold16(const R& r, typename R::T (&x)[16]) {
 template <int COLS>
 __device__ __forceinline__ uint32_t col_slot(uint32_t hi, uint32_t col) { return hi * COLS + (hi >> 4) * COLS + col; }
 
+// all a transform needs of a context
+struct SmallTables {
+    const double *twf, *itwf;
+    const ulonglong2 *tw, *itw;
+    const PrimeConst* pc;
+};
 struct CtaBarrier {
     __device__ __forceinline__ void operator()() const { __syncthreads(); }
 };

@@ -231,20 +231,6 @@ __global__ void __launch_bounds__(256) k_modup(const u64* __restrict__ dcoef, u6
 #ifndef INNER_MINB
 #define INNER_MINB 4
 #endif
-// Several sources can be summed in one pass: source s contributes sum_j dt_j(ext_s)[pi_{g_s}(t)] * key_s[j].  The giant
-// steps of a projection (different converted polynomials, different keys, one sum) and the rotate-and-add chains (one
-// converted polynomial read through several Galois permutations, one key each) then read and write the accumulators
-// once instead of once per key, and the later reads of a shared source hit L2.
-#define INNER_MAX_SRC 8
-struct InnerSrc {
-    const u64* ext;   // [batch][beta][level+K][N]
-    const u64* key;   // [beta][2][n_q+K][N]
-    u64 g;            // Galois element the digits are read through (0: none)
-};
-struct InnerSrcs {
-    InnerSrc s[INNER_MAX_SRC];
-    uint32_t n;
-};
 // PATH 0: the row's prime decides at run time; 1: the caller guarantees primes below 2^50 on rows
 // [row0, row0 + gridDim.y) (exact FP64 products only); 2: the caller sends those rows to the 128-bit integer sums.
 template <int BT, int PATH>
@@ -728,6 +714,7 @@ static int ks_decompose(fesc_ctx* ctx, const KsScratch& ws, uint32_t level, uint
     const uint32_t gx = (N + 255) / 256;
     int rc;
     RowMap m;
+    if (small_ring(ctx)) return small_decompose(ctx, ws, ws.dcoef, (size_t)level * N, false, 0, level, batch, st);
     // 1. d -> COEFF
     m.period = level;
     for (uint32_t i = 0; i < level; i++) m.prime[i] = (uint8_t)i;
@@ -772,9 +759,10 @@ static int ks_decompose(fesc_ctx* ctx, const KsScratch& ws, uint32_t level, uint
 }
 
 // Step 4: inner products of the sources `S` (converted digits, key, Galois element each) summed into ws.acc;
-// accumulate != 0 adds to what ws.acc holds (sums over several passes before one division by P).
+// accumulate != 0 adds to what ws.acc holds (sums over several passes before one division by P); last: no further pass follows.
 static int ks_inner_multi(fesc_ctx* ctx, const KsScratch& ws, const InnerSrcs& S, uint32_t level, uint32_t batch,
-                          cudaStream_t st, int accumulate) {
+                          cudaStream_t st, int accumulate, int last = 1) {
+    if (small_ring(ctx)) return small_inner(ctx, ws, S, level, batch, st, accumulate, last);
     const uint32_t N = ctx->N, K = ctx->n_p, nq = ctx->n_q, alpha = ctx->alpha;
     const uint32_t beta = (level + alpha - 1) / alpha, rows = level + K;
     const uint32_t gx = (N + 255) / 256;
@@ -826,8 +814,9 @@ static int ks_inner(fesc_ctx* ctx, const KsScratch& ws, const EvalKey& key, uint
 }
 
 // Step 5: division of ws.acc by P; the result is ADDED to out[b][p] when bit p of add_mask is set, else stored.
-// whether the last pass of the forward transform finishes the division (N = 2^16, every data prime below 2^50)
+// whether the last pass of the forward transform finishes the division (N = 2^16 with every data prime below 2^50, small rings)
 static bool moddown_fused(const fesc_ctx* ctx, uint32_t level) {
+    if (small_ring(ctx)) return true;
     bool fuse = ctx->log_n == 16;
     for (uint32_t i = 0; i < level; i++) fuse = fuse && ctx->q[i] < FESC_FP_LIMIT;
     return fuse;
@@ -836,6 +825,7 @@ static bool moddown_fused(const fesc_ctx* ctx, uint32_t level) {
 // rot_src + b * rot_stride, read through the permutation by the fused epilogue
 static int ks_moddown(fesc_ctx* ctx, const KsScratch& ws, uint32_t level, uint32_t batch, u64* out, size_t out_stride,
                       int add_mask, cudaStream_t st, const u64* rot_src = nullptr, size_t rot_stride = 0, u64 rot_g = 0) {
+    if (small_ring(ctx)) return small_moddown(ctx, ws, level, batch, out, out_stride, add_mask, st, rot_src, rot_stride, rot_g);
     const uint32_t N = ctx->N, K = ctx->n_p, nq = ctx->n_q;
     const uint32_t rows = level + K;
     const uint32_t gx = (N + 255) / 256;
@@ -889,8 +879,23 @@ static int key_switch_chunk(fesc_ctx* ctx, const KsScratch& ws, const EvalKey& k
     return ks_apply(ctx, ws, key, level, batch, out, out_stride, add_mask, st, 0);
 }
 
+
 static OwnRows own_rows(const fesc_ctx* ctx, const KsScratch& ws, uint32_t level) {
     return OwnRows{ws.ext, ctx->alpha, (level + ctx->alpha - 1) / ctx->alpha, level + ctx->n_p, ctx->log_n == 16};
+}
+__global__ void k_hoist_prepare(const u64* in, size_t in_stride, u64* out0, size_t out_stride, OwnRows d, u64* dcoef, uint32_t log_n, uint32_t level,
+                                u64 g, const PrimeConst* pcs);
+// Steps 1-3 for the second polynomial of every ciphertext at `in`, read through the permutation of g (0: none)
+static int ks_start(fesc_ctx* ctx, const KsScratch& ws, const u64* in, size_t in_stride, u64 g, uint32_t level, uint32_t batch, cudaStream_t st) {
+    if (small_ring(ctx)) return small_decompose(ctx, ws, in + (size_t)level * ctx->N, in_stride, true, g, level, batch, st);
+    const dim3 grid((ctx->N + 255) / 256, level, batch);
+    prof_begin(ctx, PF_AUTOM, st);
+    if (g)
+        k_autom_ct<<<grid, 256, 0, st>>>(in, in_stride, nullptr, 0, own_rows(ctx, ws, level), ws.dcoef, ctx->log_n, level, g, ctx->d_pc, 0);
+    else
+        k_hoist_prepare<<<grid, 256, 0, st>>>(in, in_stride, nullptr, 0, own_rows(ctx, ws, level), ws.dcoef, ctx->log_n, level, 0, ctx->d_pc);
+    prof_end(ctx, PF_AUTOM, st);
+    return ks_decompose(ctx, ws, level, batch, st);
 }
 
 size_t ks_scratch_words(const fesc_ctx* ctx, uint32_t level, uint32_t chunk, uint32_t n_ext) {
@@ -927,21 +932,20 @@ int rotate_internal(fesc_ctx* ctx, const u64* in, size_t in_stride, u64* out, si
     KsScratch ws = ks_scratch_carve(ctx, scratch, level, chunk);
     for (uint32_t b0 = 0; b0 < batch; b0 += chunk) {
         uint32_t nb = batch - b0 < chunk ? batch - b0 : chunk;
-        dim3 g((ctx->N + 255) / 256, level, nb);
-        const bool fused = moddown_fused(ctx, level);   // then the division's epilogue adds sigma_g(c0) straight from the input
-        prof_begin(ctx, PF_AUTOM, st);
-        k_autom_ct<<<g, 256, 0, st>>>(in + (size_t)b0 * in_stride, in_stride, fused ? nullptr : out + (size_t)b0 * out_stride, out_stride,
-                                      own_rows(ctx, ws, level), ws.dcoef, ctx->log_n, level, it->second.g, ctx->d_pc, accumulate);
-        prof_end(ctx, PF_AUTOM, st);
+        const u64* ib = in + (size_t)b0 * in_stride;
+        u64* ob = out + (size_t)b0 * out_stride;
         int rc;
-        if (fused) {
-            if ((rc = ks_decompose(ctx, ws, level, nb, st)) != FESC_OK) return rc;
+        if (moddown_fused(ctx, level)) {                // the division's epilogue adds sigma_g(c0) straight from the input
+            if ((rc = ks_start(ctx, ws, ib, in_stride, it->second.g, level, nb, st)) != FESC_OK) return rc;
             if ((rc = ks_inner(ctx, ws, it->second, level, nb, st, 0, 0)) != FESC_OK) return rc;
-            rc = ks_moddown(ctx, ws, level, nb, out + (size_t)b0 * out_stride, out_stride, accumulate ? 3 : 0, st,
-                            in + (size_t)b0 * in_stride, in_stride, it->second.g);
+            rc = ks_moddown(ctx, ws, level, nb, ob, out_stride, accumulate ? 3 : 0, st, ib, in_stride, it->second.g);
         } else {
-            rc = key_switch_chunk(ctx, ws, it->second, level, nb, out + (size_t)b0 * out_stride, out_stride,
-                                  accumulate ? 3 : 1, st);
+            dim3 g((ctx->N + 255) / 256, level, nb);
+            prof_begin(ctx, PF_AUTOM, st);
+            k_autom_ct<<<g, 256, 0, st>>>(ib, in_stride, ob, out_stride, own_rows(ctx, ws, level), ws.dcoef, ctx->log_n, level, it->second.g,
+                                          ctx->d_pc, accumulate);
+            prof_end(ctx, PF_AUTOM, st);
+            rc = key_switch_chunk(ctx, ws, it->second, level, nb, ob, out_stride, accumulate ? 3 : 1, st);
         }
         if (rc != FESC_OK) return rc;
     }
@@ -1008,7 +1012,7 @@ int giant_sum_deferred_internal(fesc_ctx* ctx, u64* acc, uint32_t n_terms, size_
                 if (rc != FESC_OK) return rc;
                 S.s[s] = InnerSrc{wss.ext, key.d_key, 0};
             }
-            int rc = ks_inner_multi(ctx, ws, S, level, nb, st, p0 > 1);
+            int rc = ks_inner_multi(ctx, ws, S, level, nb, st, p0 > 1, p0 + np == n_terms);
             if (rc != FESC_OK) return rc;
         }
         int rc = ks_moddown(ctx, ws, level, nb, base, stride, 3, st);
@@ -1031,10 +1035,7 @@ int rotate_hoisted_internal(fesc_ctx* ctx, const u64* in, size_t in_stride, u64*
         const uint32_t nb = batch - b0 < chunk ? batch - b0 : chunk;
         dim3 g((ctx->N + 255) / 256, level, nb);
         const u64* ib = in + (size_t)b0 * in_stride;
-        prof_begin(ctx, PF_AUTOM, st);
-        k_hoist_prepare<<<g, 256, 0, st>>>(ib, in_stride, nullptr, 0, own_rows(ctx, ws, level), ws.dcoef, ctx->log_n, level, 0, ctx->d_pc);
-        prof_end(ctx, PF_AUTOM, st);
-        int rc = ks_decompose(ctx, ws, level, nb, st);
+        int rc = ks_start(ctx, ws, ib, in_stride, 0, level, nb, st);
         if (rc != FESC_OK) return rc;
         for (uint32_t k = 0; k < n_keys; k++) {
             const EvalKey& key = ctx->keys[key_ids[k]];
@@ -1100,10 +1101,9 @@ int rotate_sum_hoisted_internal(fesc_ctx* ctx, const u64* in, size_t in_stride, 
         const u64* ib = in + (size_t)b0 * in_stride;
         u64* ob = out + (size_t)b0 * out_stride;
         prof_begin(ctx, PF_AUTOM, st);
-        k_hoist_prepare<<<g, 256, 0, st>>>(ib, in_stride, nullptr, 0, own_rows(ctx, ws, level), ws.dcoef, ctx->log_n, level, 0, ctx->d_pc);
         k_rotsum_prepare<<<g, 256, 0, st>>>(ib, in_stride, ob, out_stride, ctx->log_n, level, gs, ctx->d_pc);
-        prof_end(ctx, PF_AUTOM, st, 2);
-        int rc = ks_decompose(ctx, ws, level, nb, st);
+        prof_end(ctx, PF_AUTOM, st);
+        int rc = ks_start(ctx, ws, ib, in_stride, 0, level, nb, st);
         if (rc != FESC_OK) return rc;
         InnerSrcs S;                                   // one converted polynomial, read through every key's permutation
         S.n = n_keys;
@@ -1212,6 +1212,10 @@ int rescale_internal(fesc_ctx* ctx, const u64* in, size_t in_stride, u64* out, u
         uint32_t nb = batch - b0 < 16384 ? batch - b0 : 16384;
         const u64* ib = in + (size_t)b0 * in_stride;
         u64* ob = out + (size_t)b0 * out_stride;
+        if (small_ring(ctx)) {
+            if ((rc = small_rescale(ctx, ib, in_stride, ob, out_stride, nb, level, scratch, st)) != FESC_OK) return rc;
+            continue;
+        }
         prof_begin(ctx, PF_RESCALE, st);
         k_take_last<<<dim3(gx, nb * 2), 256, 0, st>>>(ib, in_stride, scratch, N, level);
         prof_end(ctx, PF_RESCALE, st);

@@ -11,6 +11,21 @@
 struct KsScratch {
     u64 *dcoef, *ext, *acc, *u;
 };
+// Several sources can be summed in one pass: source s contributes sum_j dt_j(ext_s)[pi_{g_s}(t)] * key_s[j].  The giant
+// steps of a projection (different converted polynomials, different keys, one sum) and the rotate-and-add chains (one
+// converted polynomial read through several Galois permutations, one key each) then read and write the accumulators
+// once instead of once per key, and the later reads of a shared source hit L2.
+#define INNER_MAX_SRC 8
+struct InnerSrc {
+    const u64* ext;   // [batch][beta][level+K][N]
+    const u64* key;   // [beta][2][n_q+K][N]
+    u64 g;            // Galois element the digits are read through (0: none)
+};
+struct InnerSrcs {
+    InnerSrc s[INNER_MAX_SRC];
+    uint32_t n;
+};
+
 size_t ks_scratch_words(const fesc_ctx* ctx, uint32_t level, uint32_t chunk, uint32_t n_ext = 1);
 KsScratch ks_scratch_carve(const fesc_ctx* ctx, u64* base, uint32_t level, uint32_t chunk, uint32_t n_ext = 1);
 // converted polynomials a deferred giant-step sum of n_terms keeps side by side (one inner-product pass over them)
@@ -106,6 +121,16 @@ void moddown_conv_imma_launch(fesc_ctx* ctx, const u64* acc, u64* u, uint32_t le
 // (Q_j/q_a)^-1
 bool modup16_supported(const fesc_ctx* ctx, uint32_t level);
 int modup16_cols_launch(fesc_ctx* ctx, const u64* y, u64* ext, uint32_t level, uint32_t batch, cudaStream_t st);
+
+// rings N = 2^10 .. 2^12 (small.cu): the steps of a key switch and of a rescale, one row per CTA.  small_inner with `last` leaves the
+// special rows of acc in the form small_moddown takes.
+bool small_ring(const fesc_ctx* ctx);
+int small_decompose(fesc_ctx* ctx, const KsScratch& ws, const u64* src, size_t src_stride, bool keep_own, u64 g, uint32_t level, uint32_t batch,
+                    cudaStream_t st);
+int small_inner(fesc_ctx* ctx, const KsScratch& ws, const InnerSrcs& S, uint32_t level, uint32_t batch, cudaStream_t st, int accumulate, int last);
+int small_moddown(fesc_ctx* ctx, const KsScratch& ws, uint32_t level, uint32_t batch, u64* out, size_t out_stride, int add_mask, cudaStream_t st,
+                  const u64* rot_src, size_t rot_stride, u64 g);
+int small_rescale(fesc_ctx* ctx, const u64* in, size_t in_stride, u64* out, size_t out_stride, uint32_t batch, uint32_t level, u64* r, cudaStream_t st);
 
 // packed-operand BSGS accumulate (packed.cu)
 size_t bsgs_packed_bytes(uint32_t N, uint32_t level, uint32_t rows, uint32_t terms);

@@ -1,0 +1,538 @@
+// Rings N = 2^10 .. 2^12: transforms and whole key-switch steps of one row per CTA.
+//
+// A row (8 to 32 KB) fits one CTA: N/16 threads keep 16 points each and run the transform as register rounds of 4, 4 and
+// log N - 8 stages with two exchanges through shared memory.  At these sizes a call is a few hundred thousand products and
+// its time is launches and latencies, so every step around a transform is done by the CTA that holds the row:
+//   k_small_coef    [permutation of c1, copy of its own rows] + inverse transform (times a constant)
+//   k_small_modup   conversion of a digit to one target + forward transform
+//   k_small_inner   key inner product of one row [+ inverse transform of the rows on special primes]
+//   k_small_down    conversion of the special rows to one limb + forward transform + last step of the division [+ permuted c0]
+//   k_small_rescale conversion of the last limb + forward transform + last step of the division
+// A rotation takes 4 launches instead of 9, a rescale 2 instead of 5.
+#define FESC_DBG_FILE 13   // file id in the sites a debug build reports
+#include "ntt16.cuh"
+#include "ops.cuh"
+
+#define SM_PAD(e) ((e) + ((e) >> 4))
+
+// Forward: x[k] = point k N/16 + tid on entry; on return the padded buffer holds the transformed row, unreduced.
+template <int LOG, class R>
+__device__ __forceinline__ void small_fwd(const R& r, typename R::T (&x)[16], u64* sm) {
+    constexpr uint32_t N = 1u << LOG, T = N / 16, L = N / 256;
+    constexpr int S = LOG - 8;
+    const uint32_t tid = threadIdx.x, top = tid / L, low = tid % L;
+    fwd_stage<0>(r, x, 1);
+    fwd_stage<1>(r, x, 1);
+    fwd_stage<2>(r, x, 1);
+    fwd_stage<3>(r, x, 1);
+    fold16(r, x);
+#pragma unroll
+    for (int k = 0; k < 16; k++) sm[SM_PAD(k * T + tid)] = R::bits(x[k]);
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 16; k++) x[k] = R::value(sm[SM_PAD(top * T + k * L + low)]);
+    fwd_stage<0>(r, x, 16 + top);
+    fwd_stage<1>(r, x, 16 + top);
+    fwd_stage<2>(r, x, 16 + top);
+    fwd_stage<3>(r, x, 16 + top);
+    fold16(r, x);
+    // a thread writes the points it has read: no barrier needed before
+#pragma unroll
+    for (int k = 0; k < 16; k++) sm[SM_PAD(top * T + k * L + low)] = R::bits(x[k]);
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 16; k++) x[k] = R::value(sm[17 * tid + k]);
+#pragma unroll
+    for (int s = 0; s < S; s++) {
+        const int d = 1 << (S - 1 - s);
+#pragma unroll
+        for (int b = 0; b < 8 / d; b++) {
+            typename R::W w;
+            r.one(w, (256u << s) + ((16 * tid + 2 * d * b) >> (S - s)));
+#pragma unroll
+            for (int k = 0; k < d; k++) r.ct(x[2 * d * b + k], x[2 * d * b + k + d], w);
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < 16; k++) sm[17 * tid + k] = R::bits(x[k]);
+    __syncthreads();
+}
+// Inverse: the padded buffer holds the row on entry (and a barrier has passed); x[k] = point k N/16 + tid on return, the last
+// stage still to be done (pairs k, k + 8).
+template <int LOG, class R>
+__device__ __forceinline__ void small_inv(const R& r, typename R::T (&x)[16], u64* sm) {
+    constexpr uint32_t N = 1u << LOG, T = N / 16, L = N / 256;
+    constexpr int S = LOG - 8;
+    const uint32_t tid = threadIdx.x, top = tid / L, low = tid % L;
+#pragma unroll
+    for (int k = 0; k < 16; k++) x[k] = R::value(sm[17 * tid + k]);
+#pragma unroll
+    for (int s = S - 1; s >= 0; s--) {
+        const int d = 1 << (S - 1 - s);
+#pragma unroll
+        for (int b = 0; b < 8 / d; b++) {
+            typename R::W w;
+            r.one(w, (256u << s) + ((16 * tid + 2 * d * b) >> (S - s)));
+#pragma unroll
+            for (int k = 0; k < d; k++) r.gs(x[2 * d * b + k], x[2 * d * b + k + d], w);
+        }
+    }
+    fold16(r, x);
+#pragma unroll
+    for (int k = 0; k < 16; k++) sm[17 * tid + k] = R::bits(x[k]);
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 16; k++) x[k] = R::value(sm[SM_PAD(top * T + k * L + low)]);
+    inv_stage<3>(r, x, 16 + top);
+    inv_stage<2>(r, x, 16 + top);
+    inv_stage<1>(r, x, 16 + top);
+    inv_stage<0>(r, x, 16 + top);
+    fold16(r, x);
+#pragma unroll
+    for (int k = 0; k < 16; k++) sm[SM_PAD(top * T + k * L + low)] = R::bits(x[k]);
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 16; k++) x[k] = R::value(sm[SM_PAD(k * T + tid)]);
+    inv_stage<3>(r, x, 1);
+    inv_stage<2>(r, x, 1);
+    inv_stage<1>(r, x, 1);
+}
+// last inverse stage of an FP64 / integer row with the constants `s` (nullptr: the plain ones), canonical words to o
+template <int LOG>
+__device__ __forceinline__ void small_inv_store(const FpRow& r, double (&x)[16], const PrimeConst& pc, const InvScale* s, u64* o) {
+    constexpr uint32_t T = (1u << LOG) / 16;
+    const double n = s ? s->nd : pc.ninvd, w = s ? s->wd : pc.ninvwd;
+#pragma unroll
+    for (int k = 0; k < 8; k++) {
+        const double u = x[k], v = x[k + 8];
+        o[k * T + threadIdx.x] = fp_store(fp_modmul(u + v, n, r.q, r.qinv), r.q, r.qinv);
+        o[(k + 8) * T + threadIdx.x] = fp_store(fp_modmul(u - v, w, r.q, r.qinv), r.q, r.qinv);
+    }
+}
+template <int LOG>
+__device__ __forceinline__ void small_inv_store(const IntRow& r, u64 (&x)[16], const PrimeConst& pc, const InvScale* s, u64* o) {
+    constexpr uint32_t T = (1u << LOG) / 16;
+    const u64 n = s ? s->n : pc.ninv, ns = s ? s->ns : pc.ninvs, w = s ? s->w : pc.ninvw, ws = s ? s->ws : pc.ninvws;
+#pragma unroll
+    for (int k = 0; k < 8; k++) {
+        const u64 u = x[k], v = x[k + 8];
+        o[k * T + threadIdx.x] = shoup(u + v, n, ns, r.q);
+        o[(k + 8) * T + threadIdx.x] = shoup(u - v + r.q2, w, ws, r.q);
+    }
+}
+// inverse transform of the canonical row in the padded buffer (barrier passed) to o
+template <int LOG>
+__device__ __forceinline__ void small_inv_row(u64* sm, const SmallTables& tb, uint32_t pi, const InvScale* s, u64* o) {
+    const PrimeConst& pc = tb.pc[pi];
+    if (pc.q < FESC_FP_LIMIT) {
+        const FpRow r{tb.itwf + ((size_t)pi << LOG), pc.qd, pc.qinvd};
+#pragma unroll
+        for (int k = 0; k < 16; k++) sm[17 * threadIdx.x + k] = FpRow::bits(fp_load(sm[17 * threadIdx.x + k], r.q));
+        double x[16];
+        small_inv<LOG>(r, x, sm);
+        small_inv_store<LOG>(r, x, pc, s, o);
+    } else {
+        const IntRow r{tb.itw + ((size_t)pi << LOG), pc.q, 2 * pc.q};
+        u64 x[16];
+        small_inv<LOG>(r, x, sm);
+        small_inv_store<LOG>(r, x, pc, s, o);
+    }
+}
+
+// ---------------------------------------------------------------------------------------
+// plain transforms, one row per CTA (skipped rows launch nothing: RowList)
+// ---------------------------------------------------------------------------------------
+template <int LOG, bool INV>
+__global__ void __launch_bounds__(1 << (LOG - 4)) k_small_ntt(u64* __restrict__ data, SmallTables tb, RowList list) {
+    constexpr uint32_t N = 1u << LOG, T = N / 16;
+    __shared__ u64 sm[SM_PAD(N)];
+    const uint32_t rep = blockIdx.x / list.count, e = blockIdx.x - rep * list.count, pi = list.prime[e], tid = threadIdx.x;
+    u64* p = data + ((size_t)rep * list.period + list.row[e]) * N;
+    if (!DBG_REGION(p, N * sizeof(u64))) return;
+    if (INV) {
+#pragma unroll
+        for (int k = 0; k < 16; k++) sm[SM_PAD(k * T + tid)] = p[k * T + tid];
+        __syncthreads();
+        small_inv_row<LOG>(sm, tb, pi, nullptr, p);
+        return;
+    }
+    const PrimeConst& pc = tb.pc[pi];
+    if (pc.q < FESC_FP_LIMIT) {
+        const FpRow r{tb.twf + ((size_t)pi << LOG), pc.qd, pc.qinvd};
+        double x[16];
+#pragma unroll
+        for (int k = 0; k < 16; k++) x[k] = fp_from_u64(p[k * T + tid]);
+        small_fwd<LOG>(r, x, sm);
+#pragma unroll
+        for (int k = 0; k < 16; k++) p[k * T + tid] = fp_store(FpRow::value(sm[SM_PAD(k * T + tid)]), r.q, r.qinv);
+    } else {
+        const IntRow r{tb.tw + ((size_t)pi << LOG), pc.q, 2 * pc.q};
+        u64 x[16];
+#pragma unroll
+        for (int k = 0; k < 16; k++) x[k] = p[k * T + tid];
+        small_fwd<LOG>(r, x, sm);
+#pragma unroll
+        for (int k = 0; k < 16; k++) p[k * T + tid] = csub(csub(sm[SM_PAD(k * T + tid)], r.q2), r.q);
+    }
+}
+
+// ---------------------------------------------------------------------------------------
+// grid (level, batch): the polynomial to be switched, src[b] = [level][N] EVAL, read through the permutation of g (0: none), its own
+// rows kept in `own` (may be nullptr), COEFF rows times (Q_j/q)^-1 to dcoef.  src may be dcoef when g = 0.
+// ---------------------------------------------------------------------------------------
+template <int LOG>
+__global__ void __launch_bounds__(1 << (LOG - 4)) k_small_coef(const u64* src, size_t src_stride, u64* own, size_t own_stride, uint32_t own_rows,
+                                                               uint32_t alpha, u64* dcoef, SmallTables tb, const InvScale* __restrict__ scale,
+                                                               uint32_t level, u64 g) {
+    constexpr uint32_t N = 1u << LOG, T = N / 16;
+    __shared__ u64 sm[SM_PAD(N)];
+    const uint32_t l = blockIdx.x, b = blockIdx.y, tid = threadIdx.x;
+    const u64* in = src + (size_t)b * src_stride + (size_t)l * N;
+    u64* o = dcoef + ((size_t)b * level + l) * N;
+    u64* w = own ? own + (size_t)b * own_stride + ((size_t)(l / alpha) * own_rows + l) * N : nullptr;
+    if (!DBG_REGION(in, N * sizeof(u64)) || !DBG_REGION(o, N * sizeof(u64)) || (w && !DBG_REGION(w, N * sizeof(u64)))) return;
+#pragma unroll
+    for (int k = 0; k < 16; k++) {
+        const uint32_t t = k * T + tid;
+        const u64 v = in[g ? galois_src(t, LOG, g) : t];
+        sm[SM_PAD(t)] = v;
+        if (w) w[t] = v;
+    }
+    __syncthreads();
+    small_inv_row<LOG>(sm, tb, l, scale + l, o);
+}
+
+// grid (rows of all digits but the own ones, batch): ext[b][j][t] = NTT(sum_a y_a m_a)
+template <int LOG>
+__global__ void __launch_bounds__(1 << (LOG - 4)) k_small_modup(const u64* __restrict__ y, u64* __restrict__ ext, const ModUpDigit* __restrict__ tab,
+                                                                SmallTables tb, uint32_t level, uint32_t n_q, uint32_t K, uint32_t alpha, uint32_t beta) {
+    constexpr uint32_t N = 1u << LOG, T = N / 16;
+    __shared__ u64 sm[SM_PAD(N)];
+    const uint32_t rows = level + K, j = blockIdx.x / rows, t = blockIdx.x - j * rows, b = blockIdx.y, tid = threadIdx.x;
+    if (t < level && t / alpha == j) return;
+    const uint32_t pt = t < level ? t : n_q + (t - level);
+    const ModUpDigit* dg = tab + j;
+    const uint32_t n_src = dg->n_src;
+    const u64* src = y + ((size_t)b * level + dg->first) * N + tid;
+    u64* o = ext + (((size_t)b * beta + j) * rows + t) * N + tid;
+    if (!DBG_REGION(src - tid, (size_t)n_src * N * sizeof(u64)) || !DBG_REGION(o - tid, N * sizeof(u64))) return;
+    const PrimeConst& pc = tb.pc[pt];
+    bool fp = pc.q < FESC_FP_LIMIT;
+    for (uint32_t a = 0; a < n_src; a++) fp = fp && tb.pc[dg->first + a].q < FESC_FP_LIMIT;
+    if (fp) {
+        const FpRow r{tb.twf + ((size_t)pt << LOG), pc.qd, pc.qinvd};
+        double x[16];
+#pragma unroll
+        for (int k = 0; k < 16; k++) x[k] = 0.0;
+        for (uint32_t a = 0; a < n_src; a++) {         // every product below 0.875 q, folded back after the fourth
+            const double m = dg->matd[a][pt];
+#pragma unroll
+            for (int k = 0; k < 16; k++) x[k] += fp_modmul(fp_from_u64(src[(size_t)a * N + k * T]), m, r.q, r.qinv);
+            if (a % 3 == 2) fold16(r, x);
+        }
+        small_fwd<LOG>(r, x, sm);
+#pragma unroll
+        for (int k = 0; k < 16; k++) o[k * T] = fp_store(FpRow::value(sm[SM_PAD(k * T + tid)]), r.q, r.qinv);
+        return;
+    }
+    u64 v[16];
+#pragma unroll
+    for (int k = 0; k < 16; k++) {
+        acc128 s{0, 0};
+        for (uint32_t a = 0; a < n_src; a++) mac128(s, src[(size_t)a * N + k * T], dg->mat[a][pt]);
+        v[k] = reduce128(s.hi, s.lo, pc);
+    }
+    if (pc.q < FESC_FP_LIMIT) {
+        const FpRow r{tb.twf + ((size_t)pt << LOG), pc.qd, pc.qinvd};
+        double x[16];
+#pragma unroll
+        for (int k = 0; k < 16; k++) x[k] = fp_from_u64(v[k]);
+        small_fwd<LOG>(r, x, sm);
+#pragma unroll
+        for (int k = 0; k < 16; k++) o[k * T] = fp_store(FpRow::value(sm[SM_PAD(k * T + tid)]), r.q, r.qinv);
+    } else {
+        const IntRow r{tb.tw + ((size_t)pt << LOG), pc.q, 2 * pc.q};
+        small_fwd<LOG>(r, v, sm);
+#pragma unroll
+        for (int k = 0; k < 16; k++) o[k * T] = csub(csub(sm[SM_PAD(k * T + tid)], r.q2), r.q);
+    }
+}
+
+// grid (level + K, 2, batch): acc[b][p][t] = sum over sources and digits of ext . key (+ what acc holds); with `last` the rows on
+// special primes are left as COEFF residues times (P/p_k)^-1
+template <int LOG>
+__global__ void __launch_bounds__(1 << (LOG - 4)) k_small_inner(InnerSrcs S, u64* __restrict__ acc, SmallTables tb, const InvScale* __restrict__ scale,
+                                                                uint32_t level, uint32_t n_q, uint32_t K, uint32_t beta, int accumulate, int last) {
+    constexpr uint32_t N = 1u << LOG, T = N / 16;
+    __shared__ u64 sm[SM_PAD(N)];
+    const uint32_t t = blockIdx.x, pol = blockIdx.y, b = blockIdx.z, tid = threadIdx.x, rows = level + K;
+    const uint32_t pt = t < level ? t : n_q + (t - level);
+    u64* o = acc + (((size_t)b * 2 + pol) * rows + t) * N;
+    bool ok = DBG_REGION(o, N * sizeof(u64));
+    for (uint32_t s = 0; s < S.n; s++)
+        for (uint32_t j = 0; j < beta; j++)
+            ok = ok && DBG_REGION(S.s[s].ext + (((size_t)b * beta + j) * rows + t) * N, N * sizeof(u64)) &&
+                 DBG_REGION(S.s[s].key + ((size_t)(2 * j + pol) * (n_q + K) + pt) * N, N * sizeof(u64));
+    if (!ok) return;
+    const PrimeConst& pc = tb.pc[pt];
+    const bool fp = pc.q < FESC_FP_LIMIT;
+    const double q = pc.qd, qinv = pc.qinvd;
+    const bool coef = last && t >= level;
+    constexpr int V = 8;           // points side by side: their loads are in flight together
+#pragma unroll 1
+    for (int k0 = 0; k0 < 16; k0 += V) {
+        const uint32_t c0 = k0 * T + tid;
+        double f[V];
+        acc128 a[V];
+#pragma unroll
+        for (int e = 0; e < V; e++) {
+            const u64 v = accumulate ? o[c0 + e * T] : 0;
+            f[e] = fp ? fp_load(v, q) : 0.0;
+            a[e] = acc128{v, 0};
+        }
+        uint32_t n = 0;
+        for (uint32_t s = 0; s < S.n; s++) {
+            const u64* x = S.s[s].ext + ((size_t)b * beta * rows + t) * N;
+            const u64* w = S.s[s].key + ((size_t)pol * (n_q + K) + pt) * N + c0;
+            uint32_t at[V];
+#pragma unroll
+            for (int e = 0; e < V; e++) at[e] = S.s[s].g ? galois_src(c0 + e * T, LOG, S.s[s].g) : c0 + e * T;
+            for (uint32_t j = 0; j < beta; j++, n++, x += (size_t)rows * N, w += (size_t)2 * (n_q + K) * N) {
+                u64 xv[V], wv[V];
+#pragma unroll
+                for (int e = 0; e < V; e++) xv[e] = x[at[e]], wv[e] = __ldg(w + e * T);
+                if (fp) {      // canonical words: products below 0.875 q, folded back every 7th (see k_inner)
+#pragma unroll
+                    for (int e = 0; e < V; e++) f[e] += fp_modmul(fp_from_u64(xv[e]), fp_from_u64(wv[e]), q, qinv);
+                    if (n % 7 == 6) {
+#pragma unroll
+                        for (int e = 0; e < V; e++) f[e] = fp_reduce(f[e], q, qinv);
+                    }
+                } else {
+#pragma unroll
+                    for (int e = 0; e < V; e++) mac128(a[e], xv[e], wv[e]);
+                    if (n % 8 == 7) {
+#pragma unroll
+                        for (int e = 0; e < V; e++) a[e] = acc128{reduce128(a[e].hi, a[e].lo, pc), 0};
+                    }
+                }
+            }
+        }
+#pragma unroll
+        for (int e = 0; e < V; e++) {
+            const u64 v = fp ? fp_store(f[e], q, qinv) : reduce128(a[e].hi, a[e].lo, pc);
+            if (coef) sm[SM_PAD(c0 + e * T)] = v;
+            else o[c0 + e * T] = v;
+        }
+    }
+    if (!coef) return;
+    __syncthreads();
+    small_inv_row<LOG>(sm, tb, pt, scale + pt, o);
+}
+
+// forward transform of x (canonical words), then out = (acc - u) c (+ the permuted c0) (+ what out holds)
+struct SmallFinish {
+    u64 cinv, cinvs;      // c and its Shoup companion
+    int add;
+    const u64* rot;       // nullptr, or the row added through the permutation of g
+    u64 g;
+};
+template <int LOG>
+__device__ __forceinline__ void small_finish(u64 (&v)[16], u64* sm, const SmallTables& tb, uint32_t pi, const u64* __restrict__ acc, u64* out,
+                                             const SmallFinish& fin) {
+    constexpr uint32_t T = (1u << LOG) / 16;
+    const uint32_t tid = threadIdx.x;
+    const PrimeConst& pc = tb.pc[pi];
+    if (pc.q < FESC_FP_LIMIT) {
+        const FpRow r{tb.twf + ((size_t)pi << LOG), pc.qd, pc.qinvd};
+        double x[16];
+#pragma unroll
+        for (int k = 0; k < 16; k++) x[k] = fp_from_u64(v[k]);
+        small_fwd<LOG>(r, x, sm);
+        const double c = fp_from_u64(fin.cinv);
+#pragma unroll
+        for (int k = 0; k < 16; k++) {      // |acc - u| below 5.4q, the lazy product below 2.6q: every sum is exact
+            const uint32_t t = k * T + tid;
+            double s = fp_modmul(fp_load(acc[t], r.q) - FpRow::value(sm[SM_PAD(t)]), c, r.q, r.qinv);
+            if (fin.rot) s += fp_load(fin.rot[galois_src(t, LOG, fin.g)], r.q);
+            if (fin.add) s += fp_load(out[t], r.q);
+            out[t] = fp_store(s, r.q, r.qinv);
+        }
+    } else {
+        const IntRow r{tb.tw + ((size_t)pi << LOG), pc.q, 2 * pc.q};
+        small_fwd<LOG>(r, v, sm);
+#pragma unroll
+        for (int k = 0; k < 16; k++) {
+            const uint32_t t = k * T + tid;
+            u64 s = shoup(submod(acc[t], csub(csub(sm[SM_PAD(t)], r.q2), r.q), r.q), fin.cinv, fin.cinvs, r.q);
+            if (fin.rot) s = addmod(s, fin.rot[galois_src(t, LOG, fin.g)], r.q);
+            if (fin.add) s = addmod(s, out[t], r.q);
+            out[t] = s;
+        }
+    }
+}
+
+// grid (level, 2, batch): out[b][p][i] = (acc[b][p][i] - u_i) P^-1 (+ ...), u_i = NTT(sum_k [y_k]_centred (P/p_k) mod q_i)
+template <int LOG>
+__global__ void __launch_bounds__(1 << (LOG - 4)) k_small_down(const u64* __restrict__ acc, u64* out, size_t out_stride, const ModDownTab* __restrict__ tab,
+                                                               SmallTables tb, uint32_t level, uint32_t n_q, uint32_t K, int add_mask,
+                                                               const u64* __restrict__ rot_src, size_t rot_stride, u64 g) {
+    constexpr uint32_t N = 1u << LOG, T = N / 16;
+    __shared__ u64 sm[SM_PAD(N)];
+    const uint32_t i = blockIdx.x, pol = blockIdx.y, b = blockIdx.z, tid = threadIdx.x;
+    const u64* a = acc + ((size_t)b * 2 + pol) * (level + K) * N;
+    u64* o = out + (size_t)b * out_stride + ((size_t)pol * level + i) * N;
+    const u64* rot = rot_src && !pol ? rot_src + (size_t)b * rot_stride + (size_t)i * N : nullptr;
+    if (!DBG_REGION(a, (size_t)(level + K) * N * sizeof(u64)) || !DBG_REGION(o, N * sizeof(u64)) || (rot && !DBG_REGION(rot, N * sizeof(u64)))) return;
+    const PrimeConst& pc = tb.pc[i];
+    const bool fp = pc.q < FESC_FP_LIMIT;
+    const double q = pc.qd, qinv = pc.qinvd;
+    u64 v[16];
+    const u64* src = a + (size_t)level * N + tid;
+    u64 cnt = 0;                   // 4 bits per point: how many of its residues are taken negative
+    if (fp) {
+        double s[16];
+#pragma unroll
+        for (int k = 0; k < 16; k++) s[k] = 0.0;
+        for (uint32_t m = 0; m < K; m++) {
+            const u64 half = tab->half[m];
+            const double m30 = tab->mat30d[m][i], m0 = tab->matd[m][i];
+#pragma unroll
+            for (int k = 0; k < 16; k++) {      // 30-bit halves: every product below 0.51 q
+                const u64 y = src[(size_t)m * N + k * T];
+                cnt += (u64)(y > half) << (4 * k);
+                s[k] += fp_modmul(fp_from_u64(y >> 30), m30, q, qinv);
+                s[k] += fp_modmul(fp_from_u64(y & ((1ull << 30) - 1)), m0, q, qinv);
+                if (m == 3) s[k] = fp_reduce(s[k], q, qinv);
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < 16; k++) v[k] = fp_store(s[k] - tab->wrapd[(cnt >> (4 * k)) & 15][i], q, qinv);
+    } else {
+#pragma unroll
+        for (int k = 0; k < 16; k++) {
+            acc128 w{0, 0};
+            uint32_t n = 0;
+            for (uint32_t m = 0; m < K; m++) {
+                const u64 y = src[(size_t)m * N + k * T];
+                n += y > tab->half[m];
+                mac128(w, y, tab->mat[m][i]);
+            }
+            v[k] = submod(reduce128(w.hi, w.lo, pc), tab->wrap[n][i], pc.q);
+        }
+    }
+    small_finish<LOG>(v, sm, tb, i, a + (size_t)i * N, o, SmallFinish{tab->pinv[i], tab->pinvs[i], (add_mask >> pol) & 1, rot, g});
+}
+
+// grid (2, batch): COEFF form of the last limb of both polynomials to r[b][p]
+template <int LOG>
+__global__ void __launch_bounds__(1 << (LOG - 4)) k_small_last(const u64* __restrict__ in, size_t in_stride, u64* __restrict__ r, SmallTables tb, uint32_t level) {
+    constexpr uint32_t N = 1u << LOG, T = N / 16;
+    __shared__ u64 sm[SM_PAD(N)];
+    const uint32_t pol = blockIdx.x, b = blockIdx.y, tid = threadIdx.x;
+    const u64* s = in + (size_t)b * in_stride + ((size_t)pol * level + level - 1) * N;
+    u64* o = r + ((size_t)b * 2 + pol) * N;
+    if (!DBG_REGION(s, N * sizeof(u64)) || !DBG_REGION(o, N * sizeof(u64))) return;
+#pragma unroll
+    for (int k = 0; k < 16; k++) sm[SM_PAD(k * T + tid)] = s[k * T + tid];
+    __syncthreads();
+    small_inv_row<LOG>(sm, tb, level - 1, nullptr, o);
+}
+// grid (level - 1, 2, batch): out = (in - NTT(centred(r) mod q_i)) q_last^-1
+template <int LOG>
+__global__ void __launch_bounds__(1 << (LOG - 4)) k_small_rescale(const u64* __restrict__ in, size_t in_stride, const u64* __restrict__ r, u64* out,
+                                                                  size_t out_stride, const RescaleTab* __restrict__ tab, SmallTables tb, uint32_t level) {
+    constexpr uint32_t N = 1u << LOG, T = N / 16;
+    __shared__ u64 sm[SM_PAD(N)];
+    const uint32_t i = blockIdx.x, pol = blockIdx.y, b = blockIdx.z, tid = threadIdx.x;
+    const u64* a = in + (size_t)b * in_stride + ((size_t)pol * level + i) * N;
+    const u64* s = r + ((size_t)b * 2 + pol) * N;
+    u64* o = out + (size_t)b * out_stride + ((size_t)pol * (level - 1) + i) * N;
+    if (!DBG_REGION(a, N * sizeof(u64)) || !DBG_REGION(s, N * sizeof(u64)) || !DBG_REGION(o, N * sizeof(u64))) return;
+    const PrimeConst& pc = tb.pc[i];
+    u64 v[16];
+#pragma unroll
+    for (int k = 0; k < 16; k++) {
+        const u64 y = s[k * T + tid];
+        u64 w = csub(y - mulhi(y, pc.mu) * pc.q, pc.q);
+        if (y > tab->half) w = submod(w, tab->wrap[i], pc.q);
+        v[k] = w;
+    }
+    small_finish<LOG>(v, sm, tb, i, a, o, SmallFinish{tab->qinv[i], tab->qinvs[i], 0, nullptr, 0});
+}
+
+// ---------------------------------------------------------------------------------------
+// launches
+// ---------------------------------------------------------------------------------------
+bool small_ring(const fesc_ctx* ctx) { return ctx->log_n >= 10 && ctx->log_n <= 12; }
+static SmallTables tables(const fesc_ctx* ctx) { return SmallTables{ctx->d_twf, ctx->d_itwf, ctx->d_tw, ctx->d_itw, ctx->d_pc}; }
+#define SMALL_LAUNCH(kern, grid, ...)                                               \
+    do {                                                                            \
+        if (ctx->log_n == 12) kern<12><<<grid, 256, 0, st>>>(__VA_ARGS__);          \
+        else if (ctx->log_n == 11) kern<11><<<grid, 128, 0, st>>>(__VA_ARGS__);     \
+        else kern<10><<<grid, 64, 0, st>>>(__VA_ARGS__);                            \
+        FESC_CHECK_CUDA(ctx, cudaGetLastError());                                   \
+    } while (0)
+
+int small_ntt_launch(fesc_ctx* ctx, u64* data, size_t rows, const RowMap& map, bool inverse, cudaStream_t st) {
+    RowList l;
+    l.period = map.period, l.count = 0;
+    for (uint32_t i = 0; i < map.period; i++)
+        if (map.prime[i] != 0xFF) l.row[l.count] = (uint8_t)i, l.prime[l.count++] = map.prime[i];
+    const unsigned grid = (unsigned)(rows / map.period * l.count);
+    if (!grid) return FESC_OK;
+    const SmallTables tb = tables(ctx);
+#define SMALL_NTT(LOG)                                                                              \
+    do {                                                                                            \
+        if (inverse) k_small_ntt<LOG, true><<<grid, 1 << (LOG - 4), 0, st>>>(data, tb, l);          \
+        else k_small_ntt<LOG, false><<<grid, 1 << (LOG - 4), 0, st>>>(data, tb, l);                 \
+    } while (0)
+    if (ctx->log_n == 12) SMALL_NTT(12);
+    else if (ctx->log_n == 11) SMALL_NTT(11);
+    else SMALL_NTT(10);
+#undef SMALL_NTT
+    FESC_CHECK_CUDA(ctx, cudaGetLastError());
+    return FESC_OK;
+}
+
+int small_decompose(fesc_ctx* ctx, const KsScratch& ws, const u64* src, size_t src_stride, bool keep_own, u64 g, uint32_t level, uint32_t batch,
+                    cudaStream_t st) {
+    const uint32_t beta = (level + ctx->alpha - 1) / ctx->alpha, rows = level + ctx->n_p;
+    prof_begin(ctx, PF_NTT, st);
+    SMALL_LAUNCH(k_small_coef, dim3(level, batch), src, src_stride, keep_own ? ws.ext : nullptr, (size_t)beta * rows * ctx->N, rows, ctx->alpha,
+                 ws.dcoef, tables(ctx), ctx->tabs.d_up_scale + (size_t)(level - 1) * ctx->n_q, level, g);
+    prof_end(ctx, PF_NTT, st);
+    prof_begin(ctx, PF_MODUP, st);
+    SMALL_LAUNCH(k_small_modup, dim3(beta * rows, batch), ws.dcoef, ws.ext, ctx->tabs.d_modup + (size_t)(level - 1) * ctx->beta_max, tables(ctx), level,
+                 ctx->n_q, ctx->n_p, ctx->alpha, beta);
+    prof_end(ctx, PF_MODUP, st);
+    ctx->counters[0] += (uint64_t)batch * (level + beta * rows - level);
+    return FESC_OK;
+}
+int small_inner(fesc_ctx* ctx, const KsScratch& ws, const InnerSrcs& S, uint32_t level, uint32_t batch, cudaStream_t st, int accumulate, int last) {
+    const uint32_t beta = (level + ctx->alpha - 1) / ctx->alpha;
+    prof_begin(ctx, PF_INNER, st);
+    SMALL_LAUNCH(k_small_inner, dim3(level + ctx->n_p, 2, batch), S, ws.acc, tables(ctx), ctx->tabs.d_down_scale, level, ctx->n_q, ctx->n_p, beta,
+                 accumulate, last);
+    prof_end(ctx, PF_INNER, st);
+    ctx->counters[1] += (uint64_t)batch * S.n;
+    if (last) ctx->counters[0] += (uint64_t)batch * 2 * ctx->n_p;
+    return FESC_OK;
+}
+int small_moddown(fesc_ctx* ctx, const KsScratch& ws, uint32_t level, uint32_t batch, u64* out, size_t out_stride, int add_mask, cudaStream_t st,
+                  const u64* rot_src, size_t rot_stride, u64 g) {
+    prof_begin(ctx, PF_MODDOWN, st);
+    SMALL_LAUNCH(k_small_down, dim3(level, 2, batch), ws.acc, out, out_stride, ctx->tabs.d_moddown, tables(ctx), level, ctx->n_q, ctx->n_p, add_mask,
+                 rot_src, rot_stride, g);
+    prof_end(ctx, PF_MODDOWN, st);
+    ctx->counters[0] += (uint64_t)batch * 2 * level;
+    return FESC_OK;
+}
+int small_rescale(fesc_ctx* ctx, const u64* in, size_t in_stride, u64* out, size_t out_stride, uint32_t batch, uint32_t level, u64* r, cudaStream_t st) {
+    prof_begin(ctx, PF_RESCALE, st);
+    SMALL_LAUNCH(k_small_last, dim3(2, batch), in, in_stride, r, tables(ctx), level);
+    SMALL_LAUNCH(k_small_rescale, dim3(level - 1, 2, batch), in, in_stride, r, out, out_stride, ctx->tabs.d_rescale + level, tables(ctx), level);
+    prof_end(ctx, PF_RESCALE, st, 2);
+    ctx->counters[0] += (uint64_t)batch * 2 * level;
+    return FESC_OK;
+}
