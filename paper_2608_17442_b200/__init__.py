@@ -20,7 +20,7 @@ NET_BRENT_KUNG, NET_KOGGE_STONE, NET_SKLANSKY = 0, 1, 2     # fesc_scan_desc.net
 RELIN_KEY_ID = 0
 
 _lib = None
-_debug_bounds = False      # the loaded library is the bounds-checking debug build
+_debug_bounds = None       # whether the loaded library is the bounds-checking debug build (None: not asked yet)
 
 
 class FescError(RuntimeError):
@@ -126,9 +126,8 @@ def debug_bounds() -> bool:
     the binding then registers the extent of every tensor it passes, and Context.sync raises FescError(EBOUNDS) after
     a kernel skipped a region outside every known extent.  The first call needs a GPU."""
     global _debug_bounds
-    if not getattr(debug_bounds, "asked", False):
+    if _debug_bounds is None:
         _debug_bounds = lib().fesc_debug_bounds_clear() == OK
-        debug_bounds.asked = True
     return _debug_bounds
 
 
@@ -156,10 +155,17 @@ def params_info(log_n: int, primes, n_q: int, n_p: int, dnum: int) -> Info:
     return out
 
 
+_raw_stream = None         # current stream handle of a device, without building a Stream object
+
+
 def _stream():
+    global _raw_stream
     import torch
 
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    if _raw_stream is None:
+        fast = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        _raw_stream = fast or (lambda device: torch.cuda.current_stream(device).cuda_stream)
+    return _raw_stream(torch.cuda.current_device())
 
 
 def _raw(t):
@@ -167,14 +173,14 @@ def _raw(t):
     if t is None:
         return None
     assert t.is_cuda and t.is_contiguous()
-    if debug_bounds():
+    if _debug_bounds or (_debug_bounds is None and debug_bounds()):
         lib().fesc_debug_bounds_register(t.data_ptr(), t.numel() * t.element_size())
     return t.data_ptr()
 
 
 def _ptr(t):
     assert t.element_size() == 8
-    return ctypes.c_void_p(_raw(t))
+    return _raw(t)
 
 
 class Context:

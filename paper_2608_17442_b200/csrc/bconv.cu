@@ -73,6 +73,7 @@ __global__ void __launch_bounds__(32 * BC_WARPS, BC_MINB) k_moddown_conv_imma(co
                                                                      const ModDownTab* __restrict__ tab, const uint4* __restrict__ frag,
                                                                      const PrimeConst* __restrict__ pcs, uint32_t N, uint32_t level,
                                                                      uint32_t n_q, uint32_t K, int out_double) {
+    pdl_begin();
     __shared__ uint4 sfrag[BC_FRAG_WORDS];
     const uint32_t tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, tg = lane & 3;
     const uint32_t bp = blockIdx.y, rows = level + K;
@@ -149,7 +150,7 @@ void moddown_conv_imma_launch(fesc_ctx* ctx, const u64* acc, u64* u, uint32_t le
     const uint32_t N = ctx->N, K = ctx->n_p;
     dim3 grid(N / (BC_WARPS * BC_COEFS), batch * 2);
     if (level > 16)
-        k_moddown_conv_imma<2><<<grid, 32 * BC_WARPS, 0, st>>>(acc, u, ctx->tabs.d_moddown, ctx->tabs.d_md_frag, ctx->d_pc, N, level, ctx->n_q, K, out_double);
+        launch(k_moddown_conv_imma<2>, grid, 32 * BC_WARPS, 0, st, acc, u, ctx->tabs.d_moddown, ctx->tabs.d_md_frag, ctx->d_pc, N, level, ctx->n_q, K, out_double);
     else
-        k_moddown_conv_imma<1><<<grid, 32 * BC_WARPS, 0, st>>>(acc, u, ctx->tabs.d_moddown, ctx->tabs.d_md_frag, ctx->d_pc, N, level, ctx->n_q, K, out_double);
+        launch(k_moddown_conv_imma<1>, grid, 32 * BC_WARPS, 0, st, acc, u, ctx->tabs.d_moddown, ctx->tabs.d_md_frag, ctx->d_pc, N, level, ctx->n_q, K, out_double);
 }

@@ -11,6 +11,7 @@
 // c0 of every ciphertext += its plaintext (pt_stride words between plaintexts)
 __global__ void __launch_bounds__(256) k_ct_add_pt(u64* __restrict__ ct, size_t ct_stride, const u64* __restrict__ pt,
                                                    size_t pt_stride, const PrimeConst* __restrict__ pcs, uint32_t N) {
+    pdl_begin();
     const uint32_t c = blockIdx.x * blockDim.x + threadIdx.x;
     const uint32_t l = blockIdx.y, b = blockIdx.z;
     if (c >= N) return;
@@ -72,7 +73,7 @@ extern "C" int fesc_conv(fesc_ctx* ctx, const uint64_t* d_ct_in, const uint64_t*
             }
         }
         prof_begin(ctx, PF_POINTWISE, st);
-        k_ct_add_pt<<<dim3((N + 255) / 256, level, blocks), 256, 0, st>>>(acc, ctw, (const u64*)d_bias, ptw, ctx->d_pc, N);
+        launch(k_ct_add_pt, dim3((N + 255) / 256, level, blocks), 256, 0, st, acc, ctw, (const u64*)d_bias, ptw, ctx->d_pc, N);
         prof_end(ctx, PF_POINTWISE, st);
         FESC_CHECK_CUDA(ctx, cudaGetLastError());
         rc = rescale_internal(ctx, acc, ctw, out + (size_t)tb * blocks * 2 * (level - 1) * N, blocks, level, ks, st);

@@ -77,6 +77,7 @@ __global__ void __launch_bounds__(MU_THREADS, 2)
     k_modup_cols(const u64* __restrict__ y, u64* __restrict__ ext, const ModUpDigit* __restrict__ tab, const double* __restrict__ twf,
                  const ulonglong2* __restrict__ tw, const PrimeConst* __restrict__ pcs, uint32_t level, uint32_t n_q, uint32_t K,
                  uint32_t beta, uint32_t splits) {
+    pdl_begin();
     extern __shared__ __align__(16) u64 smem[];      // [A][MU_SRC] source columns, then one exchange buffer per group
     __shared__ uint32_t next, taken[MU_GROUPS];
     const uint32_t tid = threadIdx.x, tile = blockIdx.x / splits, part = blockIdx.x % splits, j = blockIdx.y, b = blockIdx.z;
@@ -144,7 +145,7 @@ bool modup16_supported(const fesc_ctx* ctx, uint32_t level) {
 }
 
 template <int A>
-static int launch(fesc_ctx* ctx, const u64* y, u64* ext, uint32_t level, uint32_t batch, cudaStream_t st) {
+static int launch_modup(fesc_ctx* ctx, const u64* y, u64* ext, uint32_t level, uint32_t batch, cudaStream_t st) {
     const uint32_t beta = (level + ctx->alpha - 1) / ctx->alpha, tiles = 256 / MU_COLS;
     const size_t smem = ((size_t)A * MU_SRC + MU_GROUPS * COL_SMEM(MU_COLS)) * sizeof(u64);
     auto kern = k_modup_cols<A>;
@@ -152,12 +153,12 @@ static int launch(fesc_ctx* ctx, const u64* y, u64* ext, uint32_t level, uint32_
     // two CTAs per SM: with few ciphertexts the targets of a tile are shared by up to four CTAs, so that the last wave is full
     uint32_t splits = 1;
     while (splits < 4 && tiles * beta * batch * splits < 8 * 148) splits++;
-    kern<<<dim3(tiles * splits, beta, batch), MU_THREADS, smem, st>>>(y, ext, ctx->tabs.d_modup + (size_t)(level - 1) * ctx->beta_max,
+    launch(kern, dim3(tiles * splits, beta, batch), MU_THREADS, smem, st, y, ext, ctx->tabs.d_modup + (size_t)(level - 1) * ctx->beta_max,
                                                                      ctx->d_twf, ctx->d_tw, ctx->d_pc, level, ctx->n_q, ctx->n_p, beta, splits);
     return FESC_OK;
 }
 int modup16_cols_launch(fesc_ctx* ctx, const u64* y, u64* ext, uint32_t level, uint32_t batch, cudaStream_t st) {
-    if (ctx->alpha <= 1) return launch<1>(ctx, y, ext, level, batch, st);
-    if (ctx->alpha <= 2) return launch<2>(ctx, y, ext, level, batch, st);
-    return launch<4>(ctx, y, ext, level, batch, st);
+    if (ctx->alpha <= 1) return launch_modup<1>(ctx, y, ext, level, batch, st);
+    if (ctx->alpha <= 2) return launch_modup<2>(ctx, y, ext, level, batch, st);
+    return launch_modup<4>(ctx, y, ext, level, batch, st);
 }

@@ -12,6 +12,7 @@
 __global__ void __launch_bounds__(256) k_ct_mul_pt(const u64* ct, size_t ct_stride, const u64* __restrict__ pt,
                                                    size_t pt_stride, u64* out, size_t out_stride,
                                                    const PrimeConst* __restrict__ pcs, uint32_t N, uint32_t level) {
+    pdl_begin();
     const uint32_t c = blockIdx.x * blockDim.x + threadIdx.x;
     const uint32_t l = blockIdx.y, b = blockIdx.z;
     if (c >= N) return;
@@ -96,7 +97,7 @@ extern "C" int fesc_norm_scale(fesc_ctx* ctx, const uint64_t* d_y, const uint64_
         if (rc != FESC_OK) return rc;
         if ((rc = rescale_internal(ctx, prod, ctw, prod1, blocks, level, ks, st)) != FESC_OK) return rc;
         prof_begin(ctx, PF_POINTWISE, st);
-        k_ct_mul_pt<<<grid, 256, 0, st>>>(prod1, ctw1, (const u64*)d_gamma, (size_t)(level - 1) * N, prod1, ctw1, ctx->d_pc, N, level - 1);
+        launch(k_ct_mul_pt, grid, 256, 0, st, prod1, ctw1, (const u64*)d_gamma, (size_t)(level - 1) * N, prod1, ctw1, ctx->d_pc, N, level - 1);
         prof_end(ctx, PF_POINTWISE, st);
         FESC_CHECK_CUDA(ctx, cudaGetLastError());
         rc = rescale_internal(ctx, prod1, ctw1, out + (size_t)tb * blocks * ctw2, blocks, level - 1, ks, st);

@@ -3,7 +3,7 @@
 //
 // Forward: Cooley-Tukey butterflies with psi merged into the twiddles (natural order in, bit-reversed evaluation order
 // out); inverse: Gentleman-Sande with the inverse twiddles and N^-1 folded into the last stage.
-#define FESC_DBG_FILE 2   // file id in the sites a debug build reports
+#define FESC_DBG_FILE 13   // file id in the sites a debug build reports
 #include "common.cuh"
 
 struct Tw {
@@ -33,6 +33,7 @@ __device__ __forceinline__ void gs_bfly(u64& x, u64& y, const Tw& t, u64 q, u64 
 template <bool INV>
 __global__ void __launch_bounds__(256) ntt_small(u64* __restrict__ data, const ulonglong2* __restrict__ tw_all,
                                                  const PrimeConst* __restrict__ pcs, RowMap map, uint32_t log_n) {
+    pdl_begin();
     const uint32_t row = blockIdx.x;
     const uint32_t pi = map.prime[row % map.period];
     if (pi == 0xFF) return;
@@ -106,9 +107,9 @@ int ntt_launch(fesc_ctx* ctx, u64* d_data, size_t rows, const RowMap& map, bool 
     } else {
         size_t smem = sizeof(u64) << ctx->log_n;
         if (!inverse)
-            ntt_small<false><<<(unsigned)rows, 256, smem, st>>>(d_data, tw, ctx->d_pc, map, ctx->log_n);
+            launch(ntt_small<false>, (unsigned)rows, 256, smem, st, d_data, tw, ctx->d_pc, map, ctx->log_n);
         else
-            ntt_small<true><<<(unsigned)rows, 256, smem, st>>>(d_data, tw, ctx->d_pc, map, ctx->log_n);
+            launch(ntt_small<true>, (unsigned)rows, 256, smem, st, d_data, tw, ctx->d_pc, map, ctx->log_n);
         launches = 1;
     }
     prof_end(ctx, PF_NTT, st, launches);

@@ -34,6 +34,7 @@ template <bool FP>
 __global__ void __launch_bounds__(COL_THREADS, 1024 / COL_THREADS)
     ntt16_cols_fwd(u64* __restrict__ data, const void* __restrict__ tw, const PrimeConst* __restrict__ pcs, RowList list,
                    uint32_t y0, int in_double) {
+    pdl_begin();
     __shared__ u64 sm[COL_SMEM(NTT_COLS)];
     uint32_t pi;
     const uint32_t row = list_row(list, y0 + blockIdx.y, pi);
@@ -67,6 +68,7 @@ template <bool FP>
 __global__ void __launch_bounds__(COL_THREADS, 1024 / COL_THREADS)
     ntt16_cols_inv(u64* __restrict__ data, const void* __restrict__ tw, const PrimeConst* __restrict__ pcs, RowList list, uint32_t y0,
                    const InvScale* __restrict__ scale) {
+    pdl_begin();
     __shared__ u64 sm[COL_SMEM(NTT_COLS)];
     uint32_t pi;
     const uint32_t row = list_row(list, y0 + blockIdx.y, pi);
@@ -110,6 +112,7 @@ template <bool FP, bool FIN>
 __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
     ntt16_rows_fwd(u64* __restrict__ data, const void* __restrict__ tw, const PrimeConst* __restrict__ pcs, RowList list,
                    uint32_t y0, int out_double, NttFinish fin) {
+    pdl_begin();
     __shared__ __align__(16) u64 sm_all[NTT_WARPS * ROW_SMEM];
     uint32_t pi;
     const uint32_t row = list_row(list, y0 + blockIdx.y, pi);
@@ -184,6 +187,7 @@ __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
 template <bool FP>
 __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
     ntt16_rows_inv(u64* __restrict__ data, const void* __restrict__ tw, const PrimeConst* __restrict__ pcs, RowList list, uint32_t y0) {
+    pdl_begin();
     __shared__ __align__(16) u64 sm_all[NTT_WARPS * ROW_SMEM];
     uint32_t pi;
     const uint32_t row = list_row(list, y0 + blockIdx.y, pi);
@@ -238,18 +242,18 @@ int ntt16_launch(fesc_ctx* ctx, u64* data, size_t rows, const RowMap& map, bool 
             const dim3 gc(256 / NTT_COLS, n), gr(128 / NTT_WARPS, n);
             const uint32_t y = (uint32_t)y0;
             if (f == 0 && !inverse) {
-                if (!skip_cols) ntt16_cols_fwd<true><<<gc, COL_THREADS, 0, st>>>(data, ctx->d_twf, ctx->d_pc, l, y, in_double);
-                if (fin.acc) ntt16_rows_fwd<true, true><<<gr, ROW_THREADS, 0, st>>>(data, ctx->d_twf, ctx->d_pc, l, y, out_double, fin);
-                else ntt16_rows_fwd<true, false><<<gr, ROW_THREADS, 0, st>>>(data, ctx->d_twf, ctx->d_pc, l, y, out_double, fin);
+                if (!skip_cols) launch(ntt16_cols_fwd<true>, gc, COL_THREADS, 0, st, data, ctx->d_twf, ctx->d_pc, l, y, in_double);
+                if (fin.acc) launch(ntt16_rows_fwd<true, true>, gr, ROW_THREADS, 0, st, data, ctx->d_twf, ctx->d_pc, l, y, out_double, fin);
+                else launch(ntt16_rows_fwd<true, false>, gr, ROW_THREADS, 0, st, data, ctx->d_twf, ctx->d_pc, l, y, out_double, fin);
             } else if (f == 0) {
-                ntt16_rows_inv<true><<<gr, ROW_THREADS, 0, st>>>(data, ctx->d_itwf, ctx->d_pc, l, y);
-                ntt16_cols_inv<true><<<gc, COL_THREADS, 0, st>>>(data, ctx->d_itwf, ctx->d_pc, l, y, scale);
+                launch(ntt16_rows_inv<true>, gr, ROW_THREADS, 0, st, data, ctx->d_itwf, ctx->d_pc, l, y);
+                launch(ntt16_cols_inv<true>, gc, COL_THREADS, 0, st, data, ctx->d_itwf, ctx->d_pc, l, y, scale);
             } else if (!inverse) {
-                if (!skip_cols) ntt16_cols_fwd<false><<<gc, COL_THREADS, 0, st>>>(data, ctx->d_tw, ctx->d_pc, l, y, 0);
-                ntt16_rows_fwd<false, false><<<gr, ROW_THREADS, 0, st>>>(data, ctx->d_tw, ctx->d_pc, l, y, 0, fin);
+                if (!skip_cols) launch(ntt16_cols_fwd<false>, gc, COL_THREADS, 0, st, data, ctx->d_tw, ctx->d_pc, l, y, 0);
+                launch(ntt16_rows_fwd<false, false>, gr, ROW_THREADS, 0, st, data, ctx->d_tw, ctx->d_pc, l, y, 0, fin);
             } else {
-                ntt16_rows_inv<false><<<gr, ROW_THREADS, 0, st>>>(data, ctx->d_itw, ctx->d_pc, l, y);
-                ntt16_cols_inv<false><<<gc, COL_THREADS, 0, st>>>(data, ctx->d_itw, ctx->d_pc, l, y, scale);
+                launch(ntt16_rows_inv<false>, gr, ROW_THREADS, 0, st, data, ctx->d_itw, ctx->d_pc, l, y);
+                launch(ntt16_cols_inv<false>, gc, COL_THREADS, 0, st, data, ctx->d_itw, ctx->d_pc, l, y, scale);
             }
             launches += skip_cols ? 1 : 2;
         }

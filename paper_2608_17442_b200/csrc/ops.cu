@@ -10,6 +10,7 @@
 __global__ void __launch_bounds__(256) k_ct_pt_mac(const u64* __restrict__ ct, const u64* __restrict__ pt, size_t pt_stride,
                                                    u64* __restrict__ acc, const PrimeConst* __restrict__ pcs,
                                                    uint32_t N, uint32_t n_limbs) {
+    pdl_begin();
     const uint32_t c = blockIdx.x * blockDim.x + threadIdx.x;
     const uint32_t l = blockIdx.y, b = blockIdx.z;
     if (c >= N) return;
@@ -36,7 +37,7 @@ extern "C" int fesc_ct_pt_mac(fesc_ctx* ctx, const uint64_t* d_ct, const uint64_
     if (batch > 65535) return fesc_fail(ctx, FESC_EINVAL, "ct_pt_mac: batch too large");
     dim3 grid((ctx->N + 255) / 256, n_limbs, batch);
     prof_begin(ctx, PF_POINTWISE, (cudaStream_t)stream);
-    k_ct_pt_mac<<<grid, 256, 0, (cudaStream_t)stream>>>((const u64*)d_ct, (const u64*)d_pt, pt_stride, (u64*)d_acc,
+    launch(k_ct_pt_mac, grid, 256, 0, (cudaStream_t)stream, (const u64*)d_ct, (const u64*)d_pt, pt_stride, (u64*)d_acc,
                                                         ctx->d_pc, ctx->N, n_limbs);
     prof_end(ctx, PF_POINTWISE, (cudaStream_t)stream);
     FESC_CHECK_CUDA(ctx, cudaGetLastError());
@@ -92,6 +93,7 @@ __global__ void __launch_bounds__(256) k_autom_ct(const u64* __restrict__ in, si
                                                   size_t out_stride, OwnRows d, u64* __restrict__ dcoef,
                                                   uint32_t log_n, uint32_t level, u64 g,
                                                   const PrimeConst* __restrict__ pcs, int accumulate) {
+    pdl_begin();
     const uint32_t N = 1u << log_n;
     const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
     const uint32_t l = blockIdx.y, b = blockIdx.z;
@@ -150,6 +152,7 @@ __global__ void __launch_bounds__(256) k_modup(const u64* __restrict__ dcoef, u6
                                                const ModUpDigit* __restrict__ tab, const PrimeConst* __restrict__ pcs,
                                                uint32_t N, uint32_t level, uint32_t n_q, uint32_t K, uint32_t beta,
                                                int out_double) {
+    pdl_begin();
     // VEC adjacent coefficients per thread: every table word and every prime constant serves VEC products
     const uint32_t c = (blockIdx.x * blockDim.x + threadIdx.x) * VEC;
     const uint32_t j = blockIdx.y, b = blockIdx.z;
@@ -239,6 +242,7 @@ __global__ void __launch_bounds__(256, INNER_MINB) k_inner(InnerSrcs S, u64* __r
                                                uint32_t n_q, uint32_t K, uint32_t alpha, uint32_t beta,
                                                uint32_t batch, uint32_t log_n, int accumulate, uint32_t row0,
                                                int x_double) {
+    pdl_begin();
     const uint32_t c = blockIdx.x * blockDim.x + threadIdx.x;
     const uint32_t t = row0 + blockIdx.y, b0 = blockIdx.z * BT;
     if (c >= N) return;
@@ -408,6 +412,7 @@ __global__ void __launch_bounds__(256, INNER_MINB) k_inner(InnerSrcs S, u64* __r
 // Self-test of the bounded wait: one warp waits on a barrier phase that nothing completes, with a small poll budget;
 // the wait runs out, the status word is set and the kernel returns (no copy is in flight, nothing faults).
 __global__ void k_wait_limit_selftest(uint32_t* __restrict__ status) {
+    pdl_begin();
     __shared__ __align__(8) unsigned long long bar;
     const uint32_t b = (uint32_t)__cvta_generic_to_shared(&bar);
     if (threadIdx.x == 0) {
@@ -424,7 +429,7 @@ __global__ void k_wait_limit_selftest(uint32_t* __restrict__ status) {
 }
 extern "C" int fesc_selftest_wait_limit(fesc_ctx* ctx, void* stream) {
     if (!ctx) return FESC_EINVAL;
-    k_wait_limit_selftest<<<1, 32, 0, (cudaStream_t)stream>>>(ctx->d_status);
+    launch(k_wait_limit_selftest, 1, 32, 0, (cudaStream_t)stream, ctx->d_status);
     FESC_CHECK_CUDA(ctx, cudaGetLastError());
     return FESC_OK;
 }
@@ -436,6 +441,7 @@ __global__ void __launch_bounds__(256, 1) k_inner_tma(const u64* __restrict__ ex
                                                       uint32_t n_q, uint32_t K, uint32_t alpha, uint32_t beta,
                                                       uint32_t batch, uint32_t log_n, u64 g, int accumulate,
                                                       uint32_t n_tiles, uint32_t* __restrict__ status, int x_double) {
+    pdl_begin();
     constexpr int R = 2 + BT;                                // rows per digit: key b, key a, BT ciphertexts
     extern __shared__ __align__(128) u64 smem[];             // [2 stages][beta][R][256] then two barriers
     const uint32_t tid = threadIdx.x;
@@ -605,6 +611,7 @@ __global__ void __launch_bounds__(256) k_moddown_conv(const u64* __restrict__ ac
                                                       const ModDownTab* __restrict__ tab,
                                                       const PrimeConst* __restrict__ pcs, uint32_t N, uint32_t level,
                                                       uint32_t n_q, uint32_t K, int out_double) {
+    pdl_begin();
     // VEC adjacent coefficients per thread: every table word and every prime constant serves VEC products
     const uint32_t c = (blockIdx.x * blockDim.x + threadIdx.x) * VEC;
     const uint32_t bp = blockIdx.y;   // b*2 + p
@@ -683,6 +690,7 @@ __global__ void __launch_bounds__(256) k_moddown_finish(const u64* __restrict__ 
                                                         const ModDownTab* __restrict__ tab,
                                                         const PrimeConst* __restrict__ pcs, uint32_t N, uint32_t level,
                                                         uint32_t K, int add_mask) {
+    pdl_begin();
     const uint32_t c = blockIdx.x * blockDim.x + threadIdx.x;
     const uint32_t i = blockIdx.y, bp = blockIdx.z;
     if (c >= N) return;
@@ -742,8 +750,8 @@ static int ks_decompose(fesc_ctx* ctx, const KsScratch& ws, uint32_t level, uint
     dim3 gmu(vec2 ? N / (256 * KS_VEC) : gx, beta, batch);
 #define MODUP(A)                                                                                           \
     do {                                                                                                   \
-        if (vec2) k_modup<A, KS_VEC><<<gmu, 256, 0, st>>>(ws.dcoef, ws.ext, tab, ctx->d_pc, N, level, nq, K, beta, dbl); \
-        else k_modup<A, 1><<<gmu, 256, 0, st>>>(ws.dcoef, ws.ext, tab, ctx->d_pc, N, level, nq, K, beta, dbl);  \
+        if (vec2) launch(k_modup<A, KS_VEC>, gmu, 256, 0, st, ws.dcoef, ws.ext, tab, ctx->d_pc, N, level, nq, K, beta, dbl); \
+        else launch(k_modup<A, 1>, gmu, 256, 0, st, ws.dcoef, ws.ext, tab, ctx->d_pc, N, level, nq, K, beta, dbl);  \
     } while (0)
     prof_begin(ctx, PF_MODUP, st);
     if (alpha <= 1) MODUP(1);
@@ -771,7 +779,7 @@ static int ks_inner_multi(fesc_ctx* ctx, const KsScratch& ws, const InnerSrcs& S
 #define INNER(BT_, PATH_, ROW0_, NROWS_)                                                                        \
     do {                                                                                                        \
         dim3 gd(gx, NROWS_, (batch + BT_ - 1) / BT_);                                                           \
-        k_inner<BT_, PATH_><<<gd, 256, 0, st>>>(S, ws.acc, ctx->d_pc, N, level, nq, K, alpha, beta, batch,     \
+        launch(k_inner<BT_, PATH_>, gd, 256, 0, st, S, ws.acc, ctx->d_pc, N, level, nq, K, alpha, beta, batch,     \
                                                 ctx->log_n, accumulate, ROW0_, ctx->log_n == 16);              \
     } while (0)
     // data rows on primes below 2^50 and special rows above: one launch per kind, each compiled for its arithmetic
@@ -786,7 +794,7 @@ static int ks_inner_multi(fesc_ctx* ctx, const KsScratch& ws, const InnerSrcs& S
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         FESC_CHECK_CUDA(ctx, cudaFuncSetAttribute(k_inner_tma<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         const uint32_t grid = n_tiles < (uint32_t)sms ? n_tiles : (uint32_t)sms;
-        k_inner_tma<4><<<grid, 256, smem, st>>>(S.s[0].ext, S.s[0].key, ws.acc, ctx->d_pc, N, level, nq, K, alpha, beta,
+        launch(k_inner_tma<4>, grid, 256, smem, st, S.s[0].ext, S.s[0].key, ws.acc, ctx->d_pc, N, level, nq, K, alpha, beta,
                                                  batch, ctx->log_n, S.s[0].g, accumulate, n_tiles, ctx->d_status, ctx->log_n == 16);
     } else if (split) {
         if (batch >= 3) INNER(4, 1, 0, level);
@@ -838,9 +846,9 @@ static int ks_moddown(fesc_ctx* ctx, const KsScratch& ws, uint32_t level, uint32
     if (bconv_supported(ctx, level))
         moddown_conv_imma_launch(ctx, ws.acc, ws.u, level, batch, ctx->log_n == 16, st);
     else if (N % (256 * KS_VEC) == 0)
-        k_moddown_conv<KS_VEC><<<dim3(N / (256 * KS_VEC), batch * 2), 256, 0, st>>>(ws.acc, ws.u, ctx->tabs.d_moddown, ctx->d_pc, N, level, nq, K, ctx->log_n == 16);
+        launch(k_moddown_conv<KS_VEC>, dim3(N / (256 * KS_VEC), batch * 2), 256, 0, st, ws.acc, ws.u, ctx->tabs.d_moddown, ctx->d_pc, N, level, nq, K, ctx->log_n == 16);
     else
-        k_moddown_conv<1><<<dim3(gx, batch * 2), 256, 0, st>>>(ws.acc, ws.u, ctx->tabs.d_moddown, ctx->d_pc, N, level, nq, K, ctx->log_n == 16);
+        launch(k_moddown_conv<1>, dim3(gx, batch * 2), 256, 0, st, ws.acc, ws.u, ctx->tabs.d_moddown, ctx->d_pc, N, level, nq, K, ctx->log_n == 16);
     prof_end(ctx, PF_MODDOWN, st);
     m.period = level;
     for (uint32_t i = 0; i < level; i++) m.prime[i] = (uint8_t)i;
@@ -855,7 +863,7 @@ static int ks_moddown(fesc_ctx* ctx, const KsScratch& ws, uint32_t level, uint32
     }
     if ((rc = ntt_launch(ctx, ws.u, (size_t)batch * 2 * level, m, false, st, ctx->log_n == 16)) != FESC_OK) return rc;
     prof_begin(ctx, PF_MODDOWN, st);
-    k_moddown_finish<<<dim3(gx, level, batch * 2), 256, 0, st>>>(ws.acc, ws.u, out, out_stride, ctx->tabs.d_moddown,
+    launch(k_moddown_finish, dim3(gx, level, batch * 2), 256, 0, st, ws.acc, ws.u, out, out_stride, ctx->tabs.d_moddown,
                                                                  ctx->d_pc, N, level, K, add_mask);
     prof_end(ctx, PF_MODDOWN, st);
     FESC_CHECK_CUDA(ctx, cudaGetLastError());
@@ -891,9 +899,9 @@ static int ks_start(fesc_ctx* ctx, const KsScratch& ws, const u64* in, size_t in
     const dim3 grid((ctx->N + 255) / 256, level, batch);
     prof_begin(ctx, PF_AUTOM, st);
     if (g)
-        k_autom_ct<<<grid, 256, 0, st>>>(in, in_stride, nullptr, 0, own_rows(ctx, ws, level), ws.dcoef, ctx->log_n, level, g, ctx->d_pc, 0);
+        launch(k_autom_ct, grid, 256, 0, st, in, in_stride, nullptr, 0, own_rows(ctx, ws, level), ws.dcoef, ctx->log_n, level, g, ctx->d_pc, 0);
     else
-        k_hoist_prepare<<<grid, 256, 0, st>>>(in, in_stride, nullptr, 0, own_rows(ctx, ws, level), ws.dcoef, ctx->log_n, level, 0, ctx->d_pc);
+        launch(k_hoist_prepare, grid, 256, 0, st, in, in_stride, nullptr, 0, own_rows(ctx, ws, level), ws.dcoef, ctx->log_n, level, 0, ctx->d_pc);
     prof_end(ctx, PF_AUTOM, st);
     return ks_decompose(ctx, ws, level, batch, st);
 }
@@ -942,7 +950,7 @@ int rotate_internal(fesc_ctx* ctx, const u64* in, size_t in_stride, u64* out, si
         } else {
             dim3 g((ctx->N + 255) / 256, level, nb);
             prof_begin(ctx, PF_AUTOM, st);
-            k_autom_ct<<<g, 256, 0, st>>>(ib, in_stride, ob, out_stride, own_rows(ctx, ws, level), ws.dcoef, ctx->log_n, level, it->second.g,
+            launch(k_autom_ct, g, 256, 0, st, ib, in_stride, ob, out_stride, own_rows(ctx, ws, level), ws.dcoef, ctx->log_n, level, it->second.g,
                                           ctx->d_pc, accumulate);
             prof_end(ctx, PF_AUTOM, st);
             rc = key_switch_chunk(ctx, ws, it->second, level, nb, ob, out_stride, accumulate ? 3 : 1, st);
@@ -957,6 +965,7 @@ __global__ void __launch_bounds__(256) k_hoist_prepare(const u64* __restrict__ i
                                                        size_t out_stride, OwnRows d, u64* __restrict__ dcoef,
                                                        uint32_t log_n, uint32_t level, u64 g,
                                                        const PrimeConst* __restrict__ pcs) {
+    pdl_begin();
     const uint32_t N = 1u << log_n;
     const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
     const uint32_t l = blockIdx.y, b = blockIdx.z;
@@ -1005,7 +1014,7 @@ int giant_sum_deferred_internal(fesc_ctx* ctx, u64* acc, uint32_t n_terms, size_
                 KsScratch wss = ws;
                 wss.ext = ws.ext + (size_t)s * ext_words;
                 prof_begin(ctx, PF_AUTOM, st);
-                k_autom_ct<<<g, 256, 0, st>>>(base + (size_t)(p0 + s) * ct_words, stride, base, stride, own_rows(ctx, wss, level),
+                launch(k_autom_ct, g, 256, 0, st, base + (size_t)(p0 + s) * ct_words, stride, base, stride, own_rows(ctx, wss, level),
                                               wss.dcoef, ctx->log_n, level, key.g, ctx->d_pc, 1);
                 prof_end(ctx, PF_AUTOM, st);
                 int rc = ks_decompose(ctx, wss, level, nb, st);
@@ -1046,7 +1055,7 @@ int rotate_hoisted_internal(fesc_ctx* ctx, const u64* in, size_t in_stride, u64*
                 continue;
             }
             prof_begin(ctx, PF_AUTOM, st);
-            k_hoist_prepare<<<g, 256, 0, st>>>(ib, in_stride, ob, out_stride, OwnRows{nullptr, 1, 1, 1, 0}, nullptr, ctx->log_n, level, key.g, ctx->d_pc);
+            launch(k_hoist_prepare, g, 256, 0, st, ib, in_stride, ob, out_stride, OwnRows{nullptr, 1, 1, 1, 0}, nullptr, ctx->log_n, level, key.g, ctx->d_pc);
             prof_end(ctx, PF_AUTOM, st);
             rc = ks_apply(ctx, ws, key, level, nb, ob, out_stride, 1, st, key.g);
             if (rc != FESC_OK) return rc;
@@ -1064,6 +1073,7 @@ struct GaloisSet {
 __global__ void __launch_bounds__(256) k_rotsum_prepare(const u64* __restrict__ in, size_t in_stride, u64* __restrict__ out,
                                                         size_t out_stride, uint32_t log_n, uint32_t level, GaloisSet gs,
                                                         const PrimeConst* __restrict__ pcs) {
+    pdl_begin();
     const uint32_t N = 1u << log_n;
     const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
     const uint32_t l = blockIdx.y, b = blockIdx.z;
@@ -1101,7 +1111,7 @@ int rotate_sum_hoisted_internal(fesc_ctx* ctx, const u64* in, size_t in_stride, 
         const u64* ib = in + (size_t)b0 * in_stride;
         u64* ob = out + (size_t)b0 * out_stride;
         prof_begin(ctx, PF_AUTOM, st);
-        k_rotsum_prepare<<<g, 256, 0, st>>>(ib, in_stride, ob, out_stride, ctx->log_n, level, gs, ctx->d_pc);
+        launch(k_rotsum_prepare, g, 256, 0, st, ib, in_stride, ob, out_stride, ctx->log_n, level, gs, ctx->d_pc);
         prof_end(ctx, PF_AUTOM, st);
         int rc = ks_start(ctx, ws, ib, in_stride, 0, level, nb, st);
         if (rc != FESC_OK) return rc;
@@ -1159,6 +1169,7 @@ extern "C" int fesc_rotate(fesc_ctx* ctx, const uint64_t* d_in, uint64_t* d_out,
 // gather the last limb of every polynomial into r[b*2+p][N]
 __global__ void __launch_bounds__(256) k_take_last(const u64* __restrict__ in, size_t in_stride, u64* __restrict__ r,
                                                    uint32_t N, uint32_t level) {
+    pdl_begin();
     const uint32_t c = blockIdx.x * blockDim.x + threadIdx.x;
     const uint32_t bp = blockIdx.y;
     if (c >= N) return;
@@ -1171,6 +1182,7 @@ __global__ void __launch_bounds__(256) k_take_last(const u64* __restrict__ in, s
 __global__ void __launch_bounds__(256) k_rescale_conv(const u64* __restrict__ r, u64* __restrict__ out, size_t out_stride,
                                                       const RescaleTab* __restrict__ tab,
                                                       const PrimeConst* __restrict__ pcs, uint32_t N, uint32_t level) {
+    pdl_begin();
     const uint32_t c = blockIdx.x * blockDim.x + threadIdx.x;
     const uint32_t i = blockIdx.y, bp = blockIdx.z;
     if (c >= N) return;
@@ -1189,6 +1201,7 @@ __global__ void __launch_bounds__(256) k_rescale_finish(const u64* __restrict__ 
                                                         u64* __restrict__ out, size_t out_stride,
                                                         const RescaleTab* __restrict__ tab,
                                                         const PrimeConst* __restrict__ pcs, uint32_t N, uint32_t level) {
+    pdl_begin();
     const uint32_t c = blockIdx.x * blockDim.x + threadIdx.x;
     const uint32_t i = blockIdx.y, bp = blockIdx.z;
     if (c >= N) return;
@@ -1217,14 +1230,14 @@ int rescale_internal(fesc_ctx* ctx, const u64* in, size_t in_stride, u64* out, u
             continue;
         }
         prof_begin(ctx, PF_RESCALE, st);
-        k_take_last<<<dim3(gx, nb * 2), 256, 0, st>>>(ib, in_stride, scratch, N, level);
+        launch(k_take_last, dim3(gx, nb * 2), 256, 0, st, ib, in_stride, scratch, N, level);
         prof_end(ctx, PF_RESCALE, st);
         RowMap m;
         m.period = 1;
         m.prime[0] = (uint8_t)(level - 1);
         if ((rc = ntt_launch(ctx, scratch, (size_t)nb * 2, m, true, st)) != FESC_OK) return rc;
         prof_begin(ctx, PF_RESCALE, st);
-        k_rescale_conv<<<dim3(gx, level - 1, nb * 2), 256, 0, st>>>(scratch, ob, out_stride, tab, ctx->d_pc, N, level);
+        launch(k_rescale_conv, dim3(gx, level - 1, nb * 2), 256, 0, st, scratch, ob, out_stride, tab, ctx->d_pc, N, level);
         prof_end(ctx, PF_RESCALE, st);
         m.period = level - 1;
         for (uint32_t i = 0; i + 1 < level; i++) m.prime[i] = (uint8_t)i;
@@ -1240,7 +1253,7 @@ int rescale_internal(fesc_ctx* ctx, const u64* in, size_t in_stride, u64* out, u
         }
         if ((rc = ntt_launch(ctx, ob, (size_t)nb * 2 * (level - 1), m, false, st)) != FESC_OK) return rc;
         prof_begin(ctx, PF_RESCALE, st);
-        k_rescale_finish<<<dim3(gx, level - 1, nb * 2), 256, 0, st>>>(ib, in_stride, ob, out_stride, tab, ctx->d_pc, N,
+        launch(k_rescale_finish, dim3(gx, level - 1, nb * 2), 256, 0, st, ib, in_stride, ob, out_stride, tab, ctx->d_pc, N,
                                                                     level);
         prof_end(ctx, PF_RESCALE, st);
     }
@@ -1268,6 +1281,7 @@ __global__ void __launch_bounds__(256) k_tensor(const u64* __restrict__ a, size_
                                                 size_t b_stride, u64* __restrict__ out, size_t out_stride,
                                                 OwnRows d, u64* __restrict__ dcoef,
                                                 const PrimeConst* __restrict__ pcs, uint32_t N, uint32_t level) {
+    pdl_begin();
     const uint32_t c = blockIdx.x * blockDim.x + threadIdx.x;
     const uint32_t l = blockIdx.y, b = blockIdx.z;
     if (c >= N) return;
@@ -1299,7 +1313,7 @@ int ctmul_internal(fesc_ctx* ctx, const u64* a, size_t a_stride, const u64* b, s
         uint32_t nb = batch - b0 < chunk ? batch - b0 : chunk;
         dim3 g((ctx->N + 255) / 256, level, nb);
         prof_begin(ctx, PF_POINTWISE, st);
-        k_tensor<<<g, 256, 0, st>>>(a + (size_t)b0 * a_stride, a_stride, b + (size_t)b0 * b_stride, b_stride,
+        launch(k_tensor, g, 256, 0, st, a + (size_t)b0 * a_stride, a_stride, b + (size_t)b0 * b_stride, b_stride,
                                     out + (size_t)b0 * out_stride, out_stride, own_rows(ctx, ws, level), ws.dcoef, ctx->d_pc, ctx->N, level);
         prof_end(ctx, PF_POINTWISE, st);
         int rc = key_switch_chunk(ctx, ws, key, level, nb, out + (size_t)b0 * out_stride, out_stride, 3, st);

@@ -23,6 +23,7 @@ __global__ void __launch_bounds__(256) k_ct_addsub(const u64* __restrict__ a, si
                                                    size_t b_stride, u64* __restrict__ out, size_t out_stride,
                                                    const PrimeConst* __restrict__ pcs, uint32_t N, uint32_t level,
                                                    int sub) {
+    pdl_begin();
     const uint32_t c = blockIdx.x * blockDim.x + threadIdx.x;
     const uint32_t pl = blockIdx.y, bi = blockIdx.z;   // pl = poly*level + limb
     if (c >= N) return;
@@ -38,6 +39,7 @@ __global__ void __launch_bounds__(256) k_ct_addsub(const u64* __restrict__ a, si
 __global__ void __launch_bounds__(256) k_ct_ptmul(const u64* __restrict__ a, size_t a_stride, const u64* __restrict__ pt,
                                                   size_t pt_stride, u64* __restrict__ out, size_t out_stride,
                                                   const PrimeConst* __restrict__ pcs, uint32_t N, uint32_t level) {
+    pdl_begin();
     const uint32_t c = blockIdx.x * blockDim.x + threadIdx.x;
     const uint32_t l = blockIdx.y, bi = blockIdx.z;
     if (c >= N) return;
@@ -55,6 +57,7 @@ __global__ void __launch_bounds__(256) k_ct_ptmul(const u64* __restrict__ a, siz
 __global__ void __launch_bounds__(256) k_ct_scale_drop(const u64* __restrict__ a, size_t a_stride, u64* __restrict__ out,
                                                        size_t out_stride, const PrimeConst* __restrict__ pcs, uint32_t N,
                                                        uint32_t src, uint32_t keep, u64 k) {
+    pdl_begin();
     const uint32_t c = blockIdx.x * blockDim.x + threadIdx.x;
     const uint32_t l = blockIdx.y % keep, p = blockIdx.y / keep, bi = blockIdx.z;
     if (c >= N) return;
@@ -72,6 +75,7 @@ __global__ void __launch_bounds__(256) k_ct_mul_i(const u64* __restrict__ a, siz
                                                   size_t out_stride, const PrimeConst* __restrict__ pcs,
                                                   const ulonglong2* __restrict__ tw, uint32_t N, uint32_t level,
                                                   int times) {
+    pdl_begin();
     const uint32_t c = blockIdx.x * blockDim.x + threadIdx.x;
     const uint32_t pl = blockIdx.y, bi = blockIdx.z;
     if (c >= N) return;
@@ -90,6 +94,7 @@ __global__ void __launch_bounds__(256) k_ct_mul_i(const u64* __restrict__ a, siz
 __global__ void __launch_bounds__(256) k_ct_sum_into(const u64* __restrict__ a, size_t a_stride, uint32_t count,
                                                      u64* __restrict__ acc, const PrimeConst* __restrict__ pcs,
                                                      uint32_t N, uint32_t level) {
+    pdl_begin();
     const uint32_t c = blockIdx.x * blockDim.x + threadIdx.x;
     const uint32_t pl = blockIdx.y;
     if (c >= N) return;
@@ -112,6 +117,7 @@ __global__ void __launch_bounds__(256) k_class_mac(ClassSources s, uint32_t term
                                                    const u64* __restrict__ masks, u64* __restrict__ out,
                                                    size_t out_stride, const PrimeConst* __restrict__ pcs, uint32_t N,
                                                    uint32_t level) {
+    pdl_begin();
     const uint32_t c = blockIdx.x * blockDim.x + threadIdx.x;
     const uint32_t l = blockIdx.y, b = blockIdx.z;
     if (c >= N) return;
@@ -221,7 +227,7 @@ struct Exec {
     void addsub(const Arr& a, const Arr& b, const Arr& out, int sub) {
         if (!ok() || dry) return;
         prof_begin(ctx, PF_POINTWISE, st);
-        k_ct_addsub<<<grid(2 * a.level, a.count), 256, 0, st>>>(a.p, a.stride, b.p, b.count == 1 && a.count > 1 ? 0 : b.stride,
+        launch(k_ct_addsub, grid(2 * a.level, a.count), 256, 0, st, a.p, a.stride, b.p, b.count == 1 && a.count > 1 ? 0 : b.stride,
                                                                 out.p, out.stride, ctx->d_pc, N, a.level, sub);
         prof_end(ctx, PF_POINTWISE, st);
     }
@@ -230,7 +236,7 @@ struct Exec {
     void mul_i(const Arr& a, const Arr& out, int times) {
         if (!ok() || dry) return;
         prof_begin(ctx, PF_POINTWISE, st);
-        k_ct_mul_i<<<grid(2 * a.level, a.count), 256, 0, st>>>(a.p, a.stride, out.p, out.stride, ctx->d_pc, ctx->d_tw, N,
+        launch(k_ct_mul_i, grid(2 * a.level, a.count), 256, 0, st, a.p, a.stride, out.p, out.stride, ctx->d_pc, ctx->d_tw, N,
                                                                a.level, times);
         prof_end(ctx, PF_POINTWISE, st);
     }
@@ -247,7 +253,7 @@ struct Exec {
         Arr t = alloc(cnt, in.level);
         if (ok() && !dry) {
             prof_begin(ctx, PF_POINTWISE, st);
-            k_ct_ptmul<<<grid(in.level, cnt), 256, 0, st>>>(in.p, in.count == 1 && cnt > 1 ? 0 : in.stride, pt, pt_stride, t.p,
+            launch(k_ct_ptmul, grid(in.level, cnt), 256, 0, st, in.p, in.count == 1 && cnt > 1 ? 0 : in.stride, pt, pt_stride, t.p,
                                                             t.stride, ctx->d_pc, N, in.level);
             prof_end(ctx, PF_POINTWISE, st);
             ctx->counters[2] += cnt;
@@ -279,7 +285,7 @@ struct Exec {
             const uint64_t* tab = kind ? cs->adj_p : cs->adj_s;
             u64 k = tab[(size_t)in.level * (g.l0 + 1) + dst];
             prof_begin(ctx, PF_POINTWISE, st);
-            k_ct_scale_drop<<<grid(2 * (dst + 1), in.count), 256, 0, st>>>(in.p, in.stride, t.p, t.stride, ctx->d_pc, N,
+            launch(k_ct_scale_drop, grid(2 * (dst + 1), in.count), 256, 0, st, in.p, in.stride, t.p, t.stride, ctx->d_pc, N,
                                                                            in.level, dst + 1, k);
             prof_end(ctx, PF_POINTWISE, st);
         }
@@ -387,7 +393,7 @@ struct Exec {
                     cs_.src[j] = k == 0 ? grp.p : rots.p + (size_t)(k > 0 ? k - 1 : (int)G - 2 - k) * cnt * rots.stride;
                 }
                 prof_begin(ctx, PF_POINTWISE, st);
-                k_class_mac<<<grid(lvl, cnt), 256, 0, st>>>(cs_, G, grp.stride, masks, acc.p, acc.stride, ctx->d_pc, N, lvl);
+                launch(k_class_mac, grid(lvl, cnt), 256, 0, st, cs_, G, grp.stride, masks, acc.p, acc.stride, ctx->d_pc, N, lvl);
                 prof_end(ctx, PF_POINTWISE, st);
                 ctx->counters[2] += (uint64_t)G * cnt;
             }
@@ -715,7 +721,7 @@ static int scan_run(Exec& X, const u64* d_x, const u64* d_a, const u64* d_B, con
                     for (uint32_t sg = 0; sg < g.segs && X.ok() && !X.dry; sg++) {
                         u64* dst = d_out + (((size_t)j * g.K_s + k0 + which) * g.segs + sg) * out_ctw;
                         prof_begin(X.ctx, PF_POINTWISE, X.st);
-                        k_ct_sum_into<<<dim3((N + 255) / 256, 2 * lout), 256, 0, X.st>>>(y.p + (size_t)sg * g.Bt * y.stride, y.stride,
+                        launch(k_ct_sum_into, dim3((N + 255) / 256, 2 * lout), 256, 0, X.st, y.p + (size_t)sg * g.Bt * y.stride, y.stride,
                                                                                          g.Bt, dst, X.ctx->d_pc, N, lout);
                         prof_end(X.ctx, PF_POINTWISE, X.st);
                     }
@@ -824,9 +830,9 @@ extern "C" int fesc_split_complex(fesc_ctx* ctx, const uint64_t* d_in, uint64_t*
     if (rc != FESC_OK) return rc;
     const dim3 g((N + 255) / 256, 2 * n_limbs, batch);
     prof_begin(ctx, PF_POINTWISE, st);
-    if (im) k_ct_addsub<<<g, 256, 0, st>>>(in, ctw, re, ctw, im, ctw, ctx->d_pc, N, n_limbs, 1);
-    k_ct_addsub<<<g, 256, 0, st>>>(in, ctw, re, ctw, re, ctw, ctx->d_pc, N, n_limbs, 0);
-    if (im) k_ct_mul_i<<<g, 256, 0, st>>>(im, ctw, im, ctw, ctx->d_pc, ctx->d_tw, N, n_limbs, 3);
+    if (im) launch(k_ct_addsub, g, 256, 0, st, in, ctw, re, ctw, im, ctw, ctx->d_pc, N, n_limbs, 1);
+    launch(k_ct_addsub, g, 256, 0, st, in, ctw, re, ctw, re, ctw, ctx->d_pc, N, n_limbs, 0);
+    if (im) launch(k_ct_mul_i, g, 256, 0, st, im, ctw, im, ctw, ctx->d_pc, ctx->d_tw, N, n_limbs, 3);
     prof_end(ctx, PF_POINTWISE, st, im ? 3 : 1);
     FESC_CHECK_CUDA(ctx, cudaGetLastError());
     return FESC_OK;

@@ -9,7 +9,7 @@
 //   k_small_down    conversion of the special rows to one limb + forward transform + last step of the division [+ permuted c0]
 //   k_small_rescale conversion of the last limb + forward transform + last step of the division
 // A rotation takes 4 launches instead of 9, a rescale 2 instead of 5.
-#define FESC_DBG_FILE 13   // file id in the sites a debug build reports
+#define FESC_DBG_FILE 2   // file id in the sites a debug build reports
 #include "ntt16.cuh"
 #include "ops.cuh"
 
@@ -144,6 +144,7 @@ __device__ __forceinline__ void small_inv_row(u64* sm, const SmallTables& tb, ui
 // ---------------------------------------------------------------------------------------
 template <int LOG, bool INV>
 __global__ void __launch_bounds__(1 << (LOG - 4)) k_small_ntt(u64* __restrict__ data, SmallTables tb, RowList list) {
+    pdl_begin();
     constexpr uint32_t N = 1u << LOG, T = N / 16;
     __shared__ u64 sm[SM_PAD(N)];
     const uint32_t rep = blockIdx.x / list.count, e = blockIdx.x - rep * list.count, pi = list.prime[e], tid = threadIdx.x;
@@ -184,6 +185,7 @@ template <int LOG>
 __global__ void __launch_bounds__(1 << (LOG - 4)) k_small_coef(const u64* src, size_t src_stride, u64* own, size_t own_stride, uint32_t own_rows,
                                                                uint32_t alpha, u64* dcoef, SmallTables tb, const InvScale* __restrict__ scale,
                                                                uint32_t level, u64 g) {
+    pdl_begin();
     constexpr uint32_t N = 1u << LOG, T = N / 16;
     __shared__ u64 sm[SM_PAD(N)];
     const uint32_t l = blockIdx.x, b = blockIdx.y, tid = threadIdx.x;
@@ -206,6 +208,7 @@ __global__ void __launch_bounds__(1 << (LOG - 4)) k_small_coef(const u64* src, s
 template <int LOG>
 __global__ void __launch_bounds__(1 << (LOG - 4)) k_small_modup(const u64* __restrict__ y, u64* __restrict__ ext, const ModUpDigit* __restrict__ tab,
                                                                 SmallTables tb, uint32_t level, uint32_t n_q, uint32_t K, uint32_t alpha, uint32_t beta) {
+    pdl_begin();
     constexpr uint32_t N = 1u << LOG, T = N / 16;
     __shared__ u64 sm[SM_PAD(N)];
     const uint32_t rows = level + K, j = blockIdx.x / rows, t = blockIdx.x - j * rows, b = blockIdx.y, tid = threadIdx.x;
@@ -263,6 +266,7 @@ __global__ void __launch_bounds__(1 << (LOG - 4)) k_small_modup(const u64* __res
 template <int LOG>
 __global__ void __launch_bounds__(1 << (LOG - 4)) k_small_inner(InnerSrcs S, u64* __restrict__ acc, SmallTables tb, const InvScale* __restrict__ scale,
                                                                 uint32_t level, uint32_t n_q, uint32_t K, uint32_t beta, int accumulate, int last) {
+    pdl_begin();
     constexpr uint32_t N = 1u << LOG, T = N / 16;
     __shared__ u64 sm[SM_PAD(N)];
     const uint32_t t = blockIdx.x, pol = blockIdx.y, b = blockIdx.z, tid = threadIdx.x, rows = level + K;
@@ -377,6 +381,7 @@ template <int LOG>
 __global__ void __launch_bounds__(1 << (LOG - 4)) k_small_down(const u64* __restrict__ acc, u64* out, size_t out_stride, const ModDownTab* __restrict__ tab,
                                                                SmallTables tb, uint32_t level, uint32_t n_q, uint32_t K, int add_mask,
                                                                const u64* __restrict__ rot_src, size_t rot_stride, u64 g) {
+    pdl_begin();
     constexpr uint32_t N = 1u << LOG, T = N / 16;
     __shared__ u64 sm[SM_PAD(N)];
     const uint32_t i = blockIdx.x, pol = blockIdx.y, b = blockIdx.z, tid = threadIdx.x;
@@ -427,6 +432,7 @@ __global__ void __launch_bounds__(1 << (LOG - 4)) k_small_down(const u64* __rest
 // grid (2, batch): COEFF form of the last limb of both polynomials to r[b][p]
 template <int LOG>
 __global__ void __launch_bounds__(1 << (LOG - 4)) k_small_last(const u64* __restrict__ in, size_t in_stride, u64* __restrict__ r, SmallTables tb, uint32_t level) {
+    pdl_begin();
     constexpr uint32_t N = 1u << LOG, T = N / 16;
     __shared__ u64 sm[SM_PAD(N)];
     const uint32_t pol = blockIdx.x, b = blockIdx.y, tid = threadIdx.x;
@@ -442,6 +448,7 @@ __global__ void __launch_bounds__(1 << (LOG - 4)) k_small_last(const u64* __rest
 template <int LOG>
 __global__ void __launch_bounds__(1 << (LOG - 4)) k_small_rescale(const u64* __restrict__ in, size_t in_stride, const u64* __restrict__ r, u64* out,
                                                                   size_t out_stride, const RescaleTab* __restrict__ tab, SmallTables tb, uint32_t level) {
+    pdl_begin();
     constexpr uint32_t N = 1u << LOG, T = N / 16;
     __shared__ u64 sm[SM_PAD(N)];
     const uint32_t i = blockIdx.x, pol = blockIdx.y, b = blockIdx.z, tid = threadIdx.x;
@@ -468,9 +475,9 @@ bool small_ring(const fesc_ctx* ctx) { return ctx->log_n >= 10 && ctx->log_n <= 
 static SmallTables tables(const fesc_ctx* ctx) { return SmallTables{ctx->d_twf, ctx->d_itwf, ctx->d_tw, ctx->d_itw, ctx->d_pc}; }
 #define SMALL_LAUNCH(kern, grid, ...)                                               \
     do {                                                                            \
-        if (ctx->log_n == 12) kern<12><<<grid, 256, 0, st>>>(__VA_ARGS__);          \
-        else if (ctx->log_n == 11) kern<11><<<grid, 128, 0, st>>>(__VA_ARGS__);     \
-        else kern<10><<<grid, 64, 0, st>>>(__VA_ARGS__);                            \
+        if (ctx->log_n == 12) launch(kern<12>, grid, 256, 0, st, __VA_ARGS__);          \
+        else if (ctx->log_n == 11) launch(kern<11>, grid, 128, 0, st, __VA_ARGS__);     \
+        else launch(kern<10>, grid, 64, 0, st, __VA_ARGS__);                            \
         FESC_CHECK_CUDA(ctx, cudaGetLastError());                                   \
     } while (0)
 
@@ -484,8 +491,8 @@ int small_ntt_launch(fesc_ctx* ctx, u64* data, size_t rows, const RowMap& map, b
     const SmallTables tb = tables(ctx);
 #define SMALL_NTT(LOG)                                                                              \
     do {                                                                                            \
-        if (inverse) k_small_ntt<LOG, true><<<grid, 1 << (LOG - 4), 0, st>>>(data, tb, l);          \
-        else k_small_ntt<LOG, false><<<grid, 1 << (LOG - 4), 0, st>>>(data, tb, l);                 \
+        if (inverse) launch(k_small_ntt<LOG, true>, grid, 1 << (LOG - 4), 0, st, data, tb, l);          \
+        else launch(k_small_ntt<LOG, false>, grid, 1 << (LOG - 4), 0, st, data, tb, l);                 \
     } while (0)
     if (ctx->log_n == 12) SMALL_NTT(12);
     else if (ctx->log_n == 11) SMALL_NTT(11);
