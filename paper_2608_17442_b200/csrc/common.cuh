@@ -381,6 +381,7 @@ int ntt16_launch(fesc_ctx* ctx, u64* data, size_t rows, const RowMap& map, bool 
                  bool out_double, const NttFinish& fin, uint64_t& launches, const InvScale* scale, bool skip_cols);
 // N = 2^10 .. 2^12 (small.cu)
 bool small_ring(const fesc_ctx* ctx);
+int small_init(fesc_ctx* ctx);      // once per context
 int small_ntt_launch(fesc_ctx* ctx, u64* data, size_t rows, const RowMap& map, bool inverse, cudaStream_t st);
 // double with |x| <= q/2 as handed to the forward transform
 __device__ __forceinline__ u64 fp_handoff(double s, double q, double qinv) {

@@ -561,6 +561,7 @@ extern "C" int fesc_ctx_create(fesc_ctx** out, uint32_t log_n, const uint64_t* p
     if ((rc = upload(ctx, &ctx->d_twf, twf)) != FESC_OK) return bail(rc);
     if ((rc = upload(ctx, &ctx->d_itwf, itwf)) != FESC_OK) return bail(rc);
     if ((rc = build_tables(ctx)) != FESC_OK) return bail(rc);
+    if (small_ring(ctx) && (rc = small_init(ctx)) != FESC_OK) return bail(rc);
     // ---- secret key and relinearisation key ----
     if (dev_alloc(&ctx->d_s, (size_t)np * N * sizeof(u64)) != cudaSuccess) return bail(FESC_ENOMEM);
     if (dev_alloc(&ctx->d_status, sizeof(uint32_t)) != cudaSuccess) return bail(FESC_ENOMEM);

@@ -33,7 +33,13 @@ __device__ __forceinline__ uint32_t pad16(uint32_t e) { return e + 2 * (e >> 4);
 // round folds back.
 // IntRow: any prime below 2^62, lazy Shoup butterflies, values below 4q (forward) or 2q (inverse).
 // ---------------------------------------------------------------------------------------
-struct FpRow {
+// SHARED: the twiddle table is a copy in shared memory.
+template <bool SHARED, class V>
+__device__ __forceinline__ V tw_load(const V* p) {
+    return SHARED ? *p : __ldg(p);
+}
+template <bool SHARED>
+struct FpRowT {
     typedef double T;
     const double* __restrict__ tw;
     double q, qinv;
@@ -50,11 +56,11 @@ struct FpRow {
     template <int S>
     __device__ __forceinline__ void load(double (&w)[8], uint32_t i) const {      // 2^S twiddles from i on
         if (S == 0) {
-            w[0] = __ldg(tw + i);
+            w[0] = tw_load<SHARED>(tw + i);
         } else {
 #pragma unroll
             for (int k = 0; k < (1 << S) / 2; k++) {
-                const double2 v = __ldg(reinterpret_cast<const double2*>(tw + i) + k);
+                const double2 v = tw_load<SHARED>(reinterpret_cast<const double2*>(tw + i) + k);
                 w[2 * k] = v.x, w[2 * k + 1] = v.y;
             }
         }
@@ -63,23 +69,25 @@ struct FpRow {
     __device__ __forceinline__ void load_d(double (&w)[8], uint32_t blk, uint32_t lane) const {
         const double* t = tw + 4096 + 480 * blk;
         if (S == 0) {
-            w[0] = __ldg(t + lane);
+            w[0] = tw_load<SHARED>(t + lane);
         } else {
             const double2* p = reinterpret_cast<const double2*>(t + 32) + 32 * ((1 << S) / 2 - 1) + lane;
 #pragma unroll
             for (int k = 0; k < (1 << S) / 2; k++) {
-                const double2 v = __ldg(p + 32 * k);
+                const double2 v = tw_load<SHARED>(p + 32 * k);
                 w[2 * k] = v.x, w[2 * k + 1] = v.y;
             }
         }
     }
-    __device__ __forceinline__ void one(double& w, uint32_t i) const { w = __ldg(tw + i); }
+    __device__ __forceinline__ void one(double& w, uint32_t i) const { w = tw_load<SHARED>(tw + i); }
     typedef double W;
     __device__ __forceinline__ T fold(T x) const { return fp_reduce(x, q, qinv); }
     static __device__ __forceinline__ u64 bits(T x) { return (u64)__double_as_longlong(x); }
     static __device__ __forceinline__ T value(u64 b) { return __longlong_as_double((long long)b); }
 };
-struct IntRow {
+typedef FpRowT<false> FpRow;
+template <bool SHARED>
+struct IntRowT {
     typedef u64 T;
     typedef ulonglong2 W;
     const ulonglong2* __restrict__ tw;
@@ -97,19 +105,20 @@ struct IntRow {
     template <int S>
     __device__ __forceinline__ void load(W (&w)[8], uint32_t i) const {
 #pragma unroll
-        for (int k = 0; k < (1 << S); k++) w[k] = __ldg(tw + i + k);
+        for (int k = 0; k < (1 << S); k++) w[k] = tw_load<SHARED>(tw + i + k);
     }
     template <int S>
     __device__ __forceinline__ void load_d(W (&w)[8], uint32_t blk, uint32_t lane) const {
         const ulonglong2* t = tw + 4096 + 480 * blk + lane;
 #pragma unroll
-        for (int k = 0; k < (1 << S); k++) w[k] = __ldg(t + 32 * ((1 << S) - 1 + k));
+        for (int k = 0; k < (1 << S); k++) w[k] = tw_load<SHARED>(t + 32 * ((1 << S) - 1 + k));
     }
-    __device__ __forceinline__ void one(W& w, uint32_t i) const { w = __ldg(tw + i); }
+    __device__ __forceinline__ void one(W& w, uint32_t i) const { w = tw_load<SHARED>(tw + i); }
     __device__ __forceinline__ T fold(T x) const { return x; }
     static __device__ __forceinline__ u64 bits(T x) { return x; }
     static __device__ __forceinline__ T value(u64 b) { return b; }
 };
+typedef IntRowT<false> IntRow;
 
 // Stage S (0..3) of a forward round: distance 8 >> S, twiddles (i0 << S) + j for the j-th group of 16 >> S registers.
 template <int S, class R>

@@ -14,6 +14,32 @@
 #include "ops.cuh"
 
 #define SM_PAD(e) ((e) + ((e) >> 4))
+// dynamic shared memory: the padded row, then a copy of the row's twiddle table (8 bytes per entry for FP64 rows, 16 for integer
+// rows).  The copy is made before the kernel waits for its predecessor: at these sizes a stage's twiddles fetched from L2 one
+// stage at a time cost more than its butterflies.
+#define SM_ROW(LOG) ((SM_PAD(1u << LOG) + 1) & ~1u)
+#define SM_BYTES(LOG) (8 * (SM_ROW(LOG) + 2 * (1u << LOG)))
+typedef FpRowT<true> FpS;
+typedef IntRowT<true> IntS;
+template <int LOG>
+__device__ __forceinline__ void small_tables(u64* sm, const SmallTables& tb, uint32_t pi, bool inv) {
+    constexpr uint32_t N = 1u << LOG, T = N / 16;
+    ulonglong2* dst = reinterpret_cast<ulonglong2*>(sm + SM_ROW(LOG));
+    if (tb.pc[pi].q < FESC_FP_LIMIT) {
+        const ulonglong2* src = reinterpret_cast<const ulonglong2*>((inv ? tb.itwf : tb.twf) + (size_t)pi * N);
+#pragma unroll
+        for (int k = 0; k < 8; k++) dst[k * T + threadIdx.x] = __ldg(src + k * T + threadIdx.x);
+    } else {
+        const ulonglong2* src = (inv ? tb.itw : tb.tw) + (size_t)pi * N;
+#pragma unroll
+        for (int k = 0; k < 16; k++) dst[k * T + threadIdx.x] = __ldg(src + k * T + threadIdx.x);
+    }
+}
+#define SMALL_BEGIN(used, pi, inv)                                  \
+    extern __shared__ __align__(16) u64 sm[];                       \
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); \
+    if (used) small_tables<LOG>(sm, tb, pi, inv);                   \
+    asm volatile("griddepcontrol.wait;" ::: "memory");
 
 // Forward: x[k] = point k N/16 + tid on entry; on return the padded buffer holds the transformed row, unreduced.
 template <int LOG, class R>
@@ -21,6 +47,7 @@ __device__ __forceinline__ void small_fwd(const R& r, typename R::T (&x)[16], u6
     constexpr uint32_t N = 1u << LOG, T = N / 16, L = N / 256;
     constexpr int S = LOG - 8;
     const uint32_t tid = threadIdx.x, top = tid / L, low = tid % L;
+    __syncthreads();               // the twiddle table is complete
     fwd_stage<0>(r, x, 1);
     fwd_stage<1>(r, x, 1);
     fwd_stage<2>(r, x, 1);
@@ -99,7 +126,7 @@ __device__ __forceinline__ void small_inv(const R& r, typename R::T (&x)[16], u6
 }
 // last inverse stage of an FP64 / integer row with the constants `s` (nullptr: the plain ones), canonical words to o
 template <int LOG>
-__device__ __forceinline__ void small_inv_store(const FpRow& r, double (&x)[16], const PrimeConst& pc, const InvScale* s, u64* o) {
+__device__ __forceinline__ void small_inv_store(const FpS& r, double (&x)[16], const PrimeConst& pc, const InvScale* s, u64* o) {
     constexpr uint32_t T = (1u << LOG) / 16;
     const double n = s ? s->nd : pc.ninvd, w = s ? s->wd : pc.ninvwd;
 #pragma unroll
@@ -110,7 +137,7 @@ __device__ __forceinline__ void small_inv_store(const FpRow& r, double (&x)[16],
     }
 }
 template <int LOG>
-__device__ __forceinline__ void small_inv_store(const IntRow& r, u64 (&x)[16], const PrimeConst& pc, const InvScale* s, u64* o) {
+__device__ __forceinline__ void small_inv_store(const IntS& r, u64 (&x)[16], const PrimeConst& pc, const InvScale* s, u64* o) {
     constexpr uint32_t T = (1u << LOG) / 16;
     const u64 n = s ? s->n : pc.ninv, ns = s ? s->ns : pc.ninvs, w = s ? s->w : pc.ninvw, ws = s ? s->ws : pc.ninvws;
 #pragma unroll
@@ -125,14 +152,14 @@ template <int LOG>
 __device__ __forceinline__ void small_inv_row(u64* sm, const SmallTables& tb, uint32_t pi, const InvScale* s, u64* o) {
     const PrimeConst& pc = tb.pc[pi];
     if (pc.q < FESC_FP_LIMIT) {
-        const FpRow r{tb.itwf + ((size_t)pi << LOG), pc.qd, pc.qinvd};
+        const FpS r{reinterpret_cast<const double*>(sm + SM_ROW(LOG)), pc.qd, pc.qinvd};
 #pragma unroll
-        for (int k = 0; k < 16; k++) sm[17 * threadIdx.x + k] = FpRow::bits(fp_load(sm[17 * threadIdx.x + k], r.q));
+        for (int k = 0; k < 16; k++) sm[17 * threadIdx.x + k] = FpS::bits(fp_load(sm[17 * threadIdx.x + k], r.q));
         double x[16];
         small_inv<LOG>(r, x, sm);
         small_inv_store<LOG>(r, x, pc, s, o);
     } else {
-        const IntRow r{tb.itw + ((size_t)pi << LOG), pc.q, 2 * pc.q};
+        const IntS r{reinterpret_cast<const ulonglong2*>(sm + SM_ROW(LOG)), pc.q, 2 * pc.q};
         u64 x[16];
         small_inv<LOG>(r, x, sm);
         small_inv_store<LOG>(r, x, pc, s, o);
@@ -144,10 +171,9 @@ __device__ __forceinline__ void small_inv_row(u64* sm, const SmallTables& tb, ui
 // ---------------------------------------------------------------------------------------
 template <int LOG, bool INV>
 __global__ void __launch_bounds__(1 << (LOG - 4)) k_small_ntt(u64* __restrict__ data, SmallTables tb, RowList list) {
-    pdl_begin();
     constexpr uint32_t N = 1u << LOG, T = N / 16;
-    __shared__ u64 sm[SM_PAD(N)];
     const uint32_t rep = blockIdx.x / list.count, e = blockIdx.x - rep * list.count, pi = list.prime[e], tid = threadIdx.x;
+    SMALL_BEGIN(true, pi, INV)
     u64* p = data + ((size_t)rep * list.period + list.row[e]) * N;
     if (!DBG_REGION(p, N * sizeof(u64))) return;
     if (INV) {
@@ -159,15 +185,15 @@ __global__ void __launch_bounds__(1 << (LOG - 4)) k_small_ntt(u64* __restrict__ 
     }
     const PrimeConst& pc = tb.pc[pi];
     if (pc.q < FESC_FP_LIMIT) {
-        const FpRow r{tb.twf + ((size_t)pi << LOG), pc.qd, pc.qinvd};
+        const FpS r{reinterpret_cast<const double*>(sm + SM_ROW(LOG)), pc.qd, pc.qinvd};
         double x[16];
 #pragma unroll
         for (int k = 0; k < 16; k++) x[k] = fp_from_u64(p[k * T + tid]);
         small_fwd<LOG>(r, x, sm);
 #pragma unroll
-        for (int k = 0; k < 16; k++) p[k * T + tid] = fp_store(FpRow::value(sm[SM_PAD(k * T + tid)]), r.q, r.qinv);
+        for (int k = 0; k < 16; k++) p[k * T + tid] = fp_store(FpS::value(sm[SM_PAD(k * T + tid)]), r.q, r.qinv);
     } else {
-        const IntRow r{tb.tw + ((size_t)pi << LOG), pc.q, 2 * pc.q};
+        const IntS r{reinterpret_cast<const ulonglong2*>(sm + SM_ROW(LOG)), pc.q, 2 * pc.q};
         u64 x[16];
 #pragma unroll
         for (int k = 0; k < 16; k++) x[k] = p[k * T + tid];
@@ -185,10 +211,9 @@ template <int LOG>
 __global__ void __launch_bounds__(1 << (LOG - 4)) k_small_coef(const u64* src, size_t src_stride, u64* own, size_t own_stride, uint32_t own_rows,
                                                                uint32_t alpha, u64* dcoef, SmallTables tb, const InvScale* __restrict__ scale,
                                                                uint32_t level, u64 g) {
-    pdl_begin();
     constexpr uint32_t N = 1u << LOG, T = N / 16;
-    __shared__ u64 sm[SM_PAD(N)];
     const uint32_t l = blockIdx.x, b = blockIdx.y, tid = threadIdx.x;
+    SMALL_BEGIN(true, l, true)
     const u64* in = src + (size_t)b * src_stride + (size_t)l * N;
     u64* o = dcoef + ((size_t)b * level + l) * N;
     u64* w = own ? own + (size_t)b * own_stride + ((size_t)(l / alpha) * own_rows + l) * N : nullptr;
@@ -208,12 +233,11 @@ __global__ void __launch_bounds__(1 << (LOG - 4)) k_small_coef(const u64* src, s
 template <int LOG>
 __global__ void __launch_bounds__(1 << (LOG - 4)) k_small_modup(const u64* __restrict__ y, u64* __restrict__ ext, const ModUpDigit* __restrict__ tab,
                                                                 SmallTables tb, uint32_t level, uint32_t n_q, uint32_t K, uint32_t alpha, uint32_t beta) {
-    pdl_begin();
     constexpr uint32_t N = 1u << LOG, T = N / 16;
-    __shared__ u64 sm[SM_PAD(N)];
     const uint32_t rows = level + K, j = blockIdx.x / rows, t = blockIdx.x - j * rows, b = blockIdx.y, tid = threadIdx.x;
     if (t < level && t / alpha == j) return;
     const uint32_t pt = t < level ? t : n_q + (t - level);
+    SMALL_BEGIN(true, pt, false)
     const ModUpDigit* dg = tab + j;
     const uint32_t n_src = dg->n_src;
     const u64* src = y + ((size_t)b * level + dg->first) * N + tid;
@@ -223,7 +247,7 @@ __global__ void __launch_bounds__(1 << (LOG - 4)) k_small_modup(const u64* __res
     bool fp = pc.q < FESC_FP_LIMIT;
     for (uint32_t a = 0; a < n_src; a++) fp = fp && tb.pc[dg->first + a].q < FESC_FP_LIMIT;
     if (fp) {
-        const FpRow r{tb.twf + ((size_t)pt << LOG), pc.qd, pc.qinvd};
+        const FpS r{reinterpret_cast<const double*>(sm + SM_ROW(LOG)), pc.qd, pc.qinvd};
         double x[16];
 #pragma unroll
         for (int k = 0; k < 16; k++) x[k] = 0.0;
@@ -235,7 +259,7 @@ __global__ void __launch_bounds__(1 << (LOG - 4)) k_small_modup(const u64* __res
         }
         small_fwd<LOG>(r, x, sm);
 #pragma unroll
-        for (int k = 0; k < 16; k++) o[k * T] = fp_store(FpRow::value(sm[SM_PAD(k * T + tid)]), r.q, r.qinv);
+        for (int k = 0; k < 16; k++) o[k * T] = fp_store(FpS::value(sm[SM_PAD(k * T + tid)]), r.q, r.qinv);
         return;
     }
     u64 v[16];
@@ -246,15 +270,15 @@ __global__ void __launch_bounds__(1 << (LOG - 4)) k_small_modup(const u64* __res
         v[k] = reduce128(s.hi, s.lo, pc);
     }
     if (pc.q < FESC_FP_LIMIT) {
-        const FpRow r{tb.twf + ((size_t)pt << LOG), pc.qd, pc.qinvd};
+        const FpS r{reinterpret_cast<const double*>(sm + SM_ROW(LOG)), pc.qd, pc.qinvd};
         double x[16];
 #pragma unroll
         for (int k = 0; k < 16; k++) x[k] = fp_from_u64(v[k]);
         small_fwd<LOG>(r, x, sm);
 #pragma unroll
-        for (int k = 0; k < 16; k++) o[k * T] = fp_store(FpRow::value(sm[SM_PAD(k * T + tid)]), r.q, r.qinv);
+        for (int k = 0; k < 16; k++) o[k * T] = fp_store(FpS::value(sm[SM_PAD(k * T + tid)]), r.q, r.qinv);
     } else {
-        const IntRow r{tb.tw + ((size_t)pt << LOG), pc.q, 2 * pc.q};
+        const IntS r{reinterpret_cast<const ulonglong2*>(sm + SM_ROW(LOG)), pc.q, 2 * pc.q};
         small_fwd<LOG>(r, v, sm);
 #pragma unroll
         for (int k = 0; k < 16; k++) o[k * T] = csub(csub(sm[SM_PAD(k * T + tid)], r.q2), r.q);
@@ -266,11 +290,10 @@ __global__ void __launch_bounds__(1 << (LOG - 4)) k_small_modup(const u64* __res
 template <int LOG>
 __global__ void __launch_bounds__(1 << (LOG - 4)) k_small_inner(InnerSrcs S, u64* __restrict__ acc, SmallTables tb, const InvScale* __restrict__ scale,
                                                                 uint32_t level, uint32_t n_q, uint32_t K, uint32_t beta, int accumulate, int last) {
-    pdl_begin();
     constexpr uint32_t N = 1u << LOG, T = N / 16;
-    __shared__ u64 sm[SM_PAD(N)];
     const uint32_t t = blockIdx.x, pol = blockIdx.y, b = blockIdx.z, tid = threadIdx.x, rows = level + K;
     const uint32_t pt = t < level ? t : n_q + (t - level);
+    SMALL_BEGIN(last && t >= level, pt, true)
     u64* o = acc + (((size_t)b * 2 + pol) * rows + t) * N;
     bool ok = DBG_REGION(o, N * sizeof(u64));
     for (uint32_t s = 0; s < S.n; s++)
@@ -348,7 +371,7 @@ __device__ __forceinline__ void small_finish(u64 (&v)[16], u64* sm, const SmallT
     const uint32_t tid = threadIdx.x;
     const PrimeConst& pc = tb.pc[pi];
     if (pc.q < FESC_FP_LIMIT) {
-        const FpRow r{tb.twf + ((size_t)pi << LOG), pc.qd, pc.qinvd};
+        const FpS r{reinterpret_cast<const double*>(sm + SM_ROW(LOG)), pc.qd, pc.qinvd};
         double x[16];
 #pragma unroll
         for (int k = 0; k < 16; k++) x[k] = fp_from_u64(v[k]);
@@ -357,13 +380,13 @@ __device__ __forceinline__ void small_finish(u64 (&v)[16], u64* sm, const SmallT
 #pragma unroll
         for (int k = 0; k < 16; k++) {      // |acc - u| below 5.4q, the lazy product below 2.6q: every sum is exact
             const uint32_t t = k * T + tid;
-            double s = fp_modmul(fp_load(acc[t], r.q) - FpRow::value(sm[SM_PAD(t)]), c, r.q, r.qinv);
+            double s = fp_modmul(fp_load(acc[t], r.q) - FpS::value(sm[SM_PAD(t)]), c, r.q, r.qinv);
             if (fin.rot) s += fp_load(fin.rot[galois_src(t, LOG, fin.g)], r.q);
             if (fin.add) s += fp_load(out[t], r.q);
             out[t] = fp_store(s, r.q, r.qinv);
         }
     } else {
-        const IntRow r{tb.tw + ((size_t)pi << LOG), pc.q, 2 * pc.q};
+        const IntS r{reinterpret_cast<const ulonglong2*>(sm + SM_ROW(LOG)), pc.q, 2 * pc.q};
         small_fwd<LOG>(r, v, sm);
 #pragma unroll
         for (int k = 0; k < 16; k++) {
@@ -381,10 +404,9 @@ template <int LOG>
 __global__ void __launch_bounds__(1 << (LOG - 4)) k_small_down(const u64* __restrict__ acc, u64* out, size_t out_stride, const ModDownTab* __restrict__ tab,
                                                                SmallTables tb, uint32_t level, uint32_t n_q, uint32_t K, int add_mask,
                                                                const u64* __restrict__ rot_src, size_t rot_stride, u64 g) {
-    pdl_begin();
     constexpr uint32_t N = 1u << LOG, T = N / 16;
-    __shared__ u64 sm[SM_PAD(N)];
     const uint32_t i = blockIdx.x, pol = blockIdx.y, b = blockIdx.z, tid = threadIdx.x;
+    SMALL_BEGIN(true, i, false)
     const u64* a = acc + ((size_t)b * 2 + pol) * (level + K) * N;
     u64* o = out + (size_t)b * out_stride + ((size_t)pol * level + i) * N;
     const u64* rot = rot_src && !pol ? rot_src + (size_t)b * rot_stride + (size_t)i * N : nullptr;
@@ -432,10 +454,9 @@ __global__ void __launch_bounds__(1 << (LOG - 4)) k_small_down(const u64* __rest
 // grid (2, batch): COEFF form of the last limb of both polynomials to r[b][p]
 template <int LOG>
 __global__ void __launch_bounds__(1 << (LOG - 4)) k_small_last(const u64* __restrict__ in, size_t in_stride, u64* __restrict__ r, SmallTables tb, uint32_t level) {
-    pdl_begin();
     constexpr uint32_t N = 1u << LOG, T = N / 16;
-    __shared__ u64 sm[SM_PAD(N)];
     const uint32_t pol = blockIdx.x, b = blockIdx.y, tid = threadIdx.x;
+    SMALL_BEGIN(true, level - 1, true)
     const u64* s = in + (size_t)b * in_stride + ((size_t)pol * level + level - 1) * N;
     u64* o = r + ((size_t)b * 2 + pol) * N;
     if (!DBG_REGION(s, N * sizeof(u64)) || !DBG_REGION(o, N * sizeof(u64))) return;
@@ -448,10 +469,9 @@ __global__ void __launch_bounds__(1 << (LOG - 4)) k_small_last(const u64* __rest
 template <int LOG>
 __global__ void __launch_bounds__(1 << (LOG - 4)) k_small_rescale(const u64* __restrict__ in, size_t in_stride, const u64* __restrict__ r, u64* out,
                                                                   size_t out_stride, const RescaleTab* __restrict__ tab, SmallTables tb, uint32_t level) {
-    pdl_begin();
     constexpr uint32_t N = 1u << LOG, T = N / 16;
-    __shared__ u64 sm[SM_PAD(N)];
     const uint32_t i = blockIdx.x, pol = blockIdx.y, b = blockIdx.z, tid = threadIdx.x;
+    SMALL_BEGIN(true, i, false)
     const u64* a = in + (size_t)b * in_stride + ((size_t)pol * level + i) * N;
     const u64* s = r + ((size_t)b * 2 + pol) * N;
     u64* o = out + (size_t)b * out_stride + ((size_t)pol * (level - 1) + i) * N;
@@ -471,13 +491,24 @@ __global__ void __launch_bounds__(1 << (LOG - 4)) k_small_rescale(const u64* __r
 // ---------------------------------------------------------------------------------------
 // launches
 // ---------------------------------------------------------------------------------------
+template <int LOG>
+static int small_attr(fesc_ctx* ctx) {
+    const void* kernels[] = {(const void*)k_small_coef<LOG>, (const void*)k_small_modup<LOG>, (const void*)k_small_inner<LOG>, (const void*)k_small_down<LOG>,
+                             (const void*)k_small_last<LOG>, (const void*)k_small_rescale<LOG>, (const void*)k_small_ntt<LOG, false>,
+                             (const void*)k_small_ntt<LOG, true>};
+    for (const void* k : kernels) FESC_CHECK_CUDA(ctx, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, SM_BYTES(LOG)));
+    return FESC_OK;
+}
+int small_init(fesc_ctx* ctx) {      // up to 98 KB of shared memory per CTA
+    return ctx->log_n == 12 ? small_attr<12>(ctx) : ctx->log_n == 11 ? small_attr<11>(ctx) : small_attr<10>(ctx);
+}
 bool small_ring(const fesc_ctx* ctx) { return ctx->log_n >= 10 && ctx->log_n <= 12; }
 static SmallTables tables(const fesc_ctx* ctx) { return SmallTables{ctx->d_twf, ctx->d_itwf, ctx->d_tw, ctx->d_itw, ctx->d_pc}; }
 #define SMALL_LAUNCH(kern, grid, ...)                                               \
     do {                                                                            \
-        if (ctx->log_n == 12) launch(kern<12>, grid, 256, 0, st, __VA_ARGS__);          \
-        else if (ctx->log_n == 11) launch(kern<11>, grid, 128, 0, st, __VA_ARGS__);     \
-        else launch(kern<10>, grid, 64, 0, st, __VA_ARGS__);                            \
+        if (ctx->log_n == 12) launch(kern<12>, grid, 256, SM_BYTES(12), st, __VA_ARGS__);          \
+        else if (ctx->log_n == 11) launch(kern<11>, grid, 128, SM_BYTES(11), st, __VA_ARGS__);     \
+        else launch(kern<10>, grid, 64, SM_BYTES(10), st, __VA_ARGS__);                            \
         FESC_CHECK_CUDA(ctx, cudaGetLastError());                                   \
     } while (0)
 
@@ -491,8 +522,8 @@ int small_ntt_launch(fesc_ctx* ctx, u64* data, size_t rows, const RowMap& map, b
     const SmallTables tb = tables(ctx);
 #define SMALL_NTT(LOG)                                                                              \
     do {                                                                                            \
-        if (inverse) launch(k_small_ntt<LOG, true>, grid, 1 << (LOG - 4), 0, st, data, tb, l);          \
-        else launch(k_small_ntt<LOG, false>, grid, 1 << (LOG - 4), 0, st, data, tb, l);                 \
+        if (inverse) launch(k_small_ntt<LOG, true>, grid, 1 << (LOG - 4), SM_BYTES(LOG), st, data, tb, l);          \
+        else launch(k_small_ntt<LOG, false>, grid, 1 << (LOG - 4), SM_BYTES(LOG), st, data, tb, l);                 \
     } while (0)
     if (ctx->log_n == 12) SMALL_NTT(12);
     else if (ctx->log_n == 11) SMALL_NTT(11);
