@@ -29,8 +29,10 @@ __device__ __forceinline__ uint32_t list_row(const RowList& list, uint32_t y, ui
     return rep * list.period + list.row[e];
 }
 
+__device__ __forceinline__ void prefetch_l2(const u64* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
 // grid = (256 / NTT_COLS, rows)
-template <bool FP>
+template <int A>
 __global__ void __launch_bounds__(COL_THREADS, 1024 / COL_THREADS)
     ntt16_cols_fwd(u64* __restrict__ data, const void* __restrict__ tw, const PrimeConst* __restrict__ pcs, RowList list,
                    uint32_t y0, int in_double) {
@@ -41,7 +43,7 @@ __global__ void __launch_bounds__(COL_THREADS, 1024 / COL_THREADS)
     const uint32_t col = threadIdx.x % NTT_COLS, sub = threadIdx.x / NTT_COLS;
     if (!DBG_REGION(data + (size_t)row * N16, N16 * sizeof(u64))) return;      // the same for the whole CTA
     u64* p = data + (size_t)row * N16 + blockIdx.x * NTT_COLS + col;
-    if (FP) {
+    if constexpr (A == ROW_FP) {
         FpRow r{(const double*)tw + (size_t)pi * N16, pcs[pi].qd, pcs[pi].qinvd};
         double x[16];
 #pragma unroll
@@ -54,7 +56,7 @@ __global__ void __launch_bounds__(COL_THREADS, 1024 / COL_THREADS)
         for (int k = 0; k < 16; k++) p[(16 * sub + k) * 256] = FpRow::bits(x[k]);      // doubles below 3.7q
     } else {
         const u64 q = pcs[pi].q;
-        IntRow r{(const ulonglong2*)tw + (size_t)pi * N16, q, 2 * q};
+        const IntRow r{(const ulonglong2*)tw + (size_t)pi * N16, q, 2 * q};
         u64 x[16];
 #pragma unroll
         for (int k = 0; k < 16; k++) x[k] = p[(16 * k + sub) * 256];
@@ -64,7 +66,7 @@ __global__ void __launch_bounds__(COL_THREADS, 1024 / COL_THREADS)
     }
 }
 
-template <bool FP>
+template <int A>
 __global__ void __launch_bounds__(COL_THREADS, 1024 / COL_THREADS)
     ntt16_cols_inv(u64* __restrict__ data, const void* __restrict__ tw, const PrimeConst* __restrict__ pcs, RowList list, uint32_t y0,
                    const InvScale* __restrict__ scale) {
@@ -76,7 +78,7 @@ __global__ void __launch_bounds__(COL_THREADS, 1024 / COL_THREADS)
     if (!DBG_REGION(data + (size_t)row * N16, N16 * sizeof(u64))) return;
     u64* p = data + (size_t)row * N16 + blockIdx.x * NTT_COLS + col;
     const PrimeConst& pc = pcs[pi];
-    if (FP) {
+    if constexpr (A == ROW_FP) {
         FpRow r{(const double*)tw + (size_t)pi * N16, pc.qd, pc.qinvd};
         double x[16];
 #pragma unroll
@@ -91,7 +93,7 @@ __global__ void __launch_bounds__(COL_THREADS, 1024 / COL_THREADS)
         }
     } else {
         const u64 q = pc.q;
-        IntRow r{(const ulonglong2*)tw + (size_t)pi * N16, q, 2 * q};
+        const IntRow r{(const ulonglong2*)tw + (size_t)pi * N16, q, 2 * q};
         u64 x[16];
 #pragma unroll
         for (int k = 0; k < 16; k++) x[k] = p[(16 * sub + k) * 256];
@@ -108,7 +110,7 @@ __global__ void __launch_bounds__(COL_THREADS, 1024 / COL_THREADS)
 }
 
 // grid = (128 / NTT_WARPS, rows); FIN: the last step of a division instead of the plain store (NttFinish)
-template <bool FP, bool FIN>
+template <int A, bool FIN>
 __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
     ntt16_rows_fwd(u64* __restrict__ data, const void* __restrict__ tw, const PrimeConst* __restrict__ pcs, RowList list,
                    uint32_t y0, int out_double, NttFinish fin) {
@@ -122,11 +124,17 @@ __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
     if (!DBG_REGION(p, 512 * sizeof(u64))) return;      // warp barriers only
     const u64* in = p + 256 * (lane >> 4) + (lane & 15);
     const u64* s = sm + 2 * lane + 2 * (lane >> 3);     // the pair 2 lane (+ 64 j) of the padded buffer
-    if (FP) {
+    if constexpr (A == ROW_FP) {
         FpRow r{(const double*)tw + (size_t)pi * N16, pcs[pi].qd, pcs[pi].qinvd};
         double x[16];
 #pragma unroll
         for (int k = 0; k < 16; k++) x[k] = FpRow::value(in[16 * k]);
+        if (FIN) {
+            const uint32_t bp = row / fin.level, i = row - bp * fin.level, b = bp >> 1, pol = bp & 1;
+            prefetch_l2(fin.acc + (size_t)b * fin.acc_stride + ((size_t)pol * fin.acc_rows + i) * N16 + blk * 512 + 16 * lane);
+            if (fin.rot_src && !pol)
+                prefetch_l2(fin.rot_src + (size_t)b * fin.rot_stride + (size_t)i * N16 + (galois_src(blk * 512, 16, fin.rot_g) & ~511u) + 16 * lane);
+        }
         fwd_rows(r, x, sm, blk, lane);
         const double q = r.q, qinv = r.qinv;
         if (!FIN) {
@@ -149,28 +157,38 @@ __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
         if (!DBG_REGION(acc, N16 * sizeof(u64)) || !DBG_REGION(out, N16 * sizeof(u64)) || (rot && !DBG_REGION(rot, N16 * sizeof(u64)))) return;
         const double cinv = fin.cinv[i];
         const bool add = (fin.add_mask >> pol) & 1;
-#pragma unroll 4
-        for (int j = 0; j < 8; j++) {
-            const uint32_t t = blk * 512 + 2 * lane + 64 * j;
-            const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(s + 72 * j);
-            const ulonglong2 av = *reinterpret_cast<const ulonglong2*>(acc + t);
-            double s0 = fp_modmul(fp_load(av.x, q) - FpRow::value(v.x), cinv, q, qinv);
-            double s1 = fp_modmul(fp_load(av.y, q) - FpRow::value(v.y), cinv, q, qinv);
+        // the registers of the transform are free: all eight minuends are requested at once, the other addends by fours
+        ulonglong2 av[8];
+#pragma unroll
+        for (int j = 0; j < 8; j++) av[j] = *reinterpret_cast<const ulonglong2*>(acc + blk * 512 + 2 * lane + 64 * j);
+#pragma unroll
+        for (int h = 0; h < 8; h += 4) {
+            u64 w[8];
             if (rot) {
-                s0 += fp_load(rot[galois_src(t, 16, fin.rot_g)], q);
-                s1 += fp_load(rot[galois_src(t + 1, 16, fin.rot_g)], q);
+#pragma unroll
+                for (int j = 0; j < 8; j++) w[j] = rot[galois_src(blk * 512 + 2 * lane + 64 * (h + (j >> 1)) + (j & 1), 16, fin.rot_g)];
             }
-            ulonglong2* o = reinterpret_cast<ulonglong2*>(out + t);
-            if (add) {
-                const ulonglong2 ov = *o;
-                s0 += fp_load(ov.x, q);
-                s1 += fp_load(ov.y, q);
+#pragma unroll
+            for (int j = h; j < h + 4; j++) {
+                const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(s + 72 * j);
+                double s0 = fp_modmul(fp_load(av[j].x, q) - FpRow::value(v.x), cinv, q, qinv);
+                double s1 = fp_modmul(fp_load(av[j].y, q) - FpRow::value(v.y), cinv, q, qinv);
+                if (rot) {
+                    s0 += fp_load(w[2 * (j - h)], q);
+                    s1 += fp_load(w[2 * (j - h) + 1], q);
+                }
+                ulonglong2* o = reinterpret_cast<ulonglong2*>(out + blk * 512 + 2 * lane + 64 * j);
+                if (add) {
+                    const ulonglong2 ov = *o;
+                    s0 += fp_load(ov.x, q);
+                    s1 += fp_load(ov.y, q);
+                }
+                *o = make_ulonglong2(fp_store(s0, q, qinv), fp_store(s1, q, qinv));
             }
-            *o = make_ulonglong2(fp_store(s0, q, qinv), fp_store(s1, q, qinv));
         }
     } else {
         const u64 q = pcs[pi].q;
-        IntRow r{(const ulonglong2*)tw + (size_t)pi * N16, q, 2 * q};
+        const IntRow r{(const ulonglong2*)tw + (size_t)pi * N16, q, 2 * q};
         u64 x[16];
 #pragma unroll
         for (int k = 0; k < 16; k++) x[k] = in[16 * k];
@@ -179,12 +197,12 @@ __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
 #pragma unroll
         for (int j = 0; j < 8; j++) {
             const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(s + 72 * j);
-            o[32 * j] = make_ulonglong2(csub(csub(v.x, r.q2), q), csub(csub(v.y, r.q2), q));
+            o[32 * j] = make_ulonglong2(r.canonical(v.x), r.canonical(v.y));
         }
     }
 }
 
-template <bool FP>
+template <int A>
 __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
     ntt16_rows_inv(u64* __restrict__ data, const void* __restrict__ tw, const PrimeConst* __restrict__ pcs, RowList list, uint32_t y0) {
     pdl_begin();
@@ -198,7 +216,7 @@ __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
     const ulonglong2* in = reinterpret_cast<const ulonglong2*>(p + 2 * lane);
     u64* s = sm + 2 * lane + 2 * (lane >> 3);
     u64* o = p + 256 * (lane >> 4) + (lane & 15);
-    if (FP) {
+    if constexpr (A == ROW_FP) {
         FpRow r{(const double*)tw + (size_t)pi * N16, pcs[pi].qd, pcs[pi].qinvd};
 #pragma unroll
         for (int j = 0; j < 8; j++) {
@@ -212,7 +230,7 @@ __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
         for (int k = 0; k < 16; k++) o[16 * k] = FpRow::bits(x[k]);      // doubles, |x| <= q/2
     } else {
         const u64 q = pcs[pi].q;
-        IntRow r{(const ulonglong2*)tw + (size_t)pi * N16, q, 2 * q};
+        const IntRow r{(const ulonglong2*)tw + (size_t)pi * N16, q, 2 * q};
 #pragma unroll
         for (int j = 0; j < 8; j++) *reinterpret_cast<ulonglong2*>(s + 72 * j) = in[32 * j];
         __syncwarp();
@@ -225,11 +243,11 @@ __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
 
 int ntt16_launch(fesc_ctx* ctx, u64* data, size_t rows, const RowMap& map, bool inverse, cudaStream_t st, bool in_double,
                  bool out_double, const NttFinish& fin, uint64_t& launches, const InvScale* scale, bool skip_cols) {
-    RowList kind[2];                  // 0: primes below 2^50, 1: the rest
+    RowList kind[2];
     for (RowList& l : kind) l.period = map.period, l.count = 0;
     for (uint32_t i = 0; i < map.period; i++) {
         if (map.prime[i] == 0xFF) continue;
-        RowList& l = kind[ctx->q[map.prime[i]] < FESC_FP_LIMIT ? 0 : 1];
+        RowList& l = kind[ctx->q[map.prime[i]] < FESC_FP_LIMIT ? ROW_FP : ROW_INT];
         l.row[l.count] = (uint8_t)i;
         l.prime[l.count++] = map.prime[i];
     }
@@ -241,19 +259,21 @@ int ntt16_launch(fesc_ctx* ctx, u64* data, size_t rows, const RowMap& map, bool 
             const unsigned n = (unsigned)(total - y0 < 65535 ? total - y0 : 65535);
             const dim3 gc(256 / NTT_COLS, n), gr(128 / NTT_WARPS, n);
             const uint32_t y = (uint32_t)y0;
-            if (f == 0 && !inverse) {
-                if (!skip_cols) launch(ntt16_cols_fwd<true>, gc, COL_THREADS, 0, st, data, ctx->d_twf, ctx->d_pc, l, y, in_double);
-                if (fin.acc) launch(ntt16_rows_fwd<true, true>, gr, ROW_THREADS, 0, st, data, ctx->d_twf, ctx->d_pc, l, y, out_double, fin);
-                else launch(ntt16_rows_fwd<true, false>, gr, ROW_THREADS, 0, st, data, ctx->d_twf, ctx->d_pc, l, y, out_double, fin);
-            } else if (f == 0) {
-                launch(ntt16_rows_inv<true>, gr, ROW_THREADS, 0, st, data, ctx->d_itwf, ctx->d_pc, l, y);
-                launch(ntt16_cols_inv<true>, gc, COL_THREADS, 0, st, data, ctx->d_itwf, ctx->d_pc, l, y, scale);
-            } else if (!inverse) {
-                if (!skip_cols) launch(ntt16_cols_fwd<false>, gc, COL_THREADS, 0, st, data, ctx->d_tw, ctx->d_pc, l, y, 0);
-                launch(ntt16_rows_fwd<false, false>, gr, ROW_THREADS, 0, st, data, ctx->d_tw, ctx->d_pc, l, y, 0, fin);
+            if (f == ROW_FP) {
+                if (inverse) {
+                    launch(ntt16_rows_inv<ROW_FP>, gr, ROW_THREADS, 0, st, data, ctx->d_itwf, ctx->d_pc, l, y);
+                    launch(ntt16_cols_inv<ROW_FP>, gc, COL_THREADS, 0, st, data, ctx->d_itwf, ctx->d_pc, l, y, scale);
+                } else {
+                    if (!skip_cols) launch(ntt16_cols_fwd<ROW_FP>, gc, COL_THREADS, 0, st, data, ctx->d_twf, ctx->d_pc, l, y, in_double);
+                    if (fin.acc) launch(ntt16_rows_fwd<ROW_FP, true>, gr, ROW_THREADS, 0, st, data, ctx->d_twf, ctx->d_pc, l, y, out_double, fin);
+                    else launch(ntt16_rows_fwd<ROW_FP, false>, gr, ROW_THREADS, 0, st, data, ctx->d_twf, ctx->d_pc, l, y, out_double, fin);
+                }
+            } else if (inverse) {
+                launch(ntt16_rows_inv<ROW_INT>, gr, ROW_THREADS, 0, st, data, ctx->d_itw, ctx->d_pc, l, y);
+                launch(ntt16_cols_inv<ROW_INT>, gc, COL_THREADS, 0, st, data, ctx->d_itw, ctx->d_pc, l, y, scale);
             } else {
-                launch(ntt16_rows_inv<false>, gr, ROW_THREADS, 0, st, data, ctx->d_itw, ctx->d_pc, l, y);
-                launch(ntt16_cols_inv<false>, gc, COL_THREADS, 0, st, data, ctx->d_itw, ctx->d_pc, l, y, scale);
+                if (!skip_cols) launch(ntt16_cols_fwd<ROW_INT>, gc, COL_THREADS, 0, st, data, ctx->d_tw, ctx->d_pc, l, y, 0);
+                launch(ntt16_rows_fwd<ROW_INT, false>, gr, ROW_THREADS, 0, st, data, ctx->d_tw, ctx->d_pc, l, y, 0, fin);
             }
             launches += skip_cols ? 1 : 2;
         }

@@ -114,11 +114,14 @@ struct IntRowT {
         for (int k = 0; k < (1 << S); k++) w[k] = tw_load<SHARED>(t + 32 * ((1 << S) - 1 + k));
     }
     __device__ __forceinline__ void one(W& w, uint32_t i) const { w = tw_load<SHARED>(tw + i); }
+    __device__ __forceinline__ u64 canonical(u64 x) const { return csub(csub(x, q2), q); }
     __device__ __forceinline__ T fold(T x) const { return x; }
     static __device__ __forceinline__ u64 bits(T x) { return x; }
     static __device__ __forceinline__ T value(u64 b) { return b; }
 };
 typedef IntRowT<false> IntRow;
+// arithmetic of a launch's rows
+enum { ROW_FP = 0, ROW_INT = 1 };
 
 // Stage S (0..3) of a forward round: distance 8 >> S, twiddles (i0 << S) + j for the j-th group of 16 >> S registers.
 template <int S, class R>
