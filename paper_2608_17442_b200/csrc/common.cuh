@@ -336,6 +336,33 @@ __device__ __forceinline__ uint32_t galois_src(uint32_t t, uint32_t log_n, u64 g
     return __brev((e - 1) >> 1) >> (32 - log_n);
 }
 
+// Where the EVAL-form polynomial being switched is kept: the rows of the extended-digit buffer that belong to a
+// digit's own limbs (row l of digit l / alpha), which the basis extension leaves untouched.  The inner product then
+// reads every (digit, row) from one array.
+struct OwnRows {
+    u64* ext;
+    uint32_t alpha, beta, rows;
+    int as_double;   // rows on primes below 2^50 are kept as doubles with |x| <= q/2 (the FP64 inner product's format)
+};
+__device__ __forceinline__ u64 own_word(const OwnRows& w, u64 v, const PrimeConst& pc) {
+    return (w.as_double && pc.q < FESC_FP_LIMIT) ? (u64)__double_as_longlong(fp_load(v, pc.qd)) : v;
+}
+__device__ __forceinline__ size_t own_index(const OwnRows& w, uint32_t b, uint32_t l, uint32_t N) {
+    return (((size_t)b * w.beta + l / w.alpha) * w.rows + l) * N;
+}
+// Keys of one pass that rotates several ciphertexts by several amounts: polynomial k * nb + b belongs to key k and ciphertext b.
+#define KS_MAX_KEYS 16
+// Optional source of the first pass of an inverse N = 2^16 transform over rows r = polynomial * level + l (period `level`): row l
+// of src + k * key_stride + b * stride, read through the permutation of g[k] (0: none), kept in its own-limb row on the way.
+// Saves the kernel that permuted and copied the polynomial (8 us of a rotation's 184).
+struct NttSource {
+    const u64* src = nullptr;
+    size_t stride = 0, key_stride = 0;
+    uint32_t nb = 1;
+    u64 g[KS_MAX_KEYS] = {};
+    OwnRows own = {};
+};
+
 // Optional epilogue of the last pass of a forward N = 2^16 transform over rows r = bp * level + i (bp = ciphertext * 2 +
 // polynomial, i = data limb, all primes below 2^50): instead of storing the transformed row u, the pass stores the last
 // step of an exact division,  out[b][p][i] = (acc[bp][i] - u) * c_i  (added to what out holds when bit p of add_mask
@@ -354,7 +381,10 @@ struct NttFinish {
     // (instead of a kernel that writes the permuted c0 to `out` first and add_mask bit 0)
     const u64* rot_src = nullptr;    // ciphertext b at rot_src + b * rot_stride, first polynomial [level][N]
     size_t rot_stride = 0;
-    u64 rot_g = 0;
+    u64 rot_g[KS_MAX_KEYS] = {};
+    // several keys: ciphertext index k * nb + b is ciphertext b of key k, at out + k * out_key_stride and rot_src + k * rot_key_stride
+    uint32_t nb = 0x7fffffff;
+    size_t out_key_stride = 0, rot_key_stride = 0;
 };
 
 // internal launchers (ntt.cu)
@@ -365,7 +395,7 @@ struct NttFinish {
 // out_double (forward, N = 2^16 only): such rows are left as doubles with |x| <= q/2 for a consumer that computes in FP64.
 int ntt_launch(fesc_ctx* ctx, u64* d_data, size_t rows, const RowMap& map, bool inverse, cudaStream_t st,
                bool in_double = false, bool out_double = false, const NttFinish* finish = nullptr,
-               const InvScale* scale = nullptr, bool skip_cols = false);
+               const InvScale* scale = nullptr, bool skip_cols = false, const NttSource* source = nullptr);
 // Where twiddle i of a row of N = 2^16 points is kept.  The last four forward stages read, per 512-point block and lane, one
 // twiddle of stage 12, two of stage 13, four and eight: 15 values that lie up to 120 bytes apart between lanes.  They are
 // stored lane by lane within the block instead, in pairs for the FP64 table (16-byte loads, 512 contiguous bytes per warp), one
@@ -378,7 +408,7 @@ static inline uint32_t ntt16_twiddle_slot(uint32_t i, bool pairs) {
 }
 // N = 2^16 kernels (ntt16.cu)
 int ntt16_launch(fesc_ctx* ctx, u64* data, size_t rows, const RowMap& map, bool inverse, cudaStream_t st, bool in_double,
-                 bool out_double, const NttFinish& fin, uint64_t& launches, const InvScale* scale, bool skip_cols);
+                 bool out_double, const NttFinish& fin, uint64_t& launches, const InvScale* scale, bool skip_cols, const NttSource* source);
 // N = 2^10 .. 2^12 (small.cu)
 bool small_ring(const fesc_ctx* ctx);
 int small_init(fesc_ctx* ctx);      // once per context

@@ -38,7 +38,7 @@ extern "C" int fesc_conv(fesc_ctx* ctx, const uint64_t* d_ct_in, const uint64_t*
     cudaStream_t st = (cudaStream_t)stream;
     const size_t ctw = (size_t)2 * level * N, ptw = (size_t)level * N;
     const size_t rot_words = (size_t)2 * taps * blocks * ctw;       // one buffer: [2*taps][blocks] ciphertexts
-    const size_t ks_words = ks_scratch_words(ctx, level, ks_chunk(ctx, blocks));
+    const size_t ks_words = ks_scratch_words(ctx, level, ks_cut_hoisted(ctx, blocks, taps ? 2 * taps : 1));
     const size_t rs_words = (size_t)blocks * 2 * N;
     u64* scratch;
     int rc = ctx_scratch(ctx, (2 * rot_words + (size_t)blocks * ctw + (ks_words > rs_words ? ks_words : rs_words)) * sizeof(u64),

@@ -612,6 +612,14 @@ static size_t packed_group_bytes(size_t image_bytes) {
     return b < most ? b : most;
 }
 
+// key-switch scratch of a projection: baby rotations of `inputs` ciphertexts, giant steps of `outputs`
+static size_t linear_ks_words(const fesc_ctx* ctx, const fesc_bsgs_desc* desc, uint32_t inputs, uint32_t outputs) {
+    const uint32_t level = desc->n_limbs, babies = desc->n1 > 1 ? desc->n1 - 1 : 1, giants = desc->n2 > 1 ? desc->n2 - 1 : 1;
+    const size_t b = ks_scratch_words(ctx, level, desc->hoist ? ks_cut_hoisted(ctx, inputs, babies) : ks_cut_rotate(ctx, inputs, babies));
+    const size_t g = ks_scratch_words(ctx, level, desc->defer ? ks_cut_giant(ctx, outputs, desc->n2) : ks_cut_rotate(ctx, outputs, giants));
+    return b > g ? b : g;
+}
+
 // How a projection on packed diagonals is cut: token blocks per group and output blocks per part of a group.
 struct PackedPlan {
     uint32_t tbg, nb_part;
@@ -639,8 +647,7 @@ static PackedPlan packed_plan(const fesc_ctx* ctx, const fesc_bsgs_desc* desc, u
             PackedPlan p;
             p.tbg = tbg, p.nb_part = nb < nout ? nb : nout;
             const uint32_t parts = (nout + p.nb_part - 1) / p.nb_part;
-            const uint32_t max_batch = sub * gin > tbg * p.nb_part ? sub * gin : tbg * p.nb_part;
-            const size_t ks_words = ks_scratch_words(ctx, level, ks_chunk(ctx, max_batch), desc->defer ? giant_ext_buffers(n2) : 1);
+            const size_t ks_words = linear_ks_words(ctx, desc, sub * gin, tbg * p.nb_part);
             const size_t rs_words = (size_t)(p.nb_part < 16384 ? p.nb_part : 16384) * 2 * N;
             p.rot_words = (size_t)sub * terms * ctw, p.acc_words = (size_t)tbg * p.nb_part * n2 * ctw;
             p.xpk_words = bsgs_packed_bytes(N, level, 2 * tbg, terms) / 8;
@@ -698,11 +705,10 @@ static int linear_packed(fesc_ctx* ctx, const u64* in, const uint8_t* image, con
                                              n1 - 1, ks, st);
                 if (rc != FESC_OK) return rc;
             } else {
-                for (uint32_t q = 1; q < n1; q++) {
-                    rc = rotate_internal(ctx, gin_base, ctw, rot + (size_t)q * ctw, (size_t)n1 * ctw, ns * gin, level,
-                                         desc->baby_key_base + q, ks, st, 0);
-                    if (rc != FESC_OK) return rc;
-                }
+                std::vector<uint32_t> ids;
+                for (uint32_t q = 1; q < n1; q++) ids.push_back(desc->baby_key_base + q);
+                rc = rotate_multi_internal(ctx, gin_base, ctw, 0, rot + ctw, (size_t)n1 * ctw, ctw, ns * gin, level, ids.data(), n1 - 1, ks, st, 0);
+                if (rc != FESC_OK) return rc;
             }
             if ((rc = bsgs_pack_inputs(ctx, rot, xpk + (size_t)(s0 / 4) * tile_bytes, level, ns, terms, st)) != FESC_OK) return rc;
         }
@@ -716,11 +722,10 @@ static int linear_packed(fesc_ctx* ctx, const u64* in, const uint8_t* image, con
                 rc = giant_sum_deferred_internal(ctx, acc, n2, ctw, nt * nb, level, desc->giant_key_base, ks, st);
                 if (rc != FESC_OK) return rc;
             } else {
-                for (uint32_t p = 1; p < n2; p++) {
-                    rc = rotate_internal(ctx, acc + (size_t)p * ctw, (size_t)n2 * ctw, acc, (size_t)n2 * ctw, nt * nb, level,
-                                         desc->giant_key_base + p, ks, st, 1);
-                    if (rc != FESC_OK) return rc;
-                }
+                std::vector<uint32_t> ids;
+                for (uint32_t p = 1; p < n2; p++) ids.push_back(desc->giant_key_base + p);
+                rc = rotate_multi_internal(ctx, acc + ctw, (size_t)n2 * ctw, ctw, acc, (size_t)n2 * ctw, 0, nt * nb, level, ids.data(), n2 - 1, ks, st, 1);
+                if (rc != FESC_OK) return rc;
             }
             for (uint32_t tb = 0; tb < nt; tb++) {      // the outputs of a token block are contiguous, those of a part are not
                 rc = rescale_internal(ctx, acc + (size_t)tb * nb * n2 * ctw, (size_t)n2 * ctw,
@@ -768,8 +773,7 @@ extern "C" int fesc_linear(fesc_ctx* ctx, const uint64_t* d_ct_in, const uint64_
     u64 *scratch = nullptr, *rot = nullptr, *acc = nullptr, *ks = nullptr;
     int rc;
     for (;;) {
-        const uint32_t max_batch = tbg * (gin > nout ? gin : nout);
-        const size_t ks_words = ks_scratch_words(ctx, level, ks_chunk(ctx, max_batch), desc->defer ? giant_ext_buffers(n2) : 1);
+        const size_t ks_words = linear_ks_words(ctx, desc, tbg * gin, tbg * nout);
         const size_t rs_words = (size_t)(tbg * nout < 16384 ? tbg * nout : 16384) * 2 * N;
         const size_t rot_words = (size_t)tbg * gin * n1 * ctw, acc_words = (size_t)tbg * nout * n2 * ctw;
         rc = ctx_scratch(ctx, (rot_words + acc_words + (ks_words > rs_words ? ks_words : rs_words)) * sizeof(u64), &scratch);
@@ -806,11 +810,10 @@ extern "C" int fesc_linear(fesc_ctx* ctx, const uint64_t* d_ct_in, const uint64_
                                          n1 - 1, ks, st);
             if (rc != FESC_OK) return rc;
         } else {
-            for (uint32_t q = 1; q < n1; q++) {
-                rc = rotate_internal(ctx, gin_base, ctw, rot + (size_t)q * ctw, (size_t)n1 * ctw, nt * gin, level,
-                                     desc->baby_key_base + q, ks, st, 0);
-                if (rc != FESC_OK) return rc;
-            }
+            std::vector<uint32_t> ids;
+            for (uint32_t q = 1; q < n1; q++) ids.push_back(desc->baby_key_base + q);
+            rc = rotate_multi_internal(ctx, gin_base, ctw, 0, rot + ctw, (size_t)n1 * ctw, ctw, nt * gin, level, ids.data(), n1 - 1, ks, st, 0);
+            if (rc != FESC_OK) return rc;
         }
         const uint32_t bp_count = nout * n2;
         prof_begin(ctx, PF_BSGS, st);
@@ -879,11 +882,10 @@ extern "C" int fesc_linear(fesc_ctx* ctx, const uint64_t* d_ct_in, const uint64_
             rc = giant_sum_deferred_internal(ctx, acc, n2, ctw, nt * nout, level, desc->giant_key_base, ks, st);
             if (rc != FESC_OK) return rc;
         } else {
-            for (uint32_t p = 1; p < n2; p++) {
-                rc = rotate_internal(ctx, acc + (size_t)p * ctw, (size_t)n2 * ctw, acc, (size_t)n2 * ctw, nt * nout,
-                                     level, desc->giant_key_base + p, ks, st, 1);
-                if (rc != FESC_OK) return rc;
-            }
+            std::vector<uint32_t> ids;
+            for (uint32_t p = 1; p < n2; p++) ids.push_back(desc->giant_key_base + p);
+            rc = rotate_multi_internal(ctx, acc + ctw, (size_t)n2 * ctw, ctw, acc, (size_t)n2 * ctw, 0, nt * nout, level, ids.data(), n2 - 1, ks, st, 1);
+            if (rc != FESC_OK) return rc;
         }
         rc = rescale_internal(ctx, acc, (size_t)n2 * ctw, out + (size_t)tb0 * nout * 2 * (level - 1) * N, nt * nout, level,
                               ks, st);

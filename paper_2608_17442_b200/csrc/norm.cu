@@ -36,7 +36,7 @@ extern "C" int fesc_norm_square(fesc_ctx* ctx, const uint64_t* d_y, uint64_t* d_
     cudaStream_t st = (cudaStream_t)stream;
     const uint32_t N = ctx->N, group = batch < 16 ? batch : 16;
     const size_t ctw = (size_t)2 * n_limbs * N, outw = (size_t)2 * (n_limbs - 1) * N;
-    const size_t ks_words = ks_scratch_words(ctx, n_limbs, ks_chunk(ctx, group));
+    const size_t ks_words = ks_scratch_words(ctx, n_limbs, ks_cut_rotate(ctx, group));
     const size_t rs_words = (size_t)group * 2 * N;
     u64* scratch;
     int rc = ctx_scratch(ctx, ((size_t)group * ctw + (ks_words > rs_words ? ks_words : rs_words)) * sizeof(u64), &scratch);
@@ -71,7 +71,7 @@ extern "C" int fesc_norm_scale(fesc_ctx* ctx, const uint64_t* d_y, const uint64_
     cudaStream_t st = (cudaStream_t)stream;
     const size_t ctw = (size_t)2 * level * N, ctw1 = (size_t)2 * (level - 1) * N, ctw2 = (size_t)2 * (level - 2) * N;
     const uint32_t widest = tbs > blocks ? tbs : blocks;
-    const size_t ks_words = ks_scratch_words(ctx, level, ks_chunk(ctx, widest));
+    const size_t ks_words = ks_scratch_words(ctx, level, ks_cut_rotate(ctx, widest));
     const size_t rs_words = (size_t)widest * 2 * N;
     u64* scratch;
     int rc = ctx_scratch(ctx, ((size_t)2 * tbs * ctw + (size_t)blocks * (ctw + ctw1) + (ks_words > rs_words ? ks_words : rs_words)) *

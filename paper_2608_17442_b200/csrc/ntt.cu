@@ -85,10 +85,10 @@ __global__ void __launch_bounds__(256) ntt_small(u64* __restrict__ data, const u
 }
 
 int ntt_launch(fesc_ctx* ctx, u64* d_data, size_t rows, const RowMap& map, bool inverse, cudaStream_t st, bool in_double,
-               bool out_double, const NttFinish* finish, const InvScale* scale, bool skip_cols) {
+               bool out_double, const NttFinish* finish, const InvScale* scale, bool skip_cols, const NttSource* source) {
     const NttFinish fin = finish ? *finish : NttFinish();
     if (fin.acc && (inverse || ctx->log_n != 16)) return fesc_fail(ctx, FESC_EINVAL, "ntt: the fused epilogue belongs to a forward N = 2^16 transform");
-    if ((scale || skip_cols) && ctx->log_n != 16) return fesc_fail(ctx, FESC_EINVAL, "ntt: N = 2^16 only");
+    if ((scale || skip_cols || source) && ctx->log_n != 16) return fesc_fail(ctx, FESC_EINVAL, "ntt: N = 2^16 only");
     if (rows == 0) return FESC_OK;
     if (rows > 0x7fffffffu) return fesc_fail(ctx, FESC_EINVAL, "ntt: too many rows");
     const ulonglong2* tw = inverse ? ctx->d_itw : ctx->d_tw;
@@ -98,7 +98,7 @@ int ntt_launch(fesc_ctx* ctx, u64* d_data, size_t rows, const RowMap& map, bool 
     prof_begin(ctx, PF_NTT, st);
     uint64_t launches = 0;
     if (ctx->log_n == 16) {
-        const int rc = ntt16_launch(ctx, d_data, rows, map, inverse, st, in_double, out_double, fin, launches, scale, skip_cols);
+        const int rc = ntt16_launch(ctx, d_data, rows, map, inverse, st, in_double, out_double, fin, launches, scale, skip_cols, source);
         if (rc != FESC_OK) return rc;
     } else if (small_ring(ctx)) {
         const int rc = small_ntt_launch(ctx, d_data, rows, map, inverse, st);

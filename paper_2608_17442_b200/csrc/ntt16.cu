@@ -130,10 +130,11 @@ __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
 #pragma unroll
         for (int k = 0; k < 16; k++) x[k] = FpRow::value(in[16 * k]);
         if (FIN) {
-            const uint32_t bp = row / fin.level, i = row - bp * fin.level, b = bp >> 1, pol = bp & 1;
-            prefetch_l2(fin.acc + (size_t)b * fin.acc_stride + ((size_t)pol * fin.acc_rows + i) * N16 + blk * 512 + 16 * lane);
+            const uint32_t bp = row / fin.level, i = row - bp * fin.level, ct = bp >> 1, pol = bp & 1, k = ct / fin.nb, b = ct - k * fin.nb;
+            prefetch_l2(fin.acc + (size_t)ct * fin.acc_stride + ((size_t)pol * fin.acc_rows + i) * N16 + blk * 512 + 16 * lane);
             if (fin.rot_src && !pol)
-                prefetch_l2(fin.rot_src + (size_t)b * fin.rot_stride + (size_t)i * N16 + (galois_src(blk * 512, 16, fin.rot_g) & ~511u) + 16 * lane);
+                prefetch_l2(fin.rot_src + k * fin.rot_key_stride + b * fin.rot_stride + (size_t)i * N16 +
+                            (galois_src(blk * 512, 16, fin.rot_g[k]) & ~511u) + 16 * lane);
         }
         fwd_rows(r, x, sm, blk, lane);
         const double q = r.q, qinv = r.qinv;
@@ -150,10 +151,11 @@ __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
         }
         // (acc - u) c (+ sigma_g(c0)) (+ what the output holds); |acc - u| stays below 5.4q, the lazy product below 1.6q, so
         // every sum is exact.  Rows of the buffer: row = bp * level + i.
-        const uint32_t bp = row / fin.level, i = row - bp * fin.level, b = bp >> 1, pol = bp & 1;
-        const u64* acc = fin.acc + (size_t)b * fin.acc_stride + ((size_t)pol * fin.acc_rows + i) * N16;
-        u64* out = fin.out + (size_t)b * fin.out_stride + ((size_t)pol * fin.level + i) * N16;
-        const u64* rot = fin.rot_src && !pol ? fin.rot_src + (size_t)b * fin.rot_stride + (size_t)i * N16 : nullptr;
+        const uint32_t bp = row / fin.level, i = row - bp * fin.level, ct = bp >> 1, pol = bp & 1, kk = ct / fin.nb, b = ct - kk * fin.nb;
+        const u64* acc = fin.acc + (size_t)ct * fin.acc_stride + ((size_t)pol * fin.acc_rows + i) * N16;
+        u64* out = fin.out + kk * fin.out_key_stride + b * fin.out_stride + ((size_t)pol * fin.level + i) * N16;
+        const u64* rot = fin.rot_src && !pol ? fin.rot_src + kk * fin.rot_key_stride + b * fin.rot_stride + (size_t)i * N16 : nullptr;
+        const u64 rot_g = fin.rot_g[kk];
         if (!DBG_REGION(acc, N16 * sizeof(u64)) || !DBG_REGION(out, N16 * sizeof(u64)) || (rot && !DBG_REGION(rot, N16 * sizeof(u64)))) return;
         const double cinv = fin.cinv[i];
         const bool add = (fin.add_mask >> pol) & 1;
@@ -166,7 +168,7 @@ __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
             u64 w[8];
             if (rot) {
 #pragma unroll
-                for (int j = 0; j < 8; j++) w[j] = rot[galois_src(blk * 512 + 2 * lane + 64 * (h + (j >> 1)) + (j & 1), 16, fin.rot_g)];
+                for (int j = 0; j < 8; j++) w[j] = rot[galois_src(blk * 512 + 2 * lane + 64 * (h + (j >> 1)) + (j & 1), 16, rot_g)];
             }
 #pragma unroll
             for (int j = h; j < h + 4; j++) {
@@ -202,9 +204,10 @@ __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
     }
 }
 
-template <int A>
+template <int A, bool SRC>
 __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
-    ntt16_rows_inv(u64* __restrict__ data, const void* __restrict__ tw, const PrimeConst* __restrict__ pcs, RowList list, uint32_t y0) {
+    ntt16_rows_inv(u64* __restrict__ data, const void* __restrict__ tw, const PrimeConst* __restrict__ pcs, RowList list, uint32_t y0,
+                   NttSource src) {
     pdl_begin();
     __shared__ __align__(16) u64 sm_all[NTT_WARPS * ROW_SMEM];
     uint32_t pi;
@@ -213,15 +216,33 @@ __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
     u64* sm = sm_all + warp * ROW_SMEM;
     u64* p = data + (size_t)row * N16 + (size_t)blk * 512;
     if (!DBG_REGION(p, 512 * sizeof(u64))) return;
-    const ulonglong2* in = reinterpret_cast<const ulonglong2*>(p + 2 * lane);
+    const u64* in = p + 2 * lane;
+    uint32_t at = 0;                  // SRC: the words come from the permuted block that starts here
+    u64* own = nullptr;
+    u64 g = 0;
+    if (SRC) {                        // rows of the buffer: row = polynomial * period + limb
+        const uint32_t poly = row / list.period, l = row - poly * list.period, k = poly / src.nb, b = poly - k * src.nb;
+        g = src.g[k];
+        in = src.src + k * src.key_stride + b * src.stride + (size_t)l * N16;
+        own = src.own.ext + own_index(src.own, poly, l, N16) + blk * 512 + 2 * lane;
+        if (!DBG_REGION(in, N16 * sizeof(u64)) || !DBG_REGION(own - 2 * lane, 512 * sizeof(u64))) return;
+        at = blk * 512 + 2 * lane;
+    }
+    auto pair = [&](int j) {
+        if (!SRC) return *reinterpret_cast<const ulonglong2*>(in + 64 * j);
+        if (!g) return *reinterpret_cast<const ulonglong2*>(in + at + 64 * j);
+        return make_ulonglong2(in[galois_src(at + 64 * j, 16, g)], in[galois_src(at + 64 * j + 1, 16, g)]);
+    };
     u64* s = sm + 2 * lane + 2 * (lane >> 3);
     u64* o = p + 256 * (lane >> 4) + (lane & 15);
     if constexpr (A == ROW_FP) {
         FpRow r{(const double*)tw + (size_t)pi * N16, pcs[pi].qd, pcs[pi].qinvd};
 #pragma unroll
         for (int j = 0; j < 8; j++) {
-            const ulonglong2 v = in[32 * j];
-            *reinterpret_cast<ulonglong2*>(s + 72 * j) = make_ulonglong2(FpRow::bits(fp_load(v.x, r.q)), FpRow::bits(fp_load(v.y, r.q)));
+            ulonglong2 v = pair(j);
+            v = make_ulonglong2(FpRow::bits(fp_load(v.x, r.q)), FpRow::bits(fp_load(v.y, r.q)));
+            *reinterpret_cast<ulonglong2*>(s + 72 * j) = v;
+            if (SRC) *reinterpret_cast<ulonglong2*>(own + 64 * j) = v;
         }
         __syncwarp();
         double x[16];
@@ -232,7 +253,11 @@ __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
         const u64 q = pcs[pi].q;
         const IntRow r{(const ulonglong2*)tw + (size_t)pi * N16, q, 2 * q};
 #pragma unroll
-        for (int j = 0; j < 8; j++) *reinterpret_cast<ulonglong2*>(s + 72 * j) = in[32 * j];
+        for (int j = 0; j < 8; j++) {
+            const ulonglong2 v = pair(j);
+            *reinterpret_cast<ulonglong2*>(s + 72 * j) = v;
+            if (SRC) *reinterpret_cast<ulonglong2*>(own + 64 * j) = v;
+        }
         __syncwarp();
         u64 x[16];
         inv_rows(r, x, sm, blk, lane);
@@ -242,7 +267,7 @@ __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
 }
 
 int ntt16_launch(fesc_ctx* ctx, u64* data, size_t rows, const RowMap& map, bool inverse, cudaStream_t st, bool in_double,
-                 bool out_double, const NttFinish& fin, uint64_t& launches, const InvScale* scale, bool skip_cols) {
+                 bool out_double, const NttFinish& fin, uint64_t& launches, const InvScale* scale, bool skip_cols, const NttSource* source) {
     RowList kind[2];
     for (RowList& l : kind) l.period = map.period, l.count = 0;
     for (uint32_t i = 0; i < map.period; i++) {
@@ -252,6 +277,7 @@ int ntt16_launch(fesc_ctx* ctx, u64* data, size_t rows, const RowMap& map, bool 
         l.prime[l.count++] = map.prime[i];
     }
     const size_t reps = rows / map.period;
+    const NttSource src = source ? *source : NttSource();
     for (int f = 0; f < 2; f++) {
         const RowList& l = kind[f];
         const size_t total = reps * l.count;
@@ -261,7 +287,8 @@ int ntt16_launch(fesc_ctx* ctx, u64* data, size_t rows, const RowMap& map, bool 
             const uint32_t y = (uint32_t)y0;
             if (f == ROW_FP) {
                 if (inverse) {
-                    launch(ntt16_rows_inv<ROW_FP>, gr, ROW_THREADS, 0, st, data, ctx->d_itwf, ctx->d_pc, l, y);
+                    launch(source ? ntt16_rows_inv<ROW_FP, true> : ntt16_rows_inv<ROW_FP, false>, gr, ROW_THREADS, 0, st, data, ctx->d_itwf, ctx->d_pc, l,
+                           y, src);
                     launch(ntt16_cols_inv<ROW_FP>, gc, COL_THREADS, 0, st, data, ctx->d_itwf, ctx->d_pc, l, y, scale);
                 } else {
                     if (!skip_cols) launch(ntt16_cols_fwd<ROW_FP>, gc, COL_THREADS, 0, st, data, ctx->d_twf, ctx->d_pc, l, y, in_double);
@@ -269,7 +296,8 @@ int ntt16_launch(fesc_ctx* ctx, u64* data, size_t rows, const RowMap& map, bool 
                     else launch(ntt16_rows_fwd<ROW_FP, false>, gr, ROW_THREADS, 0, st, data, ctx->d_twf, ctx->d_pc, l, y, out_double, fin);
                 }
             } else if (inverse) {
-                launch(ntt16_rows_inv<ROW_INT>, gr, ROW_THREADS, 0, st, data, ctx->d_itw, ctx->d_pc, l, y);
+                launch(source ? ntt16_rows_inv<ROW_INT, true> : ntt16_rows_inv<ROW_INT, false>, gr, ROW_THREADS, 0, st, data, ctx->d_itw, ctx->d_pc, l, y,
+                       src);
                 launch(ntt16_cols_inv<ROW_INT>, gc, COL_THREADS, 0, st, data, ctx->d_itw, ctx->d_pc, l, y, scale);
             } else {
                 if (!skip_cols) launch(ntt16_cols_fwd<ROW_INT>, gc, COL_THREADS, 0, st, data, ctx->d_tw, ctx->d_pc, l, y, 0);

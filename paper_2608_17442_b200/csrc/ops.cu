@@ -74,21 +74,6 @@ extern "C" int fesc_intt(fesc_ctx* ctx, uint64_t* d_data, uint32_t batch, uint32
 // c0 goes to out0 (the result's first polynomial), c1 goes to BOTH d (kept in EVAL form for
 // the digit's own limbs) and dcoef (transformed in place afterwards).
 // ---------------------------------------------------------------------------------------
-// Where the EVAL-form polynomial being switched is kept: the rows of the extended-digit buffer that belong to a
-// digit's own limbs (row l of digit l / alpha), which the basis extension leaves untouched.  The inner product then
-// reads every (digit, row) from one array.
-struct OwnRows {
-    u64* ext;
-    uint32_t alpha, beta, rows;
-    int as_double;   // rows on primes below 2^50 are kept as doubles with |x| <= q/2 (the FP64 inner product's format)
-};
-__device__ __forceinline__ u64 own_word(const OwnRows& w, u64 v, const PrimeConst& pc) {
-    return (w.as_double && pc.q < FESC_FP_LIMIT) ? (u64)__double_as_longlong(fp_load(v, pc.qd)) : v;
-}
-__device__ __forceinline__ size_t own_index(const OwnRows& w, uint32_t b, uint32_t l, uint32_t N) {
-    return (((size_t)b * w.beta + l / w.alpha) * w.rows + l) * N;
-}
-struct KsScratch;
 __global__ void __launch_bounds__(256) k_autom_ct(const u64* __restrict__ in, size_t in_stride, u64* __restrict__ out0,
                                                   size_t out_stride, OwnRows d, u64* __restrict__ dcoef,
                                                   uint32_t log_n, uint32_t level, u64 g,
@@ -237,16 +222,18 @@ __global__ void __launch_bounds__(256) k_modup(const u64* __restrict__ dcoef, u6
 // PATH 0: the row's prime decides at run time; 1: the caller guarantees primes below 2^50 on rows
 // [row0, row0 + gridDim.y) (exact FP64 products only); 2: the caller sends those rows to the 128-bit integer sums.
 template <int BT, int PATH>
-__global__ void __launch_bounds__(256, INNER_MINB) k_inner(InnerSrcs S, u64* __restrict__ acc,
+__global__ void __launch_bounds__(256, INNER_MINB) k_inner(InnerSrcs S, u64* acc,
                                                const PrimeConst* __restrict__ pcs, uint32_t N, uint32_t level,
                                                uint32_t n_q, uint32_t K, uint32_t alpha, uint32_t beta,
                                                uint32_t batch, uint32_t log_n, int accumulate, uint32_t row0,
-                                               int x_double) {
+                                               int x_double, uint32_t sep) {
+    // sep != 0: the sources are not summed; source s has its own accumulators (s * batch ciphertexts on), blockIdx.z = s * sep + tile
     pdl_begin();
     const uint32_t c = blockIdx.x * blockDim.x + threadIdx.x;
-    const uint32_t t = row0 + blockIdx.y, b0 = blockIdx.z * BT;
+    const uint32_t t = row0 + blockIdx.y, s0 = sep ? blockIdx.z / sep : 0, b0 = (blockIdx.z - s0 * sep) * BT;
     if (c >= N) return;
     const uint32_t rows = level + K, np = n_q + K;
+    acc += (size_t)s0 * batch * 2 * rows * N;
     const uint32_t pt = t < level ? t : n_q + (t - level);
     // operand words of one digit: key (b, a) and the BT ciphertext words; clamped indices keep loads valid.
     // All addresses are a per-thread base plus a multiple of one stride (no per-load index products).
@@ -273,7 +260,7 @@ __global__ void __launch_bounds__(256, INNER_MINB) k_inner(InnerSrcs S, u64* __r
 #endif
     // the (source, digit) whose words are requested next; hoisted rotations: the automorphism acts on the extended
     // digits, i.e. they are read at pi_g(c)
-    uint32_t sn = 0, jn = 0;
+    uint32_t sn = s0, jn = 0;
     const u64* kp;
     const u64* xp[BT];
     auto setup = [&](uint32_t s) {
@@ -296,8 +283,8 @@ __global__ void __launch_bounds__(256, INNER_MINB) k_inner(InnerSrcs S, u64* __r
             if (++sn < S.n) setup(sn);
         }
     };
-    const uint32_t total = S.n * beta;
-    setup(0);
+    const uint32_t total = (sep ? 1 : S.n) * beta;
+    setup(s0);
     if (PATH == 1 || (PATH == 0 && pcs[pt].q < FESC_FP_LIMIT)) {
         // exact FP64 products of canonical words (both below q): every product is below 0.875q, so a running sum of
         // at most q/2 plus 7 terms stays below 2^53 = 8q; longer sums are folded back after every 7th term.  The next digit's words
@@ -392,6 +379,88 @@ __global__ void __launch_bounds__(256, INNER_MINB) k_inner(InnerSrcs S, u64* __r
                 if (accumulate) r0 = addmod(r0, *o0, pc.q), r1 = addmod(r1, *o1, pc.q);
                 *o0 = r0;
                 *o1 = r1;
+            }
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------------------
+// Inner products of ONE converted polynomial per ciphertext with several keys (hoisted rotations), N = 2^16:
+//   acc[k][b][p][t] = sum_j ext[b][j][t][pi_k(.)] * key_k[j][p][t].
+// pi_k maps aligned blocks to aligned blocks, so a CTA that owns one block of the converted rows of every ciphertext holds in
+// shared memory all that any key needs of it, and writes block pi_k^-1 of every accumulator.  The converted digits, 84 MiB per
+// ciphertext at 24 limbs, are then read once per pass of keys instead of once per key.
+// Thread = one coefficient and every fourth ciphertext: the 2 beta key words of a coefficient stay in registers meanwhile.
+// ---------------------------------------------------------------------------------------
+#define IS_BLK 64                 // coefficients per CTA
+#define IS_MAX_DIGITS 8
+struct InnerKeys {
+    const u64* key[KS_MAX_KEYS];
+    u64 g[KS_MAX_KEYS], ginv[KS_MAX_KEYS];
+    uint32_t n;
+};
+template <int BETA, bool FP>
+__global__ void __launch_bounds__(256, 4) k_inner_shared(const u64* __restrict__ ext, InnerKeys keys, u64* __restrict__ acc,
+                                                         const PrimeConst* __restrict__ pcs, uint32_t level, uint32_t n_q, uint32_t K,
+                                                         uint32_t batch, uint32_t row0) {
+    pdl_begin();
+    constexpr uint32_t N = 65536;
+    extern __shared__ __align__(16) u64 sx[];                    // [batch][BETA][IS_BLK]
+    const uint32_t tid = threadIdx.x, i = tid % IS_BLK, part = tid / IS_BLK, blk = blockIdx.x, t = row0 + blockIdx.y;
+    const uint32_t rows = level + K, np = n_q + K, pt = t < level ? t : n_q + (t - level);
+#ifdef FESC_DEBUG_BOUNDS
+    {   // the same outcome for every thread of the CTA (a barrier follows)
+        bool ok = true;
+        for (uint32_t r = 0; r < batch * BETA && ok; r++) ok = DBG_REGION(ext + ((size_t)r * rows + t) * N + blk * IS_BLK, IS_BLK * sizeof(u64));
+        for (uint32_t k = 0; k < keys.n && ok; k++) {
+            for (uint32_t j = 0; j < 2 * BETA && ok; j++) ok = DBG_REGION(keys.key[k] + ((size_t)j * np + pt) * N, N * sizeof(u64));
+            for (uint32_t b = 0; b < 2 * batch && ok; b++) ok = DBG_REGION(acc + (((size_t)k * batch * 2 + b) * rows + t) * N, N * sizeof(u64));
+        }
+        if (!ok) return;
+    }
+#endif
+    for (uint32_t r = tid / 32; r < batch * BETA; r += 8)        // a warp copies one row's block, 16 bytes per lane
+        *reinterpret_cast<ulonglong2*>(sx + r * IS_BLK + 2 * (tid % 32)) =
+            *reinterpret_cast<const ulonglong2*>(ext + ((size_t)r * rows + t) * N + blk * IS_BLK + 2 * (tid % 32));
+    __syncthreads();
+    const PrimeConst& pc = pcs[pt];
+    const double q = pc.qd, qinv = pc.qinvd;
+#pragma unroll 1
+    for (uint32_t k = 0; k < keys.n; k++) {
+        const uint32_t c = (galois_src(blk * IS_BLK, 16, keys.ginv[k]) & ~(IS_BLK - 1u)) + i;      // output coefficient
+        const u64* w = keys.key[k] + (size_t)pt * N + c;
+        const u64* x = sx + (galois_src(c, 16, keys.g[k]) & (IS_BLK - 1u));
+        u64 kw[2 * BETA];
+#pragma unroll
+        for (int j = 0; j < 2 * BETA; j++) kw[j] = __ldg(w + (size_t)j * np * N);
+        u64* o = acc + ((size_t)k * batch * 2 * rows + t) * N + c;
+        if (FP) {
+            double kd[2 * BETA];
+#pragma unroll
+            for (int j = 0; j < 2 * BETA; j++) kd[j] = fp_from_u64(kw[j]);
+            for (uint32_t b = part; b < batch; b += 256 / IS_BLK) {
+                double f0 = 0.0, f1 = 0.0;
+#pragma unroll
+                for (int j = 0; j < BETA; j++) {                 // |x| <= q/2: every product below 0.875 q, at most 7 and a rest
+                    const double xd = __longlong_as_double((long long)x[(b * BETA + j) * IS_BLK]);
+                    f0 += fp_modmul(xd, kd[2 * j], q, qinv);
+                    f1 += fp_modmul(xd, kd[2 * j + 1], q, qinv);
+                    if (j == 6) f0 = fp_reduce(f0, q, qinv), f1 = fp_reduce(f1, q, qinv);
+                }
+                o[(size_t)(2 * b) * rows * N] = fp_store(f0, q, qinv);
+                o[(size_t)(2 * b + 1) * rows * N] = fp_store(f1, q, qinv);
+            }
+        } else {
+            for (uint32_t b = part; b < batch; b += 256 / IS_BLK) {
+                acc128 a0{0, 0}, a1{0, 0};                       // at most 8 products below 2^124
+#pragma unroll
+                for (int j = 0; j < BETA; j++) {
+                    const u64 xv = x[(b * BETA + j) * IS_BLK];
+                    mac128(a0, xv, kw[2 * j]);
+                    mac128(a1, xv, kw[2 * j + 1]);
+                }
+                o[(size_t)(2 * b) * rows * N] = reduce128(a0.hi, a0.lo, pc);
+                o[(size_t)(2 * b + 1) * rows * N] = reduce128(a1.hi, a1.lo, pc);
             }
         }
     }
@@ -716,7 +785,7 @@ __global__ void __launch_bounds__(256) k_moddown_finish(const u64* __restrict__ 
 
 // Steps 1-3 of the key switch: ws.dcoef -> COEFF, digit-wise basis extension into ws.ext, NTT of the
 // converted rows.  The result (ws.ext, own-limb rows included) can serve several keys (hoisted rotations).
-static int ks_decompose(fesc_ctx* ctx, const KsScratch& ws, uint32_t level, uint32_t batch, cudaStream_t st) {
+static int ks_decompose(fesc_ctx* ctx, const KsScratch& ws, uint32_t level, uint32_t batch, cudaStream_t st, const NttSource* source = nullptr) {
     const uint32_t N = ctx->N, K = ctx->n_p, nq = ctx->n_q, alpha = ctx->alpha;
     const uint32_t beta = (level + alpha - 1) / alpha, rows = level + K;
     const uint32_t gx = (N + 255) / 256;
@@ -728,7 +797,7 @@ static int ks_decompose(fesc_ctx* ctx, const KsScratch& ws, uint32_t level, uint
     for (uint32_t i = 0; i < level; i++) m.prime[i] = (uint8_t)i;
     const bool fused = modup16_supported(ctx, level);
     if ((rc = ntt_launch(ctx, ws.dcoef, (size_t)batch * level, m, true, st, false, false, nullptr,
-                         fused ? ctx->tabs.d_up_scale + (size_t)(level - 1) * nq : nullptr)) != FESC_OK)
+                         fused ? ctx->tabs.d_up_scale + (size_t)(level - 1) * nq : nullptr, false, source)) != FESC_OK)
         return rc;
     // 2. ModUp, 3. NTT of the converted rows
     if (beta * rows > sizeof(RowMap::prime)) return fesc_fail(ctx, FESC_EINVAL, "key switch: too many digit rows");
@@ -766,26 +835,33 @@ static int ks_decompose(fesc_ctx* ctx, const KsScratch& ws, uint32_t level, uint
     return FESC_OK;
 }
 
+// data rows on primes below 2^50, special rows above
+static bool rows_split(const fesc_ctx* ctx, uint32_t level) {
+    bool split = true;
+    for (uint32_t i = 0; i < level; i++) split = split && ctx->q[i] < FESC_FP_LIMIT;
+    for (uint32_t k = 0; k < ctx->n_p; k++) split = split && ctx->q[ctx->n_q + k] >= FESC_FP_LIMIT;
+    return split;
+}
 // Step 4: inner products of the sources `S` (converted digits, key, Galois element each) summed into ws.acc;
-// accumulate != 0 adds to what ws.acc holds (sums over several passes before one division by P); last: no further pass follows.
+// accumulate != 0 adds to what ws.acc holds (sums over several passes before one division by P); last: no further pass follows;
+// separate: the sources are not summed, source s has its own batch of accumulators.
 static int ks_inner_multi(fesc_ctx* ctx, const KsScratch& ws, const InnerSrcs& S, uint32_t level, uint32_t batch,
-                          cudaStream_t st, int accumulate, int last = 1) {
+                          cudaStream_t st, int accumulate, int last = 1, bool separate = false) {
     if (small_ring(ctx)) return small_inner(ctx, ws, S, level, batch, st, accumulate, last);
     const uint32_t N = ctx->N, K = ctx->n_p, nq = ctx->n_q, alpha = ctx->alpha;
     const uint32_t beta = (level + alpha - 1) / alpha, rows = level + K;
     const uint32_t gx = (N + 255) / 256;
     prof_begin(ctx, PF_INNER, st);
-    const bool use_tma = S.n == 1 && getenv("FESC_INNER_TMA") != nullptr;   // read per call so a test can switch it
+    const bool use_tma = S.n == 1 && !separate && getenv("FESC_INNER_TMA") != nullptr;   // read per call so a test can switch it
 #define INNER(BT_, PATH_, ROW0_, NROWS_)                                                                        \
     do {                                                                                                        \
-        dim3 gd(gx, NROWS_, (batch + BT_ - 1) / BT_);                                                           \
+        const uint32_t tiles = (batch + BT_ - 1) / BT_;                                                         \
+        dim3 gd(gx, NROWS_, tiles * (separate ? S.n : 1));                                                      \
         launch(k_inner<BT_, PATH_>, gd, 256, 0, st, S, ws.acc, ctx->d_pc, N, level, nq, K, alpha, beta, batch,     \
-                                                ctx->log_n, accumulate, ROW0_, ctx->log_n == 16);              \
+                                                ctx->log_n, accumulate, ROW0_, ctx->log_n == 16, separate ? tiles : 0u); \
     } while (0)
     // data rows on primes below 2^50 and special rows above: one launch per kind, each compiled for its arithmetic
-    bool split = true;
-    for (uint32_t i = 0; i < level; i++) split = split && ctx->q[i] < FESC_FP_LIMIT;
-    for (uint32_t k = 0; k < K; k++) split = split && ctx->q[nq + k] >= FESC_FP_LIMIT;
+    const bool split = rows_split(ctx, level);
     if (use_tma && N % 256 == 0 && beta <= 8 && batch >= 3) {   // 128-bit sums of <= 8 products below 2^124 cannot wrap
         const uint32_t n_tiles = rows * (N >> 8) * ((batch + 3) / 4);
         const size_t smem = (size_t)2 * beta * 6 * 2048 + 16;
@@ -821,6 +897,71 @@ static int ks_inner(fesc_ctx* ctx, const KsScratch& ws, const EvalKey& key, uint
     return ks_inner_multi(ctx, ws, S, level, batch, st, accumulate);
 }
 
+static u64 galois_inverse(u64 g, uint32_t log_n) {      // modulo 2N, g odd: Newton's iteration doubles the correct bits
+    u64 x = g;
+    for (int i = 0; i < 5; i++) x *= 2 - g * x;
+    return x & ((2ull << log_n) - 1);
+}
+template <int BETA>
+static int inner_shared_launch(fesc_ctx* ctx, const KsScratch& ws, const InnerKeys& ik, uint32_t level, uint32_t batch, cudaStream_t st) {
+    const size_t smem = (size_t)batch * BETA * IS_BLK * sizeof(u64);
+    auto fp = k_inner_shared<BETA, true>;
+    auto in = k_inner_shared<BETA, false>;
+    FESC_CHECK_CUDA(ctx, cudaFuncSetAttribute(fp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    FESC_CHECK_CUDA(ctx, cudaFuncSetAttribute(in, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    launch(fp, dim3(65536 / IS_BLK, level), 256, smem, st, ws.ext, ik, ws.acc, ctx->d_pc, level, ctx->n_q, ctx->n_p, batch, 0u);
+    launch(in, dim3(65536 / IS_BLK, ctx->n_p), 256, smem, st, ws.ext, ik, ws.acc, ctx->d_pc, level, ctx->n_q, ctx->n_p, batch, level);
+    return FESC_OK;
+}
+// Keys of a pass: Galois elements and key words
+struct KsKeys {
+    uint32_t n;
+    u64 g[KS_MAX_KEYS];
+    const u64* key[KS_MAX_KEYS];
+};
+static int ks_keys(fesc_ctx* ctx, const char* who, const uint32_t* ids, uint32_t n, KsKeys& keys) {
+    keys.n = n;
+    for (uint32_t k = 0; k < n; k++) {
+        auto it = ctx->keys.find(ids[k]);
+        if (it == ctx->keys.end() || ids[k] == FESC_RELIN_KEY_ID)
+            return fesc_fail(ctx, FESC_ENOKEY, std::string(who) + ": no Galois key " + std::to_string(ids[k]));
+        keys.g[k] = it->second.g, keys.key[k] = it->second.d_key;
+    }
+    return FESC_OK;
+}
+// Step 4 for hoisted rotations: accumulators [key][batch] of one converted polynomial per ciphertext.  Two keys are enough for the
+// shared reading to pay (one key: the plain kernel); N = 2^16, up to 8 digits and 16 ciphertexts (64 KB of shared memory).
+static int ks_inner_hoisted(fesc_ctx* ctx, const KsScratch& ws, const KsKeys& keys, uint32_t k0, uint32_t n, uint32_t level, uint32_t batch,
+                            cudaStream_t st) {
+    const uint32_t beta = (level + ctx->alpha - 1) / ctx->alpha;
+    if (n < 2 || ctx->log_n != 16 || beta > IS_MAX_DIGITS || batch > 16 || !rows_split(ctx, level)) {
+        InnerSrcs S;
+        S.n = n;
+        for (uint32_t k = 0; k < n; k++) S.s[k] = InnerSrc{ws.ext, keys.key[k0 + k], keys.g[k0 + k]};
+        return ks_inner_multi(ctx, ws, S, level, batch, st, 0, 1, n > 1);
+    }
+    InnerKeys ik;
+    ik.n = n;
+    for (uint32_t k = 0; k < n; k++) ik.key[k] = keys.key[k0 + k], ik.g[k] = keys.g[k0 + k], ik.ginv[k] = galois_inverse(ik.g[k], 16);
+    prof_begin(ctx, PF_INNER, st);
+    int rc = FESC_OK;
+    switch (beta) {
+        case 1: rc = inner_shared_launch<1>(ctx, ws, ik, level, batch, st); break;
+        case 2: rc = inner_shared_launch<2>(ctx, ws, ik, level, batch, st); break;
+        case 3: rc = inner_shared_launch<3>(ctx, ws, ik, level, batch, st); break;
+        case 4: rc = inner_shared_launch<4>(ctx, ws, ik, level, batch, st); break;
+        case 5: rc = inner_shared_launch<5>(ctx, ws, ik, level, batch, st); break;
+        case 6: rc = inner_shared_launch<6>(ctx, ws, ik, level, batch, st); break;
+        case 7: rc = inner_shared_launch<7>(ctx, ws, ik, level, batch, st); break;
+        default: rc = inner_shared_launch<8>(ctx, ws, ik, level, batch, st); break;
+    }
+    if (rc != FESC_OK) return rc;
+    prof_end(ctx, PF_INNER, st, 2);
+    FESC_CHECK_CUDA(ctx, cudaGetLastError());
+    ctx->counters[1] += (uint64_t)batch * n;
+    return FESC_OK;
+}
+
 // Step 5: division of ws.acc by P; the result is ADDED to out[b][p] when bit p of add_mask is set, else stored.
 // whether the last pass of the forward transform finishes the division (N = 2^16 with every data prime below 2^50, small rings)
 static bool moddown_fused(const fesc_ctx* ctx, uint32_t level) {
@@ -829,11 +970,18 @@ static bool moddown_fused(const fesc_ctx* ctx, uint32_t level) {
     for (uint32_t i = 0; i < level; i++) fuse = fuse && ctx->q[i] < FESC_FP_LIMIT;
     return fuse;
 }
-// rot_src != nullptr (only when moddown_fused): out[b][0] also receives sigma_g(c0) of the ciphertext at
-// rot_src + b * rot_stride, read through the permutation by the fused epilogue
+// rot.src != nullptr (only when moddown_fused): out[b][0] also receives sigma_g(c0) of the ciphertext at
+// rot.src + b * rot.stride, read through the permutation by the fused epilogue.  Several keys (N = 2^16 only): accumulator k * batch + b
+// belongs to out + k * key_stride + b * out_stride; with key_stride 0 the keys are added one after the other.
+struct KsRot {
+    const u64* src = nullptr;
+    size_t stride = 0, key_stride = 0;
+    const u64* g = nullptr;
+};
 static int ks_moddown(fesc_ctx* ctx, const KsScratch& ws, uint32_t level, uint32_t batch, u64* out, size_t out_stride,
-                      int add_mask, cudaStream_t st, const u64* rot_src = nullptr, size_t rot_stride = 0, u64 rot_g = 0) {
-    if (small_ring(ctx)) return small_moddown(ctx, ws, level, batch, out, out_stride, add_mask, st, rot_src, rot_stride, rot_g);
+                      int add_mask, cudaStream_t st, const KsRot& rot = KsRot(), uint32_t n_keys = 1, size_t key_stride = 0) {
+    if (small_ring(ctx)) return small_moddown(ctx, ws, level, batch, out, out_stride, add_mask, st, rot.src, rot.stride, rot.src ? rot.g[0] : 0);
+    const uint32_t polys = batch * n_keys;
     const uint32_t N = ctx->N, K = ctx->n_p, nq = ctx->n_q;
     const uint32_t rows = level + K;
     const uint32_t gx = (N + 255) / 256;
@@ -841,25 +989,32 @@ static int ks_moddown(fesc_ctx* ctx, const KsScratch& ws, uint32_t level, uint32
     RowMap m;
     m.period = rows;
     for (uint32_t t = 0; t < rows; t++) m.prime[t] = t < level ? 0xFF : (uint8_t)(nq + (t - level));
-    if ((rc = ntt_launch(ctx, ws.acc, (size_t)batch * 2 * rows, m, true, st)) != FESC_OK) return rc;
+    if ((rc = ntt_launch(ctx, ws.acc, (size_t)polys * 2 * rows, m, true, st)) != FESC_OK) return rc;
     prof_begin(ctx, PF_MODDOWN, st);
     if (bconv_supported(ctx, level))
-        moddown_conv_imma_launch(ctx, ws.acc, ws.u, level, batch, ctx->log_n == 16, st);
+        moddown_conv_imma_launch(ctx, ws.acc, ws.u, level, polys, ctx->log_n == 16, st);
     else if (N % (256 * KS_VEC) == 0)
-        launch(k_moddown_conv<KS_VEC>, dim3(N / (256 * KS_VEC), batch * 2), 256, 0, st, ws.acc, ws.u, ctx->tabs.d_moddown, ctx->d_pc, N, level, nq, K, ctx->log_n == 16);
+        launch(k_moddown_conv<KS_VEC>, dim3(N / (256 * KS_VEC), polys * 2), 256, 0, st, ws.acc, ws.u, ctx->tabs.d_moddown, ctx->d_pc, N, level, nq, K, ctx->log_n == 16);
     else
-        launch(k_moddown_conv<1>, dim3(gx, batch * 2), 256, 0, st, ws.acc, ws.u, ctx->tabs.d_moddown, ctx->d_pc, N, level, nq, K, ctx->log_n == 16);
+        launch(k_moddown_conv<1>, dim3(gx, polys * 2), 256, 0, st, ws.acc, ws.u, ctx->tabs.d_moddown, ctx->d_pc, N, level, nq, K, ctx->log_n == 16);
     prof_end(ctx, PF_MODDOWN, st);
     m.period = level;
     for (uint32_t i = 0; i < level; i++) m.prime[i] = (uint8_t)i;
     const bool fuse = moddown_fused(ctx, level);
-    if (rot_src && !fuse) return fesc_fail(ctx, FESC_EINVAL, "key switch: the permuted addend needs the fused division epilogue");
+    if (rot.src && !fuse) return fesc_fail(ctx, FESC_EINVAL, "key switch: the permuted addend needs the fused division epilogue");
     if (fuse) {
-        NttFinish fin;
-        fin.acc = ws.acc, fin.acc_stride = (size_t)2 * rows * N, fin.out = out, fin.out_stride = out_stride, fin.cinv = ctx->tabs.d_moddown->pinvd;
-        fin.level = level, fin.acc_rows = rows, fin.add_mask = add_mask;
-        fin.rot_src = rot_src, fin.rot_stride = rot_stride, fin.rot_g = rot_g;
-        return ntt_launch(ctx, ws.u, (size_t)batch * 2 * level, m, false, st, true, false, &fin);
+        const uint32_t per = key_stride || n_keys == 1 ? n_keys : 1;       // keys per launch of the final pass
+        for (uint32_t k0 = 0; k0 < n_keys; k0 += per) {
+            NttFinish fin;
+            fin.acc = ws.acc + (size_t)k0 * batch * 2 * rows * N, fin.acc_stride = (size_t)2 * rows * N;
+            fin.out = out, fin.out_stride = out_stride, fin.out_key_stride = key_stride, fin.cinv = ctx->tabs.d_moddown->pinvd;
+            fin.level = level, fin.acc_rows = rows, fin.add_mask = add_mask, fin.nb = batch;
+            if (rot.src) fin.rot_src = rot.src + k0 * rot.key_stride, fin.rot_stride = rot.stride, fin.rot_key_stride = rot.key_stride;
+            for (uint32_t k = 0; k < per && rot.src; k++) fin.rot_g[k] = rot.g[k0 + k];
+            rc = ntt_launch(ctx, ws.u + (size_t)k0 * batch * 2 * level * N, (size_t)per * batch * 2 * level, m, false, st, true, false, &fin);
+            if (rc != FESC_OK) return rc;
+        }
+        return FESC_OK;
     }
     if ((rc = ntt_launch(ctx, ws.u, (size_t)batch * 2 * level, m, false, st, ctx->log_n == 16)) != FESC_OK) return rc;
     prof_begin(ctx, PF_MODDOWN, st);
@@ -893,69 +1048,119 @@ static OwnRows own_rows(const fesc_ctx* ctx, const KsScratch& ws, uint32_t level
 }
 __global__ void k_hoist_prepare(const u64* in, size_t in_stride, u64* out0, size_t out_stride, OwnRows d, u64* dcoef, uint32_t log_n, uint32_t level,
                                 u64 g, const PrimeConst* pcs);
-// Steps 1-3 for the second polynomial of every ciphertext at `in`, read through the permutation of g (0: none)
-static int ks_start(fesc_ctx* ctx, const KsScratch& ws, const u64* in, size_t in_stride, u64 g, uint32_t level, uint32_t batch, cudaStream_t st) {
-    if (small_ring(ctx)) return small_decompose(ctx, ws, in + (size_t)level * ctx->N, in_stride, true, g, level, batch, st);
+// Steps 1-3 for the second polynomial of every ciphertext at in + k * key_stride + b * in_stride, read through the permutation of g[k]
+// (g = nullptr: none).  More than one key: N = 2^16 only.
+static int ks_start(fesc_ctx* ctx, const KsScratch& ws, const u64* in, size_t in_stride, const u64* g, uint32_t level, uint32_t batch,
+                    cudaStream_t st, uint32_t n_keys = 1, size_t key_stride = 0) {
+    const u64* c1 = in + (size_t)level * ctx->N;
+    if (small_ring(ctx)) return small_decompose(ctx, ws, c1, in_stride, true, g ? g[0] : 0, level, batch, st);
+    if (ctx->log_n == 16) {
+        NttSource src;
+        src.src = c1, src.stride = in_stride, src.key_stride = key_stride, src.nb = batch, src.own = own_rows(ctx, ws, level);
+        for (uint32_t k = 0; k < n_keys && g; k++) src.g[k] = g[k];
+        return ks_decompose(ctx, ws, level, batch * n_keys, st, &src);
+    }
     const dim3 grid((ctx->N + 255) / 256, level, batch);
     prof_begin(ctx, PF_AUTOM, st);
     if (g)
-        launch(k_autom_ct, grid, 256, 0, st, in, in_stride, nullptr, 0, own_rows(ctx, ws, level), ws.dcoef, ctx->log_n, level, g, ctx->d_pc, 0);
+        launch(k_autom_ct, grid, 256, 0, st, in, in_stride, nullptr, 0, own_rows(ctx, ws, level), ws.dcoef, ctx->log_n, level, g[0], ctx->d_pc, 0);
     else
         launch(k_hoist_prepare, grid, 256, 0, st, in, in_stride, nullptr, 0, own_rows(ctx, ws, level), ws.dcoef, ctx->log_n, level, 0, ctx->d_pc);
     prof_end(ctx, PF_AUTOM, st);
     return ks_decompose(ctx, ws, level, batch, st);
 }
 
-size_t ks_scratch_words(const fesc_ctx* ctx, uint32_t level, uint32_t chunk, uint32_t n_ext) {
-    const uint32_t beta = (level + ctx->alpha - 1) / ctx->alpha, rows = level + ctx->n_p;
-    return (size_t)chunk * ctx->N * ((size_t)level + (size_t)n_ext * beta * rows + 2 * rows + 2 * level);
+// ciphertexts per key-switch pass (N = 2^16, measured: 16 is 1.5 % faster than 8 on the projection, 3 % on the scan)
+static uint32_t ks_chunk(const fesc_ctx* ctx) {
+    static const int e = getenv("FESC_KS_CHUNK") ? atoi(getenv("FESC_KS_CHUNK")) : 0;
+    return e > 0 ? (uint32_t)e : ctx->log_n == 16 ? 16 : 64;
 }
-KsScratch ks_scratch_carve(const fesc_ctx* ctx, u64* base, uint32_t level, uint32_t chunk, uint32_t n_ext) {
+static uint32_t at_least_one(uint32_t v, uint32_t most) { return v < 1 ? 1 : v < most ? v : most; }
+// The polynomial counts of a cut never shrink when the batch grows, so scratch sized for a batch serves every smaller one.
+KsCut ks_cut_rotate(const fesc_ctx* ctx, uint32_t batch, uint32_t n_keys) {
+    const uint32_t chunk = ks_chunk(ctx), most = n_keys < KS_MAX_KEYS ? n_keys : KS_MAX_KEYS;
+    KsCut c;
+    c.nb = batch < chunk ? batch : chunk;
+    c.keys = ctx->log_n == 16 ? at_least_one(chunk / c.nb, most) : 1;
+    c.src = c.ext = c.acc = ctx->log_n != 16 || (uint64_t)batch * most < chunk ? c.nb * c.keys : chunk;
+    return c;
+}
+KsCut ks_cut_hoisted(const fesc_ctx* ctx, uint32_t batch, uint32_t n_keys) {
+    const uint32_t chunk = ks_chunk(ctx), most = n_keys < KS_MAX_KEYS ? n_keys : KS_MAX_KEYS;
+    // up to 48 accumulators (2.5 GB at 24 limbs): four keys for the 12 ciphertexts of a projection's group
+    const uint32_t accs = chunk > 48 ? chunk : 48;
+    KsCut c;
+    c.nb = batch < chunk ? batch : chunk;
+    c.keys = ctx->log_n == 16 ? at_least_one(accs / c.nb, most) : 1;
+    c.src = c.ext = c.nb;
+    c.acc = ctx->log_n != 16 || (uint64_t)batch * most < accs ? c.nb * c.keys : accs;
+    return c;
+}
+KsCut ks_cut_giant(const fesc_ctx* ctx, uint32_t batch, uint32_t n_terms) {
+    const uint32_t chunk = ks_chunk(ctx);
+    KsCut c;
+    c.nb = batch < chunk ? batch : chunk;
+    c.keys = n_terms < 2 ? 1 : n_terms - 1 < 4 ? n_terms - 1 : 4;       // converted terms one inner-product pass sums
+    c.src = ctx->log_n != 16 ? c.nb : c.nb * c.keys < chunk ? c.nb * c.keys : chunk;      // decomposed together when they are few
+    c.ext = c.nb * c.keys, c.acc = c.nb;
+    return c;
+}
+size_t ks_scratch_words(const fesc_ctx* ctx, uint32_t level, const KsCut& cut) {
+    const uint32_t beta = (level + ctx->alpha - 1) / ctx->alpha, rows = level + ctx->n_p;
+    return ctx->N * ((size_t)cut.src * level + (size_t)cut.ext * beta * rows + (size_t)cut.acc * (2 * rows + 2 * level));
+}
+KsScratch ks_scratch_carve(const fesc_ctx* ctx, u64* base, uint32_t level, const KsCut& cut) {
     const uint32_t beta = (level + ctx->alpha - 1) / ctx->alpha, rows = level + ctx->n_p;
     const size_t N = ctx->N;
     KsScratch ws;
     ws.dcoef = base;
-    ws.ext = ws.dcoef + (size_t)chunk * level * N;
-    ws.acc = ws.ext + (size_t)n_ext * chunk * beta * rows * N;
-    ws.u = ws.acc + (size_t)chunk * 2 * rows * N;
+    ws.ext = ws.dcoef + (size_t)cut.src * level * N;
+    ws.acc = ws.ext + (size_t)cut.ext * beta * rows * N;
+    ws.u = ws.acc + (size_t)cut.acc * 2 * rows * N;
     return ws;
-}
-
-uint32_t ks_chunk(const fesc_ctx* ctx, uint32_t batch) {
-    // ciphertexts per key-switch pass at N = 2^16 (measured: 16 is 1.5 % faster than 8 on the projection, 3 % on the scan)
-    uint32_t c = ctx->log_n == 16 ? 16 : 64;
-    static const int e = getenv("FESC_KS_CHUNK") ? atoi(getenv("FESC_KS_CHUNK")) : 0;
-    if (e > 0) c = (uint32_t)e;
-    return batch < c ? batch : c;
 }
 
 // Rotation of `batch` ciphertexts with strides (words) between consecutive inputs / outputs.
 // accumulate != 0: the rotated ciphertext is ADDED to what `out` holds.
 int rotate_internal(fesc_ctx* ctx, const u64* in, size_t in_stride, u64* out, size_t out_stride, uint32_t batch,
                     uint32_t level, uint32_t key_id, u64* scratch, cudaStream_t st, int accumulate) {
-    auto it = ctx->keys.find(key_id);
-    if (it == ctx->keys.end() || key_id == FESC_RELIN_KEY_ID)
-        return fesc_fail(ctx, FESC_ENOKEY, "rotate: no Galois key " + std::to_string(key_id));
-    const uint32_t chunk = ks_chunk(ctx, batch);
-    KsScratch ws = ks_scratch_carve(ctx, scratch, level, chunk);
-    for (uint32_t b0 = 0; b0 < batch; b0 += chunk) {
-        uint32_t nb = batch - b0 < chunk ? batch - b0 : chunk;
-        const u64* ib = in + (size_t)b0 * in_stride;
-        u64* ob = out + (size_t)b0 * out_stride;
-        int rc;
-        if (moddown_fused(ctx, level)) {                // the division's epilogue adds sigma_g(c0) straight from the input
-            if ((rc = ks_start(ctx, ws, ib, in_stride, it->second.g, level, nb, st)) != FESC_OK) return rc;
-            if ((rc = ks_inner(ctx, ws, it->second, level, nb, st, 0, 0)) != FESC_OK) return rc;
-            rc = ks_moddown(ctx, ws, level, nb, ob, out_stride, accumulate ? 3 : 0, st, ib, in_stride, it->second.g);
-        } else {
-            dim3 g((ctx->N + 255) / 256, level, nb);
-            prof_begin(ctx, PF_AUTOM, st);
-            launch(k_autom_ct, g, 256, 0, st, ib, in_stride, ob, out_stride, own_rows(ctx, ws, level), ws.dcoef, ctx->log_n, level, it->second.g,
-                                          ctx->d_pc, accumulate);
-            prof_end(ctx, PF_AUTOM, st);
-            rc = key_switch_chunk(ctx, ws, it->second, level, nb, ob, out_stride, accumulate ? 3 : 1, st);
-        }
+    return rotate_multi_internal(ctx, in, in_stride, 0, out, out_stride, 0, batch, level, &key_id, 1, scratch, st, accumulate);
+}
+int rotate_multi_internal(fesc_ctx* ctx, const u64* in, size_t in_stride, size_t in_key_stride, u64* out, size_t out_stride,
+                          size_t out_key_stride, uint32_t batch, uint32_t level, const uint32_t* key_ids, uint32_t n_keys, u64* scratch,
+                          cudaStream_t st, int accumulate) {
+    const bool fused = moddown_fused(ctx, level);     // the division's epilogue adds sigma_g(c0) straight from the input
+    KsCut cut = ks_cut_rotate(ctx, batch, n_keys);
+    const KsScratch ws = ks_scratch_carve(ctx, scratch, level, cut);
+    if (!fused) cut.keys = 1;
+    for (uint32_t k0 = 0; k0 < n_keys; k0 += cut.keys) {
+        KsKeys keys;
+        int rc = ks_keys(ctx, "rotate", key_ids + k0, n_keys - k0 < cut.keys ? n_keys - k0 : cut.keys, keys);
         if (rc != FESC_OK) return rc;
+        for (uint32_t b0 = 0; b0 < batch; b0 += cut.nb) {
+            const uint32_t nb = batch - b0 < cut.nb ? batch - b0 : cut.nb;
+            const u64* ib = in + k0 * in_key_stride + (size_t)b0 * in_stride;
+            u64* ob = out + k0 * out_key_stride + (size_t)b0 * out_stride;
+            if (fused) {
+                if ((rc = ks_start(ctx, ws, ib, in_stride, keys.g, level, nb, st, keys.n, in_key_stride)) != FESC_OK) return rc;
+                InnerSrcs S;
+                S.n = keys.n;
+                const size_t ext_words = (size_t)nb * ((level + ctx->alpha - 1) / ctx->alpha) * (level + ctx->n_p) * ctx->N;
+                for (uint32_t k = 0; k < keys.n; k++) S.s[k] = InnerSrc{ws.ext + k * ext_words, keys.key[k], 0};
+                if ((rc = ks_inner_multi(ctx, ws, S, level, nb, st, 0, 1, keys.n > 1)) != FESC_OK) return rc;
+                KsRot rot;
+                rot.src = ib, rot.stride = in_stride, rot.key_stride = in_key_stride, rot.g = keys.g;
+                rc = ks_moddown(ctx, ws, level, nb, ob, out_stride, accumulate ? 3 : 0, st, rot, keys.n, out_key_stride);
+            } else {
+                dim3 g((ctx->N + 255) / 256, level, nb);
+                prof_begin(ctx, PF_AUTOM, st);
+                launch(k_autom_ct, g, 256, 0, st, ib, in_stride, ob, out_stride, own_rows(ctx, ws, level), ws.dcoef, ctx->log_n, level, keys.g[0],
+                       ctx->d_pc, accumulate);
+                prof_end(ctx, PF_AUTOM, st);
+                rc = key_switch_chunk(ctx, ws, ctx->keys[key_ids[k0]], level, nb, ob, out_stride, accumulate ? 3 : 1, st);
+            }
+            if (rc != FESC_OK) return rc;
+        }
     }
     return FESC_OK;
 }
@@ -986,6 +1191,25 @@ __global__ void __launch_bounds__(256) k_hoist_prepare(const u64* __restrict__ i
     }
 }
 
+// acc[b][0] first polynomial += sum_p sigma_p(first polynomial of acc[b][p]), p = 1..n: one pass over the terms
+struct GiantSet {
+    u64 g[32];
+    uint32_t n;
+};
+__global__ void __launch_bounds__(256) k_giant_c0(u64* acc, size_t stride, size_t ct_words, uint32_t log_n, GiantSet gs, const PrimeConst* __restrict__ pcs) {
+    pdl_begin();
+    const uint32_t N = 1u << log_n, t = blockIdx.x * blockDim.x + threadIdx.x, l = blockIdx.y;
+    if (t >= N) return;
+    u64* o = acc + (size_t)blockIdx.z * stride + (size_t)l * N;
+    const u64 q = pcs[l].q;
+    for (uint32_t p = 0; p <= gs.n; p++)
+        if (!DBG_REGION(o + p * ct_words, N * sizeof(u64))) return;
+    u64 v = o[t];
+#pragma unroll 4
+    for (uint32_t p = 0; p < gs.n; p++) v = addmod(v, o[(p + 1) * ct_words + galois_src(t, log_n, gs.g[p])], q);
+    o[t] = v;
+}
+
 // sum_p rot(acc[b][p], key n = key_base + p) for p = 1..n_terms-1 ADDED into acc[b][0], with one division by P
 // per ciphertext: the inner products of all p are summed on the extended basis first.  acc holds `batch` groups of
 // n_terms ciphertexts (ct_words each, group stride n_terms * ct_words).
@@ -995,34 +1219,52 @@ int giant_sum_deferred_internal(fesc_ctx* ctx, u64* acc, uint32_t n_terms, size_
     for (uint32_t p = 1; p < n_terms; p++)
         if (!ctx->keys.count(key_base + p) || key_base + p == FESC_RELIN_KEY_ID)
             return fesc_fail(ctx, FESC_ENOKEY, "giant steps: no Galois key " + std::to_string(key_base + p));
-    const uint32_t chunk = ks_chunk(ctx, batch), n_ext = giant_ext_buffers(n_terms);
-    KsScratch ws = ks_scratch_carve(ctx, scratch, level, chunk, n_ext);
+    const KsCut cut = ks_cut_giant(ctx, batch, n_terms);
+    KsScratch ws = ks_scratch_carve(ctx, scratch, level, cut);
     const size_t stride = (size_t)n_terms * ct_words;
-    const size_t ext_words = (size_t)chunk * ((level + ctx->alpha - 1) / ctx->alpha) * (level + ctx->n_p) * ctx->N;
-    for (uint32_t b0 = 0; b0 < batch; b0 += chunk) {
-        const uint32_t nb = batch - b0 < chunk ? batch - b0 : chunk;
-        dim3 g((ctx->N + 255) / 256, level, nb);
+    const size_t ext_words = (size_t)((level + ctx->alpha - 1) / ctx->alpha) * (level + ctx->n_p) * ctx->N;
+    for (uint32_t p0 = 1; p0 < n_terms; p0 += 32) {
+        GiantSet gs;
+        gs.n = n_terms - p0 < 32 ? n_terms - p0 : 32;
+        for (uint32_t p = 0; p < gs.n; p++) gs.g[p] = ctx->keys[key_base + p0 + p].g;
+        prof_begin(ctx, PF_AUTOM, st);
+        // the terms of this launch follow the ones before: shift the base so that term 0 stays the sum
+        if (p0 == 1)
+            launch(k_giant_c0, dim3((ctx->N + 255) / 256, level, batch), 256, 0, st, acc, stride, ct_words, ctx->log_n, gs, ctx->d_pc);
+        else
+            for (uint32_t p = 0; p < gs.n; p++) {
+                GiantSet one;
+                one.n = 1, one.g[0] = gs.g[p];
+                launch(k_giant_c0, dim3((ctx->N + 255) / 256, level, batch), 256, 0, st, acc, stride, (size_t)(p0 + p) * ct_words, ctx->log_n, one, ctx->d_pc);
+            }
+        prof_end(ctx, PF_AUTOM, st);
+    }
+    for (uint32_t b0 = 0; b0 < batch; b0 += cut.nb) {
+        const uint32_t nb = batch - b0 < cut.nb ? batch - b0 : cut.nb;
         u64* base = acc + (size_t)b0 * stride;
-        // up to n_ext terms are rotated and converted side by side, then one inner-product pass sums them: the
+        // up to cut.keys terms are rotated and converted side by side, then one inner-product pass sums them: the
         // accumulators on the extended basis are read and written once per pass instead of once per term
-        for (uint32_t p0 = 1; p0 < n_terms; p0 += n_ext) {
-            const uint32_t np = n_terms - p0 < n_ext ? n_terms - p0 : n_ext;
+        for (uint32_t p0 = 1; p0 < n_terms; p0 += cut.keys) {
+            const uint32_t np = n_terms - p0 < cut.keys ? n_terms - p0 : cut.keys;
+            std::vector<uint32_t> ids;
+            for (uint32_t s = 0; s < np; s++) ids.push_back(key_base + p0 + s);
+            KsKeys keys;
+            int rc = ks_keys(ctx, "giant steps", ids.data(), np, keys);
+            if (rc != FESC_OK) return rc;
             InnerSrcs S;
             S.n = np;
-            for (uint32_t s = 0; s < np; s++) {
-                const EvalKey& key = ctx->keys[key_base + p0 + s];
-                KsScratch wss = ws;
-                wss.ext = ws.ext + (size_t)s * ext_words;
-                prof_begin(ctx, PF_AUTOM, st);
-                launch(k_autom_ct, g, 256, 0, st, base + (size_t)(p0 + s) * ct_words, stride, base, stride, own_rows(ctx, wss, level),
-                                              wss.dcoef, ctx->log_n, level, key.g, ctx->d_pc, 1);
-                prof_end(ctx, PF_AUTOM, st);
-                int rc = ks_decompose(ctx, wss, level, nb, st);
+            for (uint32_t s = 0; s < np; s++) S.s[s] = InnerSrc{ws.ext + s * nb * ext_words, keys.key[s], 0};
+            if (ctx->log_n == 16 && nb * np <= cut.src) {
+                rc = ks_start(ctx, ws, base + (size_t)p0 * ct_words, stride, keys.g, level, nb, st, np, ct_words);
                 if (rc != FESC_OK) return rc;
-                S.s[s] = InnerSrc{wss.ext, key.d_key, 0};
+            } else {
+                for (uint32_t s = 0; s < np; s++) {
+                    KsScratch wss = ws;
+                    wss.ext = ws.ext + s * nb * ext_words;
+                    if ((rc = ks_start(ctx, wss, base + (size_t)(p0 + s) * ct_words, stride, &keys.g[s], level, nb, st)) != FESC_OK) return rc;
+                }
             }
-            int rc = ks_inner_multi(ctx, ws, S, level, nb, st, p0 > 1, p0 + np == n_terms);
-            if (rc != FESC_OK) return rc;
+            if ((rc = ks_inner_multi(ctx, ws, S, level, nb, st, p0 > 1, p0 + np == n_terms)) != FESC_OK) return rc;
         }
         int rc = ks_moddown(ctx, ws, level, nb, base, stride, 3, st);
         if (rc != FESC_OK) return rc;
@@ -1038,26 +1280,31 @@ int rotate_hoisted_internal(fesc_ctx* ctx, const u64* in, size_t in_stride, u64*
     for (uint32_t k = 0; k < n_keys; k++)
         if (!ctx->keys.count(key_ids[k]) || key_ids[k] == FESC_RELIN_KEY_ID)
             return fesc_fail(ctx, FESC_ENOKEY, "rotate_hoisted: no Galois key " + std::to_string(key_ids[k]));
-    const uint32_t chunk = ks_chunk(ctx, batch);
-    KsScratch ws = ks_scratch_carve(ctx, scratch, level, chunk);
-    for (uint32_t b0 = 0; b0 < batch; b0 += chunk) {
-        const uint32_t nb = batch - b0 < chunk ? batch - b0 : chunk;
+    const bool fused = moddown_fused(ctx, level);        // sigma_g(c0) is added by the division's epilogue, straight from the input
+    KsCut cut = ks_cut_hoisted(ctx, batch, n_keys);
+    const KsScratch ws = ks_scratch_carve(ctx, scratch, level, cut);
+    if (!fused) cut.keys = 1;
+    for (uint32_t b0 = 0; b0 < batch; b0 += cut.nb) {
+        const uint32_t nb = batch - b0 < cut.nb ? batch - b0 : cut.nb;
         dim3 g((ctx->N + 255) / 256, level, nb);
         const u64* ib = in + (size_t)b0 * in_stride;
-        int rc = ks_start(ctx, ws, ib, in_stride, 0, level, nb, st);
+        int rc = ks_start(ctx, ws, ib, in_stride, nullptr, level, nb, st);
         if (rc != FESC_OK) return rc;
-        for (uint32_t k = 0; k < n_keys; k++) {
-            const EvalKey& key = ctx->keys[key_ids[k]];
-            u64* ob = out + (size_t)k * key_stride + (size_t)b0 * out_stride;
-            if (moddown_fused(ctx, level)) {     // sigma_g(c0) is added by the division's epilogue, straight from the input
-                if ((rc = ks_inner(ctx, ws, key, level, nb, st, key.g, 0)) != FESC_OK) return rc;
-                if ((rc = ks_moddown(ctx, ws, level, nb, ob, out_stride, 0, st, ib, in_stride, key.g)) != FESC_OK) return rc;
+        for (uint32_t k0 = 0; k0 < n_keys; k0 += cut.keys) {
+            KsKeys keys;
+            if ((rc = ks_keys(ctx, "rotate_hoisted", key_ids + k0, n_keys - k0 < cut.keys ? n_keys - k0 : cut.keys, keys)) != FESC_OK) return rc;
+            u64* ob = out + (size_t)k0 * key_stride + (size_t)b0 * out_stride;
+            if (fused) {
+                if ((rc = ks_inner_hoisted(ctx, ws, keys, 0, keys.n, level, nb, st)) != FESC_OK) return rc;
+                KsRot rot;
+                rot.src = ib, rot.stride = in_stride, rot.g = keys.g;
+                if ((rc = ks_moddown(ctx, ws, level, nb, ob, out_stride, 0, st, rot, keys.n, key_stride)) != FESC_OK) return rc;
                 continue;
             }
             prof_begin(ctx, PF_AUTOM, st);
-            launch(k_hoist_prepare, g, 256, 0, st, ib, in_stride, ob, out_stride, OwnRows{nullptr, 1, 1, 1, 0}, nullptr, ctx->log_n, level, key.g, ctx->d_pc);
+            launch(k_hoist_prepare, g, 256, 0, st, ib, in_stride, ob, out_stride, OwnRows{nullptr, 1, 1, 1, 0}, nullptr, ctx->log_n, level, keys.g[0], ctx->d_pc);
             prof_end(ctx, PF_AUTOM, st);
-            rc = ks_apply(ctx, ws, key, level, nb, ob, out_stride, 1, st, key.g);
+            rc = ks_apply(ctx, ws, ctx->keys[key_ids[k0]], level, nb, ob, out_stride, 1, st, keys.g[0]);
             if (rc != FESC_OK) return rc;
         }
     }
@@ -1103,8 +1350,9 @@ int rotate_sum_hoisted_internal(fesc_ctx* ctx, const u64* in, size_t in_stride, 
             return fesc_fail(ctx, FESC_ENOKEY, "rotate_sum_hoisted: no Galois key " + std::to_string(key_ids[k]));
         gs.g[k] = ctx->keys[key_ids[k]].g;
     }
-    const uint32_t chunk = ks_chunk(ctx, batch);
-    KsScratch ws = ks_scratch_carve(ctx, scratch, level, chunk);
+    const KsCut cut = ks_cut_rotate(ctx, batch);
+    const uint32_t chunk = cut.nb;
+    KsScratch ws = ks_scratch_carve(ctx, scratch, level, cut);
     for (uint32_t b0 = 0; b0 < batch; b0 += chunk) {
         const uint32_t nb = batch - b0 < chunk ? batch - b0 : chunk;
         dim3 g((ctx->N + 255) / 256, level, nb);
@@ -1113,7 +1361,7 @@ int rotate_sum_hoisted_internal(fesc_ctx* ctx, const u64* in, size_t in_stride, 
         prof_begin(ctx, PF_AUTOM, st);
         launch(k_rotsum_prepare, g, 256, 0, st, ib, in_stride, ob, out_stride, ctx->log_n, level, gs, ctx->d_pc);
         prof_end(ctx, PF_AUTOM, st);
-        int rc = ks_start(ctx, ws, ib, in_stride, 0, level, nb, st);
+        int rc = ks_start(ctx, ws, ib, in_stride, nullptr, level, nb, st);
         if (rc != FESC_OK) return rc;
         InnerSrcs S;                                   // one converted polynomial, read through every key's permutation
         S.n = n_keys;
@@ -1130,7 +1378,7 @@ extern "C" int fesc_rotate_sum_hoisted(fesc_ctx* ctx, const uint64_t* d_in, uint
     if (n_limbs == 0 || n_limbs > ctx->n_q) return fesc_fail(ctx, FESC_ELEVEL, "rotate_sum_hoisted: level out of range");
     if (batch == 0) return FESC_OK;
     u64* scratch;
-    int rc = ctx_scratch(ctx, ks_scratch_words(ctx, n_limbs, ks_chunk(ctx, batch)) * sizeof(u64), &scratch);
+    int rc = ctx_scratch(ctx, ks_scratch_words(ctx, n_limbs, ks_cut_rotate(ctx, batch)) * sizeof(u64), &scratch);
     if (rc != FESC_OK) return rc;
     const size_t stride = (size_t)2 * n_limbs * ctx->N;
     return rotate_sum_hoisted_internal(ctx, (const u64*)d_in, stride, (u64*)d_out, stride, batch, n_limbs, key_ids,
@@ -1143,7 +1391,7 @@ extern "C" int fesc_rotate_hoisted(fesc_ctx* ctx, const uint64_t* d_in, uint64_t
     if (n_limbs == 0 || n_limbs > ctx->n_q) return fesc_fail(ctx, FESC_ELEVEL, "rotate_hoisted: level out of range");
     if (batch == 0 || n_keys == 0) return FESC_OK;
     u64* scratch;
-    int rc = ctx_scratch(ctx, ks_scratch_words(ctx, n_limbs, ks_chunk(ctx, batch)) * sizeof(u64), &scratch);
+    int rc = ctx_scratch(ctx, ks_scratch_words(ctx, n_limbs, ks_cut_hoisted(ctx, batch, n_keys)) * sizeof(u64), &scratch);
     if (rc != FESC_OK) return rc;
     const size_t stride = (size_t)2 * n_limbs * ctx->N;
     return rotate_hoisted_internal(ctx, (const u64*)d_in, stride, (u64*)d_out, stride, (size_t)batch * stride, batch,
@@ -1156,7 +1404,7 @@ extern "C" int fesc_rotate(fesc_ctx* ctx, const uint64_t* d_in, uint64_t* d_out,
     if (n_limbs == 0 || n_limbs > ctx->n_q) return fesc_fail(ctx, FESC_ELEVEL, "rotate: level out of range");
     if (batch == 0) return FESC_OK;
     u64* scratch;
-    int rc = ctx_scratch(ctx, ks_scratch_words(ctx, n_limbs, ks_chunk(ctx, batch)) * sizeof(u64), &scratch);
+    int rc = ctx_scratch(ctx, ks_scratch_words(ctx, n_limbs, ks_cut_rotate(ctx, batch)) * sizeof(u64), &scratch);
     if (rc != FESC_OK) return rc;
     const size_t stride = (size_t)2 * n_limbs * ctx->N;
     return rotate_internal(ctx, (const u64*)d_in, stride, (u64*)d_out, stride, batch, n_limbs, key_id, scratch,
@@ -1307,8 +1555,9 @@ __global__ void __launch_bounds__(256) k_tensor(const u64* __restrict__ a, size_
 int ctmul_internal(fesc_ctx* ctx, const u64* a, size_t a_stride, const u64* b, size_t b_stride, u64* out,
                    size_t out_stride, uint32_t batch, uint32_t level, u64* scratch, cudaStream_t st) {
     const EvalKey& key = ctx->keys[FESC_RELIN_KEY_ID];
-    const uint32_t chunk = ks_chunk(ctx, batch);
-    KsScratch ws = ks_scratch_carve(ctx, scratch, level, chunk);
+    const KsCut cut = ks_cut_rotate(ctx, batch);
+    const uint32_t chunk = cut.nb;
+    KsScratch ws = ks_scratch_carve(ctx, scratch, level, cut);
     for (uint32_t b0 = 0; b0 < batch; b0 += chunk) {
         uint32_t nb = batch - b0 < chunk ? batch - b0 : chunk;
         dim3 g((ctx->N + 255) / 256, level, nb);
@@ -1328,7 +1577,7 @@ extern "C" int fesc_ct_ct_mul(fesc_ctx* ctx, const uint64_t* d_a, const uint64_t
     if (n_limbs == 0 || n_limbs > ctx->n_q) return fesc_fail(ctx, FESC_ELEVEL, "ct_ct_mul: level out of range");
     if (batch == 0) return FESC_OK;
     u64* scratch;
-    int rc = ctx_scratch(ctx, ks_scratch_words(ctx, n_limbs, ks_chunk(ctx, batch)) * sizeof(u64), &scratch);
+    int rc = ctx_scratch(ctx, ks_scratch_words(ctx, n_limbs, ks_cut_rotate(ctx, batch)) * sizeof(u64), &scratch);
     if (rc != FESC_OK) return rc;
     const size_t stride = (size_t)2 * n_limbs * ctx->N;
     return ctmul_internal(ctx, (const u64*)d_a, stride, (const u64*)d_b, stride, (u64*)d_out, stride, batch, n_limbs,

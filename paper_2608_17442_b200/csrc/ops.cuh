@@ -15,7 +15,7 @@ struct KsScratch {
 // steps of a projection (different converted polynomials, different keys, one sum) and the rotate-and-add chains (one
 // converted polynomial read through several Galois permutations, one key each) then read and write the accumulators
 // once instead of once per key, and the later reads of a shared source hit L2.
-#define INNER_MAX_SRC 8
+#define INNER_MAX_SRC KS_MAX_KEYS
 struct InnerSrc {
     const u64* ext;   // [batch][beta][level+K][N]
     const u64* key;   // [beta][2][n_q+K][N]
@@ -26,12 +26,20 @@ struct InnerSrcs {
     uint32_t n;
 };
 
-size_t ks_scratch_words(const fesc_ctx* ctx, uint32_t level, uint32_t chunk, uint32_t n_ext = 1);
-KsScratch ks_scratch_carve(const fesc_ctx* ctx, u64* base, uint32_t level, uint32_t chunk, uint32_t n_ext = 1);
-// converted polynomials a deferred giant-step sum of n_terms keeps side by side (one inner-product pass over them)
-static inline uint32_t giant_ext_buffers(uint32_t n_terms) { return n_terms < 2 ? 1 : (n_terms - 1 < 4 ? n_terms - 1 : 4); }
-uint32_t ks_chunk(const fesc_ctx* ctx, uint32_t batch);
-
+// How a key-switch pass is cut and its scratch in polynomials: `src` are decomposed at a time (dcoef), `ext` converted ones are kept,
+// `acc` accumulators (and converted special parts) exist side by side.
+struct KsCut {
+    uint32_t nb, keys;          // ciphertexts and keys per pass
+    uint32_t src, ext, acc;
+};
+// one key per call, or several plain rotations of the same few ciphertexts: keys share a pass until it has 16 polynomials
+KsCut ks_cut_rotate(const fesc_ctx* ctx, uint32_t batch, uint32_t n_keys = 1);
+// hoisted rotations: one decomposition, the keys of a pass share one reading of the converted digits and one division launch
+KsCut ks_cut_hoisted(const fesc_ctx* ctx, uint32_t batch, uint32_t n_keys);
+// deferred giant-step sum over n_terms - 1 rotated terms
+KsCut ks_cut_giant(const fesc_ctx* ctx, uint32_t batch, uint32_t n_terms);
+size_t ks_scratch_words(const fesc_ctx* ctx, uint32_t level, const KsCut& cut);
+KsScratch ks_scratch_carve(const fesc_ctx* ctx, u64* base, uint32_t level, const KsCut& cut);
 int rotate_internal(fesc_ctx* ctx, const u64* in, size_t in_stride, u64* out, size_t out_stride, uint32_t batch,
                     uint32_t level, uint32_t key_id, u64* scratch, cudaStream_t st, int accumulate);
 int rotate_hoisted_internal(fesc_ctx* ctx, const u64* in, size_t in_stride, u64* out, size_t out_stride,
@@ -40,7 +48,11 @@ int rotate_hoisted_internal(fesc_ctx* ctx, const u64* in, size_t in_stride, u64*
 int rotate_sum_hoisted_internal(fesc_ctx* ctx, const u64* in, size_t in_stride, u64* out, size_t out_stride,
                                 uint32_t batch, uint32_t level, const uint32_t* key_ids, uint32_t n_keys, u64* scratch,
                                 cudaStream_t st);
-// scratch: ks_scratch_words(ctx, level, ks_chunk(ctx, batch), giant_ext_buffers(n_terms)) words
+// Plain rotations of the same kind of ciphertexts by n_keys keys: rotation of ciphertext b (at in + k * in_key_stride + b * in_stride) by
+// key k to out + k * out_key_stride + b * out_stride; accumulate: added to what is there.
+int rotate_multi_internal(fesc_ctx* ctx, const u64* in, size_t in_stride, size_t in_key_stride, u64* out, size_t out_stride,
+                          size_t out_key_stride, uint32_t batch, uint32_t level, const uint32_t* key_ids, uint32_t n_keys, u64* scratch,
+                          cudaStream_t st, int accumulate);
 int giant_sum_deferred_internal(fesc_ctx* ctx, u64* acc, uint32_t n_terms, size_t ct_words, uint32_t batch,
                                 uint32_t level, uint32_t key_base, u64* scratch, cudaStream_t st);
 int rescale_internal(fesc_ctx* ctx, const u64* in, size_t in_stride, u64* out, uint32_t batch, uint32_t level,

@@ -797,7 +797,11 @@ extern "C" int fesc_scan_contract(fesc_ctx* ctx, const uint64_t* d_x, const uint
     X.dry = true, X.arena = reinterpret_cast<u64*>((uintptr_t)1 << 40), X.top = 0, X.high = 0, X.ks = X.rs = nullptr;
     int rc = scan_run(X, (const u64*)d_x, (const u64*)d_a, (const u64*)d_B, (const u64*)d_C, (u64*)d_m_out);
     if (rc != FESC_OK) return rc;
-    const size_t ks_words = ks_scratch_words(ctx, g.l0, ks_chunk(ctx, 2 * g.B));
+    size_t ks_words = ks_scratch_words(ctx, g.l0, ks_cut_rotate(ctx, 2 * g.B));
+    if (desc->hoist) {           // hoisted rotations keep several accumulators per ciphertext side by side
+        const size_t hw = ks_scratch_words(ctx, g.l0, ks_cut_hoisted(ctx, 2 * g.B, KS_MAX_KEYS));
+        if (hw > ks_words) ks_words = hw;
+    }
     const size_t rs_words = (size_t)2 * g.B * 2 * ctx->N;
     u64* scratch;
     rc = ctx_scratch(ctx, (X.high + ks_words + rs_words) * sizeof(u64), &scratch);
@@ -821,7 +825,7 @@ extern "C" int fesc_split_complex(fesc_ctx* ctx, const uint64_t* d_in, uint64_t*
     const uint32_t N = ctx->N;
     const size_t ctw = (size_t)2 * n_limbs * N;
     u64* scratch;
-    int rc = ctx_scratch(ctx, ks_scratch_words(ctx, n_limbs, ks_chunk(ctx, batch)) * sizeof(u64), &scratch);
+    int rc = ctx_scratch(ctx, ks_scratch_words(ctx, n_limbs, ks_cut_rotate(ctx, batch)) * sizeof(u64), &scratch);
     if (rc != FESC_OK) return rc;
     const u64* in = (const u64*)d_in;
     u64 *re = (u64*)d_re2, *im = (u64*)d_im2;
