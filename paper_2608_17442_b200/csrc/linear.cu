@@ -584,7 +584,7 @@ __global__ void __launch_bounds__(32 * IM_CW, 1) k_bsgs_accumulate_imma(
 }
 
 // Knobs for experiments.  FESC_BSGS_KERNEL picks the accumulate kernel: "int" the 128-bit integer one, "fp" the
-// exact-FP64 one, "mixed" the mixed-pipe one, anything else the default (tensor-core byte planes where they apply).  FESC_BSGS_GROUP_GIB fixes the scratch
+// exact-FP64 one, "mixed" the mixed-pipe one, anything else the default.  FESC_BSGS_GROUP_GIB fixes the scratch
 // budget that decides how many token blocks are processed per group (default: from the free device memory).
 static int bsgs_kernel() {
     static int v = -1;
@@ -862,13 +862,17 @@ extern "C" int fesc_linear(fesc_ctx* ctx, const uint64_t* d_ct_in, const uint64_
         kern<<<grid, 32 * IM_CW, smem, st>>>(rot, diags, acc, ctx->d_pc, N, level, nt, gin * n1, bp_count, pitch); \
     } while (0)
         const bool fp_ok = qbits <= 50 && bsgs_kernel() != 2;
-        const bool imma_ok = bsgs_kernel() == 0 && qbits <= 56 && N % IM_CW == 0 && gin * n1 <= 256 && level <= 65535;
+        // Sums of at most 256 terms on primes below 2^50: the mixed-pipe kernel streams the weights near the copy bandwidth for
+        // one or two token blocks (7.25 GB of weights: 1.36 ms for one block, 2.0 for two, 3.8 for three or four; the byte-plane
+        // kernel on residues takes 4.3 to 7.0 ms, its transposition costs more than its products).  Larger primes up to 56 bits:
+        // byte planes against 128-bit integer sums.
+        const bool mixed_ok = fp_ok && (bsgs_kernel() == 0 || bsgs_kernel() == 3) && N % 256 == 0 && gin * n1 <= 256;
+        const bool imma_ok = bsgs_kernel() == 0 && !fp_ok && qbits <= 56 && N % IM_CW == 0 && gin * n1 <= 256 && level <= 65535;
         const bool deep = gin * n1 <= 128;       // room for 8 stages beside the rotated inputs
-        if (imma_ok && qbits <= 50 && deep) BSGS_IMMA(true, 8);
-        else if (imma_ok && qbits <= 50) BSGS_IMMA(true, 4);
+        if (mixed_ok && nt >= 2) BSGS_MIX(2, 8, 3);
+        else if (mixed_ok) BSGS_MIX(1, 8, 4);
         else if (imma_ok && deep) BSGS_IMMA(false, 8);
         else if (imma_ok) BSGS_IMMA(false, 4);
-        else if (fp_ok && bsgs_kernel() == 3 && N % 256 == 0 && nt >= 2 && gin * n1 <= 256) BSGS_MIX(2, 8, 3);
         else if (fp_ok && N % 256 == 0 && nt >= 2) BSGS_FPS(2, 8, 3);
         else if (fp_ok && nt >= 2) BSGS_FP(2, 8);
         else if (fp_ok) BSGS_FP(1, 8);
