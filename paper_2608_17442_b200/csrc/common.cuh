@@ -353,7 +353,8 @@ __device__ __forceinline__ size_t own_index(const OwnRows& w, uint32_t b, uint32
 // Keys of one pass that rotates several ciphertexts by several amounts: polynomial k * nb + b belongs to key k and ciphertext b.
 #define KS_MAX_KEYS 16
 // Optional source of the first pass of an inverse N = 2^16 transform over rows r = polynomial * level + l (period `level`): row l
-// of src + k * key_stride + b * stride, read through the permutation of g[k] (0: none), kept in its own-limb row on the way.
+// of src + k * key_stride + b * stride, read through the permutation of g[k] (0: none), kept in its own-limb row (own.ext
+// != nullptr) on the way.
 // Saves the kernel that permuted and copied the polynomial (8 us of a rotation's 184).
 struct NttSource {
     const u64* src = nullptr;
@@ -385,6 +386,10 @@ struct NttFinish {
     // several keys: ciphertext index k * nb + b is ciphertext b of key k, at out + k * out_key_stride and rot_src + k * rot_key_stride
     uint32_t nb = 0x7fffffff;
     size_t out_key_stride = 0, rot_key_stride = 0;
+    // rescale: the rows to transform are the centred residues of row bp of `centred` (canonical modulo centred_q, COEFF), taken by the
+    // first pass modulo every row's prime; the buffer handed to the transform is only written
+    const u64* centred = nullptr;
+    double centred_q = 0;
 };
 
 // internal launchers (ntt.cu)

@@ -3,22 +3,10 @@
 // Tap r >= 1 of token k reads token k-r: inside a token block that is rho(q; -r) masked to tokens k >= r (M_r); the
 // first r tokens of a block read the previous block's last tokens, rho(q_prev; T - r) masked to k < r (M'_r).
 // Every ciphertext is decomposed once and rotated by its 2(d_conv-1) amounts (hoisted rotations); the rotations by
-// T - r are kept for the next token block.  The masked sums use the plain ct-pt multiply-accumulate, then the bias
-// plaintext is added to c0 and the block is rescaled.
+// T - r are kept for the next token block.  The masked sum and the bias plaintext are one pass,
+// then the block is rescaled.
 #define FESC_DBG_FILE 7   // file id in the sites a debug build reports
 #include "ops.cuh"
-
-// c0 of every ciphertext += its plaintext (pt_stride words between plaintexts)
-__global__ void __launch_bounds__(256) k_ct_add_pt(u64* __restrict__ ct, size_t ct_stride, const u64* __restrict__ pt,
-                                                   size_t pt_stride, const PrimeConst* __restrict__ pcs, uint32_t N) {
-    pdl_begin();
-    const uint32_t c = blockIdx.x * blockDim.x + threadIdx.x;
-    const uint32_t l = blockIdx.y, b = blockIdx.z;
-    if (c >= N) return;
-    u64* o = ct + (size_t)b * ct_stride + (size_t)l * N + c;
-    if (!DBG_REGION(o - c, N * sizeof(u64)) || !DBG_REGION(pt + (size_t)b * pt_stride + (size_t)l * N, N * sizeof(u64))) return;
-    *o = addmod(*o, pt[(size_t)b * pt_stride + (size_t)l * N + c], pcs[l].q);
-}
 
 extern "C" int fesc_conv(fesc_ctx* ctx, const uint64_t* d_ct_in, const uint64_t* d_masks, const uint64_t* d_bias,
                          const fesc_conv_desc* desc, uint64_t* d_ct_out, void* stream) {
@@ -60,22 +48,15 @@ extern "C" int fesc_conv(fesc_ctx* ctx, const uint64_t* d_ct_in, const uint64_t*
             rc = rotate_hoisted_internal(ctx, cur, ctw, R, ctw, (size_t)blocks * ctw, blocks, level, ids.data(), n_keys, ks, st);
             if (rc != FESC_OK) return rc;
         }
-        FESC_CHECK_CUDA(ctx, cudaMemsetAsync(acc, 0, (size_t)blocks * ctw * sizeof(u64), st));
-        auto mac = [&](const u64* ct, const u64* pt) {
-            return fesc_ct_pt_mac(ctx, (const uint64_t*)ct, (const uint64_t*)pt, mask_stride, (uint64_t*)acc, blocks, level, stream);
-        };
-        if ((rc = mac(cur, masks)) != FESC_OK) return rc;
+        MaskedSum s;
+        s.n = 0;
+        auto term = [&](const u64* ct, uint32_t mask) { s.src[s.n] = ct, s.pt[s.n++] = masks + (size_t)mask * ptw; };
+        term(cur, 0);
         for (uint32_t r = 1; r < d; r++) {
-            if ((rc = mac(R + (size_t)(r - 1) * blocks * ctw, masks + (size_t)r * ptw)) != FESC_OK) return rc;
-            if (tb > 0) {
-                rc = mac(Rprev + (size_t)(taps + r - 1) * blocks * ctw, masks + (size_t)(d - 1 + r) * ptw);
-                if (rc != FESC_OK) return rc;
-            }
+            term(R + (size_t)(r - 1) * blocks * ctw, r);
+            if (tb > 0) term(Rprev + (size_t)(taps + r - 1) * blocks * ctw, d - 1 + r);
         }
-        prof_begin(ctx, PF_POINTWISE, st);
-        launch(k_ct_add_pt, dim3((N + 255) / 256, level, blocks), 256, 0, st, acc, ctw, (const u64*)d_bias, ptw, ctx->d_pc, N);
-        prof_end(ctx, PF_POINTWISE, st);
-        FESC_CHECK_CUDA(ctx, cudaGetLastError());
+        if ((rc = masked_sum(ctx, s, ctw, mask_stride, (const u64*)d_bias, ptw, acc, ctw, blocks, level, st)) != FESC_OK) return rc;
         rc = rescale_internal(ctx, acc, ctw, out + (size_t)tb * blocks * 2 * (level - 1) * N, blocks, level, ks, st);
         if (rc != FESC_OK) return rc;
     }

@@ -35,7 +35,7 @@ __device__ __forceinline__ void prefetch_l2(const u64* p) { asm volatile("prefet
 template <int A>
 __global__ void __launch_bounds__(COL_THREADS, 1024 / COL_THREADS)
     ntt16_cols_fwd(u64* __restrict__ data, const void* __restrict__ tw, const PrimeConst* __restrict__ pcs, RowList list,
-                   uint32_t y0, int in_double) {
+                   uint32_t y0, int in_double, const u64* __restrict__ centred, double centred_q) {
     pdl_begin();
     __shared__ u64 sm[COL_SMEM(NTT_COLS)];
     uint32_t pi;
@@ -46,10 +46,17 @@ __global__ void __launch_bounds__(COL_THREADS, 1024 / COL_THREADS)
     if constexpr (A == ROW_FP) {
         FpRow r{(const double*)tw + (size_t)pi * N16, pcs[pi].qd, pcs[pi].qinvd};
         double x[16];
+        if (centred) {                      // a row modulo another prime, centred, then folded modulo this one
+            const u64* s = centred + (size_t)(row / list.period) * N16 + blockIdx.x * NTT_COLS + col;
+            if (!DBG_REGION(centred + (size_t)(row / list.period) * N16, N16 * sizeof(u64))) return;
 #pragma unroll
-        for (int k = 0; k < 16; k++) {      // canonical words, or doubles with |x| <= q/2 from a conversion kernel
-            const u64 v = p[(16 * k + sub) * 256];
-            x[k] = in_double ? FpRow::value(v) : fp_from_u64(v);
+            for (int k = 0; k < 16; k++) x[k] = r.fold(fp_load(s[(16 * k + sub) * 256], centred_q));
+        } else {
+#pragma unroll
+            for (int k = 0; k < 16; k++) {  // canonical words, or doubles with |x| <= q/2 from a conversion kernel
+                const u64 v = p[(16 * k + sub) * 256];
+                x[k] = in_double ? FpRow::value(v) : fp_from_u64(v);
+            }
         }
         fwd_cols<NTT_COLS>(r, x, sm, col, sub, CtaBarrier());
 #pragma unroll
@@ -222,10 +229,10 @@ __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
     u64 g = 0;
     if (SRC) {                        // rows of the buffer: row = polynomial * period + limb
         const uint32_t poly = row / list.period, l = row - poly * list.period, k = poly / src.nb, b = poly - k * src.nb;
-        g = src.g[k];
+        g = k < KS_MAX_KEYS ? src.g[k] : 0;
         in = src.src + k * src.key_stride + b * src.stride + (size_t)l * N16;
-        own = src.own.ext + own_index(src.own, poly, l, N16) + blk * 512 + 2 * lane;
-        if (!DBG_REGION(in, N16 * sizeof(u64)) || !DBG_REGION(own - 2 * lane, 512 * sizeof(u64))) return;
+        if (src.own.ext) own = src.own.ext + own_index(src.own, poly, l, N16) + blk * 512 + 2 * lane;
+        if (!DBG_REGION(in, N16 * sizeof(u64)) || (own && !DBG_REGION(own - 2 * lane, 512 * sizeof(u64)))) return;
         at = blk * 512 + 2 * lane;
     }
     auto pair = [&](int j) {
@@ -242,7 +249,7 @@ __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
             ulonglong2 v = pair(j);
             v = make_ulonglong2(FpRow::bits(fp_load(v.x, r.q)), FpRow::bits(fp_load(v.y, r.q)));
             *reinterpret_cast<ulonglong2*>(s + 72 * j) = v;
-            if (SRC) *reinterpret_cast<ulonglong2*>(own + 64 * j) = v;
+            if (SRC && own) *reinterpret_cast<ulonglong2*>(own + 64 * j) = v;
         }
         __syncwarp();
         double x[16];
@@ -256,7 +263,7 @@ __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
         for (int j = 0; j < 8; j++) {
             const ulonglong2 v = pair(j);
             *reinterpret_cast<ulonglong2*>(s + 72 * j) = v;
-            if (SRC) *reinterpret_cast<ulonglong2*>(own + 64 * j) = v;
+            if (SRC && own) *reinterpret_cast<ulonglong2*>(own + 64 * j) = v;
         }
         __syncwarp();
         u64 x[16];
@@ -291,7 +298,7 @@ int ntt16_launch(fesc_ctx* ctx, u64* data, size_t rows, const RowMap& map, bool 
                            y, src);
                     launch(ntt16_cols_inv<ROW_FP>, gc, COL_THREADS, 0, st, data, ctx->d_itwf, ctx->d_pc, l, y, scale);
                 } else {
-                    if (!skip_cols) launch(ntt16_cols_fwd<ROW_FP>, gc, COL_THREADS, 0, st, data, ctx->d_twf, ctx->d_pc, l, y, in_double);
+                    if (!skip_cols) launch(ntt16_cols_fwd<ROW_FP>, gc, COL_THREADS, 0, st, data, ctx->d_twf, ctx->d_pc, l, y, in_double, fin.centred, fin.centred_q);
                     if (fin.acc) launch(ntt16_rows_fwd<ROW_FP, true>, gr, ROW_THREADS, 0, st, data, ctx->d_twf, ctx->d_pc, l, y, out_double, fin);
                     else launch(ntt16_rows_fwd<ROW_FP, false>, gr, ROW_THREADS, 0, st, data, ctx->d_twf, ctx->d_pc, l, y, out_double, fin);
                 }
@@ -300,7 +307,7 @@ int ntt16_launch(fesc_ctx* ctx, u64* data, size_t rows, const RowMap& map, bool 
                        src);
                 launch(ntt16_cols_inv<ROW_INT>, gc, COL_THREADS, 0, st, data, ctx->d_itw, ctx->d_pc, l, y, scale);
             } else {
-                if (!skip_cols) launch(ntt16_cols_fwd<ROW_INT>, gc, COL_THREADS, 0, st, data, ctx->d_tw, ctx->d_pc, l, y, 0);
+                if (!skip_cols) launch(ntt16_cols_fwd<ROW_INT>, gc, COL_THREADS, 0, st, data, ctx->d_tw, ctx->d_pc, l, y, 0, nullptr, 0.0);
                 launch(ntt16_rows_fwd<ROW_INT, false>, gr, ROW_THREADS, 0, st, data, ctx->d_tw, ctx->d_pc, l, y, 0, fin);
             }
             launches += skip_cols ? 1 : 2;

@@ -46,6 +46,60 @@ extern "C" int fesc_ct_pt_mac(fesc_ctx* ctx, const uint64_t* d_ct, const uint64_
 }
 
 // ---------------------------------------------------------------------------------------
+// out[b] = sum_j src_j[b] (.) pt_j[b] (+ add[b] on the first polynomial), up to 16 terms: every word of the sources is read once and the
+// accumulators stay in registers (a ct-pt MAC per term reads and writes them every time).  Two coefficients per thread.
+// Products are below 2^124: up to 16 of them fit 128 bits.
+// ---------------------------------------------------------------------------------------
+__global__ void __launch_bounds__(256) k_masked_sum(MaskedSum s, size_t src_stride, size_t pt_stride, const u64* __restrict__ add, size_t add_stride,
+                                                    u64* __restrict__ out, size_t out_stride, const PrimeConst* __restrict__ pcs, uint32_t N,
+                                                    uint32_t level) {
+    pdl_begin();
+    const uint32_t c = 2 * (blockIdx.x * blockDim.x + threadIdx.x), l = blockIdx.y, b = blockIdx.z;
+    if (c >= N) return;
+    const PrimeConst& pc = pcs[l];
+    const size_t poly = (size_t)level * N, o = (size_t)l * N;
+    for (int p = 0; p < 2; p++)
+        if (!DBG_REGION(out + b * out_stride + p * poly + o, N * sizeof(u64))) return;
+    if (add && !DBG_REGION(add + b * add_stride + o, N * sizeof(u64))) return;
+    for (uint32_t j = 0; j < s.n; j++)
+        if (!DBG_REGION(s.pt[j] + b * pt_stride + o, N * sizeof(u64)) || !DBG_REGION(s.src[j] + b * src_stride + o, N * sizeof(u64)) ||
+            !DBG_REGION(s.src[j] + b * src_stride + poly + o, N * sizeof(u64)))
+            return;
+    acc128 a[4] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}};
+#pragma unroll 4
+    for (uint32_t j = 0; j < s.n; j++) {
+        const u64* x = s.src[j] + b * src_stride + o + c;
+        const ulonglong2 w = __ldg(reinterpret_cast<const ulonglong2*>(s.pt[j] + b * pt_stride + o + c));
+        const ulonglong2 x0 = *reinterpret_cast<const ulonglong2*>(x), x1 = *reinterpret_cast<const ulonglong2*>(x + poly);
+        mac128(a[0], x0.x, w.x);
+        mac128(a[1], x0.y, w.y);
+        mac128(a[2], x1.x, w.x);
+        mac128(a[3], x1.y, w.y);
+    }
+    u64 r[4];
+#pragma unroll
+    for (int k = 0; k < 4; k++) r[k] = reduce128(a[k].hi, a[k].lo, pc);
+    if (add) {
+        const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(add + b * add_stride + o + c);
+        r[0] = addmod(r[0], v.x, pc.q), r[1] = addmod(r[1], v.y, pc.q);
+    }
+    u64* y = out + b * out_stride + o + c;
+    *reinterpret_cast<ulonglong2*>(y) = make_ulonglong2(r[0], r[1]);
+    *reinterpret_cast<ulonglong2*>(y + poly) = make_ulonglong2(r[2], r[3]);
+}
+int masked_sum(fesc_ctx* ctx, const MaskedSum& s, size_t src_stride, size_t pt_stride, const u64* add, size_t add_stride, u64* out,
+               size_t out_stride, uint32_t batch, uint32_t level, cudaStream_t st) {
+    const uint32_t N = ctx->N, threads = N / 2 < 256 ? N / 2 : 256;
+    prof_begin(ctx, PF_POINTWISE, st);
+    launch(k_masked_sum, dim3(N / 2 / threads, level, batch), threads, 0, st, s, src_stride, pt_stride, add, add_stride, out, out_stride, ctx->d_pc, N,
+           level);
+    prof_end(ctx, PF_POINTWISE, st);
+    FESC_CHECK_CUDA(ctx, cudaGetLastError());
+    ctx->counters[2] += (uint64_t)batch * s.n;
+    return FESC_OK;
+}
+
+// ---------------------------------------------------------------------------------------
 // NTT entry points
 // ---------------------------------------------------------------------------------------
 static int ntt_api(fesc_ctx* ctx, uint64_t* d_data, uint32_t batch, uint32_t first_limb, uint32_t n_limbs,
@@ -1477,28 +1531,35 @@ int rescale_internal(fesc_ctx* ctx, const u64* in, size_t in_stride, u64* out, u
             if ((rc = small_rescale(ctx, ib, in_stride, ob, out_stride, nb, level, scratch, st)) != FESC_OK) return rc;
             continue;
         }
-        prof_begin(ctx, PF_RESCALE, st);
-        launch(k_take_last, dim3(gx, nb * 2), 256, 0, st, ib, in_stride, scratch, N, level);
-        prof_end(ctx, PF_RESCALE, st);
+        // N = 2^16, FP64 rows: the inverse transform reads the last limbs in place, the forward transform's first pass takes the centred
+        // residues modulo every prime from them and its last pass stores (in - u) * q_last^-1
+        bool fuse = ctx->log_n == 16;
+        for (uint32_t i = 0; i < level; i++) fuse = fuse && ctx->q[i] < FESC_FP_LIMIT;
         RowMap m;
         m.period = 1;
         m.prime[0] = (uint8_t)(level - 1);
+        if (fuse) {
+            NttSource src;
+            src.src = ib + (size_t)(level - 1) * N, src.stride = (size_t)level * N, src.key_stride = in_stride, src.nb = 2;
+            if ((rc = ntt_launch(ctx, scratch, (size_t)nb * 2, m, true, st, false, false, nullptr, nullptr, false, &src)) != FESC_OK) return rc;
+            m.period = level - 1;
+            for (uint32_t i = 0; i + 1 < level; i++) m.prime[i] = (uint8_t)i;
+            NttFinish fin;
+            fin.acc = ib, fin.acc_stride = in_stride, fin.out = ob, fin.out_stride = out_stride, fin.cinv = tab->qinvd;
+            fin.level = level - 1, fin.acc_rows = level, fin.add_mask = 0;
+            fin.centred = scratch, fin.centred_q = (double)ctx->q[level - 1];
+            if ((rc = ntt_launch(ctx, ob, (size_t)nb * 2 * (level - 1), m, false, st, false, false, &fin)) != FESC_OK) return rc;
+            continue;
+        }
+        prof_begin(ctx, PF_RESCALE, st);
+        launch(k_take_last, dim3(gx, nb * 2), 256, 0, st, ib, in_stride, scratch, N, level);
+        prof_end(ctx, PF_RESCALE, st);
         if ((rc = ntt_launch(ctx, scratch, (size_t)nb * 2, m, true, st)) != FESC_OK) return rc;
         prof_begin(ctx, PF_RESCALE, st);
         launch(k_rescale_conv, dim3(gx, level - 1, nb * 2), 256, 0, st, scratch, ob, out_stride, tab, ctx->d_pc, N, level);
         prof_end(ctx, PF_RESCALE, st);
         m.period = level - 1;
         for (uint32_t i = 0; i + 1 < level; i++) m.prime[i] = (uint8_t)i;
-        // N = 2^16, FP64 rows: the last pass of the transform stores (in - u) * q_last^-1 itself
-        bool fuse = ctx->log_n == 16;
-        for (uint32_t i = 0; i + 1 < level; i++) fuse = fuse && ctx->q[i] < FESC_FP_LIMIT;
-        if (fuse) {
-            NttFinish fin;
-            fin.acc = ib, fin.acc_stride = in_stride, fin.out = ob, fin.out_stride = out_stride, fin.cinv = tab->qinvd;
-            fin.level = level - 1, fin.acc_rows = level, fin.add_mask = 0;
-            if ((rc = ntt_launch(ctx, ob, (size_t)nb * 2 * (level - 1), m, false, st, false, false, &fin)) != FESC_OK) return rc;
-            continue;
-        }
         if ((rc = ntt_launch(ctx, ob, (size_t)nb * 2 * (level - 1), m, false, st)) != FESC_OK) return rc;
         prof_begin(ctx, PF_RESCALE, st);
         launch(k_rescale_finish, dim3(gx, level - 1, nb * 2), 256, 0, st, ib, in_stride, ob, out_stride, tab, ctx->d_pc, N,

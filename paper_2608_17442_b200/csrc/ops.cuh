@@ -55,6 +55,13 @@ int rotate_multi_internal(fesc_ctx* ctx, const u64* in, size_t in_stride, size_t
                           cudaStream_t st, int accumulate);
 int giant_sum_deferred_internal(fesc_ctx* ctx, u64* acc, uint32_t n_terms, size_t ct_words, uint32_t batch,
                                 uint32_t level, uint32_t key_base, u64* scratch, cudaStream_t st);
+// out[b] = sum_j src_j[b] (.) pt_j[b] (+ add[b] on the first polynomial), at most 16 terms
+struct MaskedSum {
+    const u64 *src[16], *pt[16];
+    uint32_t n;
+};
+int masked_sum(fesc_ctx* ctx, const MaskedSum& s, size_t src_stride, size_t pt_stride, const u64* add, size_t add_stride, u64* out,
+               size_t out_stride, uint32_t batch, uint32_t level, cudaStream_t st);
 int rescale_internal(fesc_ctx* ctx, const u64* in, size_t in_stride, u64* out, uint32_t batch, uint32_t level,
                      u64* scratch, cudaStream_t st);
 int ctmul_internal(fesc_ctx* ctx, const u64* a, size_t a_stride, const u64* b, size_t b_stride, u64* out,

@@ -11,6 +11,7 @@
 #include <math.h>
 
 #include <map>
+#include <utility>
 
 #define FESC_DBG_FILE 6   // file id in the sites a debug build reports
 #include "ops.cuh"
@@ -106,38 +107,6 @@ __global__ void __launch_bounds__(256) k_ct_sum_into(const u64* __restrict__ a, 
     u64 s = acc[o];
     for (uint32_t i = 0; i < count; i++) s = addmod(s, a[i * a_stride + o], q);
     acc[o] = s;
-}
-
-// out[b] = sum_{j<terms} src_j[b] (.) mask_j on both polynomials (mask_j = masks + j*level*N, shared by the batch);
-// the products are summed in 128 bits and reduced once
-struct ClassSources {
-    const u64* src[16];
-};
-__global__ void __launch_bounds__(256) k_class_mac(ClassSources s, uint32_t terms, size_t src_stride,
-                                                   const u64* __restrict__ masks, u64* __restrict__ out,
-                                                   size_t out_stride, const PrimeConst* __restrict__ pcs, uint32_t N,
-                                                   uint32_t level) {
-    pdl_begin();
-    const uint32_t c = blockIdx.x * blockDim.x + threadIdx.x;
-    const uint32_t l = blockIdx.y, b = blockIdx.z;
-    if (c >= N) return;
-    const PrimeConst pc = pcs[l];
-    const size_t poly = (size_t)level * N, o = (size_t)l * N + c;
-    acc128 a0{0, 0}, a1{0, 0};
-    for (int p = 0; p < 2; p++)
-        if (!DBG_REGION(out + (size_t)b * out_stride + p * poly + o - c, N * sizeof(u64))) return;
-    for (uint32_t j = 0; j < terms; j++)
-        if (!DBG_REGION(masks + (size_t)j * poly + o - c, N * sizeof(u64)) || !DBG_REGION(s.src[j] + (size_t)b * src_stride + o - c, N * sizeof(u64)) ||
-            !DBG_REGION(s.src[j] + (size_t)b * src_stride + poly + o - c, N * sizeof(u64)))
-            return;
-    for (uint32_t j = 0; j < terms; j++) {
-        const u64 w = masks[(size_t)j * poly + o];
-        const u64* x = s.src[j] + (size_t)b * src_stride;
-        mac128(a0, x[o], w);
-        mac128(a1, x[poly + o], w);
-    }
-    out[(size_t)b * out_stride + o] = reduce128(a0.hi, a0.lo, pc);
-    out[(size_t)b * out_stride + poly + o] = reduce128(a1.hi, a1.lo, pc);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -340,7 +309,7 @@ struct Exec {
     // a + rot(a, d) + rot(a, 2d) + rot(a, 3d), d = unit * 2^b, with one decomposition and one division by P.
     void chain(const Arr& a, int64_t unit, uint32_t steps) {
         size_t mark = top;
-        Arr t = alloc(a.count, a.level);
+        Arr t = alloc(a.count, a.level), cur = a, other = t;      // the sum moves between the two buffers
         uint32_t b = 0;
         while (b < steps && ok()) {
             const int64_t d = unit * (int64_t)(1u << b);
@@ -348,16 +317,17 @@ struct Exec {
                 if (!key_ok(d) || !key_ok(2 * d) || !key_ok(3 * d)) break;
                 if (!dry) {
                     const uint32_t ids[3] = {key_for(d), key_for(2 * d), key_for(3 * d)};
-                    rc = rotate_sum_hoisted_internal(ctx, a.p, a.stride, t.p, t.stride, a.count, a.level, ids, 3, ks, st);
-                    copy(t, a);
+                    rc = rotate_sum_hoisted_internal(ctx, cur.p, cur.stride, other.p, other.stride, cur.count, cur.level, ids, 3, ks, st);
                 }
+                std::swap(cur, other);
                 b += 2;
             } else {
-                rot(a, d, t);
-                add(a, t, a);
+                rot(cur, d, other);
+                add(cur, other, cur);
                 b += 1;
             }
         }
+        copy(cur, a);
         top = mark;
     }
     void fill_right(const Arr& a, uint32_t unit, uint32_t steps) { chain(a, -(int64_t)unit, steps); }
@@ -386,16 +356,15 @@ struct Exec {
         }
         Arr acc = alloc(cnt, lvl), res = alloc(cnt, lvl - 1);
         for (uint32_t c = 0; c < G && ok(); c++) {
-            if (!dry) {
-                ClassSources cs_;
+            if (!dry && ok()) {
+                MaskedSum s;
+                s.n = G;
                 for (uint32_t j = 0; j < G; j++) {
                     const int k = (int)c - (int)j;
-                    cs_.src[j] = k == 0 ? grp.p : rots.p + (size_t)(k > 0 ? k - 1 : (int)G - 2 - k) * cnt * rots.stride;
+                    s.src[j] = k == 0 ? grp.p : rots.p + (size_t)(k > 0 ? k - 1 : (int)G - 2 - k) * cnt * rots.stride;
+                    s.pt[j] = masks + (size_t)j * lvl * N;
                 }
-                prof_begin(ctx, PF_POINTWISE, st);
-                launch(k_class_mac, grid(lvl, cnt), 256, 0, st, cs_, G, grp.stride, masks, acc.p, acc.stride, ctx->d_pc, N, lvl);
-                prof_end(ctx, PF_POINTWISE, st);
-                ctx->counters[2] += (uint64_t)G * cnt;
+                rc = masked_sum(ctx, s, grp.stride, 0, nullptr, 0, acc.p, acc.stride, cnt, lvl, st);
             }
             rescale(acc, res);
             deliver(c, res);
