@@ -29,8 +29,6 @@ __device__ __forceinline__ uint32_t list_row(const RowList& list, uint32_t y, ui
     return rep * list.period + list.row[e];
 }
 
-__device__ __forceinline__ void prefetch_l2(const u64* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
-
 // grid = (256 / NTT_COLS, rows)
 template <int A>
 __global__ void __launch_bounds__(COL_THREADS, 1024 / COL_THREADS)

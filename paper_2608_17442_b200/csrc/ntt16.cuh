@@ -181,6 +181,7 @@ __device__ __forceinline__ void fold16(const R& r, typename R::T (&x)[16]) {
 template <int COLS>
 __device__ __forceinline__ uint32_t col_slot(uint32_t hi, uint32_t col) { return hi * COLS + (hi >> 4) * COLS + col; }
 
+__device__ __forceinline__ void prefetch_l2(const u64* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 // all a transform needs of a context
 struct SmallTables {
     const double *twf, *itwf;

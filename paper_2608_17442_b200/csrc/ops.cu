@@ -837,9 +837,14 @@ __global__ void __launch_bounds__(256) k_moddown_finish(const u64* __restrict__ 
     *o = v;
 }
 
+// Whether the data rows of the converted digits can stay half transformed (`open`) for an inner product that finishes them itself
+static bool rows_split(const fesc_ctx* ctx, uint32_t level);
+static bool ks_open(const fesc_ctx* ctx, uint32_t level) { return modup16_supported(ctx, level) && rows_split(ctx, level); }
+
 // Steps 1-3 of the key switch: ws.dcoef -> COEFF, digit-wise basis extension into ws.ext, NTT of the
 // converted rows.  The result (ws.ext, own-limb rows included) can serve several keys (hoisted rotations).
-static int ks_decompose(fesc_ctx* ctx, const KsScratch& ws, uint32_t level, uint32_t batch, cudaStream_t st, const NttSource* source = nullptr) {
+static int ks_decompose(fesc_ctx* ctx, const KsScratch& ws, uint32_t level, uint32_t batch, cudaStream_t st, const NttSource* source = nullptr,
+                        bool open = false) {
     const uint32_t N = ctx->N, K = ctx->n_p, nq = ctx->n_q, alpha = ctx->alpha;
     const uint32_t beta = (level + alpha - 1) / alpha, rows = level + K;
     const uint32_t gx = (N + 255) / 256;
@@ -865,6 +870,9 @@ static int ks_decompose(fesc_ctx* ctx, const KsScratch& ws, uint32_t level, uint
         prof_begin(ctx, PF_MODUP, st);
         if ((rc = modup16_cols_launch(ctx, ws.dcoef, ws.ext, level, batch, st)) != FESC_OK) return rc;
         prof_end(ctx, PF_MODUP, st);
+        if (open)
+            for (uint32_t j = 0; j < beta; j++)
+                for (uint32_t t = 0; t < level; t++) m.prime[j * rows + t] = 0xFF;
         return ntt_launch(ctx, ws.ext, (size_t)batch * beta * rows, m, false, st, false, true, nullptr, nullptr, true);
     }
     const ModUpDigit* tab = ctx->tabs.d_modup + (size_t)(level - 1) * ctx->beta_max;
@@ -898,15 +906,16 @@ static bool rows_split(const fesc_ctx* ctx, uint32_t level) {
 }
 // Step 4: inner products of the sources `S` (converted digits, key, Galois element each) summed into ws.acc;
 // accumulate != 0 adds to what ws.acc holds (sums over several passes before one division by P); last: no further pass follows;
-// separate: the sources are not summed, source s has its own batch of accumulators.
+// separate: the sources are not summed, source s has its own batch of accumulators; open: the data rows of the digits await the last
+// pass of their transform.
 static int ks_inner_multi(fesc_ctx* ctx, const KsScratch& ws, const InnerSrcs& S, uint32_t level, uint32_t batch,
-                          cudaStream_t st, int accumulate, int last = 1, bool separate = false) {
+                          cudaStream_t st, int accumulate, int last = 1, bool separate = false, bool open = false) {
     if (small_ring(ctx)) return small_inner(ctx, ws, S, level, batch, st, accumulate, last);
     const uint32_t N = ctx->N, K = ctx->n_p, nq = ctx->n_q, alpha = ctx->alpha;
     const uint32_t beta = (level + alpha - 1) / alpha, rows = level + K;
     const uint32_t gx = (N + 255) / 256;
     prof_begin(ctx, PF_INNER, st);
-    const bool use_tma = S.n == 1 && !separate && getenv("FESC_INNER_TMA") != nullptr;   // read per call so a test can switch it
+    const bool use_tma = S.n == 1 && !separate && !open && getenv("FESC_INNER_TMA") != nullptr;   // read per call so a test can switch it
 #define INNER(BT_, PATH_, ROW0_, NROWS_)                                                                        \
     do {                                                                                                        \
         const uint32_t tiles = (batch + BT_ - 1) / BT_;                                                         \
@@ -926,6 +935,12 @@ static int ks_inner_multi(fesc_ctx* ctx, const KsScratch& ws, const InnerSrcs& S
         const uint32_t grid = n_tiles < (uint32_t)sms ? n_tiles : (uint32_t)sms;
         launch(k_inner_tma<4>, grid, 256, smem, st, S.s[0].ext, S.s[0].key, ws.acc, ctx->d_pc, N, level, nq, K, alpha, beta,
                                                  batch, ctx->log_n, S.s[0].g, accumulate, n_tiles, ctx->d_status, ctx->log_n == 16);
+    } else if (open) {
+        const int rc = rows_inner_launch(ctx, S, ws.acc, level, batch, accumulate, separate, st);
+        if (rc != FESC_OK) return rc;
+        if (batch >= 3) INNER(4, 2, level, K);
+        else if (batch == 2) INNER(2, 2, level, K);
+        else INNER(1, 2, level, K);
     } else if (split) {
         if (batch >= 3) INNER(4, 1, 0, level);
         else if (batch == 2) INNER(2, 1, 0, level);
@@ -944,11 +959,11 @@ static int ks_inner_multi(fesc_ctx* ctx, const KsScratch& ws, const InnerSrcs& S
 }
 // one source: ws.ext with `key`, digits read through the Galois permutation of g when g != 0
 static int ks_inner(fesc_ctx* ctx, const KsScratch& ws, const EvalKey& key, uint32_t level, uint32_t batch,
-                    cudaStream_t st, u64 g, int accumulate) {
+                    cudaStream_t st, u64 g, int accumulate, bool open = false) {
     InnerSrcs S;
     S.n = 1;
     S.s[0] = InnerSrc{ws.ext, key.d_key, g};
-    return ks_inner_multi(ctx, ws, S, level, batch, st, accumulate);
+    return ks_inner_multi(ctx, ws, S, level, batch, st, accumulate, 1, false, open);
 }
 
 static u64 galois_inverse(u64 g, uint32_t log_n) {      // modulo 2N, g odd: Newton's iteration doubles the correct bits
@@ -1081,8 +1096,8 @@ static int ks_moddown(fesc_ctx* ctx, const KsScratch& ws, uint32_t level, uint32
 
 // Steps 4-5 for one key.
 static int ks_apply(fesc_ctx* ctx, const KsScratch& ws, const EvalKey& key, uint32_t level, uint32_t batch, u64* out,
-                    size_t out_stride, int add_mask, cudaStream_t st, u64 g) {
-    int rc = ks_inner(ctx, ws, key, level, batch, st, g, 0);
+                    size_t out_stride, int add_mask, cudaStream_t st, u64 g, bool open = false) {
+    int rc = ks_inner(ctx, ws, key, level, batch, st, g, 0, open);
     if (rc != FESC_OK) return rc;
     return ks_moddown(ctx, ws, level, batch, out, out_stride, add_mask, st);
 }
@@ -1091,9 +1106,10 @@ static int ks_apply(fesc_ctx* ctx, const KsScratch& ws, const EvalKey& key, uint
 // dcoef (a copy of d, consumed), ext, acc, u.
 static int key_switch_chunk(fesc_ctx* ctx, const KsScratch& ws, const EvalKey& key, uint32_t level, uint32_t batch,
                             u64* out, size_t out_stride, int add_mask, cudaStream_t st) {
-    int rc = ks_decompose(ctx, ws, level, batch, st);
+    const bool open = ks_open(ctx, level);
+    int rc = ks_decompose(ctx, ws, level, batch, st, nullptr, open);
     if (rc != FESC_OK) return rc;
-    return ks_apply(ctx, ws, key, level, batch, out, out_stride, add_mask, st, 0);
+    return ks_apply(ctx, ws, key, level, batch, out, out_stride, add_mask, st, 0, open);
 }
 
 
@@ -1105,14 +1121,14 @@ __global__ void k_hoist_prepare(const u64* in, size_t in_stride, u64* out0, size
 // Steps 1-3 for the second polynomial of every ciphertext at in + k * key_stride + b * in_stride, read through the permutation of g[k]
 // (g = nullptr: none).  More than one key: N = 2^16 only.
 static int ks_start(fesc_ctx* ctx, const KsScratch& ws, const u64* in, size_t in_stride, const u64* g, uint32_t level, uint32_t batch,
-                    cudaStream_t st, uint32_t n_keys = 1, size_t key_stride = 0) {
+                    cudaStream_t st, bool open, uint32_t n_keys = 1, size_t key_stride = 0) {
     const u64* c1 = in + (size_t)level * ctx->N;
     if (small_ring(ctx)) return small_decompose(ctx, ws, c1, in_stride, true, g ? g[0] : 0, level, batch, st);
     if (ctx->log_n == 16) {
         NttSource src;
         src.src = c1, src.stride = in_stride, src.key_stride = key_stride, src.nb = batch, src.own = own_rows(ctx, ws, level);
         for (uint32_t k = 0; k < n_keys && g; k++) src.g[k] = g[k];
-        return ks_decompose(ctx, ws, level, batch * n_keys, st, &src);
+        return ks_decompose(ctx, ws, level, batch * n_keys, st, &src, open);
     }
     const dim3 grid((ctx->N + 255) / 256, level, batch);
     prof_begin(ctx, PF_AUTOM, st);
@@ -1184,6 +1200,7 @@ int rotate_multi_internal(fesc_ctx* ctx, const u64* in, size_t in_stride, size_t
                           size_t out_key_stride, uint32_t batch, uint32_t level, const uint32_t* key_ids, uint32_t n_keys, u64* scratch,
                           cudaStream_t st, int accumulate) {
     const bool fused = moddown_fused(ctx, level);     // the division's epilogue adds sigma_g(c0) straight from the input
+    const bool open = ks_open(ctx, level);
     KsCut cut = ks_cut_rotate(ctx, batch, n_keys);
     const KsScratch ws = ks_scratch_carve(ctx, scratch, level, cut);
     if (!fused) cut.keys = 1;
@@ -1196,12 +1213,12 @@ int rotate_multi_internal(fesc_ctx* ctx, const u64* in, size_t in_stride, size_t
             const u64* ib = in + k0 * in_key_stride + (size_t)b0 * in_stride;
             u64* ob = out + k0 * out_key_stride + (size_t)b0 * out_stride;
             if (fused) {
-                if ((rc = ks_start(ctx, ws, ib, in_stride, keys.g, level, nb, st, keys.n, in_key_stride)) != FESC_OK) return rc;
+                if ((rc = ks_start(ctx, ws, ib, in_stride, keys.g, level, nb, st, open, keys.n, in_key_stride)) != FESC_OK) return rc;
                 InnerSrcs S;
                 S.n = keys.n;
                 const size_t ext_words = (size_t)nb * ((level + ctx->alpha - 1) / ctx->alpha) * (level + ctx->n_p) * ctx->N;
                 for (uint32_t k = 0; k < keys.n; k++) S.s[k] = InnerSrc{ws.ext + k * ext_words, keys.key[k], 0};
-                if ((rc = ks_inner_multi(ctx, ws, S, level, nb, st, 0, 1, keys.n > 1)) != FESC_OK) return rc;
+                if ((rc = ks_inner_multi(ctx, ws, S, level, nb, st, 0, 1, keys.n > 1, open)) != FESC_OK) return rc;
                 KsRot rot;
                 rot.src = ib, rot.stride = in_stride, rot.key_stride = in_key_stride, rot.g = keys.g;
                 rc = ks_moddown(ctx, ws, level, nb, ob, out_stride, accumulate ? 3 : 0, st, rot, keys.n, out_key_stride);
@@ -1274,6 +1291,7 @@ int giant_sum_deferred_internal(fesc_ctx* ctx, u64* acc, uint32_t n_terms, size_
         if (!ctx->keys.count(key_base + p) || key_base + p == FESC_RELIN_KEY_ID)
             return fesc_fail(ctx, FESC_ENOKEY, "giant steps: no Galois key " + std::to_string(key_base + p));
     const KsCut cut = ks_cut_giant(ctx, batch, n_terms);
+    const bool open = ks_open(ctx, level);
     KsScratch ws = ks_scratch_carve(ctx, scratch, level, cut);
     const size_t stride = (size_t)n_terms * ct_words;
     const size_t ext_words = (size_t)((level + ctx->alpha - 1) / ctx->alpha) * (level + ctx->n_p) * ctx->N;
@@ -1309,16 +1327,16 @@ int giant_sum_deferred_internal(fesc_ctx* ctx, u64* acc, uint32_t n_terms, size_
             S.n = np;
             for (uint32_t s = 0; s < np; s++) S.s[s] = InnerSrc{ws.ext + s * nb * ext_words, keys.key[s], 0};
             if (ctx->log_n == 16 && nb * np <= cut.src) {
-                rc = ks_start(ctx, ws, base + (size_t)p0 * ct_words, stride, keys.g, level, nb, st, np, ct_words);
+                rc = ks_start(ctx, ws, base + (size_t)p0 * ct_words, stride, keys.g, level, nb, st, open, np, ct_words);
                 if (rc != FESC_OK) return rc;
             } else {
                 for (uint32_t s = 0; s < np; s++) {
                     KsScratch wss = ws;
                     wss.ext = ws.ext + s * nb * ext_words;
-                    if ((rc = ks_start(ctx, wss, base + (size_t)(p0 + s) * ct_words, stride, &keys.g[s], level, nb, st)) != FESC_OK) return rc;
+                    if ((rc = ks_start(ctx, wss, base + (size_t)(p0 + s) * ct_words, stride, &keys.g[s], level, nb, st, open)) != FESC_OK) return rc;
                 }
             }
-            if ((rc = ks_inner_multi(ctx, ws, S, level, nb, st, p0 > 1, p0 + np == n_terms)) != FESC_OK) return rc;
+            if ((rc = ks_inner_multi(ctx, ws, S, level, nb, st, p0 > 1, p0 + np == n_terms, false, open)) != FESC_OK) return rc;
         }
         int rc = ks_moddown(ctx, ws, level, nb, base, stride, 3, st);
         if (rc != FESC_OK) return rc;
@@ -1342,7 +1360,7 @@ int rotate_hoisted_internal(fesc_ctx* ctx, const u64* in, size_t in_stride, u64*
         const uint32_t nb = batch - b0 < cut.nb ? batch - b0 : cut.nb;
         dim3 g((ctx->N + 255) / 256, level, nb);
         const u64* ib = in + (size_t)b0 * in_stride;
-        int rc = ks_start(ctx, ws, ib, in_stride, nullptr, level, nb, st);
+        int rc = ks_start(ctx, ws, ib, in_stride, nullptr, level, nb, st, false);
         if (rc != FESC_OK) return rc;
         for (uint32_t k0 = 0; k0 < n_keys; k0 += cut.keys) {
             KsKeys keys;
@@ -1415,7 +1433,7 @@ int rotate_sum_hoisted_internal(fesc_ctx* ctx, const u64* in, size_t in_stride, 
         prof_begin(ctx, PF_AUTOM, st);
         launch(k_rotsum_prepare, g, 256, 0, st, ib, in_stride, ob, out_stride, ctx->log_n, level, gs, ctx->d_pc);
         prof_end(ctx, PF_AUTOM, st);
-        int rc = ks_start(ctx, ws, ib, in_stride, nullptr, level, nb, st);
+        int rc = ks_start(ctx, ws, ib, in_stride, nullptr, level, nb, st, false);
         if (rc != FESC_OK) return rc;
         InnerSrcs S;                                   // one converted polynomial, read through every key's permutation
         S.n = n_keys;
