@@ -230,6 +230,7 @@ struct ModUpDigit {
     u64 mat[FESC_MAX_ALPHA][FESC_MAX_PRIMES];        // (Q_j/q_i) mod q_t, t = prime index
     double matd[FESC_MAX_ALPHA][FESC_MAX_PRIMES];    // the same as doubles (exact for targets below 2^53)
     ModUpTerm term[FESC_MAX_ALPHA][FESC_MAX_PRIMES]; // the same centred (modup16.cu)
+    double start[FESC_MAX_PRIMES];                   // -2^52 times the sum of a target's mq
 };
 // Division by P = product of the special primes p_k.
 struct ModDownTab {

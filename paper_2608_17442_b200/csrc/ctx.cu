@@ -351,6 +351,7 @@ static int build_tables(fesc_ctx* ctx) {
                     d.term[a][t].m = m > q[t] / 2 ? -(long long)(q[t] - m) : (long long)m;
                     d.term[a][t].mq = (double)((long double)d.term[a][t].m / (long double)q[t]);
                 }
+                for (uint32_t t = 0; t < np; t++) d.start[t] -= 4503599627370496.0 * d.term[a][t].mq;
                 d.inv[a] = h_inv(d.mat[a][i], q[i]);
                 d.invs[a] = h_shoup(d.inv[a], q[i]);
                 scale[(size_t)(level - 1) * nq + i] = inv_scale(ctx->pc[i], d.inv[a]);

@@ -6,7 +6,7 @@
 // (level + K - n_src) rows per digit.
 //
 // The sum is an exact mixed-pipe product: its quotient c = rint(sum_a y_a (m_a / q)) comes from the FP64 pipe (one
-// multiply-add per term, m centred; |sum| < 2^51, so the error stays below 0.75 and |v| <= 1.25 q < 2^63), its value
+// multiply-add per term, m centred; the roundings at up to 2^53 add up to less than 2.63, so |v| <= 2.63 q < 2^63), its value
 // v = sum_a y_a m_a - c q from wrapping 64-bit integer products on the multiplier pipe, which the FP64 butterflies leave idle.
 //
 // A CTA owns 4 columns of one digit of one ciphertext: the source columns (8 KB per limb) are read once into shared memory
@@ -35,39 +35,42 @@ struct GroupBarrier {
 #define FP_MAGIC 6755399441055744.0      // 1.5 * 2^52: the low mantissa bits of FP_MAGIC + c hold the integer c, |c| < 2^51
 #define FP_MAGIC_HI 0x43380000u
 
-// v[0..3] = sum_a y_a m_a - c q (two's complement) for the points p, p + 16 MU_COLS, ... of the source columns
+// v[0..3] = sum_a y_a m_a - c q (two's complement) for the points p, p + 16 MU_COLS, ... of the source columns.  The columns hold
+// the doubles 2^52 + y, whose low 50 bits are y: one word serves both pipes without a conversion.  What 2^52 adds to the FP64 sum is
+// in its starting value c0, what the exponent bits add to the cross products (weight 2^32, modulo 2^32) is taken off at the end.
 template <int A>
 __device__ __forceinline__ void convert4(const u64* p, uint32_t n_src, const ModUpTerm (*__restrict__ term)[FESC_MAX_PRIMES], uint32_t pt,
-                                         u64 q, u64* v) {
+                                         double c0, u64 q, u64* v) {
     u64 acc[4];            // low product words, and the cross terms of weight 2^32 apart from them
-    uint32_t cross[4];
+    uint32_t cross[4], msum = 0;
     double s[4];
 #pragma unroll
-    for (int e = 0; e < 4; e++) acc[e] = 0, cross[e] = 0, s[e] = 0.0;
+    for (int e = 0; e < 4; e++) acc[e] = 0, cross[e] = 0, s[e] = c0;
 #pragma unroll
     for (int a = 0; a < A; a++) {
         if (a >= n_src) break;
         const ulonglong2 t = __ldg(reinterpret_cast<const ulonglong2*>(&term[a][pt]));
         const uint32_t ml = (uint32_t)t.x, mh = (uint32_t)(t.x >> 32);
         const double mq = __longlong_as_double((long long)t.y);
+        msum += ml;
 #pragma unroll
         for (int e = 0; e < 4; e++) {
             const u64 y = p[a * MU_SRC + e * 16 * MU_COLS];
             const uint32_t yl = (uint32_t)y, yh = (uint32_t)(y >> 32);
-            s[e] = __fma_rn(fp_from_u64(y), mq, s[e]);
+            s[e] = __fma_rn(__longlong_as_double((long long)y), mq, s[e]);
             asm("mad.wide.u32 %0, %1, %2, %0;" : "+l"(acc[e]) : "r"(yl), "r"(ml));
             asm("mad.lo.u32 %0, %1, %2, %0;" : "+r"(cross[e]) : "r"(yl), "r"(mh));
             asm("mad.lo.u32 %0, %1, %2, %0;" : "+r"(cross[e]) : "r"(yh), "r"(ml));
         }
     }
     const u64 nq = 0 - q;
-    const uint32_t ql = (uint32_t)nq, qh = (uint32_t)(nq >> 32);
+    const uint32_t ql = (uint32_t)nq, qh = (uint32_t)(nq >> 32), corr = 0u - 0x43300000u * msum;
 #pragma unroll
     for (int e = 0; e < 4; e++) {
         const u64 c = (u64)__double_as_longlong(__dadd_rn(s[e], FP_MAGIC));
         const uint32_t cl = (uint32_t)c, ch = (uint32_t)(c >> 32) - FP_MAGIC_HI;
         asm("mad.wide.u32 %0, %1, %2, %0;" : "+l"(acc[e]) : "r"(cl), "r"(ql));
-        const uint32_t hi = (uint32_t)(acc[e] >> 32) + (cross[e] + cl * qh + ch * ql);
+        const uint32_t hi = (uint32_t)(acc[e] >> 32) + (cross[e] + corr + cl * qh + ch * ql);
         v[e] = ((u64)hi << 32) | (uint32_t)acc[e];
     }
 }
@@ -90,8 +93,9 @@ __global__ void __launch_bounds__(MU_THREADS, 2)
         return;                                     // the same for the whole CTA
     for (uint32_t i = tid; i < n_src * (MU_SRC / 2); i += MU_THREADS) {
         const uint32_t a = i / (MU_SRC / 2), r = (i / (MU_COLS / 2)) & 255, c = 2 * (i % (MU_COLS / 2));
+        const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(src + (size_t)a * N16 + r * 256 + c);
         *reinterpret_cast<ulonglong2*>(smem + a * MU_SRC + r * MU_COLS + c) =
-            *reinterpret_cast<const ulonglong2*>(src + (size_t)a * N16 + r * 256 + c);
+            make_ulonglong2(v.x | 0x4330000000000000ull, v.y | 0x4330000000000000ull);
     }
     if (tid == 0) next = 0;
     __syncthreads();
@@ -108,13 +112,14 @@ __global__ void __launch_bounds__(MU_THREADS, 2)
         const uint32_t t = o < K ? level + o : (d < first ? d : d + n_src), pt = o < K ? n_q + o : t;
         u64* p = out + (size_t)t * N16 + col;
         const u64 q = pcs[pt].q;
+        const double c0 = __ldg(&dg->start[pt]);
         if (q < FESC_FP_LIMIT) {
             FpRow r{twf + (size_t)pt * N16, pcs[pt].qd, pcs[pt].qinvd};
             double x[16];
 #pragma unroll
             for (int k = 0; k < 16; k += 4) {
                 u64 v[4];
-                convert4<A>(ys + k * 16 * MU_COLS, n_src, dg->term, pt, q, v);
+                convert4<A>(ys + k * 16 * MU_COLS, n_src, dg->term, pt, c0, q, v);
 #pragma unroll
                 for (int e = 0; e < 4; e++) x[k + e] = __dadd_rn(FpRow::value(v[e] + ((u64)FP_MAGIC_HI << 32)), -FP_MAGIC);
             }
@@ -126,9 +131,9 @@ __global__ void __launch_bounds__(MU_THREADS, 2)
             u64 x[16];
 #pragma unroll
             for (int k = 0; k < 16; k += 4) {
-                convert4<A>(ys + k * 16 * MU_COLS, n_src, dg->term, pt, q, x + k);
+                convert4<A>(ys + k * 16 * MU_COLS, n_src, dg->term, pt, c0, q, x + k);
 #pragma unroll
-                for (int e = 0; e < 4; e++) x[k + e] += r.q2;      // |v| <= 1.25 q: below 4q
+                for (int e = 0; e < 4; e++) x[k + e] = csub(x[k + e] + 3 * q, r.q2);      // |v| <= 2.63 q: below 4q
             }
             fwd_cols<MU_COLS>(r, x, sm, col, sub, bar);
 #pragma unroll
@@ -141,6 +146,8 @@ bool modup16_supported(const fesc_ctx* ctx, uint32_t level) {
     if (ctx->log_n != 16 || ctx->alpha > 4 || ctx->n_p > 4) return false;
     for (uint32_t i = 0; i < level; i++)
         if (ctx->q[i] >= FESC_FP_LIMIT) return false;
+    for (uint32_t k = 0; k < ctx->n_p; k++)
+        if (ctx->q[ctx->n_q + k] >= (1ull << 61)) return false;
     return true;
 }
 
