@@ -242,6 +242,7 @@ struct ModDownTab {
     u64 pinv[FESC_MAX_PRIMES], pinvs[FESC_MAX_PRIMES];   // P^-1 mod q_i
     double matd[FESC_MAX_SPECIAL][FESC_MAX_PRIMES], mat30d[FESC_MAX_SPECIAL][FESC_MAX_PRIMES];   // as doubles
     double wrapd[FESC_MAX_SPECIAL + 1][FESC_MAX_PRIMES], pinvd[FESC_MAX_PRIMES];
+    ModUpTerm term[4][FESC_MAX_PRIMES];                  // (P/p_k) mod q_i centred, and divided by 2^10 q_i (modup16.cu)
 };
 // Rescale from level l (drops limb l-1); entry index l.
 struct RescaleTab {

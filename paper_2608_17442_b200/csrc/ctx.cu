@@ -380,6 +380,10 @@ static int build_tables(fesc_ctx* ctx) {
             md.mat[k][i] = m;
             md.mat30[k][i] = h_mul(m, (1ull << 30) % q[i], q[i]);
             md.matd[k][i] = (double)md.mat[k][i];
+            if (k < 4) {
+                md.term[k][i].m = m > q[i] / 2 ? -(long long)(q[i] - m) : (long long)m;
+                md.term[k][i].mq = (double)((long double)md.term[k][i].m / ((long double)q[i] * 1024));
+            }
             md.mat30d[k][i] = (double)md.mat30[k][i];
         }
     }

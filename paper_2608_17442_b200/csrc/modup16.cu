@@ -169,3 +169,131 @@ int modup16_cols_launch(fesc_ctx* ctx, const u64* y, u64* ext, uint32_t level, u
     if (ctx->alpha <= 2) return launch_modup<2>(ctx, y, ext, level, batch, st);
     return launch_modup<4>(ctx, y, ext, level, batch, st);
 }
+
+// ---------------------------------------------------------------------------------------
+// Division by P, conversion step fused with the first pass of the forward transform in the same way:
+//   u_i = sum_k y_k m_k mod q_i,  y_k = r_k (P/p_k)^-1 mod p_k centred (the constant rides on the inverse transform's last stage),
+//   m_k = (P/p_k) mod q_i.
+// The sources have 60 bits, so the quotient is taken in units of 2^10: c = rint(sum_k y_k (m_k / (q 2^10))), |c| <= 2^50, and
+// v = sum_k y_k m_k - c 2^10 q is below 2.1 2^10 q < 2^62; a second quotient from the high word of v leaves |v| <= 0.7 q.  Per source
+// that is one FP64 multiply-add, one wide and two narrow integer ones, and no counting of negative residues.
+// ---------------------------------------------------------------------------------------
+#define MD_GROUPS 3
+#define MD_THREADS (MD_GROUPS * MU_TARGET_THREADS)
+
+template <int A>
+__global__ void __launch_bounds__(MD_THREADS, 2)
+    k_moddown_cols(const u64* __restrict__ acc, u64* __restrict__ u, const ModDownTab* __restrict__ tab, const double* __restrict__ twf,
+                   const PrimeConst* __restrict__ pcs, uint32_t level, uint32_t n_q, uint32_t K, uint32_t splits) {
+    pdl_begin();
+    extern __shared__ __align__(16) u64 smem[];      // [A][MU_SRC] sources, the same as doubles, then one exchange buffer per group
+    __shared__ uint32_t next, taken[MD_GROUPS];
+    const uint32_t tid = threadIdx.x, tile = blockIdx.x / splits, part = blockIdx.x % splits, bp = blockIdx.y;
+    const u64* src = acc + ((size_t)bp * (level + K) + level) * N16 + tile * MU_COLS;
+    u64* out = u + (size_t)bp * level * N16 + tile * MU_COLS;
+    if (!DBG_REGION(tab, sizeof(ModDownTab)) || !DBG_REGION(src - tile * MU_COLS, (size_t)K * N16 * sizeof(u64)) ||
+        !DBG_REGION(out - tile * MU_COLS, (size_t)level * N16 * sizeof(u64)))
+        return;                                     // the same for the whole CTA
+    double* smd = reinterpret_cast<double*>(smem + A * MU_SRC);
+    for (uint32_t i = tid; i < A * (MU_SRC / 2); i += MD_THREADS) {
+        const uint32_t a = i / (MU_SRC / 2), r = (i / (MU_COLS / 2)) & 255, c = 2 * (i % (MU_COLS / 2)), at = a * MU_SRC + r * MU_COLS + c;
+        ulonglong2 v = make_ulonglong2(0, 0);
+        if (a < K) {
+            v = *reinterpret_cast<const ulonglong2*>(src + (size_t)a * N16 + r * 256 + c);
+            const u64 p = pcs[n_q + a].q, half = tab->half[a];
+            if (v.x > half) v.x -= p;
+            if (v.y > half) v.y -= p;
+        }
+        *reinterpret_cast<ulonglong2*>(smem + at) = v;
+        *reinterpret_cast<double2*>(smd + at) = make_double2(__ll2double_rn((long long)v.x), __ll2double_rn((long long)v.y));
+    }
+    if (tid == 0) next = 0;
+    __syncthreads();
+    const uint32_t group = tid / MU_TARGET_THREADS, gt = tid % MU_TARGET_THREADS, col = gt % MU_COLS, sub = gt / MU_COLS;
+    const GroupBarrier bar{1 + group};
+    u64* sm = smem + 2 * A * MU_SRC + group * COL_SMEM(MU_COLS);
+    const u64* ys = smem + sub * MU_COLS + col;
+    const double* yd = smd + sub * MU_COLS + col;
+    for (;;) {
+        if (gt == 0) taken[group] = atomicAdd(&next, 1u);
+        bar();
+        const uint32_t i = taken[group] * splits + part;
+        if (i >= level) return;
+        const FpRow r{twf + (size_t)i * N16, pcs[i].qd, pcs[i].qinvd};
+        const u64 nq = 0 - pcs[i].q, nq10 = nq << 10;
+        const uint32_t ql = (uint32_t)nq, qh = (uint32_t)(nq >> 32), tl = (uint32_t)nq10, th = (uint32_t)(nq10 >> 32);
+        const double q32 = 4294967296.0 * r.qinv;
+        double x[16];
+#pragma unroll
+        for (int k = 0; k < 16; k += 4) {
+            u64 v[4];
+            uint32_t cross[4];
+            double s[4];
+#pragma unroll
+            for (int e = 0; e < 4; e++) v[e] = 0, cross[e] = 0, s[e] = FP_MAGIC;
+#pragma unroll
+            for (int a = 0; a < A; a++) {
+                const ulonglong2 t = __ldg(reinterpret_cast<const ulonglong2*>(&tab->term[a][i]));
+                const uint32_t ml = (uint32_t)t.x, mh = (uint32_t)(t.x >> 32);
+                const double mq = __longlong_as_double((long long)t.y);
+#pragma unroll
+                for (int e = 0; e < 4; e++) {
+                    const uint32_t at = a * MU_SRC + (k + e) * 16 * MU_COLS;
+                    const u64 y = ys[at];
+                    const uint32_t yl = (uint32_t)y, yh = (uint32_t)(y >> 32);
+                    s[e] = __fma_rn(yd[at], mq, s[e]);
+                    asm("mad.wide.u32 %0, %1, %2, %0;" : "+l"(v[e]) : "r"(yl), "r"(ml));
+                    asm("mad.lo.u32 %0, %1, %2, %0;" : "+r"(cross[e]) : "r"(yl), "r"(mh));
+                    asm("mad.lo.u32 %0, %1, %2, %0;" : "+r"(cross[e]) : "r"(yh), "r"(ml));
+                }
+            }
+#pragma unroll
+            for (int e = 0; e < 4; e++) {
+                // every rounding of s is to an integer: four terms leave c within 2.1 of the quotient, |v| <= 2.1 2^10 q
+                const u64 c = (u64)__double_as_longlong(s[e]);
+                const uint32_t cl = (uint32_t)c, ch = (uint32_t)(c >> 32) - FP_MAGIC_HI;
+                asm("mad.wide.u32 %0, %1, %2, %0;" : "+l"(v[e]) : "r"(cl), "r"(tl));
+                uint32_t hi = (uint32_t)(v[e] >> 32) + (cross[e] + cl * th + ch * tl);
+                // second quotient: the signed high word times 2^32 / q
+                const double d = __dadd_rn(__hiloint2double(0x43300000, (int)(hi ^ 0x80000000u)), -4503601774854144.0);
+                const u64 c2 = (u64)__double_as_longlong(__fma_rn(d, q32, FP_MAGIC));
+                const uint32_t dl = (uint32_t)c2, dh = (uint32_t)(c2 >> 32) - FP_MAGIC_HI;
+                u64 w = ((u64)hi << 32) | (uint32_t)v[e];
+                asm("mad.wide.u32 %0, %1, %2, %0;" : "+l"(w) : "r"(dl), "r"(ql));
+                hi = (uint32_t)(w >> 32) + (dl * qh + dh * ql);
+                x[k + e] = __dadd_rn(__hiloint2double((int)(hi + FP_MAGIC_HI), (int)(uint32_t)w), -FP_MAGIC);
+            }
+        }
+        fwd_cols<MU_COLS>(r, x, sm, col, sub, bar);
+        u64* p = out + (size_t)i * N16 + col;
+#pragma unroll
+        for (int k = 0; k < 16; k++) p[(16 * sub + k) * 256] = FpRow::bits(x[k]);
+    }
+}
+
+// special primes below 2^60 (|y| < 2^59), data primes of 2^40 to 2^50 (the second quotient ignores the low word of v)
+bool moddown16_supported(const fesc_ctx* ctx, uint32_t level) {
+    if (ctx->log_n != 16 || ctx->n_p > 4) return false;
+    for (uint32_t i = 0; i < level; i++)
+        if (ctx->q[i] >= FESC_FP_LIMIT || ctx->q[i] < (1ull << 40)) return false;
+    for (uint32_t k = 0; k < ctx->n_p; k++)
+        if (ctx->q[ctx->n_q + k] >= (1ull << 60)) return false;
+    return true;
+}
+template <int A>
+static int launch_moddown(fesc_ctx* ctx, const u64* acc, u64* u, uint32_t level, uint32_t polys, cudaStream_t st) {
+    const uint32_t tiles = 256 / MU_COLS;
+    const size_t smem = ((size_t)2 * A * MU_SRC + MD_GROUPS * COL_SMEM(MU_COLS)) * sizeof(u64);
+    auto kern = k_moddown_cols<A>;
+    FESC_CHECK_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    uint32_t splits = 1;
+    while (splits < 4 && tiles * polys * splits < 8 * 148) splits++;
+    launch(kern, dim3(tiles * splits, polys), MD_THREADS, smem, st, acc, u, ctx->tabs.d_moddown, ctx->d_twf, ctx->d_pc, level, ctx->n_q, ctx->n_p,
+           splits);
+    return FESC_OK;
+}
+int moddown16_cols_launch(fesc_ctx* ctx, const u64* acc, u64* u, uint32_t level, uint32_t polys, cudaStream_t st) {
+    if (ctx->n_p <= 1) return launch_moddown<1>(ctx, acc, u, level, polys, st);
+    if (ctx->n_p <= 2) return launch_moddown<2>(ctx, acc, u, level, polys, st);
+    return launch_moddown<4>(ctx, acc, u, level, polys, st);
+}

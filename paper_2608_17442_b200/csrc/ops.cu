@@ -1058,9 +1058,13 @@ static int ks_moddown(fesc_ctx* ctx, const KsScratch& ws, uint32_t level, uint32
     RowMap m;
     m.period = rows;
     for (uint32_t t = 0; t < rows; t++) m.prime[t] = t < level ? 0xFF : (uint8_t)(nq + (t - level));
-    if ((rc = ntt_launch(ctx, ws.acc, (size_t)polys * 2 * rows, m, true, st)) != FESC_OK) return rc;
+    const bool cols = moddown16_supported(ctx, level);      // the conversion feeds the forward transform's first pass
+    if ((rc = ntt_launch(ctx, ws.acc, (size_t)polys * 2 * rows, m, true, st, false, false, nullptr, cols ? ctx->tabs.d_down_scale : nullptr)) != FESC_OK)
+        return rc;
     prof_begin(ctx, PF_MODDOWN, st);
-    if (bconv_supported(ctx, level))
+    if (cols) {
+        if ((rc = moddown16_cols_launch(ctx, ws.acc, ws.u, level, polys * 2, st)) != FESC_OK) return rc;
+    } else if (bconv_supported(ctx, level))
         moddown_conv_imma_launch(ctx, ws.acc, ws.u, level, polys, ctx->log_n == 16, st);
     else if (N % (256 * KS_VEC) == 0)
         launch(k_moddown_conv<KS_VEC>, dim3(N / (256 * KS_VEC), polys * 2), 256, 0, st, ws.acc, ws.u, ctx->tabs.d_moddown, ctx->d_pc, N, level, nq, K, ctx->log_n == 16);
@@ -1080,7 +1084,7 @@ static int ks_moddown(fesc_ctx* ctx, const KsScratch& ws, uint32_t level, uint32
             fin.level = level, fin.acc_rows = rows, fin.add_mask = add_mask, fin.nb = batch;
             if (rot.src) fin.rot_src = rot.src + k0 * rot.key_stride, fin.rot_stride = rot.stride, fin.rot_key_stride = rot.key_stride;
             for (uint32_t k = 0; k < per && rot.src; k++) fin.rot_g[k] = rot.g[k0 + k];
-            rc = ntt_launch(ctx, ws.u + (size_t)k0 * batch * 2 * level * N, (size_t)per * batch * 2 * level, m, false, st, true, false, &fin);
+            rc = ntt_launch(ctx, ws.u + (size_t)k0 * batch * 2 * level * N, (size_t)per * batch * 2 * level, m, false, st, true, false, &fin, nullptr, cols);
             if (rc != FESC_OK) return rc;
         }
         return FESC_OK;

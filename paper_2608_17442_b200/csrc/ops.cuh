@@ -139,6 +139,9 @@ void moddown_conv_imma_launch(fesc_ctx* ctx, const u64* acc, u64* u, uint32_t le
 // ModUp fused with the first eight stages of the forward transform (N = 2^16, modup16.cu): y = the COEFF rows times
 // (Q_j/q_a)^-1
 bool modup16_supported(const fesc_ctx* ctx, uint32_t level);
+// the same for the division by P: the special rows of acc hold COEFF residues times (P/p_k)^-1
+bool moddown16_supported(const fesc_ctx* ctx, uint32_t level);
+int moddown16_cols_launch(fesc_ctx* ctx, const u64* acc, u64* u, uint32_t level, uint32_t polys, cudaStream_t st);
 int modup16_cols_launch(fesc_ctx* ctx, const u64* y, u64* ext, uint32_t level, uint32_t batch, cudaStream_t st);
 
 // rows on primes below 2^50: last pass of the forward transform of the converted digits and key inner product in one kernel (inner16.cu)
