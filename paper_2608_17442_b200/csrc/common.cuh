@@ -135,6 +135,8 @@ __device__ __forceinline__ double fp_load(u64 a, double q) {
     const double d = fp_from_u64(a);
     return d + d >= q ? d - q : d;
 }
+// any integer modulo q < 2^50, as a double
+__device__ __forceinline__ double fp_mod_u64(u64 a, const PrimeConst& pc) { return fp_from_u64(csub(a - mulhi(a, pc.mu) * pc.q, pc.q)); }
 // integer-valued double below 2^53 -> canonical residue
 __device__ __forceinline__ u64 fp_store(double x, double q, double qinv) {
     x = fp_reduce(x, q, qinv);
@@ -364,6 +366,10 @@ struct NttSource {
     uint32_t nb = 1;
     u64 g[KS_MAX_KEYS] = {};
     OwnRows own = {};
+    // rescale of a product: the words are multiplied by the plaintext row pt + k * pt_stride (FP64 rows), or by the integer `mul`
+    const u64* pt = nullptr;
+    size_t pt_stride = 0;
+    u64 mul = 0;
 };
 
 // Optional epilogue of the last pass of a forward N = 2^16 transform over rows r = bp * level + i (bp = ciphertext * 2 +
@@ -392,6 +398,10 @@ struct NttFinish {
     // first pass modulo every row's prime; the buffer handed to the transform is only written
     const u64* centred = nullptr;
     double centred_q = 0;
+    // rescale of a product: the minuend is multiplied by the plaintext row pt + ct * pt_stride + i * N, or by the integer `mul`
+    const u64* pt = nullptr;
+    size_t pt_stride = 0;
+    u64 mul = 0;
 };
 
 // internal launchers (ntt.cu)

@@ -96,11 +96,18 @@ extern "C" int fesc_norm_scale(fesc_ctx* ctx, const uint64_t* d_y, const uint64_
         rc = ctmul_internal(ctx, y + (size_t)tb * blocks * ctw, ctw, f[cur] + (size_t)tb * ctw, 0, prod, ctw, blocks, level, ks, st);
         if (rc != FESC_OK) return rc;
         if ((rc = rescale_internal(ctx, prod, ctw, prod1, blocks, level, ks, st)) != FESC_OK) return rc;
-        prof_begin(ctx, PF_POINTWISE, st);
-        launch(k_ct_mul_pt, grid, 256, 0, st, prod1, ctw1, (const u64*)d_gamma, (size_t)(level - 1) * N, prod1, ctw1, ctx->d_pc, N, level - 1);
-        prof_end(ctx, PF_POINTWISE, st);
-        FESC_CHECK_CUDA(ctx, cudaGetLastError());
-        rc = rescale_internal(ctx, prod1, ctw1, out + (size_t)tb * blocks * ctw2, blocks, level - 1, ks, st);
+        const u64* gamma = (const u64*)d_gamma;
+        const size_t pt_stride = (size_t)(level - 1) * N;
+        RescaleView view;
+        if (rescale_fused(ctx, level - 1)) {             // the product is formed by the rescale itself
+            view.pt = gamma, view.pt_stride = pt_stride;
+        } else {
+            prof_begin(ctx, PF_POINTWISE, st);
+            launch(k_ct_mul_pt, grid, 256, 0, st, prod1, ctw1, gamma, pt_stride, prod1, ctw1, ctx->d_pc, N, level - 1);
+            prof_end(ctx, PF_POINTWISE, st);
+            FESC_CHECK_CUDA(ctx, cudaGetLastError());
+        }
+        rc = rescale_internal(ctx, prod1, ctw1, out + (size_t)tb * blocks * ctw2, blocks, level - 1, ks, st, view);
         if (rc != FESC_OK) return rc;
     }
     return FESC_OK;

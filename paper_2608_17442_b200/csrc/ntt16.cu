@@ -114,8 +114,8 @@ __global__ void __launch_bounds__(COL_THREADS, 1024 / COL_THREADS)
     }
 }
 
-// grid = (128 / NTT_WARPS, rows); FIN: the last step of a division instead of the plain store (NttFinish)
-template <int A, bool FIN>
+// grid = (128 / NTT_WARPS, rows); FIN: the last step of a division instead of the plain store (NttFinish), 2: of a product
+template <int A, int FIN>
 __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
     ntt16_rows_fwd(u64* __restrict__ data, const void* __restrict__ tw, const PrimeConst* __restrict__ pcs, RowList list,
                    uint32_t y0, int out_double, NttFinish fin) {
@@ -165,27 +165,36 @@ __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
         const double cinv = fin.cinv[i];
         const bool add = (fin.add_mask >> pol) & 1;
         // the registers of the transform are free: all eight minuends are requested at once, the other addends by fours
+        const u64* pt = FIN == 2 && fin.pt ? fin.pt + ct * fin.pt_stride + (size_t)i * N16 + blk * 512 + 2 * lane : nullptr;
+        if (pt && !DBG_REGION(pt - 2 * lane, 512 * sizeof(u64))) return;
+        const double mul = FIN == 2 ? fp_mod_u64(fin.mul, pcs[pi]) : 0.0;
         ulonglong2 av[8];
 #pragma unroll
         for (int j = 0; j < 8; j++) av[j] = *reinterpret_cast<const ulonglong2*>(acc + blk * 512 + 2 * lane + 64 * j);
 #pragma unroll
         for (int h = 0; h < 8; h += 4) {
             u64 w[8];
-            if (rot) {
+            if (FIN == 1 && rot) {
 #pragma unroll
                 for (int j = 0; j < 8; j++) w[j] = rot[galois_src(blk * 512 + 2 * lane + 64 * (h + (j >> 1)) + (j & 1), 16, rot_g)];
             }
 #pragma unroll
             for (int j = h; j < h + 4; j++) {
                 const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(s + 72 * j);
-                double s0 = fp_modmul(fp_load(av[j].x, q) - FpRow::value(v.x), cinv, q, qinv);
-                double s1 = fp_modmul(fp_load(av[j].y, q) - FpRow::value(v.y), cinv, q, qinv);
-                if (rot) {
+                double a0 = fp_load(av[j].x, q), a1 = fp_load(av[j].y, q);
+                if (FIN == 2) {             // lazy products below 0.7 q
+                    const ulonglong2 w2 = pt ? __ldg(reinterpret_cast<const ulonglong2*>(pt + 64 * j)) : make_ulonglong2(0, 0);
+                    a0 = fp_modmul(a0, pt ? fp_from_u64(w2.x) : mul, q, qinv);
+                    a1 = fp_modmul(a1, pt ? fp_from_u64(w2.y) : mul, q, qinv);
+                }
+                double s0 = fp_modmul(a0 - FpRow::value(v.x), cinv, q, qinv);
+                double s1 = fp_modmul(a1 - FpRow::value(v.y), cinv, q, qinv);
+                if (FIN == 1 && rot) {
                     s0 += fp_load(w[2 * (j - h)], q);
                     s1 += fp_load(w[2 * (j - h) + 1], q);
                 }
                 ulonglong2* o = reinterpret_cast<ulonglong2*>(out + blk * 512 + 2 * lane + 64 * j);
-                if (add) {
+                if (FIN == 1 && add) {
                     const ulonglong2 ov = *o;
                     s0 += fp_load(ov.x, q);
                     s1 += fp_load(ov.y, q);
@@ -224,6 +233,7 @@ __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
     const u64* in = p + 2 * lane;
     uint32_t at = 0;                  // SRC: the words come from the permuted block that starts here
     u64* own = nullptr;
+    const u64* pt = nullptr;
     u64 g = 0;
     if (SRC) {                        // rows of the buffer: row = polynomial * period + limb
         const uint32_t poly = row / list.period, l = row - poly * list.period, k = poly / src.nb, b = poly - k * src.nb;
@@ -232,6 +242,10 @@ __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
         if (src.own.ext) own = src.own.ext + own_index(src.own, poly, l, N16) + blk * 512 + 2 * lane;
         if (!DBG_REGION(in, N16 * sizeof(u64)) || (own && !DBG_REGION(own - 2 * lane, 512 * sizeof(u64)))) return;
         at = blk * 512 + 2 * lane;
+        if (src.pt) {
+            pt = src.pt + k * src.pt_stride + at;
+            if (!DBG_REGION(pt - 2 * lane, 512 * sizeof(u64))) return;
+        }
     }
     auto pair = [&](int j) {
         if (!SRC) return *reinterpret_cast<const ulonglong2*>(in + 64 * j);
@@ -242,10 +256,17 @@ __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
     u64* o = p + 256 * (lane >> 4) + (lane & 15);
     if constexpr (A == ROW_FP) {
         FpRow r{(const double*)tw + (size_t)pi * N16, pcs[pi].qd, pcs[pi].qinvd};
+        const double mul = SRC ? fp_mod_u64(src.mul, pcs[pi]) : 0.0;
 #pragma unroll
         for (int j = 0; j < 8; j++) {
             ulonglong2 v = pair(j);
-            v = make_ulonglong2(FpRow::bits(fp_load(v.x, r.q)), FpRow::bits(fp_load(v.y, r.q)));
+            double a = fp_load(v.x, r.q), b = fp_load(v.y, r.q);
+            if (SRC && (pt || src.mul)) {
+                const ulonglong2 w = pt ? __ldg(reinterpret_cast<const ulonglong2*>(pt + 64 * j)) : make_ulonglong2(0, 0);
+                a = r.fold(fp_modmul(a, pt ? fp_from_u64(w.x) : mul, r.q, r.qinv));
+                b = r.fold(fp_modmul(b, pt ? fp_from_u64(w.y) : mul, r.q, r.qinv));
+            }
+            v = make_ulonglong2(FpRow::bits(a), FpRow::bits(b));
             *reinterpret_cast<ulonglong2*>(s + 72 * j) = v;
             if (SRC && own) *reinterpret_cast<ulonglong2*>(own + 64 * j) = v;
         }
@@ -297,8 +318,9 @@ int ntt16_launch(fesc_ctx* ctx, u64* data, size_t rows, const RowMap& map, bool 
                     launch(ntt16_cols_inv<ROW_FP>, gc, COL_THREADS, 0, st, data, ctx->d_itwf, ctx->d_pc, l, y, scale);
                 } else {
                     if (!skip_cols) launch(ntt16_cols_fwd<ROW_FP>, gc, COL_THREADS, 0, st, data, ctx->d_twf, ctx->d_pc, l, y, in_double, fin.centred, fin.centred_q);
-                    if (fin.acc) launch(ntt16_rows_fwd<ROW_FP, true>, gr, ROW_THREADS, 0, st, data, ctx->d_twf, ctx->d_pc, l, y, out_double, fin);
-                    else launch(ntt16_rows_fwd<ROW_FP, false>, gr, ROW_THREADS, 0, st, data, ctx->d_twf, ctx->d_pc, l, y, out_double, fin);
+                    if (fin.pt || fin.mul) launch(ntt16_rows_fwd<ROW_FP, 2>, gr, ROW_THREADS, 0, st, data, ctx->d_twf, ctx->d_pc, l, y, out_double, fin);
+                    else if (fin.acc) launch(ntt16_rows_fwd<ROW_FP, 1>, gr, ROW_THREADS, 0, st, data, ctx->d_twf, ctx->d_pc, l, y, out_double, fin);
+                    else launch(ntt16_rows_fwd<ROW_FP, 0>, gr, ROW_THREADS, 0, st, data, ctx->d_twf, ctx->d_pc, l, y, out_double, fin);
                 }
             } else if (inverse) {
                 launch(source ? ntt16_rows_inv<ROW_INT, true> : ntt16_rows_inv<ROW_INT, false>, gr, ROW_THREADS, 0, st, data, ctx->d_itw, ctx->d_pc, l, y,
@@ -306,7 +328,7 @@ int ntt16_launch(fesc_ctx* ctx, u64* data, size_t rows, const RowMap& map, bool 
                 launch(ntt16_cols_inv<ROW_INT>, gc, COL_THREADS, 0, st, data, ctx->d_itw, ctx->d_pc, l, y, scale);
             } else {
                 if (!skip_cols) launch(ntt16_cols_fwd<ROW_INT>, gc, COL_THREADS, 0, st, data, ctx->d_tw, ctx->d_pc, l, y, 0, nullptr, 0.0);
-                launch(ntt16_rows_fwd<ROW_INT, false>, gr, ROW_THREADS, 0, st, data, ctx->d_tw, ctx->d_pc, l, y, 0, fin);
+                launch(ntt16_rows_fwd<ROW_INT, 0>, gr, ROW_THREADS, 0, st, data, ctx->d_tw, ctx->d_pc, l, y, 0, fin);
             }
             launches += skip_cols ? 1 : 2;
         }

@@ -473,6 +473,14 @@ __global__ void __launch_bounds__(256, 4) k_inner_shared(const u64* __restrict__
         if (!ok) return;
     }
 #endif
+    // the key words of a pass arrive in L2 one key ahead: 2 BETA rows of four lines
+    auto prefetch_key = [&](uint32_t k) {
+        if (tid < 8 * BETA) {
+            const uint32_t c = galois_src(blk * IS_BLK, 16, keys.ginv[k]) & ~(IS_BLK - 1u);
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(keys.key[k] + ((size_t)(tid >> 2) * np + pt) * N + c + 16 * (tid & 3)));
+        }
+    };
+    prefetch_key(0);
     for (uint32_t r = tid / 32; r < batch * BETA; r += 8)        // a warp copies one row's block, 16 bytes per lane
         *reinterpret_cast<ulonglong2*>(sx + r * IS_BLK + 2 * (tid % 32)) =
             *reinterpret_cast<const ulonglong2*>(ext + ((size_t)r * rows + t) * N + blk * IS_BLK + 2 * (tid % 32));
@@ -481,6 +489,7 @@ __global__ void __launch_bounds__(256, 4) k_inner_shared(const u64* __restrict__
     const double q = pc.qd, qinv = pc.qinvd;
 #pragma unroll 1
     for (uint32_t k = 0; k < keys.n; k++) {
+        if (k + 1 < keys.n) prefetch_key(k + 1);
         const uint32_t c = (galois_src(blk * IS_BLK, 16, keys.ginv[k]) & ~(IS_BLK - 1u)) + i;      // output coefficient
         const u64* w = keys.key[k] + (size_t)pt * N + c;
         const u64* x = sx + (galois_src(c, 16, keys.g[k]) & (IS_BLK - 1u));
@@ -1538,11 +1547,21 @@ __global__ void __launch_bounds__(256) k_rescale_finish(const u64* __restrict__ 
     *o = shoup(submod(x, *o, q), tab->qinv[i], tab->qinvs[i], q);
 }
 
-// out must be a contiguous batch [batch][2][level-1][N]; scratch holds batch*2*N words.
+// whether the rescale needs no conversion kernels: N = 2^16, every prime of the level below 2^50
+bool rescale_fused(const fesc_ctx* ctx, uint32_t level) {
+    bool fuse = ctx->log_n == 16;
+    for (uint32_t i = 0; i < level; i++) fuse = fuse && ctx->q[i] < FESC_FP_LIMIT;
+    return fuse;
+}
+// out: a contiguous batch [batch][2][level-1][N] unless the view says otherwise; scratch holds batch*2*N words.
 int rescale_internal(fesc_ctx* ctx, const u64* in, size_t in_stride, u64* out, uint32_t batch, uint32_t level,
-                     u64* scratch, cudaStream_t st) {
+                     u64* scratch, cudaStream_t st, const RescaleView& view) {
     const uint32_t N = ctx->N, gx = (N + 255) / 256;
-    const size_t out_stride = (size_t)2 * (level - 1) * N;
+    const size_t row_stride = (size_t)2 * (level - 1) * N, out_stride = view.out_stride ? view.out_stride : row_stride;
+    const uint32_t in_rows = view.in_rows ? view.in_rows : level;
+    const bool fuse = rescale_fused(ctx, level);
+    if (!fuse && (view.in_rows || view.pt || view.mul || view.out_stride))
+        return fesc_fail(ctx, FESC_EINVAL, "rescale: products and strided results belong to the fused kernels");
     const RescaleTab* tab = ctx->tabs.d_rescale + level;
     int rc;
     for (uint32_t b0 = 0; b0 < batch; b0 += 16384) {
@@ -1555,22 +1574,25 @@ int rescale_internal(fesc_ctx* ctx, const u64* in, size_t in_stride, u64* out, u
         }
         // N = 2^16, FP64 rows: the inverse transform reads the last limbs in place, the forward transform's first pass takes the centred
         // residues modulo every prime from them and its last pass stores (in - u) * q_last^-1
-        bool fuse = ctx->log_n == 16;
-        for (uint32_t i = 0; i < level; i++) fuse = fuse && ctx->q[i] < FESC_FP_LIMIT;
         RowMap m;
         m.period = 1;
         m.prime[0] = (uint8_t)(level - 1);
         if (fuse) {
             NttSource src;
-            src.src = ib + (size_t)(level - 1) * N, src.stride = (size_t)level * N, src.key_stride = in_stride, src.nb = 2;
+            src.src = ib + (size_t)(level - 1) * N, src.stride = (size_t)in_rows * N, src.key_stride = in_stride, src.nb = 2;
+            const u64* pt = view.pt ? view.pt + b0 * view.pt_stride : nullptr;
+            if (pt) src.pt = pt + (size_t)(level - 1) * N, src.pt_stride = view.pt_stride;
+            src.mul = view.mul;
             if ((rc = ntt_launch(ctx, scratch, (size_t)nb * 2, m, true, st, false, false, nullptr, nullptr, false, &src)) != FESC_OK) return rc;
             m.period = level - 1;
             for (uint32_t i = 0; i + 1 < level; i++) m.prime[i] = (uint8_t)i;
             NttFinish fin;
             fin.acc = ib, fin.acc_stride = in_stride, fin.out = ob, fin.out_stride = out_stride, fin.cinv = tab->qinvd;
-            fin.level = level - 1, fin.acc_rows = level, fin.add_mask = 0;
+            fin.level = level - 1, fin.acc_rows = in_rows, fin.add_mask = 0;
             fin.centred = scratch, fin.centred_q = (double)ctx->q[level - 1];
-            if ((rc = ntt_launch(ctx, ob, (size_t)nb * 2 * (level - 1), m, false, st, false, false, &fin)) != FESC_OK) return rc;
+            fin.pt = pt, fin.pt_stride = view.pt_stride, fin.mul = view.mul;
+            u64* rows = view.rows ? view.rows + (size_t)b0 * row_stride : ob;
+            if ((rc = ntt_launch(ctx, rows, (size_t)nb * 2 * (level - 1), m, false, st, false, false, &fin)) != FESC_OK) return rc;
             continue;
         }
         prof_begin(ctx, PF_RESCALE, st);

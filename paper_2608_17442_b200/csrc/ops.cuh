@@ -62,8 +62,20 @@ struct MaskedSum {
 };
 int masked_sum(fesc_ctx* ctx, const MaskedSum& s, size_t src_stride, size_t pt_stride, const u64* add, size_t add_stride, u64* out,
                size_t out_stride, uint32_t batch, uint32_t level, cudaStream_t st);
+// What the rescale takes beyond a contiguous batch, where rescale_fused holds: polynomials stored with more limbs than `level`, a product
+// (by plaintexts at pt + b * pt_stride, or by an integer) that is formed on the way, results with a stride (then `rows` holds the
+// batch * 2 * (level - 1) rows of the transform).
+struct RescaleView {
+    uint32_t in_rows = 0;           // limbs per stored polynomial; 0: level
+    const u64* pt = nullptr;        // [level][N]
+    size_t pt_stride = 0;
+    u64 mul = 0;                    // 0: none
+    size_t out_stride = 0;          // 0: contiguous
+    u64* rows = nullptr;
+};
+bool rescale_fused(const fesc_ctx* ctx, uint32_t level);
 int rescale_internal(fesc_ctx* ctx, const u64* in, size_t in_stride, u64* out, uint32_t batch, uint32_t level,
-                     u64* scratch, cudaStream_t st);
+                     u64* scratch, cudaStream_t st, const RescaleView& view = RescaleView());
 int ctmul_internal(fesc_ctx* ctx, const u64* a, size_t a_stride, const u64* b, size_t b_stride, u64* out,
                    size_t out_stride, uint32_t batch, uint32_t level, u64* scratch, cudaStream_t st);
 

@@ -209,28 +209,47 @@ struct Exec {
                                                                a.level, times);
         prof_end(ctx, PF_POINTWISE, st);
     }
-    // contiguous `in` at level l -> contiguous `out` at level l-1
-    void rescale(const Arr& in, const Arr& out) {
-        if (!ok() || dry) return;
-        rc = rescale_internal(ctx, in.p, in.stride, out.p, in.count, in.level, rs, st);
-    }
-    // out (level-1, contiguous) = rescale(in (.) pt); pt_stride != 0: plaintext i for element i; a single `in` with
-    // out.count plaintexts multiplies that one ciphertext by each of them
-    void ptmul_rescale(const Arr& in, const u64* pt, const Arr& out, size_t pt_stride = 0) {
+    // out = rescale of the first `level` limbs of in (.) factor; factor: plaintexts (pt_stride apart), an integer, or none.  A single `in`
+    // with out.count plaintexts multiplies that one ciphertext by each of them.  Where the rescale is fused the product is never stored.
+    void product_rescale(const Arr& in, uint32_t level, const u64* pt, size_t pt_stride, u64 mul, const Arr& out) {
+        if (!ok()) return;
         size_t mark = top;
         const uint32_t cnt = out.count;
-        Arr t = alloc(cnt, in.level);
-        if (ok() && !dry) {
-            prof_begin(ctx, PF_POINTWISE, st);
-            launch(k_ct_ptmul, grid(in.level, cnt), 256, 0, st, in.p, in.count == 1 && cnt > 1 ? 0 : in.stride, pt, pt_stride, t.p,
-                                                            t.stride, ctx->d_pc, N, in.level);
-            prof_end(ctx, PF_POINTWISE, st);
-            ctx->counters[2] += cnt;
+        const bool strided_out = out.stride != ctw(level - 1) && cnt > 1;
+        const size_t in_stride = in.count == 1 && cnt > 1 ? 0 : in.stride;
+        if (rescale_fused(ctx, level) && (pt || mul || in.level == level)) {
+            RescaleView v;
+            v.in_rows = in.level, v.pt = pt, v.pt_stride = pt_stride, v.mul = mul;
+            if (strided_out) {
+                Arr rows = alloc(cnt, level - 1);
+                v.rows = rows.p, v.out_stride = out.stride;
+            }
+            if (!dry) rc = rescale_internal(ctx, in.p, in_stride, out.p, cnt, level, rs, st, v);
+        } else {
+            Arr t{in.p, cnt, level, in_stride};
+            if (pt || mul || in.level != level) {
+                t = alloc(cnt, level);
+                if (!dry) {
+                    prof_begin(ctx, PF_POINTWISE, st);
+                    if (pt)
+                        launch(k_ct_ptmul, grid(level, cnt), 256, 0, st, in.p, in_stride, pt, pt_stride, t.p, t.stride, ctx->d_pc, N, level);
+                    else
+                        launch(k_ct_scale_drop, grid(2 * level, cnt), 256, 0, st, in.p, in_stride, t.p, t.stride, ctx->d_pc, N, in.level, level, mul);
+                    prof_end(ctx, PF_POINTWISE, st);
+                }
+            }
+            Arr r = strided_out ? alloc(cnt, level - 1) : out;
+            if (!dry) rc = rescale_internal(ctx, t.p, t.stride, r.p, cnt, level, rs, st);
+            if (strided_out) copy(r, out);
         }
-        rescale(t, out);
+        if (pt && !dry) ctx->counters[2] += cnt;
         top = mark;
     }
-    // out (level-1, contiguous) = rescale(a * b); b may be a single ciphertext shared by the batch
+    // `in` at level l -> `out` at level l-1
+    void rescale(const Arr& in, const Arr& out) { product_rescale(in, in.level, nullptr, 0, 0, out); }
+    // out (level-1) = rescale(in (.) pt); pt_stride != 0: plaintext i for element i
+    void ptmul_rescale(const Arr& in, const u64* pt, const Arr& out, size_t pt_stride = 0) { product_rescale(in, in.level, pt, pt_stride, 0, out); }
+    // out (level-1) = rescale(a * b); b may be a single ciphertext shared by the batch
     void mul_rescale(const Arr& a, const Arr& b, const Arr& out) {
         size_t mark = top;
         Arr t = alloc(a.count, a.level);
@@ -240,7 +259,7 @@ struct Exec {
         rescale(t, out);
         top = mark;
     }
-    // out (level dst, contiguous) = in brought from its level to dst; kind 0: state-like, 1: multiplicand
+    // out (level dst) = in brought from its level to dst; kind 0: state-like, 1: multiplicand
     void adjust(const Arr& in, uint32_t dst, int kind, const Arr& out) {
         if (!ok()) return;
         if (in.level == dst) return copy(in, out);
@@ -248,18 +267,23 @@ struct Exec {
             rc = fesc_fail(ctx, FESC_ELEVEL, "scan_contract: level schedule violated");
             return;
         }
-        size_t mark = top;
-        Arr t = alloc(in.count, dst + 1);
-        if (!dry) {
-            const uint64_t* tab = kind ? cs->adj_p : cs->adj_s;
-            u64 k = tab[(size_t)in.level * (g.l0 + 1) + dst];
-            prof_begin(ctx, PF_POINTWISE, st);
-            launch(k_ct_scale_drop, grid(2 * (dst + 1), in.count), 256, 0, st, in.p, in.stride, t.p, t.stride, ctx->d_pc, N,
-                                                                           in.level, dst + 1, k);
-            prof_end(ctx, PF_POINTWISE, st);
-        }
-        rescale(t, out);
-        top = mark;
+        const uint64_t* tab = kind ? cs->adj_p : cs->adj_s;
+        product_rescale(in, dst + 1, nullptr, 0, tab[(size_t)in.level * (g.l0 + 1) + dst], out);
+    }
+    static bool equally_spaced(const std::vector<uint32_t>& pos, uint32_t& step) {
+        step = pos.size() > 1 ? pos[1] - pos[0] : 1;
+        bool ok = pos.size() < 2 || pos[1] > pos[0];
+        for (size_t k = 1; k < pos.size(); k++) ok = ok && pos[k] == pos[k - 1] + step;
+        return ok;
+    }
+    // The slots `pos` of `base` at level dst: in place when they are all there and equally spaced, brought down into `out` otherwise.
+    Arr at_level(const Arr& base, const std::vector<uint32_t>& pos, const std::vector<uint32_t>& lev, uint32_t dst, int kind, const Arr& out) {
+        uint32_t step;
+        bool there = equally_spaced(pos, step);
+        for (uint32_t p : pos) there = there && lev[p] == dst;
+        if (there) return Arr{base.p + (size_t)pos[0] * base.stride, (uint32_t)pos.size(), dst, base.stride * step};
+        adjust_many(base, pos, lev, dst, kind, out);
+        return out;
     }
     // out[i] (level dst, contiguous) = slot pos[i] of `base` (capacity stride base.stride, current level lev[pos[i]])
     // brought to dst.  Slots that sit at the same level go down in ONE batch: straight from the slots when their
@@ -334,10 +358,10 @@ struct Exec {
     // Broadcasts of the tokens of filled group ciphertexts (grouped leaf build): for class c < G
     //   out_c[u] = rescale( sum_{j<G} masks[j] (.) rot(grp[u], (c - j) unit) ),
     // with the 2(G-1) rotations by +unit..+(G-1)unit, -unit..-(G-1)unit taken once for the whole batch of groups
-    // (hoisted mode: one decomposition per group).  `deliver(c, res)` receives the batch of class c (level - 1,
-    // contiguous, valid until it returns).
+    // (hoisted mode: one decomposition per group).  `finish(c, sum)` receives the sum of class c before the rescale (valid until it
+    // returns).
     template <class F>
-    void class_broadcasts(const Arr& grp, const u64* masks, uint32_t G, uint32_t unit, F deliver) {
+    void class_broadcasts(const Arr& grp, const u64* masks, uint32_t G, uint32_t unit, F finish) {
         size_t mark = top;
         const uint32_t nk = 2 * (G - 1), cnt = grp.count, lvl = grp.level;
         Arr rots = alloc(nk * cnt, lvl);       // [shift][group]
@@ -354,7 +378,7 @@ struct Exec {
         } else {
             for (uint32_t i = 0; i < nk; i++) rot(grp, shifts[i], at(rots, i * cnt, cnt));
         }
-        Arr acc = alloc(cnt, lvl), res = alloc(cnt, lvl - 1);
+        Arr acc = alloc(cnt, lvl);
         for (uint32_t c = 0; c < G && ok(); c++) {
             if (!dry && ok()) {
                 MaskedSum s;
@@ -366,8 +390,7 @@ struct Exec {
                 }
                 rc = masked_sum(ctx, s, grp.stride, 0, nullptr, 0, acc.p, acc.stride, cnt, lvl, st);
             }
-            rescale(acc, res);
-            deliver(c, res);
+            finish(c, acc);
         }
         top = mark;
     }
@@ -427,7 +450,7 @@ static int scan_run(Exec& X, const u64* d_x, const u64* d_a, const u64* d_B, con
                 X.ptmul_rescale(exg, (const u64*)X.cs->d_mask_bg, gb);
                 X.fill_right(gb, unit, ilog2(g.n / unit));
                 X.class_broadcasts(gb, (const u64*)X.cs->d_mask_b2, G, g.d_s,
-                                   [&](uint32_t c, const Arr& res) { X.copy(res, X.strided(brB, c, G, ng)); });
+                                   [&](uint32_t c, const Arr& sum) { X.rescale(sum, X.strided(brB, c, G, ng)); });
                 X.top = m;
                 continue;
             }
@@ -464,7 +487,7 @@ static int scan_run(Exec& X, const u64* d_x, const u64* d_a, const u64* d_B, con
                     X.ptmul_rescale(ex, (const u64*)X.cs->d_mask_xg, xg);
                     X.fill_right(xg, G, ilog2(g.d_s / G));
                     X.class_broadcasts(xg, (const u64*)X.cs->d_mask_x2, G, 1,
-                                       [&](uint32_t c, const Arr& res) { X.copy(res, X.strided(xr, c, G, ng)); });
+                                       [&](uint32_t c, const Arr& sum) { X.rescale(sum, X.strided(xr, c, G, ng)); });
                 } else {
                     Arr ex = X.alloc(B, l0);
                     for (uint32_t sg = 0; sg < g.segs; sg++) X.extract_n(X.at(srcx, sg), 1, g.Bt, X.at(ex, sg * g.Bt, g.Bt));
@@ -489,13 +512,13 @@ static int scan_run(Exec& X, const u64* d_x, const u64* d_a, const u64* d_B, con
                     X.extract_n(X.at(apre, sg), (int64_t)G * g.P, ngs, X.at(ex, sg * ngs, ngs));
                 X.ptmul_rescale(ex, (const u64*)X.cs->d_mask_ag, ag);
                 X.fill_right(ag, G * g.P, ilog2(g.R / (G * g.P)));
-                Arr xr = X.alloc(B, l0 - 2), cls1 = X.alloc(ng, l1);
+                Arr xr = X.alloc(B, l0 - 2), cls = X.alloc(ng, l0 - 2);
                 // class c = the tokens u*G + c of every group u
                 X.class_broadcasts(xg, (const u64*)X.cs->d_mask_x2, G, 1,
-                                   [&](uint32_t c, const Arr& res) { X.copy(res, X.strided(xr, c, G, ng)); });
-                X.class_broadcasts(ag, (const u64*)X.cs->d_mask_a2, G, g.P, [&](uint32_t c, const Arr& res) {
-                    X.adjust(res, l1, 1, cls1);          // p_t = br(a_t) at the leaf level
-                    X.copy(cls1, X.strided(Ps, c, G, ng));
+                                   [&](uint32_t c, const Arr& sum) { X.rescale(sum, X.strided(xr, c, G, ng)); });
+                X.class_broadcasts(ag, (const u64*)X.cs->d_mask_a2, G, g.P, [&](uint32_t c, const Arr& sum) {
+                    X.rescale(sum, cls);
+                    X.adjust(cls, l1, 1, X.strided(Ps, c, G, ng));      // p_t = br(a_t) at the leaf level
                 });
                 X.mul_rescale(xr, brB, Ss);      // s_t = br(x_t) (.) br(B_t), level l1 = l0-3
                 X.top = m;
@@ -524,38 +547,31 @@ static int scan_run(Exec& X, const u64* d_x, const u64* d_a, const u64* d_B, con
                 const uint32_t cnt = (uint32_t)left.size();
                 if (!cnt || !X.ok()) return;
                 size_t m = X.top;
-                if (plain) {        // s <- abar^span (.) s_L + s_R: one ct-pt product per node
-                    Arr sL = X.alloc(cnt, lvl), sR = X.alloc(cnt, lvl - 1), ns = X.alloc(cnt, lvl - 1);
-                    X.adjust_many(Ss, left, ls, lvl, 0, sL);
-                    X.adjust_many(Ss, right, ls, lvl - 1, 0, sR);
-                    X.ptmul_rescale(sL, stage_pt, ns);
-                    X.add(ns, sR, ns);
+                // results go straight to the slots of the right positions when those are equally spaced
+                uint32_t step;
+                const bool spaced = Exec::equally_spaced(right, step);
+                auto deliver = [&](const Arr& base, std::vector<uint32_t>& lev, auto make) {
+                    Arr dst = spaced ? Arr{base.p + (size_t)right[0] * base.stride, cnt, lvl - 1, base.stride * step} : X.alloc(cnt, lvl - 1);
+                    make(dst);
                     for (uint32_t i = 0; i < cnt; i++) {
-                        const uint32_t b = right[i];
-                        X.copy(X.at(ns, i), Arr{Ss.p + (size_t)b * Ss.stride, 1, lvl - 1, X.ctw(lvl - 1)});
-                        ls[b] = lvl - 1;
+                        if (!spaced) X.copy(X.at(dst, i), Arr{base.p + (size_t)right[i] * base.stride, 1, lvl - 1, X.ctw(lvl - 1)});
+                        lev[right[i]] = lvl - 1;
                     }
+                };
+                Arr sL = X.at_level(Ss, left, ls, lvl, 0, X.alloc(cnt, lvl)), sR = X.at_level(Ss, right, ls, lvl - 1, 0, X.alloc(cnt, lvl - 1));
+                Arr ns = X.alloc(cnt, lvl - 1);
+                if (plain) {        // s <- abar^span (.) s_L + s_R: one ct-pt product per node
+                    X.ptmul_rescale(sL, stage_pt, ns);
+                    deliver(Ss, ls, [&](const Arr& dst) { X.add(ns, sR, dst); });
                     X.top = m;
                     return;
                 }
-                Arr pL = X.alloc(cnt, lvl), sL = X.alloc(cnt, lvl), pR = X.alloc(cnt, lvl), sR = X.alloc(cnt, lvl - 1);
-                Arr np_ = X.alloc(cnt, lvl - 1), ns = X.alloc(cnt, lvl - 1);
-                if (need_p) X.adjust_many(Ps, left, lp, lvl, 1, pL);
-                X.adjust_many(Ss, left, ls, lvl, 0, sL);
-                X.adjust_many(Ps, right, lp, lvl, 1, pR);
-                X.adjust_many(Ss, right, ls, lvl - 1, 0, sR);
-                if (need_p) X.mul_rescale(pR, pL, np_);
+                // both products read their operands before a slot is overwritten: s_R is added where it lies, p_R p_L leaves its slot last
+                Arr pR = X.at_level(Ps, right, lp, lvl, 1, X.alloc(cnt, lvl));
+                Arr pL = need_p ? X.at_level(Ps, left, lp, lvl, 1, X.alloc(cnt, lvl)) : pR;
                 X.mul_rescale(pR, sL, ns);
-                X.add(ns, sR, ns);
-                for (uint32_t i = 0; i < cnt; i++) {
-                    const uint32_t b = right[i];
-                    if (need_p) {
-                        X.copy(X.at(np_, i), Arr{Ps.p + (size_t)b * Ps.stride, 1, lvl - 1, X.ctw(lvl - 1)});
-                        lp[b] = lvl - 1;
-                    }
-                    X.copy(X.at(ns, i), Arr{Ss.p + (size_t)b * Ss.stride, 1, lvl - 1, X.ctw(lvl - 1)});
-                    ls[b] = lvl - 1;
-                }
+                deliver(Ss, ls, [&](const Arr& dst) { X.add(ns, sR, dst); });
+                if (need_p) deliver(Ps, lp, [&](const Arr& dst) { X.mul_rescale(pR, pL, dst); });
                 X.top = m;
             };
             const uint32_t network = X.desc->network;
