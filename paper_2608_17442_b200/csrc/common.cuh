@@ -333,6 +333,16 @@ static inline int fesc_fail(fesc_ctx* ctx, int code, const std::string& msg) {
     return code;
 }
 
+// Two adjacent words of a buffer that the caller owns, which need not lie on a 16-byte boundary (`wide`: it does).
+__device__ __forceinline__ bool pair_aligned(const u64* p) { return ((size_t)p & 15) == 0; }
+__device__ __forceinline__ ulonglong2 ld_pair(const u64* p, bool wide) {
+    return wide ? *reinterpret_cast<const ulonglong2*>(p) : make_ulonglong2(p[0], p[1]);
+}
+__device__ __forceinline__ void st_pair(u64* p, ulonglong2 v, bool wide) {
+    if (wide) *reinterpret_cast<ulonglong2*>(p) = v;
+    else p[0] = v.x, p[1] = v.y;
+}
+
 // Galois automorphism X -> X^g in evaluation (bit-reversed) order: out[t] = in[galois_src(t)]
 __device__ __forceinline__ uint32_t galois_src(uint32_t t, uint32_t log_n, u64 g) {
     uint32_t u = __brev(t) >> (32 - log_n);

@@ -168,9 +168,10 @@ __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
         const u64* pt = FIN == 2 && fin.pt ? fin.pt + ct * fin.pt_stride + (size_t)i * N16 + blk * 512 + 2 * lane : nullptr;
         if (pt && !DBG_REGION(pt - 2 * lane, 512 * sizeof(u64))) return;
         const double mul = FIN == 2 ? fp_mod_u64(fin.mul, pcs[pi]) : 0.0;
+        const bool wide = FIN == 2 && pair_aligned(acc), wide_pt = FIN == 2 && pair_aligned(pt);
         ulonglong2 av[8];
 #pragma unroll
-        for (int j = 0; j < 8; j++) av[j] = *reinterpret_cast<const ulonglong2*>(acc + blk * 512 + 2 * lane + 64 * j);
+        for (int j = 0; j < 8; j++) av[j] = ld_pair(acc + blk * 512 + 2 * lane + 64 * j, FIN == 1 || wide);
 #pragma unroll
         for (int h = 0; h < 8; h += 4) {
             u64 w[8];
@@ -183,7 +184,7 @@ __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
                 const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(s + 72 * j);
                 double a0 = fp_load(av[j].x, q), a1 = fp_load(av[j].y, q);
                 if (FIN == 2) {             // lazy products below 0.7 q
-                    const ulonglong2 w2 = pt ? __ldg(reinterpret_cast<const ulonglong2*>(pt + 64 * j)) : make_ulonglong2(0, 0);
+                    const ulonglong2 w2 = pt ? ld_pair(pt + 64 * j, wide_pt) : make_ulonglong2(0, 0);
                     a0 = fp_modmul(a0, pt ? fp_from_u64(w2.x) : mul, q, qinv);
                     a1 = fp_modmul(a1, pt ? fp_from_u64(w2.y) : mul, q, qinv);
                 }
@@ -247,9 +248,10 @@ __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
             if (!DBG_REGION(pt - 2 * lane, 512 * sizeof(u64))) return;
         }
     }
+    const bool wide = SRC && pair_aligned(in), wide_pt = SRC && pair_aligned(pt);
     auto pair = [&](int j) {
         if (!SRC) return *reinterpret_cast<const ulonglong2*>(in + 64 * j);
-        if (!g) return *reinterpret_cast<const ulonglong2*>(in + at + 64 * j);
+        if (!g) return ld_pair(in + at + 64 * j, wide);
         return make_ulonglong2(in[galois_src(at + 64 * j, 16, g)], in[galois_src(at + 64 * j + 1, 16, g)]);
     };
     u64* s = sm + 2 * lane + 2 * (lane >> 3);
@@ -262,7 +264,7 @@ __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
             ulonglong2 v = pair(j);
             double a = fp_load(v.x, r.q), b = fp_load(v.y, r.q);
             if (SRC && (pt || src.mul)) {
-                const ulonglong2 w = pt ? __ldg(reinterpret_cast<const ulonglong2*>(pt + 64 * j)) : make_ulonglong2(0, 0);
+                const ulonglong2 w = pt ? ld_pair(pt + 64 * j, wide_pt) : make_ulonglong2(0, 0);
                 a = r.fold(fp_modmul(a, pt ? fp_from_u64(w.x) : mul, r.q, r.qinv));
                 b = r.fold(fp_modmul(b, pt ? fp_from_u64(w.y) : mul, r.q, r.qinv));
             }

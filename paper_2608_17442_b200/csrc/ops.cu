@@ -68,9 +68,9 @@ __global__ void __launch_bounds__(256) k_masked_sum(MaskedSum s, size_t src_stri
     acc128 a[4] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}};
 #pragma unroll 4
     for (uint32_t j = 0; j < s.n; j++) {
-        const u64* x = s.src[j] + b * src_stride + o + c;
-        const ulonglong2 w = __ldg(reinterpret_cast<const ulonglong2*>(s.pt[j] + b * pt_stride + o + c));
-        const ulonglong2 x0 = *reinterpret_cast<const ulonglong2*>(x), x1 = *reinterpret_cast<const ulonglong2*>(x + poly);
+        const u64 *x = s.src[j] + b * src_stride + o + c, *m = s.pt[j] + b * pt_stride + o + c;
+        const bool wide = pair_aligned(x);
+        const ulonglong2 w = ld_pair(m, pair_aligned(m)), x0 = ld_pair(x, wide), x1 = ld_pair(x + poly, wide);
         mac128(a[0], x0.x, w.x);
         mac128(a[1], x0.y, w.y);
         mac128(a[2], x1.x, w.x);
@@ -80,12 +80,13 @@ __global__ void __launch_bounds__(256) k_masked_sum(MaskedSum s, size_t src_stri
 #pragma unroll
     for (int k = 0; k < 4; k++) r[k] = reduce128(a[k].hi, a[k].lo, pc);
     if (add) {
-        const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(add + b * add_stride + o + c);
+        const ulonglong2 v = ld_pair(add + b * add_stride + o + c, pair_aligned(add + c));
         r[0] = addmod(r[0], v.x, pc.q), r[1] = addmod(r[1], v.y, pc.q);
     }
     u64* y = out + b * out_stride + o + c;
-    *reinterpret_cast<ulonglong2*>(y) = make_ulonglong2(r[0], r[1]);
-    *reinterpret_cast<ulonglong2*>(y + poly) = make_ulonglong2(r[2], r[3]);
+    const bool wide = pair_aligned(y);
+    st_pair(y, make_ulonglong2(r[0], r[1]), wide);
+    st_pair(y + poly, make_ulonglong2(r[2], r[3]), wide);
 }
 int masked_sum(fesc_ctx* ctx, const MaskedSum& s, size_t src_stride, size_t pt_stride, const u64* add, size_t add_stride, u64* out,
                size_t out_stride, uint32_t batch, uint32_t level, cudaStream_t st) {
