@@ -691,6 +691,7 @@ static int linear_packed(fesc_ctx* ctx, const u64* in, const uint8_t* image, con
     const size_t tile_bytes = bsgs_packed_bytes(N, level, 8, terms);     // one tile of 8 rows of packed inputs
     const uint32_t dshift = desc->diag_run_log2;
     const size_t image_tile_bytes = bsgs_packed_bytes(N >> dshift, level, 8, terms);
+    const bool periodic = bsgs_periodic_supported(terms, (nb_part < nout ? nb_part : nout) * n2, dshift);
     for (uint32_t tb0 = 0; tb0 < tbs; tb0 += tbg) {
         const uint32_t nt = tbs - tb0 < tbg ? tbs - tb0 : tbg;
         for (uint32_t s0 = 0; s0 < nt; s0 += 4) {        // baby rotations of 4 token blocks, packed into their tile
@@ -710,12 +711,12 @@ static int linear_packed(fesc_ctx* ctx, const u64* in, const uint8_t* image, con
                 rc = rotate_multi_internal(ctx, gin_base, ctw, 0, rot + ctw, (size_t)n1 * ctw, ctw, ns * gin, level, ids.data(), n1 - 1, ks, st, 0);
                 if (rc != FESC_OK) return rc;
             }
-            if ((rc = bsgs_pack_inputs(ctx, rot, xpk + (size_t)(s0 / 4) * tile_bytes, level, ns, terms, st)) != FESC_OK) return rc;
+            if ((rc = bsgs_pack_inputs(ctx, rot, xpk + (size_t)(s0 / 4) * tile_bytes, level, ns, terms, periodic, st)) != FESC_OK) return rc;
         }
         for (uint32_t b0 = 0; b0 < nout; b0 += nb_part) {
             const uint32_t nb = nout - b0 < nb_part ? nout - b0 : nb_part;
-            rc = bsgs_accumulate_packed(ctx, xpk, image + (size_t)(b0 * n2 / 8) * image_tile_bytes, acc, level, nt, terms, nb * n2,
-                                        qbits <= 50, dshift, st);
+            const auto accumulate = periodic ? bsgs_accumulate_periodic : bsgs_accumulate_packed;
+            rc = accumulate(ctx, xpk, image + (size_t)(b0 * n2 / 8) * image_tile_bytes, acc, level, nt, terms, nb * n2, qbits <= 50, dshift, st);
             if (rc != FESC_OK) return rc;
             ctx->counters[2] += (uint64_t)nt * nb * n2 * terms;
             if (desc->defer) {

@@ -121,15 +121,7 @@ __device__ __forceinline__ void byte_planes4(u64 w0, u64 w1, u64 w2, u64 w3, uin
 // primes below 2^50 (|fp_reduce| <= q/2 and every lazy product within 2q, so the sum stays below 6.5 q < 2^53), as a
 // 128-bit integer otherwise.  c32, c64, c96 = 2^32, 2^64, 2^96 mod q (FP path only).
 template <bool FP>
-__device__ __forceinline__ u64 imma_recombine(const int (&d)[4][7][4], int sel, const PrimeConst& pc, double c32, double c64,
-                                              double c96) {
-    uint32_t e[13];
-#pragma unroll
-    for (int x = 0; x < 13; x++) e[x] = 0;
-#pragma unroll
-    for (int k = 0; k < 7; k++)
-#pragma unroll
-        for (int j = 0; j < 7; j++) e[k + j] += (uint32_t)d[k >> 1][j][(k & 1) * 2 + sel];
+__device__ __forceinline__ u64 imma_reduce(const uint32_t (&e)[13], const PrimeConst& pc, double c32, double c64, double c96) {
     const u64 w0 = e[0] + ((u64)e[1] << 8) + ((u64)e[2] << 16) + ((u64)e[3] << 24);
     const u64 w1 = e[4] + ((u64)e[5] << 8) + ((u64)e[6] << 16) + ((u64)e[7] << 24);
     const u64 w2 = e[8] + ((u64)e[9] << 8) + ((u64)e[10] << 16) + ((u64)e[11] << 24);
@@ -141,6 +133,18 @@ __device__ __forceinline__ u64 imma_recombine(const int (&d)[4][7][4], int sel, 
     }
     const u128 S = (u128)w0 + ((u128)w1 << 32) + ((u128)w2 << 64) + ((u128)e[12] << 96);
     return reduce128((u64)(S >> 64), (u64)S, pc);
+}
+template <bool FP>
+__device__ __forceinline__ u64 imma_recombine(const int (&d)[4][7][4], int sel, const PrimeConst& pc, double c32, double c64,
+                                              double c96) {
+    uint32_t e[13];
+#pragma unroll
+    for (int x = 0; x < 13; x++) e[x] = 0;
+#pragma unroll
+    for (int k = 0; k < 7; k++)
+#pragma unroll
+        for (int j = 0; j < 7; j++) e[k + j] += (uint32_t)d[k >> 1][j][(k & 1) * 2 + sel];
+    return imma_reduce<FP>(e, pc, c32, c64, c96);
 }
 #endif
 
@@ -172,6 +176,10 @@ int small_rescale(fesc_ctx* ctx, const u64* in, size_t in_stride, u64* out, size
 // packed-operand BSGS accumulate (packed.cu)
 size_t bsgs_packed_bytes(uint32_t N, uint32_t level, uint32_t rows, uint32_t terms);
 bool bsgs_packed_supported(const fesc_ctx* ctx, uint32_t level, uint32_t terms, uint32_t dshift);
-int bsgs_pack_inputs(fesc_ctx* ctx, const u64* rot, uint8_t* xpk, uint32_t level, uint32_t tbs, uint32_t terms, cudaStream_t st);
+int bsgs_pack_inputs(fesc_ctx* ctx, const u64* rot, uint8_t* xpk, uint32_t level, uint32_t tbs, uint32_t terms, bool cores, cudaStream_t st);
 int bsgs_accumulate_packed(fesc_ctx* ctx, const uint8_t* xpk, const uint8_t* dpk, u64* acc, uint32_t level, uint32_t tbs,
                            uint32_t terms, uint32_t bp_count, bool fp, uint32_t dshift, cudaStream_t st);
+// the same for periodic diagonals (packed_tc.cu); its inputs are packed with `cores`
+bool bsgs_periodic_supported(uint32_t terms, uint32_t bp_count, uint32_t dshift);
+int bsgs_accumulate_periodic(fesc_ctx* ctx, const uint8_t* xpk, const uint8_t* dpk, u64* acc, uint32_t level, uint32_t tbs, uint32_t terms,
+                             uint32_t bp_count, bool fp, uint32_t dshift, cudaStream_t st);

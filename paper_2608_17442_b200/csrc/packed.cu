@@ -42,7 +42,7 @@ size_t bsgs_packed_bytes(uint32_t N, uint32_t level, uint32_t rows, uint32_t ter
 template <bool A_SIDE>
 __global__ void __launch_bounds__(256) k_pack_fragments(const u64* __restrict__ src, uint8_t* __restrict__ dst, uint32_t N,
                                                         uint32_t level, uint32_t rows, uint32_t terms, uint32_t ksteps,
-                                                        size_t stride_hi, size_t stride_lo, size_t term_stride) {
+                                                        size_t stride_hi, size_t stride_lo, size_t term_stride, bool cores) {
     __shared__ u64 sm[8 * PK_BLK];
     const uint32_t tid = threadIdx.x, cw = tid & 7, rw = tid >> 3;
     const uint32_t ct = blockIdx.x, l = blockIdx.y, tile = blockIdx.z / ksteps, ks = blockIdx.z - tile * ksteps;
@@ -82,6 +82,12 @@ __global__ void __launch_bounds__(256) k_pack_fragments(const u64* __restrict__ 
         for (int m = 0; m < 3; m++)
             *(uint4*)(out + m * 512 + lane * 16) = make_uint4(lo[2 * m], lo[2 * m + 1], hi[2 * m], hi[2 * m + 1]);
         *(uint2*)(out + 1536 + lane * 8) = make_uint2(lo[6], hi[6]);
+    } else if (cores) {                      // inputs of the periodic accumulate: terms 0-15 and 16-31 of the 8 columns, 128 bytes each
+#pragma unroll
+        for (int j = 0; j < 7; j++) {
+            *(uint32_t*)(out + j * 256 + lane * 4) = lo[j];
+            *(uint32_t*)(out + j * 256 + 128 + lane * 4) = hi[j];
+        }
     } else {
 #pragma unroll
         for (int j = 0; j < 7; j++) *(uint2*)(out + j * 256 + lane * 8) = make_uint2(lo[j], hi[j]);
@@ -89,13 +95,13 @@ __global__ void __launch_bounds__(256) k_pack_fragments(const u64* __restrict__ 
 }
 
 int bsgs_pack_inputs(fesc_ctx* ctx, const u64* rot, uint8_t* xpk, uint32_t level, uint32_t tbs, uint32_t terms,
-                     cudaStream_t st) {
+                     bool cores, cudaStream_t st) {
     const uint32_t N = ctx->N, ksteps = (terms + 31) / 32, tiles = (2 * tbs + 7) / 8;
     const size_t poly = (size_t)level * N, ctw = 2 * poly;
     dim3 grid(N / PK_CW, level, tiles * ksteps);
     if (grid.z > 65535 || level > 65535) return fesc_fail(ctx, FESC_EINVAL, "linear: too many packing tiles");
     prof_begin(ctx, PF_POINTWISE, st);
-    k_pack_fragments<false><<<grid, 256, 0, st>>>(rot, xpk, N, level, 2 * tbs, terms, ksteps, (size_t)terms * ctw, poly, ctw);
+    k_pack_fragments<false><<<grid, 256, 0, st>>>(rot, xpk, N, level, 2 * tbs, terms, ksteps, (size_t)terms * ctw, poly, ctw, cores);
     prof_end(ctx, PF_POINTWISE, st);
     FESC_CHECK_CUDA(ctx, cudaGetLastError());
     return FESC_OK;
@@ -342,7 +348,7 @@ extern "C" int fesc_linear_pack_diags(fesc_ctx* ctx, const uint64_t* d_diags, co
     if (grid.z > 65535 || level > 65535) return fesc_fail(ctx, FESC_EINVAL, "pack_diags: range too large for one call");
     uint8_t* dst = (uint8_t*)d_packed + (size_t)(first / 8) * level * N * ksteps * PK_FRAG;
     k_pack_fragments<true><<<grid, 256, 0, (cudaStream_t)stream>>>((const u64*)d_diags, dst, N, level, count, terms, ksteps,
-                                                                   (size_t)terms * poly, 0, poly);
+                                                                   (size_t)terms * poly, 0, poly, false);
     ctx->counters[4] += 1;
     FESC_CHECK_CUDA(ctx, cudaGetLastError());
     return FESC_OK;
