@@ -7,11 +7,12 @@
 // images its tensor pipe was 0.62 busy and is several times narrower.
 //
 // One instruction multiplies byte plane k of the 128 outputs with all planes j of the inputs, and the sums of equal weight 256^(k+j)
-// belong together.  They land together without any arithmetic: the input planes lie in shared memory between six groups of zeros, and
-// the instruction for plane k takes the window that starts k groups early, so that plane j meets accumulator column group k + j.  The
-// 13 sums of a product then sit in one row of tensor memory: a thread owns an output, and no exchange between lanes is left.
+// belong together.  They land together without any arithmetic: the accumulator of planes 2m and 2m + 1 starts 2m column groups to the
+// right, and plane 2m + 1 takes its inputs from one group early, where a group of zeros lies.  The 13 sums of a product then sit in one row
+// of tensor memory: a thread owns an output, and no exchange between lanes is left.  64 columns per instruction (windows of all 14 groups, 112
+// columns, took 111 ms for 8 token blocks of 210 outputs x 189 terms).
 //
-// CTA = 6 warps: 4 recombine (thread = output), one issues the products, one fetches the inputs.  Two accumulators (2 x 128 columns of
+// CTA = 10 warps: 8 recombine (thread = output and half of the columns), one issues the products, one fetches the inputs.  Two accumulators (2 x 128 columns of
 // tensor memory) let the recombination of a coefficient run beside the products of the next.  Every wait is bounded (status word 4).
 #define FESC_DBG_FILE 15   // file id in the sites a debug build reports
 #include "ops.cuh"
@@ -19,11 +20,12 @@
 #define TC_FRAG 1792                       // bytes of one coefficient's inputs per k-step of 32 terms: [plane][k half][8 rows][16]
 #define TC_CORE 256                        // 8 rows x 32 terms: two core matrices of 8 x 16 bytes
 #define TC_MAX_KSTEPS 6
-#define TC_THREADS 192
+#define TC_THREADS 320
+#define TC_OUT_WARPS 8
 #define TC_BUFFERS 4
-#define TC_N 112                           // 14 groups of 8 columns; the last one is never read
 #define TC_A_BYTES(ksteps) (7u * (ksteps) * 16 * TC_CORE)
-#define TC_B_BYTES(ksteps) ((7u + 13 * (ksteps)) * TC_CORE)      // 6 groups of zeros around every k-step, one spare at the end
+#define TC_B_BYTES(ksteps) ((1u + 8 * (ksteps)) * TC_CORE)       // a group of zeros before and after every k-step's seven
+#define TC_ZERO_BYTES (6u * TC_CORE)       // the right operand that clears the columns which the first product does not reach
 
 // shared-memory operand without swizzle, both core matrices of a row group side by side: K direction 128 bytes, row groups 256
 __device__ __forceinline__ u64 tc_desc(uint32_t addr) {
@@ -69,21 +71,21 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     }
 #endif
     const uint32_t a_base = (uint32_t)__cvta_generic_to_shared(smem), a_bytes = TC_A_BYTES(ksteps), b_bytes = TC_B_BYTES(ksteps);
-    const uint32_t bar = (uint32_t)__cvta_generic_to_shared(bars);
+    const uint32_t b_base = a_base + a_bytes + TC_ZERO_BYTES, bar = (uint32_t)__cvta_generic_to_shared(bars);
     const uint32_t b_full = bar, b_free = bar + 8 * TC_BUFFERS, d_full = bar + 16 * TC_BUFFERS, d_free = d_full + 16, drained = d_free + 16;
-    if (warp == 4) {
+    if (warp == TC_OUT_WARPS) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 256;" ::"r"((uint32_t)__cvta_generic_to_shared(&tmem_base))
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     if (tid == 0) {
         for (uint32_t i = 0; i < TC_BUFFERS; i++) mbar_init(b_full + 8 * i, 1), mbar_init(b_free + 8 * i, 1);
-        for (uint32_t i = 0; i < 2; i++) mbar_init(d_full + 8 * i, 1), mbar_init(d_free + 8 * i, 4);
+        for (uint32_t i = 0; i < 2; i++) mbar_init(d_full + 8 * i, 1), mbar_init(d_free + 8 * i, TC_OUT_WARPS);
         mbar_init(drained, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     // zeros around the inputs, and the left operand: [plane][k-step][16 row groups][k half][8 rows][16 bytes]
-    for (uint32_t i = tid; i < buffers * (b_bytes / 16); i += TC_THREADS) *reinterpret_cast<uint4*>(smem + a_bytes + 16 * i) = make_uint4(0, 0, 0, 0);
+    for (uint32_t i = tid; i < (TC_ZERO_BYTES + buffers * b_bytes) / 16; i += TC_THREADS) *reinterpret_cast<uint4*>(smem + a_bytes + 16 * i) = make_uint4(0, 0, 0, 0);
     for (uint32_t i = warp; i < 16 * ksteps; i += TC_THREADS / 32) {
         const uint32_t rg = i / ksteps, ks = i - rg * ksteps, bt = mt * 16 + rg;
         uint32_t lo[7] = {}, hi[7] = {};
@@ -109,7 +111,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = tmem_base;
     bool ok = true;
-    if (warp == 5) {                       // fetches the inputs
+    if (warp == TC_OUT_WARPS + 1) {                       // fetches the inputs
         if (lane == 0) {
             uint32_t i = 0;
             for (; i < coefs; i++) {
@@ -121,16 +123,16 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                 const uint8_t* src = xsrc + (size_t)(c >> 3) * ksteps * stage + (c & 7) * TC_FRAG;
                 mbar_expect_tx(b_full + 8 * buf, ksteps * TC_FRAG);
                 for (uint32_t k = 0; k < ksteps; k++)
-                    bulk_g2s(a_base + a_bytes + buf * b_bytes + (6 + 13 * k) * TC_CORE, src + k * stage, TC_FRAG, b_full + 8 * buf);
+                    bulk_g2s(b_base + buf * b_bytes + (1 + 8 * k) * TC_CORE, src + k * stage, TC_FRAG, b_full + 8 * buf);
             }
             // copies in flight when a wait ran out: the last `buffers` of them
             if (!ok)
                 for (uint32_t s = i > buffers ? i - buffers : 0; s < i; s++) mbar_wait_bounded(b_full + 8 * (s % buffers), (s / buffers) & 1);
         }
-    } else if (warp == 4) {                // issues the products
+    } else if (warp == TC_OUT_WARPS) {                // issues the products
         if (lane == 0) {
-            // u8 x u8 -> s32, both operands K-major, 128 x TC_N
-            const uint32_t idesc = (2u << 4) | ((TC_N / 8u) << 17) | ((128u / 16) << 24);
+            // u8 x u8 -> s32, both operands K-major, 128 rows x 64 or 48 columns
+            const uint32_t idesc = (2u << 4) | (8u << 17) | (8u << 24), idesc48 = (2u << 4) | (6u << 17) | (8u << 24);
             for (uint32_t i = 0; i < coefs; i++) {
                 const uint32_t buf = i % buffers, use = i / buffers, db = i & 1, du = i >> 1;
                 if (mbar_wait_bounded(b_full + 8 * buf, use & 1) || (du && mbar_wait_bounded(d_free + 8 * db, (du - 1) & 1))) {
@@ -138,11 +140,13 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                     break;
                 }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t b0 = a_base + a_bytes + buf * b_bytes, d = tmem + 128 * db;
+                const uint32_t b0 = b_base + buf * b_bytes, d = tmem + 128 * db;
+                tc_mma(d + 64, tc_desc(a_base), tc_desc(a_base + a_bytes), idesc48, false);
                 for (uint32_t k = 0; k < ksteps; k++)
 #pragma unroll
                     for (uint32_t p = 0; p < 7; p++)
-                        tc_mma(d, tc_desc(a_base + (p * ksteps + k) * 16 * TC_CORE), tc_desc(b0 + (6 + 13 * k - p) * TC_CORE), idesc, k || p);
+                        tc_mma(d + 16 * (p >> 1), tc_desc(a_base + (p * ksteps + k) * 16 * TC_CORE), tc_desc(b0 + (1 + 8 * k - (p & 1)) * TC_CORE), idesc,
+                               k || p);
                 tc_commit(b_free + 8 * buf);
                 tc_commit(d_full + 8 * db);
             }
@@ -157,42 +161,37 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             c64 = fp_modmul(c32, c32, pc.qd, pc.qinvd);
             c96 = fp_modmul(c64, c32, pc.qd, pc.qinvd);
         }
-        const uint32_t bp = mt * 128 + tid;
+        const uint32_t row = tid & 127, half = warp >> 2, bp = mt * 128 + row;
         u64* out = acc + (size_t)bp * ctw + (size_t)l * N + c_first;
         for (uint32_t i0 = 0; i0 < coefs && ok; i0 += 4) {      // four coefficients make a full sector of every output row
-            u64 r[8][4];
+            u64 r[4][4];
 #pragma unroll
             for (uint32_t e = 0; e < 4; e++) {
                 const uint32_t i = i0 + e, db = i & 1, du = i >> 1;
                 if (ok && mbar_wait_bounded(d_full + 8 * db, du & 1)) ok = false;
                 ok = __all_sync(0xFFFFFFFFu, ok);
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                uint32_t s[13][4];
 #pragma unroll
-                for (int h = 0; h < 2; h++) {
-                    uint32_t s[13][4];
+                for (int x = 0; x < 13; x++) tc_ld4(s[x], tmem + 128 * db + 8 * x + 4 * half + ((32 * (warp & 3)) << 16));
+                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-                    for (int x = 0; x < 13; x++) tc_ld4(s[x], tmem + 128 * db + 8 * x + 4 * h + ((32 * warp) << 16));
-                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                for (int x = 0; x < 13; x++)          // no use of a loaded word moves above the wait
+                    asm volatile("" : "+r"(s[x][0]), "+r"(s[x][1]), "+r"(s[x][2]), "+r"(s[x][3]));
+                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                if (lane == 0) mbar_arrive(d_free + 8 * db);
 #pragma unroll
-                    for (int x = 0; x < 13; x++)          // no use of a loaded word moves above the wait
-                        asm volatile("" : "+r"(s[x][0]), "+r"(s[x][1]), "+r"(s[x][2]), "+r"(s[x][3]));
-                    if (h) {
-                        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                        if (lane == 0) mbar_arrive(d_free + 8 * db);
-                    }
+                for (int n = 0; n < 4; n++) {
+                    uint32_t v[13];
 #pragma unroll
-                    for (int n = 0; n < 4; n++) {
-                        uint32_t v[13];
-#pragma unroll
-                        for (int x = 0; x < 13; x++) v[x] = s[x][n];
-                        r[4 * h + n][e] = imma_reduce<FP>(v, pc, c32, c64, c96);
-                    }
+                    for (int x = 0; x < 13; x++) v[x] = s[x][n];
+                    r[n][e] = imma_reduce<FP>(v, pc, c32, c64, c96);
                 }
             }
             if (ok && bp < bp_count) {
 #pragma unroll
-                for (uint32_t n = 0; n < 8; n++) {
-                    const uint32_t tb = tbt * 4 + (n >> 1);
+                for (uint32_t n = 0; n < 4; n++) {
+                    const uint32_t tb = tbt * 4 + 2 * half + (n >> 1);
                     if (tb >= tbs) break;
                     u64* o = out + (size_t)tb * bp_count * ctw + (n & 1) * poly + i0;
                     *reinterpret_cast<ulonglong2*>(o) = make_ulonglong2(r[n][0], r[n][1]);
@@ -205,11 +204,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     __syncwarp();
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    if (warp == 4) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 256;" ::"r"(tmem));
+    if (warp == TC_OUT_WARPS) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 256;" ::"r"(tmem));
 }
 
 static uint32_t tc_buffers(uint32_t ksteps) {
-    const uint32_t fit = (226u * 1024 - TC_A_BYTES(ksteps)) / TC_B_BYTES(ksteps);
+    const uint32_t fit = (226u * 1024 - TC_ZERO_BYTES - TC_A_BYTES(ksteps)) / TC_B_BYTES(ksteps);
     return fit < TC_BUFFERS ? fit : TC_BUFFERS;
 }
 // The left operand is worth its place in shared memory when at least 16 coefficients use it and a good part of its 128 rows is filled
@@ -221,7 +220,7 @@ int bsgs_accumulate_periodic(fesc_ctx* ctx, const uint8_t* xpk, const uint8_t* d
                              uint32_t bp_count, bool fp, uint32_t dshift, cudaStream_t st) {
     const uint32_t N = ctx->N, ksteps = (terms + 31) / 32, buffers = tc_buffers(ksteps);
     const dim3 grid((N >> dshift) * ((bp_count + 127) / 128) * ((tbs + 3) / 4), level);
-    size_t smem = TC_A_BYTES(ksteps) + (size_t)buffers * TC_B_BYTES(ksteps);
+    size_t smem = TC_A_BYTES(ksteps) + TC_ZERO_BYTES + (size_t)buffers * TC_B_BYTES(ksteps);
     if (smem < 120 * 1024) smem = 120 * 1024;          // one CTA per SM: no CTA waits for another one's tensor memory
     auto kern = fp ? k_bsgs_accumulate_periodic<true> : k_bsgs_accumulate_periodic<false>;
     FESC_CHECK_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
