@@ -9,8 +9,12 @@
 // One instruction multiplies byte plane k of the 128 outputs with all planes j of the inputs, and the sums of equal weight 256^(k+j)
 // belong together.  They land together without any arithmetic: the accumulator of planes 2m and 2m + 1 starts 2m column groups to the
 // right, and plane 2m + 1 takes its inputs from one group early, where a group of zeros lies.  The 13 sums of a product then sit in one row
-// of tensor memory: a thread owns an output, and no exchange between lanes is left.  64 columns per instruction (windows of all 14 groups, 112
-// columns, took 111 ms for 8 token blocks of 210 outputs x 189 terms).
+// of tensor memory: a thread owns an output, and no exchange between lanes is left.  64 columns per instruction.
+//
+// 8 token blocks of 210 outputs x 189 terms at 24 limbs: 78 ms (167 ms in packed.cu).  Windows of all 14 column groups and one recombining
+// warp per scheduler 111; 16-byte stores and descriptors computed per product 90.  An instruction of 128 x 64 x 32 takes 48 cycles, what
+// reading its operands from shared memory takes, so the products alone need 46 ms; with issue, operand set-up and hand-over 62 without any recombination; the
+// scattered sectors of the outputs 35 by themselves.  Four accumulators instead of two: no change.
 //
 // CTA = 10 warps: 8 recombine (thread = output and half of the columns), one issues the products, one fetches the inputs.  Two accumulators (2 x 128 columns of
 // tensor memory) let the recombination of a coefficient run beside the products of the next.  Every wait is bounded (status word 4).
@@ -27,13 +31,13 @@
 #define TC_B_BYTES(ksteps) ((1u + 8 * (ksteps)) * TC_CORE)       // a group of zeros before and after every k-step's seven
 #define TC_ZERO_BYTES (6u * TC_CORE)       // the right operand that clears the columns which the first product does not reach
 
-// shared-memory operand without swizzle, both core matrices of a row group side by side: K direction 128 bytes, row groups 256
-__device__ __forceinline__ u64 tc_desc(uint32_t addr) {
-    return (u64)((addr & 0x3FFFF) >> 4) | ((u64)(128 >> 4) << 16) | ((u64)(TC_CORE >> 4) << 32) | (1ull << 46);
-}
-__device__ __forceinline__ void tc_mma(uint32_t d, u64 a, u64 b, uint32_t idesc, bool add) {
-    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %4, 0;\n\ttcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n\t}" ::"r"(d), "l"(a),
-                 "l"(b), "r"(idesc), "r"((uint32_t)add)
+// Shared-memory operand without swizzle, both core matrices of a row group side by side: K direction 128 bytes, row groups 256.  Only the
+// address, in the low word, differs between operands: one thread issues all products, and what it computes per product counts.
+#define TC_DESC_HI ((uint32_t)(TC_CORE >> 4) | (1u << 14))
+__device__ __forceinline__ uint32_t tc_desc(uint32_t addr) { return (addr >> 4) | ((uint32_t)(128 >> 4) << 16); }
+__device__ __forceinline__ void tc_mma(uint32_t d, uint32_t a, uint32_t b, uint32_t idesc, bool add) {
+    asm volatile("{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\tmov.b64 a, {%1, %5};\n\tmov.b64 b, {%2, %5};\n\tsetp.ne.u32 p, %4, 0;\n\t"
+                 "tcgen05.mma.cta_group::1.kind::i8 [%0], a, b, %3, p;\n\t}" ::"r"(d), "r"(a), "r"(b), "r"(idesc), "r"((uint32_t)add), "r"(TC_DESC_HI)
                  : "memory");
 }
 __device__ __forceinline__ void tc_commit(uint32_t bar) {
@@ -43,11 +47,12 @@ __device__ __forceinline__ void tc_ld4(uint32_t* r, uint32_t addr) {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
 }
 
-template <bool FP>
+template <bool FP, int KS>
 __global__ void __launch_bounds__(TC_THREADS, 1)
     k_bsgs_accumulate_periodic(const uint8_t* __restrict__ xpk, const uint8_t* __restrict__ dpk, u64* __restrict__ acc,
-                               const PrimeConst* __restrict__ pcs, uint32_t N, uint32_t level, uint32_t tbs, uint32_t ksteps, uint32_t bp_count,
-                               uint32_t dshift, uint32_t buffers, uint32_t* __restrict__ status) {
+                               const PrimeConst* __restrict__ pcs, uint32_t N, uint32_t level, uint32_t tbs, uint32_t bp_count, uint32_t dshift,
+                               uint32_t buffers, uint32_t* __restrict__ status) {
+    constexpr uint32_t ksteps = KS;
     extern __shared__ __align__(128) uint8_t smem[];
     __shared__ __align__(8) u64 bars[2 * TC_BUFFERS + 5];
     __shared__ uint32_t tmem_base;
@@ -84,7 +89,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         mbar_init(drained, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    // zeros around the inputs, and the left operand: [plane][k-step][16 row groups][k half][8 rows][16 bytes]
+    // zeros around the inputs, and the left operand: [k-step][plane][16 row groups][k half][8 rows][16 bytes]
     for (uint32_t i = tid; i < (TC_ZERO_BYTES + buffers * b_bytes) / 16; i += TC_THREADS) *reinterpret_cast<uint4*>(smem + a_bytes + 16 * i) = make_uint4(0, 0, 0, 0);
     for (uint32_t i = warp; i < 16 * ksteps; i += TC_THREADS / 32) {
         const uint32_t rg = i / ksteps, ks = i - rg * ksteps, bt = mt * 16 + rg;
@@ -101,7 +106,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         }
 #pragma unroll
         for (int p = 0; p < 7; p++) {
-            uint32_t* dst = reinterpret_cast<uint32_t*>(smem + ((p * ksteps + ks) * 16 + rg) * TC_CORE) + lane;
+            uint32_t* dst = reinterpret_cast<uint32_t*>(smem + ((ks * 7 + p) * 16 + rg) * TC_CORE) + lane;
             dst[0] = lo[p], dst[32] = hi[p];
         }
     }
@@ -133,6 +138,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         if (lane == 0) {
             // u8 x u8 -> s32, both operands K-major, 128 rows x 64 or 48 columns
             const uint32_t idesc = (2u << 4) | (8u << 17) | (8u << 24), idesc48 = (2u << 4) | (6u << 17) | (8u << 24);
+            const uint32_t a0 = tc_desc(a_base), zero = tc_desc(a_base + a_bytes);
             for (uint32_t i = 0; i < coefs; i++) {
                 const uint32_t buf = i % buffers, use = i / buffers, db = i & 1, du = i >> 1;
                 if (mbar_wait_bounded(b_full + 8 * buf, use & 1) || (du && mbar_wait_bounded(d_free + 8 * db, (du - 1) & 1))) {
@@ -140,13 +146,13 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                     break;
                 }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t b0 = b_base + buf * b_bytes, d = tmem + 128 * db;
-                tc_mma(d + 64, tc_desc(a_base), tc_desc(a_base + a_bytes), idesc48, false);
-                for (uint32_t k = 0; k < ksteps; k++)
+                const uint32_t b0 = tc_desc(b_base + TC_CORE + buf * b_bytes), d = tmem + 128 * db;
+                tc_mma(d + 64, a0, zero, idesc48, false);
+#pragma unroll
+                for (uint32_t k = 0; k < KS; k++)
 #pragma unroll
                     for (uint32_t p = 0; p < 7; p++)
-                        tc_mma(d + 16 * (p >> 1), tc_desc(a_base + (p * ksteps + k) * 16 * TC_CORE), tc_desc(b0 + (1 + 8 * k - (p & 1)) * TC_CORE), idesc,
-                               k || p);
+                        tc_mma(d + 16 * (p >> 1), a0 + (k * 7 + p) * TC_CORE, b0 + (8 * k - (p & 1)) * (TC_CORE / 16), idesc, k || p);
                 tc_commit(b_free + 8 * buf);
                 tc_commit(d_full + 8 * db);
             }
@@ -194,8 +200,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                     const uint32_t tb = tbt * 4 + 2 * half + (n >> 1);
                     if (tb >= tbs) break;
                     u64* o = out + (size_t)tb * bp_count * ctw + (n & 1) * poly + i0;
-                    *reinterpret_cast<ulonglong2*>(o) = make_ulonglong2(r[n][0], r[n][1]);
-                    *reinterpret_cast<ulonglong2*>(o + 2) = make_ulonglong2(r[n][2], r[n][3]);
+                    // whole sectors: 16-byte stores took twice the time (59 against 35 ms with the arithmetic left out)
+                    asm volatile("st.global.v4.b64 [%0], {%1, %2, %3, %4};" ::"l"(o), "l"(r[n][0]), "l"(r[n][1]), "l"(r[n][2]), "l"(r[n][3]) : "memory");
                 }
             }
         }
@@ -222,10 +228,19 @@ int bsgs_accumulate_periodic(fesc_ctx* ctx, const uint8_t* xpk, const uint8_t* d
     const dim3 grid((N >> dshift) * ((bp_count + 127) / 128) * ((tbs + 3) / 4), level);
     size_t smem = TC_A_BYTES(ksteps) + TC_ZERO_BYTES + (size_t)buffers * TC_B_BYTES(ksteps);
     if (smem < 120 * 1024) smem = 120 * 1024;          // one CTA per SM: no CTA waits for another one's tensor memory
-    auto kern = fp ? k_bsgs_accumulate_periodic<true> : k_bsgs_accumulate_periodic<false>;
-    FESC_CHECK_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+#define TC_LAUNCH(FP, KS)                                                                                                               \
+    case KS: {                                                                                                                          \
+        auto kern = k_bsgs_accumulate_periodic<FP, KS>;                                                                                 \
+        FESC_CHECK_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));                       \
+        kern<<<grid, TC_THREADS, smem, st>>>(xpk, dpk, acc, ctx->d_pc, N, level, tbs, bp_count, dshift, buffers, ctx->d_status);        \
+    } break;
+#define TC_PICK(FP) \
+    switch (ksteps) { TC_LAUNCH(FP, 1) TC_LAUNCH(FP, 2) TC_LAUNCH(FP, 3) TC_LAUNCH(FP, 4) TC_LAUNCH(FP, 5) TC_LAUNCH(FP, 6) }
     prof_begin(ctx, PF_BSGS, st);
-    kern<<<grid, TC_THREADS, smem, st>>>(xpk, dpk, acc, ctx->d_pc, N, level, tbs, ksteps, bp_count, dshift, buffers, ctx->d_status);
+    if (fp) TC_PICK(true)
+    else TC_PICK(false)
+#undef TC_PICK
+#undef TC_LAUNCH
     prof_end(ctx, PF_BSGS, st);
     FESC_CHECK_CUDA(ctx, cudaGetLastError());
     return FESC_OK;
