@@ -148,7 +148,7 @@ int fesc_ctx_export_secret(fesc_ctx* ctx, uint64_t* d_dst, void* stream);
 uint32_t fesc_ctx_num_digits(const fesc_ctx* ctx);
 /* Counters since creation: [0] limb transforms, [1] key switches, [2] ct-pt MACs (per
  * ciphertext), [3] bytes of scratch currently reserved, [4] kernel launches, [5] token blocks per group of the last
- * fesc_linear call; [6..7] zero. */
+ * fesc_linear call, [6] passes of limb transforms outside fused conversions and inner products (two per transform); [7] zero. */
 int fesc_ctx_counters(const fesc_ctx* ctx, uint64_t out[8]);
 /*
  * Optional timing of kernel families with CUDA events recorded on the launching stream

@@ -95,6 +95,7 @@ int ntt_launch(fesc_ctx* ctx, u64* d_data, size_t rows, const RowMap& map, bool 
     size_t live = 0;
     for (uint32_t i = 0; i < map.period; i++) live += map.prime[i] != 0xFF;
     ctx->counters[0] += rows / map.period * live;
+    ctx->counters[6] += rows / map.period * live * (skip_cols ? 1 : 2);
     prof_begin(ctx, PF_NTT, st);
     uint64_t launches = 0;
     if (ctx->log_n == 16) {

@@ -958,6 +958,7 @@ static int ks_inner_multi(fesc_ctx* ctx, const KsScratch& ws, const InnerSrcs& S
     } else if (open) {
         const int rc = rows_inner_launch(ctx, S, ws.acc, level, batch, accumulate, separate, st);
         if (rc != FESC_OK) return rc;
+        ctx->counters[0] += (uint64_t)batch * S.n * level * (beta - 1);      // transforms that end in the inner product
     } else if (split) {
         INNER_BATCH(1, 0, level);
         INNER_BATCH(2, level, K);
