@@ -350,6 +350,13 @@ __device__ __forceinline__ uint32_t galois_src(uint32_t t, uint32_t log_n, u64 g
     return __brev((e - 1) >> 1) >> (32 - log_n);
 }
 
+// the words that the automorphism takes to t and t + 1 (t even): it maps aligned pairs to aligned pairs, in either order
+__device__ __forceinline__ ulonglong2 galois_pair(const u64* __restrict__ in, uint32_t t, uint32_t log_n, u64 g, bool wide) {
+    const uint32_t src = galois_src(t, log_n, g);
+    const ulonglong2 v = ld_pair(in + (src & ~1u), wide);
+    return src & 1 ? make_ulonglong2(v.y, v.x) : v;
+}
+
 // Where the EVAL-form polynomial being switched is kept: the rows of the extended-digit buffer that belong to a
 // digit's own limbs (row l of digit l / alpha), which the basis extension leaves untouched.  The inner product then
 // reads every (digit, row) from one array.

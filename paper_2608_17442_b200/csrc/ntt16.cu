@@ -168,16 +168,16 @@ __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
         const u64* pt = FIN == 2 && fin.pt ? fin.pt + ct * fin.pt_stride + (size_t)i * N16 + blk * 512 + 2 * lane : nullptr;
         if (pt && !DBG_REGION(pt - 2 * lane, 512 * sizeof(u64))) return;
         const double mul = FIN == 2 ? fp_mod_u64(fin.mul, pcs[pi]) : 0.0;
-        const bool wide = FIN == 2 && pair_aligned(acc), wide_pt = FIN == 2 && pair_aligned(pt);
+        const bool wide = pair_aligned(FIN == 2 ? acc : rot), wide_pt = FIN == 2 && pair_aligned(pt);
         ulonglong2 av[8];
 #pragma unroll
         for (int j = 0; j < 8; j++) av[j] = ld_pair(acc + blk * 512 + 2 * lane + 64 * j, FIN == 1 || wide);
 #pragma unroll
         for (int h = 0; h < 8; h += 4) {
-            u64 w[8];
+            ulonglong2 w[4];
             if (FIN == 1 && rot) {
 #pragma unroll
-                for (int j = 0; j < 8; j++) w[j] = rot[galois_src(blk * 512 + 2 * lane + 64 * (h + (j >> 1)) + (j & 1), 16, rot_g)];
+                for (int j = 0; j < 4; j++) w[j] = galois_pair(rot, blk * 512 + 2 * lane + 64 * (h + j), 16, rot_g, wide);
             }
 #pragma unroll
             for (int j = h; j < h + 4; j++) {
@@ -191,8 +191,8 @@ __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
                 double s0 = fp_modmul(a0 - FpRow::value(v.x), cinv, q, qinv);
                 double s1 = fp_modmul(a1 - FpRow::value(v.y), cinv, q, qinv);
                 if (FIN == 1 && rot) {
-                    s0 += fp_load(w[2 * (j - h)], q);
-                    s1 += fp_load(w[2 * (j - h) + 1], q);
+                    s0 += fp_load(w[j - h].x, q);
+                    s1 += fp_load(w[j - h].y, q);
                 }
                 ulonglong2* o = reinterpret_cast<ulonglong2*>(out + blk * 512 + 2 * lane + 64 * j);
                 if (FIN == 1 && add) {
@@ -252,7 +252,7 @@ __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
     auto pair = [&](int j) {
         if (!SRC) return *reinterpret_cast<const ulonglong2*>(in + 64 * j);
         if (!g) return ld_pair(in + at + 64 * j, wide);
-        return make_ulonglong2(in[galois_src(at + 64 * j, 16, g)], in[galois_src(at + 64 * j + 1, 16, g)]);
+        return galois_pair(in, at + 64 * j, 16, g, wide);
     };
     u64* s = sm + 2 * lane + 2 * (lane >> 3);
     u64* o = p + 256 * (lane >> 4) + (lane & 15);

@@ -1428,10 +1428,9 @@ __global__ void __launch_bounds__(256) k_rotsum_prepare(const u64* __restrict__ 
     ulonglong2 v = ld_pair(c0 + t, wide);
 #pragma unroll 4
     for (uint32_t k = 0; k < gs.n; k++) {
-        const uint32_t src = galois_src(t, log_n, gs.g[k]);
-        const ulonglong2 w = ld_pair(c0 + (src & ~1u), wide);
-        v.x = addmod(v.x, src & 1 ? w.y : w.x, q);
-        v.y = addmod(v.y, src & 1 ? w.x : w.y, q);
+        const ulonglong2 w = galois_pair(c0, t, log_n, gs.g[k], wide);
+        v.x = addmod(v.x, w.x, q);
+        v.y = addmod(v.y, w.y, q);
     }
     st_pair(ob + (size_t)l * N + t, v, wide_out);
     st_pair(ob + ((size_t)level + l) * N + t, c1, wide_out);
@@ -1645,12 +1644,18 @@ extern "C" int fesc_rescale(fesc_ctx* ctx, const uint64_t* d_in, uint64_t* d_out
 // ---------------------------------------------------------------------------------------
 // ct x ct: tensor product, then relinearisation of d2
 // ---------------------------------------------------------------------------------------
+__device__ __forceinline__ void tensor_word(u64 a0, u64 a1, u64 b0, u64 b1, const PrimeConst& pc, u64& d0, u64& d1, u64& d2) {
+    acc128 s{0, 0};
+    mac128(s, a0, b1);
+    mac128(s, a1, b0);
+    d0 = mulmod(a0, b0, pc), d1 = reduce128(s.hi, s.lo, pc), d2 = mulmod(a1, b1, pc);
+}
 __global__ void __launch_bounds__(256) k_tensor(const u64* __restrict__ a, size_t a_stride, const u64* __restrict__ bb,
                                                 size_t b_stride, u64* __restrict__ out, size_t out_stride,
                                                 OwnRows d, u64* __restrict__ dcoef,
                                                 const PrimeConst* __restrict__ pcs, uint32_t N, uint32_t level) {
     pdl_begin();
-    const uint32_t c = blockIdx.x * blockDim.x + threadIdx.x;
+    const uint32_t c = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
     const uint32_t l = blockIdx.y, b = blockIdx.z;
     if (c >= N) return;
     const PrimeConst pc = pcs[l];
@@ -1660,16 +1665,17 @@ __global__ void __launch_bounds__(256) k_tensor(const u64* __restrict__ a, size_
             !DBG_REGION(out + b * out_stride + p * poly + o - c, N * sizeof(u64)))
             return;
     if (!DBG_REGION(d.ext + own_index(d, b, l, N), N * sizeof(u64)) || !DBG_REGION(dcoef + ((size_t)b * level + l) * N, N * sizeof(u64))) return;
-    const u64 a0 = a[b * a_stride + o], a1 = a[b * a_stride + poly + o];
-    const u64 b0 = bb[b * b_stride + o], b1 = bb[b * b_stride + poly + o];
-    out[b * out_stride + o] = mulmod(a0, b0, pc);
-    acc128 s{0, 0};
-    mac128(s, a0, b1);
-    mac128(s, a1, b0);
-    out[b * out_stride + poly + o] = reduce128(s.hi, s.lo, pc);
-    const u64 d2 = mulmod(a1, b1, pc);
-    d.ext[own_index(d, b, l, N) + c] = own_word(d, d2, pc);
-    dcoef[((size_t)b * level + l) * N + c] = d2;
+    const bool wide_a = pair_aligned(a), wide_b = pair_aligned(bb), wide_out = pair_aligned(out);
+    const ulonglong2 va[2] = {ld_pair(a + b * a_stride + o, wide_a), ld_pair(a + b * a_stride + poly + o, wide_a)};
+    const ulonglong2 vb[2] = {ld_pair(bb + b * b_stride + o, wide_b), ld_pair(bb + b * b_stride + poly + o, wide_b)};
+    ulonglong2 d0, d1, d2, own;
+    tensor_word(va[0].x, va[1].x, vb[0].x, vb[1].x, pc, d0.x, d1.x, d2.x);
+    tensor_word(va[0].y, va[1].y, vb[0].y, vb[1].y, pc, d0.y, d1.y, d2.y);
+    own.x = own_word(d, d2.x, pc), own.y = own_word(d, d2.y, pc);
+    st_pair(out + b * out_stride + o, d0, wide_out);
+    st_pair(out + b * out_stride + poly + o, d1, wide_out);
+    *reinterpret_cast<ulonglong2*>(d.ext + own_index(d, b, l, N) + c) = own;
+    *reinterpret_cast<ulonglong2*>(dcoef + ((size_t)b * level + l) * N + c) = d2;
 }
 
 int ctmul_internal(fesc_ctx* ctx, const u64* a, size_t a_stride, const u64* b, size_t b_stride, u64* out,
@@ -1680,7 +1686,7 @@ int ctmul_internal(fesc_ctx* ctx, const u64* a, size_t a_stride, const u64* b, s
     KsScratch ws = ks_scratch_carve(ctx, scratch, level, cut);
     for (uint32_t b0 = 0; b0 < batch; b0 += chunk) {
         uint32_t nb = batch - b0 < chunk ? batch - b0 : chunk;
-        dim3 g((ctx->N + 255) / 256, level, nb);
+        dim3 g((ctx->N + 511) / 512, level, nb);
         prof_begin(ctx, PF_POINTWISE, st);
         launch(k_tensor, g, 256, 0, st, a + (size_t)b0 * a_stride, a_stride, b + (size_t)b0 * b_stride, b_stride,
                                     out + (size_t)b0 * out_stride, out_stride, own_rows(ctx, ws, level), ws.dcoef, ctx->d_pc, ctx->N, level);
