@@ -488,7 +488,7 @@ def measure_variants(args, ctx, ct, diags, out, gin, nout, tbs, n, dev):
     return variants
 
 
-def bsgs_roofline(args, gin, nout, n, tb_per_launch, timed, hbm_peak, sm_mhz):
+def bsgs_roofline(args, gin, nout, n, tbs, tb_per_launch, steps, timed, hbm_peak, sm_mhz):
     """Roofline of the accumulate family from (milliseconds, launches).  Packed operands: the kernel streams the
     byte-plane image once per launch (7 bytes per diagonal word), the packed inputs of its token blocks and writes the
     partial sums: HBM-bound; the tensor-core ceiling (u8 mma.sync m16n8k32 at 8 cycles per scheduler, measured) is
@@ -497,13 +497,15 @@ def bsgs_roofline(args, gin, nout, n, tb_per_launch, timed, hbm_peak, sm_mhz):
     t = ms * 1e-3 / max(1, launches)
     ctw = 2 * LEVEL * n * 8
     terms, bp = gin * N1, nout * N2
+    # a group of token blocks may take its outputs in several parts: a launch has its share of the image and of the outputs
+    bp /= max(1.0, launches / (steps * -(-tbs // tb_per_launch)))
     macs = tb_per_launch * bp * terms * 2 * LEVEL * n
     if args.packed:
         ksteps = -(-terms // 32)
-        image = -(-bp // 8) * LEVEL * n * ksteps * 1792                      # bytes: 8 rows x 32 terms x 7 planes per image
+        image = bp / 8 * LEVEL * n * ksteps * 1792                      # bytes: 8 rows x 32 terms x 7 planes per image
         xpk = -(-2 * tb_per_launch // 8) * LEVEL * n * ksteps * 1792
         alg = image + xpk + tb_per_launch * bp * ctw
-        mma = -(-bp // 8) * ksteps * 28 * LEVEL * n * -(-tb_per_launch // 4)      # m16n8k32 instructions per launch
+        mma = bp / 8 * ksteps * 28 * LEVEL * n * -(-tb_per_launch // 4)      # m16n8k32 instructions per launch
         tensor_peak = SM_COUNT * 4 * sm_mhz * 1e6 / 8                            # instructions / s
         return {"kernel": "bsgs", "variant": "k_bsgs_accumulate_packed (byte planes on the tensor cores)", "bound": "hbm",
                 "achieved": alg / t / 1e9, "peak": hbm_peak, "unit": "GB/s", "frac": alg / t / 1e9 / hbm_peak,
@@ -636,12 +638,12 @@ def run_ours(args):
     hbm_peak, peak_kind = peaks()
     sm_mhz = clocks.get("sm_mhz") or 1350.0
     tb_per_launch = int(ctx.counters()[5]) or tbs
-    fam_roofs = {"bsgs": bsgs_roofline(args, gin, nout, n, tb_per_launch, fam["bsgs"], hbm_peak, sm_mhz),
+    fam_roofs = {"bsgs": bsgs_roofline(args, gin, nout, n, tbs, tb_per_launch, 1, fam["bsgs"], hbm_peak, sm_mhz),
                  "ntt": ntt_roofline(p, n, fam["ntt"], passes_profiled, hbm_peak, sm_mhz)}
     if dominant in fam_roofs:
         # the dominant family was event-timed over the whole timed region: use those launches
         if dominant == "bsgs":
-            fam_roofs["bsgs"] = bsgs_roofline(args, gin, nout, n, tb_per_launch, (dom_ms, dom_records), hbm_peak, sm_mhz)
+            fam_roofs["bsgs"] = bsgs_roofline(args, gin, nout, n, tbs, tb_per_launch, args.steps, (dom_ms, dom_records), hbm_peak, sm_mhz)
         else:
             fam_roofs["ntt"] = ntt_roofline(p, n, (dom_ms, dom_records), passes, hbm_peak, sm_mhz)
         roof = dict(fam_roofs[dominant], timed="all launches of the timed steps")

@@ -639,6 +639,10 @@ static PackedPlan packed_plan(const fesc_ctx* ctx, const fesc_bsgs_desc* desc, u
     while (bstep > 1 && (bstep / 2) * n2 % 8 == 0) bstep /= 2;
     const double image = (double)bsgs_packed_bytes(N >> desc->diag_run_log2, level, nout * n2, terms);
     const double tensor = 0.5 * (double)bsgs_packed_bytes(N, level, nout * n2, terms);
+    // a CTA of the accumulate (one part, one tile) pays for its input fragments, the filling of its ring and its last recombination what 8
+    // images cost: 112 (b,p) pairs in 2 x 4 parts of tiles of 8 token blocks took 132 ms for the 14 outputs of
+    // in_proj and 16 token blocks, in 4 whole groups of 4 112
+    const double start = 8.0 * (double)bsgs_packed_bytes(N >> desc->diag_run_log2, level, 8, 32);
     PackedPlan best{};
     double best_cost = 0;
     for (uint32_t tbg = tbg_max;; tbg = tbg > 4 ? 4 : (tbg + 1) / 2) {
@@ -652,7 +656,7 @@ static PackedPlan packed_plan(const fesc_ctx* ctx, const fesc_bsgs_desc* desc, u
             p.rot_words = (size_t)sub * terms * ctw, p.acc_words = (size_t)tbg * p.nb_part * n2 * ctw;
             p.xpk_words = bsgs_packed_bytes(N, level, 2 * tbg, terms) / 8;
             p.total = (p.rot_words + p.acc_words + p.xpk_words + (ks_words > rs_words ? ks_words : rs_words)) * sizeof(u64);
-            const double cost = groups * (image + parts * 8.0 * (double)p.xpk_words + tiles * tensor);
+            const double cost = groups * (image + parts * (8.0 * (double)p.xpk_words + tiles * start) + tiles * tensor);
             const bool least = tbg == 1 && nb <= bstep;
             if ((p.total <= budget && (best.tbg == 0 || cost < best_cost)) || (best.tbg == 0 && least)) best = p, best_cost = cost;
             if (nb <= bstep) break;
