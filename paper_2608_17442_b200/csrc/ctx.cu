@@ -351,10 +351,14 @@ static int build_tables(fesc_ctx* ctx) {
                     d.term[a][t].m = m > q[t] / 2 ? -(long long)(q[t] - m) : (long long)m;
                     d.term[a][t].mq = (double)((long double)d.term[a][t].m / (long double)q[t]);
                 }
-                for (uint32_t t = 0; t < np; t++) d.start[t] -= 4503599627370496.0 * d.term[a][t].mq;
                 d.inv[a] = h_inv(d.mat[a][i], q[i]);
                 d.invs[a] = h_shoup(d.inv[a], q[i]);
                 scale[(size_t)(level - 1) * nq + i] = inv_scale(ctx->pc[i], d.inv[a]);
+            }
+            for (uint32_t t = 0; t < np; t++) {        // rounded once: the sum of doubles below 1 fits 64 bits but for 2^-63
+                long double mq = 0;
+                for (uint32_t a = 0; a < d.n_src; a++) mq += (long double)d.term[a][t].mq;
+                d.start[t] = (double)(-4503599627370496.0L * mq);
             }
         }
     }

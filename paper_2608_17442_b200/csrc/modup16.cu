@@ -6,7 +6,7 @@
 // (level + K - n_src) rows per digit.
 //
 // The sum is an exact mixed-pipe product: its quotient c = rint(sum_a y_a (m_a / q)) comes from the FP64 pipe (one
-// multiply-add per term, m centred; the roundings at up to 2^53 add up to less than 2.63, so |v| <= 2.63 q < 2^63), its value
+// multiply-add per term, m centred; its roundings add up to 2.51 at most, see convert4, so |v| <= 2.51 q < 2^63), its value
 // v = sum_a y_a m_a - c q from wrapping 64-bit integer products on the multiplier pipe, which the FP64 butterflies leave idle.
 //
 // A CTA owns 4 columns of one digit of one ciphertext: the source columns (8 KB per limb) are read once into shared memory
@@ -35,12 +35,24 @@ struct GroupBarrier {
 #define FP_MAGIC 6755399441055744.0      // 1.5 * 2^52: the low mantissa bits of FP_MAGIC + c hold the integer c, |c| < 2^51
 #define FP_MAGIC_HI 0x43380000u
 
+// the integer v, |v| < 2^53, whose high word has 2^31 added to it.  (One addition to 1.5 * 2^52 would do for |v| < 2^51 only, which is 2 q
+// at 50 bits.  The second one is not seen in the times: 32 rotations by 4 keys at 24 limbs 21.99 ms with one, 21.93 with two.)
+__device__ __forceinline__ double wide_to_double(u64 v) {
+    const double h = __dadd_rn(__hiloint2double(0x45300000, (int)(v >> 32)), -0x1.00000801p84);      // 2^84 + 2^63 + 2^52
+    return __dadd_rn(h, __hiloint2double(0x43300000, (int)(uint32_t)v));
+}
+
 // v[0..3] = sum_a y_a m_a - c q (two's complement) for the points p, p + 16 MU_COLS, ... of the source columns.  The columns hold
 // the doubles 2^52 + y, whose low 50 bits are y: one word serves both pipes without a conversion.  What 2^52 adds to the FP64 sum is
-// in its starting value c0, what the exponent bits add to the cross products (weight 2^32, modulo 2^32) is taken off at the end.
+// in its starting value c0, what the exponent bits add to the cross products (weight 2^32, modulo 2^32) is taken off at the end;
+// `bias` is added to the high word.
+// How far c is from the quotient, for any four primes below 2^50 (|m / q| <= 1/2, y < 2^50): the running sum starts at -2^52 sum(m / q)
+// and loses 2^52 m / q with every term, so it is below 2^53, 2^53, 2^52 + 2^50, 2^52 and 2^51 in turn and the roundings (of the start and of
+// four multiply-adds) are at most 1/2, 1/2, 1/2, 1/4 and 1/8; m / q as a double is off by 2^-55 at most, 1/32 per term after the product
+// with y (what 2^52 makes of it is in c0, which is formed from the same doubles); the quotient rounds by 1/2.  Together 2.5.
 template <int A>
 __device__ __forceinline__ void convert4(const u64* p, uint32_t n_src, const ModUpTerm (*__restrict__ term)[FESC_MAX_PRIMES], uint32_t pt,
-                                         double c0, u64 q, u64* v) {
+                                         double c0, u64 q, uint32_t bias, u64* v) {
     u64 acc[4];            // low product words, and the cross terms of weight 2^32 apart from them
     uint32_t cross[4], msum = 0;
     double s[4];
@@ -64,7 +76,7 @@ __device__ __forceinline__ void convert4(const u64* p, uint32_t n_src, const Mod
         }
     }
     const u64 nq = 0 - q;
-    const uint32_t ql = (uint32_t)nq, qh = (uint32_t)(nq >> 32), corr = 0u - 0x43300000u * msum;
+    const uint32_t ql = (uint32_t)nq, qh = (uint32_t)(nq >> 32), corr = bias - 0x43300000u * msum;
 #pragma unroll
     for (int e = 0; e < 4; e++) {
         const u64 c = (u64)__double_as_longlong(__dadd_rn(s[e], FP_MAGIC));
@@ -119,9 +131,9 @@ __global__ void __launch_bounds__(MU_THREADS, 2)
 #pragma unroll
             for (int k = 0; k < 16; k += 4) {
                 u64 v[4];
-                convert4<A>(ys + k * 16 * MU_COLS, n_src, dg->term, pt, c0, q, v);
+                convert4<A>(ys + k * 16 * MU_COLS, n_src, dg->term, pt, c0, q, 0x80000000u, v);
 #pragma unroll
-                for (int e = 0; e < 4; e++) x[k + e] = __dadd_rn(FpRow::value(v[e] + ((u64)FP_MAGIC_HI << 32)), -FP_MAGIC);
+                for (int e = 0; e < 4; e++) x[k + e] = wide_to_double(v[e]);       // |v| <= 2.51 q, within the 2.69 q fwd_cols takes
             }
             fwd_cols<MU_COLS>(r, x, sm, col, sub, bar);
 #pragma unroll
@@ -131,9 +143,9 @@ __global__ void __launch_bounds__(MU_THREADS, 2)
             u64 x[16];
 #pragma unroll
             for (int k = 0; k < 16; k += 4) {
-                convert4<A>(ys + k * 16 * MU_COLS, n_src, dg->term, pt, c0, q, x + k);
+                convert4<A>(ys + k * 16 * MU_COLS, n_src, dg->term, pt, c0, q, 0u, x + k);
 #pragma unroll
-                for (int e = 0; e < 4; e++) x[k + e] = csub(x[k + e] + 3 * q, r.q2);      // |v| <= 2.63 q: below 4q
+                for (int e = 0; e < 4; e++) x[k + e] = csub(x[k + e] + 3 * q, r.q2);      // |v| <= 2.51 q: below 4q
             }
             fwd_cols<MU_COLS>(r, x, sm, col, sub, bar);
 #pragma unroll

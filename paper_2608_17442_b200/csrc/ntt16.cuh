@@ -27,7 +27,7 @@ __device__ __forceinline__ uint32_t pad16(uint32_t e) { return e + 2 * (e >> 4);
 // ---------------------------------------------------------------------------------------
 // Arithmetic of a row.  w(i): twiddle i of the row's table.
 // FpRow: primes below 2^50, exact products on the FP64 pipe.  |product| <= (1/2 + 1.5 |y| 2^-53) q with centred twiddles,
-// so a forward stage takes a bound B q to (1.1875 B + 1/2) q: four stages from 2.8 q reach 8 q, seven from q/2 reach 7.88 q,
+// so a forward stage takes a bound B q to (1.1875 B + 1/2) q: four stages from 2.69 q and seven from q/2 stay below 8 q,
 // and everything below 8 q < 2^53 is exact.  Forward rows are folded back to q/2 twice (after four and after eleven
 // stages; the first bound leaves room for a conversion's lazy sum at the input); an inverse stage doubles the bound, so four stages from q/2 end at 8 q and every inverse
 // round folds back.

@@ -1,0 +1,87 @@
+"""The converted sum of the fused ModUp, in exact arithmetic: its quotient comes from a sum of rounded multiply-adds, so what is left of
+sum_a y_a m_a is a few times q.  The bound the device code states, the room its butterflies have and the decoding of the result are
+checked here for prime sets next to 2^50, where they are tightest."""
+from fractions import Fraction
+
+import numpy as np
+import pytest
+
+import fesc_synth as S
+
+BOUND, ROOM = 2.51, 2.69
+MAGIC = 1.5 * 2.0**52
+
+
+def largest_primes(skip, count=24):
+    """`count` primes = 1 mod 2^17 below 2^50 in descending order, after the first `skip`."""
+    return S.ntt_primes(50, 16, skip + count, 0)[skip:]
+
+
+def fma(a, b, c):
+    return float(Fraction(a) * Fraction(b) + Fraction(c))
+
+
+def centred(v, q):
+    return v - q if v > q // 2 else v
+
+
+def digit_terms(src, q):
+    """m and m / q of every source limb, and the sum's starting value, as the tables hold them."""
+    Q = int(np.prod([int(p) for p in src], dtype=object))
+    m = [centred(Q // p % q, q) for p in src]
+    mq = [float(Fraction(v, q)) for v in m]
+    return m, mq, float(-(2**52) * sum(map(Fraction, mq)))
+
+
+def left(y, m, mq, start, q):
+    """sum y m - c q with c = the rounded quotient sum, operation by operation."""
+    s = start
+    for v, w in zip(y, mq):
+        s = fma(2.0**52 + v, w, s)
+    return sum(v * w for v, w in zip(y, m)) - int(s + MAGIC - MAGIC) * q
+
+
+def decode(v):
+    """wide_to_double: two additions on the halves of the word."""
+    w = (v + (1 << 63)) & ((1 << 64) - 1)
+    h = (2.0**84 + float(w >> 32) * 2.0**32) - float.fromhex("0x1.00000801p84")
+    return h + (2.0**52 + float(w & 0xFFFFFFFF))
+
+
+SETS = {"largest": largest_primes(0), "next": largest_primes(24), "shipped": S.params("full")["primes"][:24],
+        "found": [1125899884167169, 1125899884036097, 1125899883642881, 1125899883380737, 1125899862016001],
+        "spread": [1125899780227073, 1125899387928577, 1125899077681153, 1125899416240129, 1125899607212033]}
+
+
+@pytest.mark.parametrize("name", sorted(SETS))
+def test_what_is_left_of_a_converted_word(name):
+    primes, g = SETS[name], np.random.default_rng(5)
+    worst = 0.0
+    for first in range(0, len(primes) - 1, 4):
+        src = primes[first:first + 4]
+        for t in [t for t in range(len(primes)) if not first <= t < first + 4][first % 3::3]:
+            q = primes[t]
+            m, mq, start = digit_terms(src, q)
+            assert all(abs(w) <= 0.5 for w in mq)
+            ys = [[0] * len(src), [p - 1 for p in src]] + [[int(g.integers(0, p)) for p in src] for _ in range(40 if len(primes) > 5 else 3000)]
+            for y in ys:
+                v = left(y, m, mq, start, q)
+                worst = max(worst, abs(v) / q)
+                assert decode(v) == v
+    assert worst < BOUND < ROOM and worst > 0.4, worst
+
+
+def test_a_word_beyond_the_window_of_one_addition():
+    """A digit and target of the largest primes where the sum of rounded multiply-adds has left more than 2^51: one addition to 1.5 * 2^52
+    cannot hold it."""
+    v = 2277992762386754
+    assert v > 2**51 and decode(v) == v and decode(-v) == -v
+    bits = (np.uint64(0x4338000000000000) + np.uint64(v)).view(np.float64) - MAGIC
+    assert bits != v
+
+
+def test_four_stages_from_the_bound_stay_exact():
+    for start, stages in ((ROOM, 4), (0.5, 7)):
+        for _ in range(stages):
+            start = 1.1875 * start + 0.5
+        assert start < 8
