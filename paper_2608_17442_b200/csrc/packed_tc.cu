@@ -7,16 +7,19 @@
 // images its tensor pipe was 0.62 busy and is several times narrower.
 //
 // One instruction multiplies byte plane k of the 128 outputs with all planes j of the inputs, and the sums of equal weight 256^(k+j)
-// belong together.  They land together without any arithmetic: the accumulator of planes 2m and 2m + 1 starts 2m column groups to the
-// right, and plane 2m + 1 takes its inputs from one group early, where a group of zeros lies.  The 13 sums of a product then sit in one row
-// of tensor memory: a thread owns an output, and no exchange between lanes is left.  64 columns per instruction.
+// belong together.  Those of planes 2m and 2m + 1 land together: both have the accumulator m of eight column groups, plane 2m + 1 takes its
+// inputs from one group early, where a group of zeros lies, so that column group y holds the weight 256^(2m + y).  A thread owns an output:
+// it adds the groups of equal weight of the four accumulators, and no exchange between lanes is left.  64 columns per instruction.
 //
-// 8 token blocks of 210 outputs x 189 terms at 24 limbs: 78 ms (167 ms in packed.cu).  Windows of all 14 column groups and one recombining
-// warp per scheduler 111; 16-byte stores and descriptors computed per product 90.  An instruction of 128 x 64 x 32 takes 48 cycles, what
-// reading its operands from shared memory takes, so the products alone need 46 ms; with issue, operand set-up and hand-over 62 without any recombination; the
-// scattered sectors of the outputs 35 by themselves.  Four accumulators instead of two: no change.
+// Two tcgen05.mma are ordered without a wait between them only when they have the same accumulator and the same shape.  Products that
+// depend on one another therefore share both, and the accumulators share no column; all of tensor memory is taken (2 x 4 x 64).
 //
-// CTA = 10 warps: 8 recombine (thread = output and half of the columns), one issues the products, one fetches the inputs.  Two accumulators (2 x 128 columns of
+// 8 token blocks of 210 outputs x 189 terms at 6 limbs: 20.1 ms (40.8 ms in packed.cu).  With accumulators that overlap, so that the 13 sums
+// are read without an addition, 19.6, but on an order that nothing promises; two accumulators of four planes in 80 columns 21.1, one of seven in 112
+// columns 22.8; the products in other orders 20.3.  An instruction of 128 x 64 x 32 takes 48 cycles, what reading its operands from shared memory
+// takes, so the products alone need 11.5 ms; outputs are scattered sectors.
+//
+// CTA = 10 warps: 8 recombine (thread = output and half of the columns), one issues the products, one fetches the inputs.  Two sets of accumulators (2 x 256 columns of
 // tensor memory) let the recombination of a coefficient run beside the products of the next.  Every wait is bounded (status word 4).
 #define FESC_DBG_FILE 15   // file id in the sites a debug build reports
 #include "ops.cuh"
@@ -28,8 +31,14 @@
 #define TC_OUT_WARPS 8
 #define TC_BUFFERS 4
 #define TC_A_BYTES(ksteps) (7u * (ksteps) * 16 * TC_CORE)
-#define TC_B_BYTES(ksteps) ((1u + 8 * (ksteps)) * TC_CORE)       // a group of zeros before and after every k-step's seven
-#define TC_ZERO_BYTES (6u * TC_CORE)       // the right operand that clears the columns which the first product does not reach
+#define TC_PLANES 2                        // byte planes of the outputs per accumulator
+#define TC_ACCS ((7 + TC_PLANES - 1) / TC_PLANES)
+#define TC_GROUPS ((7 + TC_PLANES) / 2 * 2)                      // 7 + TC_PLANES - 1 column groups of 8, made even (columns come in 16s)
+#define TC_GAP (TC_GROUPS - 7)                                   // groups of zeros before and after every k-step's seven planes
+#define TC_ACC_COLS (256 / TC_ACCS / 32 * 32)                    // columns of tensor memory from one accumulator to the next
+#define TC_B_BYTES(ksteps) ((TC_GAP + (7u + TC_GAP) * (ksteps)) * TC_CORE)
+static_assert(8 * TC_GROUPS <= TC_ACC_COLS && TC_ACCS * TC_ACC_COLS <= 256, "accumulators do not share columns");
+static_assert(TC_PLANES - 1 <= TC_GAP, "a window starts at most TC_PLANES - 1 groups early");
 
 // Shared-memory operand without swizzle, both core matrices of a row group side by side: K direction 128 bytes, row groups 256.  Only the
 // address, in the low word, differs between operands: one thread issues all products, and what it computes per product counts.
@@ -46,6 +55,9 @@ __device__ __forceinline__ void tc_commit(uint32_t bar) {
 __device__ __forceinline__ void tc_ld4(uint32_t* r, uint32_t addr) {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
 }
+
+// column groups of accumulator a that hold sums: its planes plus the seven of the inputs, less one
+__host__ __device__ constexpr int tc_groups(int a) { return (7 - TC_PLANES * a < TC_PLANES ? 7 - TC_PLANES * a : TC_PLANES) + 6; }
 
 template <bool FP, int KS>
 __global__ void __launch_bounds__(TC_THREADS, 1)
@@ -76,10 +88,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     }
 #endif
     const uint32_t a_base = (uint32_t)__cvta_generic_to_shared(smem), a_bytes = TC_A_BYTES(ksteps), b_bytes = TC_B_BYTES(ksteps);
-    const uint32_t b_base = a_base + a_bytes + TC_ZERO_BYTES, bar = (uint32_t)__cvta_generic_to_shared(bars);
+    const uint32_t b_base = a_base + a_bytes, bar = (uint32_t)__cvta_generic_to_shared(bars);
     const uint32_t b_full = bar, b_free = bar + 8 * TC_BUFFERS, d_full = bar + 16 * TC_BUFFERS, d_free = d_full + 16, drained = d_free + 16;
     if (warp == TC_OUT_WARPS) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 256;" ::"r"((uint32_t)__cvta_generic_to_shared(&tmem_base))
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"((uint32_t)__cvta_generic_to_shared(&tmem_base))
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
@@ -90,7 +102,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     // zeros around the inputs, and the left operand: [k-step][plane][16 row groups][k half][8 rows][16 bytes]
-    for (uint32_t i = tid; i < (TC_ZERO_BYTES + buffers * b_bytes) / 16; i += TC_THREADS) *reinterpret_cast<uint4*>(smem + a_bytes + 16 * i) = make_uint4(0, 0, 0, 0);
+    for (uint32_t i = tid; i < buffers * b_bytes / 16; i += TC_THREADS) *reinterpret_cast<uint4*>(smem + a_bytes + 16 * i) = make_uint4(0, 0, 0, 0);
     for (uint32_t i = warp; i < 16 * ksteps; i += TC_THREADS / 32) {
         const uint32_t rg = i / ksteps, ks = i - rg * ksteps, bt = mt * 16 + rg;
         uint32_t lo[7] = {}, hi[7] = {};
@@ -128,7 +140,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                 const uint8_t* src = xsrc + (size_t)(c >> 3) * ksteps * stage + (c & 7) * TC_FRAG;
                 mbar_expect_tx(b_full + 8 * buf, ksteps * TC_FRAG);
                 for (uint32_t k = 0; k < ksteps; k++)
-                    bulk_g2s(b_base + buf * b_bytes + (1 + 8 * k) * TC_CORE, src + k * stage, TC_FRAG, b_full + 8 * buf);
+                    bulk_g2s(b_base + buf * b_bytes + (TC_GAP + (7 + TC_GAP) * k) * TC_CORE, src + k * stage, TC_FRAG, b_full + 8 * buf);
             }
             // copies in flight when a wait ran out: the last `buffers` of them
             if (!ok)
@@ -136,9 +148,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         }
     } else if (warp == TC_OUT_WARPS) {                // issues the products
         if (lane == 0) {
-            // u8 x u8 -> s32, both operands K-major, 128 rows x 64 or 48 columns
-            const uint32_t idesc = (2u << 4) | (8u << 17) | (8u << 24), idesc48 = (2u << 4) | (6u << 17) | (8u << 24);
-            const uint32_t a0 = tc_desc(a_base), zero = tc_desc(a_base + a_bytes);
+            // u8 x u8 -> s32, both operands K-major, 128 rows
+            const uint32_t idesc = (2u << 4) | (TC_GROUPS << 17) | (8u << 24), a0 = tc_desc(a_base);
             for (uint32_t i = 0; i < coefs; i++) {
                 const uint32_t buf = i % buffers, use = i / buffers, db = i & 1, du = i >> 1;
                 if (mbar_wait_bounded(b_full + 8 * buf, use & 1) || (du && mbar_wait_bounded(d_free + 8 * db, (du - 1) & 1))) {
@@ -146,13 +157,13 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                     break;
                 }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t b0 = tc_desc(b_base + TC_CORE + buf * b_bytes), d = tmem + 128 * db;
-                tc_mma(d + 64, a0, zero, idesc48, false);
+                const uint32_t b0 = tc_desc(b_base + TC_GAP * TC_CORE + buf * b_bytes), d = tmem + 256 * db;
 #pragma unroll
                 for (uint32_t k = 0; k < KS; k++)
 #pragma unroll
                     for (uint32_t p = 0; p < 7; p++)
-                        tc_mma(d + 16 * (p >> 1), a0 + (k * 7 + p) * TC_CORE, b0 + (8 * k - (p & 1)) * (TC_CORE / 16), idesc, k || p);
+                        tc_mma(d + TC_ACC_COLS * (p / TC_PLANES), a0 + (k * 7 + p) * TC_CORE,
+                               b0 + ((7 + TC_GAP) * k - p % TC_PLANES) * (TC_CORE / 16), idesc, k || p % TC_PLANES);
                 tc_commit(b_free + 8 * buf);
                 tc_commit(d_full + 8 * db);
             }
@@ -177,20 +188,28 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                 if (ok && mbar_wait_bounded(d_full + 8 * db, du & 1)) ok = false;
                 ok = __all_sync(0xFFFFFFFFu, ok);
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                uint32_t s[13][4];
+                uint32_t s[TC_ACCS][TC_GROUPS][4];       // group y of accumulator a: weight 256^(TC_PLANES a + y)
 #pragma unroll
-                for (int x = 0; x < 13; x++) tc_ld4(s[x], tmem + 128 * db + 8 * x + 4 * half + ((32 * (warp & 3)) << 16));
+                for (int a = 0; a < TC_ACCS; a++)
+#pragma unroll
+                    for (int y = 0; y < TC_GROUPS; y++)
+                        if (y < tc_groups(a)) tc_ld4(s[a][y], tmem + 256 * db + TC_ACC_COLS * a + 8 * y + 4 * half + ((32 * (warp & 3)) << 16));
                 asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-                for (int x = 0; x < 13; x++)          // no use of a loaded word moves above the wait
-                    asm volatile("" : "+r"(s[x][0]), "+r"(s[x][1]), "+r"(s[x][2]), "+r"(s[x][3]));
+                for (int a = 0; a < TC_ACCS; a++)
+#pragma unroll
+                    for (int y = 0; y < TC_GROUPS; y++)      // no use of a loaded word moves above the wait
+                        if (y < tc_groups(a)) asm volatile("" : "+r"(s[a][y][0]), "+r"(s[a][y][1]), "+r"(s[a][y][2]), "+r"(s[a][y][3]));
                 asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                 if (lane == 0) mbar_arrive(d_free + 8 * db);
 #pragma unroll
                 for (int n = 0; n < 4; n++) {
-                    uint32_t v[13];
+                    uint32_t v[13] = {};
 #pragma unroll
-                    for (int x = 0; x < 13; x++) v[x] = s[x][n];
+                    for (int a = 0; a < TC_ACCS; a++)
+#pragma unroll
+                        for (int y = 0; y < TC_GROUPS; y++)
+                            if (y < tc_groups(a)) v[TC_PLANES * a + y] += s[a][y][n];
                     r[n][e] = imma_reduce<FP>(v, pc, c32, c64, c96);
                 }
             }
@@ -210,15 +229,16 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     __syncwarp();
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    if (warp == TC_OUT_WARPS) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 256;" ::"r"(tmem));
+    if (warp == TC_OUT_WARPS) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem));
 }
 
 static uint32_t tc_buffers(uint32_t ksteps) {
-    const uint32_t fit = (226u * 1024 - TC_ZERO_BYTES - TC_A_BYTES(ksteps)) / TC_B_BYTES(ksteps);
+    const uint32_t fit = (226u * 1024 - TC_A_BYTES(ksteps)) / TC_B_BYTES(ksteps);
     return fit < TC_BUFFERS ? fit : TC_BUFFERS;
 }
-// The left operand is worth its place in shared memory when at least 16 coefficients use it and a good part of its 128 rows is filled
-// (a tile of 128 costs what the other kernel takes for 5 tiles of 8); more than 192 terms do not fit.
+// The left operand is worth its place in shared memory when at least 16 coefficients use it and half of a tile's 128 rows are filled; more than
+// 192 terms do not fit.  8 token blocks x 189 terms at 6 limbs, here against packed.cu: 31 outputs 9.9 / 6.7 ms, 45 outputs 9.9 / 9.7, 64 outputs
+// 10.0 / 12.7, 130 outputs (two tiles) 19.9 / 26.0, 210 outputs 20.1 / 40.8; one token block the same to a scale of 1/2.
 bool bsgs_periodic_supported(uint32_t terms, uint32_t bp_count, uint32_t dshift) {
     return dshift >= 4 && (terms + 31) / 32 <= TC_MAX_KSTEPS && bp_count >= 64;
 }
@@ -226,7 +246,7 @@ int bsgs_accumulate_periodic(fesc_ctx* ctx, const uint8_t* xpk, const uint8_t* d
                              uint32_t bp_count, bool fp, uint32_t dshift, cudaStream_t st) {
     const uint32_t N = ctx->N, ksteps = (terms + 31) / 32, buffers = tc_buffers(ksteps);
     const dim3 grid((N >> dshift) * ((bp_count + 127) / 128) * ((tbs + 3) / 4), level);
-    size_t smem = TC_A_BYTES(ksteps) + TC_ZERO_BYTES + (size_t)buffers * TC_B_BYTES(ksteps);
+    size_t smem = TC_A_BYTES(ksteps) + (size_t)buffers * TC_B_BYTES(ksteps);
     if (smem < 120 * 1024) smem = 120 * 1024;          // one CTA per SM: no CTA waits for another one's tensor memory
 #define TC_LAUNCH(FP, KS)                                                                                                               \
     case KS: {                                                                                                                          \
