@@ -14,7 +14,9 @@
  *   - A ciphertext at level l (l active data limbs) is [2][l][N]: c0 then c1, EVAL form.
  *     A batch is [batch][2][l][N].  Limb i of a ciphertext uses data prime i.
  *   - Pointers named `d_*` or documented "device" are device pointers owned by the
- *     caller; the library never frees or reallocates them.  `stream` is a cudaStream_t
+ *     caller; the library never frees or reallocates them.  Arrays of words need the
+ *     alignment of a word (8 bytes; 16 are faster), a packed image (below) 16 bytes:
+ *     FESC_EINVAL otherwise.  `stream` is a cudaStream_t
  *     passed as void* (NULL = default stream).  Calls enqueue work on `stream` and return
  *     without synchronising, unless stated otherwise.
  *   - Scratch memory belongs to the context.  It grows (cudaFree + cudaMalloc, which

@@ -333,13 +333,29 @@ static inline int fesc_fail(fesc_ctx* ctx, int code, const std::string& msg) {
     return code;
 }
 
-// Two adjacent words of a buffer that the caller owns, which need not lie on a 16-byte boundary (`wide`: it does).
-__device__ __forceinline__ bool pair_aligned(const u64* p) { return ((size_t)p & 15) == 0; }
+// Two adjacent words of a buffer that the caller owns, which need not lie on a 16-byte boundary (`wide`: it does).  The wide accesses are
+// instructions of their own: written as accesses to a ulonglong2, unrolled loops over both kinds made misaligned accesses with
+// `wide` false.
+__host__ __device__ __forceinline__ bool pair_aligned(const u64* p) { return ((size_t)p & 15) == 0; }
 __device__ __forceinline__ ulonglong2 ld_pair(const u64* p, bool wide) {
-    return wide ? *reinterpret_cast<const ulonglong2*>(p) : make_ulonglong2(p[0], p[1]);
+    ulonglong2 v;
+    if (wide) asm volatile("ld.global.v2.b64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "l"(p));
+    else v.x = p[0], v.y = p[1];
+    return v;
 }
 __device__ __forceinline__ void st_pair(u64* p, ulonglong2 v, bool wide) {
-    if (wide) *reinterpret_cast<ulonglong2*>(p) = v;
+    if (wide) asm volatile("st.global.v2.b64 [%0], {%1, %2};" ::"l"(p), "l"(v.x), "l"(v.y) : "memory");
+    else p[0] = v.x, p[1] = v.y;
+}
+// the same where the host has chosen between two kernels
+template <bool WIDE>
+__device__ __forceinline__ ulonglong2 ld_pair(const u64* p) {
+    if constexpr (WIDE) return *reinterpret_cast<const ulonglong2*>(p);
+    else return make_ulonglong2(p[0], p[1]);
+}
+template <bool WIDE>
+__device__ __forceinline__ void st_pair(u64* p, ulonglong2 v) {
+    if constexpr (WIDE) *reinterpret_cast<ulonglong2*>(p) = v;
     else p[0] = v.x, p[1] = v.y;
 }
 
@@ -354,6 +370,12 @@ __device__ __forceinline__ uint32_t galois_src(uint32_t t, uint32_t log_n, u64 g
 __device__ __forceinline__ ulonglong2 galois_pair(const u64* __restrict__ in, uint32_t t, uint32_t log_n, u64 g, bool wide) {
     const uint32_t src = galois_src(t, log_n, g);
     const ulonglong2 v = ld_pair(in + (src & ~1u), wide);
+    return src & 1 ? make_ulonglong2(v.y, v.x) : v;
+}
+template <bool WIDE>
+__device__ __forceinline__ ulonglong2 galois_pair(const u64* __restrict__ in, uint32_t t, uint32_t log_n, u64 g) {
+    const uint32_t src = galois_src(t, log_n, g);
+    const ulonglong2 v = ld_pair<WIDE>(in + (src & ~1u));
     return src & 1 ? make_ulonglong2(v.y, v.x) : v;
 }
 

@@ -762,6 +762,7 @@ extern "C" int fesc_linear(fesc_ctx* ctx, const uint64_t* d_ct_in, const uint64_
         return fesc_fail(ctx, FESC_EINVAL, "linear: periodic diagonals (diag_run_log2) are a property of the packed image");
     if (packed && !bsgs_packed_supported(ctx, level, gin * n1, desc->diag_run_log2))
         return fesc_fail(ctx, FESC_EINVAL, "linear: packed diagonals need N a multiple of 8, primes below 2^56, at most 512 terms and runs that leave 8 words per limb");
+    if (packed && (size_t)d_diags & 15) return fesc_fail(ctx, FESC_EINVAL, "linear: a packed image must start on a 16-byte boundary");
     if (packed) {
         uint32_t bits = 0;
         for (uint32_t i = 0; i < level; i++) {

@@ -115,7 +115,8 @@ __global__ void __launch_bounds__(COL_THREADS, 1024 / COL_THREADS)
 }
 
 // grid = (128 / NTT_WARPS, rows); FIN: the last step of a division instead of the plain store (NttFinish), 2: of a product
-template <int A, int FIN>
+// WIDE: every buffer lies on a 16-byte boundary (a template and not a flag: tests of a flag at every access cost 0.4 % of a rotation)
+template <int A, int FIN, bool WIDE>
 __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
     ntt16_rows_fwd(u64* __restrict__ data, const void* __restrict__ tw, const PrimeConst* __restrict__ pcs, RowList list,
                    uint32_t y0, int out_double, NttFinish fin) {
@@ -144,13 +145,12 @@ __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
         fwd_rows(r, x, sm, blk, lane);
         const double q = r.q, qinv = r.qinv;
         if (!FIN) {
-            ulonglong2* o = reinterpret_cast<ulonglong2*>(p + 2 * lane);
 #pragma unroll
             for (int j = 0; j < 8; j++) {
                 const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(s + 72 * j);
                 const double a = FpRow::value(v.x), b = FpRow::value(v.y);
-                o[32 * j] = out_double ? make_ulonglong2(fp_handoff(a, q, qinv), fp_handoff(b, q, qinv))
-                                       : make_ulonglong2(fp_store(a, q, qinv), fp_store(b, q, qinv));
+                st_pair<WIDE>(p + 2 * lane + 64 * j, out_double ? make_ulonglong2(fp_handoff(a, q, qinv), fp_handoff(b, q, qinv))
+                                                                : make_ulonglong2(fp_store(a, q, qinv), fp_store(b, q, qinv)));
             }
             return;
         }
@@ -168,23 +168,22 @@ __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
         const u64* pt = FIN == 2 && fin.pt ? fin.pt + ct * fin.pt_stride + (size_t)i * N16 + blk * 512 + 2 * lane : nullptr;
         if (pt && !DBG_REGION(pt - 2 * lane, 512 * sizeof(u64))) return;
         const double mul = FIN == 2 ? fp_mod_u64(fin.mul, pcs[pi]) : 0.0;
-        const bool wide = pair_aligned(FIN == 2 ? acc : rot), wide_pt = FIN == 2 && pair_aligned(pt);
         ulonglong2 av[8];
 #pragma unroll
-        for (int j = 0; j < 8; j++) av[j] = ld_pair(acc + blk * 512 + 2 * lane + 64 * j, FIN == 1 || wide);
+        for (int j = 0; j < 8; j++) av[j] = ld_pair<WIDE>(acc + blk * 512 + 2 * lane + 64 * j);
 #pragma unroll
         for (int h = 0; h < 8; h += 4) {
             ulonglong2 w[4];
             if (FIN == 1 && rot) {
 #pragma unroll
-                for (int j = 0; j < 4; j++) w[j] = galois_pair(rot, blk * 512 + 2 * lane + 64 * (h + j), 16, rot_g, wide);
+                for (int j = 0; j < 4; j++) w[j] = galois_pair<WIDE>(rot, blk * 512 + 2 * lane + 64 * (h + j), 16, rot_g);
             }
 #pragma unroll
             for (int j = h; j < h + 4; j++) {
                 const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(s + 72 * j);
                 double a0 = fp_load(av[j].x, q), a1 = fp_load(av[j].y, q);
                 if (FIN == 2) {             // lazy products below 0.7 q
-                    const ulonglong2 w2 = pt ? ld_pair(pt + 64 * j, wide_pt) : make_ulonglong2(0, 0);
+                    const ulonglong2 w2 = pt ? ld_pair<WIDE>(pt + 64 * j) : make_ulonglong2(0, 0);
                     a0 = fp_modmul(a0, pt ? fp_from_u64(w2.x) : mul, q, qinv);
                     a1 = fp_modmul(a1, pt ? fp_from_u64(w2.y) : mul, q, qinv);
                 }
@@ -194,13 +193,13 @@ __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
                     s0 += fp_load(w[j - h].x, q);
                     s1 += fp_load(w[j - h].y, q);
                 }
-                ulonglong2* o = reinterpret_cast<ulonglong2*>(out + blk * 512 + 2 * lane + 64 * j);
+                u64* o = out + blk * 512 + 2 * lane + 64 * j;
                 if (FIN == 1 && add) {
-                    const ulonglong2 ov = *o;
+                    const ulonglong2 ov = ld_pair<WIDE>(o);
                     s0 += fp_load(ov.x, q);
                     s1 += fp_load(ov.y, q);
                 }
-                *o = make_ulonglong2(fp_store(s0, q, qinv), fp_store(s1, q, qinv));
+                st_pair<WIDE>(o, make_ulonglong2(fp_store(s0, q, qinv), fp_store(s1, q, qinv)));
             }
         }
     } else {
@@ -210,16 +209,15 @@ __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
 #pragma unroll
         for (int k = 0; k < 16; k++) x[k] = in[16 * k];
         fwd_rows(r, x, sm, blk, lane);
-        ulonglong2* o = reinterpret_cast<ulonglong2*>(p + 2 * lane);
 #pragma unroll
         for (int j = 0; j < 8; j++) {
             const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(s + 72 * j);
-            o[32 * j] = make_ulonglong2(r.canonical(v.x), r.canonical(v.y));
+            st_pair<WIDE>(p + 2 * lane + 64 * j, make_ulonglong2(r.canonical(v.x), r.canonical(v.y)));
         }
     }
 }
 
-template <int A, bool SRC>
+template <int A, bool SRC, bool WIDE>
 __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
     ntt16_rows_inv(u64* __restrict__ data, const void* __restrict__ tw, const PrimeConst* __restrict__ pcs, RowList list, uint32_t y0,
                    NttSource src) {
@@ -248,11 +246,10 @@ __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
             if (!DBG_REGION(pt - 2 * lane, 512 * sizeof(u64))) return;
         }
     }
-    const bool wide = SRC && pair_aligned(in), wide_pt = SRC && pair_aligned(pt);
     auto pair = [&](int j) {
-        if (!SRC) return *reinterpret_cast<const ulonglong2*>(in + 64 * j);
-        if (!g) return ld_pair(in + at + 64 * j, wide);
-        return galois_pair(in, at + 64 * j, 16, g, wide);
+        if (!SRC) return ld_pair<WIDE>(in + 64 * j);
+        if (!g) return ld_pair<WIDE>(in + at + 64 * j);
+        return galois_pair<WIDE>(in, at + 64 * j, 16, g);
     };
     u64* s = sm + 2 * lane + 2 * (lane >> 3);
     u64* o = p + 256 * (lane >> 4) + (lane & 15);
@@ -264,7 +261,7 @@ __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
             ulonglong2 v = pair(j);
             double a = fp_load(v.x, r.q), b = fp_load(v.y, r.q);
             if (SRC && (pt || src.mul)) {
-                const ulonglong2 w = pt ? ld_pair(pt + 64 * j, wide_pt) : make_ulonglong2(0, 0);
+                const ulonglong2 w = pt ? ld_pair<WIDE>(pt + 64 * j) : make_ulonglong2(0, 0);
                 a = r.fold(fp_modmul(a, pt ? fp_from_u64(w.x) : mul, r.q, r.qinv));
                 b = r.fold(fp_modmul(b, pt ? fp_from_u64(w.y) : mul, r.q, r.qinv));
             }
@@ -294,8 +291,15 @@ __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
     }
 }
 
-int ntt16_launch(fesc_ctx* ctx, u64* data, size_t rows, const RowMap& map, bool inverse, cudaStream_t st, bool in_double,
-                 bool out_double, const NttFinish& fin, uint64_t& launches, const InvScale* scale, bool skip_cols, const NttSource* source) {
+static bool all_aligned(const u64* data, const NttFinish& fin, const NttSource& src) {      // strides are multiples of N words
+    const u64* all[] = {data, fin.acc, fin.out, fin.rot_src, fin.pt, src.src, src.pt};
+    for (const u64* p : all)
+        if (!pair_aligned(p)) return false;
+    return true;
+}
+template <bool WIDE>
+static int launch_all(fesc_ctx* ctx, u64* data, size_t rows, const RowMap& map, bool inverse, cudaStream_t st, bool in_double, bool out_double,
+                      const NttFinish& fin, uint64_t& launches, const InvScale* scale, bool skip_cols, const NttSource* source) {
     RowList kind[2];
     for (RowList& l : kind) l.period = map.period, l.count = 0;
     for (uint32_t i = 0; i < map.period; i++) {
@@ -315,25 +319,31 @@ int ntt16_launch(fesc_ctx* ctx, u64* data, size_t rows, const RowMap& map, bool 
             const uint32_t y = (uint32_t)y0;
             if (f == ROW_FP) {
                 if (inverse) {
-                    launch(source ? ntt16_rows_inv<ROW_FP, true> : ntt16_rows_inv<ROW_FP, false>, gr, ROW_THREADS, 0, st, data, ctx->d_itwf, ctx->d_pc, l,
+                    launch(source ? ntt16_rows_inv<ROW_FP, true, WIDE> : ntt16_rows_inv<ROW_FP, false, WIDE>, gr, ROW_THREADS, 0, st, data, ctx->d_itwf, ctx->d_pc, l,
                            y, src);
                     launch(ntt16_cols_inv<ROW_FP>, gc, COL_THREADS, 0, st, data, ctx->d_itwf, ctx->d_pc, l, y, scale);
                 } else {
                     if (!skip_cols) launch(ntt16_cols_fwd<ROW_FP>, gc, COL_THREADS, 0, st, data, ctx->d_twf, ctx->d_pc, l, y, in_double, fin.centred, fin.centred_q);
-                    if (fin.pt || fin.mul) launch(ntt16_rows_fwd<ROW_FP, 2>, gr, ROW_THREADS, 0, st, data, ctx->d_twf, ctx->d_pc, l, y, out_double, fin);
-                    else if (fin.acc) launch(ntt16_rows_fwd<ROW_FP, 1>, gr, ROW_THREADS, 0, st, data, ctx->d_twf, ctx->d_pc, l, y, out_double, fin);
-                    else launch(ntt16_rows_fwd<ROW_FP, 0>, gr, ROW_THREADS, 0, st, data, ctx->d_twf, ctx->d_pc, l, y, out_double, fin);
+                    if (fin.pt || fin.mul) launch(ntt16_rows_fwd<ROW_FP, 2, WIDE>, gr, ROW_THREADS, 0, st, data, ctx->d_twf, ctx->d_pc, l, y, out_double, fin);
+                    else if (fin.acc) launch(ntt16_rows_fwd<ROW_FP, 1, WIDE>, gr, ROW_THREADS, 0, st, data, ctx->d_twf, ctx->d_pc, l, y, out_double, fin);
+                    else launch(ntt16_rows_fwd<ROW_FP, 0, WIDE>, gr, ROW_THREADS, 0, st, data, ctx->d_twf, ctx->d_pc, l, y, out_double, fin);
                 }
             } else if (inverse) {
-                launch(source ? ntt16_rows_inv<ROW_INT, true> : ntt16_rows_inv<ROW_INT, false>, gr, ROW_THREADS, 0, st, data, ctx->d_itw, ctx->d_pc, l, y,
+                launch(source ? ntt16_rows_inv<ROW_INT, true, WIDE> : ntt16_rows_inv<ROW_INT, false, WIDE>, gr, ROW_THREADS, 0, st, data, ctx->d_itw, ctx->d_pc, l, y,
                        src);
                 launch(ntt16_cols_inv<ROW_INT>, gc, COL_THREADS, 0, st, data, ctx->d_itw, ctx->d_pc, l, y, scale);
             } else {
                 if (!skip_cols) launch(ntt16_cols_fwd<ROW_INT>, gc, COL_THREADS, 0, st, data, ctx->d_tw, ctx->d_pc, l, y, 0, nullptr, 0.0);
-                launch(ntt16_rows_fwd<ROW_INT, 0>, gr, ROW_THREADS, 0, st, data, ctx->d_tw, ctx->d_pc, l, y, 0, fin);
+                launch(ntt16_rows_fwd<ROW_INT, 0, WIDE>, gr, ROW_THREADS, 0, st, data, ctx->d_tw, ctx->d_pc, l, y, 0, fin);
             }
             launches += skip_cols ? 1 : 2;
         }
     }
     return FESC_OK;
+}
+
+int ntt16_launch(fesc_ctx* ctx, u64* data, size_t rows, const RowMap& map, bool inverse, cudaStream_t st, bool in_double,
+                 bool out_double, const NttFinish& fin, uint64_t& launches, const InvScale* scale, bool skip_cols, const NttSource* source) {
+    const auto all = all_aligned(data, fin, source ? *source : NttSource()) ? launch_all<true> : launch_all<false>;
+    return all(ctx, data, rows, map, inverse, st, in_double, out_double, fin, launches, scale, skip_cols, source);
 }

@@ -334,6 +334,7 @@ extern "C" size_t fesc_linear_packed_bytes(const fesc_ctx* ctx, const fesc_bsgs_
 extern "C" int fesc_linear_pack_diags(fesc_ctx* ctx, const uint64_t* d_diags, const fesc_bsgs_desc* desc, uint32_t first,
                                       uint32_t count, void* d_packed, void* stream) {
     if (!ctx || !d_diags || !desc || !d_packed) return FESC_EINVAL;
+    if ((size_t)d_packed & 15) return fesc_fail(ctx, FESC_EINVAL, "pack_diags: the image must start on a 16-byte boundary");
     const uint32_t level = desc->n_limbs, terms = desc->in_blocks * desc->n1, bp_count = desc->out_blocks * desc->n2;
     if (!bsgs_packed_supported(ctx, level, terms, desc->diag_run_log2))
         return fesc_fail(ctx, FESC_EINVAL, "pack_diags: needs N a multiple of 8, primes below 2^56, at most 512 terms and runs that leave 8 words per limb");
