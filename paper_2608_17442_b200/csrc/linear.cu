@@ -623,6 +623,7 @@ static size_t linear_ks_words(const fesc_ctx* ctx, const fesc_bsgs_desc* desc, u
 // How a projection on packed diagonals is cut: token blocks per group and output blocks per part of a group.
 struct PackedPlan {
     uint32_t tbg, nb_part;
+    bool least;                                          // no cut needs less
     size_t rot_words, acc_words, xpk_words, total;      // words; bytes of scratch in all
 };
 // Every cut is charged what its accumulate launches have to read plus the tensor work of its tiles of 4 token blocks in the
@@ -631,7 +632,7 @@ struct PackedPlan {
 // tiles, full or not.  A group of 1 or 2 pays for a whole tile, which is why a projection whose rotated inputs are large (189
 // terms, 210 accumulators per token block) is worth 58 GiB of scratch: 1086 ms with groups of 1, 592 ms with groups of 4
 // (8 token blocks).
-static PackedPlan packed_plan(const fesc_ctx* ctx, const fesc_bsgs_desc* desc, uint32_t tbg_max, size_t budget) {
+static PackedPlan packed_plan(const fesc_ctx* ctx, const fesc_bsgs_desc* desc, size_t budget) {
     const uint32_t n2 = desc->n2, gin = desc->in_blocks, nout = desc->out_blocks, tbs = desc->token_blocks;
     const uint32_t level = desc->n_limbs, N = ctx->N, terms = gin * desc->n1;
     const size_t ctw = (size_t)2 * level * N;
@@ -645,7 +646,7 @@ static PackedPlan packed_plan(const fesc_ctx* ctx, const fesc_bsgs_desc* desc, u
     const double start = 8.0 * (double)bsgs_packed_bytes(N >> desc->diag_run_log2, level, 8, 32);
     PackedPlan best{};
     double best_cost = 0;
-    for (uint32_t tbg = tbg_max;; tbg = tbg > 4 ? 4 : (tbg + 1) / 2) {
+    for (uint32_t tbg = tbs >= 8 ? 8 : tbs;; tbg = tbg > 4 ? 4 : (tbg + 1) / 2) {
         const uint32_t tiles = (tbg + 3) / 4, sub = tbg < 4 ? tbg : 4, groups = (tbs + tbg - 1) / tbg;
         for (uint32_t nb = (nout + bstep - 1) / bstep * bstep;; nb -= bstep) {
             PackedPlan p;
@@ -657,8 +658,8 @@ static PackedPlan packed_plan(const fesc_ctx* ctx, const fesc_bsgs_desc* desc, u
             p.xpk_words = bsgs_packed_bytes(N, level, 2 * tbg, terms) / 8;
             p.total = (p.rot_words + p.acc_words + p.xpk_words + (ks_words > rs_words ? ks_words : rs_words)) * sizeof(u64);
             const double cost = groups * (image + parts * (8.0 * (double)p.xpk_words + tiles * start) + tiles * tensor);
-            const bool least = tbg == 1 && nb <= bstep;
-            if ((p.total <= budget && (best.tbg == 0 || cost < best_cost)) || (best.tbg == 0 && least)) best = p, best_cost = cost;
+            p.least = tbg == 1 && nb <= bstep;
+            if ((p.total <= budget && (best.tbg == 0 || cost < best_cost)) || (best.tbg == 0 && p.least)) best = p, best_cost = cost;
             if (nb <= bstep) break;
         }
         if (tbg == 1) return best;
@@ -677,15 +678,15 @@ static int linear_packed(fesc_ctx* ctx, const u64* in, const uint8_t* image, con
     const uint32_t tbs = desc->token_blocks, level = desc->n_limbs, N = ctx->N, terms = gin * n1;
     const size_t ctw = (size_t)2 * level * N, ctw_out = (size_t)2 * (level - 1) * N;
     u64* scratch = nullptr;
-    const size_t budget = packed_group_bytes(bsgs_packed_bytes(N >> desc->diag_run_log2, level, nout * n2, terms));
+    size_t budget = packed_group_bytes(bsgs_packed_bytes(N >> desc->diag_run_log2, level, nout * n2, terms));
     PackedPlan plan;
     int rc = FESC_ENOMEM;
-    for (uint32_t most = tbs >= 8 ? 8 : tbs;; most = most > 4 ? 4 : (most + 1) / 2) {     // smaller groups until the scratch can be had
-        plan = packed_plan(ctx, desc, most, budget);
-        most = plan.tbg;
+    for (;;) {          // smaller groups, then smaller parts, until the scratch can be had
+        plan = packed_plan(ctx, desc, budget);
         rc = ctx_scratch(ctx, plan.total, &scratch);
         if (rc == FESC_OK) break;
-        if (rc != FESC_ENOMEM || most == 1) return rc;
+        if (rc != FESC_ENOMEM || plan.least) return rc;
+        budget = plan.total - plan.total / 16;
     }
     const uint32_t tbg = plan.tbg, nb_part = plan.nb_part;
     u64 *rot = scratch, *acc = rot + plan.rot_words;

@@ -367,6 +367,32 @@ def test_linear_falls_back_to_smaller_groups_when_scratch_cannot_be_had(packed):
     assert np.array_equal(_run_gpu(ctx, cts, diags, n1, n2, dims, level, key_base=kb, packed=packed), want)
 
 
+def test_one_token_block_falls_back_to_smaller_parts_of_its_outputs():
+    """A projection of one token block cannot be cut into smaller groups; when its scratch cannot be reserved (failure injected on the
+    host) the output blocks are processed in parts, down to one that starts and ends on whole tiles of the image."""
+    import paper_2608_17442_b200 as fesc
+
+    T, C, n1, n2, tokens, d_in, d_out, level = 16, 32, 1, 32, 16, 32, 128, 3      # 1 token block, 4 output blocks
+    pair = ctx_pair("small")
+    ctx, orc, _ = pair
+    kb = 1000 + 41 * T
+    X, W, cts, diags, dims = _setup(pair, T, C, n1, n2, tokens, d_in, d_out, level, 2.0**40, wscale=10.0, key_base=kb)
+    want = orc.linear(cts, diags, dict(n1=n1, n2=n2), {q: kb + q for q in range(1, n1)}, {g: kb + 500 + g for g in range(1, n2)})
+    reserved = []
+    for failures in (0, 1, 2):
+        ctx.trim()
+        ctx.test_fail_allocs(failures)
+        assert np.array_equal(_run_gpu(ctx, cts, diags, n1, n2, dims, level, key_base=kb, packed=1), want)
+        reserved.append(ctx.counters()[3])
+    assert reserved[0] > reserved[1] > reserved[2]
+    ctx.trim()
+    ctx.test_fail_allocs(4)                    # every cut of the four outputs
+    with pytest.raises(fesc.FescError) as e:
+        _run_gpu(ctx, cts, diags, n1, n2, dims, level, key_base=kb, packed=1)
+    assert e.value.code == fesc.ENOMEM
+    ctx.test_fail_allocs(0)
+
+
 @pytest.mark.parametrize("gin", [7, 9, 11])
 def test_linear_packed_input_fragments_of_4_to_6_ksteps(gin):
     """Sums of 112, 144 and 176 terms: the packed accumulate keeps the input fragments of 4, 5 and 6 k-steps in shared
