@@ -267,8 +267,12 @@ struct Exec {
             rc = fesc_fail(ctx, FESC_ELEVEL, "scan_contract: level schedule violated");
             return;
         }
-        const uint64_t* tab = kind ? cs->adj_p : cs->adj_s;
-        product_rescale(in, dst + 1, nullptr, 0, tab[(size_t)in.level * (g.l0 + 1) + dst], out);
+        const uint64_t k = (kind ? cs->adj_p : cs->adj_s)[(size_t)in.level * (g.l0 + 1) + dst];
+        if (k) return product_rescale(in, dst + 1, nullptr, 0, k, out);
+        // a factor of zero (0 stands for none there): the rescale of zeros
+        if (dry) return;
+        const cudaError_t e = cudaMemset2DAsync(out.p, out.stride * sizeof(u64), 0, ctw(dst) * sizeof(u64), out.count, st);
+        if (e != cudaSuccess) rc = fesc_fail(ctx, FESC_ECUDA, cudaGetErrorString(e));
     }
     static bool equally_spaced(const std::vector<uint32_t>& pos, uint32_t& step) {
         step = pos.size() > 1 ? pos[1] - pos[0] : 1;

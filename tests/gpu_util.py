@@ -48,9 +48,10 @@ def random_ct(orc, seed: int, stream: int, level: int, batch: int) -> np.ndarray
     return out
 
 
-def run_scan_parity(name, hoist=0, network="bk", group=0, **kw):
+def run_scan_parity(name, hoist=0, network="bk", group=0, adj_zero=(), **kw):
     """fesc_scan_contract against ScanEvaluator.run on the named parameter set and shape: asserts that every output
-    residue is equal and returns the largest deviation of the decrypted result from the float64 recurrence."""
+    residue is equal and returns the largest deviation of the decrypted result from the float64 recurrence.  adj_zero: (source,
+    target) level pairs whose factors are set to zero."""
     import torch
     import fesc_synth as S
     import paper_2608_17442_b200 as fesc
@@ -63,6 +64,8 @@ def run_scan_parity(name, hoist=0, network="bk", group=0, **kw):
     l0 = p["n_q"]
     x, a, B, C = S.scan_inputs(p["seed"] + sh.L, sh.L, sh.H, sh.P, 1, sh.d_s)
     c = ScanConsts(orc, sh, l0, p["log_scale"], network, group)
+    for pair in adj_zero:
+        c.adj_s[pair] = c.adj_p[pair] = 0
     add_scan_keys(orc, sh, hoist=bool(hoist), group=group)
     for r in sh.rotation_amounts(bool(hoist), group) + [CONJ]:
         ctx.add_galois_key(r, key_id_for(sh, r))

@@ -28,6 +28,13 @@ def test_scan_two_digit_offsets_and_odd_chunk_count(hoist):
     assert _run("scan_small", hoist, L=64, H=3, P=4, d_s=4, B_blk=32) < 2.0**-22
 
 
+def test_scan_factors_of_zero_between_adjacent_levels():
+    """The tables that bring ciphertexts down are the caller's: a factor of zero gives zeros, also one level down, where no limb is
+    dropped before the product."""
+    every = [(a, a - 1) for a in range(2, 11)]
+    _run("scan_toy", 0, adj_zero=every, L=4, H=2, P=4, d_s=2, B_blk=4)
+
+
 @pytest.mark.parametrize("network", ["ks", "sk"])
 def test_scan_other_prefix_networks(network):
     """Kogge-Stone and Sklansky networks: bit-exact against the oracle's network of the same name (toy shape; carries
