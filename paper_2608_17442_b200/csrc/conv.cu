@@ -14,6 +14,7 @@ extern "C" int fesc_conv(fesc_ctx* ctx, const uint64_t* d_ct_in, const uint64_t*
     const uint32_t d = desc->d_conv, T = desc->T, blocks = desc->blocks, tbs = desc->token_blocks, level = desc->n_limbs;
     const uint32_t N = ctx->N;
     if (!d || d > 8 || !blocks || !tbs) return fesc_fail(ctx, FESC_EINVAL, "conv: empty dimension or more than 8 taps");
+    if (blocks > 65535) return fesc_fail(ctx, FESC_EINVAL, "conv: too many channel blocks");
     if (!T || (N / 2) % T || d > T) return fesc_fail(ctx, FESC_EINVAL, "conv: T must divide the slot count and exceed the taps");
     if (level < 2 || level > ctx->n_q) return fesc_fail(ctx, FESC_ELEVEL, "conv: level out of range");
     const uint32_t taps = d - 1;

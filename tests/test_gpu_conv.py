@@ -78,3 +78,14 @@ def test_conv_missing_key_is_reported():
     with pytest.raises(fesc.FescError) as e:
         ctx.conv(z, z, z, fesc.ConvDesc(4, 32, 1, 2, 3, 7900000), z)
     assert e.value.code == fesc.ENOKEY
+
+
+def test_conv_refuses_more_channel_blocks_than_a_launch_takes():
+    import torch
+    import paper_2608_17442_b200 as fesc
+
+    ctx, orc, _ = ctx_pair("toy")
+    word = torch.zeros((1,), dtype=torch.int64, device="cuda")          # refused before any buffer is touched
+    with pytest.raises(fesc.FescError) as e:
+        ctx.conv(word, word, word, fesc.ConvDesc(1, orc.N // 2, 65536, 1, 2, 1000), word)
+    assert e.value.code == fesc.EINVAL
