@@ -1312,22 +1312,20 @@ int giant_sum_deferred_internal(fesc_ctx* ctx, u64* acc, uint32_t n_terms, size_
     KsScratch ws = ks_scratch_carve(ctx, scratch, level, cut);
     const size_t stride = (size_t)n_terms * ct_words;
     const size_t ext_words = (size_t)((level + ctx->alpha - 1) / ctx->alpha) * (level + ctx->n_p) * ctx->N;
-    for (uint32_t p0 = 1; p0 < n_terms; p0 += 32) {
-        GiantSet gs;
-        gs.n = n_terms - p0 < 32 ? n_terms - p0 : 32;
-        for (uint32_t p = 0; p < gs.n; p++) gs.g[p] = ctx->keys[key_base + p0 + p].g;
-        prof_begin(ctx, PF_AUTOM, st);
-        // the terms of this launch follow the ones before: shift the base so that term 0 stays the sum
-        if (p0 == 1)
-            launch(k_giant_c0, dim3((ctx->N + 255) / 256, level, batch), 256, 0, st, acc, stride, ct_words, ctx->log_n, gs, ctx->d_pc);
-        else
-            for (uint32_t p = 0; p < gs.n; p++) {
-                GiantSet one;
-                one.n = 1, one.g[0] = gs.g[p];
-                launch(k_giant_c0, dim3((ctx->N + 255) / 256, level, batch), 256, 0, st, acc, stride, (size_t)(p0 + p) * ct_words, ctx->log_n, one, ctx->d_pc);
-            }
-        prof_end(ctx, PF_AUTOM, st);
+    prof_begin(ctx, PF_AUTOM, st);
+    uint64_t launches = 0;
+    for (uint32_t b0 = 0; b0 < batch; b0 += 65535) {              // gridDim.z
+        const dim3 grid((ctx->N + 255) / 256, level, batch - b0 < 65535 ? batch - b0 : 65535);
+        // up to 32 terms at a time; beyond the first 32 one by one (a launch finds its terms ct_words apart, term 0 being the sum)
+        for (uint32_t p0 = 1, n; p0 < n_terms; p0 += n) {
+            GiantSet gs;
+            gs.n = n = p0 > 1 ? 1 : n_terms - p0 < 32 ? n_terms - p0 : 32;
+            for (uint32_t p = 0; p < n; p++) gs.g[p] = ctx->keys[key_base + p0 + p].g;
+            launch(k_giant_c0, grid, 256, 0, st, acc + (size_t)b0 * stride, stride, p0 * ct_words, ctx->log_n, gs, ctx->d_pc);
+            launches++;
+        }
     }
+    prof_end(ctx, PF_AUTOM, st, launches);
     for (uint32_t b0 = 0; b0 < batch; b0 += cut.nb) {
         const uint32_t nb = batch - b0 < cut.nb ? batch - b0 : cut.nb;
         u64* base = acc + (size_t)b0 * stride;

@@ -393,6 +393,47 @@ def test_one_token_block_falls_back_to_smaller_parts_of_its_outputs():
     ctx.test_fail_allocs(0)
 
 
+def test_deferred_giant_steps_over_more_outputs_than_a_launch_covers():
+    """65 536 outputs in one group and more giant steps than one pass over the first polynomials takes: residues equal those of the
+    same projection over fewer token blocks."""
+    import torch
+    import paper_2608_17442_b200 as fesc
+
+    pair = ctx_pair("toy")
+    ctx, orc, p = pair
+    level, N, n2, tbs, kb = 2, orc.N, 3, 16384, 60000
+    for g in range(1, n2):
+        add_key(pair, g, kb + 500 + g)
+    few = np.stack([S.uniform_residues_np(p["seed"], 5000 + i, orc.q[:level], N) for i in range(4 * 2)]).reshape(4, 1, 2, level, N)
+    w = to_dev(np.stack([S.uniform_residues_np(p["seed"], 5100 + i, orc.q[:level], N) for i in range(4 * n2)]).reshape(4, n2, 1, 1, level, N))
+    out = []
+    for ct in (to_dev(few), to_dev(few).repeat(tbs // 4, 1, 1, 1, 1)):
+        y = torch.empty((ct.shape[0], 4, 2, level - 1, N), dtype=torch.int64, device="cuda")
+        ctx.linear(ct, w, fesc.BsgsDesc(1, n2, 1, 4, ct.shape[0], level, kb, kb + 500, 1, 1, 0), y)
+        ctx.sync()
+        out.append(y)
+    assert ctx.counters()[5] == tbs and bool(out[0].any())
+    assert torch.equal(out[1].view(tbs // 4, 4, 4, 2, level - 1, N), out[0].expand(tbs // 4, -1, -1, -1, -1, -1))
+
+
+def test_deferred_giant_steps_beyond_one_pass():
+    """40 giant amounts: the first polynomials are summed in several launches; residues equal the oracle's."""
+    import torch
+    import paper_2608_17442_b200 as fesc
+
+    pair = ctx_pair("small")
+    ctx, orc, p = pair
+    level, N, n2, kb = 3, orc.N, 41, 61000
+    for g in range(1, n2):
+        add_key(pair, g, kb + 500 + g)
+    cts = np.stack([S.uniform_residues_np(p["seed"], 5200 + i, orc.q[:level], N) for i in range(2)]).reshape(1, 1, 2, level, N)
+    w = np.stack([S.uniform_residues_np(p["seed"], 5300 + i, orc.q[:level], N) for i in range(n2)]).reshape(1, n2, 1, 1, level, N)
+    out = torch.empty((1, 1, 2, level - 1, N), dtype=torch.int64, device="cuda")
+    ctx.linear(to_dev(cts), to_dev(w), fesc.BsgsDesc(1, n2, 1, 1, 1, level, kb, kb + 500, 0, 1, 0), out)
+    ctx.sync()
+    assert np.array_equal(to_host(out), orc.linear(cts, w, dict(n1=1, n2=n2), {}, {g: kb + 500 + g for g in range(1, n2)}, defer=True))
+
+
 @pytest.mark.parametrize("gin", [7, 9, 11])
 def test_linear_packed_input_fragments_of_4_to_6_ksteps(gin):
     """Sums of 112, 144 and 176 terms: the packed accumulate keeps the input fragments of 4, 5 and 6 k-steps in shared
