@@ -1616,6 +1616,13 @@ int rescale_internal(fesc_ctx* ctx, const u64* in, size_t in_stride, u64* out, u
         prof_end(ctx, PF_RESCALE, st);
         m.period = level - 1;
         for (uint32_t i = 0; i + 1 < level; i++) m.prime[i] = (uint8_t)i;
+        if (rescale_fused(ctx, level - 1)) {      // the dropped prime alone is 2^50 or more: the last pass still finishes the division
+            NttFinish fin;
+            fin.acc = ib, fin.acc_stride = in_stride, fin.out = ob, fin.out_stride = out_stride, fin.cinv = tab->qinvd;
+            fin.level = level - 1, fin.acc_rows = level, fin.add_mask = 0;
+            if ((rc = ntt_launch(ctx, ob, (size_t)nb * 2 * (level - 1), m, false, st, false, false, &fin)) != FESC_OK) return rc;
+            continue;
+        }
         if ((rc = ntt_launch(ctx, ob, (size_t)nb * 2 * (level - 1), m, false, st)) != FESC_OK) return rc;
         prof_begin(ctx, PF_RESCALE, st);
         launch(k_rescale_finish, dim3(gx, level - 1, nb * 2), 256, 0, st, ib, in_stride, ob, out_stride, tab, ctx->d_pc, N,

@@ -443,6 +443,25 @@ def test_inner_product_staged_by_bulk_copies(monkeypatch):
             assert np.array_equal(sgot[b], orc.rotate_sum_hoisted(ct[b], [81, 82]))
 
 
+def test_rescale_drops_a_prime_of_52_bits_onto_primes_of_50():
+    """Only the dropped prime is above the FP64 range: the last pass of the transform finishes the division (no kernel after it)."""
+    import torch
+    import paper_2608_17442_b200 as fesc
+    from oracle.ckks import Oracle
+
+    args = (16, S.ntt_primes(50, 16, 2, 0) + S.ntt_primes(52, 16, 1, 0) + S.ntt_primes(60, 16, 1, 0), 3, 1, 3, 99)
+    ctx, orc = fesc.Context(*args), Oracle(*args)
+    ct = random_ct(orc, 31, 0, 3, 2)
+    ct[0, :, 2] = orc.q[2] - 1
+    out = torch.empty((2, 2, 2, orc.N), dtype=torch.int64, device="cuda")
+    before = ctx.counters()[4]
+    ctx.rescale(to_dev(ct), out, 2, 3)
+    assert ctx.counters()[4] - before == 6
+    got = to_host(out)
+    for b in range(2):
+        assert np.array_equal(got[b], orc.rescale(ct[b]))
+
+
 def test_integer_paths_with_primes_above_50_bits():
     """Primes of 52 and 55 bits take the integer kernels (wide-lazy transform at N = 2^16, 128-bit lazy
     accumulation in ModUp / inner product / ModDown); same bit-exact bar."""
