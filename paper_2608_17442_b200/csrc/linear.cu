@@ -604,12 +604,27 @@ static size_t bsgs_group_bytes() {
 }
 // Packed operands: the budget is what an image of in_proj's size (110 GiB) leaves on a device of 178 GiB, 37 GiB, and
 // grows by what a smaller image leaves free, up to 64 GiB.
+#define PACKED_LEAST ((size_t)37 << 30)
 static size_t packed_group_bytes(size_t image_bytes) {
     const char* e = getenv("FESC_BSGS_GROUP_GIB");
     if (e && atoi(e) > 0) return (size_t)atoi(e) << 30;
-    const size_t full = (size_t)111 << 30, least = (size_t)37 << 30, most = (size_t)64 << 30;
-    const size_t b = image_bytes < full ? least + (full - image_bytes) : least;
+    const size_t full = (size_t)111 << 30, most = (size_t)64 << 30;
+    const size_t b = image_bytes < full ? PACKED_LEAST + (full - image_bytes) : PACKED_LEAST;
     return b < most ? b : most;
+}
+// What lies above 37 GiB may take half of what the device has free beyond them (the arena is given back before it grows), so that
+// the other half stays the caller's.  Nothing is asked of the device when the arena holds the plan already, or during a capture.
+static size_t packed_spare_bytes(const fesc_ctx* ctx, cudaStream_t st) {
+    const char* e = getenv("FESC_BSGS_GROUP_GIB");
+    if (e && atoi(e) > 0) return SIZE_MAX;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    size_t free = 0, total = 0;
+    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone || cudaMemGetInfo(&free, &total) != cudaSuccess) {
+        cudaGetLastError();
+        return PACKED_LEAST;
+    }
+    const size_t have = free + ctx->scratch_bytes;
+    return have > PACKED_LEAST ? PACKED_LEAST + (have - PACKED_LEAST) / 2 : PACKED_LEAST;
 }
 
 // key-switch scratch of a projection: baby rotations of `inputs` ciphertexts, giant steps of `outputs`
@@ -683,6 +698,10 @@ static int linear_packed(fesc_ctx* ctx, const u64* in, const uint8_t* image, con
     int rc = FESC_ENOMEM;
     for (;;) {          // smaller groups, then smaller parts, until the scratch can be had
         plan = packed_plan(ctx, desc, budget);
+        if (plan.total > PACKED_LEAST && plan.total > ctx->scratch_bytes) {
+            const size_t spare = packed_spare_bytes(ctx, st);
+            if (plan.total > spare) plan = packed_plan(ctx, desc, spare);
+        }
         rc = ctx_scratch(ctx, plan.total, &scratch);
         if (rc == FESC_OK) break;
         if (rc != FESC_ENOMEM || plan.least) return rc;

@@ -434,6 +434,40 @@ def test_deferred_giant_steps_beyond_one_pass():
     assert np.array_equal(to_host(out), orc.linear(cts, w, dict(n1=1, n2=n2), {}, {g: kb + 500 + g for g in range(1, n2)}, defer=True))
 
 
+def test_scratch_beyond_the_usual_amount_leaves_the_caller_half_of_what_is_free():
+    """A projection that is cut best with more than 37 GiB of scratch takes no more of a nearly full device than 37 GiB and half of the
+    rest; the cut does not change the result."""
+    import torch
+    import paper_2608_17442_b200 as fesc
+
+    ctx, orc, p = ctx_pair("full")
+    level, N, gin, nout, tbs, GiB = 24, orc.N, 64, 192, 8, 2**30
+    free = torch.cuda.mem_get_info()[0]
+    if free < 130 * GiB:
+        pytest.skip("needs most of a 180 GB device")
+    desc = fesc.BsgsDesc(1, 1, gin, nout, tbs, level, 0, 0, 0, 0, 1, 7)
+    g = torch.Generator(device="cuda").manual_seed(3)
+    rand = lambda *shape: torch.randint(0, 1 << 49, shape, generator=g, dtype=torch.int64, device="cuda")
+    x, image = rand(tbs, gin, 2, level, N), torch.empty((ctx.linear_packed_bytes(desc),), dtype=torch.uint8, device="cuda")
+    ctx.linear_pack_diags(rand(nout, gin, 1, level, N >> 7), desc, 0, nout, image)
+    out, scratch = torch.empty((tbs, nout, 2, level - 1, N), dtype=torch.int64, device="cuda"), []
+    for spare in (None, 43):
+        ctx.trim()
+        torch.cuda.empty_cache()
+        hog = torch.empty((torch.cuda.mem_get_info()[0] - spare * GiB,), dtype=torch.uint8, device="cuda") if spare else None
+        ctx.linear(x, image, desc, out)
+        ctx.sync()
+        scratch.append(ctx.counters()[3])
+        del hog
+        if spare is None:
+            want = out[:, ::37, :, ::5].clone()
+    assert scratch[0] > 42 * GiB and scratch[1] <= 40 * GiB + 2**20
+    assert torch.equal(out[:, ::37, :, ::5], want)
+    ctx.trim()
+    del x, image, out, want
+    torch.cuda.empty_cache()
+
+
 @pytest.mark.parametrize("gin", [7, 9, 11])
 def test_linear_packed_input_fragments_of_4_to_6_ksteps(gin):
     """Sums of 112, 144 and 176 terms: the packed accumulate keeps the input fragments of 4, 5 and 6 k-steps in shared
