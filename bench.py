@@ -207,7 +207,8 @@ MAC_MIXED_CYCLES = 8              # mixed-pipe multiply-accumulate: multiplier-p
 # read once per launch and every output byte written once, traffic grows in proportion to the algorithmic bytes.
 BSGS_TRAFFIC_RATIO = {"packed": 1.000, "residues": 1.001}     # measured DRAM bytes / algorithmic bytes (small case)
 PACKED_BYTES_PER_WORD = 7                                     # a residue below 2^56 as byte planes
-NTT_DISPATCH_CYCLES = 27.1        # dispatch-port cycles per warp-butterfly of the FP64 transforms: 9.5 x 2 + 8.1 (ncu opcode mix)
+NTT_DISPATCH_CYCLES = 17.0        # dispatch-port cycles per warp-butterfly of the FP64 transforms, arithmetic alone: two multiply-adds of
+                                  # three registers (3 each), two multiplications and three additions (2 each), one rounding (1)
 NTT_TRAFFIC_RATIO = 1.0           # the transforms read and write every word of both passes through DRAM once
 INT_LIMB_SHARE = 32.0 / 224.0     # transforms on the 60-bit special primes per key switch (integer path)
 
@@ -535,10 +536,8 @@ def ntt_roofline(p, n, timed, passes, hbm_peak, sm_mhz):
     alu_peak = 1.0 / ((1.0 - INT_LIMB_SHARE) / peak_fp + INT_LIMB_SHARE / peak_int)
     ach = bfly / (ms * 1e-3) / 1e12
     moved = limb_ntts * 2 * 2 * n * 8           # two passes, each reads and writes the limb
-    # What the dispatch port allows with the measured instruction mix of the FP64 path (ncu opcode counts: 17.6 warp
-    # instructions per warp-butterfly, 9.5 of them FP64, which hold the port for two cycles): 27.1 cycles per
-    # warp-butterfly on each of the 4 schedulers of an SM.  The kernels also have to load, exchange and store, so this,
-    # not the FP64-pipe figure above, is the ceiling they can approach.
+    # What the dispatch port allows for the arithmetic of the FP64 path alone (loads, exchanges and stores take dispatch
+    # cycles of their own, so the kernels cannot reach it).
     issue_peak = SM_COUNT * 4 * 32 * sm_mhz * 1e6 / NTT_DISPATCH_CYCLES / 1e12
     return {"kernel": "ntt", "variant": "ntt16_cols + ntt16_rows (two passes per limb transform)", "bound": "alu",
             "achieved": ach, "peak": alu_peak, "unit": "T butterflies/s (FP64 pipe for 50-bit primes, integer pipe for 60-bit)",

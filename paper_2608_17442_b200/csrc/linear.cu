@@ -438,7 +438,7 @@ __global__ void __launch_bounds__(MIX_THREADS, (TT * PT >= 12 ? 256 / MIX_THREAD
         }
 }
 
-// Tensor-core accumulate for primes below 2^56 (at most 256 terms).  For one coefficient of one limb the sums
+// Tensor-core accumulate for primes of 50 to 55 bits (at most 256 terms).  For one coefficient of one limb the sums
 //   S[tb,p][bp] = sum_t x_t[tb,p] * w_t[bp]
 // are a small dense integer matrix product over the terms.  Every residue is cut into 7 bytes; the byte planes
 // form u8 matrices and  S = sum_{k,j} 256^(k+j) D[k][j],  D[k][j] = sum_t w_t.byte(k) * x_t.byte(j),  where each
@@ -453,8 +453,7 @@ __global__ void __launch_bounds__(MIX_THREADS, (TT * PT >= 12 ? 256 / MIX_THREAD
 // launch.  Fragments are built in registers from the raw 64-bit words: four words of consecutive terms are
 // byte-transposed with 15 byte permutes into the seven 4-term registers the instruction expects.
 // Recombination: E_d = sum_{k+j=d} D[k][j] (13 values below 2^27), groups of four E_d are packed exactly into
-// doubles T_m < 2^52, and S mod q = T_0 + T_1 2^32 + T_2 2^64 + T_3 2^96 mod q with exact FP64 products (primes below
-// 2^50) or as a 128-bit integer followed by the usual reduction (primes of 50..55 bits).
+// T_m < 2^52, and S = T_0 + T_1 2^32 + T_2 2^64 + T_3 2^96 is a 128-bit integer followed by the usual reduction.
 #define IM_CW 8
 #define IM_ROWP 9                      // words per (row, 8 coefficients): one word of padding
 #define IM_BPP (32 * IM_ROWP + 1)      // words between the (b,p) blocks of a stage (= 1 mod 16: conflict-free fragment loads)
@@ -465,7 +464,7 @@ __device__ __forceinline__ void cp_async8z(uint32_t smem_dst, const void* gmem_s
     asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(smem_dst), "l"(gmem_src), "r"(n) : "memory");
 }
 
-template <bool FP, int IM_STAGES>
+template <int IM_STAGES>
 __global__ void __launch_bounds__(32 * IM_CW, 1) k_bsgs_accumulate_imma(
     const u64* __restrict__ rot, const u64* __restrict__ diags, u64* __restrict__ acc,
     const PrimeConst* __restrict__ pcs, uint32_t N, uint32_t level, uint32_t tbs, uint32_t terms, uint32_t bp_count,
@@ -522,14 +521,6 @@ __global__ void __launch_bounds__(32 * IM_CW, 1) k_bsgs_accumulate_imma(
         if (s < total) issue();
         cp_async_commit();
     }
-    // constants of the recombination
-    const double q = pc.qd, qinv = pc.qinvd;
-    double c32 = 0, c64 = 0, c96 = 0;
-    if (FP) {
-        c32 = fp_reduce(4294967296.0, q, qinv);
-        c64 = fp_modmul(c32, c32, q, qinv);
-        c96 = fp_modmul(c64, c32, q, qinv);
-    }
     int d[4][7][4];
     int z0 = 0, z1 = 0, z2 = 0, z3 = 0;       // a fixed quad of zero addends (see imma_u8_zero)
     asm volatile("" : "+r"(z0), "+r"(z1), "+r"(z2), "+r"(z3));
@@ -576,8 +567,8 @@ __global__ void __launch_bounds__(32 * IM_CW, 1) k_bsgs_accumulate_imma(
         const bool live = bp < bp_count && tb < tbs;
         u64* dst = acc + ((size_t)(live ? tb : 0) * bp_count + (live ? bp : 0)) * ctw + (size_t)l * N + c0 + warp;
         if (live) {
-            dst[0] = imma_recombine<FP>(d, 0, pc, c32, c64, c96);
-            dst[poly] = imma_recombine<FP>(d, 1, pc, c32, c64, c96);
+            dst[0] = imma_recombine<false>(d, 0, pc, 0, 0, 0);
+            dst[poly] = imma_recombine<false>(d, 1, pc, 0, 0, 0);
         }
     }
     cp_async_wait<0>();
@@ -585,7 +576,7 @@ __global__ void __launch_bounds__(32 * IM_CW, 1) k_bsgs_accumulate_imma(
 
 // Knobs for experiments.  FESC_BSGS_KERNEL picks the accumulate kernel: "int" the 128-bit integer one, "fp" the
 // exact-FP64 one, "mixed" the mixed-pipe one, anything else the default.  FESC_BSGS_GROUP_GIB fixes the scratch
-// budget that decides how many token blocks are processed per group (default: from the free device memory).
+// budget that decides how many token blocks are processed per group (default: the functions below).
 static int bsgs_kernel() {
     static int v = -1;
     if (v < 0) {
@@ -876,14 +867,14 @@ extern "C" int fesc_linear(fesc_ctx* ctx, const uint64_t* d_ct_in, const uint64_
         FESC_CHECK_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)); \
         kern<<<grid, MIX_THREADS, smem, st>>>(rot, diags, acc, ctx->d_pc, N, level, nt, gin * n1, bp_count);  \
     } while (0)
-#define BSGS_IMMA(FP, ST)                                                                                       \
+#define BSGS_IMMA(ST)                                                                                           \
     do {                                                                                                      \
         const uint32_t tp = ((gin * n1 + 31) / 32) * 32;                                                      \
         uint32_t pitch = tp * IM_ROWP;                                                                        \
         pitch += (17 - pitch % 16) % 16;          /* = 1 mod 16 */                                            \
         dim3 grid(N / IM_CW, level, (nt + 3) / 4);                                                            \
         const size_t smem = ((size_t)8 * pitch + (size_t)ST * IM_STAGE_WORDS) * 8;                            \
-        auto kern = k_bsgs_accumulate_imma<FP, ST>;                                                           \
+        auto kern = k_bsgs_accumulate_imma<ST>;                                                               \
         FESC_CHECK_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)); \
         kern<<<grid, 32 * IM_CW, smem, st>>>(rot, diags, acc, ctx->d_pc, N, level, nt, gin * n1, bp_count, pitch); \
     } while (0)
@@ -897,8 +888,8 @@ extern "C" int fesc_linear(fesc_ctx* ctx, const uint64_t* d_ct_in, const uint64_
         const bool deep = gin * n1 <= 128;       // room for 8 stages beside the rotated inputs
         if (mixed_ok && nt >= 2) BSGS_MIX(2, 8, 3);
         else if (mixed_ok) BSGS_MIX(1, 8, 4);
-        else if (imma_ok && deep) BSGS_IMMA(false, 8);
-        else if (imma_ok) BSGS_IMMA(false, 4);
+        else if (imma_ok && deep) BSGS_IMMA(8);
+        else if (imma_ok) BSGS_IMMA(4);
         else if (fp_ok && N % 256 == 0 && nt >= 2) BSGS_FPS(2, 8, 3);
         else if (fp_ok && nt >= 2) BSGS_FP(2, 8);
         else if (fp_ok) BSGS_FP(1, 8);

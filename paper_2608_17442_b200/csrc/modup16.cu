@@ -169,7 +169,7 @@ static int launch_modup(fesc_ctx* ctx, const u64* y, u64* ext, uint32_t level, u
     const size_t smem = ((size_t)A * MU_SRC + MU_GROUPS * COL_SMEM(MU_COLS)) * sizeof(u64);
     auto kern = k_modup_cols<A>;
     FESC_CHECK_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    // two CTAs per SM: with few ciphertexts the targets of a tile are shared by up to four CTAs, so that the last wave is full
+    // with few ciphertexts up to four CTAs share the targets of a tile, until there are four CTAs for every place (two per SM)
     uint32_t splits = 1;
     while (splits < 4 && tiles * beta * batch * splits < 8 * 148) splits++;
     launch(kern, dim3(tiles * splits, beta, batch), MU_THREADS, smem, st, y, ext, ctx->tabs.d_modup + (size_t)(level - 1) * ctx->beta_max,

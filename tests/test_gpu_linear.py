@@ -443,8 +443,8 @@ def test_scratch_beyond_the_usual_amount_leaves_the_caller_half_of_what_is_free(
     ctx, orc, p = ctx_pair("full")
     level, N, gin, nout, tbs, GiB = 24, orc.N, 64, 192, 8, 2**30
     free = torch.cuda.mem_get_info()[0]
-    if free < 130 * GiB:
-        pytest.skip("needs most of a 180 GB device")
+    if free < 130 * GiB or fesc.debug_bounds():
+        pytest.skip("needs most of a 180 GB device and the release kernels")
     desc = fesc.BsgsDesc(1, 1, gin, nout, tbs, level, 0, 0, 0, 0, 1, 7)
     g = torch.Generator(device="cuda").manual_seed(3)
     rand = lambda *shape: torch.randint(0, 1 << 49, shape, generator=g, dtype=torch.int64, device="cuda")
