@@ -441,6 +441,16 @@ static void free_tables(fesc_ctx* ctx) {
     dev_free(ctx->tabs.d_md_frag);
 }
 
+// Key rows between canonical residues and the doubles that N = 2^16 keys are kept in (EvalKey); rows on larger primes are copied.
+__global__ void __launch_bounds__(256) k_key_format(const u64* in, u64* out, const PrimeConst* __restrict__ pcs, uint32_t N, int to_double) {
+    const uint32_t c = blockIdx.x * blockDim.x + threadIdx.x;
+    const size_t at = ((size_t)blockIdx.z * gridDim.y + blockIdx.y) * N + c;
+    if (c >= N || !DBG_REGION(in + at, sizeof(u64)) || !DBG_REGION(out + at, sizeof(u64))) return;
+    const PrimeConst& pc = pcs[blockIdx.y];
+    const u64 v = in[at];
+    if (pc.q >= FESC_FP_LIMIT) out[at] = v;
+    else out[at] = to_double ? (u64)__double_as_longlong(fp_load(v, pc.qd)) : fp_store(__longlong_as_double((long long)v), pc.qd, pc.qinvd);
+}
 // Generate the switching key from s' (EVAL on all limbs, device) to s.
 static int gen_key(fesc_ctx* ctx, uint32_t key_id, const u64* d_sp, u64 g) {
     const uint32_t N = ctx->N, np = ctx->n_primes;
@@ -469,6 +479,7 @@ static int gen_key(fesc_ctx* ctx, uint32_t key_id, const u64* d_sp, u64 g) {
         if (hi > ctx->n_q) hi = ctx->n_q;
         k_make_b<<<grid, 256>>>(b, a, ctx->d_s, d_e, d_sp, ctx->d_pc, ctx->tabs.d_Pmod_all, N, lo, hi);
     }
+    if (rc == FESC_OK && ctx->log_n == 16) k_key_format<<<dim3((N + 255) / 256, np, 2 * ctx->beta_max), 256>>>(d_key, d_key, ctx->d_pc, N, 1);
     cudaError_t e = cudaDeviceSynchronize();
     dev_free(d_e);
     if (rc == FESC_OK && e != cudaSuccess) {
@@ -733,6 +744,12 @@ extern "C" int fesc_ctx_export_key(fesc_ctx* ctx, uint32_t key_id, uint64_t* d_d
     if (!ctx || !d_dst) return FESC_EINVAL;
     auto it = ctx->keys.find(key_id);
     if (it == ctx->keys.end()) return fesc_fail(ctx, FESC_ENOKEY, "no key " + std::to_string(key_id));
+    if (ctx->log_n == 16) {
+        k_key_format<<<dim3((ctx->N + 255) / 256, ctx->n_primes, 2 * ctx->beta_max), 256, 0, (cudaStream_t)stream>>>(it->second.d_key, (u64*)d_dst, ctx->d_pc,
+                                                                                                                    ctx->N, 0);
+        FESC_CHECK_CUDA(ctx, cudaGetLastError());
+        return FESC_OK;
+    }
     size_t bytes = (size_t)ctx->beta_max * 2 * ctx->n_primes * ctx->N * sizeof(u64);
     FESC_CHECK_CUDA(ctx, cudaMemcpyAsync(d_dst, it->second.d_key, bytes, cudaMemcpyDeviceToDevice, (cudaStream_t)stream));
     return FESC_OK;

@@ -4,9 +4,10 @@
 // the transformed digits for several keys).  The transformed rows are never stored: 75 MB written and 88 MB read per ciphertext at
 // 24 limbs.
 //
-// Measured on 128 rotations at 24 limbs (batches of 16): 5.84 ms and 2.7 ms less in the transforms, against 3.45 ms for the inner
-// product on stored digits; FP64 pipe 55 %, the rest is latency at 16 warps per SM.  Staging the next digit's points through shared
-// memory with asynchronous copies was slower (9.2 ms): it takes the L1 from the key words and twiddles that the warps share.
+// What bounds it: the dispatch port (issue slots 50 %, FP64 pipe 47 %, its instructions hold the port for two or three cycles) at 16 warps
+// per SM; 16 rotations at 24 limbs 0.77 -> 0.63 ms when the next digit's points and key words came to be fetched by bulk copies, while a
+// digit is transformed: a warp's 4 KB of points and the CTA's 8 KB of keys (one copy for its ciphertexts) have their own shared memory and the
+// L1 keeps the twiddles.  (Points by 8-byte asynchronous copies instead 1.2 ms, points alone by bulk copies 0.15 ms more.)
 //
 // The special rows arrive transformed and are multiplied by the last CTAs of the same launch: their products and loads run beside the
 // data rows' arithmetic and fill its last wave (5.36 + 0.98 ms in two launches, 5.84 ms in one; first instead of last 6.02).  Two warps per 512 points with
@@ -14,7 +15,8 @@
 //
 // A warp owns 512 points of one row of one ciphertext.  It runs rounds C and D of every digit in turn (the digit that holds the row
 // itself needs no transform), multiplies with the two key words of each point and keeps both sums in registers; 128 registers, 16
-// warps per SM.  The four warps of a CTA are four ciphertexts on the same points, so that the key words come from L1 after the first.
+// warps per SM.  The warps of a CTA (up to four, shared out evenly: 5 run as 3 + 2) are ciphertexts on the same points.  Every wait is bounded
+// (status word 5).
 #define FESC_DBG_FILE 14   // file id in the sites a debug build reports
 #include "ntt16.cuh"
 #include "ops.cuh"
@@ -60,15 +62,28 @@ __device__ __forceinline__ void int_rows(const InnerSrcs& S, uint32_t s0, uint32
     }
 }
 
+#define RI_X 512                    // words of a warp's staged points
+#define RI_WARP_WORDS (RI_X + ROW_SMEM)
+#define RI_KEY_WORDS 1024
+// bytes of shared memory for a CTA of `warps`: keys, per warp the staged points and the exchange buffer, barriers
+#define RI_SMEM(warps) (8 * (RI_KEY_WORDS + (warps) * RI_WARP_WORDS + (warps) + 2))
 __global__ void __launch_bounds__(32 * RI_WARPS, 4)
     k_rows_inner(InnerSrcs S, u64* acc, const double* __restrict__ twf, const PrimeConst* __restrict__ pcs, uint32_t level, uint32_t n_q,
-                 uint32_t K, uint32_t alpha, uint32_t beta, uint32_t batch, int accumulate, int sep) {
-    pdl_begin();
-    __shared__ __align__(16) u64 sm_all[RI_WARPS * ROW_SMEM];
-    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, id = blockIdx.x * RI_WARPS + warp;
-    const uint32_t blk = id / batch, b = id - blk * batch, t = blockIdx.y, rows = level + K, np = n_q + K;
+                 uint32_t K, uint32_t alpha, uint32_t beta, uint32_t batch, uint32_t groups, int accumulate, int sep, uint32_t* __restrict__ status) {
+    extern __shared__ __align__(128) u64 smem[];
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+    const uint32_t blk = blockIdx.x / groups, b0 = (blockIdx.x - blk * groups) * warps, b = b0 + warp, t = blockIdx.y, rows = level + K, np = n_q + K;
     const uint32_t pt = t < level ? t : n_q + (t - level), own = t / alpha;
-    if (blk >= 128) return;                             // warp barriers only
+    const uint32_t base = (uint32_t)__cvta_generic_to_shared(smem), bars = base + 8 * (RI_KEY_WORDS + warps * RI_WARP_WORDS);
+    const uint32_t x_bar = bars + 8 * warp, key_full = bars + 8 * warps, last = (batch - b0 < warps ? batch - b0 : warps) - 1;
+    if (threadIdx.x == 0) {
+        for (uint32_t i = 0; i <= warps; i++) mbar_init(bars + 8 * i, 1);
+        smem[RI_KEY_WORDS + warps * RI_WARP_WORDS + warps + 1] = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    pdl_begin();
+    __syncthreads();
+    if (b >= batch) return;
     const uint32_t s0 = sep ? blockIdx.z : 0, s1 = sep ? s0 + 1 : S.n;
     acc += (size_t)s0 * batch * 2 * rows * N16;         // separate sources have their own accumulators
     u64* o0 = acc + ((size_t)b * 2 * rows + t) * N16 + blk * 512 + 2 * lane;
@@ -85,7 +100,21 @@ __global__ void __launch_bounds__(32 * RI_WARPS, 4)
         int_rows(S, s0, s1, o0, o1, pcs[pt], x_at + 2 * lane, (size_t)rows * N16, key_at, (size_t)np * N16, beta, accumulate);
         return;
     }
-    u64* sm = sm_all + warp * ROW_SMEM;
+    const uint32_t total = (s1 - s0) * beta;
+    auto load_x = [&](uint32_t s, uint32_t j) {         // lane 0
+        mbar_expect_tx(x_bar, 8 * RI_X);
+        bulk_g2s(base + 8 * (RI_KEY_WORDS + warp * RI_WARP_WORDS), S.s[s].ext + x_at + (size_t)j * rows * N16, 8 * RI_X, x_bar);
+    };
+    auto load_keys = [&](uint32_t s, uint32_t j) {      // one lane of the CTA
+        const u64* k = S.s[s].key + (size_t)pt * N16 + blk * 512 + (size_t)(2 * j) * np * N16;
+        mbar_expect_tx(key_full, 8 * 1024);
+        bulk_g2s(base, k, 8 * 512, key_full);
+        bulk_g2s(base + 8 * 512, k + (size_t)np * N16, 8 * 512, key_full);
+    };
+    if (lane == 0) load_x(s0, 0);
+    if (threadIdx.x == 0) load_keys(s0, 0);
+    const u64* sx = smem + RI_KEY_WORDS + warp * RI_WARP_WORDS;
+    u64* sm = smem + RI_KEY_WORDS + warp * RI_WARP_WORDS + RI_X;
     const u64* sp = sm + 2 * lane + 2 * (lane >> 3);    // the pair 2 lane (+ 64 j) of the padded buffer
     const FpRow r{twf + (size_t)t * N16, pcs[t].qd, pcs[t].qinvd};
     const double q = r.q, qinv = r.qinv;
@@ -99,47 +128,55 @@ __global__ void __launch_bounds__(32 * RI_WARPS, 4)
             f1[2 * k] = fp_load(v1.x, q), f1[2 * k + 1] = fp_load(v1.y, q);
         }
     }
-    uint32_t n = 0;
-    for (uint32_t s = s0; s < s1; s++) {
-        const u64* row = S.s[s].ext + x_at;
-        const u64* key = S.s[s].key + key_at;
+    uint32_t s = s0, j = 0, room = accumulate || beta > 6 ? 5 : 6;
 #pragma unroll 1
-        for (uint32_t j = 0; j < beta; j++, row += (size_t)rows * N16, key += (size_t)2 * np * N16) {
-            // the next digit's points and this digit's key words arrive in L2 while the digit is transformed (6.2 -> 5.8 ms below)
-            if (j + 1 < beta) prefetch_l2(row + (size_t)rows * N16 + 16 * lane);
-            prefetch_l2(key + 14 * lane);
-            prefetch_l2(key + (size_t)np * N16 + 14 * lane);
-            if (j != own) {
-                const u64* in = row + 256 * (lane >> 4) + (lane & 15);
-                double x[16];
+    for (uint32_t n = 0; n < total; n++) {
+        const uint32_t s_next = j + 1 < beta ? s : s + 1, j_next = j + 1 < beta ? j + 1 : 0;
+        if (mbar_wait_bounded(x_bar, n & 1)) {          // gives up: the other copy in flight is waited for as well (bounded)
+            if (lane == 0) atomicExch(status, 5u);
+            mbar_wait_bounded(key_full, n & 1);
+            return;
+        }
+        if (j != own) {
+            const u64* in = sx + 256 * (lane >> 4) + (lane & 15);
+            double x[16];
 #pragma unroll
-                for (int k = 0; k < 16; k++) x[k] = FpRow::value(in[16 * k]);
-                __syncwarp();                           // the previous digit's values have been read
-                fwd_rows(r, x, sm, blk, lane);
-            }
-            // |x| <= q/2 once folded: products below 0.7 q, seven and a rest of q/2 below 8 q
-            const bool fold = ++n % 7 == 0;
+            for (int k = 0; k < 16; k++) x[k] = FpRow::value(in[16 * k]);
+            __syncwarp();                               // the staged points and the previous digit's values have been read
+            if (lane == 0 && n + 1 < total) load_x(s_next, j_next);
+            fwd_rows(r, x, sm, blk, lane);
+        }
+        if (mbar_wait_bounded(key_full, n & 1)) {
+            if (lane == 0) atomicExch(status, 5u);
+            if (j != own && n + 1 < total) mbar_wait_bounded(x_bar, (n + 1) & 1);
+            return;
+        }
+        const u64* key = smem + 2 * lane;
 #pragma unroll
-            for (int k = 0; k < 8; k++) {
-                const ulonglong2 w0 = __ldg(reinterpret_cast<const ulonglong2*>(key + 64 * k));
-                const ulonglong2 w1 = __ldg(reinterpret_cast<const ulonglong2*>(key + (size_t)np * N16 + 64 * k));
-                double xa, xb;
-                if (j != own) {
-                    const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(sp + 72 * k);
-                    xa = r.fold(FpRow::value(v.x)), xb = r.fold(FpRow::value(v.y));
-                } else {
-                    const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(row + 2 * lane + 64 * k);
-                    xa = FpRow::value(v.x), xb = FpRow::value(v.y);
-                }
-                f0[2 * k] += fp_modmul(xa, fp_from_u64(w0.x), q, qinv);
-                f0[2 * k + 1] += fp_modmul(xb, fp_from_u64(w0.y), q, qinv);
-                f1[2 * k] += fp_modmul(xa, fp_from_u64(w1.x), q, qinv);
-                f1[2 * k + 1] += fp_modmul(xb, fp_from_u64(w1.y), q, qinv);
+        for (int k = 0; k < 8; k++) {
+            const double2 w0 = *reinterpret_cast<const double2*>(key + 64 * k);
+            const double2 w1 = *reinterpret_cast<const double2*>(key + 512 + 64 * k);
+            const double2 v = *reinterpret_cast<const double2*>(j != own ? sp + 72 * k : sx + 2 * lane + 64 * k);
+            f0[2 * k] += fp_modmul(v.x, w0.x, q, qinv);
+            f0[2 * k + 1] += fp_modmul(v.y, w0.y, q, qinv);
+            f1[2 * k] += fp_modmul(v.x, w1.x, q, qinv);
+            f1[2 * k + 1] += fp_modmul(v.y, w1.y, q, qinv);
+        }
+        if (n + 1 < total) {
+            __syncwarp();
+            if (lane == 0) {
+                if (j == own) load_x(s_next, j_next);
+                // the last warp to have read the key words requests the next ones
+                if (atomicInc(reinterpret_cast<uint32_t*>(smem + RI_KEY_WORDS + warps * RI_WARP_WORDS + warps + 1), last) == last) load_keys(s_next, j_next);
             }
-            if (fold) {
-                fold16(r, f0);
-                fold16(r, f1);
-            }
+        }
+        s = s_next, j = j_next;
+        // A transformed point stays below 4.82 q (five stages from q/2), its product below 1.41 q, an own digit's below 0.6 q: five products and
+        // a rest of q/2 stay below 8 q, and so do six that start from zero and have an own one among them (a source of up to six digits)
+        if (--room == 0 && n + 1 < total) {
+            fold16(r, f0);
+            fold16(r, f1);
+            room = 5;
         }
     }
 #pragma unroll
@@ -150,10 +187,11 @@ __global__ void __launch_bounds__(32 * RI_WARPS, 4)
 }
 
 int rows_inner_launch(fesc_ctx* ctx, const InnerSrcs& S, u64* acc, uint32_t level, uint32_t batch, int accumulate, bool separate, cudaStream_t st) {
-    const uint32_t beta = (level + ctx->alpha - 1) / ctx->alpha;
-    const dim3 grid((128 * batch + RI_WARPS - 1) / RI_WARPS, level + ctx->n_p, separate ? S.n : 1);
-    launch(k_rows_inner, grid, 32 * RI_WARPS, 0, st, S, acc, ctx->d_twf, ctx->d_pc, level, ctx->n_q, ctx->n_p, ctx->alpha, beta, batch, accumulate,
-           separate ? 1 : 0);
+    const uint32_t beta = (level + ctx->alpha - 1) / ctx->alpha, groups = (batch + RI_WARPS - 1) / RI_WARPS, warps = (batch + groups - 1) / groups;
+    const dim3 grid(128 * groups, level + ctx->n_p, separate ? S.n : 1);
+    FESC_CHECK_CUDA(ctx, cudaFuncSetAttribute(k_rows_inner, cudaFuncAttributeMaxDynamicSharedMemorySize, RI_SMEM(RI_WARPS)));
+    launch(k_rows_inner, grid, 32 * warps, RI_SMEM(warps), st, S, acc, ctx->d_twf, ctx->d_pc, level, ctx->n_q, ctx->n_p, ctx->alpha, beta, batch, groups, accumulate,
+           separate ? 1 : 0, ctx->d_status);
     FESC_CHECK_CUDA(ctx, cudaGetLastError());
     return FESC_OK;
 }

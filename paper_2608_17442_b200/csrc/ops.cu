@@ -274,6 +274,8 @@ __global__ void __launch_bounds__(256) k_modup(const u64* __restrict__ dcoef, u6
 #ifndef INNER_MINB
 #define INNER_MINB 4
 #endif
+// a key word of a row on a prime below 2^50: a double at N = 2^16 (EvalKey), a canonical residue in smaller rings
+__device__ __forceinline__ double key_double(u64 w, int as_double) { return as_double ? __longlong_as_double((long long)w) : fp_from_u64(w); }
 // PATH 0: the row's prime decides at run time; 1: the caller guarantees primes below 2^50 on rows
 // [row0, row0 + gridDim.y) (exact FP64 products only); 2: the caller sends those rows to the 128-bit integer sums.
 template <int BT, int PATH>
@@ -366,7 +368,7 @@ __global__ void __launch_bounds__(256, INNER_MINB) k_inner(InnerSrcs S, u64* acc
 #pragma unroll 1
         for (uint32_t it = 0; it < total; it++) {
             if (it + 1 < total) load_next(nkb, nka, nx);
-            const double dkb = fp_from_u64(kb), dka = fp_from_u64(ka);
+            const double dkb = key_double(kb, x_double), dka = key_double(ka, x_double);
 #pragma unroll
             for (int i = 0; i < BT; i++) {
                 // canonical words (every product below 0.875q) or doubles with |x| <= q/2 left by the producers
@@ -502,7 +504,7 @@ __global__ void __launch_bounds__(256, 4) k_inner_shared(const u64* __restrict__
         if (FP) {
             double kd[2 * BETA];
 #pragma unroll
-            for (int j = 0; j < 2 * BETA; j++) kd[j] = fp_from_u64(kw[j]);
+            for (int j = 0; j < 2 * BETA; j++) kd[j] = __longlong_as_double((long long)kw[j]);
             for (uint32_t b = part; b < batch; b += 256 / IS_BLK) {
                 double f0 = 0.0, f1 = 0.0;
 #pragma unroll
@@ -679,7 +681,7 @@ __global__ void __launch_bounds__(256, 1) k_inner_tma(const u64* __restrict__ ex
             }
             for (uint32_t j = 0; j < beta; j++) {
                 const u64* dj = sm + (size_t)j * R * 256;
-                const double dkb = fp_from_u64(dj[tid]), dka = fp_from_u64(dj[256 + tid]);
+                const double dkb = key_double(dj[tid], x_double), dka = key_double(dj[256 + tid], x_double);
 #pragma unroll
                 for (int i = 0; i < BT; i++) {
                     const u64 xw = dj[(2 + i) * 256 + si];

@@ -1,0 +1,72 @@
+"""Key switches over the sizes of special primes (N = 2^16) and sums over many products."""
+import numpy as np
+import pytest
+
+import fesc_synth as S
+from gpu_util import add_key, ctx_pair, random_ct, to_dev, to_host
+
+pytestmark = pytest.mark.gpu
+
+
+def _pair(bits, n_p):
+    import paper_2608_17442_b200 as fesc
+    from oracle.ckks import Oracle
+
+    args = (16, S.ntt_primes(50, 16, 5, 0) + S.ntt_primes(bits, 16, n_p, 0), 5, n_p, 2, 61)
+    return fesc.Context(*args), Oracle(*args), None
+
+
+@pytest.mark.parametrize("bits,n_p", [(60, 4), (55, 2), (51, 1), (61, 2)])
+def test_key_switches_by_size_of_the_special_primes(bits, n_p):
+    """Special primes next to 2^60 and next to 2^51 from below, and 61 bits, which the fused division does not take: their transforms at the
+    ends of the range, a relinearisation, a rotation, hoisted rotations and their sum."""
+    import torch
+
+    pair = _pair(bits, n_p)
+    ctx, orc, _ = pair
+    for k, rot in enumerate((3, -8, 4096)):
+        add_key(pair, rot, 70 + k)
+    idx = list(range(5, 5 + n_p))
+    rows = np.empty((2, n_p, orc.N), dtype=np.uint64)
+    for k, i in enumerate(idx):
+        rows[0, k] = orc.q[i] - 1
+        rows[1, k] = np.where((np.arange(orc.N) * 2654435761 >> 7) % 3 == 0, 0, orc.q[i] // 2 + 1)
+    for gpu, ref in ((ctx.ntt, orc.ntt), (ctx.intt, orc.intt)):
+        d = to_dev(rows)
+        gpu(d, 2, 5, n_p)
+        got = to_host(d)
+        for b in range(2):
+            assert np.array_equal(got[b], ref(rows[b], idx))
+    ct, ids = random_ct(orc, 5, 5, 5, 3), [70, 71, 72]
+    d, out = to_dev(ct), torch.empty((3, 3, 2, 5, orc.N), dtype=torch.int64, device="cuda")
+    ctx.rotate(d, out[0], 3, 5, 71)
+    ctx.rotate_sum_hoisted(d, out[1], 3, 5, ids)
+    ctx.ct_ct_mul(d, d, out[2], 3, 5)
+    got = to_host(out)
+    for b in range(3):
+        assert np.array_equal(got[0, b], orc.rotate(ct[b], 71))
+        assert np.array_equal(got[1, b], orc.rotate_sum_hoisted(ct[b], ids))
+        assert np.array_equal(got[2, b], orc.ct_ct_mul(ct[b], ct[b]))
+    ctx.rotate_hoisted(d, out, 3, 5, ids)
+    got = to_host(out)
+    for b in range(3):
+        assert np.array_equal(got[:, b], np.stack(orc.rotate_hoisted(ct[b], ids)))
+
+
+@pytest.mark.parametrize("level,batch,n_keys", [(24, 2, 8), (9, 4, 3), (4, 1, 7)])
+def test_sums_that_are_reduced_in_between(level, batch, n_keys):
+    """Up to 48 products per sum, and batches of one, two and four ciphertexts per thread."""
+    import torch
+
+    pair = ctx_pair("full")
+    ctx, orc, _ = pair
+    ids = [700 + k for k in range(n_keys)]
+    for k, i in enumerate(ids):
+        add_key(pair, 16 * k + 1, i)
+    ct = random_ct(orc, 41, level, level, batch)
+    ct[0] = (np.array(orc.q[:level], dtype=np.uint64) - np.uint64(1))[None, :, None]
+    out = torch.empty_like(to_dev(ct))
+    ctx.rotate_sum_hoisted(to_dev(ct), out, batch, level, ids)
+    got = to_host(out)
+    for b in sorted({0, batch - 1}):
+        assert np.array_equal(got[b], orc.rotate_sum_hoisted(ct[b], ids))
