@@ -244,7 +244,8 @@ struct ModDownTab {
     u64 pinv[FESC_MAX_PRIMES], pinvs[FESC_MAX_PRIMES];   // P^-1 mod q_i
     double matd[FESC_MAX_SPECIAL][FESC_MAX_PRIMES], mat30d[FESC_MAX_SPECIAL][FESC_MAX_PRIMES];   // as doubles
     double wrapd[FESC_MAX_SPECIAL + 1][FESC_MAX_PRIMES], pinvd[FESC_MAX_PRIMES];
-    ModUpTerm term[4][FESC_MAX_PRIMES];                  // (P/p_k) mod q_i centred, and divided by 2^10 q_i (modup16.cu)
+    ModUpTerm term[4][FESC_MAX_PRIMES];                  // (P/p_k) mod q_i centred, and divided by 4 q_i (modup16.cu)
+    double start[FESC_MAX_PRIMES];                       // 1.5 * 2^52 times (1 - the sum of a target's mq)
 };
 // Rescale from level l (drops limb l-1); entry index l.
 struct RescaleTab {
@@ -448,7 +449,8 @@ struct NttFinish {
 // rows: number of N-word rows starting at d_data; map gives the prime per row.
 // in_double (forward, N = 2^16 only): rows on primes below 2^50 hold doubles with |x| <= q/2 (bit patterns) written by a
 // basis-conversion kernel instead of canonical words.
-// scale (inverse, N = 2^16 only): per prime index, constants in place of those of the last stage.  skip_cols (forward, N = 2^16 only): the first eight stages are already done.
+// scale (inverse, N = 2^16 only): per prime index, constants in place of those of the last stage.  skip_cols (N = 2^16 only): without the eight
+// stages of distance 256 and more (forward: they are done; inverse: the consumer does them).
 // out_double (forward, N = 2^16 only): such rows are left as doubles with |x| <= q/2 for a consumer that computes in FP64.
 int ntt_launch(fesc_ctx* ctx, u64* d_data, size_t rows, const RowMap& map, bool inverse, cudaStream_t st,
                bool in_double = false, bool out_double = false, const NttFinish* finish = nullptr,

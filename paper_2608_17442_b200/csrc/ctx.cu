@@ -386,7 +386,7 @@ static int build_tables(fesc_ctx* ctx) {
             md.matd[k][i] = (double)md.mat[k][i];
             if (k < 4) {
                 md.term[k][i].m = m > q[i] / 2 ? -(long long)(q[i] - m) : (long long)m;
-                md.term[k][i].mq = (double)((long double)md.term[k][i].m / ((long double)q[i] * 1024));
+                md.term[k][i].mq = (double)((long double)md.term[k][i].m / ((long double)q[i] * 4));
             }
             md.mat30d[k][i] = (double)md.mat30[k][i];
         }
@@ -395,6 +395,9 @@ static int build_tables(fesc_ctx* ctx) {
         u64 P = 1;
         for (uint32_t b = 0; b < K; b++) P = h_mul(P, q[nq + b] % q[i], q[i]);
         Pmod[i] = P;
+        long double mq = 0;
+        for (uint32_t k = 0; k < K && k < 4; k++) mq += (long double)md.term[k][i].mq;
+        md.start[i] = (double)(0x1.8p52L * (1 - mq));
         md.pinv[i] = h_inv(P, q[i]);
         md.pinvs[i] = h_shoup(md.pinv[i], q[i]);
         for (uint32_t c = 0; c <= K; c++) md.wrap[c][i] = h_mul(c, P, q[i]);

@@ -11,7 +11,8 @@
 //
 // The special rows arrive transformed and are multiplied by the last CTAs of the same launch: their products and loads run beside the
 // data rows' arithmetic and fill its last wave (5.36 + 0.98 ms in two launches, 5.84 ms in one; first instead of last 6.02).  Two warps per 512 points with
-// half the digits each, for single ciphertexts: 103 us against 86.
+// half the digits each, for single ciphertexts: 103 us against 86.  Where the division by P follows, the special rows are left after the first
+// pass of their inverse transform, on the 512 points that a warp has just summed: 0.071 ms of a launch for 0.057 here.
 //
 // A warp owns 512 points of one row of one ciphertext.  It runs rounds C and D of every digit in turn (the digit that holds the row
 // itself needs no transform), multiplies with the two key words of each point and keeps both sums in registers; 128 registers, 16
@@ -67,9 +68,29 @@ __device__ __forceinline__ void int_rows(const InnerSrcs& S, uint32_t s0, uint32
 #define RI_KEY_WORDS 1024
 // bytes of shared memory for a CTA of `warps`: keys, per warp the staged points and the exchange buffer, barriers
 #define RI_SMEM(warps) (8 * (RI_KEY_WORDS + (warps) * RI_WARP_WORDS + (warps) + 2))
+// first pass of the inverse transform of 512 canonical points at o, which this lane's earlier stores have put there (words 2 lane + 64 j of the block)
+__device__ __forceinline__ void int_rows_inv(const IntRow& r, u64* o, u64* sm, uint32_t blk, uint32_t lane) {
+    u64* s = sm + 2 * lane + 2 * (lane >> 3);
+#pragma unroll
+    for (int j = 0; j < 8; j++) {
+        const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(o + 2 * lane + 64 * j);
+        *reinterpret_cast<ulonglong2*>(s + 72 * j) = v;
+    }
+    __syncwarp();
+    u64 x[16];
+    inv_rows(r, x, sm, blk, lane);
+    u64* d = o + 256 * (lane >> 4) + (lane & 15);
+#pragma unroll
+    for (int k = 0; k < 16; k++) d[16 * k] = x[k];
+    __syncwarp();
+}
+
+// itw: not nullptr where the sums are complete and the division by P takes the special rows after the first pass of their inverse transform
+// (no launch for that pass, and its rows are still in L2)
 __global__ void __launch_bounds__(32 * RI_WARPS, 4)
-    k_rows_inner(InnerSrcs S, u64* acc, const double* __restrict__ twf, const PrimeConst* __restrict__ pcs, uint32_t level, uint32_t n_q,
-                 uint32_t K, uint32_t alpha, uint32_t beta, uint32_t batch, uint32_t groups, int accumulate, int sep, uint32_t* __restrict__ status) {
+    k_rows_inner(InnerSrcs S, u64* acc, const double* __restrict__ twf, const ulonglong2* __restrict__ itw, const PrimeConst* __restrict__ pcs,
+                 uint32_t level, uint32_t n_q, uint32_t K, uint32_t alpha, uint32_t beta, uint32_t batch, uint32_t groups, int accumulate, int sep,
+                 uint32_t* __restrict__ status) {
     extern __shared__ __align__(128) u64 smem[];
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
     const uint32_t blk = blockIdx.x / groups, b0 = (blockIdx.x - blk * groups) * warps, b = b0 + warp, t = blockIdx.y, rows = level + K, np = n_q + K;
@@ -98,6 +119,12 @@ __global__ void __launch_bounds__(32 * RI_WARPS, 4)
     const size_t x_at = ((size_t)b * beta * rows + t) * N16 + blk * 512, key_at = (size_t)pt * N16 + blk * 512 + 2 * lane;
     if (t >= level) {
         int_rows(S, s0, s1, o0, o1, pcs[pt], x_at + 2 * lane, (size_t)rows * N16, key_at, (size_t)np * N16, beta, accumulate);
+        if (itw) {
+            const IntRow r{itw + (size_t)pt * N16, pcs[pt].q, 2 * pcs[pt].q};
+            u64* buf = smem + RI_KEY_WORDS + warp * RI_WARP_WORDS + RI_X;
+#pragma unroll 1
+            for (int p = 0; p < 2; p++) int_rows_inv(r, (p ? o1 : o0) - 2 * lane, buf, blk, lane);
+        }
         return;
     }
     const uint32_t total = (s1 - s0) * beta;
@@ -186,12 +213,14 @@ __global__ void __launch_bounds__(32 * RI_WARPS, 4)
     }
 }
 
-int rows_inner_launch(fesc_ctx* ctx, const InnerSrcs& S, u64* acc, uint32_t level, uint32_t batch, int accumulate, bool separate, cudaStream_t st) {
+int rows_inner_launch(fesc_ctx* ctx, const InnerSrcs& S, u64* acc, uint32_t level, uint32_t batch, int accumulate, bool separate, bool inv_special,
+                      cudaStream_t st) {
     const uint32_t beta = (level + ctx->alpha - 1) / ctx->alpha, groups = (batch + RI_WARPS - 1) / RI_WARPS, warps = (batch + groups - 1) / groups;
     const dim3 grid(128 * groups, level + ctx->n_p, separate ? S.n : 1);
     FESC_CHECK_CUDA(ctx, cudaFuncSetAttribute(k_rows_inner, cudaFuncAttributeMaxDynamicSharedMemorySize, RI_SMEM(RI_WARPS)));
-    launch(k_rows_inner, grid, 32 * warps, RI_SMEM(warps), st, S, acc, ctx->d_twf, ctx->d_pc, level, ctx->n_q, ctx->n_p, ctx->alpha, beta, batch, groups, accumulate,
-           separate ? 1 : 0, ctx->d_status);
+    launch(k_rows_inner, grid, 32 * warps, RI_SMEM(warps), st, S, acc, ctx->d_twf,
+           inv_special ? ctx->d_itw : nullptr, ctx->d_pc, level, ctx->n_q, ctx->n_p, ctx->alpha, beta, batch, groups,
+           accumulate, separate ? 1 : 0, ctx->d_status);
     FESC_CHECK_CUDA(ctx, cudaGetLastError());
     return FESC_OK;
 }

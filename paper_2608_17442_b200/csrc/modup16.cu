@@ -89,7 +89,7 @@ __device__ __forceinline__ void convert4(const u64* p, uint32_t n_src, const Mod
 
 template <int A>
 __global__ void __launch_bounds__(MU_THREADS, 2)
-    k_modup_cols(const u64* __restrict__ y, u64* __restrict__ ext, const ModUpDigit* __restrict__ tab, const double* __restrict__ twf,
+    k_modup_cols(const u64* y, u64* ext, const ModUpDigit* __restrict__ tab, const double* __restrict__ twf,
                  const ulonglong2* __restrict__ tw, const PrimeConst* __restrict__ pcs, uint32_t level, uint32_t n_q, uint32_t K,
                  uint32_t beta, uint32_t splits) {
     pdl_begin();
@@ -187,18 +187,27 @@ int modup16_cols_launch(fesc_ctx* ctx, const u64* y, u64* ext, uint32_t level, u
 //   u_i = sum_k y_k m_k mod q_i,  y_k = r_k (P/p_k)^-1 mod p_k centred (the constant rides on the inverse transform's last stage),
 //   m_k = (P/p_k) mod q_i.
 // The sources have 60 bits, so the quotient is taken in units of 2^10: c = rint(sum_k y_k (m_k / (q 2^10))), |c| <= 2^50, and
-// v = sum_k y_k m_k - c 2^10 q is below 2.1 2^10 q < 2^62; a second quotient from the high word of v leaves |v| <= 0.7 q.  Per source
-// that is one FP64 multiply-add, one wide and two narrow integer ones, and no counting of negative residues.
+// v = sum_k y_k m_k - c 2^10 q is below 5.2 2^10 q < 2^63; a second quotient from the high word of v leaves |v| <= 0.7 q.  A source word is
+// kept once, with 2^59 added: its upper 52 bits below the exponent of 2^52 are the double that the quotient needs (a shift by eight in
+// registers), the word itself goes to the integer products, what the additions contribute is in the sum's starting value and in the
+// cross terms.  Reading the doubles as well loaded shared memory to 67 % and left room for three groups per CTA.
+//
+// How far c is from the quotient: the running sum stays within [0.75, 2.25] 2^52, so the start and the first three multiply-adds round by at most
+// 1, the last by 1/2; the bits shifted out are below 1 each, times |m / 4q| <= 1/8; errors of m / 4q are below 2^-5.  Together 5.2.
 // ---------------------------------------------------------------------------------------
-#define MD_GROUPS 3
+#define MD_GROUPS 4
 #define MD_THREADS (MD_GROUPS * MU_TARGET_THREADS)
+#define MD_BIAS (1ull << 59)
 
-template <int A>
+// OPEN: the special rows await the last eight stages of their inverse transform, which are done here on the columns that the CTA
+// needs anyway, one group per row: no pass of its own, 8 rows per ciphertext less to write and read (division of 42 rotations at 24 limbs,
+// with the passes it replaces: 1.12 -> 0.98 ms).
+template <int A, bool OPEN>
 __global__ void __launch_bounds__(MD_THREADS, 2)
-    k_moddown_cols(const u64* __restrict__ acc, u64* __restrict__ u, const ModDownTab* __restrict__ tab, const double* __restrict__ twf,
-                   const PrimeConst* __restrict__ pcs, uint32_t level, uint32_t n_q, uint32_t K, uint32_t splits) {
+    k_moddown_cols(const u64* acc, u64* u, const ModDownTab* __restrict__ tab, const double* __restrict__ twf,
+                   const ulonglong2* __restrict__ itw, const InvScale* __restrict__ scale, const PrimeConst* __restrict__ pcs, uint32_t level, uint32_t n_q, uint32_t K, uint32_t splits) {
     pdl_begin();
-    extern __shared__ __align__(16) u64 smem[];      // [A][MU_SRC] sources, the same as doubles, then one exchange buffer per group
+    extern __shared__ __align__(16) u64 smem[];      // [A][MU_SRC] sources, then one exchange buffer per group
     __shared__ uint32_t next, taken[MD_GROUPS];
     const uint32_t tid = threadIdx.x, tile = blockIdx.x / splits, part = blockIdx.x % splits, bp = blockIdx.y;
     const u64* src = acc + ((size_t)bp * (level + K) + level) * N16 + tile * MU_COLS;
@@ -206,26 +215,49 @@ __global__ void __launch_bounds__(MD_THREADS, 2)
     if (!DBG_REGION(tab, sizeof(ModDownTab)) || !DBG_REGION(src - tile * MU_COLS, (size_t)K * N16 * sizeof(u64)) ||
         !DBG_REGION(out - tile * MU_COLS, (size_t)level * N16 * sizeof(u64)))
         return;                                     // the same for the whole CTA
-    double* smd = reinterpret_cast<double*>(smem + A * MU_SRC);
-    for (uint32_t i = tid; i < A * (MU_SRC / 2); i += MD_THREADS) {
-        const uint32_t a = i / (MU_SRC / 2), r = (i / (MU_COLS / 2)) & 255, c = 2 * (i % (MU_COLS / 2)), at = a * MU_SRC + r * MU_COLS + c;
-        ulonglong2 v = make_ulonglong2(0, 0);
-        if (a < K) {
-            v = *reinterpret_cast<const ulonglong2*>(src + (size_t)a * N16 + r * 256 + c);
+    const uint32_t group = tid / MU_TARGET_THREADS, gt = tid % MU_TARGET_THREADS, col = gt % MU_COLS, sub = gt / MU_COLS;
+    const GroupBarrier bar{1 + group};
+    u64* sm = smem + A * MU_SRC + group * COL_SMEM(MU_COLS);
+    if (OPEN) {
+        for (uint32_t a = group; a < A; a += MD_GROUPS) {
+            u64* y = smem + a * MU_SRC + sub * MU_COLS + col;
+            if (a >= K) {
+#pragma unroll
+                for (int k = 0; k < 16; k++) y[k * 16 * MU_COLS] = MD_BIAS;
+                continue;
+            }
             const u64 p = pcs[n_q + a].q, half = tab->half[a];
-            if (v.x > half) v.x -= p;
-            if (v.y > half) v.y -= p;
+            const IntRow r{itw + (size_t)(n_q + a) * N16, p, 2 * p};
+            const InvScale& c = scale[n_q + a];
+            u64 x[16];
+#pragma unroll
+            for (int k = 0; k < 16; k++) x[k] = src[(size_t)a * N16 + (16 * sub + k) * 256 + col];
+            bar();                                  // the buffer's last reader
+            inv_cols<MU_COLS>(r, x, sm, col, sub, bar);
+            const u64 n = c.n, ns = c.ns, nw = c.w, nws = c.ws;
+#pragma unroll
+            for (int k = 0; k < 8; k++) {           // as in ntt16_cols_inv
+                const u64 e = x[k], v = x[k + 8], y0 = shoup(e + v, n, ns, p), y1 = shoup(e - v + r.q2, nw, nws, p);
+                y[k * 16 * MU_COLS] = y0 + (y0 > half ? MD_BIAS - p : MD_BIAS);
+                y[(k + 8) * 16 * MU_COLS] = y1 + (y1 > half ? MD_BIAS - p : MD_BIAS);
+            }
         }
-        *reinterpret_cast<ulonglong2*>(smem + at) = v;
-        *reinterpret_cast<double2*>(smd + at) = make_double2(__ll2double_rn((long long)v.x), __ll2double_rn((long long)v.y));
+    } else {
+        for (uint32_t i = tid; i < A * (MU_SRC / 2); i += MD_THREADS) {
+            const uint32_t a = i / (MU_SRC / 2), r = (i / (MU_COLS / 2)) & 255, c = 2 * (i % (MU_COLS / 2)), at = a * MU_SRC + r * MU_COLS + c;
+            ulonglong2 v = make_ulonglong2(MD_BIAS, MD_BIAS);
+            if (a < K) {
+                v = *reinterpret_cast<const ulonglong2*>(src + (size_t)a * N16 + r * 256 + c);
+                const u64 p = pcs[n_q + a].q, half = tab->half[a];
+                v.x += v.x > half ? MD_BIAS - p : MD_BIAS;
+                v.y += v.y > half ? MD_BIAS - p : MD_BIAS;
+            }
+            *reinterpret_cast<ulonglong2*>(smem + at) = v;
+        }
     }
     if (tid == 0) next = 0;
     __syncthreads();
-    const uint32_t group = tid / MU_TARGET_THREADS, gt = tid % MU_TARGET_THREADS, col = gt % MU_COLS, sub = gt / MU_COLS;
-    const GroupBarrier bar{1 + group};
-    u64* sm = smem + 2 * A * MU_SRC + group * COL_SMEM(MU_COLS);
     const u64* ys = smem + sub * MU_COLS + col;
-    const double* yd = smd + sub * MU_COLS + col;
     for (;;) {
         if (gt == 0) taken[group] = atomicAdd(&next, 1u);
         bar();
@@ -239,21 +271,21 @@ __global__ void __launch_bounds__(MD_THREADS, 2)
 #pragma unroll
         for (int k = 0; k < 16; k += 4) {
             u64 v[4];
-            uint32_t cross[4];
+            uint32_t cross[4], msum = 0;
             double s[4];
 #pragma unroll
-            for (int e = 0; e < 4; e++) v[e] = 0, cross[e] = 0, s[e] = FP_MAGIC;
+            for (int e = 0; e < 4; e++) v[e] = 0, cross[e] = 0, s[e] = __ldg(&tab->start[i]);
 #pragma unroll
             for (int a = 0; a < A; a++) {
                 const ulonglong2 t = __ldg(reinterpret_cast<const ulonglong2*>(&tab->term[a][i]));
                 const uint32_t ml = (uint32_t)t.x, mh = (uint32_t)(t.x >> 32);
                 const double mq = __longlong_as_double((long long)t.y);
+                msum += ml;
 #pragma unroll
                 for (int e = 0; e < 4; e++) {
-                    const uint32_t at = a * MU_SRC + (k + e) * 16 * MU_COLS;
-                    const u64 y = ys[at];
+                    const u64 y = ys[a * MU_SRC + (k + e) * 16 * MU_COLS];
                     const uint32_t yl = (uint32_t)y, yh = (uint32_t)(y >> 32);
-                    s[e] = __fma_rn(yd[at], mq, s[e]);
+                    s[e] = __fma_rn(__hiloint2double((int)(0x43300000u + (yh >> 8)), (int)__funnelshift_r(yl, yh, 8)), mq, s[e]);
                     asm("mad.wide.u32 %0, %1, %2, %0;" : "+l"(v[e]) : "r"(yl), "r"(ml));
                     asm("mad.lo.u32 %0, %1, %2, %0;" : "+r"(cross[e]) : "r"(yl), "r"(mh));
                     asm("mad.lo.u32 %0, %1, %2, %0;" : "+r"(cross[e]) : "r"(yh), "r"(ml));
@@ -261,11 +293,10 @@ __global__ void __launch_bounds__(MD_THREADS, 2)
             }
 #pragma unroll
             for (int e = 0; e < 4; e++) {
-                // every rounding of s is to an integer: four terms leave c within 2.1 of the quotient, |v| <= 2.1 2^10 q
                 const u64 c = (u64)__double_as_longlong(s[e]);
                 const uint32_t cl = (uint32_t)c, ch = (uint32_t)(c >> 32) - FP_MAGIC_HI;
                 asm("mad.wide.u32 %0, %1, %2, %0;" : "+l"(v[e]) : "r"(cl), "r"(tl));
-                uint32_t hi = (uint32_t)(v[e] >> 32) + (cross[e] + cl * th + ch * tl);
+                uint32_t hi = (uint32_t)(v[e] >> 32) + (cross[e] + cl * th + ch * tl - (msum << 27));      // the bias times the sum of m
                 // second quotient: the signed high word times 2^32 / q
                 const double d = __dadd_rn(__hiloint2double(0x43300000, (int)(hi ^ 0x80000000u)), -4503601774854144.0);
                 const u64 c2 = (u64)__double_as_longlong(__fma_rn(d, q32, FP_MAGIC));
@@ -292,17 +323,26 @@ bool moddown16_supported(const fesc_ctx* ctx, uint32_t level) {
         if (ctx->q[ctx->n_q + k] >= (1ull << 60)) return false;
     return true;
 }
-template <int A>
+bool moddown16_open(const fesc_ctx* ctx, uint32_t level) {
+    bool open = moddown16_supported(ctx, level);
+    for (uint32_t k = 0; k < ctx->n_p; k++) open = open && ctx->q[ctx->n_q + k] >= FESC_FP_LIMIT;
+    return open;
+}
+template <int A, bool OPEN>
 static int launch_moddown(fesc_ctx* ctx, const u64* acc, u64* u, uint32_t level, uint32_t polys, cudaStream_t st) {
     const uint32_t tiles = 256 / MU_COLS;
-    const size_t smem = ((size_t)2 * A * MU_SRC + MD_GROUPS * COL_SMEM(MU_COLS)) * sizeof(u64);
-    auto kern = k_moddown_cols<A>;
+    const size_t smem = ((size_t)A * MU_SRC + MD_GROUPS * COL_SMEM(MU_COLS)) * sizeof(u64);
+    auto kern = k_moddown_cols<A, OPEN>;
     FESC_CHECK_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     uint32_t splits = 1;
     while (splits < 4 && tiles * polys * splits < 8 * 148) splits++;
-    launch(kern, dim3(tiles * splits, polys), MD_THREADS, smem, st, acc, u, ctx->tabs.d_moddown, ctx->d_twf, ctx->d_pc, level, ctx->n_q, ctx->n_p,
-           splits);
+    launch(kern, dim3(tiles * splits, polys), MD_THREADS, smem, st, acc, u, ctx->tabs.d_moddown, ctx->d_twf, ctx->d_itw, ctx->tabs.d_down_scale, ctx->d_pc,
+           level, ctx->n_q, ctx->n_p, splits);
     return FESC_OK;
+}
+template <int A>
+static int launch_moddown(fesc_ctx* ctx, const u64* acc, u64* u, uint32_t level, uint32_t polys, cudaStream_t st) {
+    return moddown16_open(ctx, level) ? launch_moddown<A, true>(ctx, acc, u, level, polys, st) : launch_moddown<A, false>(ctx, acc, u, level, polys, st);
 }
 int moddown16_cols_launch(fesc_ctx* ctx, const u64* acc, u64* u, uint32_t level, uint32_t polys, cudaStream_t st) {
     if (ctx->n_p <= 1) return launch_moddown<1>(ctx, acc, u, level, polys, st);

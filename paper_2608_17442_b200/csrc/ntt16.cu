@@ -88,7 +88,7 @@ __global__ void __launch_bounds__(COL_THREADS, 1024 / COL_THREADS)
         double x[16];
 #pragma unroll
         for (int k = 0; k < 16; k++) x[k] = FpRow::value(p[(16 * sub + k) * 256]);
-        inv_cols<NTT_COLS>(r, x, sm, col, sub);
+        inv_cols<NTT_COLS>(r, x, sm, col, sub, CtaBarrier());
         const double ninv = scale ? scale[pi].nd : pc.ninvd, ninvw = scale ? scale[pi].wd : pc.ninvwd;
 #pragma unroll
         for (int k = 0; k < 8; k++) {        // last stage, N^-1 folded in
@@ -102,7 +102,7 @@ __global__ void __launch_bounds__(COL_THREADS, 1024 / COL_THREADS)
         u64 x[16];
 #pragma unroll
         for (int k = 0; k < 16; k++) x[k] = p[(16 * sub + k) * 256];
-        inv_cols<NTT_COLS>(r, x, sm, col, sub);
+        inv_cols<NTT_COLS>(r, x, sm, col, sub, CtaBarrier());
         const u64 n = scale ? scale[pi].n : pc.ninv, ns = scale ? scale[pi].ns : pc.ninvs;
         const u64 nw = scale ? scale[pi].w : pc.ninvw, nws = scale ? scale[pi].ws : pc.ninvws;
 #pragma unroll
@@ -321,7 +321,7 @@ static int launch_all(fesc_ctx* ctx, u64* data, size_t rows, const RowMap& map, 
                 if (inverse) {
                     launch(source ? ntt16_rows_inv<ROW_FP, true, WIDE> : ntt16_rows_inv<ROW_FP, false, WIDE>, gr, ROW_THREADS, 0, st, data, ctx->d_itwf, ctx->d_pc, l,
                            y, src);
-                    launch(ntt16_cols_inv<ROW_FP>, gc, COL_THREADS, 0, st, data, ctx->d_itwf, ctx->d_pc, l, y, scale);
+                    if (!skip_cols) launch(ntt16_cols_inv<ROW_FP>, gc, COL_THREADS, 0, st, data, ctx->d_itwf, ctx->d_pc, l, y, scale);
                 } else {
                     if (!skip_cols) launch(ntt16_cols_fwd<ROW_FP>, gc, COL_THREADS, 0, st, data, ctx->d_twf, ctx->d_pc, l, y, in_double, fin.centred, fin.centred_q);
                     if (fin.pt || fin.mul) launch(ntt16_rows_fwd<ROW_FP, 2, WIDE>, gr, ROW_THREADS, 0, st, data, ctx->d_twf, ctx->d_pc, l, y, out_double, fin);
@@ -331,7 +331,7 @@ static int launch_all(fesc_ctx* ctx, u64* data, size_t rows, const RowMap& map, 
             } else if (inverse) {
                 launch(source ? ntt16_rows_inv<ROW_INT, true, WIDE> : ntt16_rows_inv<ROW_INT, false, WIDE>, gr, ROW_THREADS, 0, st, data, ctx->d_itw, ctx->d_pc, l, y,
                        src);
-                launch(ntt16_cols_inv<ROW_INT>, gc, COL_THREADS, 0, st, data, ctx->d_itw, ctx->d_pc, l, y, scale);
+                if (!skip_cols) launch(ntt16_cols_inv<ROW_INT>, gc, COL_THREADS, 0, st, data, ctx->d_itw, ctx->d_pc, l, y, scale);
             } else {
                 if (!skip_cols) launch(ntt16_cols_fwd<ROW_INT>, gc, COL_THREADS, 0, st, data, ctx->d_tw, ctx->d_pc, l, y, 0, nullptr, 0.0);
                 launch(ntt16_rows_fwd<ROW_INT, 0, WIDE>, gr, ROW_THREADS, 0, st, data, ctx->d_tw, ctx->d_pc, l, y, 0, fin);

@@ -212,8 +212,8 @@ __device__ __forceinline__ void fwd_cols(const R& r, typename R::T (&x)[16], u64
     fwd_stage<3>(r, x, i0);
 }
 // Rounds B and A without the last stage.
-template <int COLS, class R>
-__device__ __forceinline__ void inv_cols(const R& r, typename R::T (&x)[16], u64* sm, uint32_t col, uint32_t sub) {
+template <int COLS, class R, class B>
+__device__ __forceinline__ void inv_cols(const R& r, typename R::T (&x)[16], u64* sm, uint32_t col, uint32_t sub, B bar) {
     const uint32_t i0 = 16 + sub;
     inv_stage<3>(r, x, i0);
     inv_stage<2>(r, x, i0);
@@ -223,7 +223,7 @@ __device__ __forceinline__ void inv_cols(const R& r, typename R::T (&x)[16], u64
     u64* s = sm + col_slot<COLS>(16 * sub, col);
 #pragma unroll
     for (int k = 0; k < 16; k++) s[k * COLS] = R::bits(x[k]);
-    __syncthreads();
+    bar();
 #pragma unroll
     for (int k = 0; k < 16; k++) x[k] = R::value(sm[col_slot<COLS>(16 * k, col) + sub * COLS]);
     inv_stage<3>(r, x, 1);

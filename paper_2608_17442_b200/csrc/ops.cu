@@ -958,7 +958,7 @@ static int ks_inner_multi(fesc_ctx* ctx, const KsScratch& ws, const InnerSrcs& S
         launch(k_inner_tma<4>, grid, 256, smem, st, S.s[0].ext, S.s[0].key, ws.acc, ctx->d_pc, N, level, nq, K, alpha, beta,
                                                  batch, ctx->log_n, S.s[0].g, accumulate, n_tiles, ctx->d_status, ctx->log_n == 16);
     } else if (open) {
-        const int rc = rows_inner_launch(ctx, S, ws.acc, level, batch, accumulate, separate, st);
+        const int rc = rows_inner_launch(ctx, S, ws.acc, level, batch, accumulate, separate, last && moddown16_open(ctx, level), st);
         if (rc != FESC_OK) return rc;
         ctx->counters[0] += (uint64_t)batch * S.n * level * (beta - 1);      // transforms that end in the inner product
     } else if (split) {
@@ -1046,7 +1046,8 @@ static int ks_inner_hoisted(fesc_ctx* ctx, const KsScratch& ws, const KsKeys& ke
     return FESC_OK;
 }
 
-// Step 5: division of ws.acc by P; the result is ADDED to out[b][p] when bit p of add_mask is set, else stored.
+// Step 5: division of ws.acc by P; the result is ADDED to out[b][p] when bit p of add_mask is set, else stored.  open: the sums come from
+// ks_inner_multi with `open`.
 // whether the last pass of the forward transform finishes the division (N = 2^16 with every data prime below 2^50, small rings)
 static bool moddown_fused(const fesc_ctx* ctx, uint32_t level) {
     if (small_ring(ctx)) return true;
@@ -1063,7 +1064,7 @@ struct KsRot {
     const u64* g = nullptr;
 };
 static int ks_moddown(fesc_ctx* ctx, const KsScratch& ws, uint32_t level, uint32_t batch, u64* out, size_t out_stride,
-                      int add_mask, cudaStream_t st, const KsRot& rot = KsRot(), uint32_t n_keys = 1, size_t key_stride = 0) {
+                      int add_mask, cudaStream_t st, bool open, const KsRot& rot = KsRot(), uint32_t n_keys = 1, size_t key_stride = 0) {
     if (small_ring(ctx)) return small_moddown(ctx, ws, level, batch, out, out_stride, add_mask, st, rot.src, rot.stride, rot.src ? rot.g[0] : 0);
     const uint32_t polys = batch * n_keys;
     const uint32_t N = ctx->N, K = ctx->n_p, nq = ctx->n_q;
@@ -1074,7 +1075,11 @@ static int ks_moddown(fesc_ctx* ctx, const KsScratch& ws, uint32_t level, uint32
     m.period = rows;
     for (uint32_t t = 0; t < rows; t++) m.prime[t] = t < level ? 0xFF : (uint8_t)(nq + (t - level));
     const bool cols = moddown16_supported(ctx, level);      // the conversion feeds the forward transform's first pass
-    if ((rc = ntt_launch(ctx, ws.acc, (size_t)polys * 2 * rows, m, true, st, false, false, nullptr, cols ? ctx->tabs.d_down_scale : nullptr)) != FESC_OK)
+    if (open && moddown16_open(ctx, level)) {       // the inner product has done the first pass
+        ctx->counters[0] += (uint64_t)polys * 2 * K;
+        ctx->counters[6] += (uint64_t)polys * 2 * K;
+    } else if ((rc = ntt_launch(ctx, ws.acc, (size_t)polys * 2 * rows, m, true, st, false, false, nullptr, cols ? ctx->tabs.d_down_scale : nullptr,
+                                moddown16_open(ctx, level))) != FESC_OK)
         return rc;
     prof_begin(ctx, PF_MODDOWN, st);
     if (cols) {
@@ -1118,7 +1123,7 @@ static int ks_apply(fesc_ctx* ctx, const KsScratch& ws, const EvalKey& key, uint
                     size_t out_stride, int add_mask, cudaStream_t st, u64 g, bool open = false) {
     int rc = ks_inner(ctx, ws, key, level, batch, st, g, 0, open);
     if (rc != FESC_OK) return rc;
-    return ks_moddown(ctx, ws, level, batch, out, out_stride, add_mask, st);
+    return ks_moddown(ctx, ws, level, batch, out, out_stride, add_mask, st, open);
 }
 
 // Hybrid key switch of `batch` polynomials d[b] ([level][N], EVAL, contiguous) with scratch
@@ -1240,7 +1245,7 @@ int rotate_multi_internal(fesc_ctx* ctx, const u64* in, size_t in_stride, size_t
                 if ((rc = ks_inner_multi(ctx, ws, S, level, nb, st, 0, 1, keys.n > 1, open)) != FESC_OK) return rc;
                 KsRot rot;
                 rot.src = ib, rot.stride = in_stride, rot.key_stride = in_key_stride, rot.g = keys.g;
-                rc = ks_moddown(ctx, ws, level, nb, ob, out_stride, accumulate ? 3 : 0, st, rot, keys.n, out_key_stride);
+                rc = ks_moddown(ctx, ws, level, nb, ob, out_stride, accumulate ? 3 : 0, st, open, rot, keys.n, out_key_stride);
             } else {
                 dim3 g((ctx->N + 255) / 256, level, nb);
                 prof_begin(ctx, PF_AUTOM, st);
@@ -1355,7 +1360,7 @@ int giant_sum_deferred_internal(fesc_ctx* ctx, u64* acc, uint32_t n_terms, size_
             }
             if ((rc = ks_inner_multi(ctx, ws, S, level, nb, st, p0 > 1, p0 + np == n_terms, false, open)) != FESC_OK) return rc;
         }
-        int rc = ks_moddown(ctx, ws, level, nb, base, stride, 3, st);
+        int rc = ks_moddown(ctx, ws, level, nb, base, stride, 3, st, open);
         if (rc != FESC_OK) return rc;
     }
     return FESC_OK;
@@ -1387,7 +1392,7 @@ int rotate_hoisted_internal(fesc_ctx* ctx, const u64* in, size_t in_stride, u64*
                 if ((rc = ks_inner_hoisted(ctx, ws, keys, 0, keys.n, level, nb, st)) != FESC_OK) return rc;
                 KsRot rot;
                 rot.src = ib, rot.stride = in_stride, rot.g = keys.g;
-                if ((rc = ks_moddown(ctx, ws, level, nb, ob, out_stride, 0, st, rot, keys.n, key_stride)) != FESC_OK) return rc;
+                if ((rc = ks_moddown(ctx, ws, level, nb, ob, out_stride, 0, st, false, rot, keys.n, key_stride)) != FESC_OK) return rc;
                 continue;
             }
             prof_begin(ctx, PF_AUTOM, st);
@@ -1466,7 +1471,7 @@ int rotate_sum_hoisted_internal(fesc_ctx* ctx, const u64* in, size_t in_stride, 
         S.n = n_keys;
         for (uint32_t k = 0; k < n_keys; k++) S.s[k] = InnerSrc{ws.ext, ctx->keys[key_ids[k]].d_key, gs.g[k]};
         if ((rc = ks_inner_multi(ctx, ws, S, level, nb, st, 0)) != FESC_OK) return rc;
-        if ((rc = ks_moddown(ctx, ws, level, nb, ob, out_stride, 3, st)) != FESC_OK) return rc;
+        if ((rc = ks_moddown(ctx, ws, level, nb, ob, out_stride, 3, st, false)) != FESC_OK) return rc;
     }
     return FESC_OK;
 }

@@ -157,11 +157,14 @@ void moddown_conv_imma_launch(fesc_ctx* ctx, const u64* acc, u64* u, uint32_t le
 bool modup16_supported(const fesc_ctx* ctx, uint32_t level);
 // the same for the division by P: the special rows of acc hold COEFF residues times (P/p_k)^-1
 bool moddown16_supported(const fesc_ctx* ctx, uint32_t level);
+bool moddown16_open(const fesc_ctx* ctx, uint32_t level);      // the special rows arrive without the last pass of their inverse transform
 int moddown16_cols_launch(fesc_ctx* ctx, const u64* acc, u64* u, uint32_t level, uint32_t polys, cudaStream_t st);
 int modup16_cols_launch(fesc_ctx* ctx, const u64* y, u64* ext, uint32_t level, uint32_t batch, cudaStream_t st);
 
 // rows on primes below 2^50: last pass of the forward transform of the converted digits and key inner product in one kernel (inner16.cu)
-int rows_inner_launch(fesc_ctx* ctx, const InnerSrcs& S, u64* acc, uint32_t level, uint32_t batch, int accumulate, bool separate, cudaStream_t st);
+// inv_special: the special rows are left after the first pass of their inverse transform
+int rows_inner_launch(fesc_ctx* ctx, const InnerSrcs& S, u64* acc, uint32_t level, uint32_t batch, int accumulate, bool separate, bool inv_special,
+                      cudaStream_t st);
 
 // rings N = 2^10 .. 2^12 (small.cu): the steps of a key switch and of a rescale, one row per CTA.  small_inner with `last` leaves the
 // special rows of acc in the form small_moddown takes.

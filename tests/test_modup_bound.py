@@ -85,3 +85,30 @@ def test_four_stages_from_the_bound_stay_exact():
         for _ in range(stages):
             start = 1.1875 * start + 0.5
         assert start < 8
+
+
+@pytest.mark.parametrize("bits", [40, 45, 50])
+def test_first_quotient_of_the_division_by_p(bits):
+    """The fused division by P (special primes below 2^60, data primes of 2^40 to 2^50): a source word is centred, offset by 2^59 and seen by the
+    FP64 sum as 2^52 plus its upper 52 bits; the quotient is in units of 2^10.  What it leaves is at most 5.2 2^10 q, which fits a signed word."""
+    g = np.random.default_rng(7)
+    specials = S.ntt_primes(60, 16, 4, 0)
+    P = int(np.prod([int(p) for p in specials], dtype=object))
+    worst = 0.0
+    for q in S.ntt_primes(bits, 16, 3, 0):
+        m = [centred(P // p % q, q) for p in specials]
+        mq = [float(Fraction(v, 4 * q)) for v in m]
+        start = float(Fraction(3, 2) * 2**52 * (1 - sum(map(Fraction, mq))))
+        ys = [[0] * 4, [p - 1 for p in specials], [p // 2 for p in specials], [p // 2 + 1 for p in specials]]
+        ys += [[p // 2 + (w < 0) for p, w in zip(specials, m)], [p // 2 + (w > 0) for p, w in zip(specials, m)]]      # all terms of one sign
+        ys += [[int(g.integers(0, p)) for p in specials] for _ in range(2000)]
+        for y in ys:
+            c = [centred(v, p) for v, p in zip(y, specials)]
+            s = start
+            for v, w in zip(c, mq):
+                s = fma(2.0**52 + ((v + 2**59) >> 8), w, s)
+            assert 2.0**52 <= s < 2.0**53 and s == int(s)
+            v = sum(a * b for a, b in zip(c, m)) - (int(s) - int(MAGIC)) * 2**10 * q
+            worst = max(worst, abs(v) / (2**10 * q))
+            assert abs(v) < 2**63
+    assert worst < 5.2, worst
