@@ -231,8 +231,9 @@ struct ModUpDigit {
     u64 inv[FESC_MAX_ALPHA], invs[FESC_MAX_ALPHA];   // (Q_j/q_i)^-1 mod q_i and its Shoup companion
     u64 mat[FESC_MAX_ALPHA][FESC_MAX_PRIMES];        // (Q_j/q_i) mod q_t, t = prime index
     double matd[FESC_MAX_ALPHA][FESC_MAX_PRIMES];    // the same as doubles (exact for targets below 2^53)
-    ModUpTerm term[FESC_MAX_ALPHA][FESC_MAX_PRIMES]; // the same centred (modup16.cu)
-    double start[FESC_MAX_PRIMES];                   // -2^52 times the sum of a target's mq
+    // the same centred, [0] as they are and [1] times the target's twiddle of the transform's first stage (modup16.cu)
+    ModUpTerm term[2][FESC_MAX_ALPHA][FESC_MAX_PRIMES];
+    double start[2][FESC_MAX_PRIMES];                // -2^52 times the sum of a target's mq
 };
 // Division by P = product of the special primes p_k.
 struct ModDownTab {
@@ -244,8 +245,9 @@ struct ModDownTab {
     u64 pinv[FESC_MAX_PRIMES], pinvs[FESC_MAX_PRIMES];   // P^-1 mod q_i
     double matd[FESC_MAX_SPECIAL][FESC_MAX_PRIMES], mat30d[FESC_MAX_SPECIAL][FESC_MAX_PRIMES];   // as doubles
     double wrapd[FESC_MAX_SPECIAL + 1][FESC_MAX_PRIMES], pinvd[FESC_MAX_PRIMES];
-    ModUpTerm term[4][FESC_MAX_PRIMES];                  // (P/p_k) mod q_i centred, and divided by 4 q_i (modup16.cu)
-    double start[FESC_MAX_PRIMES];                       // 1.5 * 2^52 times (1 - the sum of a target's mq)
+    // (P/p_k) mod q_i, and that times the twiddle of the transform's first stage: centred, and divided by 4 q_i (modup16.cu)
+    ModUpTerm term[2][4][FESC_MAX_PRIMES];
+    double start[2][FESC_MAX_PRIMES];                    // 1.5 * 2^52 times (1 - the sum of a target's mq)
 };
 // Rescale from level l (drops limb l-1); entry index l.
 struct RescaleTab {
@@ -288,6 +290,7 @@ struct fesc_ctx {
     u64 seed;
     std::vector<u64> q;           // host primes
     std::vector<PrimeConst> pc;   // host copy
+    std::vector<u64> w1;          // twiddle of the forward transform's first stage
     PrimeConst* d_pc;             // device [n_primes]
     ulonglong2* d_tw;             // forward twiddles [n_primes][N] (w, shoup); N = 2^16: entries from 4096 on regrouped
                                   // (ntt16_twiddle_slot), here and in the three tables below
@@ -449,8 +452,7 @@ struct NttFinish {
 // rows: number of N-word rows starting at d_data; map gives the prime per row.
 // in_double (forward, N = 2^16 only): rows on primes below 2^50 hold doubles with |x| <= q/2 (bit patterns) written by a
 // basis-conversion kernel instead of canonical words.
-// scale (inverse, N = 2^16 only): per prime index, constants in place of those of the last stage.  skip_cols (N = 2^16 only): without the eight
-// stages of distance 256 and more (forward: they are done; inverse: the consumer does them).
+// scale (inverse, N = 2^16 only): per prime index, constants in place of those of the last stage.  skip_cols (N = 2^16 only): without the eight stages of distance 256 and more (forward: they are done; inverse: the consumer does them).
 // out_double (forward, N = 2^16 only): such rows are left as doubles with |x| <= q/2 for a consumer that computes in FP64.
 int ntt_launch(fesc_ctx* ctx, u64* d_data, size_t rows, const RowMap& map, bool inverse, cudaStream_t st,
                bool in_double = false, bool out_double = false, const NttFinish* finish = nullptr,

@@ -325,6 +325,13 @@ static InvScale inv_scale(const PrimeConst& pc, u64 f) {
     s.nd = centred(s.n), s.wd = centred(s.w);
     return s;
 }
+// m modulo q centred, and that divided by `unit` q
+static ModUpTerm centred_term(u64 m, u64 q, int unit) {
+    ModUpTerm t;
+    t.m = m > q / 2 ? -(long long)(q - m) : (long long)m;
+    t.mq = (double)((long double)t.m / ((long double)q * unit));
+    return t;
+}
 static int build_tables(fesc_ctx* ctx) {
     const uint32_t nq = ctx->n_q, np = ctx->n_primes, K = ctx->n_p, alpha = ctx->alpha;
     const std::vector<u64>& q = ctx->q;
@@ -348,18 +355,18 @@ static int build_tables(fesc_ctx* ctx) {
                         if (b != a) m = h_mul(m, q[d.first + b] % q[t], q[t]);
                     d.mat[a][t] = m;
                     d.matd[a][t] = (double)m;
-                    d.term[a][t].m = m > q[t] / 2 ? -(long long)(q[t] - m) : (long long)m;
-                    d.term[a][t].mq = (double)((long double)d.term[a][t].m / (long double)q[t]);
+                    for (int w = 0; w < 2; w++) d.term[w][a][t] = centred_term(w ? h_mul(m, ctx->w1[t], q[t]) : m, q[t], 1);
                 }
                 d.inv[a] = h_inv(d.mat[a][i], q[i]);
                 d.invs[a] = h_shoup(d.inv[a], q[i]);
                 scale[(size_t)(level - 1) * nq + i] = inv_scale(ctx->pc[i], d.inv[a]);
             }
-            for (uint32_t t = 0; t < np; t++) {        // rounded once: the sum of doubles below 1 fits 64 bits but for 2^-63
-                long double mq = 0;
-                for (uint32_t a = 0; a < d.n_src; a++) mq += (long double)d.term[a][t].mq;
-                d.start[t] = (double)(-4503599627370496.0L * mq);
-            }
+            for (uint32_t t = 0; t < np; t++)          // rounded once: the sum of doubles below 1 fits 64 bits but for 2^-63
+                for (int w = 0; w < 2; w++) {
+                    long double mq = 0;
+                    for (uint32_t a = 0; a < d.n_src; a++) mq += (long double)d.term[w][a][t].mq;
+                    d.start[w][t] = (double)(-4503599627370496.0L * mq);
+                }
         }
     }
     if ((rc = upload(ctx, &ctx->tabs.d_up_scale, scale)) != FESC_OK) return rc;
@@ -384,10 +391,7 @@ static int build_tables(fesc_ctx* ctx) {
             md.mat[k][i] = m;
             md.mat30[k][i] = h_mul(m, (1ull << 30) % q[i], q[i]);
             md.matd[k][i] = (double)md.mat[k][i];
-            if (k < 4) {
-                md.term[k][i].m = m > q[i] / 2 ? -(long long)(q[i] - m) : (long long)m;
-                md.term[k][i].mq = (double)((long double)md.term[k][i].m / ((long double)q[i] * 4));
-            }
+            for (int w = 0; w < 2 && k < 4; w++) md.term[w][k][i] = centred_term(w ? h_mul(m, ctx->w1[i], q[i]) : m, q[i], 4);
             md.mat30d[k][i] = (double)md.mat30[k][i];
         }
     }
@@ -395,9 +399,11 @@ static int build_tables(fesc_ctx* ctx) {
         u64 P = 1;
         for (uint32_t b = 0; b < K; b++) P = h_mul(P, q[nq + b] % q[i], q[i]);
         Pmod[i] = P;
-        long double mq = 0;
-        for (uint32_t k = 0; k < K && k < 4; k++) mq += (long double)md.term[k][i].mq;
-        md.start[i] = (double)(0x1.8p52L * (1 - mq));
+        for (int w = 0; w < 2; w++) {
+            long double mq = 0;
+            for (uint32_t k = 0; k < K && k < 4; k++) mq += (long double)md.term[w][k][i].mq;
+            md.start[w][i] = (double)(0x1.8p52L * (1 - mq));
+        }
         md.pinv[i] = h_inv(P, q[i]);
         md.pinvs[i] = h_shoup(md.pinv[i], q[i]);
         for (uint32_t c = 0; c <= K; c++) md.wrap[c][i] = h_mul(c, P, q[i]);
@@ -577,6 +583,7 @@ extern "C" int fesc_ctx_create(fesc_ctx** out, uint32_t log_n, const uint64_t* p
         pc.ninvd = (double)pc.ninv;
         pc.ninvwd = (double)pc.ninvw;
         ctx->pc.push_back(pc);
+        ctx->w1.push_back(pw[h_brev(1, log_n)]);
     }
     if ((rc = upload(ctx, &ctx->d_pc, ctx->pc)) != FESC_OK) return bail(rc);
     if ((rc = upload(ctx, &ctx->d_tw, tw)) != FESC_OK) return bail(rc);

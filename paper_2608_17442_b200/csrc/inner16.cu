@@ -155,7 +155,7 @@ __global__ void __launch_bounds__(32 * RI_WARPS, 4)
             f1[2 * k] = fp_load(v1.x, q), f1[2 * k + 1] = fp_load(v1.y, q);
         }
     }
-    uint32_t s = s0, j = 0, room = accumulate || beta > 6 ? 5 : 6;
+    uint32_t s = s0, j = 0, room = accumulate || beta > 5 ? 4 : 5;
 #pragma unroll 1
     for (uint32_t n = 0; n < total; n++) {
         const uint32_t s_next = j + 1 < beta ? s : s + 1, j_next = j + 1 < beta ? j + 1 : 0;
@@ -171,7 +171,7 @@ __global__ void __launch_bounds__(32 * RI_WARPS, 4)
             for (int k = 0; k < 16; k++) x[k] = FpRow::value(in[16 * k]);
             __syncwarp();                               // the staged points and the previous digit's values have been read
             if (lane == 0 && n + 1 < total) load_x(s_next, j_next);
-            fwd_rows(r, x, sm, blk, lane);
+            fwd_rows<false>(r, x, sm, blk, lane);
         }
         if (mbar_wait_bounded(key_full, n & 1)) {
             if (lane == 0) atomicExch(status, 5u);
@@ -198,12 +198,12 @@ __global__ void __launch_bounds__(32 * RI_WARPS, 4)
             }
         }
         s = s_next, j = j_next;
-        // A transformed point stays below 4.82 q (five stages from q/2), its product below 1.41 q, an own digit's below 0.6 q: five products and
-        // a rest of q/2 stay below 8 q, and so do six that start from zero and have an own one among them (a source of up to six digits)
+        // A transformed point stays below 6.75 q, its product below 1.77 q, an own digit's below 0.6 q: four products and a rest of q/2 stay below
+        // 8 q, and so do five that start from zero and have an own one among them (a source of up to five digits, or any first four)
         if (--room == 0 && n + 1 < total) {
             fold16(r, f0);
             fold16(r, f1);
-            room = 5;
+            room = 4;
         }
     }
 #pragma unroll

@@ -12,11 +12,14 @@
 // A CTA owns 4 columns of one digit of one ciphertext: the source columns (8 KB per limb) are read once into shared memory
 // and serve all targets; six groups of 64 threads take targets from a counter, the slower rows on the 60-bit primes first.
 //
+// The first stage of the transform has one twiddle, so the constants of the lower half of the points carry it: those words are converted to
+// their product, and the stage is additions only.
+//
 // What bounds it: the dispatch of wide operands (an FP64 multiply-add of three registers holds its port for three cycles), which
 // conversion and butterflies share; 0.38 us per converted row at 24 limbs and 16 ciphertexts against 0.41 for a conversion kernel
-// and a first pass of their own, and 1.2 GB less traffic per launch.  8 columns with 8 groups 0.39; four exact FP64 products
-// per word instead of the mixed sum 0.53 (the rounding unit takes nine cycles per product); byte planes on the tensor cores,
-// eight targets at a time through shared memory, 0.45; the same for the division by P 0.51 against 0.36 unfused.
+// and a first pass of their own, and 1.2 GB less traffic per launch.  8 columns with 6 groups 0.38, division by P 0.39 against 0.33 ms; four exact
+// FP64 products per word instead of the mixed sum 0.53 (the rounding unit takes nine cycles per product); byte planes on the tensor
+// cores, eight targets at a time through shared memory, 0.45; the same for the division by P 0.51 against 0.36 unfused.
 #define FESC_DBG_FILE 12   // file id in the sites a debug build reports
 #include "ntt16.cuh"
 #include "ops.cuh"
@@ -35,24 +38,16 @@ struct GroupBarrier {
 #define FP_MAGIC 6755399441055744.0      // 1.5 * 2^52: the low mantissa bits of FP_MAGIC + c hold the integer c, |c| < 2^51
 #define FP_MAGIC_HI 0x43380000u
 
-// the integer v, |v| < 2^53, whose high word has 2^31 added to it.  (One addition to 1.5 * 2^52 would do for |v| < 2^51 only, which is 2 q
-// at 50 bits.  The second one is not seen in the times: 32 rotations by 4 keys at 24 limbs 21.99 ms with one, 21.93 with two.)
-__device__ __forceinline__ double wide_to_double(u64 v) {
-    const double h = __dadd_rn(__hiloint2double(0x45300000, (int)(v >> 32)), -0x1.00000801p84);      // 2^84 + 2^63 + 2^52
-    return __dadd_rn(h, __hiloint2double(0x43300000, (int)(uint32_t)v));
-}
-
 // v[0..3] = sum_a y_a m_a - c q (two's complement) for the points p, p + 16 MU_COLS, ... of the source columns.  The columns hold
 // the doubles 2^52 + y, whose low 50 bits are y: one word serves both pipes without a conversion.  What 2^52 adds to the FP64 sum is
-// in its starting value c0, what the exponent bits add to the cross products (weight 2^32, modulo 2^32) is taken off at the end;
-// `bias` is added to the high word.
+// in its starting value c0, what the exponent bits add to the cross products (weight 2^32, modulo 2^32) is taken off at the end.
 // How far c is from the quotient, for any four primes below 2^50 (|m / q| <= 1/2, y < 2^50): the running sum starts at -2^52 sum(m / q)
 // and loses 2^52 m / q with every term, so it is below 2^53, 2^53, 2^52 + 2^50, 2^52 and 2^51 in turn and the roundings (of the start and of
 // four multiply-adds) are at most 1/2, 1/2, 1/2, 1/4 and 1/8; m / q as a double is off by 2^-55 at most, 1/32 per term after the product
 // with y (what 2^52 makes of it is in c0, which is formed from the same doubles); the quotient rounds by 1/2.  Together 2.5.
 template <int A>
 __device__ __forceinline__ void convert4(const u64* p, uint32_t n_src, const ModUpTerm (*__restrict__ term)[FESC_MAX_PRIMES], uint32_t pt,
-                                         double c0, u64 q, uint32_t bias, u64* v) {
+                                         double c0, u64 q, u64* v) {
     u64 acc[4];            // low product words, and the cross terms of weight 2^32 apart from them
     uint32_t cross[4], msum = 0;
     double s[4];
@@ -76,11 +71,11 @@ __device__ __forceinline__ void convert4(const u64* p, uint32_t n_src, const Mod
         }
     }
     const u64 nq = 0 - q;
-    const uint32_t ql = (uint32_t)nq, qh = (uint32_t)(nq >> 32), corr = bias - 0x43300000u * msum;
+    const uint32_t ql = (uint32_t)nq, qh = (uint32_t)(nq >> 32), corr = 0u - 0x43300000u * msum - FP_MAGIC_HI * ql;      // the exponent bits of y and c
 #pragma unroll
     for (int e = 0; e < 4; e++) {
         const u64 c = (u64)__double_as_longlong(__dadd_rn(s[e], FP_MAGIC));
-        const uint32_t cl = (uint32_t)c, ch = (uint32_t)(c >> 32) - FP_MAGIC_HI;
+        const uint32_t cl = (uint32_t)c, ch = (uint32_t)(c >> 32);
         asm("mad.wide.u32 %0, %1, %2, %0;" : "+l"(acc[e]) : "r"(cl), "r"(ql));
         const uint32_t hi = (uint32_t)(acc[e] >> 32) + (cross[e] + corr + cl * qh + ch * ql);
         v[e] = ((u64)hi << 32) | (uint32_t)acc[e];
@@ -94,7 +89,7 @@ __global__ void __launch_bounds__(MU_THREADS, 2)
                  uint32_t beta, uint32_t splits) {
     pdl_begin();
     extern __shared__ __align__(16) u64 smem[];      // [A][MU_SRC] source columns, then one exchange buffer per group
-    __shared__ uint32_t next, taken[MU_GROUPS];
+    __shared__ uint32_t next, taken[2][MU_GROUPS];
     const uint32_t tid = threadIdx.x, tile = blockIdx.x / splits, part = blockIdx.x % splits, j = blockIdx.y, b = blockIdx.z;
     const ModUpDigit* dg = tab + j;
     const uint32_t first = dg->first, n_src = dg->n_src, rows = level + K, others = rows - n_src;
@@ -115,39 +110,41 @@ __global__ void __launch_bounds__(MU_THREADS, 2)
     const GroupBarrier bar{1 + group};
     u64* sm = smem + A * MU_SRC + group * COL_SMEM(MU_COLS);
     const u64* ys = smem + sub * MU_COLS + col;
-    for (;;) {
-        if (gt == 0) taken[group] = atomicAdd(&next, 1u);
-        bar();
-        const uint32_t o = taken[group] * splits + part;      // (the exchange's barrier keeps the next write behind this read)
+    if (gt == 0) taken[0][group] = atomicAdd(&next, 1u);
+    bar();
+    // the next target is taken while this one is worked on; the exchange's barrier publishes it.  (A barrier before the exchange and not
+    // at the head of the loop: a group's two warps may be half a target apart.)
+    for (uint32_t slot = 0;; slot ^= 1) {
+        const uint32_t o = taken[slot][group] * splits + part;
         if (o >= others) return;
+        if (gt == 0) taken[slot ^ 1][group] = atomicAdd(&next, 1u);
         const uint32_t d = o < K ? 0 : o - K;
         const uint32_t t = o < K ? level + o : (d < first ? d : d + n_src), pt = o < K ? n_q + o : t;
         u64* p = out + (size_t)t * N16 + col;
         const u64 q = pcs[pt].q;
-        const double c0 = __ldg(&dg->start[pt]);
         if (q < FESC_FP_LIMIT) {
             FpRow r{twf + (size_t)pt * N16, pcs[pt].qd, pcs[pt].qinvd};
             double x[16];
 #pragma unroll
             for (int k = 0; k < 16; k += 4) {
                 u64 v[4];
-                convert4<A>(ys + k * 16 * MU_COLS, n_src, dg->term, pt, c0, q, 0x80000000u, v);
+                convert4<A>(ys + k * 16 * MU_COLS, n_src, dg->term[k / 8], pt, __ldg(&dg->start[k / 8][pt]), q, v);
 #pragma unroll
-                for (int e = 0; e < 4; e++) x[k + e] = wide_to_double(v[e]);       // |v| <= 2.51 q, within the 2.69 q fwd_cols takes
+                for (int e = 0; e < 4; e++) x[k + e] = __ll2double_rn((long long)v[e]);       // |v| <= 2.51 q, as COLS_MODUP takes them
             }
-            fwd_cols<MU_COLS>(r, x, sm, col, sub, bar);
+            fwd_cols<MU_COLS, COLS_MODUP>(r, x, sm, col, sub, bar);
 #pragma unroll
             for (int k = 0; k < 16; k++) p[(16 * sub + k) * 256] = FpRow::bits(x[k]);
         } else {
-            IntRow r{tw + (size_t)pt * N16, q, 2 * q};
+            const IntRow r{tw + (size_t)pt * N16, q, 2 * q};
             u64 x[16];
 #pragma unroll
             for (int k = 0; k < 16; k += 4) {
-                convert4<A>(ys + k * 16 * MU_COLS, n_src, dg->term, pt, c0, q, 0u, x + k);
+                convert4<A>(ys + k * 16 * MU_COLS, n_src, dg->term[k / 8], pt, __ldg(&dg->start[k / 8][pt]), q, x + k);
 #pragma unroll
                 for (int e = 0; e < 4; e++) x[k + e] = csub(x[k + e] + 3 * q, r.q2);      // |v| <= 2.51 q: below 4q
             }
-            fwd_cols<MU_COLS>(r, x, sm, col, sub, bar);
+            fwd_cols<MU_COLS, COLS_MODUP>(r, x, sm, col, sub, bar);
 #pragma unroll
             for (int k = 0; k < 16; k++) p[(16 * sub + k) * 256] = x[k];
         }
@@ -208,7 +205,7 @@ __global__ void __launch_bounds__(MD_THREADS, 2)
                    const ulonglong2* __restrict__ itw, const InvScale* __restrict__ scale, const PrimeConst* __restrict__ pcs, uint32_t level, uint32_t n_q, uint32_t K, uint32_t splits) {
     pdl_begin();
     extern __shared__ __align__(16) u64 smem[];      // [A][MU_SRC] sources, then one exchange buffer per group
-    __shared__ uint32_t next, taken[MD_GROUPS];
+    __shared__ uint32_t next, taken[2][MD_GROUPS];
     const uint32_t tid = threadIdx.x, tile = blockIdx.x / splits, part = blockIdx.x % splits, bp = blockIdx.y;
     const u64* src = acc + ((size_t)bp * (level + K) + level) * N16 + tile * MU_COLS;
     u64* out = u + (size_t)bp * level * N16 + tile * MU_COLS;
@@ -258,14 +255,16 @@ __global__ void __launch_bounds__(MD_THREADS, 2)
     if (tid == 0) next = 0;
     __syncthreads();
     const u64* ys = smem + sub * MU_COLS + col;
-    for (;;) {
-        if (gt == 0) taken[group] = atomicAdd(&next, 1u);
-        bar();
-        const uint32_t i = taken[group] * splits + part;
+    if (gt == 0) taken[0][group] = atomicAdd(&next, 1u);
+    bar();
+    for (uint32_t slot = 0;; slot ^= 1) {
+        const uint32_t i = taken[slot][group] * splits + part;
         if (i >= level) return;
+        if (gt == 0) taken[slot ^ 1][group] = atomicAdd(&next, 1u);
         const FpRow r{twf + (size_t)i * N16, pcs[i].qd, pcs[i].qinvd};
         const u64 nq = 0 - pcs[i].q, nq10 = nq << 10;
         const uint32_t ql = (uint32_t)nq, qh = (uint32_t)(nq >> 32), tl = (uint32_t)nq10, th = (uint32_t)(nq10 >> 32);
+        const uint32_t corr2 = 0u - FP_MAGIC_HI * ql;
         const double q32 = 4294967296.0 * r.qinv;
         double x[16];
 #pragma unroll
@@ -274,10 +273,10 @@ __global__ void __launch_bounds__(MD_THREADS, 2)
             uint32_t cross[4], msum = 0;
             double s[4];
 #pragma unroll
-            for (int e = 0; e < 4; e++) v[e] = 0, cross[e] = 0, s[e] = __ldg(&tab->start[i]);
+            for (int e = 0; e < 4; e++) v[e] = 0, cross[e] = 0, s[e] = __ldg(&tab->start[k / 8][i]);
 #pragma unroll
             for (int a = 0; a < A; a++) {
-                const ulonglong2 t = __ldg(reinterpret_cast<const ulonglong2*>(&tab->term[a][i]));
+                const ulonglong2 t = __ldg(reinterpret_cast<const ulonglong2*>(&tab->term[k / 8][a][i]));
                 const uint32_t ml = (uint32_t)t.x, mh = (uint32_t)(t.x >> 32);
                 const double mq = __longlong_as_double((long long)t.y);
                 msum += ml;
@@ -293,21 +292,22 @@ __global__ void __launch_bounds__(MD_THREADS, 2)
             }
 #pragma unroll
             for (int e = 0; e < 4; e++) {
+                const uint32_t corr = 0u - (msum << 27) - FP_MAGIC_HI * tl;      // the bias times the sum of m; the exponent bits of c
                 const u64 c = (u64)__double_as_longlong(s[e]);
-                const uint32_t cl = (uint32_t)c, ch = (uint32_t)(c >> 32) - FP_MAGIC_HI;
+                const uint32_t cl = (uint32_t)c, ch = (uint32_t)(c >> 32);
                 asm("mad.wide.u32 %0, %1, %2, %0;" : "+l"(v[e]) : "r"(cl), "r"(tl));
-                uint32_t hi = (uint32_t)(v[e] >> 32) + (cross[e] + cl * th + ch * tl - (msum << 27));      // the bias times the sum of m
+                uint32_t hi = (uint32_t)(v[e] >> 32) + (cross[e] + cl * th + ch * tl + corr);
                 // second quotient: the signed high word times 2^32 / q
-                const double d = __dadd_rn(__hiloint2double(0x43300000, (int)(hi ^ 0x80000000u)), -4503601774854144.0);
+                const double d = __int2double_rn((int)hi);
                 const u64 c2 = (u64)__double_as_longlong(__fma_rn(d, q32, FP_MAGIC));
-                const uint32_t dl = (uint32_t)c2, dh = (uint32_t)(c2 >> 32) - FP_MAGIC_HI;
+                const uint32_t dl = (uint32_t)c2, dh = (uint32_t)(c2 >> 32);
                 u64 w = ((u64)hi << 32) | (uint32_t)v[e];
                 asm("mad.wide.u32 %0, %1, %2, %0;" : "+l"(w) : "r"(dl), "r"(ql));
-                hi = (uint32_t)(w >> 32) + (dl * qh + dh * ql);
-                x[k + e] = __dadd_rn(__hiloint2double((int)(hi + FP_MAGIC_HI), (int)(uint32_t)w), -FP_MAGIC);
+                hi = (uint32_t)(w >> 32) + (dl * qh + dh * ql + corr2);
+                x[k + e] = __ll2double_rn((long long)((u64)hi << 32 | (uint32_t)w));
             }
         }
-        fwd_cols<MU_COLS>(r, x, sm, col, sub, bar);
+        fwd_cols<MU_COLS, COLS_MODDOWN>(r, x, sm, col, sub, bar);
         u64* p = out + (size_t)i * N16 + col;
 #pragma unroll
         for (int k = 0; k < 16; k++) p[(16 * sub + k) * 256] = FpRow::bits(x[k]);

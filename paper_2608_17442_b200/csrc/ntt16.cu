@@ -56,16 +56,16 @@ __global__ void __launch_bounds__(COL_THREADS, 1024 / COL_THREADS)
                 x[k] = in_double ? FpRow::value(v) : fp_from_u64(v);
             }
         }
-        fwd_cols<NTT_COLS>(r, x, sm, col, sub, CtaBarrier());
+        fwd_cols<NTT_COLS, COLS_WORDS>(r, x, sm, col, sub, CtaBarrier());
 #pragma unroll
-        for (int k = 0; k < 16; k++) p[(16 * sub + k) * 256] = FpRow::bits(x[k]);      // doubles below 3.7q
+        for (int k = 0; k < 16; k++) p[(16 * sub + k) * 256] = FpRow::bits(x[k]);      // doubles below 3.4q
     } else {
         const u64 q = pcs[pi].q;
         const IntRow r{(const ulonglong2*)tw + (size_t)pi * N16, q, 2 * q};
         u64 x[16];
 #pragma unroll
         for (int k = 0; k < 16; k++) x[k] = p[(16 * k + sub) * 256];
-        fwd_cols<NTT_COLS>(r, x, sm, col, sub, CtaBarrier());
+        fwd_cols<NTT_COLS, COLS_WORDS>(r, x, sm, col, sub, CtaBarrier());
 #pragma unroll
         for (int k = 0; k < 16; k++) p[(16 * sub + k) * 256] = x[k];                   // below 4q
     }
@@ -84,7 +84,7 @@ __global__ void __launch_bounds__(COL_THREADS, 1024 / COL_THREADS)
     u64* p = data + (size_t)row * N16 + blockIdx.x * NTT_COLS + col;
     const PrimeConst& pc = pcs[pi];
     if constexpr (A == ROW_FP) {
-        FpRow r{(const double*)tw + (size_t)pi * N16, pc.qd, pc.qinvd};
+        FpRow r{(const double*)tw + (size_t)pi * N16, pcs[pi].qd, pcs[pi].qinvd};
         double x[16];
 #pragma unroll
         for (int k = 0; k < 16; k++) x[k] = FpRow::value(p[(16 * sub + k) * 256]);
@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
                 prefetch_l2(fin.rot_src + k * fin.rot_key_stride + b * fin.rot_stride + (size_t)i * N16 +
                             (galois_src(blk * 512, 16, fin.rot_g[k]) & ~511u) + 16 * lane);
         }
-        fwd_rows(r, x, sm, blk, lane);
+        fwd_rows<FIN != 0>(r, x, sm, blk, lane);
         const double q = r.q, qinv = r.qinv;
         if (!FIN) {
 #pragma unroll
@@ -154,8 +154,8 @@ __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
             }
             return;
         }
-        // (acc - u) c (+ sigma_g(c0)) (+ what the output holds); |acc - u| stays below 5.4q, the lazy product below 1.6q, so
-        // every sum is exact.  Rows of the buffer: row = bp * level + i.
+        // (acc - u) c (+ sigma_g(c0)) (+ what the output holds); |acc - u| stays below 3.1q, the lazy product below 1.7q, the sum below 3.7q, so
+        // every sum is exact and the words need not be centred first.  Rows of the buffer: row = bp * level + i.
         const uint32_t bp = row / fin.level, i = row - bp * fin.level, ct = bp >> 1, pol = bp & 1, kk = ct / fin.nb, b = ct - kk * fin.nb;
         const u64* acc = fin.acc + (size_t)ct * fin.acc_stride + ((size_t)pol * fin.acc_rows + i) * N16;
         u64* out = fin.out + kk * fin.out_key_stride + b * fin.out_stride + ((size_t)pol * fin.level + i) * N16;
@@ -181,7 +181,7 @@ __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
 #pragma unroll
             for (int j = h; j < h + 4; j++) {
                 const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(s + 72 * j);
-                double a0 = fp_load(av[j].x, q), a1 = fp_load(av[j].y, q);
+                double a0 = fp_from_u64(av[j].x), a1 = fp_from_u64(av[j].y);
                 if (FIN == 2) {             // lazy products below 0.7 q
                     const ulonglong2 w2 = pt ? ld_pair<WIDE>(pt + 64 * j) : make_ulonglong2(0, 0);
                     a0 = fp_modmul(a0, pt ? fp_from_u64(w2.x) : mul, q, qinv);
@@ -190,14 +190,14 @@ __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
                 double s0 = fp_modmul(a0 - FpRow::value(v.x), cinv, q, qinv);
                 double s1 = fp_modmul(a1 - FpRow::value(v.y), cinv, q, qinv);
                 if (FIN == 1 && rot) {
-                    s0 += fp_load(w[j - h].x, q);
-                    s1 += fp_load(w[j - h].y, q);
+                    s0 += fp_from_u64(w[j - h].x);
+                    s1 += fp_from_u64(w[j - h].y);
                 }
                 u64* o = out + blk * 512 + 2 * lane + 64 * j;
                 if (FIN == 1 && add) {
                     const ulonglong2 ov = ld_pair<WIDE>(o);
-                    s0 += fp_load(ov.x, q);
-                    s1 += fp_load(ov.y, q);
+                    s0 += fp_from_u64(ov.x);
+                    s1 += fp_from_u64(ov.y);
                 }
                 st_pair<WIDE>(o, make_ulonglong2(fp_store(s0, q, qinv), fp_store(s1, q, qinv)));
             }
@@ -208,7 +208,7 @@ __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
         u64 x[16];
 #pragma unroll
         for (int k = 0; k < 16; k++) x[k] = in[16 * k];
-        fwd_rows(r, x, sm, blk, lane);
+        fwd_rows<false>(r, x, sm, blk, lane);
 #pragma unroll
         for (int j = 0; j < 8; j++) {
             const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(s + 72 * j);

@@ -27,10 +27,13 @@ __device__ __forceinline__ uint32_t pad16(uint32_t e) { return e + 2 * (e >> 4);
 // ---------------------------------------------------------------------------------------
 // Arithmetic of a row.  w(i): twiddle i of the row's table.
 // FpRow: primes below 2^50, exact products on the FP64 pipe.  |product| <= (1/2 + 1.5 |y| 2^-53) q with centred twiddles,
-// so a forward stage takes a bound B q to (1.1875 B + 1/2) q: four stages from 2.69 q and seven from q/2 stay below 8 q,
-// and everything below 8 q < 2^53 is exact.  Forward rows are folded back to q/2 twice (after four and after eleven
-// stages; the first bound leaves room for a conversion's lazy sum at the input); an inverse stage doubles the bound, so four stages from q/2 end at 8 q and every inverse
-// round folds back.
+// so a forward stage takes a bound B q to (1.1875 B + 1/2) q, and everything below 8 q < 2^53 is exact.  Where a bound would pass that, a stage
+// folds the addends of its butterflies (half the points; the products reduce themselves) and leaves (1 + 0.1875 B) q.  Column pass of
+// canonical words or words up to q: six stages to 7.62 q, folded at the seventh, 3.39 q; of converted words up to 2.51 q whose first stage has
+// no products: 5.02, 6.47, folded at the third 2.22, 7.04 after the seventh, folded at the eighth 2.32 q; of words up to 0.7 q from the division by P
+// likewise: 6.94 after the sixth, folded at the seventh, 3.24 q.  Row pass: 7.47 q at most after three stages, folded at the fourth 2.40, and
+// 7.41 q at the end, or 2.10 q where the last stage folds as well.  An inverse stage doubles the bound, so four stages from q/2 end at 8 q and every
+// inverse round folds back.
 // IntRow: any prime below 2^62, lazy Shoup butterflies, values below 4q (forward) or 2q (inverse).
 // ---------------------------------------------------------------------------------------
 // SHARED: the twiddle table is a copy in shared memory.
@@ -45,6 +48,11 @@ struct FpRowT {
     double q, qinv;
     __device__ __forceinline__ void ct(T& x, T& y, double w) const {
         const double v = fp_modmul(y, w, q, qinv), u = x;
+        x = u + v;
+        y = u - v;
+    }
+    __device__ __forceinline__ void sums(T& x, T& y) const {       // a butterfly whose product is done
+        const double u = x, v = y;
         x = u + v;
         y = u - v;
     }
@@ -97,6 +105,11 @@ struct IntRowT {
         x = u + v;
         y = u - v + q2;
     }
+    __device__ __forceinline__ void sums(T& x, T& y) const {       // a butterfly whose product is done
+        const u64 u = csub(x, q2), v = csub(y, q2);
+        x = u + v;
+        y = u - v + q2;
+    }
     __device__ __forceinline__ void gs(T& x, T& y, const W& w) const {
         const u64 u = x, v = y;
         x = csub(u + v, q2);
@@ -123,8 +136,9 @@ typedef IntRowT<false> IntRow;
 // arithmetic of a launch's rows
 enum { ROW_FP = 0, ROW_INT = 1 };
 
-// Stage S (0..3) of a forward round: distance 8 >> S, twiddles (i0 << S) + j for the j-th group of 16 >> S registers.
-template <int S, class R>
+// Stage S (0..3) of a forward round: distance 8 >> S, twiddles (i0 << S) + j for the j-th group of 16 >> S registers.  FOLD: the addends are
+// folded first.
+template <int S, bool FOLD = false, class R>
 __device__ __forceinline__ void fwd_stage(const R& r, typename R::T (&x)[16], uint32_t i0) {
     typename R::W w[8];
     r.template load<S>(w, i0 << S);
@@ -132,6 +146,7 @@ __device__ __forceinline__ void fwd_stage(const R& r, typename R::T (&x)[16], ui
 #pragma unroll
     for (int k = 0; k < 8; k++) {
         const int i = (k / d) * 2 * d + k % d;
+        if (FOLD) x[i] = r.fold(x[i]);
         r.ct(x[i], x[i + d], w[k / d]);
     }
 }
@@ -148,7 +163,7 @@ __device__ __forceinline__ void inv_stage(const R& r, typename R::T (&x)[16], ui
 }
 // The same with the twiddles of round D: those of a 512-point block lie together, regrouped so that a warp's loads are
 // contiguous (ntt16_twiddle_slot).
-template <int S, class R>
+template <int S, bool FOLD = false, class R>
 __device__ __forceinline__ void fwd_stage_d(const R& r, typename R::T (&x)[16], uint32_t blk, uint32_t lane) {
     typename R::W w[8];
     r.template load_d<S>(w, blk, lane);
@@ -156,6 +171,7 @@ __device__ __forceinline__ void fwd_stage_d(const R& r, typename R::T (&x)[16], 
 #pragma unroll
     for (int k = 0; k < 8; k++) {
         const int i = (k / d) * 2 * d + k % d;
+        if (FOLD) x[i] = r.fold(x[i]);
         r.ct(x[i], x[i + d], w[k / d]);
     }
 }
@@ -191,14 +207,22 @@ struct SmallTables {
 struct CtaBarrier {
     __device__ __forceinline__ void operator()() const { __syncthreads(); }
 };
+// What a column pass starts from: words up to q; converted words; words of the division by P.  The last two come with the products of the
+// first stage done (their constants carry its twiddle) and share an exchange buffer that has been used before.
+enum { COLS_WORDS, COLS_MODUP, COLS_MODDOWN };
 // Rounds A and B on the registers of one thread (column, sub = 0..15); bar: barrier of the threads that share the columns.
-template <int COLS, class R, class B>
+template <int COLS, int FROM, class R, class B>
 __device__ __forceinline__ void fwd_cols(const R& r, typename R::T (&x)[16], u64* sm, uint32_t col, uint32_t sub, B bar) {
-    fwd_stage<0>(r, x, 1);
+    if (FROM == COLS_WORDS) {
+        fwd_stage<0>(r, x, 1);
+    } else {
+#pragma unroll
+        for (int k = 0; k < 8; k++) r.sums(x[k], x[k + 8]);
+    }
     fwd_stage<1>(r, x, 1);
-    fwd_stage<2>(r, x, 1);
+    fwd_stage<2, FROM == COLS_MODUP>(r, x, 1);
     fwd_stage<3>(r, x, 1);
-    fold16(r, x);
+    if (FROM != COLS_WORDS) bar();
 #pragma unroll
     for (int k = 0; k < 16; k++) sm[col_slot<COLS>(16 * k, col) + sub * COLS] = R::bits(x[k]);
     bar();
@@ -208,8 +232,8 @@ __device__ __forceinline__ void fwd_cols(const R& r, typename R::T (&x)[16], u64
     const uint32_t i0 = 16 + sub;
     fwd_stage<0>(r, x, i0);
     fwd_stage<1>(r, x, i0);
-    fwd_stage<2>(r, x, i0);
-    fwd_stage<3>(r, x, i0);
+    fwd_stage<2, FROM != COLS_MODUP>(r, x, i0);
+    fwd_stage<3, FROM == COLS_MODUP>(r, x, i0);
 }
 // Rounds B and A without the last stage.
 template <int COLS, class R, class B>
@@ -231,15 +255,14 @@ __device__ __forceinline__ void inv_cols(const R& r, typename R::T (&x)[16], u64
     inv_stage<1>(r, x, 1);
 }
 // Rounds C and D of one warp's 512 points (blk = index of the 512-point block in the row).  x holds round C's points on
-// entry; on return the warp's padded buffer holds the transformed points, unreduced.
-template <class R>
+// entry; on return the warp's padded buffer holds the transformed points, unreduced (FOLD: the last stage folds).
+template <bool FOLD, class R>
 __device__ __forceinline__ void fwd_rows(const R& r, typename R::T (&x)[16], u64* sm, uint32_t blk, uint32_t lane) {
     const uint32_t i1 = 256 + 2 * blk + (lane >> 4);
     fwd_stage<0>(r, x, i1);
     fwd_stage<1>(r, x, i1);
     fwd_stage<2>(r, x, i1);
-    fold16(r, x);
-    fwd_stage<3>(r, x, i1);
+    fwd_stage<3, true>(r, x, i1);
     u64* c = sm + 288 * (lane >> 4) + (lane & 15);
 #pragma unroll
     for (int k = 0; k < 16; k++) c[18 * k] = R::bits(x[k]);
@@ -253,7 +276,7 @@ __device__ __forceinline__ void fwd_rows(const R& r, typename R::T (&x)[16], u64
     fwd_stage_d<0>(r, x, blk, lane);
     fwd_stage_d<1>(r, x, blk, lane);
     fwd_stage_d<2>(r, x, blk, lane);
-    fwd_stage_d<3>(r, x, blk, lane);
+    fwd_stage_d<3, FOLD>(r, x, blk, lane);
 #pragma unroll
     for (int k = 0; k < 8; k++) d[k] = make_ulonglong2(R::bits(x[2 * k]), R::bits(x[2 * k + 1]));
     __syncwarp();

@@ -112,3 +112,21 @@ def test_first_quotient_of_the_division_by_p(bits):
             worst = max(worst, abs(v) / (2**10 * q))
             assert abs(v) < 2**63
     assert worst < 5.2, worst
+
+
+def test_passes_whose_stages_fold_their_addends_stay_exact():
+    """A stage takes a bound B (in q) to 1.1875 B + 0.5, one that folds its addends first leaves 1 + 0.1875 B: nothing passes 8 q."""
+    def run(b, folds, stages):
+        for s in range(stages):
+            b = 1 + 0.1875 * b if s in folds else 1.1875 * b + 0.5
+            assert b < 8, (s, b)
+        return b
+
+    words = run(1.0, {6}, 8)
+    modup = run(2 * BOUND, {1, 6}, 7)            # the first stage only adds
+    moddown = run(2 * 0.7, {5}, 7)
+    assert (round(words, 2), round(modup, 2), round(moddown, 2)) == (3.38, 2.32, 3.23)
+    for b in (words, modup, moddown):
+        assert run(b, {3}, 8) < 7.41 and run(b, {3, 7}, 8) < 2.10
+    product = 0.5 + 0.1875 * run(modup, {3}, 8)  # in the key inner product
+    assert 4 * product + 0.5 + 0.1875 / 2 < 8 and 4 * product + 0.5 < 8
