@@ -63,6 +63,12 @@ struct PrimeConst {
     double ninvd;
     double ninvwd;
 };
+// q and 1/q of every prime as doubles, handed to kernels by value: read with an index that is the same for a CTA they stay in uniform registers,
+// and an FP64 multiply-add with one uniform operand holds its port for two cycles and not three (a butterfly 16.1 cycles against 17.3; the
+// end of a division on 768 rows 0.325 -> 0.309 ms; k_rows_inner spills with it, 0.70 -> 0.74 ms, and has its constants in registers)
+struct PrimeDoubles {
+    double q[FESC_MAX_PRIMES], qinv[FESC_MAX_PRIMES];
+};
 // Constants of an inverse transform's last stage (N^-1 and N^-1 psi^-brev(1), times a factor of the caller's): Shoup pairs, and
 // centred doubles for primes below 2^50.
 struct InvScale {
@@ -290,6 +296,7 @@ struct fesc_ctx {
     u64 seed;
     std::vector<u64> q;           // host primes
     std::vector<PrimeConst> pc;   // host copy
+    PrimeDoubles pd;              // of the same primes
     std::vector<u64> w1;          // twiddle of the forward transform's first stage
     PrimeConst* d_pc;             // device [n_primes]
     ulonglong2* d_tw;             // forward twiddles [n_primes][N] (w, shoup); N = 2^16: entries from 4096 on regrouped

@@ -532,6 +532,7 @@ extern "C" int fesc_ctx_create(fesc_ctx** out, uint32_t log_n, const uint64_t* p
     ctx->scratch_bytes = 0;
     memset(ctx->counters, 0, sizeof(ctx->counters));
     memset(&ctx->tabs, 0, sizeof(ctx->tabs));
+    memset(&ctx->pd, 0, sizeof(ctx->pd));
     const uint32_t N = ctx->N, np = ctx->n_primes;
     int rc = FESC_OK;
     auto bail = [&](int code) {
@@ -583,6 +584,7 @@ extern "C" int fesc_ctx_create(fesc_ctx** out, uint32_t log_n, const uint64_t* p
         pc.ninvd = (double)pc.ninv;
         pc.ninvwd = (double)pc.ninvw;
         ctx->pc.push_back(pc);
+        ctx->pd.q[i] = pc.qd, ctx->pd.qinv[i] = pc.qinvd;
         ctx->w1.push_back(pw[h_brev(1, log_n)]);
     }
     if ((rc = upload(ctx, &ctx->d_pc, ctx->pc)) != FESC_OK) return bail(rc);

@@ -32,7 +32,7 @@ __device__ __forceinline__ uint32_t list_row(const RowList& list, uint32_t y, ui
 // grid = (256 / NTT_COLS, rows)
 template <int A>
 __global__ void __launch_bounds__(COL_THREADS, 1024 / COL_THREADS)
-    ntt16_cols_fwd(u64* __restrict__ data, const void* __restrict__ tw, const PrimeConst* __restrict__ pcs, RowList list,
+    ntt16_cols_fwd(u64* __restrict__ data, const void* __restrict__ tw, const PrimeConst* __restrict__ pcs, const __grid_constant__ PrimeDoubles pd, RowList list,
                    uint32_t y0, int in_double, const u64* __restrict__ centred, double centred_q) {
     pdl_begin();
     __shared__ u64 sm[COL_SMEM(NTT_COLS)];
@@ -42,7 +42,7 @@ __global__ void __launch_bounds__(COL_THREADS, 1024 / COL_THREADS)
     if (!DBG_REGION(data + (size_t)row * N16, N16 * sizeof(u64))) return;      // the same for the whole CTA
     u64* p = data + (size_t)row * N16 + blockIdx.x * NTT_COLS + col;
     if constexpr (A == ROW_FP) {
-        FpRow r{(const double*)tw + (size_t)pi * N16, pcs[pi].qd, pcs[pi].qinvd};
+        FpRow r{(const double*)tw + (size_t)pi * N16, pd.q[pi], pd.qinv[pi]};
         double x[16];
         if (centred) {                      // a row modulo another prime, centred, then folded modulo this one
             const u64* s = centred + (size_t)(row / list.period) * N16 + blockIdx.x * NTT_COLS + col;
@@ -73,7 +73,7 @@ __global__ void __launch_bounds__(COL_THREADS, 1024 / COL_THREADS)
 
 template <int A>
 __global__ void __launch_bounds__(COL_THREADS, 1024 / COL_THREADS)
-    ntt16_cols_inv(u64* __restrict__ data, const void* __restrict__ tw, const PrimeConst* __restrict__ pcs, RowList list, uint32_t y0,
+    ntt16_cols_inv(u64* __restrict__ data, const void* __restrict__ tw, const PrimeConst* __restrict__ pcs, const __grid_constant__ PrimeDoubles pd, RowList list, uint32_t y0,
                    const InvScale* __restrict__ scale) {
     pdl_begin();
     __shared__ u64 sm[COL_SMEM(NTT_COLS)];
@@ -84,7 +84,7 @@ __global__ void __launch_bounds__(COL_THREADS, 1024 / COL_THREADS)
     u64* p = data + (size_t)row * N16 + blockIdx.x * NTT_COLS + col;
     const PrimeConst& pc = pcs[pi];
     if constexpr (A == ROW_FP) {
-        FpRow r{(const double*)tw + (size_t)pi * N16, pcs[pi].qd, pcs[pi].qinvd};
+        FpRow r{(const double*)tw + (size_t)pi * N16, pd.q[pi], pd.qinv[pi]};
         double x[16];
 #pragma unroll
         for (int k = 0; k < 16; k++) x[k] = FpRow::value(p[(16 * sub + k) * 256]);
@@ -118,7 +118,7 @@ __global__ void __launch_bounds__(COL_THREADS, 1024 / COL_THREADS)
 // WIDE: every buffer lies on a 16-byte boundary (a template and not a flag: tests of a flag at every access cost 0.4 % of a rotation)
 template <int A, int FIN, bool WIDE>
 __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
-    ntt16_rows_fwd(u64* __restrict__ data, const void* __restrict__ tw, const PrimeConst* __restrict__ pcs, RowList list,
+    ntt16_rows_fwd(u64* __restrict__ data, const void* __restrict__ tw, const PrimeConst* __restrict__ pcs, const __grid_constant__ PrimeDoubles pd, RowList list,
                    uint32_t y0, int out_double, NttFinish fin) {
     pdl_begin();
     __shared__ __align__(16) u64 sm_all[NTT_WARPS * ROW_SMEM];
@@ -131,7 +131,7 @@ __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
     const u64* in = p + 256 * (lane >> 4) + (lane & 15);
     const u64* s = sm + 2 * lane + 2 * (lane >> 3);     // the pair 2 lane (+ 64 j) of the padded buffer
     if constexpr (A == ROW_FP) {
-        FpRow r{(const double*)tw + (size_t)pi * N16, pcs[pi].qd, pcs[pi].qinvd};
+        FpRow r{(const double*)tw + (size_t)pi * N16, pd.q[pi], pd.qinv[pi]};
         double x[16];
 #pragma unroll
         for (int k = 0; k < 16; k++) x[k] = FpRow::value(in[16 * k]);
@@ -219,7 +219,7 @@ __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
 
 template <int A, bool SRC, bool WIDE>
 __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
-    ntt16_rows_inv(u64* __restrict__ data, const void* __restrict__ tw, const PrimeConst* __restrict__ pcs, RowList list, uint32_t y0,
+    ntt16_rows_inv(u64* __restrict__ data, const void* __restrict__ tw, const PrimeConst* __restrict__ pcs, const __grid_constant__ PrimeDoubles pd, RowList list, uint32_t y0,
                    NttSource src) {
     pdl_begin();
     __shared__ __align__(16) u64 sm_all[NTT_WARPS * ROW_SMEM];
@@ -254,7 +254,7 @@ __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
     u64* s = sm + 2 * lane + 2 * (lane >> 3);
     u64* o = p + 256 * (lane >> 4) + (lane & 15);
     if constexpr (A == ROW_FP) {
-        FpRow r{(const double*)tw + (size_t)pi * N16, pcs[pi].qd, pcs[pi].qinvd};
+        FpRow r{(const double*)tw + (size_t)pi * N16, pd.q[pi], pd.qinv[pi]};
         const double mul = SRC ? fp_mod_u64(src.mul, pcs[pi]) : 0.0;
 #pragma unroll
         for (int j = 0; j < 8; j++) {
@@ -319,22 +319,22 @@ static int launch_all(fesc_ctx* ctx, u64* data, size_t rows, const RowMap& map, 
             const uint32_t y = (uint32_t)y0;
             if (f == ROW_FP) {
                 if (inverse) {
-                    launch(source ? ntt16_rows_inv<ROW_FP, true, WIDE> : ntt16_rows_inv<ROW_FP, false, WIDE>, gr, ROW_THREADS, 0, st, data, ctx->d_itwf, ctx->d_pc, l,
+                    launch(source ? ntt16_rows_inv<ROW_FP, true, WIDE> : ntt16_rows_inv<ROW_FP, false, WIDE>, gr, ROW_THREADS, 0, st, data, ctx->d_itwf, ctx->d_pc, ctx->pd, l,
                            y, src);
-                    if (!skip_cols) launch(ntt16_cols_inv<ROW_FP>, gc, COL_THREADS, 0, st, data, ctx->d_itwf, ctx->d_pc, l, y, scale);
+                    if (!skip_cols) launch(ntt16_cols_inv<ROW_FP>, gc, COL_THREADS, 0, st, data, ctx->d_itwf, ctx->d_pc, ctx->pd, l, y, scale);
                 } else {
-                    if (!skip_cols) launch(ntt16_cols_fwd<ROW_FP>, gc, COL_THREADS, 0, st, data, ctx->d_twf, ctx->d_pc, l, y, in_double, fin.centred, fin.centred_q);
-                    if (fin.pt || fin.mul) launch(ntt16_rows_fwd<ROW_FP, 2, WIDE>, gr, ROW_THREADS, 0, st, data, ctx->d_twf, ctx->d_pc, l, y, out_double, fin);
-                    else if (fin.acc) launch(ntt16_rows_fwd<ROW_FP, 1, WIDE>, gr, ROW_THREADS, 0, st, data, ctx->d_twf, ctx->d_pc, l, y, out_double, fin);
-                    else launch(ntt16_rows_fwd<ROW_FP, 0, WIDE>, gr, ROW_THREADS, 0, st, data, ctx->d_twf, ctx->d_pc, l, y, out_double, fin);
+                    if (!skip_cols) launch(ntt16_cols_fwd<ROW_FP>, gc, COL_THREADS, 0, st, data, ctx->d_twf, ctx->d_pc, ctx->pd, l, y, in_double, fin.centred, fin.centred_q);
+                    if (fin.pt || fin.mul) launch(ntt16_rows_fwd<ROW_FP, 2, WIDE>, gr, ROW_THREADS, 0, st, data, ctx->d_twf, ctx->d_pc, ctx->pd, l, y, out_double, fin);
+                    else if (fin.acc) launch(ntt16_rows_fwd<ROW_FP, 1, WIDE>, gr, ROW_THREADS, 0, st, data, ctx->d_twf, ctx->d_pc, ctx->pd, l, y, out_double, fin);
+                    else launch(ntt16_rows_fwd<ROW_FP, 0, WIDE>, gr, ROW_THREADS, 0, st, data, ctx->d_twf, ctx->d_pc, ctx->pd, l, y, out_double, fin);
                 }
             } else if (inverse) {
-                launch(source ? ntt16_rows_inv<ROW_INT, true, WIDE> : ntt16_rows_inv<ROW_INT, false, WIDE>, gr, ROW_THREADS, 0, st, data, ctx->d_itw, ctx->d_pc, l, y,
+                launch(source ? ntt16_rows_inv<ROW_INT, true, WIDE> : ntt16_rows_inv<ROW_INT, false, WIDE>, gr, ROW_THREADS, 0, st, data, ctx->d_itw, ctx->d_pc, ctx->pd, l, y,
                        src);
-                if (!skip_cols) launch(ntt16_cols_inv<ROW_INT>, gc, COL_THREADS, 0, st, data, ctx->d_itw, ctx->d_pc, l, y, scale);
+                if (!skip_cols) launch(ntt16_cols_inv<ROW_INT>, gc, COL_THREADS, 0, st, data, ctx->d_itw, ctx->d_pc, ctx->pd, l, y, scale);
             } else {
-                if (!skip_cols) launch(ntt16_cols_fwd<ROW_INT>, gc, COL_THREADS, 0, st, data, ctx->d_tw, ctx->d_pc, l, y, 0, nullptr, 0.0);
-                launch(ntt16_rows_fwd<ROW_INT, 0, WIDE>, gr, ROW_THREADS, 0, st, data, ctx->d_tw, ctx->d_pc, l, y, 0, fin);
+                if (!skip_cols) launch(ntt16_cols_fwd<ROW_INT>, gc, COL_THREADS, 0, st, data, ctx->d_tw, ctx->d_pc, ctx->pd, l, y, 0, nullptr, 0.0);
+                launch(ntt16_rows_fwd<ROW_INT, 0, WIDE>, gr, ROW_THREADS, 0, st, data, ctx->d_tw, ctx->d_pc, ctx->pd, l, y, 0, fin);
             }
             launches += skip_cols ? 1 : 2;
         }
