@@ -53,20 +53,23 @@ def test_key_switches_by_size_of_the_special_primes(bits, n_p):
         assert np.array_equal(got[:, b], np.stack(orc.rotate_hoisted(ct[b], ids)))
 
 
-@pytest.mark.parametrize("level,batch,n_keys", [(24, 2, 8), (9, 4, 3), (4, 1, 7)])
-def test_sums_that_are_reduced_in_between(level, batch, n_keys):
-    """Up to 48 products per sum, and batches of one, two and four ciphertexts per thread."""
+@pytest.mark.parametrize("batch,n_keys", [(2, 8), (4, 3), (1, 7)])
+def test_sums_that_are_reduced_in_between(batch, n_keys):
+    """Six digits of one limb: up to 48 products per sum, and batches of one, two and four ciphertexts per thread."""
     import torch
+    import paper_2608_17442_b200 as fesc
+    from oracle.ckks import Oracle
 
-    pair = ctx_pair("full")
+    args = (16, S.ntt_primes(50, 16, 6, 0) + S.ntt_primes(60, 16, 1, 0), 6, 1, 6, 62)
+    pair = (fesc.Context(*args), Oracle(*args), None)
     ctx, orc, _ = pair
     ids = [700 + k for k in range(n_keys)]
     for k, i in enumerate(ids):
         add_key(pair, 16 * k + 1, i)
-    ct = random_ct(orc, 41, level, level, batch)
-    ct[0] = (np.array(orc.q[:level], dtype=np.uint64) - np.uint64(1))[None, :, None]
+    ct = random_ct(orc, 41, 6, 6, batch)
+    ct[0] = (np.array(orc.q[:6], dtype=np.uint64) - np.uint64(1))[None, :, None]
     out = torch.empty_like(to_dev(ct))
-    ctx.rotate_sum_hoisted(to_dev(ct), out, batch, level, ids)
+    ctx.rotate_sum_hoisted(to_dev(ct), out, batch, 6, ids)
     got = to_host(out)
     for b in sorted({0, batch - 1}):
         assert np.array_equal(got[b], orc.rotate_sum_hoisted(ct[b], ids))
