@@ -1,8 +1,10 @@
 // Rings N = 2^10 .. 2^12: transforms and whole key-switch steps of one row per CTA.
 //
-// A row (8 to 32 KB) fits one CTA: N/16 threads keep 16 points each and run the transform as register rounds of 4, 4 and
-// log N - 8 stages with two exchanges through shared memory.  At these sizes a call is a few hundred thousand products and
-// its time is launches and latencies, so every step around a transform is done by the CTA that holds the row:
+// A row (8 to 32 KB) fits one CTA: N/8 threads keep eight points each and run the transform as register rounds of 3, 3, 3 and
+// log N - 9 stages with three exchanges through shared memory.  At these sizes a call is a few hundred thousand products and
+// its time is launches and latencies, so every step around a transform is done by the CTA that holds the row.  Eight points a
+// thread and not sixteen: a row is one CTA's chain of dependent instructions, and twice the warps hide twice as much of it (a product
+// with a plaintext and two rotations of 4 / 40 / 200 ciphertexts of 3 limbs at N = 2^12: 95.2 -> 72.0, 137 -> 128, 697 -> 587 us).
 //   k_small_coef    [permutation of c1, copy of its own rows] + inverse transform (times a constant)
 //   k_small_modup   conversion of a digit to one target + forward transform
 //   k_small_inner   key inner product of one row [+ inverse transform of the rows on special primes]
@@ -13,7 +15,7 @@
 #include "ntt16.cuh"
 #include "ops.cuh"
 
-#define SM_PAD(e) ((e) + ((e) >> 4))
+#define SM_PAD(e) ((e) + ((e) >> 3))      // a thread's eight adjacent points start nine words apart
 // dynamic shared memory: the padded row, then a copy of the row's twiddle table (8 bytes per entry for FP64 rows, 16 for integer
 // rows).  The copy is made before the kernel waits for its predecessor: at these sizes a stage's twiddles fetched from L2 one
 // stage at a time cost more than its butterflies.
@@ -23,128 +25,179 @@ typedef FpRowT<true> FpS;
 typedef IntRowT<true> IntS;
 template <int LOG>
 __device__ __forceinline__ void small_tables(u64* sm, const SmallTables& tb, uint32_t pi, bool inv) {
-    constexpr uint32_t N = 1u << LOG, T = N / 16;
+    constexpr uint32_t N = 1u << LOG, T = N / 8;
     ulonglong2* dst = reinterpret_cast<ulonglong2*>(sm + SM_ROW(LOG));
     if (tb.pc[pi].q < FESC_FP_LIMIT) {
         const ulonglong2* src = reinterpret_cast<const ulonglong2*>((inv ? tb.itwf : tb.twf) + (size_t)pi * N);
 #pragma unroll
-        for (int k = 0; k < 8; k++) dst[k * T + threadIdx.x] = __ldg(src + k * T + threadIdx.x);
+        for (int k = 0; k < 4; k++) dst[k * T + threadIdx.x] = __ldg(src + k * T + threadIdx.x);
     } else {
         const ulonglong2* src = (inv ? tb.itw : tb.tw) + (size_t)pi * N;
 #pragma unroll
-        for (int k = 0; k < 16; k++) dst[k * T + threadIdx.x] = __ldg(src + k * T + threadIdx.x);
+        for (int k = 0; k < 8; k++) dst[k * T + threadIdx.x] = __ldg(src + k * T + threadIdx.x);
     }
 }
+// (Buffers that kernels write carry no __restrict__: reads through the read-only path may be moved ahead of the wait.)
 #define SMALL_BEGIN(used, pi, inv)                                  \
     extern __shared__ __align__(16) u64 sm[];                       \
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); \
     if (used) small_tables<LOG>(sm, tb, pi, inv);                   \
     asm volatile("griddepcontrol.wait;" ::: "memory");
 
-// Forward: x[k] = point k N/16 + tid on entry; on return the padded buffer holds the transformed row, unreduced.
-template <int LOG, class R>
-__device__ __forceinline__ void small_fwd(const R& r, typename R::T (&x)[16], u64* sm) {
-    constexpr uint32_t N = 1u << LOG, T = N / 16, L = N / 256;
-    constexpr int S = LOG - 8;
-    const uint32_t tid = threadIdx.x, top = tid / L, low = tid % L;
-    __syncthreads();               // the twiddle table is complete
-    fwd_stage<0>(r, x, 1);
-    fwd_stage<1>(r, x, 1);
-    fwd_stage<2>(r, x, 1);
-    fwd_stage<3>(r, x, 1);
-    fold16(r, x);
+// Stage S (0..2) of a round on eight registers: distance 4 >> S, twiddles (i0 << S) + j for the j-th group.  FOLD: as in fwd_stage.
+template <int S, bool FOLD, class R>
+__device__ __forceinline__ void fwd8(const R& r, typename R::T (&x)[8], uint32_t i0) {
+    typename R::W w[8];
+    r.template load<S>(w, i0 << S);
+    constexpr int d = 4 >> S;
 #pragma unroll
-    for (int k = 0; k < 16; k++) sm[SM_PAD(k * T + tid)] = R::bits(x[k]);
+    for (int k = 0; k < 4; k++) {
+        const int i = (k / d) * 2 * d + k % d;
+        if (FOLD) x[i] = r.fold(x[i]);
+        r.ct(x[i], x[i + d], w[k / d]);
+    }
+}
+template <int S, class R>
+__device__ __forceinline__ void inv8(const R& r, typename R::T (&x)[8], uint32_t i0) {
+    typename R::W w[8];
+    r.template load<S>(w, i0 << S);
+    constexpr int d = 4 >> S;
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+        const int i = (k / d) * 2 * d + k % d;
+        r.gs(x[i], x[i + d], w[k / d]);
+    }
+}
+template <class R>
+__device__ __forceinline__ void fold8(const R& r, typename R::T (&x)[8]) {
+#pragma unroll
+    for (int k = 0; k < 8; k++) x[k] = r.fold(x[k]);
+}
+// position in the padded buffer of point k of a thread in the rounds of stride N/8 (1), N/64 (2) and N/512 (3)
+template <int LOG, int ROUND>
+__device__ __forceinline__ uint32_t at8(uint32_t k) {
+    constexpr uint32_t N = 1u << LOG, L = ROUND == 1 ? N / 8 : ROUND == 2 ? N / 64 : N / 512;
+    return SM_PAD(threadIdx.x / L * 8 * L + k * L + threadIdx.x % L);
+}
+// Forward: x[k] = point k N/8 + tid on entry, up to q; on return the padded buffer holds the transformed row, unreduced.  Six stages reach
+// 7.62 q; the folded seventh leaves 2.43, the eleventh 7.47, the folded twelfth 2.40 q.
+template <int LOG, class R>
+__device__ __forceinline__ void small_fwd(const R& r, typename R::T (&x)[8], u64* sm) {
+    constexpr uint32_t N = 1u << LOG, L2 = N / 64, L3 = N / 512;
+    constexpr int S = LOG - 9;
+    const uint32_t tid = threadIdx.x;
+    __syncthreads();               // the twiddle table is complete
+    fwd8<0, false>(r, x, 1);
+    fwd8<1, false>(r, x, 1);
+    fwd8<2, false>(r, x, 1);
+#pragma unroll
+    for (int k = 0; k < 8; k++) sm[at8<LOG, 1>(k)] = R::bits(x[k]);
     __syncthreads();
 #pragma unroll
-    for (int k = 0; k < 16; k++) x[k] = R::value(sm[SM_PAD(top * T + k * L + low)]);
-    fwd_stage<0>(r, x, 16 + top);
-    fwd_stage<1>(r, x, 16 + top);
-    fwd_stage<2>(r, x, 16 + top);
-    fwd_stage<3>(r, x, 16 + top);
-    fold16(r, x);
+    for (int k = 0; k < 8; k++) x[k] = R::value(sm[at8<LOG, 2>(k)]);
+    fwd8<0, false>(r, x, 8 + tid / L2);
+    fwd8<1, false>(r, x, 8 + tid / L2);
+    fwd8<2, false>(r, x, 8 + tid / L2);
     // a thread writes the points it has read: no barrier needed before
 #pragma unroll
-    for (int k = 0; k < 16; k++) sm[SM_PAD(top * T + k * L + low)] = R::bits(x[k]);
+    for (int k = 0; k < 8; k++) sm[at8<LOG, 2>(k)] = R::bits(x[k]);
     __syncthreads();
 #pragma unroll
-    for (int k = 0; k < 16; k++) x[k] = R::value(sm[17 * tid + k]);
+    for (int k = 0; k < 8; k++) x[k] = R::value(sm[at8<LOG, 3>(k)]);
+    fwd8<0, true>(r, x, 64 + tid / L3);
+    fwd8<1, false>(r, x, 64 + tid / L3);
+    fwd8<2, false>(r, x, 64 + tid / L3);
+#pragma unroll
+    for (int k = 0; k < 8; k++) sm[at8<LOG, 3>(k)] = R::bits(x[k]);
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 8; k++) x[k] = R::value(sm[9 * tid + k]);
 #pragma unroll
     for (int s = 0; s < S; s++) {
         const int d = 1 << (S - 1 - s);
 #pragma unroll
-        for (int b = 0; b < 8 / d; b++) {
+        for (int b = 0; b < 4 / d; b++) {
             typename R::W w;
-            r.one(w, (256u << s) + ((16 * tid + 2 * d * b) >> (S - s)));
+            r.one(w, (512u << s) + ((8 * tid + 2 * d * b) >> (S - s)));
 #pragma unroll
-            for (int k = 0; k < d; k++) r.ct(x[2 * d * b + k], x[2 * d * b + k + d], w);
+            for (int k = 0; k < d; k++) {
+                if (s == 2) x[2 * d * b + k] = r.fold(x[2 * d * b + k]);
+                r.ct(x[2 * d * b + k], x[2 * d * b + k + d], w);
+            }
         }
     }
 #pragma unroll
-    for (int k = 0; k < 16; k++) sm[17 * tid + k] = R::bits(x[k]);
+    for (int k = 0; k < 8; k++) sm[9 * tid + k] = R::bits(x[k]);
     __syncthreads();
 }
-// Inverse: the padded buffer holds the row on entry (and a barrier has passed); x[k] = point k N/16 + tid on return, the last
-// stage still to be done (pairs k, k + 8).
+// Inverse: the padded buffer holds the row on entry (and a barrier has passed); x[k] = point k N/8 + tid on return, the last
+// stage still to be done (pairs k, k + 4).
 template <int LOG, class R>
-__device__ __forceinline__ void small_inv(const R& r, typename R::T (&x)[16], u64* sm) {
-    constexpr uint32_t N = 1u << LOG, T = N / 16, L = N / 256;
-    constexpr int S = LOG - 8;
-    const uint32_t tid = threadIdx.x, top = tid / L, low = tid % L;
+__device__ __forceinline__ void small_inv(const R& r, typename R::T (&x)[8], u64* sm) {
+    constexpr uint32_t N = 1u << LOG, L2 = N / 64, L3 = N / 512;
+    constexpr int S = LOG - 9;
+    const uint32_t tid = threadIdx.x;
 #pragma unroll
-    for (int k = 0; k < 16; k++) x[k] = R::value(sm[17 * tid + k]);
+    for (int k = 0; k < 8; k++) x[k] = R::value(sm[9 * tid + k]);
 #pragma unroll
     for (int s = S - 1; s >= 0; s--) {
         const int d = 1 << (S - 1 - s);
 #pragma unroll
-        for (int b = 0; b < 8 / d; b++) {
+        for (int b = 0; b < 4 / d; b++) {
             typename R::W w;
-            r.one(w, (256u << s) + ((16 * tid + 2 * d * b) >> (S - s)));
+            r.one(w, (512u << s) + ((8 * tid + 2 * d * b) >> (S - s)));
 #pragma unroll
             for (int k = 0; k < d; k++) r.gs(x[2 * d * b + k], x[2 * d * b + k + d], w);
         }
     }
-    fold16(r, x);
+    fold8(r, x);
 #pragma unroll
-    for (int k = 0; k < 16; k++) sm[17 * tid + k] = R::bits(x[k]);
+    for (int k = 0; k < 8; k++) sm[9 * tid + k] = R::bits(x[k]);
     __syncthreads();
 #pragma unroll
-    for (int k = 0; k < 16; k++) x[k] = R::value(sm[SM_PAD(top * T + k * L + low)]);
-    inv_stage<3>(r, x, 16 + top);
-    inv_stage<2>(r, x, 16 + top);
-    inv_stage<1>(r, x, 16 + top);
-    inv_stage<0>(r, x, 16 + top);
-    fold16(r, x);
+    for (int k = 0; k < 8; k++) x[k] = R::value(sm[at8<LOG, 3>(k)]);
+    inv8<2>(r, x, 64 + tid / L3);
+    inv8<1>(r, x, 64 + tid / L3);
+    inv8<0>(r, x, 64 + tid / L3);
+    fold8(r, x);
 #pragma unroll
-    for (int k = 0; k < 16; k++) sm[SM_PAD(top * T + k * L + low)] = R::bits(x[k]);
+    for (int k = 0; k < 8; k++) sm[at8<LOG, 3>(k)] = R::bits(x[k]);
     __syncthreads();
 #pragma unroll
-    for (int k = 0; k < 16; k++) x[k] = R::value(sm[SM_PAD(k * T + tid)]);
-    inv_stage<3>(r, x, 1);
-    inv_stage<2>(r, x, 1);
-    inv_stage<1>(r, x, 1);
+    for (int k = 0; k < 8; k++) x[k] = R::value(sm[at8<LOG, 2>(k)]);
+    inv8<2>(r, x, 8 + tid / L2);
+    inv8<1>(r, x, 8 + tid / L2);
+    inv8<0>(r, x, 8 + tid / L2);
+    fold8(r, x);
+#pragma unroll
+    for (int k = 0; k < 8; k++) sm[at8<LOG, 2>(k)] = R::bits(x[k]);
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 8; k++) x[k] = R::value(sm[at8<LOG, 1>(k)]);
+    inv8<2>(r, x, 1);
+    inv8<1>(r, x, 1);
 }
 // last inverse stage of an FP64 / integer row with the constants `s` (nullptr: the plain ones), canonical words to o
 template <int LOG>
-__device__ __forceinline__ void small_inv_store(const FpS& r, double (&x)[16], const PrimeConst& pc, const InvScale* s, u64* o) {
-    constexpr uint32_t T = (1u << LOG) / 16;
+__device__ __forceinline__ void small_inv_store(const FpS& r, double (&x)[8], const PrimeConst& pc, const InvScale* s, u64* o) {
+    constexpr uint32_t T = (1u << LOG) / 8;
     const double n = s ? s->nd : pc.ninvd, w = s ? s->wd : pc.ninvwd;
 #pragma unroll
-    for (int k = 0; k < 8; k++) {
-        const double u = x[k], v = x[k + 8];
+    for (int k = 0; k < 4; k++) {
+        const double u = x[k], v = x[k + 4];
         o[k * T + threadIdx.x] = fp_store(fp_modmul(u + v, n, r.q, r.qinv), r.q, r.qinv);
-        o[(k + 8) * T + threadIdx.x] = fp_store(fp_modmul(u - v, w, r.q, r.qinv), r.q, r.qinv);
+        o[(k + 4) * T + threadIdx.x] = fp_store(fp_modmul(u - v, w, r.q, r.qinv), r.q, r.qinv);
     }
 }
 template <int LOG>
-__device__ __forceinline__ void small_inv_store(const IntS& r, u64 (&x)[16], const PrimeConst& pc, const InvScale* s, u64* o) {
-    constexpr uint32_t T = (1u << LOG) / 16;
+__device__ __forceinline__ void small_inv_store(const IntS& r, u64 (&x)[8], const PrimeConst& pc, const InvScale* s, u64* o) {
+    constexpr uint32_t T = (1u << LOG) / 8;
     const u64 n = s ? s->n : pc.ninv, ns = s ? s->ns : pc.ninvs, w = s ? s->w : pc.ninvw, ws = s ? s->ws : pc.ninvws;
 #pragma unroll
-    for (int k = 0; k < 8; k++) {
-        const u64 u = x[k], v = x[k + 8];
+    for (int k = 0; k < 4; k++) {
+        const u64 u = x[k], v = x[k + 4];
         o[k * T + threadIdx.x] = shoup(u + v, n, ns, r.q);
-        o[(k + 8) * T + threadIdx.x] = shoup(u - v + r.q2, w, ws, r.q);
+        o[(k + 4) * T + threadIdx.x] = shoup(u - v + r.q2, w, ws, r.q);
     }
 }
 // inverse transform of the canonical row in the padded buffer (barrier passed) to o
@@ -154,13 +207,13 @@ __device__ __forceinline__ void small_inv_row(u64* sm, const SmallTables& tb, ui
     if (pc.q < FESC_FP_LIMIT) {
         const FpS r{reinterpret_cast<const double*>(sm + SM_ROW(LOG)), pc.qd, pc.qinvd};
 #pragma unroll
-        for (int k = 0; k < 16; k++) sm[17 * threadIdx.x + k] = FpS::bits(fp_load(sm[17 * threadIdx.x + k], r.q));
-        double x[16];
+        for (int k = 0; k < 8; k++) sm[9 * threadIdx.x + k] = FpS::bits(fp_load(sm[9 * threadIdx.x + k], r.q));
+        double x[8];
         small_inv<LOG>(r, x, sm);
         small_inv_store<LOG>(r, x, pc, s, o);
     } else {
         const IntS r{reinterpret_cast<const ulonglong2*>(sm + SM_ROW(LOG)), pc.q, 2 * pc.q};
-        u64 x[16];
+        u64 x[8];
         small_inv<LOG>(r, x, sm);
         small_inv_store<LOG>(r, x, pc, s, o);
     }
@@ -170,15 +223,15 @@ __device__ __forceinline__ void small_inv_row(u64* sm, const SmallTables& tb, ui
 // plain transforms, one row per CTA (skipped rows launch nothing: RowList)
 // ---------------------------------------------------------------------------------------
 template <int LOG, bool INV>
-__global__ void __launch_bounds__(1 << (LOG - 4)) k_small_ntt(u64* __restrict__ data, SmallTables tb, RowList list) {
-    constexpr uint32_t N = 1u << LOG, T = N / 16;
+__global__ void __launch_bounds__(1 << (LOG - 3)) k_small_ntt(u64* data, SmallTables tb, RowList list) {
+    constexpr uint32_t N = 1u << LOG, T = N / 8;
     const uint32_t rep = blockIdx.x / list.count, e = blockIdx.x - rep * list.count, pi = list.prime[e], tid = threadIdx.x;
     SMALL_BEGIN(true, pi, INV)
     u64* p = data + ((size_t)rep * list.period + list.row[e]) * N;
     if (!DBG_REGION(p, N * sizeof(u64))) return;
     if (INV) {
 #pragma unroll
-        for (int k = 0; k < 16; k++) sm[SM_PAD(k * T + tid)] = p[k * T + tid];
+        for (int k = 0; k < 8; k++) sm[SM_PAD(k * T + tid)] = p[k * T + tid];
         __syncthreads();
         small_inv_row<LOG>(sm, tb, pi, nullptr, p);
         return;
@@ -186,20 +239,20 @@ __global__ void __launch_bounds__(1 << (LOG - 4)) k_small_ntt(u64* __restrict__ 
     const PrimeConst& pc = tb.pc[pi];
     if (pc.q < FESC_FP_LIMIT) {
         const FpS r{reinterpret_cast<const double*>(sm + SM_ROW(LOG)), pc.qd, pc.qinvd};
-        double x[16];
+        double x[8];
 #pragma unroll
-        for (int k = 0; k < 16; k++) x[k] = fp_from_u64(p[k * T + tid]);
+        for (int k = 0; k < 8; k++) x[k] = fp_from_u64(p[k * T + tid]);
         small_fwd<LOG>(r, x, sm);
 #pragma unroll
-        for (int k = 0; k < 16; k++) p[k * T + tid] = fp_store(FpS::value(sm[SM_PAD(k * T + tid)]), r.q, r.qinv);
+        for (int k = 0; k < 8; k++) p[k * T + tid] = fp_store(FpS::value(sm[SM_PAD(k * T + tid)]), r.q, r.qinv);
     } else {
         const IntS r{reinterpret_cast<const ulonglong2*>(sm + SM_ROW(LOG)), pc.q, 2 * pc.q};
-        u64 x[16];
+        u64 x[8];
 #pragma unroll
-        for (int k = 0; k < 16; k++) x[k] = p[k * T + tid];
+        for (int k = 0; k < 8; k++) x[k] = p[k * T + tid];
         small_fwd<LOG>(r, x, sm);
 #pragma unroll
-        for (int k = 0; k < 16; k++) p[k * T + tid] = csub(csub(sm[SM_PAD(k * T + tid)], r.q2), r.q);
+        for (int k = 0; k < 8; k++) p[k * T + tid] = csub(csub(sm[SM_PAD(k * T + tid)], r.q2), r.q);
     }
 }
 
@@ -208,18 +261,17 @@ __global__ void __launch_bounds__(1 << (LOG - 4)) k_small_ntt(u64* __restrict__ 
 // rows kept in `own` (may be nullptr), COEFF rows times (Q_j/q)^-1 to dcoef.  src may be dcoef when g = 0.
 // ---------------------------------------------------------------------------------------
 template <int LOG>
-__global__ void __launch_bounds__(1 << (LOG - 4)) k_small_coef(const u64* src, size_t src_stride, u64* own, size_t own_stride, uint32_t own_rows,
-                                                               uint32_t alpha, u64* dcoef, SmallTables tb, const InvScale* __restrict__ scale,
-                                                               uint32_t level, u64 g) {
-    constexpr uint32_t N = 1u << LOG, T = N / 16;
-    const uint32_t l = blockIdx.x, b = blockIdx.y, tid = threadIdx.x;
-    SMALL_BEGIN(true, l, true)
+__device__ __forceinline__ void coef_row(u64* sm, uint32_t l, uint32_t b, const u64* src, size_t src_stride, u64* own, size_t own_stride,
+                                         uint32_t own_rows, uint32_t alpha, u64* dcoef, const SmallTables& tb, const InvScale* __restrict__ scale,
+                                         uint32_t level, u64 g) {
+    constexpr uint32_t N = 1u << LOG, T = N / 8;
+    const uint32_t tid = threadIdx.x;
     const u64* in = src + (size_t)b * src_stride + (size_t)l * N;
     u64* o = dcoef + ((size_t)b * level + l) * N;
     u64* w = own ? own + (size_t)b * own_stride + ((size_t)(l / alpha) * own_rows + l) * N : nullptr;
     if (!DBG_REGION(in, N * sizeof(u64)) || !DBG_REGION(o, N * sizeof(u64)) || (w && !DBG_REGION(w, N * sizeof(u64)))) return;
 #pragma unroll
-    for (int k = 0; k < 16; k++) {
+    for (int k = 0; k < 8; k++) {
         const uint32_t t = k * T + tid;
         const u64 v = in[g ? galois_src(t, LOG, g) : t];
         sm[SM_PAD(t)] = v;
@@ -228,16 +280,20 @@ __global__ void __launch_bounds__(1 << (LOG - 4)) k_small_coef(const u64* src, s
     __syncthreads();
     small_inv_row<LOG>(sm, tb, l, scale + l, o);
 }
+template <int LOG>
+__global__ void __launch_bounds__(1 << (LOG - 3)) k_small_coef(const u64* src, size_t src_stride, u64* own, size_t own_stride, uint32_t own_rows,
+                                                               uint32_t alpha, u64* dcoef, SmallTables tb, const InvScale* __restrict__ scale,
+                                                               uint32_t level, u64 g) {
+    SMALL_BEGIN(true, blockIdx.x, true)
+    coef_row<LOG>(sm, blockIdx.x, blockIdx.y, src, src_stride, own, own_stride, own_rows, alpha, dcoef, tb, scale, level, g);
+}
 
 // grid (rows of all digits but the own ones, batch): ext[b][j][t] = NTT(sum_a y_a m_a)
 template <int LOG>
-__global__ void __launch_bounds__(1 << (LOG - 4)) k_small_modup(const u64* __restrict__ y, u64* __restrict__ ext, const ModUpDigit* __restrict__ tab,
-                                                                SmallTables tb, uint32_t level, uint32_t n_q, uint32_t K, uint32_t alpha, uint32_t beta) {
-    constexpr uint32_t N = 1u << LOG, T = N / 16;
-    const uint32_t rows = level + K, j = blockIdx.x / rows, t = blockIdx.x - j * rows, b = blockIdx.y, tid = threadIdx.x;
-    if (t < level && t / alpha == j) return;
-    const uint32_t pt = t < level ? t : n_q + (t - level);
-    SMALL_BEGIN(true, pt, false)
+__device__ __forceinline__ void modup_row(u64* sm, uint32_t j, uint32_t t, uint32_t pt, uint32_t b, const u64* y, u64* ext,
+                                          const ModUpDigit* __restrict__ tab, const SmallTables& tb, uint32_t level, uint32_t rows, uint32_t beta) {
+    constexpr uint32_t N = 1u << LOG, T = N / 8;
+    const uint32_t tid = threadIdx.x;
     const ModUpDigit* dg = tab + j;
     const uint32_t n_src = dg->n_src;
     const u64* src = y + ((size_t)b * level + dg->first) * N + tid;
@@ -248,52 +304,62 @@ __global__ void __launch_bounds__(1 << (LOG - 4)) k_small_modup(const u64* __res
     for (uint32_t a = 0; a < n_src; a++) fp = fp && tb.pc[dg->first + a].q < FESC_FP_LIMIT;
     if (fp) {
         const FpS r{reinterpret_cast<const double*>(sm + SM_ROW(LOG)), pc.qd, pc.qinvd};
-        double x[16];
+        double x[8];
 #pragma unroll
-        for (int k = 0; k < 16; k++) x[k] = 0.0;
+        for (int k = 0; k < 8; k++) x[k] = 0.0;
         for (uint32_t a = 0; a < n_src; a++) {         // every product below 0.875 q, folded back after the fourth
             const double m = dg->matd[a][pt];
 #pragma unroll
-            for (int k = 0; k < 16; k++) x[k] += fp_modmul(fp_from_u64(src[(size_t)a * N + k * T]), m, r.q, r.qinv);
-            if (a % 3 == 2) fold16(r, x);
+            for (int k = 0; k < 8; k++) x[k] += fp_modmul(fp_from_u64(src[(size_t)a * N + k * T]), m, r.q, r.qinv);
+            if (a % 3 == 2) fold8(r, x);
         }
+        if (n_src > 1) fold8(r, x);
         small_fwd<LOG>(r, x, sm);
 #pragma unroll
-        for (int k = 0; k < 16; k++) o[k * T] = fp_store(FpS::value(sm[SM_PAD(k * T + tid)]), r.q, r.qinv);
+        for (int k = 0; k < 8; k++) o[k * T] = fp_store(FpS::value(sm[SM_PAD(k * T + tid)]), r.q, r.qinv);
         return;
     }
-    u64 v[16];
+    u64 v[8];
 #pragma unroll
-    for (int k = 0; k < 16; k++) {
+    for (int k = 0; k < 8; k++) {
         acc128 s{0, 0};
         for (uint32_t a = 0; a < n_src; a++) mac128(s, src[(size_t)a * N + k * T], dg->mat[a][pt]);
         v[k] = reduce128(s.hi, s.lo, pc);
     }
     if (pc.q < FESC_FP_LIMIT) {
         const FpS r{reinterpret_cast<const double*>(sm + SM_ROW(LOG)), pc.qd, pc.qinvd};
-        double x[16];
+        double x[8];
 #pragma unroll
-        for (int k = 0; k < 16; k++) x[k] = fp_from_u64(v[k]);
+        for (int k = 0; k < 8; k++) x[k] = fp_from_u64(v[k]);
         small_fwd<LOG>(r, x, sm);
 #pragma unroll
-        for (int k = 0; k < 16; k++) o[k * T] = fp_store(FpS::value(sm[SM_PAD(k * T + tid)]), r.q, r.qinv);
+        for (int k = 0; k < 8; k++) o[k * T] = fp_store(FpS::value(sm[SM_PAD(k * T + tid)]), r.q, r.qinv);
     } else {
         const IntS r{reinterpret_cast<const ulonglong2*>(sm + SM_ROW(LOG)), pc.q, 2 * pc.q};
         small_fwd<LOG>(r, v, sm);
 #pragma unroll
-        for (int k = 0; k < 16; k++) o[k * T] = csub(csub(sm[SM_PAD(k * T + tid)], r.q2), r.q);
+        for (int k = 0; k < 8; k++) o[k * T] = csub(csub(sm[SM_PAD(k * T + tid)], r.q2), r.q);
     }
+}
+
+template <int LOG>
+__global__ void __launch_bounds__(1 << (LOG - 3)) k_small_modup(const u64* y, u64* ext, const ModUpDigit* __restrict__ tab,
+                                                                SmallTables tb, uint32_t level, uint32_t n_q, uint32_t K, uint32_t alpha, uint32_t beta) {
+    const uint32_t rows = level + K, j = blockIdx.x / rows, t = blockIdx.x - j * rows;
+    if (t < level && t / alpha == j) return;
+    const uint32_t pt = t < level ? t : n_q + (t - level);
+    SMALL_BEGIN(true, pt, false)
+    modup_row<LOG>(sm, j, t, pt, blockIdx.y, y, ext, tab, tb, level, rows, beta);
 }
 
 // grid (level + K, 2, batch): acc[b][p][t] = sum over sources and digits of ext . key (+ what acc holds); with `last` the rows on
 // special primes are left as COEFF residues times (P/p_k)^-1
 template <int LOG>
-__global__ void __launch_bounds__(1 << (LOG - 4)) k_small_inner(InnerSrcs S, u64* __restrict__ acc, SmallTables tb, const InvScale* __restrict__ scale,
-                                                                uint32_t level, uint32_t n_q, uint32_t K, uint32_t beta, int accumulate, int last) {
-    constexpr uint32_t N = 1u << LOG, T = N / 16;
-    const uint32_t t = blockIdx.x, pol = blockIdx.y, b = blockIdx.z, tid = threadIdx.x, rows = level + K;
-    const uint32_t pt = t < level ? t : n_q + (t - level);
-    SMALL_BEGIN(last && t >= level, pt, true)
+__device__ __forceinline__ void inner_row(u64* sm, uint32_t t, uint32_t pol, uint32_t pt, uint32_t b, const InnerSrcs& S, u64* acc, const SmallTables& tb,
+                                          const InvScale* __restrict__ scale, uint32_t level, uint32_t n_q, uint32_t K, uint32_t beta, int accumulate,
+                                          int last) {
+    constexpr uint32_t N = 1u << LOG, T = N / 8;
+    const uint32_t tid = threadIdx.x, rows = level + K;
     u64* o = acc + (((size_t)b * 2 + pol) * rows + t) * N;
     bool ok = DBG_REGION(o, N * sizeof(u64));
     for (uint32_t s = 0; s < S.n; s++)
@@ -305,83 +371,114 @@ __global__ void __launch_bounds__(1 << (LOG - 4)) k_small_inner(InnerSrcs S, u64
     const bool fp = pc.q < FESC_FP_LIMIT;
     const double q = pc.qd, qinv = pc.qinvd;
     const bool coef = last && t >= level;
-    constexpr int V = 8;           // points side by side: their loads are in flight together
-#pragma unroll 1
-    for (int k0 = 0; k0 < 16; k0 += V) {
-        const uint32_t c0 = k0 * T + tid;
-        double f[V];
-        acc128 a[V];
+    uint32_t n = 0, at[8];
+    auto positions = [&](u64 g) {
 #pragma unroll
-        for (int e = 0; e < V; e++) {
-            const u64 v = accumulate ? o[c0 + e * T] : 0;
-            f[e] = fp ? fp_load(v, q) : 0.0;
-            a[e] = acc128{v, 0};
-        }
-        uint32_t n = 0;
+        for (int e = 0; e < 8; e++) at[e] = g ? galois_src(tid + e * T, LOG, g) : tid + e * T;
+    };
+    auto put = [&](int e, u64 v) {
+        if (coef) sm[SM_PAD(tid + e * T)] = v;
+        else o[tid + e * T] = v;
+    };
+    const size_t x_step = (size_t)rows * N, w_step = (size_t)2 * (n_q + K) * N;
+    if (fp) {      // canonical words: products below 0.875 q, folded back every 7th (see k_inner)
+        constexpr uint32_t G = 2;      // digits whose words are in flight together: a call of few ciphertexts is a chain of such waits
+        double f[8];
+#pragma unroll
+        for (int e = 0; e < 8; e++) f[e] = accumulate ? fp_load(o[tid + e * T], q) : 0.0;
         for (uint32_t s = 0; s < S.n; s++) {
             const u64* x = S.s[s].ext + ((size_t)b * beta * rows + t) * N;
-            const u64* w = S.s[s].key + ((size_t)pol * (n_q + K) + pt) * N + c0;
-            uint32_t at[V];
+            const u64* w = S.s[s].key + ((size_t)pol * (n_q + K) + pt) * N + tid;
+            positions(S.s[s].g);
+            for (uint32_t j = 0; j < beta; j += G, x += G * x_step, w += G * w_step) {
+                u64 xv[G][8], wv[G][8];
 #pragma unroll
-            for (int e = 0; e < V; e++) at[e] = S.s[s].g ? galois_src(c0 + e * T, LOG, S.s[s].g) : c0 + e * T;
-            for (uint32_t j = 0; j < beta; j++, n++, x += (size_t)rows * N, w += (size_t)2 * (n_q + K) * N) {
-                u64 xv[V], wv[V];
+                for (uint32_t g = 0; g < G; g++)
+                    if (j + g < beta) {
 #pragma unroll
-                for (int e = 0; e < V; e++) xv[e] = x[at[e]], wv[e] = __ldg(w + e * T);
-                if (fp) {      // canonical words: products below 0.875 q, folded back every 7th (see k_inner)
-#pragma unroll
-                    for (int e = 0; e < V; e++) f[e] += fp_modmul(fp_from_u64(xv[e]), fp_from_u64(wv[e]), q, qinv);
-                    if (n % 7 == 6) {
-#pragma unroll
-                        for (int e = 0; e < V; e++) f[e] = fp_reduce(f[e], q, qinv);
+                        for (int e = 0; e < 8; e++) xv[g][e] = x[g * x_step + at[e]], wv[g][e] = __ldg(w + g * w_step + e * T);
                     }
-                } else {
 #pragma unroll
-                    for (int e = 0; e < V; e++) mac128(a[e], xv[e], wv[e]);
-                    if (n % 8 == 7) {
+                for (uint32_t g = 0; g < G; g++) {
+                    if (j + g >= beta) break;
 #pragma unroll
-                        for (int e = 0; e < V; e++) a[e] = acc128{reduce128(a[e].hi, a[e].lo, pc), 0};
+                    for (int e = 0; e < 8; e++) f[e] += fp_modmul(fp_from_u64(xv[g][e]), fp_from_u64(wv[g][e]), q, qinv);
+                    if (n++ % 7 == 6) {
+#pragma unroll
+                        for (int e = 0; e < 8; e++) f[e] = fp_reduce(f[e], q, qinv);
                     }
                 }
             }
         }
 #pragma unroll
-        for (int e = 0; e < V; e++) {
-            const u64 v = fp ? fp_store(f[e], q, qinv) : reduce128(a[e].hi, a[e].lo, pc);
-            if (coef) sm[SM_PAD(c0 + e * T)] = v;
-            else o[c0 + e * T] = v;
+        for (int e = 0; e < 8; e++) put(e, fp_store(f[e], q, qinv));
+    } else {
+        acc128 a[8];
+#pragma unroll
+        for (int e = 0; e < 8; e++) a[e] = acc128{accumulate ? o[tid + e * T] : 0, 0};
+        for (uint32_t s = 0; s < S.n; s++) {
+            const u64* x = S.s[s].ext + ((size_t)b * beta * rows + t) * N;
+            const u64* w = S.s[s].key + ((size_t)pol * (n_q + K) + pt) * N + tid;
+            positions(S.s[s].g);
+            for (uint32_t j = 0; j < beta; j++, x += x_step, w += w_step) {
+                u64 xv[8], wv[8];
+#pragma unroll
+                for (int e = 0; e < 8; e++) xv[e] = x[at[e]], wv[e] = __ldg(w + e * T);
+#pragma unroll
+                for (int e = 0; e < 8; e++) mac128(a[e], xv[e], wv[e]);
+                if (n++ % 8 == 7) {
+#pragma unroll
+                    for (int e = 0; e < 8; e++) a[e] = acc128{reduce128(a[e].hi, a[e].lo, pc), 0};
+                }
+            }
         }
+#pragma unroll
+        for (int e = 0; e < 8; e++) put(e, reduce128(a[e].hi, a[e].lo, pc));
     }
     if (!coef) return;
     __syncthreads();
     small_inv_row<LOG>(sm, tb, pt, scale + pt, o);
 }
+template <int LOG>
+__global__ void __launch_bounds__(1 << (LOG - 3)) k_small_inner(InnerSrcs S, u64* acc, SmallTables tb, const InvScale* __restrict__ scale,
+                                                                uint32_t level, uint32_t n_q, uint32_t K, uint32_t beta, int accumulate, int last) {
+    const uint32_t t = blockIdx.x, pt = t < level ? t : n_q + (t - level);
+    SMALL_BEGIN(last && t >= level, pt, true)
+    inner_row<LOG>(sm, t, blockIdx.y, pt, blockIdx.z, S, acc, tb, scale, level, n_q, K, beta, accumulate, last);
+}
 
-// forward transform of x (canonical words), then out = (acc - u) c (+ the permuted c0) (+ what out holds)
+// forward transform of v (canonical words), then out = (a - u) c (+ rot) (+ what out holds).  a and rot are a thread's words of the minuend
+// and of the permuted c0 (zero: none), fetched by the caller before the transform needs its own.
 struct SmallFinish {
     u64 cinv, cinvs;      // c and its Shoup companion
     int add;
-    const u64* rot;       // nullptr, or the row added through the permutation of g
-    u64 g;
 };
 template <int LOG>
-__device__ __forceinline__ void small_finish(u64 (&v)[16], u64* sm, const SmallTables& tb, uint32_t pi, const u64* __restrict__ acc, u64* out,
+__device__ __forceinline__ void small_words(u64 (&v)[8], const u64* p, u64 g) {      // words tid + k N/8 of the row p, through the permutation of g
+    constexpr uint32_t T = (1u << LOG) / 8;
+#pragma unroll
+    for (int k = 0; k < 8; k++) {
+        const uint32_t t = k * T + threadIdx.x;
+        v[k] = !p ? 0 : p[g ? galois_src(t, LOG, g) : t];
+    }
+}
+template <int LOG>
+__device__ __forceinline__ void small_finish(u64 (&v)[8], u64* sm, const SmallTables& tb, uint32_t pi, const u64 (&a)[8], const u64 (&rot)[8], u64* out,
                                              const SmallFinish& fin) {
-    constexpr uint32_t T = (1u << LOG) / 16;
+    constexpr uint32_t T = (1u << LOG) / 8;
     const uint32_t tid = threadIdx.x;
     const PrimeConst& pc = tb.pc[pi];
     if (pc.q < FESC_FP_LIMIT) {
         const FpS r{reinterpret_cast<const double*>(sm + SM_ROW(LOG)), pc.qd, pc.qinvd};
-        double x[16];
+        double x[8];
 #pragma unroll
-        for (int k = 0; k < 16; k++) x[k] = fp_from_u64(v[k]);
+        for (int k = 0; k < 8; k++) x[k] = fp_from_u64(v[k]);
         small_fwd<LOG>(r, x, sm);
         const double c = fp_from_u64(fin.cinv);
 #pragma unroll
-        for (int k = 0; k < 16; k++) {      // |acc - u| below 5.4q, the lazy product below 2.6q: every sum is exact
+        for (int k = 0; k < 8; k++) {      // u is below 7.48q at the most (N = 2^11), a - u below 8q, the lazy product below 3.5q
             const uint32_t t = k * T + tid;
-            double s = fp_modmul(fp_load(acc[t], r.q) - FpS::value(sm[SM_PAD(t)]), c, r.q, r.qinv);
-            if (fin.rot) s += fp_load(fin.rot[galois_src(t, LOG, fin.g)], r.q);
+            double s = fp_modmul(fp_load(a[k], r.q) - FpS::value(sm[SM_PAD(t)]), c, r.q, r.qinv) + fp_load(rot[k], r.q);
             if (fin.add) s += fp_load(out[t], r.q);
             out[t] = fp_store(s, r.q, r.qinv);
         }
@@ -389,10 +486,9 @@ __device__ __forceinline__ void small_finish(u64 (&v)[16], u64* sm, const SmallT
         const IntS r{reinterpret_cast<const ulonglong2*>(sm + SM_ROW(LOG)), pc.q, 2 * pc.q};
         small_fwd<LOG>(r, v, sm);
 #pragma unroll
-        for (int k = 0; k < 16; k++) {
+        for (int k = 0; k < 8; k++) {
             const uint32_t t = k * T + tid;
-            u64 s = shoup(submod(acc[t], csub(csub(sm[SM_PAD(t)], r.q2), r.q), r.q), fin.cinv, fin.cinvs, r.q);
-            if (fin.rot) s = addmod(s, fin.rot[galois_src(t, LOG, fin.g)], r.q);
+            u64 s = addmod(shoup(submod(a[k], csub(csub(sm[SM_PAD(t)], r.q2), r.q), r.q), fin.cinv, fin.cinvs, r.q), rot[k], r.q);
             if (fin.add) s = addmod(s, out[t], r.q);
             out[t] = s;
         }
@@ -401,12 +497,11 @@ __device__ __forceinline__ void small_finish(u64 (&v)[16], u64* sm, const SmallT
 
 // grid (level, 2, batch): out[b][p][i] = (acc[b][p][i] - u_i) P^-1 (+ ...), u_i = NTT(sum_k [y_k]_centred (P/p_k) mod q_i)
 template <int LOG>
-__global__ void __launch_bounds__(1 << (LOG - 4)) k_small_down(const u64* __restrict__ acc, u64* out, size_t out_stride, const ModDownTab* __restrict__ tab,
-                                                               SmallTables tb, uint32_t level, uint32_t n_q, uint32_t K, int add_mask,
-                                                               const u64* __restrict__ rot_src, size_t rot_stride, u64 g) {
-    constexpr uint32_t N = 1u << LOG, T = N / 16;
-    const uint32_t i = blockIdx.x, pol = blockIdx.y, b = blockIdx.z, tid = threadIdx.x;
-    SMALL_BEGIN(true, i, false)
+__device__ __forceinline__ void down_row(u64* sm, uint32_t i, uint32_t pol, uint32_t b, const u64* acc, u64* out, size_t out_stride,
+                                         const ModDownTab* __restrict__ tab, const SmallTables& tb, uint32_t level, uint32_t K, int add_mask,
+                                         const u64* rot_src, size_t rot_stride, u64 g) {
+    constexpr uint32_t N = 1u << LOG, T = N / 8;
+    const uint32_t tid = threadIdx.x;
     const u64* a = acc + ((size_t)b * 2 + pol) * (level + K) * N;
     u64* o = out + (size_t)b * out_stride + ((size_t)pol * level + i) * N;
     const u64* rot = rot_src && !pol ? rot_src + (size_t)b * rot_stride + (size_t)i * N : nullptr;
@@ -414,30 +509,32 @@ __global__ void __launch_bounds__(1 << (LOG - 4)) k_small_down(const u64* __rest
     const PrimeConst& pc = tb.pc[i];
     const bool fp = pc.q < FESC_FP_LIMIT;
     const double q = pc.qd, qinv = pc.qinvd;
-    u64 v[16];
+    u64 v[8], av[8], rv[8];
+    small_words<LOG>(av, a + (size_t)i * N, 0);
+    small_words<LOG>(rv, rot, g);
     const u64* src = a + (size_t)level * N + tid;
-    u64 cnt = 0;                   // 4 bits per point: how many of its residues are taken negative
     if (fp) {
-        double s[16];
+        double s[8];
 #pragma unroll
-        for (int k = 0; k < 16; k++) s[k] = 0.0;
+        for (int k = 0; k < 8; k++) s[k] = 0.0;
+        const double wrap = tab->wrapd[1][i], w = wrap + wrap >= q ? wrap - q : wrap;      // P, subtracted for every residue taken negative
         for (uint32_t m = 0; m < K; m++) {
             const u64 half = tab->half[m];
             const double m30 = tab->mat30d[m][i], m0 = tab->matd[m][i];
 #pragma unroll
-            for (int k = 0; k < 16; k++) {      // 30-bit halves: every product below 0.51 q
+            for (int k = 0; k < 8; k++) {      // 30-bit halves: every product below 0.51 q, four times two of them and 4 w below 6.1 q
                 const u64 y = src[(size_t)m * N + k * T];
-                cnt += (u64)(y > half) << (4 * k);
                 s[k] += fp_modmul(fp_from_u64(y >> 30), m30, q, qinv);
                 s[k] += fp_modmul(fp_from_u64(y & ((1ull << 30) - 1)), m0, q, qinv);
+                if (y > half) s[k] -= w;
                 if (m == 3) s[k] = fp_reduce(s[k], q, qinv);
             }
         }
 #pragma unroll
-        for (int k = 0; k < 16; k++) v[k] = fp_store(s[k] - tab->wrapd[(cnt >> (4 * k)) & 15][i], q, qinv);
+        for (int k = 0; k < 8; k++) v[k] = fp_store(s[k], q, qinv);
     } else {
 #pragma unroll
-        for (int k = 0; k < 16; k++) {
+        for (int k = 0; k < 8; k++) {
             acc128 w{0, 0};
             uint32_t n = 0;
             for (uint32_t m = 0; m < K; m++) {
@@ -448,28 +545,35 @@ __global__ void __launch_bounds__(1 << (LOG - 4)) k_small_down(const u64* __rest
             v[k] = submod(reduce128(w.hi, w.lo, pc), tab->wrap[n][i], pc.q);
         }
     }
-    small_finish<LOG>(v, sm, tb, i, a + (size_t)i * N, o, SmallFinish{tab->pinv[i], tab->pinvs[i], (add_mask >> pol) & 1, rot, g});
+    small_finish<LOG>(v, sm, tb, i, av, rv, o, SmallFinish{tab->pinv[i], tab->pinvs[i], (add_mask >> pol) & 1});
+}
+template <int LOG>
+__global__ void __launch_bounds__(1 << (LOG - 3)) k_small_down(const u64* acc, u64* out, size_t out_stride, const ModDownTab* __restrict__ tab,
+                                                               SmallTables tb, uint32_t level, uint32_t K, int add_mask, const u64* rot_src,
+                                                               size_t rot_stride, u64 g) {
+    SMALL_BEGIN(true, blockIdx.x, false)
+    down_row<LOG>(sm, blockIdx.x, blockIdx.y, blockIdx.z, acc, out, out_stride, tab, tb, level, K, add_mask, rot_src, rot_stride, g);
 }
 
 // grid (2, batch): COEFF form of the last limb of both polynomials to r[b][p]
 template <int LOG>
-__global__ void __launch_bounds__(1 << (LOG - 4)) k_small_last(const u64* __restrict__ in, size_t in_stride, u64* __restrict__ r, SmallTables tb, uint32_t level) {
-    constexpr uint32_t N = 1u << LOG, T = N / 16;
+__global__ void __launch_bounds__(1 << (LOG - 3)) k_small_last(const u64* in, size_t in_stride, u64* r, SmallTables tb, uint32_t level) {
+    constexpr uint32_t N = 1u << LOG, T = N / 8;
     const uint32_t pol = blockIdx.x, b = blockIdx.y, tid = threadIdx.x;
     SMALL_BEGIN(true, level - 1, true)
     const u64* s = in + (size_t)b * in_stride + ((size_t)pol * level + level - 1) * N;
     u64* o = r + ((size_t)b * 2 + pol) * N;
     if (!DBG_REGION(s, N * sizeof(u64)) || !DBG_REGION(o, N * sizeof(u64))) return;
 #pragma unroll
-    for (int k = 0; k < 16; k++) sm[SM_PAD(k * T + tid)] = s[k * T + tid];
+    for (int k = 0; k < 8; k++) sm[SM_PAD(k * T + tid)] = s[k * T + tid];
     __syncthreads();
     small_inv_row<LOG>(sm, tb, level - 1, nullptr, o);
 }
 // grid (level - 1, 2, batch): out = (in - NTT(centred(r) mod q_i)) q_last^-1
 template <int LOG>
-__global__ void __launch_bounds__(1 << (LOG - 4)) k_small_rescale(const u64* __restrict__ in, size_t in_stride, const u64* __restrict__ r, u64* out,
+__global__ void __launch_bounds__(1 << (LOG - 3)) k_small_rescale(const u64* in, size_t in_stride, const u64* r, u64* out,
                                                                   size_t out_stride, const RescaleTab* __restrict__ tab, SmallTables tb, uint32_t level) {
-    constexpr uint32_t N = 1u << LOG, T = N / 16;
+    constexpr uint32_t N = 1u << LOG, T = N / 8;
     const uint32_t i = blockIdx.x, pol = blockIdx.y, b = blockIdx.z, tid = threadIdx.x;
     SMALL_BEGIN(true, i, false)
     const u64* a = in + (size_t)b * in_stride + ((size_t)pol * level + i) * N;
@@ -477,15 +581,17 @@ __global__ void __launch_bounds__(1 << (LOG - 4)) k_small_rescale(const u64* __r
     u64* o = out + (size_t)b * out_stride + ((size_t)pol * (level - 1) + i) * N;
     if (!DBG_REGION(a, N * sizeof(u64)) || !DBG_REGION(s, N * sizeof(u64)) || !DBG_REGION(o, N * sizeof(u64))) return;
     const PrimeConst& pc = tb.pc[i];
-    u64 v[16];
+    u64 v[8], av[8], zero[8];
+    small_words<LOG>(av, a, 0);
+    small_words<LOG>(zero, nullptr, 0);
 #pragma unroll
-    for (int k = 0; k < 16; k++) {
+    for (int k = 0; k < 8; k++) {
         const u64 y = s[k * T + tid];
         u64 w = csub(y - mulhi(y, pc.mu) * pc.q, pc.q);
         if (y > tab->half) w = submod(w, tab->wrap[i], pc.q);
         v[k] = w;
     }
-    small_finish<LOG>(v, sm, tb, i, a, o, SmallFinish{tab->qinv[i], tab->qinvs[i], 0, nullptr, 0});
+    small_finish<LOG>(v, sm, tb, i, av, zero, o, SmallFinish{tab->qinv[i], tab->qinvs[i], 0});
 }
 
 // ---------------------------------------------------------------------------------------
@@ -506,9 +612,9 @@ bool small_ring(const fesc_ctx* ctx) { return ctx->log_n >= 10 && ctx->log_n <= 
 static SmallTables tables(const fesc_ctx* ctx) { return SmallTables{ctx->d_twf, ctx->d_itwf, ctx->d_tw, ctx->d_itw, ctx->d_pc}; }
 #define SMALL_LAUNCH(kern, grid, ...)                                               \
     do {                                                                            \
-        if (ctx->log_n == 12) launch(kern<12>, grid, 256, SM_BYTES(12), st, __VA_ARGS__);          \
-        else if (ctx->log_n == 11) launch(kern<11>, grid, 128, SM_BYTES(11), st, __VA_ARGS__);     \
-        else launch(kern<10>, grid, 64, SM_BYTES(10), st, __VA_ARGS__);                            \
+        if (ctx->log_n == 12) launch(kern<12>, grid, 512, SM_BYTES(12), st, __VA_ARGS__);          \
+        else if (ctx->log_n == 11) launch(kern<11>, grid, 256, SM_BYTES(11), st, __VA_ARGS__);     \
+        else launch(kern<10>, grid, 128, SM_BYTES(10), st, __VA_ARGS__);                            \
         FESC_CHECK_CUDA(ctx, cudaGetLastError());                                   \
     } while (0)
 
@@ -522,8 +628,8 @@ int small_ntt_launch(fesc_ctx* ctx, u64* data, size_t rows, const RowMap& map, b
     const SmallTables tb = tables(ctx);
 #define SMALL_NTT(LOG)                                                                              \
     do {                                                                                            \
-        if (inverse) launch(k_small_ntt<LOG, true>, grid, 1 << (LOG - 4), SM_BYTES(LOG), st, data, tb, l);          \
-        else launch(k_small_ntt<LOG, false>, grid, 1 << (LOG - 4), SM_BYTES(LOG), st, data, tb, l);                 \
+        if (inverse) launch(k_small_ntt<LOG, true>, grid, 1 << (LOG - 3), SM_BYTES(LOG), st, data, tb, l);          \
+        else launch(k_small_ntt<LOG, false>, grid, 1 << (LOG - 3), SM_BYTES(LOG), st, data, tb, l);                 \
     } while (0)
     if (ctx->log_n == 12) SMALL_NTT(12);
     else if (ctx->log_n == 11) SMALL_NTT(11);
@@ -560,7 +666,7 @@ int small_inner(fesc_ctx* ctx, const KsScratch& ws, const InnerSrcs& S, uint32_t
 int small_moddown(fesc_ctx* ctx, const KsScratch& ws, uint32_t level, uint32_t batch, u64* out, size_t out_stride, int add_mask, cudaStream_t st,
                   const u64* rot_src, size_t rot_stride, u64 g) {
     prof_begin(ctx, PF_MODDOWN, st);
-    SMALL_LAUNCH(k_small_down, dim3(level, 2, batch), ws.acc, out, out_stride, ctx->tabs.d_moddown, tables(ctx), level, ctx->n_q, ctx->n_p, add_mask,
+    SMALL_LAUNCH(k_small_down, dim3(level, 2, batch), ws.acc, out, out_stride, ctx->tabs.d_moddown, tables(ctx), level, ctx->n_p, add_mask,
                  rot_src, rot_stride, g);
     prof_end(ctx, PF_MODDOWN, st);
     ctx->counters[0] += (uint64_t)batch * 2 * level;
