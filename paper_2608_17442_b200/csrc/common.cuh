@@ -311,6 +311,7 @@ struct fesc_ctx {
     u64* d_scratch;
     size_t scratch_bytes;
     uint32_t fail_allocs = 0;     // test hook: this many scratch allocations report FESC_ENOMEM
+    uint32_t small_clusters[2] = {0, 0};   // rings 2^10 .. 2^12: clusters of 8 and of 16 CTAs of k_small_switch that run at the same time
     uint32_t* d_status;           // device word: non-zero after a bounded device-side wait gave up
     uint64_t counters[8];
     Profiler prof;

@@ -1127,11 +1127,15 @@ static int ks_apply(fesc_ctx* ctx, const KsScratch& ws, const EvalKey& key, uint
 }
 
 // Hybrid key switch of `batch` polynomials d[b] ([level][N], EVAL, contiguous) with scratch
-// dcoef (a copy of d, consumed), ext, acc, u.
+// dcoef (a copy of d, consumed), ext, acc, u; only: the call has no other chunk.
 static int key_switch_chunk(fesc_ctx* ctx, const KsScratch& ws, const EvalKey& key, uint32_t level, uint32_t batch,
-                            u64* out, size_t out_stride, int add_mask, cudaStream_t st) {
+                            u64* out, size_t out_stride, int add_mask, cudaStream_t st, bool only) {
     const bool open = ks_open(ctx, level);
-    int rc = ks_decompose(ctx, ws, level, batch, st, nullptr, open);
+    int rc;
+    if (small_ring(ctx) && only &&
+        small_switch(ctx, ws, ws.dcoef, (size_t)level * ctx->N, false, 0, key.d_key, level, batch, out, out_stride, add_mask, st, nullptr, 0, rc))
+        return rc;
+    rc = ks_decompose(ctx, ws, level, batch, st, nullptr, open);
     if (rc != FESC_OK) return rc;
     return ks_apply(ctx, ws, key, level, batch, out, out_stride, add_mask, st, 0, open);
 }
@@ -1236,7 +1240,10 @@ int rotate_multi_internal(fesc_ctx* ctx, const u64* in, size_t in_stride, size_t
             const uint32_t nb = batch - b0 < cut.nb ? batch - b0 : cut.nb;
             const u64* ib = in + k0 * in_key_stride + (size_t)b0 * in_stride;
             u64* ob = out + k0 * out_key_stride + (size_t)b0 * out_stride;
-            if (fused) {
+            if (small_ring(ctx) && nb == batch &&
+                small_switch(ctx, ws, ib + (size_t)level * ctx->N, in_stride, true, keys.g[0], keys.key[0], level, nb, ob, out_stride,
+                             accumulate ? 3 : 0, st, ib, in_stride, rc)) {
+            } else if (fused) {
                 if ((rc = ks_start(ctx, ws, ib, in_stride, keys.g, level, nb, st, open, keys.n, in_key_stride)) != FESC_OK) return rc;
                 InnerSrcs S;
                 S.n = keys.n;
@@ -1252,7 +1259,7 @@ int rotate_multi_internal(fesc_ctx* ctx, const u64* in, size_t in_stride, size_t
                 launch(k_autom_ct, g, 256, 0, st, ib, in_stride, ob, out_stride, own_rows(ctx, ws, level), ws.dcoef, ctx->log_n, level, keys.g[0],
                        ctx->d_pc, accumulate);
                 prof_end(ctx, PF_AUTOM, st);
-                rc = key_switch_chunk(ctx, ws, ctx->keys[key_ids[k0]], level, nb, ob, out_stride, accumulate ? 3 : 1, st);
+                rc = key_switch_chunk(ctx, ws, ctx->keys[key_ids[k0]], level, nb, ob, out_stride, accumulate ? 3 : 1, st, nb == batch);
             }
             if (rc != FESC_OK) return rc;
         }
@@ -1703,7 +1710,7 @@ int ctmul_internal(fesc_ctx* ctx, const u64* a, size_t a_stride, const u64* b, s
         launch(k_tensor, g, 256, 0, st, a + (size_t)b0 * a_stride, a_stride, b + (size_t)b0 * b_stride, b_stride,
                                     out + (size_t)b0 * out_stride, out_stride, own_rows(ctx, ws, level), ws.dcoef, ctx->d_pc, ctx->N, level);
         prof_end(ctx, PF_POINTWISE, st);
-        int rc = key_switch_chunk(ctx, ws, key, level, nb, out + (size_t)b0 * out_stride, out_stride, 3, st);
+        int rc = key_switch_chunk(ctx, ws, key, level, nb, out + (size_t)b0 * out_stride, out_stride, 3, st, nb == batch);
         if (rc != FESC_OK) return rc;
     }
     return FESC_OK;

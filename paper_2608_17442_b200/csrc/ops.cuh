@@ -174,6 +174,9 @@ int small_decompose(fesc_ctx* ctx, const KsScratch& ws, const u64* src, size_t s
 int small_inner(fesc_ctx* ctx, const KsScratch& ws, const InnerSrcs& S, uint32_t level, uint32_t batch, cudaStream_t st, int accumulate, int last);
 int small_moddown(fesc_ctx* ctx, const KsScratch& ws, uint32_t level, uint32_t batch, u64* out, size_t out_stride, int add_mask, cudaStream_t st,
                   const u64* rot_src, size_t rot_stride, u64 g);
+// a whole key switch with one key in one launch where the call is small enough (false: the steps above have to be used)
+bool small_switch(fesc_ctx* ctx, const KsScratch& ws, const u64* src, size_t src_stride, bool keep_own, u64 g, const u64* key, uint32_t level, uint32_t batch,
+                  u64* out, size_t out_stride, int add_mask, cudaStream_t st, const u64* rot_src, size_t rot_stride, int& rc);
 int small_rescale(fesc_ctx* ctx, const u64* in, size_t in_stride, u64* out, size_t out_stride, uint32_t batch, uint32_t level, u64* r, cudaStream_t st);
 
 // packed-operand BSGS accumulate (packed.cu)

@@ -11,6 +11,7 @@
 //   k_small_down    conversion of the special rows to one limb + forward transform + last step of the division [+ permuted c0]
 //   k_small_rescale conversion of the last limb + forward transform + last step of the division
 // A rotation takes 4 launches instead of 9, a rescale 2 instead of 5.
+//   k_small_switch  the first four as one launch of clusters, for calls that leave most of the device idle (rule: switch_ctas)
 #define FESC_DBG_FILE 2   // file id in the sites a debug build reports
 #include "ntt16.cuh"
 #include "ops.cuh"
@@ -555,6 +556,102 @@ __global__ void __launch_bounds__(1 << (LOG - 3)) k_small_down(const u64* acc, u
     down_row<LOG>(sm, blockIdx.x, blockIdx.y, blockIdx.z, acc, out, out_stride, tab, tb, level, K, add_mask, rot_src, rot_stride, g);
 }
 
+// ---------------------------------------------------------------------------------------
+// The four steps of a key switch with one key in one launch: a cluster of CTAs holds a ciphertext, its CTAs take the rows of a step in
+// turn and meet at the cluster's barrier between steps (whose release and acquire also order the rows in global memory, so nothing
+// written here is read through the read-only path).  The twiddle table of a CTA's first row of the next step is fetched while it waits.
+// ---------------------------------------------------------------------------------------
+struct SmallSwitch {
+    const u64* src;              // the polynomial to be switched (k_small_coef)
+    size_t src_stride;
+    u64 *dcoef, *ext, *acc;
+    int keep_own;
+    u64 g;
+    const u64* key;
+    u64* out;
+    size_t out_stride;
+    int add_mask;
+    const u64* rot_src;
+    size_t rot_stride;
+    const InvScale *up_scale, *down_scale;
+    const ModUpDigit* up;
+    const ModDownTab* down;
+    uint32_t level, n_q, K, alpha, beta;
+};
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+
+// grid (CTAs of a cluster, batch)
+template <int LOG>
+__global__ void __launch_bounds__(1 << (LOG - 3)) k_small_switch(SmallSwitch a, SmallTables tb) {
+    extern __shared__ __align__(16) u64 sm[];
+    constexpr uint32_t N = 1u << LOG;
+    const uint32_t rank = blockIdx.x, C = gridDim.x, b = blockIdx.y, level = a.level, rows = level + a.K, beta = a.beta, others = rows - a.alpha;
+    const uint32_t n_up = beta * rows - level;
+    // converted row `task`: every digit but the last has `others` of them
+    struct Up {
+        uint32_t j, t, pt;
+    };
+    auto up_row = [&](uint32_t task) {
+        Up u;
+        u.j = task / others < beta - 1 ? task / others : beta - 1;
+        const uint32_t d = task - u.j * others, first = u.j * a.alpha, n = first + a.alpha < level ? a.alpha : level - first;
+        u.t = d < first ? d : d + n;
+        u.pt = u.t < level ? u.t : a.n_q + (u.t - level);
+        return u;
+    };
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (rank < level) small_tables<LOG>(sm, tb, rank, true);
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    for (uint32_t l = rank; l < level; l += C) {
+        if (l != rank) {
+            __syncthreads();
+            small_tables<LOG>(sm, tb, l, true);
+        }
+        coef_row<LOG>(sm, l, b, a.src, a.src_stride, a.keep_own ? a.ext : nullptr, (size_t)beta * rows * N, rows, a.alpha, a.dcoef, tb, a.up_scale, level, a.g);
+    }
+    __syncthreads();
+    cluster_arrive();
+    if (rank < n_up) small_tables<LOG>(sm, tb, up_row(rank).pt, false);
+    cluster_wait();
+    for (uint32_t task = rank; task < n_up; task += C) {
+        const Up u = up_row(task);
+        if (task != rank) {
+            __syncthreads();
+            small_tables<LOG>(sm, tb, u.pt, false);
+        }
+        modup_row<LOG>(sm, u.j, u.t, u.pt, b, a.dcoef, a.ext, a.up, tb, level, rows, beta);
+    }
+    __syncthreads();
+    cluster_arrive();
+    // the special rows first: they are transformed as well
+    auto row_of = [&](uint32_t task) { return rows - 1 - (task >> 1); };
+    if (rank < 2 * a.K) small_tables<LOG>(sm, tb, a.n_q + (row_of(rank) - level), true);
+    cluster_wait();
+    InnerSrcs S;
+    S.n = 1;
+    S.s[0] = InnerSrc{a.ext, a.key, 0};
+    for (uint32_t task = rank; task < 2 * rows; task += C) {
+        const uint32_t t = row_of(task), pt = t < level ? t : a.n_q + (t - level);
+        if (task != rank && t >= level) {
+            __syncthreads();
+            small_tables<LOG>(sm, tb, pt, true);
+        }
+        inner_row<LOG>(sm, t, task & 1, pt, b, S, a.acc, tb, a.down_scale, level, a.n_q, a.K, beta, 0, 1);
+    }
+    __syncthreads();
+    cluster_arrive();
+    if (rank < 2 * level) small_tables<LOG>(sm, tb, rank >> 1, false);
+    cluster_wait();
+    for (uint32_t task = rank; task < 2 * level; task += C) {
+        if (task != rank) {
+            __syncthreads();
+            small_tables<LOG>(sm, tb, task >> 1, false);
+        }
+        down_row<LOG>(sm, task >> 1, task & 1, b, a.acc, a.out, a.out_stride, a.down, tb, level, a.K, a.add_mask, a.rot_src, a.rot_stride, a.g);
+    }
+}
+
 // grid (2, batch): COEFF form of the last limb of both polynomials to r[b][p]
 template <int LOG>
 __global__ void __launch_bounds__(1 << (LOG - 3)) k_small_last(const u64* in, size_t in_stride, u64* r, SmallTables tb, uint32_t level) {
@@ -597,12 +694,28 @@ __global__ void __launch_bounds__(1 << (LOG - 3)) k_small_rescale(const u64* in,
 // ---------------------------------------------------------------------------------------
 // launches
 // ---------------------------------------------------------------------------------------
+static cudaLaunchConfig_t cluster_config(uint32_t ctas, uint32_t batch, uint32_t threads, size_t smem, cudaStream_t st, cudaLaunchAttribute* attr) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(ctas, batch), cfg.blockDim = threads, cfg.dynamicSmemBytes = smem, cfg.stream = st;
+    attr->id = cudaLaunchAttributeClusterDimension;
+    attr->val.clusterDim.x = ctas, attr->val.clusterDim.y = attr->val.clusterDim.z = 1;
+    cfg.attrs = attr, cfg.numAttrs = 1;
+    return cfg;
+}
 template <int LOG>
 static int small_attr(fesc_ctx* ctx) {
     const void* kernels[] = {(const void*)k_small_coef<LOG>, (const void*)k_small_modup<LOG>, (const void*)k_small_inner<LOG>, (const void*)k_small_down<LOG>,
                              (const void*)k_small_last<LOG>, (const void*)k_small_rescale<LOG>, (const void*)k_small_ntt<LOG, false>,
-                             (const void*)k_small_ntt<LOG, true>};
+                             (const void*)k_small_ntt<LOG, true>, (const void*)k_small_switch<LOG>};
     for (const void* k : kernels) FESC_CHECK_CUDA(ctx, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, SM_BYTES(LOG)));
+    FESC_CHECK_CUDA(ctx, cudaFuncSetAttribute((const void*)k_small_switch<LOG>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    for (int i = 0; i < 2; i++) {
+        cudaLaunchAttribute attr;
+        const cudaLaunchConfig_t cfg = cluster_config(8u << i, 1, 1u << (LOG - 3), SM_BYTES(LOG), 0, &attr);
+        int n = 0;
+        if (cudaOccupancyMaxActiveClusters(&n, k_small_switch<LOG>, &cfg) != cudaSuccess) cudaGetLastError(), n = 0;      // no cluster of this size
+        ctx->small_clusters[i] = (uint32_t)n;
+    }
     return FESC_OK;
 }
 int small_init(fesc_ctx* ctx) {      // up to 98 KB of shared memory per CTA
@@ -679,4 +792,40 @@ int small_rescale(fesc_ctx* ctx, const u64* in, size_t in_stride, u64* out, size
     prof_end(ctx, PF_RESCALE, st, 2);
     ctx->counters[0] += (uint64_t)batch * 2 * level;
     return FESC_OK;
+}
+// CTAs per ciphertext for one launch of k_small_switch, 0: the four kernels.  A barrier of a cluster costs less than a launch, but a
+// step's rows are taken by 8 or 16 CTAs in turn: one launch while all clusters run at once and a CTA has at most two rows to convert.
+// Product with a plaintext and two rotations at N = 2^12, 3 limbs (9 converted rows, up to 18 clusters of 16), four launches / one:
+// 1 ciphertext 69.0 / 67.0 us, 4: 72.4 / 68.1, 9: 79.9 / 78.8, 16: 84.5 / 84.3; 40 would need two waves of clusters.
+static uint32_t switch_ctas(const fesc_ctx* ctx, uint32_t level, uint32_t batch) {
+    const uint32_t beta = (level + ctx->alpha - 1) / ctx->alpha, n_up = beta * (level + ctx->n_p) - level;
+    if (batch <= ctx->small_clusters[1] && n_up > 8 && n_up <= 32) return 16;
+    if (batch <= ctx->small_clusters[0] && n_up <= 16) return 8;
+    return 0;
+}
+template <int LOG>
+static int switch_launch(fesc_ctx* ctx, const SmallSwitch& a, uint32_t ctas, uint32_t batch, cudaStream_t st) {
+    cudaLaunchAttribute attr[2];
+    cudaLaunchConfig_t cfg = cluster_config(ctas, batch, 1u << (LOG - 3), SM_BYTES(LOG), st, attr);
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.numAttrs = 2;
+    FESC_CHECK_CUDA(ctx, cudaLaunchKernelEx(&cfg, k_small_switch<LOG>, a, tables(ctx)));
+    return FESC_OK;
+}
+bool small_switch(fesc_ctx* ctx, const KsScratch& ws, const u64* src, size_t src_stride, bool keep_own, u64 g, const u64* key, uint32_t level, uint32_t batch,
+                  u64* out, size_t out_stride, int add_mask, cudaStream_t st, const u64* rot_src, size_t rot_stride, int& rc) {
+    const uint32_t ctas = switch_ctas(ctx, level, batch), beta = (level + ctx->alpha - 1) / ctx->alpha, rows = level + ctx->n_p;
+    if (!ctas) return false;
+    const SmallSwitch a = {src, src_stride, ws.dcoef, ws.ext, ws.acc, keep_own, g, key, out, out_stride, add_mask, rot_src, rot_stride,
+                           ctx->tabs.d_up_scale + (size_t)(level - 1) * ctx->n_q, ctx->tabs.d_down_scale, ctx->tabs.d_modup + (size_t)(level - 1) * ctx->beta_max,
+                           ctx->tabs.d_moddown, level, ctx->n_q, ctx->n_p, ctx->alpha, beta};
+    prof_begin(ctx, PF_NTT, st);
+    rc = ctx->log_n == 12 ? switch_launch<12>(ctx, a, ctas, batch, st) : ctx->log_n == 11 ? switch_launch<11>(ctx, a, ctas, batch, st)
+                                                                                          : switch_launch<10>(ctx, a, ctas, batch, st);
+    if (rc != FESC_OK) return true;
+    prof_end(ctx, PF_NTT, st);
+    ctx->counters[0] += (uint64_t)batch * (beta * rows + 2 * ctx->n_p + 2 * level);
+    ctx->counters[1] += batch;
+    return true;
 }

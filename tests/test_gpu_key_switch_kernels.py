@@ -73,3 +73,22 @@ def test_sums_that_are_reduced_in_between(batch, n_keys):
     got = to_host(out)
     for b in sorted({0, batch - 1}):
         assert np.array_equal(got[b], orc.rotate_sum_hoisted(ct[b], ids))
+
+
+@pytest.mark.parametrize("name,batch", [("tiny", 1), ("tiny", 18), ("tiny", 19), ("tiny", 40), ("tiny", 70), ("small", 2)])
+def test_small_rings_in_one_launch_and_in_four(name, batch):
+    """Key switches of small rings run as one launch while their clusters fit the device at once, as four beyond that."""
+    import torch
+
+    pair = ctx_pair(name)
+    ctx, orc, _ = pair
+    add_key(pair, 5, 91)
+    for lv in (24, 5, 1) if name == "small" else (3, 2, 1):
+        ct = random_ct(orc, 51, lv, lv, batch)
+        d, out = to_dev(ct), torch.empty((2, batch, 2, lv, orc.N), dtype=torch.int64, device="cuda")
+        ctx.rotate(d, out[0], batch, lv, 91)
+        ctx.ct_ct_mul(d, d, out[1], batch, lv)
+        got = to_host(out)
+        for b in sorted({0, batch // 2, batch - 1}):
+            assert np.array_equal(got[0, b], orc.rotate(ct[b], 91))
+            assert np.array_equal(got[1, b], orc.ct_ct_mul(ct[b], ct[b]))
