@@ -208,8 +208,8 @@ __global__ void __launch_bounds__(32 * RI_WARPS, 4)
     }
 #pragma unroll
     for (int k = 0; k < 8; k++) {
-        *reinterpret_cast<ulonglong2*>(o0 + 64 * k) = make_ulonglong2(fp_store(f0[2 * k], q, qinv), fp_store(f0[2 * k + 1], q, qinv));
-        *reinterpret_cast<ulonglong2*>(o1 + 64 * k) = make_ulonglong2(fp_store(f1[2 * k], q, qinv), fp_store(f1[2 * k + 1], q, qinv));
+        st_pair_once<true>(o0 + 64 * k, make_ulonglong2(fp_store(f0[2 * k], q, qinv), fp_store(f0[2 * k + 1], q, qinv)));
+        st_pair_once<true>(o1 + 64 * k, make_ulonglong2(fp_store(f1[2 * k], q, qinv), fp_store(f1[2 * k + 1], q, qinv)));
     }
 }
 

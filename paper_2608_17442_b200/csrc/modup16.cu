@@ -16,7 +16,7 @@
 // their product, and the stage is additions only.
 //
 // What bounds it: the dispatch of wide operands (an FP64 multiply-add of three registers holds its port for three cycles), which
-// conversion and butterflies share; 0.38 us per converted row at 24 limbs and 16 ciphertexts against 0.41 for a conversion kernel
+// conversion and butterflies share; 0.36 us per converted row at 24 limbs and 16 ciphertexts against 0.41 for a conversion kernel
 // and a first pass of their own, and 1.2 GB less traffic per launch.  8 columns with 6 groups 0.38, division by P 0.39 against 0.33 ms; four exact
 // FP64 products per word instead of the mixed sum 0.53 (the rounding unit takes nine cycles per product); byte planes on the tensor
 // cores, eight targets at a time through shared memory, 0.45; the same for the division by P 0.51 against 0.36 unfused.
@@ -100,7 +100,7 @@ __global__ void __launch_bounds__(MU_THREADS, 2)
         return;                                     // the same for the whole CTA
     for (uint32_t i = tid; i < n_src * (MU_SRC / 2); i += MU_THREADS) {
         const uint32_t a = i / (MU_SRC / 2), r = (i / (MU_COLS / 2)) & 255, c = 2 * (i % (MU_COLS / 2));
-        const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(src + (size_t)a * N16 + r * 256 + c);
+        const ulonglong2 v = ld_pair_once<true>(src + (size_t)a * N16 + r * 256 + c);
         *reinterpret_cast<ulonglong2*>(smem + a * MU_SRC + r * MU_COLS + c) =
             make_ulonglong2(v.x | 0x4330000000000000ull, v.y | 0x4330000000000000ull);
     }
@@ -134,7 +134,7 @@ __global__ void __launch_bounds__(MU_THREADS, 2)
             }
             fwd_cols<MU_COLS, COLS_MODUP>(r, x, sm, col, sub, bar);
 #pragma unroll
-            for (int k = 0; k < 16; k++) p[(16 * sub + k) * 256] = FpRow::bits(x[k]);
+            for (int k = 0; k < 16; k++) st_once(p + (16 * sub + k) * 256, FpRow::bits(x[k]));
         } else {
             const IntRow r{tw + (size_t)pt * N16, q, 2 * q};
             u64 x[16];
@@ -146,7 +146,7 @@ __global__ void __launch_bounds__(MU_THREADS, 2)
             }
             fwd_cols<MU_COLS, COLS_MODUP>(r, x, sm, col, sub, bar);
 #pragma unroll
-            for (int k = 0; k < 16; k++) p[(16 * sub + k) * 256] = x[k];
+            for (int k = 0; k < 16; k++) st_once(p + (16 * sub + k) * 256, x[k]);
         }
     }
 }
@@ -228,7 +228,7 @@ __global__ void __launch_bounds__(MD_THREADS, 2)
             const InvScale& c = scale[n_q + a];
             u64 x[16];
 #pragma unroll
-            for (int k = 0; k < 16; k++) x[k] = src[(size_t)a * N16 + (16 * sub + k) * 256 + col];
+            for (int k = 0; k < 16; k++) x[k] = ld_once(src + (size_t)a * N16 + (16 * sub + k) * 256 + col);
             bar();                                  // the buffer's last reader
             inv_cols<MU_COLS>(r, x, sm, col, sub, bar);
             const u64 n = c.n, ns = c.ns, nw = c.w, nws = c.ws;
@@ -310,7 +310,7 @@ __global__ void __launch_bounds__(MD_THREADS, 2)
         fwd_cols<MU_COLS, COLS_MODDOWN>(r, x, sm, col, sub, bar);
         u64* p = out + (size_t)i * N16 + col;
 #pragma unroll
-        for (int k = 0; k < 16; k++) p[(16 * sub + k) * 256] = FpRow::bits(x[k]);
+        for (int k = 0; k < 16; k++) st_once(p + (16 * sub + k) * 256, FpRow::bits(x[k]));
     }
 }
 

@@ -12,7 +12,7 @@
 // The inverse runs D, C, B, A.
 //
 // What bounds it: a transform moves 2 MiB (0.32 us at the 6.55 TB/s a copy reaches) and issues about 17 cycles of FP64 work
-// per warp-butterfly (0.26 us); measured 0.383 us per transform on 1536 rows, 0.41 on 384 (8 points per thread and two
+// per warp-butterfly (0.26 us); measured 0.365 us per transform on 1536 rows, 0.41 on 384 (8 points per thread and two
 // exchanges per kernel: 0.487 and 0.513).  Sixteen points per thread halve the shared-memory traffic and the barriers per
 // butterfly and still fit 64 registers, i.e. 32 warps per SM; CTAs of four warps drift apart, so that loads, exchanges and
 // butterflies of different CTAs overlap.  Measured beside it: 4 / 16 columns per CTA 0.432 / 0.372-0.381, 1 / 8 warps 0.397 /
@@ -52,7 +52,7 @@ __global__ void __launch_bounds__(COL_THREADS, 1024 / COL_THREADS)
         } else {
 #pragma unroll
             for (int k = 0; k < 16; k++) {  // canonical words, or doubles with |x| <= q/2 from a conversion kernel
-                const u64 v = p[(16 * k + sub) * 256];
+                const u64 v = ld_once(p + (16 * k + sub) * 256);
                 x[k] = in_double ? FpRow::value(v) : fp_from_u64(v);
             }
         }
@@ -87,7 +87,7 @@ __global__ void __launch_bounds__(COL_THREADS, 1024 / COL_THREADS)
         FpRow r{(const double*)tw + (size_t)pi * N16, pd.q[pi], pd.qinv[pi]};
         double x[16];
 #pragma unroll
-        for (int k = 0; k < 16; k++) x[k] = FpRow::value(p[(16 * sub + k) * 256]);
+        for (int k = 0; k < 16; k++) x[k] = FpRow::value(ld_once(p + (16 * sub + k) * 256));
         inv_cols<NTT_COLS>(r, x, sm, col, sub, CtaBarrier());
         const double ninv = scale ? scale[pi].nd : pc.ninvd, ninvw = scale ? scale[pi].wd : pc.ninvwd;
 #pragma unroll
@@ -134,7 +134,7 @@ __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
         FpRow r{(const double*)tw + (size_t)pi * N16, pd.q[pi], pd.qinv[pi]};
         double x[16];
 #pragma unroll
-        for (int k = 0; k < 16; k++) x[k] = FpRow::value(in[16 * k]);
+        for (int k = 0; k < 16; k++) x[k] = FpRow::value(ld_once(in + 16 * k));
         if (FIN) {
             const uint32_t bp = row / fin.level, i = row - bp * fin.level, ct = bp >> 1, pol = bp & 1, k = ct / fin.nb, b = ct - k * fin.nb;
             prefetch_l2(fin.acc + (size_t)ct * fin.acc_stride + ((size_t)pol * fin.acc_rows + i) * N16 + blk * 512 + 16 * lane);
@@ -170,7 +170,7 @@ __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
         const double mul = FIN == 2 ? fp_mod_u64(fin.mul, pcs[pi]) : 0.0;
         ulonglong2 av[8];
 #pragma unroll
-        for (int j = 0; j < 8; j++) av[j] = ld_pair<WIDE>(acc + blk * 512 + 2 * lane + 64 * j);
+        for (int j = 0; j < 8; j++) av[j] = ld_pair_once<WIDE>(acc + blk * 512 + 2 * lane + 64 * j);
 #pragma unroll
         for (int h = 0; h < 8; h += 4) {
             ulonglong2 w[4];
@@ -183,7 +183,7 @@ __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
                 const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(s + 72 * j);
                 double a0 = fp_from_u64(av[j].x), a1 = fp_from_u64(av[j].y);
                 if (FIN == 2) {             // lazy products below 0.7 q
-                    const ulonglong2 w2 = pt ? ld_pair<WIDE>(pt + 64 * j) : make_ulonglong2(0, 0);
+                    const ulonglong2 w2 = pt ? ld_pair_once<WIDE>(pt + 64 * j) : make_ulonglong2(0, 0);
                     a0 = fp_modmul(a0, pt ? fp_from_u64(w2.x) : mul, q, qinv);
                     a1 = fp_modmul(a1, pt ? fp_from_u64(w2.y) : mul, q, qinv);
                 }
@@ -195,11 +195,11 @@ __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
                 }
                 u64* o = out + blk * 512 + 2 * lane + 64 * j;
                 if (FIN == 1 && add) {
-                    const ulonglong2 ov = ld_pair<WIDE>(o);
+                    const ulonglong2 ov = ld_pair_once<WIDE>(o);
                     s0 += fp_from_u64(ov.x);
                     s1 += fp_from_u64(ov.y);
                 }
-                st_pair<WIDE>(o, make_ulonglong2(fp_store(s0, q, qinv), fp_store(s1, q, qinv)));
+                st_pair_once<WIDE>(o, make_ulonglong2(fp_store(s0, q, qinv), fp_store(s1, q, qinv)));
             }
         }
     } else {
@@ -207,7 +207,7 @@ __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
         const IntRow r{(const ulonglong2*)tw + (size_t)pi * N16, q, 2 * q};
         u64 x[16];
 #pragma unroll
-        for (int k = 0; k < 16; k++) x[k] = in[16 * k];
+        for (int k = 0; k < 16; k++) x[k] = ld_once(in + 16 * k);
         fwd_rows<false>(r, x, sm, blk, lane);
 #pragma unroll
         for (int j = 0; j < 8; j++) {
@@ -273,7 +273,7 @@ __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
         double x[16];
         inv_rows(r, x, sm, blk, lane);
 #pragma unroll
-        for (int k = 0; k < 16; k++) o[16 * k] = FpRow::bits(x[k]);      // doubles, |x| <= q/2
+        for (int k = 0; k < 16; k++) st_once(o + 16 * k, FpRow::bits(x[k]));      // doubles, |x| <= q/2
     } else {
         const u64 q = pcs[pi].q;
         const IntRow r{(const ulonglong2*)tw + (size_t)pi * N16, q, 2 * q};
@@ -287,7 +287,7 @@ __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
         u64 x[16];
         inv_rows(r, x, sm, blk, lane);
 #pragma unroll
-        for (int k = 0; k < 16; k++) o[16 * k] = x[k];                   // below 2q
+        for (int k = 0; k < 16; k++) st_once(o + 16 * k, x[k]);                   // below 2q
     }
 }
 

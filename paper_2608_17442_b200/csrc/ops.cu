@@ -487,7 +487,7 @@ __global__ void __launch_bounds__(256, 4) k_inner_shared(const u64* __restrict__
     prefetch_key(0);
     for (uint32_t r = tid / 32; r < batch * BETA; r += 8)        // a warp copies one row's block, 16 bytes per lane
         *reinterpret_cast<ulonglong2*>(sx + r * IS_BLK + 2 * (tid % 32)) =
-            *reinterpret_cast<const ulonglong2*>(ext + ((size_t)r * rows + t) * N + blk * IS_BLK + 2 * (tid % 32));
+            ld_pair_once<true>(ext + ((size_t)r * rows + t) * N + blk * IS_BLK + 2 * (tid % 32));
     __syncthreads();
     const PrimeConst& pc = pcs[pt];
     const double q = pc.qd, qinv = pc.qinvd;
@@ -514,8 +514,8 @@ __global__ void __launch_bounds__(256, 4) k_inner_shared(const u64* __restrict__
                     f1 += fp_modmul(xd, kd[2 * j + 1], q, qinv);
                     if (j == 6) f0 = fp_reduce(f0, q, qinv), f1 = fp_reduce(f1, q, qinv);
                 }
-                o[(size_t)(2 * b) * rows * N] = fp_store(f0, q, qinv);
-                o[(size_t)(2 * b + 1) * rows * N] = fp_store(f1, q, qinv);
+                st_once(o + (size_t)(2 * b) * rows * N, fp_store(f0, q, qinv));
+                st_once(o + (size_t)(2 * b + 1) * rows * N, fp_store(f1, q, qinv));
             }
         } else {
             for (uint32_t b = part; b < batch; b += 256 / IS_BLK) {
@@ -526,8 +526,8 @@ __global__ void __launch_bounds__(256, 4) k_inner_shared(const u64* __restrict__
                     mac128(a0, xv, kw[2 * j]);
                     mac128(a1, xv, kw[2 * j + 1]);
                 }
-                o[(size_t)(2 * b) * rows * N] = reduce128(a0.hi, a0.lo, pc);
-                o[(size_t)(2 * b + 1) * rows * N] = reduce128(a1.hi, a1.lo, pc);
+                st_once(o + (size_t)(2 * b) * rows * N, reduce128(a0.hi, a0.lo, pc));
+                st_once(o + (size_t)(2 * b + 1) * rows * N, reduce128(a1.hi, a1.lo, pc));
             }
         }
     }
