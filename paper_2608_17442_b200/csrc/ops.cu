@@ -1669,7 +1669,15 @@ __device__ __forceinline__ void tensor_word(u64 a0, u64 a1, u64 b0, u64 b1, cons
     mac128(s, a1, b0);
     d0 = mulmod(a0, b0, pc), d1 = reduce128(s.hi, s.lo, pc), d2 = mulmod(a1, b1, pc);
 }
-__global__ void __launch_bounds__(256) k_tensor(const u64* __restrict__ a, size_t a_stride, const u64* __restrict__ bb,
+// The same below 2^50: a product of canonical words stays below 0.875 q, the sum of two below 1.75 q.  The kernel moves 48 bytes per word of a
+// square (64 of a product): 12 squares of 17 limbs 0.165 ms with the integer products, bound by them, 0.104 with these, at 0.94 of the copy rate.
+__device__ __forceinline__ void tensor_word_fp(u64 a0, u64 a1, u64 b0, u64 b1, double q, double qinv, u64& d0, u64& d1, u64& d2) {
+    const double x0 = fp_from_u64(a0), x1 = fp_from_u64(a1), y0 = fp_from_u64(b0), y1 = fp_from_u64(b1);
+    d0 = fp_store(fp_modmul(x0, y0, q, qinv), q, qinv);
+    d1 = fp_store(fp_modmul(x0, y1, q, qinv) + fp_modmul(x1, y0, q, qinv), q, qinv);
+    d2 = fp_store(fp_modmul(x1, y1, q, qinv), q, qinv);
+}
+__global__ void __launch_bounds__(256) k_tensor(const u64* a, size_t a_stride, const u64* bb,
                                                 size_t b_stride, u64* __restrict__ out, size_t out_stride,
                                                 OwnRows d, u64* __restrict__ dcoef,
                                                 const PrimeConst* __restrict__ pcs, uint32_t N, uint32_t level) {
@@ -1688,8 +1696,13 @@ __global__ void __launch_bounds__(256) k_tensor(const u64* __restrict__ a, size_
     const ulonglong2 va[2] = {ld_pair(a + b * a_stride + o, wide_a), ld_pair(a + b * a_stride + poly + o, wide_a)};
     const ulonglong2 vb[2] = {ld_pair(bb + b * b_stride + o, wide_b), ld_pair(bb + b * b_stride + poly + o, wide_b)};
     ulonglong2 d0, d1, d2, own;
-    tensor_word(va[0].x, va[1].x, vb[0].x, vb[1].x, pc, d0.x, d1.x, d2.x);
-    tensor_word(va[0].y, va[1].y, vb[0].y, vb[1].y, pc, d0.y, d1.y, d2.y);
+    if (pc.q < FESC_FP_LIMIT) {
+        tensor_word_fp(va[0].x, va[1].x, vb[0].x, vb[1].x, pc.qd, pc.qinvd, d0.x, d1.x, d2.x);
+        tensor_word_fp(va[0].y, va[1].y, vb[0].y, vb[1].y, pc.qd, pc.qinvd, d0.y, d1.y, d2.y);
+    } else {
+        tensor_word(va[0].x, va[1].x, vb[0].x, vb[1].x, pc, d0.x, d1.x, d2.x);
+        tensor_word(va[0].y, va[1].y, vb[0].y, vb[1].y, pc, d0.y, d1.y, d2.y);
+    }
     own.x = own_word(d, d2.x, pc), own.y = own_word(d, d2.y, pc);
     st_pair(out + b * out_stride + o, d0, wide_out);
     st_pair(out + b * out_stride + poly + o, d1, wide_out);

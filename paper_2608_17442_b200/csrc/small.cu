@@ -795,8 +795,8 @@ int small_rescale(fesc_ctx* ctx, const u64* in, size_t in_stride, u64* out, size
 }
 // CTAs per ciphertext for one launch of k_small_switch, 0: the four kernels.  A barrier of a cluster costs less than a launch, but a
 // step's rows are taken by 8 or 16 CTAs in turn: one launch while all clusters run at once and a CTA has at most two rows to convert.
-// Product with a plaintext and two rotations at N = 2^12, 3 limbs (9 converted rows, up to 18 clusters of 16), four launches / one:
-// 1 ciphertext 69.0 / 67.0 us, 4: 72.4 / 68.1, 9: 79.9 / 78.8, 16: 84.5 / 84.3; 40 would need two waves of clusters.
+// Product with a plaintext and two rotations at N = 2^12, 3 limbs (9 converted rows; 14 clusters of 16 run at once, 15 of 8), four launches /
+// one: 1 ciphertext 69.0 / 67.0 us, 4: 72.4 / 68.1 (8 CTAs 76.7), 9: 79.9 / 78.8, 16: 84.5 and no longer in one.
 static uint32_t switch_ctas(const fesc_ctx* ctx, uint32_t level, uint32_t batch) {
     const uint32_t beta = (level + ctx->alpha - 1) / ctx->alpha, n_up = beta * (level + ctx->n_p) - level;
     if (batch <= ctx->small_clusters[1] && n_up > 8 && n_up <= 32) return 16;

@@ -75,7 +75,7 @@ def test_sums_that_are_reduced_in_between(batch, n_keys):
         assert np.array_equal(got[b], orc.rotate_sum_hoisted(ct[b], ids))
 
 
-@pytest.mark.parametrize("name,batch", [("tiny", 1), ("tiny", 18), ("tiny", 19), ("tiny", 40), ("tiny", 70), ("small", 2)])
+@pytest.mark.parametrize("name,batch", [("tiny", 1), ("tiny", 14), ("tiny", 15), ("tiny", 16), ("tiny", 40), ("small", 2)])
 def test_small_rings_in_one_launch_and_in_four(name, batch):
     """Key switches of small rings run as one launch while their clusters fit the device at once, as four beyond that."""
     import torch
@@ -92,3 +92,28 @@ def test_small_rings_in_one_launch_and_in_four(name, batch):
         for b in sorted({0, batch // 2, batch - 1}):
             assert np.array_equal(got[0, b], orc.rotate(ct[b], 91))
             assert np.array_equal(got[1, b], orc.ct_ct_mul(ct[b], ct[b]))
+
+
+@pytest.mark.parametrize("bits", [36, 50, 51, 55])
+def test_products_of_the_largest_words(bits):
+    """Products with relinearisation on both sides of 2^50, where FP64 products end: words 0, 1, (q +- 1)/2, q - 2 and q - 1 against each other."""
+    import torch
+    import paper_2608_17442_b200 as fesc
+    from oracle.ckks import Oracle
+
+    args = (12, S.ntt_primes(bits, 12, 3, 0) + S.ntt_primes(60, 12, 1, 0), 3, 1, 3, 63)
+    ctx, orc = fesc.Context(*args), Oracle(*args)
+    ct = np.empty((2, 2, 3, orc.N), dtype=np.uint64)
+    at = np.arange(orc.N)
+    for l in range(3):
+        q = orc.q[l]
+        words = np.array([0, 1, (q - 1) // 2, (q + 1) // 2, q - 2, q - 1], dtype=np.uint64)
+        for k in range(4):
+            ct[k // 2, k % 2, l] = words[at // 6**k % 6]
+    out = torch.empty((2, 2, 3, orc.N), dtype=torch.int64, device="cuda")
+    a, b = to_dev(ct), to_dev(ct[::-1].copy())
+    ctx.ct_ct_mul(a, b, out[:1], 1, 3)
+    ctx.ct_ct_mul(a, a, out[1:], 1, 3)
+    got = to_host(out)
+    assert np.array_equal(got[0], orc.ct_ct_mul(ct[0], ct[1]))
+    assert np.array_equal(got[1], orc.ct_ct_mul(ct[0], ct[0]))
