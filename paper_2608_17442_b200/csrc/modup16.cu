@@ -86,11 +86,11 @@ template <int A>
 __global__ void __launch_bounds__(MU_THREADS, 2)
     k_modup_cols(const u64* y, u64* ext, const ModUpDigit* __restrict__ tab, const double* __restrict__ twf,
                  const ulonglong2* __restrict__ tw, const PrimeConst* __restrict__ pcs, uint32_t level, uint32_t n_q, uint32_t K,
-                 uint32_t beta, uint32_t splits) {
+                 uint32_t beta) {
     pdl_begin();
     extern __shared__ __align__(16) u64 smem[];      // [A][MU_SRC] source columns, then one exchange buffer per group
     __shared__ uint32_t next, taken[2][MU_GROUPS];
-    const uint32_t tid = threadIdx.x, tile = blockIdx.x / splits, part = blockIdx.x % splits, j = blockIdx.y, b = blockIdx.z;
+    const uint32_t tid = threadIdx.x, tile = blockIdx.x, j = blockIdx.y, b = blockIdx.z;
     const ModUpDigit* dg = tab + j;
     const uint32_t first = dg->first, n_src = dg->n_src, rows = level + K, others = rows - n_src;
     const u64* src = y + ((size_t)b * level + first) * N16 + tile * MU_COLS;
@@ -115,7 +115,7 @@ __global__ void __launch_bounds__(MU_THREADS, 2)
     // the next target is taken while this one is worked on; the exchange's barrier publishes it.  (A barrier before the exchange and not
     // at the head of the loop: a group's two warps may be half a target apart.)
     for (uint32_t slot = 0;; slot ^= 1) {
-        const uint32_t o = taken[slot][group] * splits + part;
+        const uint32_t o = taken[slot][group];
         if (o >= others) return;
         if (gt == 0) taken[slot ^ 1][group] = atomicAdd(&next, 1u);
         const uint32_t d = o < K ? 0 : o - K;
@@ -166,11 +166,10 @@ static int launch_modup(fesc_ctx* ctx, const u64* y, u64* ext, uint32_t level, u
     const size_t smem = ((size_t)A * MU_SRC + MU_GROUPS * COL_SMEM(MU_COLS)) * sizeof(u64);
     auto kern = k_modup_cols<A>;
     FESC_CHECK_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    // with few ciphertexts up to four CTAs share the targets of a tile, until there are four CTAs for every place (two per SM)
-    uint32_t splits = 1;
-    while (splits < 4 && tiles * beta * batch * splits < 8 * 148) splits++;
-    launch(kern, dim3(tiles * splits, beta, batch), MU_THREADS, smem, st, y, ext, ctx->tabs.d_modup + (size_t)(level - 1) * ctx->beta_max,
-                                                                     ctx->d_twf, ctx->d_tw, ctx->d_pc, level, ctx->n_q, ctx->n_p, beta, splits);
+    // One CTA takes all targets of a tile, however few tiles there are: shared by two to four CTAs, each of which loads the sources again, one rotation of
+    // 24 / 15 / 9 / 5 limbs takes 267-275 / 187-195 / 150-162 / 109-111 us against 266 / 181 / 149 / 107, four of 15 limbs 444-469 against 419.
+    launch(kern, dim3(tiles, beta, batch), MU_THREADS, smem, st, y, ext, ctx->tabs.d_modup + (size_t)(level - 1) * ctx->beta_max,
+                                                                     ctx->d_twf, ctx->d_tw, ctx->d_pc, level, ctx->n_q, ctx->n_p, beta);
     return FESC_OK;
 }
 int modup16_cols_launch(fesc_ctx* ctx, const u64* y, u64* ext, uint32_t level, uint32_t batch, cudaStream_t st) {
@@ -334,8 +333,10 @@ static int launch_moddown(fesc_ctx* ctx, const u64* acc, u64* u, uint32_t level,
     const size_t smem = ((size_t)A * MU_SRC + MD_GROUPS * COL_SMEM(MU_COLS)) * sizeof(u64);
     auto kern = k_moddown_cols<A, OPEN>;
     FESC_CHECK_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    uint32_t splits = 1;
-    while (splits < 4 && tiles * polys * splits < 8 * 148) splits++;
+    // Two CTAs share the limbs of a tile where its places (two per SM) would be half empty otherwise.  Each opens the special rows again, which costs as
+    // much as a third of 24 limbs: one rotation of 24 / 15 / 9 / 5 limbs with 1, 2, 4 CTAs per tile 277, 260, 271 / 194, 188, 194 / 155, 147, 160 /
+    // 114, 106, 113 us; two: 395, 400, 416 / 250, 257, 269 / 195, 205, 219 / 138, 150, 163; eight of 24 limbs 1239, 1265, 1341.
+    const uint32_t splits = tiles * polys <= 148 ? 2 : 1;
     launch(kern, dim3(tiles * splits, polys), MD_THREADS, smem, st, acc, u, ctx->tabs.d_moddown, ctx->d_twf, ctx->d_itw, ctx->tabs.d_down_scale, ctx->d_pc,
            level, ctx->n_q, ctx->n_p, splits);
     return FESC_OK;
