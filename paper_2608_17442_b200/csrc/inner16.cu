@@ -218,6 +218,10 @@ int rows_inner_launch(fesc_ctx* ctx, const InnerSrcs& S, u64* acc, uint32_t leve
     const uint32_t beta = (level + ctx->alpha - 1) / ctx->alpha, groups = (batch + RI_WARPS - 1) / RI_WARPS, warps = (batch + groups - 1) / groups;
     const dim3 grid(128 * groups, level + ctx->n_p, separate ? S.n : 1);
     FESC_CHECK_CUDA(ctx, cudaFuncSetAttribute(k_rows_inner, cudaFuncAttributeMaxDynamicSharedMemorySize, RI_SMEM(RI_WARPS)));
+    // Shared memory for four CTAs of four warps and no more: CTAs of one or two warps would fill all of it and leave the L1 too small for their twiddles
+    // (one rotation of 24 limbs 254.6 -> 244.9 us, two 395 -> 379; three and more the same, with a smaller share 3 % slower).
+    const int share = (int)((400 * (RI_SMEM(RI_WARPS) + 1024) + 228 * 1024 - 1) / (228 * 1024));
+    FESC_CHECK_CUDA(ctx, cudaFuncSetAttribute(k_rows_inner, cudaFuncAttributePreferredSharedMemoryCarveout, share));
     launch(k_rows_inner, grid, 32 * warps, RI_SMEM(warps), st, S, acc, ctx->d_twf,
            inv_special ? ctx->d_itw : nullptr, ctx->d_pc, level, ctx->n_q, ctx->n_p, ctx->alpha, beta, batch, groups,
            accumulate, separate ? 1 : 0, ctx->d_status);
