@@ -69,7 +69,7 @@ __device__ __forceinline__ u64 bconv_int(u64 lo, u64 hi, const PrimeConst& pc) {
 // grid = (N / 256, polynomials), 4 warps x 64 coefficients.
 // ---------------------------------------------------------------------------------------
 template <int TILES>
-__global__ void __launch_bounds__(32 * BC_WARPS, BC_MINB) k_moddown_conv_imma(const u64* __restrict__ acc, u64* __restrict__ u,
+__global__ void __launch_bounds__(32 * BC_WARPS, BC_MINB) k_moddown_conv_imma(const u64* acc, u64* u,
                                                                      const ModDownTab* __restrict__ tab, const uint4* __restrict__ frag,
                                                                      const PrimeConst* __restrict__ pcs, uint32_t N, uint32_t level,
                                                                      uint32_t n_q, uint32_t K, int out_double) {

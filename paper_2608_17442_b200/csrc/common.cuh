@@ -188,6 +188,8 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
 // waits, before it touches memory that a kernel writes, until everything before it on the stream has completed.  A key
 // switch of one ciphertext is a chain of 10 launches of 5 to 70 us; the hand-overs cost 1 to 2 us less each (one rotation
 // 303 -> 289 us).
+// Buffers that kernels write are passed to these kernels without __restrict__: a read-only __restrict__ parameter is read through the
+// read-only path, whose loads the compiler takes for constant and may move ahead of the wait.  Tables of the context may carry it.
 // ---------------------------------------------------------------------------------------
 __device__ __forceinline__ void pdl_begin() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -404,13 +406,13 @@ __device__ __forceinline__ uint32_t galois_src(uint32_t t, uint32_t log_n, u64 g
 }
 
 // the words that the automorphism takes to t and t + 1 (t even): it maps aligned pairs to aligned pairs, in either order
-__device__ __forceinline__ ulonglong2 galois_pair(const u64* __restrict__ in, uint32_t t, uint32_t log_n, u64 g, bool wide) {
+__device__ __forceinline__ ulonglong2 galois_pair(const u64* in, uint32_t t, uint32_t log_n, u64 g, bool wide) {
     const uint32_t src = galois_src(t, log_n, g);
     const ulonglong2 v = ld_pair(in + (src & ~1u), wide);
     return src & 1 ? make_ulonglong2(v.y, v.x) : v;
 }
 template <bool WIDE>
-__device__ __forceinline__ ulonglong2 galois_pair(const u64* __restrict__ in, uint32_t t, uint32_t log_n, u64 g) {
+__device__ __forceinline__ ulonglong2 galois_pair(const u64* in, uint32_t t, uint32_t log_n, u64 g) {
     const uint32_t src = galois_src(t, log_n, g);
     const ulonglong2 v = ld_pair_once<WIDE>(in + (src & ~1u));
     return src & 1 ? make_ulonglong2(v.y, v.x) : v;

@@ -9,7 +9,7 @@
 
 // out[b] = ct[b] (.) pt[b] on both polynomials (pt_stride words between plaintexts)
 // (out may be ct itself: every thread reads its words before it writes them)
-__global__ void __launch_bounds__(256) k_ct_mul_pt(const u64* ct, size_t ct_stride, const u64* __restrict__ pt,
+__global__ void __launch_bounds__(256) k_ct_mul_pt(const u64* ct, size_t ct_stride, const u64* pt,
                                                    size_t pt_stride, u64* out, size_t out_stride,
                                                    const PrimeConst* __restrict__ pcs, uint32_t N, uint32_t level) {
     pdl_begin();

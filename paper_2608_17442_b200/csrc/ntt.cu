@@ -31,7 +31,7 @@ __device__ __forceinline__ void gs_bfly(u64& x, u64& y, const Tw& t, u64 q, u64 
 // N <= 2^9: one CTA per row, radix-2 stages in shared memory.
 // ---------------------------------------------------------------------------------------
 template <bool INV>
-__global__ void __launch_bounds__(256) ntt_small(u64* __restrict__ data, const ulonglong2* __restrict__ tw_all,
+__global__ void __launch_bounds__(256) ntt_small(u64* data, const ulonglong2* __restrict__ tw_all,
                                                  const PrimeConst* __restrict__ pcs, RowMap map, uint32_t log_n) {
     pdl_begin();
     const uint32_t row = blockIdx.x;

@@ -32,8 +32,8 @@ __device__ __forceinline__ uint32_t list_row(const RowList& list, uint32_t y, ui
 // grid = (256 / NTT_COLS, rows)
 template <int A>
 __global__ void __launch_bounds__(COL_THREADS, 1024 / COL_THREADS)
-    ntt16_cols_fwd(u64* __restrict__ data, const void* __restrict__ tw, const PrimeConst* __restrict__ pcs, const __grid_constant__ PrimeDoubles pd, RowList list,
-                   uint32_t y0, int in_double, const u64* __restrict__ centred, double centred_q) {
+    ntt16_cols_fwd(u64* data, const void* __restrict__ tw, const PrimeConst* __restrict__ pcs, const __grid_constant__ PrimeDoubles pd, RowList list,
+                   uint32_t y0, int in_double, const u64* centred, double centred_q) {
     pdl_begin();
     __shared__ u64 sm[COL_SMEM(NTT_COLS)];
     uint32_t pi;
@@ -73,7 +73,7 @@ __global__ void __launch_bounds__(COL_THREADS, 1024 / COL_THREADS)
 
 template <int A>
 __global__ void __launch_bounds__(COL_THREADS, 1024 / COL_THREADS)
-    ntt16_cols_inv(u64* __restrict__ data, const void* __restrict__ tw, const PrimeConst* __restrict__ pcs, const __grid_constant__ PrimeDoubles pd, RowList list, uint32_t y0,
+    ntt16_cols_inv(u64* data, const void* __restrict__ tw, const PrimeConst* __restrict__ pcs, const __grid_constant__ PrimeDoubles pd, RowList list, uint32_t y0,
                    const InvScale* __restrict__ scale) {
     pdl_begin();
     __shared__ u64 sm[COL_SMEM(NTT_COLS)];
@@ -118,7 +118,7 @@ __global__ void __launch_bounds__(COL_THREADS, 1024 / COL_THREADS)
 // WIDE: every buffer lies on a 16-byte boundary (a template and not a flag: tests of a flag at every access cost 0.4 % of a rotation)
 template <int A, int FIN, bool WIDE>
 __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
-    ntt16_rows_fwd(u64* __restrict__ data, const void* __restrict__ tw, const PrimeConst* __restrict__ pcs, const __grid_constant__ PrimeDoubles pd, RowList list,
+    ntt16_rows_fwd(u64* data, const void* __restrict__ tw, const PrimeConst* __restrict__ pcs, const __grid_constant__ PrimeDoubles pd, RowList list,
                    uint32_t y0, int out_double, NttFinish fin) {
     pdl_begin();
     __shared__ __align__(16) u64 sm_all[NTT_WARPS * ROW_SMEM];
@@ -219,7 +219,7 @@ __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
 
 template <int A, bool SRC, bool WIDE>
 __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
-    ntt16_rows_inv(u64* __restrict__ data, const void* __restrict__ tw, const PrimeConst* __restrict__ pcs, const __grid_constant__ PrimeDoubles pd, RowList list, uint32_t y0,
+    ntt16_rows_inv(u64* data, const void* __restrict__ tw, const PrimeConst* __restrict__ pcs, const __grid_constant__ PrimeDoubles pd, RowList list, uint32_t y0,
                    NttSource src) {
     pdl_begin();
     __shared__ __align__(16) u64 sm_all[NTT_WARPS * ROW_SMEM];

@@ -7,8 +7,8 @@
 // ---------------------------------------------------------------------------------------
 // ct-pt multiply-accumulate:  acc[b][p][l][c] += ct[b][p][l][c] * pt[b][l][c]
 // ---------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_ct_pt_mac(const u64* __restrict__ ct, const u64* __restrict__ pt, size_t pt_stride,
-                                                   u64* __restrict__ acc, const PrimeConst* __restrict__ pcs,
+__global__ void __launch_bounds__(256) k_ct_pt_mac(const u64* ct, const u64* pt, size_t pt_stride,
+                                                   u64* acc, const PrimeConst* __restrict__ pcs,
                                                    uint32_t N, uint32_t n_limbs) {
     pdl_begin();
     const uint32_t c = blockIdx.x * blockDim.x + threadIdx.x;
@@ -20,12 +20,12 @@ __global__ void __launch_bounds__(256) k_ct_pt_mac(const u64* __restrict__ ct, c
     if (!DBG_REGION(pt + (size_t)b * pt_stride + (size_t)l * N, N * sizeof(u64))) return;
     for (int p = 0; p < 2; p++)
         if (!DBG_REGION(ct + o - c + p * poly, N * sizeof(u64)) || !DBG_REGION(acc + o - c + p * poly, N * sizeof(u64))) return;
-    const u64 w = pt[(size_t)b * pt_stride + (size_t)l * N + c];
+    const u64 w = pt[(size_t)b * pt_stride + (size_t)l * N + c], x[2] = {ct[o], ct[o + poly]};
+    acc128 a[2] = {{acc[o], 0}, {acc[o + poly], 0}};
 #pragma unroll
     for (int p = 0; p < 2; p++) {
-        acc128 a{acc[o + p * poly], 0};
-        mac128(a, ct[o + p * poly], w);
-        acc[o + p * poly] = reduce128(a.hi, a.lo, pc);
+        mac128(a[p], x[p], w);
+        acc[o + p * poly] = reduce128(a[p].hi, a[p].lo, pc);
     }
 }
 
@@ -50,8 +50,8 @@ extern "C" int fesc_ct_pt_mac(fesc_ctx* ctx, const uint64_t* d_ct, const uint64_
 // accumulators stay in registers (a ct-pt MAC per term reads and writes them every time).  Two coefficients per thread.
 // Products are below 2^124: up to 16 of them fit 128 bits.
 // ---------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_masked_sum(MaskedSum s, size_t src_stride, size_t pt_stride, const u64* __restrict__ add, size_t add_stride,
-                                                    u64* __restrict__ out, size_t out_stride, const PrimeConst* __restrict__ pcs, uint32_t N,
+__global__ void __launch_bounds__(256) k_masked_sum(MaskedSum s, size_t src_stride, size_t pt_stride, const u64* add, size_t add_stride,
+                                                    u64* out, size_t out_stride, const PrimeConst* __restrict__ pcs, uint32_t N,
                                                     uint32_t level) {
     pdl_begin();
     const uint32_t c = 2 * (blockIdx.x * blockDim.x + threadIdx.x), l = blockIdx.y, b = blockIdx.z;
@@ -129,8 +129,8 @@ extern "C" int fesc_intt(fesc_ctx* ctx, uint64_t* d_data, uint32_t batch, uint32
 // c0 goes to out0 (the result's first polynomial), c1 goes to BOTH d (kept in EVAL form for
 // the digit's own limbs) and dcoef (transformed in place afterwards).
 // ---------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_autom_ct(const u64* __restrict__ in, size_t in_stride, u64* __restrict__ out0,
-                                                  size_t out_stride, OwnRows d, u64* __restrict__ dcoef,
+__global__ void __launch_bounds__(256) k_autom_ct(const u64* in, size_t in_stride, u64* out0,
+                                                  size_t out_stride, OwnRows d, u64* dcoef,
                                                   uint32_t log_n, uint32_t level, u64 g,
                                                   const PrimeConst* __restrict__ pcs, int accumulate) {
     pdl_begin();
@@ -166,7 +166,7 @@ __global__ void __launch_bounds__(256) k_autom_ct(const u64* __restrict__ in, si
 // ---------------------------------------------------------------------------------------
 // VEC (1, 2 or 4) adjacent words with 16-byte accesses where possible
 template <int VEC>
-__device__ __forceinline__ void ldv(const u64* __restrict__ src, u64 (&w)[VEC]) {
+__device__ __forceinline__ void ldv(const u64* src, u64 (&w)[VEC]) {
     if (VEC == 1) {
         w[0] = *src;
     } else {
@@ -178,7 +178,7 @@ __device__ __forceinline__ void ldv(const u64* __restrict__ src, u64 (&w)[VEC]) 
     }
 }
 template <int VEC>
-__device__ __forceinline__ void stv(u64* __restrict__ dst, const u64 (&r)[VEC]) {
+__device__ __forceinline__ void stv(u64* dst, const u64 (&r)[VEC]) {
     if (VEC == 1) {
         *dst = r[0];
     } else {
@@ -188,7 +188,7 @@ __device__ __forceinline__ void stv(u64* __restrict__ dst, const u64 (&r)[VEC]) 
 }
 
 template <int ALPHA, int VEC>
-__global__ void __launch_bounds__(256) k_modup(const u64* __restrict__ dcoef, u64* __restrict__ ext,
+__global__ void __launch_bounds__(256) k_modup(const u64* dcoef, u64* ext,
                                                const ModUpDigit* __restrict__ tab, const PrimeConst* __restrict__ pcs,
                                                uint32_t N, uint32_t level, uint32_t n_q, uint32_t K, uint32_t beta,
                                                int out_double) {
@@ -458,7 +458,7 @@ struct InnerKeys {
     uint32_t n;
 };
 template <int BETA, bool FP>
-__global__ void __launch_bounds__(256, 4) k_inner_shared(const u64* __restrict__ ext, InnerKeys keys, u64* __restrict__ acc,
+__global__ void __launch_bounds__(256, 4) k_inner_shared(const u64* ext, InnerKeys keys, u64* acc,
                                                          const PrimeConst* __restrict__ pcs, uint32_t level, uint32_t n_q, uint32_t K,
                                                          uint32_t batch, uint32_t row0) {
     pdl_begin();
@@ -571,8 +571,8 @@ extern "C" int fesc_selftest_wait_limit(fesc_ctx* ctx, void* stream) {
 }
 
 template <int BT>
-__global__ void __launch_bounds__(256, 1) k_inner_tma(const u64* __restrict__ ext,
-                                                      const u64* __restrict__ key, u64* __restrict__ acc,
+__global__ void __launch_bounds__(256, 1) k_inner_tma(const u64* ext,
+                                                      const u64* key, u64* acc,
                                                       const PrimeConst* __restrict__ pcs, uint32_t N, uint32_t level,
                                                       uint32_t n_q, uint32_t K, uint32_t alpha, uint32_t beta,
                                                       uint32_t batch, uint32_t log_n, u64 g, int accumulate,
@@ -743,7 +743,7 @@ __global__ void __launch_bounds__(256, 1) k_inner_tma(const u64* __restrict__ ex
 //   u_i = sum_k y_k (P/p_k) mod q_i = sum_k [y_k]_canonical (P/p_k) - #{y_k > p_k/2} * P  (mod q_i).
 // ---------------------------------------------------------------------------------------
 template <int VEC>
-__global__ void __launch_bounds__(256) k_moddown_conv(const u64* __restrict__ acc, u64* __restrict__ u,
+__global__ void __launch_bounds__(256) k_moddown_conv(const u64* acc, u64* u,
                                                       const ModDownTab* __restrict__ tab,
                                                       const PrimeConst* __restrict__ pcs, uint32_t N, uint32_t level,
                                                       uint32_t n_q, uint32_t K, int out_double) {
@@ -821,8 +821,8 @@ __global__ void __launch_bounds__(256) k_moddown_conv(const u64* __restrict__ ac
 }
 
 // out[b][p][i] = (acc[b][p][i] - u[b][p][i]) * P^-1 + add[b][p][i]   (all EVAL)
-__global__ void __launch_bounds__(256) k_moddown_finish(const u64* __restrict__ acc, const u64* __restrict__ u,
-                                                        u64* __restrict__ out, size_t out_stride,
+__global__ void __launch_bounds__(256) k_moddown_finish(const u64* acc, const u64* u,
+                                                        u64* out, size_t out_stride,
                                                         const ModDownTab* __restrict__ tab,
                                                         const PrimeConst* __restrict__ pcs, uint32_t N, uint32_t level,
                                                         uint32_t K, int add_mask) {
@@ -1268,8 +1268,8 @@ int rotate_multi_internal(fesc_ctx* ctx, const u64* in, size_t in_stride, size_t
 }
 
 // c0 of every ciphertext through the Galois permutation into out[b][0]; with g == 0, c1 copied to d and dcoef
-__global__ void __launch_bounds__(256) k_hoist_prepare(const u64* __restrict__ in, size_t in_stride, u64* __restrict__ out0,
-                                                       size_t out_stride, OwnRows d, u64* __restrict__ dcoef,
+__global__ void __launch_bounds__(256) k_hoist_prepare(const u64* in, size_t in_stride, u64* out0,
+                                                       size_t out_stride, OwnRows d, u64* dcoef,
                                                        uint32_t log_n, uint32_t level, u64 g,
                                                        const PrimeConst* __restrict__ pcs) {
     pdl_begin();
@@ -1420,7 +1420,7 @@ struct GaloisSet {
 };
 // Two coefficients per thread and 16-byte accesses: a permutation maps aligned pairs to aligned pairs (either order).  75 limb rows and
 // 3 elements: 62 -> 41 us.
-__global__ void __launch_bounds__(256) k_rotsum_prepare(const u64* __restrict__ in, size_t in_stride, u64* __restrict__ out,
+__global__ void __launch_bounds__(256) k_rotsum_prepare(const u64* in, size_t in_stride, u64* out,
                                                         size_t out_stride, uint32_t log_n, uint32_t level, GaloisSet gs,
                                                         const PrimeConst* __restrict__ pcs) {
     pdl_begin();
@@ -1526,7 +1526,7 @@ extern "C" int fesc_rotate(fesc_ctx* ctx, const uint64_t* d_in, uint64_t* d_out,
 // Rescale
 // ---------------------------------------------------------------------------------------
 // gather the last limb of every polynomial into r[b*2+p][N]
-__global__ void __launch_bounds__(256) k_take_last(const u64* __restrict__ in, size_t in_stride, u64* __restrict__ r,
+__global__ void __launch_bounds__(256) k_take_last(const u64* in, size_t in_stride, u64* r,
                                                    uint32_t N, uint32_t level) {
     pdl_begin();
     const uint32_t c = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1538,7 +1538,7 @@ __global__ void __launch_bounds__(256) k_take_last(const u64* __restrict__ in, s
     r[(size_t)bp * N + c] = in[(size_t)(bp >> 1) * in_stride + ((size_t)(bp & 1) * level + level - 1) * N + c];
 }
 // out[b][p][i] = centred(r) mod q_i  (COEFF)
-__global__ void __launch_bounds__(256) k_rescale_conv(const u64* __restrict__ r, u64* __restrict__ out, size_t out_stride,
+__global__ void __launch_bounds__(256) k_rescale_conv(const u64* r, u64* out, size_t out_stride,
                                                       const RescaleTab* __restrict__ tab,
                                                       const PrimeConst* __restrict__ pcs, uint32_t N, uint32_t level) {
     pdl_begin();
@@ -1556,8 +1556,8 @@ __global__ void __launch_bounds__(256) k_rescale_conv(const u64* __restrict__ r,
     out[(size_t)(bp >> 1) * out_stride + ((size_t)(bp & 1) * (level - 1) + i) * N + c] = w;
 }
 // out = (in - out) * q_last^-1
-__global__ void __launch_bounds__(256) k_rescale_finish(const u64* __restrict__ in, size_t in_stride,
-                                                        u64* __restrict__ out, size_t out_stride,
+__global__ void __launch_bounds__(256) k_rescale_finish(const u64* in, size_t in_stride,
+                                                        u64* out, size_t out_stride,
                                                         const RescaleTab* __restrict__ tab,
                                                         const PrimeConst* __restrict__ pcs, uint32_t N, uint32_t level) {
     pdl_begin();
@@ -1678,8 +1678,8 @@ __device__ __forceinline__ void tensor_word_fp(u64 a0, u64 a1, u64 b0, u64 b1, d
     d2 = fp_store(fp_modmul(x1, y1, q, qinv), q, qinv);
 }
 __global__ void __launch_bounds__(256) k_tensor(const u64* a, size_t a_stride, const u64* bb,
-                                                size_t b_stride, u64* __restrict__ out, size_t out_stride,
-                                                OwnRows d, u64* __restrict__ dcoef,
+                                                size_t b_stride, u64* out, size_t out_stride,
+                                                OwnRows d, u64* dcoef,
                                                 const PrimeConst* __restrict__ pcs, uint32_t N, uint32_t level) {
     pdl_begin();
     const uint32_t c = 2 * (blockIdx.x * blockDim.x + threadIdx.x);

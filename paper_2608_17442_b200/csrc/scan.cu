@@ -20,8 +20,8 @@
 // pointwise kernels on batches of compact ciphertexts [2][level][N]
 // ---------------------------------------------------------------------------------------
 // out = a + b (sub = 0) or a - b (sub = 1); b_stride may be 0
-__global__ void __launch_bounds__(256) k_ct_addsub(const u64* __restrict__ a, size_t a_stride, const u64* __restrict__ b,
-                                                   size_t b_stride, u64* __restrict__ out, size_t out_stride,
+__global__ void __launch_bounds__(256) k_ct_addsub(const u64* a, size_t a_stride, const u64* b,
+                                                   size_t b_stride, u64* out, size_t out_stride,
                                                    const PrimeConst* __restrict__ pcs, uint32_t N, uint32_t level,
                                                    int sub) {
     pdl_begin();
@@ -37,8 +37,8 @@ __global__ void __launch_bounds__(256) k_ct_addsub(const u64* __restrict__ a, si
     out[bi * out_stride + o] = sub ? submod(x, y, q) : addmod(x, y, q);
 }
 // out[b] = ct[b] (.) pt[b]  (pt [level][N]; pt_stride = 0: one plaintext for the batch; a_stride = 0: one ciphertext)
-__global__ void __launch_bounds__(256) k_ct_ptmul(const u64* __restrict__ a, size_t a_stride, const u64* __restrict__ pt,
-                                                  size_t pt_stride, u64* __restrict__ out, size_t out_stride,
+__global__ void __launch_bounds__(256) k_ct_ptmul(const u64* a, size_t a_stride, const u64* pt,
+                                                  size_t pt_stride, u64* out, size_t out_stride,
                                                   const PrimeConst* __restrict__ pcs, uint32_t N, uint32_t level) {
     pdl_begin();
     const uint32_t c = blockIdx.x * blockDim.x + threadIdx.x;
@@ -50,12 +50,12 @@ __global__ void __launch_bounds__(256) k_ct_ptmul(const u64* __restrict__ a, siz
     for (int p = 0; p < 2; p++)
         if (!DBG_REGION(a + bi * a_stride + p * poly + o - c, N * sizeof(u64)) || !DBG_REGION(out + bi * out_stride + p * poly + o - c, N * sizeof(u64)))
             return;
-    const u64 w = pt[bi * pt_stride + o];
-    out[bi * out_stride + o] = mulmod(a[bi * a_stride + o], w, pc);
-    out[bi * out_stride + poly + o] = mulmod(a[bi * a_stride + poly + o], w, pc);
+    const u64 w = pt[bi * pt_stride + o], x0 = a[bi * a_stride + o], x1 = a[bi * a_stride + poly + o];
+    out[bi * out_stride + o] = mulmod(x0, w, pc);
+    out[bi * out_stride + poly + o] = mulmod(x1, w, pc);
 }
 // keep the first `keep` limbs of a level-`src` ciphertext and multiply them by the integer k
-__global__ void __launch_bounds__(256) k_ct_scale_drop(const u64* __restrict__ a, size_t a_stride, u64* __restrict__ out,
+__global__ void __launch_bounds__(256) k_ct_scale_drop(const u64* a, size_t a_stride, u64* out,
                                                        size_t out_stride, const PrimeConst* __restrict__ pcs, uint32_t N,
                                                        uint32_t src, uint32_t keep, u64 k) {
     pdl_begin();
@@ -72,7 +72,7 @@ __global__ void __launch_bounds__(256) k_ct_scale_drop(const u64* __restrict__ a
 }
 // multiply by the monomial X^(N/2) `times` times (times = 1: slots * i; times = 3: slots * -i).
 // In evaluation order X^(N/2) is I = psi^(N/2) on the first half of the indices and -I on the second.
-__global__ void __launch_bounds__(256) k_ct_mul_i(const u64* __restrict__ a, size_t a_stride, u64* __restrict__ out,
+__global__ void __launch_bounds__(256) k_ct_mul_i(const u64* a, size_t a_stride, u64* out,
                                                   size_t out_stride, const PrimeConst* __restrict__ pcs,
                                                   const ulonglong2* __restrict__ tw, uint32_t N, uint32_t level,
                                                   int times) {
@@ -92,8 +92,8 @@ __global__ void __launch_bounds__(256) k_ct_mul_i(const u64* __restrict__ a, siz
     out[bi * out_stride + o] = (neg && v) ? q - v : v;
 }
 // acc += sum over the batch
-__global__ void __launch_bounds__(256) k_ct_sum_into(const u64* __restrict__ a, size_t a_stride, uint32_t count,
-                                                     u64* __restrict__ acc, const PrimeConst* __restrict__ pcs,
+__global__ void __launch_bounds__(256) k_ct_sum_into(const u64* a, size_t a_stride, uint32_t count,
+                                                     u64* acc, const PrimeConst* __restrict__ pcs,
                                                      uint32_t N, uint32_t level) {
     pdl_begin();
     const uint32_t c = blockIdx.x * blockDim.x + threadIdx.x;

@@ -38,7 +38,7 @@ __device__ __forceinline__ void small_tables(u64* sm, const SmallTables& tb, uin
         for (int k = 0; k < 8; k++) dst[k * T + threadIdx.x] = __ldg(src + k * T + threadIdx.x);
     }
 }
-// (Buffers that kernels write carry no __restrict__: reads through the read-only path may be moved ahead of the wait.)
+// (No __restrict__ on buffers that kernels write: see pdl_begin.)
 #define SMALL_BEGIN(used, pi, inv)                                  \
     extern __shared__ __align__(16) u64 sm[];                       \
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); \
