@@ -179,6 +179,15 @@ __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t
                  "l"(src), "r"(bytes), "r"(bar) : "memory");
 }
 
+// Between the last reads of words in shared memory and a bulk copy over them.  The copy's issuer executes it after its own reads and those that a
+// barrier has ordered before it; other readers execute it before they count themselves out.
+__device__ __forceinline__ void before_refill() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+// Counts up to `last` and wraps; the one who sees `last` comes after the reads of all who counted before.
+__device__ __forceinline__ uint32_t count_readers(uint32_t counter, uint32_t last) {
+    uint32_t seen;
+    asm volatile("atom.acq_rel.cta.shared::cta.inc.u32 %0, [%1], %2;" : "=r"(seen) : "r"(counter), "r"(last) : "memory");
+    return seen;
+}
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }

@@ -170,7 +170,10 @@ __global__ void __launch_bounds__(32 * RI_WARPS, 4)
 #pragma unroll
             for (int k = 0; k < 16; k++) x[k] = FpRow::value(in[16 * k]);
             __syncwarp();                               // the staged points and the previous digit's values have been read
-            if (lane == 0 && n + 1 < total) load_x(s_next, j_next);
+            if (lane == 0 && n + 1 < total) {
+                before_refill();
+                load_x(s_next, j_next);
+            }
             fwd_rows<false>(r, x, sm, blk, lane);
         }
         if (mbar_wait_bounded(key_full, n & 1)) {
@@ -192,9 +195,9 @@ __global__ void __launch_bounds__(32 * RI_WARPS, 4)
         if (n + 1 < total) {
             __syncwarp();
             if (lane == 0) {
+                before_refill();
                 if (j == own) load_x(s_next, j_next);
-                // the last warp to have read the key words requests the next ones
-                if (atomicInc(reinterpret_cast<uint32_t*>(smem + RI_KEY_WORDS + warps * RI_WARP_WORDS + warps + 1), last) == last) load_keys(s_next, j_next);
+                if (count_readers(key_full + 8, last) == last) load_keys(s_next, j_next);      // the last warp to have read the key words requests the next ones
             }
         }
         s = s_next, j = j_next;

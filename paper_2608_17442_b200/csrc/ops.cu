@@ -615,7 +615,7 @@ __global__ void __launch_bounds__(256, 1) k_inner_tma(const u64* ext,
             }
         }
 #endif
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // earlier reads of this half precede the refill
+        before_refill();
         mbar_expect_tx(bar, stage_words * 8);
         for (uint32_t j = 0; j < beta; j++) {
             bulk_g2s(dst, key + ((size_t)(2 * j) * np + pt) * N + (cblk << 8), 2048, bar);

@@ -53,3 +53,17 @@ def test_kernels_that_start_early_read_no_written_buffer_through_the_read_only_p
             continue
         bad = [p.strip() for p in params.split(",") if "__restrict__" in p and re.search(r"\b(u64|uint64_t|uint8_t)\b", p)]
         assert not bad, (name, bad)
+
+
+def test_words_that_were_read_are_handed_to_bulk_copies_in_order():
+    """k_rows_inner and k_inner_tma refill shared memory that other threads have read: the copies belong to the asynchronous proxy, and the
+    one who starts them learns that the others are done from a count that releases and acquires (or from a CTA barrier)."""
+    seen = 0
+    for f in ("inner16.cu", "ops.cu"):
+        for name, _, body in functions(open(os.path.join(CSRC, f)).read(), r"__global__ void"):
+            if "bulk_g2s(" in body:
+                seen += 1
+                assert "before_refill()" in body and not re.search(r"\batomic(Inc|Add)\(", body), name
+    assert seen == 2
+    common = open(os.path.join(CSRC, "common.cuh")).read()
+    assert "atom.acq_rel.cta.shared::cta.inc.u32" in common and "fence.proxy.async.shared::cta" in common
