@@ -458,6 +458,10 @@ __global__ void __launch_bounds__(MIX_THREADS, (TT * PT >= 12 ? 256 / MIX_THREAD
 #define IM_ROWP 9                      // words per (row, 8 coefficients): one word of padding
 #define IM_BPP (32 * IM_ROWP + 1)      // words between the (b,p) blocks of a stage (= 1 mod 16: conflict-free fragment loads)
 #define IM_STAGE_WORDS (8 * IM_BPP)
+#define IM_DEEP_TERMS 128              // sums of so many terms leave room for 8 stages
+#define IM_ROWS(terms) (((terms) + 31) / 32 * 32 * IM_ROWP)
+#define IM_PITCH(terms) (IM_ROWS(terms) + (17 - IM_ROWS(terms) % 16) % 16)      // = 1 mod 16
+#define IM_SMEM(pitch, st) (((size_t)8 * (pitch) + (size_t)(st) * IM_STAGE_WORDS) * 8)
 
 __device__ __forceinline__ void cp_async8z(uint32_t smem_dst, const void* gmem_src, bool valid) {
     const uint32_t n = valid ? 8u : 0u;      // 0 source bytes: the destination is filled with zeros
@@ -869,13 +873,13 @@ extern "C" int fesc_linear(fesc_ctx* ctx, const uint64_t* d_ct_in, const uint64_
     } while (0)
 #define BSGS_IMMA(ST)                                                                                           \
     do {                                                                                                      \
-        const uint32_t tp = ((gin * n1 + 31) / 32) * 32;                                                      \
-        uint32_t pitch = tp * IM_ROWP;                                                                        \
-        pitch += (17 - pitch % 16) % 16;          /* = 1 mod 16 */                                            \
+        const uint32_t pitch = IM_PITCH(gin * n1);                                                            \
         dim3 grid(N / IM_CW, level, (nt + 3) / 4);                                                            \
-        const size_t smem = ((size_t)8 * pitch + (size_t)ST * IM_STAGE_WORDS) * 8;                            \
+        const size_t smem = IM_SMEM(pitch, ST);                                                               \
         auto kern = k_bsgs_accumulate_imma<ST>;                                                               \
-        FESC_CHECK_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)); \
+        /* the limit is the process's, not the call's: the largest of this variant, the same from every thread */ \
+        const int most = IM_SMEM(IM_PITCH(ST == 8 ? IM_DEEP_TERMS : 256), ST);                                \
+        FESC_CHECK_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, most));  \
         kern<<<grid, 32 * IM_CW, smem, st>>>(rot, diags, acc, ctx->d_pc, N, level, nt, gin * n1, bp_count, pitch); \
     } while (0)
         const bool fp_ok = qbits <= 50 && bsgs_kernel() != 2;
@@ -885,7 +889,7 @@ extern "C" int fesc_linear(fesc_ctx* ctx, const uint64_t* d_ct_in, const uint64_
         // byte planes against 128-bit integer sums.
         const bool mixed_ok = fp_ok && (bsgs_kernel() == 0 || bsgs_kernel() == 3) && N % 256 == 0 && gin * n1 <= 256;
         const bool imma_ok = bsgs_kernel() == 0 && !fp_ok && qbits <= 56 && N % IM_CW == 0 && gin * n1 <= 256 && level <= 65535;
-        const bool deep = gin * n1 <= 128;       // room for 8 stages beside the rotated inputs
+        const bool deep = gin * n1 <= IM_DEEP_TERMS;       // room for 8 stages beside the rotated inputs
         if (mixed_ok && nt >= 2) BSGS_MIX(2, 8, 3);
         else if (mixed_ok) BSGS_MIX(1, 8, 4);
         else if (imma_ok && deep) BSGS_IMMA(8);

@@ -452,6 +452,7 @@ __global__ void __launch_bounds__(256, INNER_MINB) k_inner(InnerSrcs S, u64* acc
 // ---------------------------------------------------------------------------------------
 #define IS_BLK 64                 // coefficients per CTA
 #define IS_MAX_DIGITS 8
+#define IS_MAX_BATCH 16
 struct InnerKeys {
     const u64* key[KS_MAX_KEYS];
     u64 g[KS_MAX_KEYS], ginv[KS_MAX_KEYS];
@@ -950,10 +951,11 @@ static int ks_inner_multi(fesc_ctx* ctx, const KsScratch& ws, const InnerSrcs& S
     if (use_tma && N % 256 == 0 && beta <= 8 && batch >= 3) {   // 128-bit sums of <= 8 products below 2^124 cannot wrap
         const uint32_t n_tiles = rows * (N >> 8) * ((batch + 3) / 4);
         const size_t smem = (size_t)2 * beta * 6 * 2048 + 16;
+        const int most = 2 * 8 * 6 * 2048 + 16;             // the same from every thread of the process
         int dev = 0, sms = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        FESC_CHECK_CUDA(ctx, cudaFuncSetAttribute(k_inner_tma<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        FESC_CHECK_CUDA(ctx, cudaFuncSetAttribute(k_inner_tma<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
         const uint32_t grid = n_tiles < (uint32_t)sms ? n_tiles : (uint32_t)sms;
         launch(k_inner_tma<4>, grid, 256, smem, st, S.s[0].ext, S.s[0].key, ws.acc, ctx->d_pc, N, level, nq, K, alpha, beta,
                                                  batch, ctx->log_n, S.s[0].g, accumulate, n_tiles, ctx->d_status, ctx->log_n == 16);
@@ -991,8 +993,10 @@ static int inner_shared_launch(fesc_ctx* ctx, const KsScratch& ws, const InnerKe
     const size_t smem = (size_t)batch * BETA * IS_BLK * sizeof(u64);
     auto fp = k_inner_shared<BETA, true>;
     auto in = k_inner_shared<BETA, false>;
-    FESC_CHECK_CUDA(ctx, cudaFuncSetAttribute(fp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    FESC_CHECK_CUDA(ctx, cudaFuncSetAttribute(in, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    // the limit is the process's, not the call's: the same from every thread, whatever its batch
+    const int most = IS_MAX_BATCH * BETA * IS_BLK * sizeof(u64);
+    FESC_CHECK_CUDA(ctx, cudaFuncSetAttribute(fp, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+    FESC_CHECK_CUDA(ctx, cudaFuncSetAttribute(in, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
     launch(fp, dim3(65536 / IS_BLK, level), 256, smem, st, ws.ext, ik, ws.acc, ctx->d_pc, level, ctx->n_q, ctx->n_p, batch, 0u);
     launch(in, dim3(65536 / IS_BLK, ctx->n_p), 256, smem, st, ws.ext, ik, ws.acc, ctx->d_pc, level, ctx->n_q, ctx->n_p, batch, level);
     return FESC_OK;
@@ -1018,7 +1022,7 @@ static int ks_keys(fesc_ctx* ctx, const char* who, const uint32_t* ids, uint32_t
 static int ks_inner_hoisted(fesc_ctx* ctx, const KsScratch& ws, const KsKeys& keys, uint32_t k0, uint32_t n, uint32_t level, uint32_t batch,
                             cudaStream_t st) {
     const uint32_t beta = (level + ctx->alpha - 1) / ctx->alpha;
-    if (n < 2 || ctx->log_n != 16 || beta > IS_MAX_DIGITS || batch > 16 || !rows_split(ctx, level)) {
+    if (n < 2 || ctx->log_n != 16 || beta > IS_MAX_DIGITS || batch > IS_MAX_BATCH || !rows_split(ctx, level)) {
         InnerSrcs S;
         S.n = n;
         for (uint32_t k = 0; k < n; k++) S.s[k] = InnerSrc{ws.ext, keys.key[k0 + k], keys.g[k0 + k]};

@@ -117,3 +117,40 @@ def test_products_of_the_largest_words(bits):
     got = to_host(out)
     assert np.array_equal(got[0], orc.ct_ct_mul(ct[0], ct[1]))
     assert np.array_equal(got[1], orc.ct_ct_mul(ct[0], ct[0]))
+
+
+def test_threads_with_contexts_of_their_own():
+    """Hoisted rotations of 1 and of 16 ciphertexts from two threads at a time: kernels whose shared memory depends on the call."""
+    import threading
+
+    import torch
+    import paper_2608_17442_b200 as fesc
+
+    args = (16, S.ntt_primes(50, 16, 8, 0) + S.ntt_primes(60, 16, 4, 0), 8, 4, 2, 64)
+    errors, results = [], {}
+    go = threading.Barrier(2)
+
+    def work(batch):
+        try:
+            torch.cuda.set_device(0)
+            with torch.cuda.stream(torch.cuda.Stream()):
+                ctx = fesc.Context(*args)
+                for k in (1, 2):
+                    ctx.add_galois_key(k, k)
+                ct = torch.arange(batch * 2 * 8 << 16, dtype=torch.int64, device="cuda").view(batch, 2, 8, 1 << 16)
+                out = torch.empty((2, batch, 2, 8, 1 << 16), dtype=torch.int64, device="cuda")
+                go.wait(60)
+                for _ in range(300 if batch == 16 else 3000):
+                    ctx.rotate_hoisted(ct, out, batch, 8, [1, 2])
+                ctx.sync()
+                results[batch] = out[:, 0].cpu()
+        except Exception as e:      # reported by the test, not by the thread
+            errors.append(e)
+
+    threads = [threading.Thread(target=work, args=(b,)) for b in (1, 16)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
+    assert torch.equal(results[1], results[16])       # the first ciphertext of both batches is the same
