@@ -29,10 +29,19 @@ __device__ __forceinline__ uint32_t list_row(const RowList& list, uint32_t y, ui
     return rep * list.period + list.row[e];
 }
 
+// Constants of the primes that a kernel takes by value: none for integer rows (1 KB of parameters is 0.1 us of a
+// launch: a rotation of one ciphertext of three 55-bit limbs 121.7 us with it, 120.5 without).
+template <int A>
+struct RowPrimes : PrimeDoubles {
+    explicit RowPrimes(const fesc_ctx* ctx) : PrimeDoubles(ctx->pd) {}
+};
+template <>
+struct RowPrimes<ROW_INT> {};
+
 // grid = (256 / NTT_COLS, rows)
 template <int A>
 __global__ void __launch_bounds__(COL_THREADS, 1024 / COL_THREADS)
-    ntt16_cols_fwd(u64* data, const void* __restrict__ tw, const PrimeConst* __restrict__ pcs, const __grid_constant__ PrimeDoubles pd, RowList list,
+    ntt16_cols_fwd(u64* data, const void* __restrict__ tw, const PrimeConst* __restrict__ pcs, const __grid_constant__ RowPrimes<A> pd, RowList list,
                    uint32_t y0, int in_double, const u64* centred, double centred_q) {
     pdl_begin();
     __shared__ u64 sm[COL_SMEM(NTT_COLS)];
@@ -73,7 +82,7 @@ __global__ void __launch_bounds__(COL_THREADS, 1024 / COL_THREADS)
 
 template <int A>
 __global__ void __launch_bounds__(COL_THREADS, 1024 / COL_THREADS)
-    ntt16_cols_inv(u64* data, const void* __restrict__ tw, const PrimeConst* __restrict__ pcs, const __grid_constant__ PrimeDoubles pd, RowList list, uint32_t y0,
+    ntt16_cols_inv(u64* data, const void* __restrict__ tw, const PrimeConst* __restrict__ pcs, const __grid_constant__ RowPrimes<A> pd, RowList list, uint32_t y0,
                    const InvScale* __restrict__ scale) {
     pdl_begin();
     __shared__ u64 sm[COL_SMEM(NTT_COLS)];
@@ -118,7 +127,7 @@ __global__ void __launch_bounds__(COL_THREADS, 1024 / COL_THREADS)
 // WIDE: every buffer lies on a 16-byte boundary (a template and not a flag: tests of a flag at every access cost 0.4 % of a rotation)
 template <int A, int FIN, bool WIDE>
 __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
-    ntt16_rows_fwd(u64* data, const void* __restrict__ tw, const PrimeConst* __restrict__ pcs, const __grid_constant__ PrimeDoubles pd, RowList list,
+    ntt16_rows_fwd(u64* data, const void* __restrict__ tw, const PrimeConst* __restrict__ pcs, const __grid_constant__ RowPrimes<A> pd, RowList list,
                    uint32_t y0, int out_double, NttFinish fin) {
     pdl_begin();
     __shared__ __align__(16) u64 sm_all[NTT_WARPS * ROW_SMEM];
@@ -219,7 +228,7 @@ __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
 
 template <int A, bool SRC, bool WIDE>
 __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
-    ntt16_rows_inv(u64* data, const void* __restrict__ tw, const PrimeConst* __restrict__ pcs, const __grid_constant__ PrimeDoubles pd, RowList list, uint32_t y0,
+    ntt16_rows_inv(u64* data, const void* __restrict__ tw, const PrimeConst* __restrict__ pcs, const __grid_constant__ RowPrimes<A> pd, RowList list, uint32_t y0,
                    NttSource src) {
     pdl_begin();
     __shared__ __align__(16) u64 sm_all[NTT_WARPS * ROW_SMEM];
@@ -319,22 +328,22 @@ static int launch_all(fesc_ctx* ctx, u64* data, size_t rows, const RowMap& map, 
             const uint32_t y = (uint32_t)y0;
             if (f == ROW_FP) {
                 if (inverse) {
-                    launch(source ? ntt16_rows_inv<ROW_FP, true, WIDE> : ntt16_rows_inv<ROW_FP, false, WIDE>, gr, ROW_THREADS, 0, st, data, ctx->d_itwf, ctx->d_pc, ctx->pd, l,
+                    launch(source ? ntt16_rows_inv<ROW_FP, true, WIDE> : ntt16_rows_inv<ROW_FP, false, WIDE>, gr, ROW_THREADS, 0, st, data, ctx->d_itwf, ctx->d_pc, RowPrimes<ROW_FP>(ctx), l,
                            y, src);
-                    if (!skip_cols) launch(ntt16_cols_inv<ROW_FP>, gc, COL_THREADS, 0, st, data, ctx->d_itwf, ctx->d_pc, ctx->pd, l, y, scale);
+                    if (!skip_cols) launch(ntt16_cols_inv<ROW_FP>, gc, COL_THREADS, 0, st, data, ctx->d_itwf, ctx->d_pc, RowPrimes<ROW_FP>(ctx), l, y, scale);
                 } else {
-                    if (!skip_cols) launch(ntt16_cols_fwd<ROW_FP>, gc, COL_THREADS, 0, st, data, ctx->d_twf, ctx->d_pc, ctx->pd, l, y, in_double, fin.centred, fin.centred_q);
-                    if (fin.pt || fin.mul) launch(ntt16_rows_fwd<ROW_FP, 2, WIDE>, gr, ROW_THREADS, 0, st, data, ctx->d_twf, ctx->d_pc, ctx->pd, l, y, out_double, fin);
-                    else if (fin.acc) launch(ntt16_rows_fwd<ROW_FP, 1, WIDE>, gr, ROW_THREADS, 0, st, data, ctx->d_twf, ctx->d_pc, ctx->pd, l, y, out_double, fin);
-                    else launch(ntt16_rows_fwd<ROW_FP, 0, WIDE>, gr, ROW_THREADS, 0, st, data, ctx->d_twf, ctx->d_pc, ctx->pd, l, y, out_double, fin);
+                    if (!skip_cols) launch(ntt16_cols_fwd<ROW_FP>, gc, COL_THREADS, 0, st, data, ctx->d_twf, ctx->d_pc, RowPrimes<ROW_FP>(ctx), l, y, in_double, fin.centred, fin.centred_q);
+                    if (fin.pt || fin.mul) launch(ntt16_rows_fwd<ROW_FP, 2, WIDE>, gr, ROW_THREADS, 0, st, data, ctx->d_twf, ctx->d_pc, RowPrimes<ROW_FP>(ctx), l, y, out_double, fin);
+                    else if (fin.acc) launch(ntt16_rows_fwd<ROW_FP, 1, WIDE>, gr, ROW_THREADS, 0, st, data, ctx->d_twf, ctx->d_pc, RowPrimes<ROW_FP>(ctx), l, y, out_double, fin);
+                    else launch(ntt16_rows_fwd<ROW_FP, 0, WIDE>, gr, ROW_THREADS, 0, st, data, ctx->d_twf, ctx->d_pc, RowPrimes<ROW_FP>(ctx), l, y, out_double, fin);
                 }
             } else if (inverse) {
-                launch(source ? ntt16_rows_inv<ROW_INT, true, WIDE> : ntt16_rows_inv<ROW_INT, false, WIDE>, gr, ROW_THREADS, 0, st, data, ctx->d_itw, ctx->d_pc, ctx->pd, l, y,
+                launch(source ? ntt16_rows_inv<ROW_INT, true, WIDE> : ntt16_rows_inv<ROW_INT, false, WIDE>, gr, ROW_THREADS, 0, st, data, ctx->d_itw, ctx->d_pc, RowPrimes<ROW_INT>(), l, y,
                        src);
-                if (!skip_cols) launch(ntt16_cols_inv<ROW_INT>, gc, COL_THREADS, 0, st, data, ctx->d_itw, ctx->d_pc, ctx->pd, l, y, scale);
+                if (!skip_cols) launch(ntt16_cols_inv<ROW_INT>, gc, COL_THREADS, 0, st, data, ctx->d_itw, ctx->d_pc, RowPrimes<ROW_INT>(), l, y, scale);
             } else {
-                if (!skip_cols) launch(ntt16_cols_fwd<ROW_INT>, gc, COL_THREADS, 0, st, data, ctx->d_tw, ctx->d_pc, ctx->pd, l, y, 0, nullptr, 0.0);
-                launch(ntt16_rows_fwd<ROW_INT, 0, WIDE>, gr, ROW_THREADS, 0, st, data, ctx->d_tw, ctx->d_pc, ctx->pd, l, y, 0, fin);
+                if (!skip_cols) launch(ntt16_cols_fwd<ROW_INT>, gc, COL_THREADS, 0, st, data, ctx->d_tw, ctx->d_pc, RowPrimes<ROW_INT>(), l, y, 0, nullptr, 0.0);
+                launch(ntt16_rows_fwd<ROW_INT, 0, WIDE>, gr, ROW_THREADS, 0, st, data, ctx->d_tw, ctx->d_pc, RowPrimes<ROW_INT>(), l, y, 0, fin);
             }
             launches += skip_cols ? 1 : 2;
         }
