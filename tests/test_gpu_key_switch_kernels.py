@@ -119,6 +119,40 @@ def test_products_of_the_largest_words(bits):
     assert np.array_equal(got[1], orc.ct_ct_mul(ct[0], ct[0]))
 
 
+@pytest.mark.parametrize("bits", [50, 55])
+@pytest.mark.parametrize("log_n", [10, 11, 12])
+def test_small_ring_transforms_and_rescale_at_the_ends_of_the_range(log_n, bits):
+    """Rings with one, two and three stages after the rounds of three: transforms of the largest words and of words 0, (q +- 1)/2 and q - 1, and
+    rescales of one CTA per SM and of several."""
+    import torch
+    import paper_2608_17442_b200 as fesc
+    from oracle.ckks import Oracle
+
+    args = (log_n, S.ntt_primes(bits, log_n, 3, 0) + S.ntt_primes(60, log_n, 1, 0), 3, 1, 3, 67)
+    ctx, orc = fesc.Context(*args), Oracle(*args)
+    at = np.arange(orc.N)
+    rows = np.empty((3, 4, orc.N), dtype=np.uint64)
+    for i, q in enumerate(orc.q):
+        words = np.array([0, (q - 1) // 2, (q + 1) // 2, q - 1], dtype=np.uint64)
+        rows[0, i] = q - 1
+        rows[1, i] = words[(at * 2654435761 >> 7) % 4]
+        rows[2, i] = np.where(at % 2 == 0, (q - 1) // 2, (q + 1) // 2)
+    for gpu, ref in ((ctx.ntt, orc.ntt), (ctx.intt, orc.intt)):
+        d = to_dev(rows)
+        gpu(d, 3, 0, 4)
+        got = to_host(d)
+        for b in range(3):
+            assert np.array_equal(got[b], ref(rows[b], list(range(4)))), b
+    for batch in (1, 37, 150):      # 4, 148 and 600 CTAs
+        ct = np.ascontiguousarray(np.broadcast_to(rows[:2, :3], (batch, 2, 3, orc.N)))
+        ct[-1] = rows[1:, :3]
+        out = torch.empty((batch, 2, 2, orc.N), dtype=torch.int64, device="cuda")
+        ctx.rescale(to_dev(ct), out, batch, 3)
+        got = to_host(out)
+        for b in sorted({0, batch // 2, batch - 1}):
+            assert np.array_equal(got[b], orc.rescale(ct[b])), (batch, b)
+
+
 def test_threads_with_contexts_of_their_own():
     """Hoisted rotations of 1 and of 16 ciphertexts from two threads at a time: kernels whose shared memory depends on the call."""
     import threading
