@@ -136,7 +136,20 @@ __device__ __forceinline__ void small_fwd(const R& r, typename R::T (&x)[8], u64
     for (int k = 0; k < 8; k++) sm[at8<LOG, 4>(k)] = R::bits(x[k]);
     __syncthreads();
 }
-// Inverse: the buffer holds the row on entry (and a barrier has passed); x[k] = point k N/8 + tid on return, the last
+// Three stages of an inverse round on words up to 2 q, and the same for two of the three (LAST: the third is the caller's).  A stage doubles
+// the sums and leaves its products at (1/2 + 0.1875 B) q: after two stages words 0 and 4 may have reached 8 q and are folded; after three, words 1
+// (5 q) and 2 (4 q) are, and the rest stay below 2 q.  (All eight words folded after every round:
+// inverse transforms of 80 polynomials of 8 limbs at N = 2^11 10.3 us, so 9.9.)
+template <bool LAST, class R>
+__device__ __forceinline__ void inv_round(const R& r, typename R::T (&x)[8], uint32_t i0) {
+    inv8<2>(r, x, i0);
+    inv8<1>(r, x, i0);
+    x[0] = r.fold(x[0]), x[4] = r.fold(x[4]);
+    if (LAST) return;
+    inv8<0>(r, x, i0);
+    x[1] = r.fold(x[1]), x[2] = r.fold(x[2]);
+}
+// Inverse: the buffer holds the row on entry, centred (and a barrier has passed); x[k] = point k N/8 + tid on return, the last
 // stage still to be done (pairs k, k + 4).
 template <int LOG, class R>
 __device__ __forceinline__ void small_inv(const R& r, typename R::T (&x)[8], u64* sm) {
@@ -156,32 +169,25 @@ __device__ __forceinline__ void small_inv(const R& r, typename R::T (&x)[8], u64
             for (int k = 0; k < d; k++) r.gs(x[2 * d * b + k], x[2 * d * b + k + d], w);
         }
     }
-    fold8(r, x);
+    if (S == 3) x[0] = r.fold(x[0]), x[1] = r.fold(x[1]);      // 4 q and 2.75 q
 #pragma unroll
     for (int k = 0; k < 8; k++) sm[at8<LOG, 4>(k)] = R::bits(x[k]);
     __syncthreads();
 #pragma unroll
     for (int k = 0; k < 8; k++) x[k] = R::value(sm[at8<LOG, 3>(k)]);
-    inv8<2>(r, x, 64 + tid / L3);
-    inv8<1>(r, x, 64 + tid / L3);
-    inv8<0>(r, x, 64 + tid / L3);
-    fold8(r, x);
+    inv_round<false>(r, x, 64 + tid / L3);
 #pragma unroll
     for (int k = 0; k < 8; k++) sm[at8<LOG, 3>(k)] = R::bits(x[k]);
     __syncthreads();
 #pragma unroll
     for (int k = 0; k < 8; k++) x[k] = R::value(sm[at8<LOG, 2>(k)]);
-    inv8<2>(r, x, 8 + tid / L2);
-    inv8<1>(r, x, 8 + tid / L2);
-    inv8<0>(r, x, 8 + tid / L2);
-    fold8(r, x);
+    inv_round<false>(r, x, 8 + tid / L2);
 #pragma unroll
     for (int k = 0; k < 8; k++) sm[at8<LOG, 2>(k)] = R::bits(x[k]);
     __syncthreads();
 #pragma unroll
     for (int k = 0; k < 8; k++) x[k] = R::value(sm[at8<LOG, 1>(k)]);
-    inv8<2>(r, x, 1);
-    inv8<1>(r, x, 1);
+    inv_round<true>(r, x, 1);
 }
 // last inverse stage of an FP64 / integer row with the constants `s` (nullptr: the plain ones), canonical words to o
 template <int LOG>

@@ -130,3 +130,35 @@ def test_passes_whose_stages_fold_their_addends_stay_exact():
         assert run(b, {3}, 8) < 7.41 and run(b, {3, 7}, 8) < 2.10
     product = 0.5 + 0.1875 * run(modup, {3}, 8)  # in the key inner product
     assert 4 * product + 0.5 + 0.1875 / 2 < 8 and 4 * product + 0.5 < 8
+
+
+def inverse_stage(b, d):
+    """Bounds of eight words after an inverse stage of distance d: sums, and products of differences with centred twiddles."""
+    out = list(b)
+    for i in range(8):
+        if not i & d:
+            out[i] = b[i] + b[i + d]
+            out[i + d] = 0.5 + 0.1875 * (b[i] + b[i + d])
+    assert max(out) <= 8, out
+    return out
+
+
+@pytest.mark.parametrize("log_n", [10, 11, 12])
+def test_inverse_rounds_of_the_small_rings_stay_exact(log_n):
+    """Words enter centred; log N - 9 stages, then rounds of three that fold words 0 and 4 before their last stage and 1 and 2 after it.  The words
+    of a thread have one bound, as they had one place in the round before."""
+    first = log_n - 9
+    b = [0.5] * 8
+    for s in range(first):
+        b = inverse_stage(b, 1 << s)
+    if first == 3:
+        b[0] = b[1] = 0.5
+    for last in (False, False, True):
+        enter = max(b)
+        assert enter <= 2
+        b = inverse_stage(inverse_stage([enter] * 8, 1), 2)
+        b[0] = b[4] = 0.5
+        b = inverse_stage(b, 4)              # of the last round: sums and differences that the scaled products take
+        if not last:
+            b[1] = b[2] = 0.5
+    assert 0.5 + 0.375 * max(b) < 8
