@@ -26,6 +26,9 @@
 // stage at a time cost more than its butterflies.
 #define SM_ROW(LOG) (1u << LOG)
 #define SM_BYTES(LOG) (8 * (SM_ROW(LOG) + 2 * (1u << LOG)))
+// CTAs per SM that their shared memory leaves room for.  A rescale takes its 64 registers for it: 150 ciphertexts of 3 limbs at N = 2^12 41.4 us with 74
+// registers and one CTA per SM, 33.8 so.
+#define SM_CTAS(LOG) (32 >> ((LOG) - 8))
 typedef FpRowT<true> FpS;
 typedef IntRowT<true> IntS;
 template <int LOG>
@@ -43,11 +46,14 @@ __device__ __forceinline__ void small_tables(u64* sm, const SmallTables& tb, uin
     }
 }
 // (No __restrict__ on buffers that kernels write: see pdl_begin.)
+// The next kernel is let in after the wait and not before it: a kernel that still waits would let in the one after it, whose CTAs then sit on the SMs
+// that the first one's are to run on.  Rescales one after the other of 16 ciphertexts of 3 limbs at N = 2^12 17.8 us with the trigger first, 10.8 so; of
+// 40 of 6 limbs at N = 2^11 12.3 and 10.9; a rotation of one ciphertext of 2 limbs at N = 2^10 in four launches 30.8 and 25.1.
 #define SMALL_BEGIN(used, pi, inv)                                  \
     extern __shared__ __align__(16) u64 sm[];                       \
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); \
     if (used) small_tables<LOG>(sm, tb, pi, inv);                   \
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");              \
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
 // Stage S (0..2) of a round on eight registers: distance 4 >> S, twiddles (i0 << S) + j for the j-th group.  FOLD: as in fwd_stage.
 template <int S, bool FOLD, class R>
@@ -611,9 +617,9 @@ __global__ void __launch_bounds__(1 << (LOG - 3)) k_small_switch(SmallSwitch a, 
         u.pt = u.t < level ? u.t : a.n_q + (u.t - level);
         return u;
     };
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (rank < level) small_tables<LOG>(sm, tb, rank, true);
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     for (uint32_t l = rank; l < level; l += C) {
         if (l != rank) {
             __syncthreads();
@@ -679,7 +685,7 @@ __global__ void __launch_bounds__(1 << (LOG - 3)) k_small_last(const u64* in, si
 }
 // grid (level - 1, 2, batch): out = (in - NTT(centred(r) mod q_i)) q_last^-1
 template <int LOG>
-__global__ void __launch_bounds__(1 << (LOG - 3)) k_small_rescale(const u64* in, size_t in_stride, const u64* r, u64* out,
+__global__ void __launch_bounds__(1 << (LOG - 3), SM_CTAS(LOG)) k_small_rescale(const u64* in, size_t in_stride, const u64* r, u64* out,
                                                                   size_t out_stride, const RescaleTab* __restrict__ tab, SmallTables tb, uint32_t level) {
     constexpr uint32_t N = 1u << LOG, T = N / 8;
     const uint32_t i = blockIdx.x, pol = blockIdx.y, b = blockIdx.z, tid = threadIdx.x;
