@@ -598,9 +598,9 @@ struct SmallSwitch {
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
-// grid (CTAs of a cluster, batch)
+// grid (CTAs of a cluster, batch); 128 registers, so that an SM takes as many CTAs as the rule's figures were measured with
 template <int LOG>
-__global__ void __launch_bounds__(1 << (LOG - 3)) k_small_switch(SmallSwitch a, SmallTables tb) {
+__global__ void __launch_bounds__(1 << (LOG - 3), 16 >> (LOG - 8)) k_small_switch(SmallSwitch a, SmallTables tb) {
     extern __shared__ __align__(16) u64 sm[];
     constexpr uint32_t N = 1u << LOG;
     const uint32_t rank = blockIdx.x, C = gridDim.x, b = blockIdx.y, level = a.level, rows = level + a.K, beta = a.beta, others = rows - a.alpha;
@@ -810,14 +810,20 @@ int small_rescale(fesc_ctx* ctx, const u64* in, size_t in_stride, u64* out, size
     ctx->counters[0] += (uint64_t)batch * 2 * level;
     return FESC_OK;
 }
-// CTAs per ciphertext for one launch of k_small_switch, 0: the four kernels.  A barrier of a cluster costs less than a launch, but a
-// step's rows are taken by 8 or 16 CTAs in turn: one launch while all clusters run at once and a CTA has at most two rows to convert.
-// Product with a plaintext and two rotations at N = 2^12, 3 limbs (9 converted rows; 14 clusters of 16 run at once, 15 of 8), four launches /
-// one: 1 ciphertext 69.0 / 67.0 us, 4: 72.4 / 68.1 (8 CTAs 76.7), 9: 79.9 / 78.8, 16: 84.5 and no longer in one.
+// CTAs per ciphertext for one launch of k_small_switch, 0: the four kernels.  A barrier of a cluster costs less than a launch, but a step's rows are taken
+// by the cluster's CTAs in turn: one launch while a CTA converts at most one row and the clusters leave a sixteenth of the device free (N = 2^10 / 2^11 /
+// 2^12: 71 / 33 / 15 clusters of 8 and 31 / 14 / 7 of 16 fit; all 31 take 48 us where 28 take 30).  For five to eight rows both sizes will do: 16 while
+// they are few.  One rotation each, four launches / 8 / 16 CTAs, us:
+//   N = 2^12   3 limbs, 9 rows: 1 ciphertext 27.3 / 31.2 / 26.6, 6: 27.6 / 31.5 / 27.1, 15: 31.0 / 32.0 / -     4 limbs, 8 rows: 1: 38.2 / 41.0 / 38.8, 15: 51.7 / 41.6 / -
+//              6 limbs, 18 rows: 1: 38.4 / 60.2 / 45.0       N = 2^11   2 limbs, 2 rows: 1: 27.7 / 28.9 / 28.7, 28: 36.8 / 32.6 / -
+//   N = 2^11   4 limbs, 8 rows: 1: 28.4 / 31.0 / 29.3, 4: 30.9 / 31.5 / 29.8, 12: 36.9 / 31.7 / 33.6, 28: 43.9 / 35.9 / -     6 limbs, 18 rows: 8: 34.9 / 43.1 / 38.5
+//   N = 2^10   4 limbs, 4 rows: 1: 31.1 / 29.0 / 27.3, 28: 38.0 / 30.6 / 32.6, 64: 49.2 / 34.0 / -     8 limbs, 16 rows: 1: 33.0 / 41.4 / 29.1, 28: 45.1 / 44.8 / 35.4
 static uint32_t switch_ctas(const fesc_ctx* ctx, uint32_t level, uint32_t batch) {
     const uint32_t beta = (level + ctx->alpha - 1) / ctx->alpha, n_up = beta * (level + ctx->n_p) - level;
-    if (batch <= ctx->small_clusters[1] && n_up > 8 && n_up <= 32) return 16;
-    if (batch <= ctx->small_clusters[0] && n_up <= 16) return 8;
+    uint32_t most[2];      // clusters of 8 and of 16
+    for (int i = 0; i < 2; i++) most[i] = ctx->small_clusters[i] - (ctx->small_clusters[i] + 15) / 16;
+    if (n_up > (batch <= 6 ? 4 : 8) && n_up <= 16 && batch <= most[1]) return 16;
+    if (n_up <= 8 && batch <= most[0]) return 8;
     return 0;
 }
 template <int LOG>

@@ -75,23 +75,52 @@ def test_sums_that_are_reduced_in_between(batch, n_keys):
         assert np.array_equal(got[b], orc.rotate_sum_hoisted(ct[b], ids))
 
 
-@pytest.mark.parametrize("name,batch", [("tiny", 1), ("tiny", 14), ("tiny", 15), ("tiny", 16), ("tiny", 40), ("small", 2)])
-def test_small_rings_in_one_launch_and_in_four(name, batch):
-    """Key switches of small rings run as one launch while their clusters fit the device at once, as four beyond that."""
+def _launches(ctx, call):
+    before = ctx.counters()[4]
+    call()
+    return ctx.counters()[4] - before
+
+
+def _boundaries(ctx, orc, lv, key_id, most):
+    """Batches on both sides of every change of the number of launches of a rotation, the first and the last; launches by batch."""
     import torch
 
-    pair = ctx_pair(name)
+    d = torch.zeros((most, 2, lv, orc.N), dtype=torch.int64, device="cuda")
+    out = torch.empty_like(d)
+    n = [_launches(ctx, lambda: ctx.rotate(d, out, b, lv, key_id)) for b in range(1, most + 1)]
+    return sorted({1, most} | {b + k for b in range(1, most) if n[b - 1] != n[b] for k in (0, 1)}), n
+
+
+def _ring_of_2048():
+    import paper_2608_17442_b200 as fesc
+    from oracle.ckks import Oracle
+
+    args = (11, S.ntt_primes(50, 11, 6, 0) + S.ntt_primes(60, 11, 2, 0), 6, 2, 3, 65)
+    return fesc.Context(*args), Oracle(*args), None
+
+
+@pytest.mark.parametrize("name,levels", [("tiny", {3: (1, 4), 2: (1, 4), 1: (1, 4)}), ("2048", {6: (4, 4), 4: (1, 4), 1: (1, 4)}),
+                                         ("small", {24: (4, 4), 8: (1, 4), 5: (1, 4), 1: (1, 1)})])
+def test_small_rings_in_one_launch_and_in_four(name, levels):
+    """Key switches of small rings run as one launch while their clusters fit the device and convert few rows each, as four beyond that: the
+    launches of 1 and of 64 ciphertexts by level, and the oracle's words on either side of every change."""
+    import torch
+
+    pair = _ring_of_2048() if name == "2048" else ctx_pair(name)
     ctx, orc, _ = pair
     add_key(pair, 5, 91)
-    for lv in (24, 5, 1) if name == "small" else (3, 2, 1):
-        ct = random_ct(orc, 51, lv, lv, batch)
-        d, out = to_dev(ct), torch.empty((2, batch, 2, lv, orc.N), dtype=torch.int64, device="cuda")
-        ctx.rotate(d, out[0], batch, lv, 91)
-        ctx.ct_ct_mul(d, d, out[1], batch, lv)
-        got = to_host(out)
-        for b in sorted({0, batch // 2, batch - 1}):
-            assert np.array_equal(got[0, b], orc.rotate(ct[b], 91))
-            assert np.array_equal(got[1, b], orc.ct_ct_mul(ct[b], ct[b]))
+    for lv, ends in levels.items():
+        batches, launches = _boundaries(ctx, orc, lv, 91, 64)
+        assert (launches[0], launches[-1]) == ends and set(launches) <= {1, 4}, (lv, launches)
+        for batch in batches:
+            ct = random_ct(orc, 51, lv, lv, batch)
+            d, out = to_dev(ct), torch.empty((2, batch, 2, lv, orc.N), dtype=torch.int64, device="cuda")
+            assert _launches(ctx, lambda: ctx.rotate(d, out[0], batch, lv, 91)) == launches[batch - 1]
+            assert _launches(ctx, lambda: ctx.ct_ct_mul(d, d, out[1], batch, lv)) == 1 + launches[batch - 1]
+            got = to_host(out)
+            for b in sorted({0, batch // 2, batch - 1}):
+                assert np.array_equal(got[0, b], orc.rotate(ct[b], 91)), (lv, batch, b)
+                assert np.array_equal(got[1, b], orc.ct_ct_mul(ct[b], ct[b])), (lv, batch, b)
 
 
 @pytest.mark.parametrize("bits", [36, 50, 51, 55])
