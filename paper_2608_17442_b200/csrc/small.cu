@@ -605,14 +605,14 @@ __global__ void __launch_bounds__(1 << (LOG - 3), 16 >> (LOG - 8)) k_small_switc
     constexpr uint32_t N = 1u << LOG;
     const uint32_t rank = blockIdx.x, C = gridDim.x, b = blockIdx.y, level = a.level, rows = level + a.K, beta = a.beta, others = rows - a.alpha;
     const uint32_t n_up = beta * rows - level;
-    // converted row `task`: every digit but the last has `others` of them
+    // converted row `task`: every digit but the last has `others` of them (with one digit `others` may be anything)
     struct Up {
         uint32_t j, t, pt;
     };
     auto up_row = [&](uint32_t task) {
         Up u;
-        u.j = task / others < beta - 1 ? task / others : beta - 1;
-        const uint32_t d = task - u.j * others, first = u.j * a.alpha, n = first + a.alpha < level ? a.alpha : level - first;
+        u.j = beta == 1 ? 0 : task / others < beta - 1 ? task / others : beta - 1;
+        const uint32_t d = u.j ? task - u.j * others : task, first = u.j * a.alpha, n = first + a.alpha < level ? a.alpha : level - first;
         u.t = d < first ? d : d + n;
         u.pt = u.t < level ? u.t : a.n_q + (u.t - level);
         return u;

@@ -182,6 +182,26 @@ def test_small_ring_transforms_and_rescale_at_the_ends_of_the_range(log_n, bits)
             assert np.array_equal(got[b], orc.rescale(ct[b])), (batch, b)
 
 
+@pytest.mark.parametrize("log_n", [10, 11, 12])
+def test_one_digit_of_more_limbs_than_the_level_and_the_special_primes(log_n):
+    """Levels below the digit's size: every converted row belongs to the one digit there is."""
+    import torch
+    import paper_2608_17442_b200 as fesc
+    from oracle.ckks import Oracle
+
+    args = (log_n, S.ntt_primes(45, log_n, 4, 0) + S.ntt_primes(60, log_n, 1, 0), 4, 1, 1, 66)
+    pair = (fesc.Context(*args), Oracle(*args), None)
+    ctx, orc, _ = pair
+    add_key(pair, 3, 92)
+    for lv in (1, 2, 3, 4):
+        ct = random_ct(orc, 52, lv, lv, 2)
+        d, out = to_dev(ct), torch.empty((2, 2, lv, orc.N), dtype=torch.int64, device="cuda")
+        assert _launches(ctx, lambda: ctx.rotate(d, out, 2, lv, 92)) == 1
+        got = to_host(out)
+        for b in range(2):
+            assert np.array_equal(got[b], orc.rotate(ct[b], 92)), (lv, b)
+
+
 def test_threads_with_contexts_of_their_own():
     """Hoisted rotations of 1 and of 16 ciphertexts from two threads at a time: kernels whose shared memory depends on the call."""
     import threading
