@@ -159,7 +159,8 @@ int fesc_ctx_counters(const fesc_ctx* ctx, uint64_t out[8]);
  * the summed milliseconds and record counts per family and clears the records.  Families:
  * 0 NTT/INTT, 1 ModUp conversion, 2 key inner product, 3 ModDown conversion and finish,
  * 4 automorphism gather, 5 BSGS accumulate, 6 rescale pointwise parts, 7 ct-pt MAC / tensor.
- * Launches beyond the reserved records are not timed.
+ * Launches beyond the reserved records are not timed.  Rings 2^10 .. 2^12: a key switch that would be one launch runs as its
+ * steps while one of the families 0 to 3 is timed.
  */
 int fesc_profile_enable(fesc_ctx* ctx, int mask, uint32_t max_records);
 int fesc_profile_read(fesc_ctx* ctx, float ms[8], uint64_t records[8]);

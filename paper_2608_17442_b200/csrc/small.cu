@@ -819,6 +819,7 @@ int small_rescale(fesc_ctx* ctx, const u64* in, size_t in_stride, u64* out, size
 //   N = 2^11   4 limbs, 8 rows: 1: 28.4 / 31.0 / 29.3, 4: 30.9 / 31.5 / 29.8, 12: 36.9 / 31.7 / 33.6, 28: 43.9 / 35.9 / -     6 limbs, 18 rows: 8: 34.9 / 43.1 / 38.5
 //   N = 2^10   4 limbs, 4 rows: 1: 31.1 / 29.0 / 27.3, 28: 38.0 / 30.6 / 32.6, 64: 49.2 / 34.0 / -     8 limbs, 16 rows: 1: 33.0 / 41.4 / 29.1, 28: 45.1 / 44.8 / 35.4
 static uint32_t switch_ctas(const fesc_ctx* ctx, uint32_t level, uint32_t batch) {
+    if (ctx->prof.on & (1u << PF_NTT | 1u << PF_MODUP | 1u << PF_INNER | 1u << PF_MODDOWN)) return 0;      // the steps are timed one by one
     const uint32_t beta = (level + ctx->alpha - 1) / ctx->alpha, n_up = beta * (level + ctx->n_p) - level;
     uint32_t most[2];      // clusters of 8 and of 16
     for (int i = 0; i < 2; i++) most[i] = ctx->small_clusters[i] - (ctx->small_clusters[i] + 15) / 16;

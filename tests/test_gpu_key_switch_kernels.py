@@ -202,6 +202,27 @@ def test_one_digit_of_more_limbs_than_the_level_and_the_special_primes(log_n):
             assert np.array_equal(got[b], orc.rotate(ct[b], 92)), (lv, b)
 
 
+def test_steps_of_a_small_key_switch_are_timed_apart():
+    """While the families of a key switch are timed, it runs as its four steps, one record each."""
+    import torch
+
+    pair = ctx_pair("tiny")
+    ctx, orc, _ = pair
+    add_key(pair, 5, 91)
+    ct = random_ct(orc, 53, 3, 3, 1)
+    d, out = to_dev(ct), torch.empty((1, 2, 3, orc.N), dtype=torch.int64, device="cuda")
+    families = ("ntt", "modup", "inner", "moddown")
+    ctx.profile_enable(families, 64)
+    try:
+        ctx.rotate(d, out, 1, 3, 91)
+        read = ctx.profile_read()
+    finally:
+        ctx.profile_enable(())
+    assert [read[f][1] for f in families] == [1, 1, 1, 1]
+    assert np.array_equal(to_host(out)[0], orc.rotate(ct[0], 91))
+    assert _launches(ctx, lambda: ctx.rotate(d, out, 1, 3, 91)) == 1
+
+
 def test_threads_with_contexts_of_their_own():
     """Hoisted rotations of 1 and of 16 ciphertexts from two threads at a time: kernels whose shared memory depends on the call."""
     import threading
