@@ -16,16 +16,18 @@ def _pair(bits, n_p):
     return fesc.Context(*args), Oracle(*args), None
 
 
-@pytest.mark.parametrize("bits,n_p", [(60, 4), (55, 2), (51, 1), (61, 2)])
+@pytest.mark.parametrize("bits,n_p", [(60, 4), (55, 2), (51, 1), (61, 2), (49, 4), (40, 2)])
 def test_key_switches_by_size_of_the_special_primes(bits, n_p):
-    """Special primes next to 2^60 and next to 2^51 from below, and 61 bits, which the fused division does not take: their transforms at the
-    ends of the range, a relinearisation, a rotation, hoisted rotations and their sum."""
+    """Special primes next to 2^60 and next to 2^51 from below, 61 bits, which the fused division does not take, and 49 and 40 bits, whose rows
+    (and key words) are FP64 rows like the data primes': their keys, their transforms at the ends of the range, a relinearisation, a
+    rotation, hoisted rotations and their sum."""
     import torch
 
     pair = _pair(bits, n_p)
     ctx, orc, _ = pair
     for k, rot in enumerate((3, -8, 4096)):
         add_key(pair, rot, 70 + k)
+    assert np.array_equal(to_host(ctx.export_key(71)), orc.keys[71][1])      # kept in another form, handed out as residues
     idx = list(range(5, 5 + n_p))
     rows = np.empty((2, n_p, orc.N), dtype=np.uint64)
     for k, i in enumerate(idx):
@@ -123,29 +125,24 @@ def test_small_rings_in_one_launch_and_in_four(name, levels):
                 assert np.array_equal(got[1, b], orc.ct_ct_mul(ct[b], ct[b])), (lv, batch, b)
 
 
-@pytest.mark.parametrize("bits", [36, 50, 51, 55])
-def test_products_of_the_largest_words(bits):
-    """Products with relinearisation on both sides of 2^50, where FP64 products end: words 0, 1, (q +- 1)/2, q - 2 and q - 1 against each other."""
+@pytest.mark.parametrize("log_n", [10, 11, 12])
+def test_one_digit_of_more_limbs_than_the_level_and_the_special_primes(log_n):
+    """Levels below the digit's size: every converted row belongs to the one digit there is."""
     import torch
     import paper_2608_17442_b200 as fesc
     from oracle.ckks import Oracle
 
-    args = (12, S.ntt_primes(bits, 12, 3, 0) + S.ntt_primes(60, 12, 1, 0), 3, 1, 3, 63)
-    ctx, orc = fesc.Context(*args), Oracle(*args)
-    ct = np.empty((2, 2, 3, orc.N), dtype=np.uint64)
-    at = np.arange(orc.N)
-    for l in range(3):
-        q = orc.q[l]
-        words = np.array([0, 1, (q - 1) // 2, (q + 1) // 2, q - 2, q - 1], dtype=np.uint64)
-        for k in range(4):
-            ct[k // 2, k % 2, l] = words[at // 6**k % 6]
-    out = torch.empty((2, 2, 3, orc.N), dtype=torch.int64, device="cuda")
-    a, b = to_dev(ct), to_dev(ct[::-1].copy())
-    ctx.ct_ct_mul(a, b, out[:1], 1, 3)
-    ctx.ct_ct_mul(a, a, out[1:], 1, 3)
-    got = to_host(out)
-    assert np.array_equal(got[0], orc.ct_ct_mul(ct[0], ct[1]))
-    assert np.array_equal(got[1], orc.ct_ct_mul(ct[0], ct[0]))
+    args = (log_n, S.ntt_primes(45, log_n, 4, 0) + S.ntt_primes(60, log_n, 1, 0), 4, 1, 1, 66)
+    pair = (fesc.Context(*args), Oracle(*args), None)
+    ctx, orc, _ = pair
+    add_key(pair, 3, 92)
+    for lv in (1, 2, 3, 4):
+        ct = random_ct(orc, 52, lv, lv, 2)
+        d, out = to_dev(ct), torch.empty((2, 2, lv, orc.N), dtype=torch.int64, device="cuda")
+        assert _launches(ctx, lambda: ctx.rotate(d, out, 2, lv, 92)) == 1
+        got = to_host(out)
+        for b in range(2):
+            assert np.array_equal(got[b], orc.rotate(ct[b], 92)), (lv, b)
 
 
 @pytest.mark.parametrize("bits", [50, 55])
@@ -182,26 +179,6 @@ def test_small_ring_transforms_and_rescale_at_the_ends_of_the_range(log_n, bits)
             assert np.array_equal(got[b], orc.rescale(ct[b])), (batch, b)
 
 
-@pytest.mark.parametrize("log_n", [10, 11, 12])
-def test_one_digit_of_more_limbs_than_the_level_and_the_special_primes(log_n):
-    """Levels below the digit's size: every converted row belongs to the one digit there is."""
-    import torch
-    import paper_2608_17442_b200 as fesc
-    from oracle.ckks import Oracle
-
-    args = (log_n, S.ntt_primes(45, log_n, 4, 0) + S.ntt_primes(60, log_n, 1, 0), 4, 1, 1, 66)
-    pair = (fesc.Context(*args), Oracle(*args), None)
-    ctx, orc, _ = pair
-    add_key(pair, 3, 92)
-    for lv in (1, 2, 3, 4):
-        ct = random_ct(orc, 52, lv, lv, 2)
-        d, out = to_dev(ct), torch.empty((2, 2, lv, orc.N), dtype=torch.int64, device="cuda")
-        assert _launches(ctx, lambda: ctx.rotate(d, out, 2, lv, 92)) == 1
-        got = to_host(out)
-        for b in range(2):
-            assert np.array_equal(got[b], orc.rotate(ct[b], 92)), (lv, b)
-
-
 def test_steps_of_a_small_key_switch_are_timed_apart():
     """While the families of a key switch are timed, it runs as its four steps, one record each."""
     import torch
@@ -221,6 +198,31 @@ def test_steps_of_a_small_key_switch_are_timed_apart():
     assert [read[f][1] for f in families] == [1, 1, 1, 1]
     assert np.array_equal(to_host(out)[0], orc.rotate(ct[0], 91))
     assert _launches(ctx, lambda: ctx.rotate(d, out, 1, 3, 91)) == 1
+
+
+@pytest.mark.parametrize("bits", [36, 50, 51, 55])
+def test_products_of_the_largest_words(bits):
+    """Products with relinearisation on both sides of 2^50, where FP64 products end: words 0, 1, (q +- 1)/2, q - 2 and q - 1 against each other."""
+    import torch
+    import paper_2608_17442_b200 as fesc
+    from oracle.ckks import Oracle
+
+    args = (12, S.ntt_primes(bits, 12, 3, 0) + S.ntt_primes(60, 12, 1, 0), 3, 1, 3, 63)
+    ctx, orc = fesc.Context(*args), Oracle(*args)
+    ct = np.empty((2, 2, 3, orc.N), dtype=np.uint64)
+    at = np.arange(orc.N)
+    for l in range(3):
+        q = orc.q[l]
+        words = np.array([0, 1, (q - 1) // 2, (q + 1) // 2, q - 2, q - 1], dtype=np.uint64)
+        for k in range(4):
+            ct[k // 2, k % 2, l] = words[at // 6**k % 6]
+    out = torch.empty((2, 2, 3, orc.N), dtype=torch.int64, device="cuda")
+    a, b = to_dev(ct), to_dev(ct[::-1].copy())
+    ctx.ct_ct_mul(a, b, out[:1], 1, 3)
+    ctx.ct_ct_mul(a, a, out[1:], 1, 3)
+    got = to_host(out)
+    assert np.array_equal(got[0], orc.ct_ct_mul(ct[0], ct[1]))
+    assert np.array_equal(got[1], orc.ct_ct_mul(ct[0], ct[0]))
 
 
 def test_threads_with_contexts_of_their_own():
