@@ -333,10 +333,10 @@ static int launch_moddown(fesc_ctx* ctx, const u64* acc, u64* u, uint32_t level,
     const size_t smem = ((size_t)A * MU_SRC + MD_GROUPS * COL_SMEM(MU_COLS)) * sizeof(u64);
     auto kern = k_moddown_cols<A, OPEN>;
     FESC_CHECK_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    // Two CTAs share the limbs of a tile where its places (two per SM) would be half empty otherwise.  Each opens the special rows again, which costs as
-    // much as a third of 24 limbs: one rotation of 24 / 15 / 9 / 5 limbs with 1, 2, 4 CTAs per tile 277, 260, 271 / 194, 188, 194 / 155, 147, 160 /
+    // Two CTAs share the limbs of a tile for the two polynomials of one ciphertext, which would leave more than half of the places (two per SM) empty
+    // otherwise.  Each opens the special rows again, which costs as much as a third of 24 limbs: one rotation of 24 / 15 / 9 / 5 limbs with 1, 2, 4 CTAs per tile 277, 260, 271 / 194, 188, 194 / 155, 147, 160 /
     // 114, 106, 113 us; two: 395, 400, 416 / 250, 257, 269 / 195, 205, 219 / 138, 150, 163; eight of 24 limbs 1239, 1265, 1341.
-    const uint32_t splits = tiles * polys <= 148 ? 2 : 1;
+    const uint32_t splits = polys <= 2 ? 2 : 1;
     launch(kern, dim3(tiles * splits, polys), MD_THREADS, smem, st, acc, u, ctx->tabs.d_moddown, ctx->d_twf, ctx->d_itw, ctx->tabs.d_down_scale, ctx->d_pc,
            level, ctx->n_q, ctx->n_p, splits);
     return FESC_OK;

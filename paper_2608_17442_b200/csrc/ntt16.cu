@@ -191,7 +191,7 @@ __global__ void __launch_bounds__(ROW_THREADS, 1024 / ROW_THREADS)
             for (int j = h; j < h + 4; j++) {
                 const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(s + 72 * j);
                 double a0 = fp_from_u64(av[j].x), a1 = fp_from_u64(av[j].y);
-                if (FIN == 2) {             // lazy products below 0.7 q
+                if (FIN == 2) {             // lazy products below 0.875 q, the difference below 3 q
                     const ulonglong2 w2 = pt ? ld_pair_once<WIDE>(pt + 64 * j) : make_ulonglong2(0, 0);
                     a0 = fp_modmul(a0, pt ? fp_from_u64(w2.x) : mul, q, qinv);
                     a1 = fp_modmul(a1, pt ? fp_from_u64(w2.y) : mul, q, qinv);

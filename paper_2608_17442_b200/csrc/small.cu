@@ -325,7 +325,7 @@ __device__ __forceinline__ void modup_row(u64* sm, uint32_t j, uint32_t t, uint3
         double x[8];
 #pragma unroll
         for (int k = 0; k < 8; k++) x[k] = 0.0;
-        for (uint32_t a = 0; a < n_src; a++) {         // every product below 0.875 q, folded back after the fourth
+        for (uint32_t a = 0; a < n_src; a++) {         // every product below 0.875 q, folded back after every third
             const double m = dg->matd[a][pt];
 #pragma unroll
             for (int k = 0; k < 8; k++) x[k] += fp_modmul(fp_from_u64(src[(size_t)a * N + k * T]), m, r.q, r.qinv);
@@ -735,7 +735,7 @@ static int small_attr(fesc_ctx* ctx) {
     }
     return FESC_OK;
 }
-int small_init(fesc_ctx* ctx) {      // up to 98 KB of shared memory per CTA
+int small_init(fesc_ctx* ctx) {      // up to 96 KB of shared memory per CTA
     return ctx->log_n == 12 ? small_attr<12>(ctx) : ctx->log_n == 11 ? small_attr<11>(ctx) : small_attr<10>(ctx);
 }
 bool small_ring(const fesc_ctx* ctx) { return ctx->log_n >= 10 && ctx->log_n <= 12; }
