@@ -3,7 +3,7 @@ import numpy as np
 import pytest
 
 import fesc_synth as S
-from gpu_util import add_key, ctx_pair, random_ct, to_dev, to_host
+from gpu_util import add_key, random_ct, to_dev, to_host
 
 pytestmark = pytest.mark.gpu
 
@@ -93,11 +93,16 @@ def _boundaries(ctx, orc, lv, key_id, most):
     return sorted({1, most} | {b + k for b in range(1, most) if n[b - 1] != n[b] for k in (0, 1)}), n
 
 
-def _ring_of_2048():
+def _small_pair(name):
+    """Contexts of the test's own: their scratch goes with them (a later test of the suite fills the device)."""
     import paper_2608_17442_b200 as fesc
     from oracle.ckks import Oracle
 
-    args = (11, S.ntt_primes(50, 11, 6, 0) + S.ntt_primes(60, 11, 2, 0), 6, 2, 3, 65)
+    if name == "2048":
+        args = (11, S.ntt_primes(50, 11, 6, 0) + S.ntt_primes(60, 11, 2, 0), 6, 2, 3, 65)
+    else:
+        p = S.params(name)
+        args = (p["log_n"], p["primes"], p["n_q"], p["n_p"], p["dnum"], p["seed"])
     return fesc.Context(*args), Oracle(*args), None
 
 
@@ -108,7 +113,7 @@ def test_small_rings_in_one_launch_and_in_four(name, levels):
     launches of 1 and of 64 ciphertexts by level, and the oracle's words on either side of every change."""
     import torch
 
-    pair = _ring_of_2048() if name == "2048" else ctx_pair(name)
+    pair = _small_pair(name)
     ctx, orc, _ = pair
     add_key(pair, 5, 91)
     for lv, ends in levels.items():
@@ -183,7 +188,7 @@ def test_steps_of_a_small_key_switch_are_timed_apart():
     """While the families of a key switch are timed, it runs as its four steps, one record each."""
     import torch
 
-    pair = ctx_pair("tiny")
+    pair = _small_pair("tiny")
     ctx, orc, _ = pair
     add_key(pair, 5, 91)
     ct = random_ct(orc, 53, 3, 3, 1)
@@ -258,5 +263,6 @@ def test_threads_with_contexts_of_their_own():
         t.start()
     for t in threads:
         t.join()
+    torch.cuda.empty_cache()
     assert not errors, errors
     assert torch.equal(results[1], results[16])       # the first ciphertext of both batches is the same
